@@ -100,13 +100,17 @@ void head_widths(const cerb_config* g, int w[CERB_MAX_HEADS][CERB_MAX_LEVELS + 1
   *wmax = mx;
 }
 
-size_t part_floats_needed(const cerb_config* g, int Mmax, int sm_count) {
+// Mmax: rows of the widest forward; lm_rows: rows of the widest LM head (a prefill needs its logits at one row per sequence).
+size_t part_floats_needed(const cerb_config* g, int Mmax, int lm_rows, int sm_count) {
   const int HD = g->n_heads * g->head_dim;
   const int shapes[5][2] = {{3 * HD, g->d_model}, {g->d_model, HD}, {2 * g->mlp_dim, g->d_model},
                             {g->d_model, g->mlp_dim}, {g->vocab, g->d_model}};
   size_t best = 0;
   for (int i = 0; i < 5; ++i)
-    for (int M = 1; M <= Mmax; ++M) {
+    // the plan depends on whether M exceeds 128 and on the number of 256-row chunks, so the last M of each class decides
+    for (int M = 0, top = i == 4 ? lm_rows : Mmax; M < top;) {
+      M = M == 0 ? (top < 128 ? top : 128) : M == 128 ? (top < kGemmRowsPerPass ? top : kGemmRowsPerPass)
+                                                     : (top < M + kGemmRowsPerPass ? top : M + kGemmRowsPerPass);
       int ns = g->dtype == CERB_BF16 ? gemm_plan_split(sm_count, M, shapes[i][0], shapes[i][1]) : 1;
       size_t f = (size_t)ns * M * shapes[i][0];
       if (f > best) best = f;
@@ -130,6 +134,7 @@ size_t carve(cerb_ctx* c, char* base) {
   c->d_naccept = b.take<int32_t>(MB);
   c->d_kper = b.take<int32_t>(CERB_MAX_HEADS);
   c->d_rowoff = b.take<int32_t>(CERB_MAX_BATCH + 1);
+  c->d_iota = b.take<int32_t>(c->Mmax);
   c->d_S = b.take<float>(MB);
   c->d_path = b.take<int32_t>(MB * kPathMax);
   c->d_outtok = b.take<int32_t>(MB * kPathMax);
@@ -162,13 +167,17 @@ void init_sizes(cerb_ctx* c, const cerb_config* g, int sm_count) {
   c->cfg = *g;
   c->bf16 = g->dtype == CERB_BF16;
   c->esize = c->bf16 ? 2 : 4;
-  // rows per sequence of one forward: the widest tree, or a prefill chunk (128 prompt tokens whatever max_nodes is)
-  const int rows_seq = g->max_nodes > kPrefillChunkMax ? g->max_nodes : kPrefillChunkMax;
+  // rows per sequence of one forward: the widest tree, or the least that a prefill forward takes of every sequence
+  const int rows_seq = g->max_nodes > kPrefillQuantum ? g->max_nodes : kPrefillQuantum;
   c->Mmax = g->max_batch * rows_seq;
   c->max_pos = g->max_pages * CERB_PAGE;
+  // ... or a whole prefill forward, as far as the caches can hold one
+  const long long cap = (long long)g->max_batch * c->max_pos;
+  const int pre = cap < kPrefillRows ? round_up((int)cap, kPrefillQuantum) : kPrefillRows;
+  if (pre > c->Mmax) c->Mmax = pre;
   c->sm_count = sm_count;
   head_widths(g, c->head_w, &c->head_wmax);
-  c->part_floats = part_floats_needed(g, c->Mmax, sm_count);
+  c->part_floats = part_floats_needed(g, c->Mmax, g->max_batch * g->max_nodes, sm_count);
   c->attn_scratch_bytes = attn_scratch_bytes(g->max_batch, rows_seq, g->n_heads, g->head_dim);
 }
 
@@ -257,7 +266,7 @@ struct OrderCheck {
 // rows / row_off: with ragged rows (cerb_step on a batch whose sequences chose different modes) sequence b owns the
 // rows row_off[b] .. row_off[b] + n_active[b] - 1 of every activation buffer and `rows` is their total; otherwise
 // row_off is null and sequence b owns rows b * n .. b * n + n - 1.
-// need: per sequence, how many of the n rows are live (host; a prefill chunk near the end of a prompt), or null = n.
+// need: per sequence, how many of the n rows are live (host; a prefill chunk), or null = n.
 int forward_rows(cerb_ctx* c, const cerb_tree* tree, const int32_t* tok, int tok_stride, int tok_off, int n,
                  cudaStream_t st, int rows = 0, const int32_t* row_off = nullptr, const int* need = nullptr) {
   const cerb_config& g = c->cfg;
@@ -320,7 +329,7 @@ int forward_rows(cerb_ctx* c, const cerb_tree* tree, const int32_t* tok, int tok
     CERB_ORDER(oc, LO_ATTN);
     { ProfScope ps(c, K_ATTN, st);
       CERB_TRY(launch_tree_attention(c, &a, c->bf16 ? &c->tm_kpool[l] : nullptr, c->bf16 ? &c->tm_vpool[l] : nullptr,
-                                     c->sm_count, c->d_status, st, row_off)); }
+                                     c->sm_count, c->d_status, st, row_off, tree == c->chain)); }
     CERB_ORDER(oc, LO_GEMM_WO);
     { ProfScope ps(c, K_GEMM, st);
       CERB_TRY(gemm(c, c->d_attn, &c->tm_attn, c->wo[l], c->bf16 ? &c->tm_wo[l] : nullptr, M, d, HD, &ns, st)); }
@@ -491,11 +500,14 @@ int cerb_load(const cerb_config* cfg, const cerb_weights* w, void* workspace_dev
       if ((rc = make_act_maps(&c->tm_hlast, c->d_hlast, CERB_MAX_BATCH, g.d_model)) != CERB_OK) break;
     }
     if ((rc = launch_rope_table(c, 0)) != CERB_OK) break;
-    const int chunk = kPrefillChunkMax;
-    std::vector<int32_t> par(chunk);
+    const int chunk = kPrefillQuantum;
+    std::vector<int32_t> par(chunk), iota(c->Mmax);
+    for (int v = 0; v < c->Mmax; ++v) iota[v] = v;
+    if (cudaMemcpy(c->d_iota, iota.data(), iota.size() * sizeof(int32_t), cudaMemcpyHostToDevice) != cudaSuccess) { rc = CERB_E_CUDA; break; }
     for (int v = 0; v < chunk; ++v) par[v] = v - 1;
     // the prefill chain is deeper than an acceptable path may be: no depth limit for it
     if ((rc = tree_build(c, par.data(), nullptr, nullptr, chunk, CERB_MAX_TREES, false, false, &c->chain)) != CERB_OK) break;
+    c->chain->dev.depth = c->d_iota;        // (a chunk may be longer than a tree; its attention windows are chains of 128)
     int32_t one = -1;
     if ((rc = tree_build(c, &one, nullptr, nullptr, 1, CERB_MAX_TREES + 1, false, true, &c->single)) != CERB_OK) break;
     if (cudaDeviceSynchronize() != cudaSuccess) { rc = CERB_E_CUDA; break; }
@@ -561,17 +573,30 @@ int cerb_prefill(cerb_ctx* c, const int32_t* tokens_dev, const int32_t* lens_hos
   CERB_CUDA_OK(cudaStreamSynchronize(st));
   for (int b = 0; b < B; ++b) c->h_stage[b] = lens_host[b];
   CERB_CUDA_OK(cudaMemcpyAsync(c->d_lens_in, c->h_stage, B * sizeof(int32_t), cudaMemcpyHostToDevice, st));
-  const int C = c->chain->n;          // 128 tokens per chunk
-  for (int off = 0; off < longest; off += C) {
-    int need[CERB_MAX_BATCH];
-    for (int b = 0; b < B; ++b) {
-      c->h_len[b] = lens_host[b] < off ? lens_host[b] : off;
-      const int left = lens_host[b] - off;
-      need[b] = left < 0 ? 0 : left < C ? left : C;
+  // Every forward takes the next C tokens of each prompt (fewer where a prompt ends), C the largest multiple of 128 whose
+  // live tokens fit a forward; only live tokens have rows.
+  for (int off = 0, C; off < longest; off += C) {
+    int need[CERB_MAX_BATCH], rows = 0;
+    auto take = [&](int chunk) {
+      rows = 0;
+      for (int b = 0; b < B; ++b) {
+        const int left = lens_host[b] - off;
+        need[b] = left < 0 ? 0 : left < chunk ? left : chunk;
+        rows += need[b];
+      }
+    };
+    C = kPrefillQuantum;
+    for (int more = C + kPrefillQuantum; C < longest - off; more += kPrefillQuantum) {
+      take(more);
+      if (rows > c->Mmax) break;
+      C = more;
     }
+    if (C > longest - off) C = longest - off;
+    take(C);
+    for (int b = 0; b < B; ++b) c->h_len[b] = lens_host[b] < off ? lens_host[b] : off;
     CERB_TRY(launch_set_nactive(c, 1, off, C, st));
-    CERB_TRY(forward_rows(c, c->chain, tokens_dev, max_len, off, C, st, 0, nullptr, need));
-    CERB_TRY(launch_prefill_commit(c, C, st));
+    CERB_TRY(forward_rows(c, c->chain, tokens_dev, max_len, off, C, st, rows, c->d_rowoff, need));
+    CERB_TRY(launch_prefill_commit(c, st));
   }
   for (int b = 0; b < B; ++b) c->h_len[b] = lens_host[b];
   // root = argmax LH(h_last)

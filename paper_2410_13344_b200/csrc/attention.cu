@@ -27,6 +27,7 @@ constexpr int kTargetCtas = 296;          // two CTAs per SM on a 148-SM part
 constexpr int kMaxSplit = 32;
 constexpr int kMaxPagesPerCta = 1024;
 constexpr size_t kCounterBytes = 4096;    // one ticket counter per (sequence, head)
+constexpr int kAttnRowsPerLaunch = 128;   // query rows a CTA holds at most
 
 // K/V tiles are read once per step (the next layer's tiles, and 13 GB of weights, come before they are needed
 // again): they enter L2 with evict-first priority so that they do not push out activations and partial sums.
@@ -78,6 +79,9 @@ struct AttnParams {
   unsigned int* counters;   // [B*H]
   int32_t* status;
   int n, H, max_pages, nsplit, oob_row;
+  int B;
+  int win;                  // > 1: a prefill chunk of up to win * 128 consecutive tokens per sequence, one window of 128 query
+                            // rows per blockIdx.z (locate_window); 1 otherwise
   int row0, rows;           // query rows row0 .. row0 + rows - 1 of the tree are this launch's (q, out, lse and anc already point
                             // at row0); a tree of more than 128 nodes takes two launches.  n stays the tree's node count
                             // (the row stride between sequences); only keys below row0 + rows can be ancestors of these rows.
@@ -87,6 +91,15 @@ struct AttnParams {
   int cluster;              // tensor-core path: the splits of a (sequence, head) form one cluster and merge through shared memory
   float scale_log2;
 };
+
+// Which sequence, and which window of 128 query rows of it, a CTA's blockIdx.z stands for.  A prefill chunk is one long
+// chain: window w is a chain of 128 nodes behind `shift` = 128 w more prefix keys, all of them in the cache before this
+// launch.  The last windows see the most keys and come first, so that the short ones fill the launch's tail.
+__device__ __forceinline__ void locate_window(const AttnParams& p, int& b, int& shift) {
+  const int z = (int)blockIdx.z;
+  b = p.win > 1 ? z % p.B : z;
+  shift = p.win > 1 ? (p.win - 1 - z / p.B) * kAttnRowsPerLaunch : 0;
+}
 
 template <int DH, int WQ, int WK, int STAGES>
 __global__ void __launch_bounds__((WQ * WK + 1) * 32) tree_attn_bf16_kernel(const __grid_constant__ CUtensorMap tmK,
@@ -119,10 +132,12 @@ __global__ void __launch_bounds__((WQ * WK + 1) * 32) tree_attn_bf16_kernel(cons
   // set-up, the page list and the first prefix tiles run before griddep_wait() and overlap the previous
   // kernel's tail; Q and this step's tree keys are only touched after it.
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int split = blockIdx.x, h = blockIdx.y, b = blockIdx.z;
-  const int L = p.len[b];
-  const int nq_all = p.n_active ? min(p.n_active[b], p.n) : p.n;      // live nodes of this sequence
-  const size_t qrow = p.row_off ? (size_t)p.row_off[b] : (size_t)b * p.n;   // this sequence's first row of q and out
+  const int split = blockIdx.x, h = blockIdx.y;
+  int b, shift;
+  locate_window(p, b, shift);
+  const int L_old = p.len[b], L = L_old + shift;                      // keys written by earlier launches; keys every row sees
+  const int nq_all = (p.n_active ? min(p.n_active[b], p.n) : p.n) - shift;   // live nodes of this sequence (from the window on)
+  const size_t qrow = (p.row_off ? (size_t)p.row_off[b] : (size_t)b * p.n) + shift;   // its first row of q and out
   const int nq = min(nq_all - p.row0, p.rows);                        // live query rows of this launch
   if (nq <= 0) return;
   const int kv_total = L + min(nq_all, p.row0 + p.rows);
@@ -160,7 +175,7 @@ __global__ void __launch_bounds__((WQ * WK + 1) * 32) tree_attn_bf16_kernel(cons
     __syncwarp();
     if (lane == 0) {
       int early = 0;
-      while (t0 + early < t_end && early < STAGES && (t0 + early + 1) * TILE <= L) ++early;
+      while (t0 + early < t_end && early < STAGES && (t0 + early + 1) * TILE <= L_old) ++early;
       // (the abort flag itself is looked at once, for a launch that starts after a time-out: nothing is issued then;
       // later a wait that gives up says so in its return value, which costs the loop nothing)
       const int t_stop = *aborted ? t0 : t_end;
@@ -387,12 +402,12 @@ __global__ void __launch_bounds__((WQ * WK + 1) * 32) tree_attn_bf16_kernel(cons
         for (int r = ct; r < nq; r += nct)
           p.lse[((size_t)b * p.H + h) * p.n + r] = (mrg[(size_t)r * ROWF + DH] + log2f(mrg[(size_t)r * ROWF + DH + 1])) * LN2;
     } else {
-      float* part = p.partial + (((size_t)b * p.H + h) * p.nsplit) * (size_t)(NQ * ROWF);
+      float* part = p.partial + (((size_t)blockIdx.z * p.H + h) * p.nsplit) * (size_t)(NQ * ROWF);
       float* mine = part + (size_t)split * (NQ * ROWF);
       for (int idx = ct; idx < nq * ROWF; idx += nct) __stcg(mine + idx, mrg[idx]);
       __threadfence();
       compute_bar(NW * 32);
-      if (ct == 0) ticket_s = atomicAdd(&p.counters[b * p.H + h], 1u);
+      if (ct == 0) ticket_s = atomicAdd(&p.counters[blockIdx.z * p.H + h], 1u);
       compute_bar(NW * 32);
       if (ticket_s == (unsigned)p.nsplit - 1) {
         __threadfence();
@@ -427,7 +442,7 @@ __global__ void __launch_bounds__((WQ * WK + 1) * 32) tree_attn_bf16_kernel(cons
           uint2 packed = make_uint2(pack_bf16(acc.x, acc.y), pack_bf16(acc.z, acc.w));
           *reinterpret_cast<uint2*>(p.out + ((qrow + r) * p.H + h) * DH + c4 * 4) = packed;
         }
-        if (ct == 0) p.counters[b * p.H + h] = 0u;       // ready for the next launch
+        if (ct == 0) p.counters[blockIdx.z * p.H + h] = 0u;       // ready for the next launch
       }
     }
   }
@@ -541,10 +556,12 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tree_attn_tc_kernel(const __gri
   const uint32_t k_ring = q_base + TC_Q_BYTES;
   const uint32_t v_ring = k_ring + SK * TC_KV_BYTES;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int split = blockIdx.x, h = blockIdx.y, b = blockIdx.z;
-  const int L = p.len[b];
-  const int nq_all = p.n_active ? min(p.n_active[b], p.n) : p.n;      // live nodes of this sequence
-  const size_t qrow = p.row_off ? (size_t)p.row_off[b] : (size_t)b * p.n;   // this sequence's first row of q and out
+  const int split = blockIdx.x, h = blockIdx.y;
+  int b, shift;
+  locate_window(p, b, shift);
+  const int L_old = p.len[b], L = L_old + shift;                      // keys written by earlier launches; keys every row sees
+  const int nq_all = (p.n_active ? min(p.n_active[b], p.n) : p.n) - shift;   // live nodes of this sequence (from the window on)
+  const size_t qrow = (p.row_off ? (size_t)p.row_off[b] : (size_t)b * p.n) + shift;   // its first row of q and out
   const int nq = min(nq_all - p.row0, p.rows);                        // live query rows of this launch
   if (nq <= 0) return;
   const int kv_total = L + min(nq_all, p.row0 + p.rows);
@@ -603,7 +620,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tree_attn_tc_kernel(const __gri
     __syncwarp();
     // tiles of the first ring that lie wholly inside the prefix may be fetched before the wait
     int early = 0;
-    while (early < T && early < SK && (t0 + early + 1) * TILE <= L) ++early;
+    while (early < T && early < SK && (t0 + early + 1) * TILE <= L_old) ++early;
     if constexpr (!UNI) {
       // A tile is 16 boxes of 2 KB (K and V, four pages, two 64-wide halves).  With separate K and V rings
       // (128 query rows) 16 lanes issue one box each: 4-7 % faster than one lane issuing them in turn
@@ -923,12 +940,12 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tree_attn_tc_kernel(const __gri
         for (int r = ct; r < nq; r += nct)
           p.lse[((size_t)b * p.H + h) * p.n + r] = (mrg[(size_t)r * ROWF + DH] + log2f(mrg[(size_t)r * ROWF + DH + 1])) * LN2;
     } else {
-      float* part = p.partial + (((size_t)b * p.H + h) * p.nsplit) * (size_t)(RP * ROWF);
+      float* part = p.partial + (((size_t)blockIdx.z * p.H + h) * p.nsplit) * (size_t)(RP * ROWF);
       float* mine = part + (size_t)split * (RP * ROWF);
       for (int idx = ct; idx < nq * ROWF; idx += nct) __stcg(mine + idx, mrg[idx]);
       __threadfence();
       compute_bar(256);
-      if (ct == 0) ticket_s = atomicAdd(&p.counters[b * p.H + h], 1u);
+      if (ct == 0) ticket_s = atomicAdd(&p.counters[blockIdx.z * p.H + h], 1u);
       compute_bar(256);
       if (ticket_s == (unsigned)p.nsplit - 1) {
         __threadfence();
@@ -961,7 +978,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tree_attn_tc_kernel(const __gri
           *reinterpret_cast<uint2*>(p.out + ((qrow + r) * p.H + h) * DH + c4 * 4) =
               make_uint2(pack_bf16(acc.x, acc.y), pack_bf16(acc.z, acc.w));
         }
-        if (ct == 0) p.counters[b * p.H + h] = 0u;          // ready for the next launch
+        if (ct == 0) p.counters[blockIdx.z * p.H + h] = 0u;          // ready for the next launch
       }
     }
   }
@@ -1028,19 +1045,21 @@ __global__ void __launch_bounds__(128) tree_attn_f32_kernel(const float* __restr
                                                             const int32_t* __restrict__ n_active,
                                                             const uint64_t* __restrict__ anc, float* __restrict__ out,
                                                             float* __restrict__ lse, int n, int H, int max_pages,
-                                                            float scale, const int32_t* __restrict__ row_off) {
+                                                            float scale, const int32_t* __restrict__ row_off, int win) {
   constexpr int E = DH / 32;
   __shared__ float s_o[4][DH];
   __shared__ float s_m[4], s_l[4];
   griddep_wait();
   griddep_launch();
-  const int i = blockIdx.x, h = blockIdx.y, b = blockIdx.z;
-  const int nq = n_active ? min(n_active[b], n) : n;
+  // (windows of 128 rows of a prefill chunk: see locate_window)
+  const int i = blockIdx.x, h = blockIdx.y, b = blockIdx.z / win, shift = (blockIdx.z % win) * kAttnRowsPerLaunch;
+  const int nq_all = (n_active ? min(n_active[b], n) : n) - shift;
+  const int nq = win > 1 ? min(nq_all, kAttnRowsPerLaunch) : nq_all;
   if (i >= nq) return;
-  const int L = len[b], warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int L = len[b] + shift, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint64_t a0 = anc[i * CERB_ANC_WORDS], a1 = anc[i * CERB_ANC_WORDS + 1], a2 = anc[i * CERB_ANC_WORDS + 2];
   float qv[E], acc[E];
-  const size_t qrow = row_off ? (size_t)row_off[b] : (size_t)b * n;
+  const size_t qrow = (row_off ? (size_t)row_off[b] : (size_t)b * n) + shift;
   const float* qp = q + ((qrow + i) * H + h) * DH;
   for (int e = 0; e < E; ++e) { qv[e] = qp[lane + 32 * e]; acc[e] = 0.f; }
   float m = -INFINITY, l = 0.f;
@@ -1118,12 +1137,14 @@ size_t attn_scratch_bytes(int B, int n, int H, int Dh) {
   return kCounterBytes + rows * (size_t)nq_pad(n) * (size_t)(Dh + 4) * sizeof(float);
 }
 
-constexpr int kAttnRowsPerLaunch = 128;
-
 // One launch of the bf16 kernels over query rows row0 .. row0 + rows - 1 (rows <= 128) of every sequence's tree.
+// win > 1: `rows` is 128 and the launch covers that many windows of a prefill chunk per sequence side by side.
 static int launch_attn_window(const cerb_attn_args* a, int row0, int rows, const CUtensorMap* tmK, const CUtensorMap* tmV,
-                              int32_t* status, cudaStream_t st, const int32_t* row_off) {
+                              int32_t* status, cudaStream_t st, const int32_t* row_off, int win = 1) {
   AttnParams p;
+  const int Bw = a->B * win;             // (sequence, window) pairs
+  p.B = a->B;
+  p.win = win;
   const size_t row_elems = (size_t)a->n_heads * a->head_dim;
   p.q = (const bf16*)a->q + (size_t)row0 * row_elems;
   p.page_table = a->page_table;
@@ -1156,7 +1177,7 @@ static int launch_attn_window(const cerb_attn_args* a, int row0, int rows, const
   // CTAs that fit at once: one per SM for the tensor-core kernel and for the warp-MMA layouts of 32 rows and more
   // (288 threads x 168 registers), two per SM for the 16-row layout (160 threads); the grid is planned to fit one wave
   const int resident = (tensor_path || np_ > 16) ? 148 : kTargetCtas;
-  p.nsplit = plan_nsplit(a->B, a->n_heads, nq_pad(rows), a->max_len, resident, true, use_cluster ? 8 : kMaxSplit);
+  p.nsplit = plan_nsplit(Bw, a->n_heads, nq_pad(rows), a->max_len, resident, true, use_cluster ? 8 : kMaxSplit);
   if (p.nsplit < 1) return CERB_E_SHAPE;
   p.oob_row = a->n_pool_pages * a->n_heads * CERB_PAGE;
   p.scale_log2 = a->scale * 1.4426950408889634f;
@@ -1176,7 +1197,7 @@ static int launch_attn_window(const cerb_attn_args* a, int row0, int rows, const
   const bool kt_path = a->head_dim == 128 && force_tc < 0 && rows <= 64 && (force_kt < 0 ? rows > 16 : force_kt != 0);
   if (kt_path) {
     const int tiles = (a->max_len + KT_TILE - 1) / KT_TILE;
-    int want = 148 / (a->B * a->n_heads);
+    int want = 148 / (Bw * a->n_heads);
     const int max_split = use_cluster ? 8 : kMaxSplit;
     if (want > max_split) want = max_split;
     if (want > tiles) want = tiles;
@@ -1192,7 +1213,7 @@ static int launch_attn_window(const cerb_attn_args* a, int row0, int rows, const
       kt_configured = true;
     }
     auto kern = tree_attn_kt_kernel<2>;
-    const dim3 grid(p.nsplit, p.H, a->B), block(kt_threads(ncb));
+    const dim3 grid(p.nsplit, p.H, Bw), block(kt_threads(ncb));
     if (p.cluster)
       rc = launch_pdl_cluster(kern, grid, block, kt_smem(ncb), st, (unsigned)p.nsplit, *tmK, *tmV, p) == cudaSuccess ? CERB_OK : CERB_E_CUDA;
     else
@@ -1207,44 +1228,52 @@ static int launch_attn_window(const cerb_attn_args* a, int row0, int rows, const
     auto kern = rows <= 64 ? tree_attn_tc_kernel<5, 5, 64, true> : tree_attn_tc_kernel<2, 5, 128, false>;
     const size_t TC_SMEM = rows <= 64 ? tc_smem(5, 5, 64) : tc_smem(2, 5, 128);
     if (p.cluster)
-      rc = launch_pdl_cluster(kern, dim3(p.nsplit, p.H, a->B), dim3(TC_THREADS), TC_SMEM, st, (unsigned)p.nsplit,
+      rc = launch_pdl_cluster(kern, dim3(p.nsplit, p.H, Bw), dim3(TC_THREADS), TC_SMEM, st, (unsigned)p.nsplit,
                               *tmK, *tmV, p) == cudaSuccess ? CERB_OK : CERB_E_CUDA;
     else
-      rc = launch_pdl(kern, dim3(p.nsplit, p.H, a->B), dim3(TC_THREADS), TC_SMEM, st, *tmK, *tmV, p) == cudaSuccess
+      rc = launch_pdl(kern, dim3(p.nsplit, p.H, Bw), dim3(TC_THREADS), TC_SMEM, st, *tmK, *tmV, p) == cudaSuccess
                ? CERB_OK : CERB_E_CUDA;
   } else if (a->head_dim == 128) {
-    if (np == 16) rc = launch_cfg<128, 1, 4, 3>(p, tmK, tmV, a->B, st);
-    else if (np == 32) rc = launch_cfg<128, 2, 4, 3>(p, tmK, tmV, a->B, st);
-    else if (np == 64) rc = launch_cfg<128, 4, 2, 3>(p, tmK, tmV, a->B, st);
-    else rc = launch_cfg<128, 8, 1, 3>(p, tmK, tmV, a->B, st);
+    if (np == 16) rc = launch_cfg<128, 1, 4, 3>(p, tmK, tmV, Bw, st);
+    else if (np == 32) rc = launch_cfg<128, 2, 4, 3>(p, tmK, tmV, Bw, st);
+    else if (np == 64) rc = launch_cfg<128, 4, 2, 3>(p, tmK, tmV, Bw, st);
+    else rc = launch_cfg<128, 8, 1, 3>(p, tmK, tmV, Bw, st);
   } else if (a->head_dim == 64) {
-    if (np == 16) rc = launch_cfg<64, 1, 4, 4>(p, tmK, tmV, a->B, st);
-    else if (np == 32) rc = launch_cfg<64, 2, 4, 4>(p, tmK, tmV, a->B, st);
-    else if (np == 64) rc = launch_cfg<64, 4, 2, 4>(p, tmK, tmV, a->B, st);
-    else rc = launch_cfg<64, 8, 1, 4>(p, tmK, tmV, a->B, st);
+    if (np == 16) rc = launch_cfg<64, 1, 4, 4>(p, tmK, tmV, Bw, st);
+    else if (np == 32) rc = launch_cfg<64, 2, 4, 4>(p, tmK, tmV, Bw, st);
+    else if (np == 64) rc = launch_cfg<64, 4, 2, 4>(p, tmK, tmV, Bw, st);
+    else rc = launch_cfg<64, 8, 1, 4>(p, tmK, tmV, Bw, st);
   }
   return rc;
 }
 
 int launch_tree_attention(cerb_ctx* c, const cerb_attn_args* a, const CUtensorMap* tmK, const CUtensorMap* tmV,
-                          int sm_count, int32_t* status, cudaStream_t st, const int32_t* row_off) {
+                          int sm_count, int32_t* status, cudaStream_t st, const int32_t* row_off, bool chain) {
   (void)sm_count;
+  const int win = chain ? (a->n + kAttnRowsPerLaunch - 1) / kAttnRowsPerLaunch : 1;
   if (a->dtype == CERB_F32) {
-    dim3 grid(a->n, a->n_heads, a->B);
+    dim3 grid(win > 1 ? kAttnRowsPerLaunch : a->n, a->n_heads, a->B * win);
     if (a->head_dim == 64)
       tree_attn_f32_kernel<64><<<grid, 128, 0, st>>>((const float*)a->q, (const float*)a->k_pool, (const float*)a->v_pool,
                                                      a->page_table, a->len, a->n_active, a->anc, (float*)a->out, a->lse,
-                                                     a->n, a->n_heads, a->max_pages, a->scale, row_off);
+                                                     a->n, a->n_heads, a->max_pages, a->scale, row_off, win);
     else if (a->head_dim == 128)
       tree_attn_f32_kernel<128><<<grid, 128, 0, st>>>((const float*)a->q, (const float*)a->k_pool, (const float*)a->v_pool,
                                                       a->page_table, a->len, a->n_active, a->anc, (float*)a->out, a->lse,
-                                                      a->n, a->n_heads, a->max_pages, a->scale, row_off);
+                                                      a->n, a->n_heads, a->max_pages, a->scale, row_off, win);
     else
       return CERB_E_SHAPE;
     CERB_LAUNCH_CHECK(c);
     return CERB_OK;
   }
   if (a->B * a->n_heads > (int)(kCounterBytes / sizeof(unsigned int)) - 4) return CERB_E_SHAPE;   // last 16 bytes: status word
+  if (win > 1) {
+    // a prefill chunk of more than 128 tokens per sequence: its windows are CTAs of one launch
+    if (a->scratch_bytes < attn_scratch_bytes(a->B, kAttnRowsPerLaunch, a->n_heads, a->head_dim)) return CERB_E_NOMEM;
+    CERB_TRY(launch_attn_window(a, 0, kAttnRowsPerLaunch, tmK, tmV, status, st, row_off, win));
+    CERB_LAUNCH_CHECK(c);
+    return CERB_OK;
+  }
   if (a->scratch_bytes < attn_scratch_bytes(a->B, a->n, a->n_heads, a->head_dim)) return CERB_E_NOMEM;
   // A CTA holds at most 128 query rows (the tensor-core MMA's height, eight 16-row warps in the warp-MMA kernel).
   // A wider tree (Sec. 5.1 goes up to 150 candidates + the root) takes one launch per window of 128 rows; the

@@ -101,12 +101,14 @@ __global__ void __launch_bounds__(kt_threads(NCB), 1) tree_attn_kt_kernel(const 
   const uint32_t q_base = p_base + PB * 2 * P_TERM;                       // [half of head_dim][NQ rows][128 B]
   const uint32_t ring = q_base + 2 * QHALF;                          // NU units
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int split = blockIdx.x, h = blockIdx.y, b = blockIdx.z;
+  const int split = blockIdx.x, h = blockIdx.y;
+  int b, shift;
+  locate_window(p, b, shift);
   // Lengths, live node counts, the page table, the tree and the prefix keys are at least two kernels old:
   // everything up to the first use of Q or of this step's tree keys runs before griddep_wait().
-  const int L = p.len[b];
-  const int nq_all = p.n_active ? min(p.n_active[b], p.n) : p.n;      // live nodes of this sequence
-  const size_t qrow = p.row_off ? (size_t)p.row_off[b] : (size_t)b * p.n;   // this sequence's first row of q and out
+  const int L_old = p.len[b], L = L_old + shift;                      // keys written by earlier launches; keys every row sees
+  const int nq_all = (p.n_active ? min(p.n_active[b], p.n) : p.n) - shift;   // live nodes of this sequence (from the window on)
+  const size_t qrow = (p.row_off ? (size_t)p.row_off[b] : (size_t)b * p.n) + shift;   // its first row of q and out
   const int nq = min(nq_all - p.row0, p.rows);                        // live query rows of this launch
   if (nq <= 0) return;                                                // (uniform over a cluster)
   const int n_tree = min(nq_all, p.row0 + p.rows);                    // tree keys these rows can see
@@ -179,7 +181,7 @@ __global__ void __launch_bounds__(kt_threads(NCB), 1) tree_attn_kt_kernel(const 
     asm volatile("bar.sync 3, %0;" ::"r"(32 * NPROD) : "memory");      // the page list is complete
     // units (K and V) of tiles that lie wholly inside the prefix may be fetched before the wait
     int early = 0;
-    while (early < T && 2 * early < NU && (t0 + early + 1) * KT_TILE <= L) ++early;
+    while (early < T && 2 * early < NU && (t0 + early + 1) * KT_TILE <= L_old) ++early;
     const int early_units = min(2 * early, NU);
     static_assert(KT_PAGES == 8, "the lane -> box map below assumes eight pages per tile");
     const int box = pw + NPROD * lane;               // lanes 0 .. BOXES-1
@@ -536,12 +538,12 @@ __global__ void __launch_bounds__(kt_threads(NCB), 1) tree_attn_kt_kernel(const 
         for (int rr = ct; rr < nq; rr += nct)
           p.lse[((size_t)b * p.H + h) * p.n + rr] = (mrg[(size_t)rr * ROWF + DH] + log2f(mrg[(size_t)rr * ROWF + DH + 1])) * LN2;
     } else {
-      float* part = p.partial + (((size_t)b * p.H + h) * p.nsplit) * (size_t)(RP * ROWF);
+      float* part = p.partial + (((size_t)blockIdx.z * p.H + h) * p.nsplit) * (size_t)(RP * ROWF);
       float* mine = part + (size_t)split * (RP * ROWF);
       for (int idx = ct; idx < nq * ROWF; idx += nct) __stcg(mine + idx, mrg[idx]);
       __threadfence();
       asm volatile("bar.sync 2, %0;" ::"r"(nst) : "memory");
-      if (ct == 0) ticket_s = atomicAdd(&p.counters[b * p.H + h], 1u);
+      if (ct == 0) ticket_s = atomicAdd(&p.counters[blockIdx.z * p.H + h], 1u);
       asm volatile("bar.sync 2, %0;" ::"r"(nst) : "memory");
       if (ticket_s == (unsigned)p.nsplit - 1) {
         __threadfence();
@@ -576,7 +578,7 @@ __global__ void __launch_bounds__(kt_threads(NCB), 1) tree_attn_kt_kernel(const 
           *reinterpret_cast<uint2*>(p.out + ((qrow + rr) * p.H + h) * DH + c4 * 4) =
               make_uint2(pack_bf16(acc.x, acc.y), pack_bf16(acc.z, acc.w));
         }
-        if (ct == 0) p.counters[b * p.H + h] = 0u;          // ready for the next launch
+        if (ct == 0) p.counters[blockIdx.z * p.H + h] = 0u;          // ready for the next launch
       }
     }
   }

@@ -90,7 +90,11 @@ inline cudaError_t launch_pdl_cluster(void (*kernel)(KArgs...), dim3 grid, dim3 
 }
 
 constexpr int kPathMax = CERB_MAX_DEPTH + 1;
-constexpr int kPrefillChunkMax = 128;   // prompt tokens per prefill chunk (a chain-shaped tree), whatever max_nodes is
+// Rows of one prefill forward.  A forward streams all the weights whatever its row count, so short chunks pay for the
+// stream again and again: a 2048-token prompt of the 7B shape took 73.7 ms in 128-token chunks (16 weight streams,
+// 0.23 of the tensor peak).  2048 rows are where the GEMMs are tensor-bound; the sequences of a batch share them.
+constexpr int kPrefillRows = 2048;
+constexpr int kPrefillQuantum = 128;    // tokens per sequence and forward come in multiples of this (the attention window)
 constexpr int kGemmRowsPerPass = 256;   // activation rows one tcgen05 pass covers at most (the MMA's N extent; CTA pairs)
 constexpr int kGemmMaxSplit = 16;
 
@@ -124,7 +128,7 @@ struct cerb_ctx {
   cerb_config cfg;
   bool bf16;
   size_t esize;                       // bytes per model element
-  int Mmax;                           // max rows of one forward (max_batch * max_nodes)
+  int Mmax;                           // max rows of one forward (max_batch * max_nodes, or a prefill forward's)
   int max_pos;                        // 16 * max_pages
   int head_w[CERB_MAX_HEADS][CERB_MAX_LEVELS + 1];   // state width entering each level
   int head_wmax;
@@ -146,6 +150,7 @@ struct cerb_ctx {
   int32_t *d_len, *d_len_old, *d_root, *d_nactive, *d_status, *d_lens_in, *d_mode, *d_naccept;
   int32_t *d_path, *d_outtok, *d_argmax, *d_treetok, *d_topk, *d_kper;
   int32_t* d_rowoff;                  // [CERB_MAX_BATCH + 1] first row of every sequence when the rows of a step are ragged
+  int32_t* d_iota;                    // [Mmax] 0, 1, 2, ...: the depths of a prefill chunk
   float* d_S;
   void *d_hlast, *d_x, *d_xn, *d_q, *d_attn, *d_act, *d_hidden;
   float *d_part, *d_logits, *d_hlogits;
@@ -159,7 +164,7 @@ struct cerb_ctx {
   size_t attn_scratch_bytes;
   char* d_tree_store;
   bool tree_used[CERB_MAX_TREES];
-  cerb_tree* chain;                   // chain tree of max_nodes for the prefill
+  cerb_tree* chain;                   // stands for the prompt tokens of a prefill chunk
   cerb_tree* single;                  // one-node tree for auto-regressive steps
 
   // pinned host staging
@@ -215,7 +220,7 @@ int launch_swiglu(cerb_ctx* c, const float* part, int nsplit, size_t split_strid
 int launch_argmax_rows(cerb_ctx* c, const float* part, int nsplit, size_t split_stride, int rows, int V, int32_t* out,
                        float* summed, cudaStream_t st);
 int launch_set_nactive(cerb_ctx* c, int mode, int a, int b, cudaStream_t st);
-int launch_prefill_commit(cerb_ctx* c, int n, cudaStream_t st);
+int launch_prefill_commit(cerb_ctx* c, cudaStream_t st);
 
 // gemm_f32.cu / gemm_bf16.cu : out[split][M][N] fp32 partial sums of X[M][K] . W[N][K]^T
 int launch_gemm_f32(cerb_ctx* c, const float* X, const float* W, float* out, int M, int N, int K, cudaStream_t st);
@@ -252,8 +257,10 @@ int init_driver_api();
 size_t attn_scratch_bytes(int B, int n, int H, int Dh);
 int make_pool_map(CUtensorMap* out, const void* pool, int n_pool_pages, int H, int Dh);
 // row_off: first row of every sequence in q / out when the rows of a batch are ragged (device, [B]); null = b * n
+// chain: the n nodes of every sequence are consecutive prompt tokens (n may then exceed CERB_MAX_NODES; anc describes a
+// chain of 128)
 int launch_tree_attention(cerb_ctx* c, const cerb_attn_args* a, const CUtensorMap* tmK, const CUtensorMap* tmV,
-                          int sm_count, int32_t* status, cudaStream_t st, const int32_t* row_off = nullptr);
+                          int sm_count, int32_t* status, cudaStream_t st, const int32_t* row_off = nullptr, bool chain = false);
 
 // heads.cu
 int launch_heads(cerb_ctx* c, const cerb_tree* tree, int32_t* tree_tok, const int32_t* plant, int32_t* topk_out,

@@ -256,28 +256,41 @@ __global__ void argmax_rows_kernel(const float* __restrict__ part, int nsplit, s
   }
 }
 
-// mode 0: n_active[b] = a.  mode 1 (prefill chunk): n_active[b] = clamp(lens_in[b] - a, 0, b_).
-__global__ void set_nactive_kernel(int32_t* n_active, const int32_t* lens_in, int B, int mode, int a, int b_) {
+// mode 0: n_active[b] = a.  mode 1 (prefill chunk): n_active[b] = clamp(lens_in[b] - a, 0, b_), and row_off[b] = the first
+// of the rows that sequence b owns when only live tokens have rows.
+__global__ void set_nactive_kernel(int32_t* n_active, const int32_t* lens_in, int32_t* row_off, int B, int mode, int a, int b_) {
   griddep_wait();
   griddep_launch();
-  int b = threadIdx.x;
-  if (b >= B) return;
-  if (mode == 0) n_active[b] = a;
-  else {
-    int r = lens_in[b] - a;
-    n_active[b] = r < 0 ? 0 : (r > b_ ? b_ : r);
+  const int b = threadIdx.x;
+  int r = 0;
+  if (b < B) {
+    r = a;
+    if (mode == 1) {
+      r = lens_in[b] - a;
+      r = r < 0 ? 0 : (r > b_ ? b_ : r);
+    }
+    n_active[b] = r;
+  }
+  if (mode == 1) {
+    int sum = r;
+    for (int o = 1; o < 32; o <<= 1) {
+      const int t = __shfl_up_sync(0xffffffffu, sum, o);
+      if (b >= o) sum += t;
+    }
+    if (b <= B) row_off[b] = sum - r;
   }
 }
 
 // After a chain-shaped prefill chunk: everything is accepted in place.
 template <typename T>
 __global__ void prefill_commit_kernel(const int32_t* __restrict__ n_active, int32_t* __restrict__ len,
-                                      const T* __restrict__ hidden, T* __restrict__ h_last, int n, int d) {
+                                      const T* __restrict__ hidden, T* __restrict__ h_last,
+                                      const int32_t* __restrict__ row_off, int d) {
   griddep_wait();
   griddep_launch();
   int b = blockIdx.x, na = n_active[b];
   if (na <= 0) return;
-  const T* src = hidden + ((size_t)b * n + na - 1) * d;
+  const T* src = hidden + ((size_t)row_off[b] + na - 1) * d;
   for (int j = threadIdx.x; j < d; j += blockDim.x) h_last[(size_t)b * d + j] = src[j];
   __syncthreads();
   if (threadIdx.x == 0) len[b] += na;
@@ -343,19 +356,19 @@ int launch_argmax_rows(cerb_ctx* c, const float* part, int nsplit, size_t split_
 }
 
 int launch_set_nactive(cerb_ctx* c, int mode, int a, int b, cudaStream_t st) {
-  set_nactive_kernel<<<1, 32, 0, st>>>(c->d_nactive, c->d_lens_in, c->B, mode, a, b);
+  set_nactive_kernel<<<1, 32, 0, st>>>(c->d_nactive, c->d_lens_in, c->d_rowoff, c->B, mode, a, b);
   CERB_LAUNCH_CHECK(c);
   return CERB_OK;
 }
 
-int launch_prefill_commit(cerb_ctx* c, int n, cudaStream_t st) {
+int launch_prefill_commit(cerb_ctx* c, cudaStream_t st) {
   int d = c->cfg.d_model;
   if (c->bf16)
     prefill_commit_kernel<bf16><<<c->B, 256, 0, st>>>(c->d_nactive, c->d_len, (const bf16*)c->d_hidden,
-                                                      (bf16*)c->d_hlast, n, d);
+                                                      (bf16*)c->d_hlast, (const int32_t*)c->d_rowoff, d);
   else
     prefill_commit_kernel<float><<<c->B, 256, 0, st>>>(c->d_nactive, c->d_len, (const float*)c->d_hidden,
-                                                       (float*)c->d_hlast, n, d);
+                                                       (float*)c->d_hlast, (const int32_t*)c->d_rowoff, d);
   CERB_LAUNCH_CHECK(c);
   return CERB_OK;
 }

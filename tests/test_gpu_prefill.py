@@ -1,0 +1,41 @@
+"""Prefill forwards of many tokens: windows of 128 query rows side by side, packed rows, several forwards per prompt."""
+import pytest
+import torch
+
+from oracle import cerberus_oracle as orc
+from paper_2410_13344_b200 import binding as cb
+from paper_2410_13344_b200 import synth
+from tests.helpers import close
+from tests.test_gpu_model import TOL, Rig
+
+pytestmark = pytest.mark.gpu
+
+SHAPES = {"fp32": synth.tiny_shape("fp32"), "bf16 head_dim 64": synth.tiny_shape("bf16"),
+          "bf16 head_dim 128": synth.ModelShape(2, 256, 2, 128, 512, 1024, "bf16")}
+
+
+# a window edge on both sides; one row and several forwards beside each other (the forward holds 2048 rows: 2049 tokens
+# leave one for the second, and three prompts of unequal length share it); a whole forward of 16 sequences
+@pytest.mark.parametrize("shape", list(SHAPES))
+@pytest.mark.parametrize("lens", [(127, 1, 129), (128, 256, 255), (2049,), (1300, 5, 900), tuple(range(131, 147))],
+                         ids=lambda l: "-".join(map(str, l[:3])))
+def test_prefill_matches_oracle(shape, lens):
+    ms = SHAPES[shape]
+    B = len(lens)
+    rig = Rig(cb, ms, max_batch=B, max_tokens=max(lens) + 16, max_nodes=16)
+    prompts = [[int(t) for t in synth.make_prompt(ms.vocab, n, seq=70 + b)] for b, n in enumerate(lens)]
+    tok = torch.zeros(B, max(lens), dtype=torch.int32, device="cuda")
+    for b, p in enumerate(prompts):
+        tok[b, :len(p)] = torch.tensor(p, dtype=torch.int32)
+    rig.eng.prefill(tok, list(lens))
+    got_len, got_root, h_last = rig.eng.read_state()
+    assert rig.eng.device_status() == 0 and list(got_len) == list(lens)
+    tol = TOL[ms.dtype]                              # the repository's bound for a small model against the oracle
+    for b in {0, B // 2, B - 1}:
+        st = orc.prefill(rig.cmodel, rig.sh, prompts[b], lens[b] + 16)
+        assert close(h_last[b], st.h_last, 0) < tol
+        for l in range(ms.n_layers):
+            k, v = rig.eng.gather_kv(b, l, lens[b])
+            assert close(k, st.k[l][:lens[b]], 0) < tol and close(v, st.v[l][:lens[b]], 0) < tol, (b, l)
+        if ms.dtype == "fp32":
+            assert int(got_root[b]) == st.root
