@@ -336,7 +336,8 @@ int cerb_set_wait_cycles(int64_t cycles);
  * programmatic dependent launch).  Writes one line per launch, "id|name|writes|reads-before-wait", for one set-up
  * launch, three layers and the tail, into buf (host).  variant 0: separate SwiGLU and RoPE kernels; 1: SwiGLU inside the
  * gate-up GEMM (steps of at most 16 rows); 2: RoPE + cache append inside the QKV GEMM as well (such steps at
- * head_dim 128).  Returns CERB_OK when no kernel reads, ahead of its wait, a buffer
+ * head_dim 128).  3..7: the other combinations, with the residual add inside the O and down GEMMs (3, 5, 6, 7), which occur
+ * above 128 rows.  Returns CERB_OK when no kernel reads, ahead of its wait, a buffer
  * that the kernel right in front of it writes, CERB_E_STATE otherwise, CERB_E_NOMEM when buf is too small. */
 int cerb_launch_order_table(int32_t variant, char* buf_host, size_t cap);
 

@@ -153,6 +153,7 @@ size_t carve(cerb_ctx* c, char* base) {
   c->d_attn = b.take<char>((size_t)Mr * HD * es);
   c->d_act = b.take<char>((size_t)Mr * g.mlp_dim * es);
   c->d_part = b.take<float>(c->part_floats);
+  c->d_gemm_fix = b.take<float>(c->bf16 && c->Mmax > 128 ? gemm_fix_floats() : 0);
   int Hc = g.n_cheads > 0 ? g.n_cheads : 1;
   c->d_hstate[0] = b.take<float>((size_t)MB * Hc * c->head_wmax);
   c->d_hstate[1] = b.take<float>((size_t)MB * Hc * c->head_wmax);
@@ -232,13 +233,17 @@ unsigned long long* gemm_clock_slot(cerb_ctx* c) {
   return c->d_gemm_clock + c->gemm_clock_used++;
 }
 
-// out = X . W^T as fp32 split partials in d_part; returns the split count.
+// X . W^T as fp32 split partials in d_part; returns the split count.  A caller that knows there is one slot (more than 128
+// rows) may have it elsewhere (out).
 int gemm(cerb_ctx* c, const void* X, const ActMaps* xm, const void* W, const CUtensorMap* wm, int M, int N, int K,
-         int* nsplit, cudaStream_t st) {
+         int* nsplit, cudaStream_t st, float* out = nullptr) {
   if (c->bf16) {
     int ns = gemm_plan_split(c->sm_count, M, N, K);
     if ((size_t)ns * M * N > c->part_floats) return CERB_E_NOMEM;
     *nsplit = ns;
+    if (M > 128)
+      return launch_gemm_tile(c, wm, xm, make_tile_plan(M, N, K), out ? out : c->d_part, c->d_gemm_fix, c->d_gemm_tickets, M, N, c->d_status, st,
+                              nullptr, gemm_clock_slot(c));
     return launch_gemm_bf16(c, wm, xm, c->d_part, M, N, K, ns, c->d_status, st, nullptr, gemm_clock_slot(c));
   }
   if ((size_t)M * N > c->part_floats) return CERB_E_NOMEM;
@@ -246,12 +251,19 @@ int gemm(cerb_ctx* c, const void* X, const ActMaps* xm, const void* W, const CUt
   return launch_gemm_f32(c, (const float*)X, (const float*)W, c->d_part, M, N, K, st);
 }
 
+// The same for a GEMM of more than 128 rows that ends in a fused epilogue.
+int gemm_fused(cerb_ctx* c, const ActMaps* xm, const CUtensorMap* wm, int M, int N, int K, const GemmEpilogue& epi, cudaStream_t st) {
+  ProfScope ps(c, K_GEMM, st);
+  return launch_gemm_tile(c, wm, xm, make_tile_plan(M, N, K), nullptr, c->d_gemm_fix, c->d_gemm_tickets, M, N, c->d_status, st, &epi,
+                          gemm_clock_slot(c));
+}
+
 // Steps through the layer sequence of launch_order.cu while forward_rows launches: a kernel announced out of
 // turn means the table of pre-wait reads no longer describes the code.
 struct OrderCheck {
-  const int* ids;
+  int ids[kLayerLaunches];
   int n, pos;
-  explicit OrderCheck(int variant) : pos(0) { n = launch_order_layer(variant, &ids); }
+  explicit OrderCheck(int variant) : pos(0) { n = launch_order_layer(variant, ids); }
   bool next(int id) {
     if (id == LO_NORM_FINAL) return pos == 0;
     const bool ok = ids[pos] == id;
@@ -293,9 +305,12 @@ int forward_rows(cerb_ctx* c, const cerb_tree* tree, const int32_t* tok, int tok
   }
   // Steps of up to 16 rows: SwiGLU runs in the gate-up GEMM's epilogue and (head_dim 128) RoPE + cache append in the
   // QKV GEMM's.
-  const bool fuse_swiglu = c->bf16 && gemm_swiglu_fusable(M, F);
-  const bool fuse_rope = fuse_swiglu && gemm_rope_fusable(M, g.head_dim);
-  OrderCheck oc(fuse_rope ? 2 : fuse_swiglu ? 1 : 0);
+  // More than 128 rows: so does whatever follows a GEMM whose plan has whole tiles, the residual adds included.
+  const bool wide = c->bf16 && M > 128;
+  const bool fuse_swiglu = wide ? F % 16 == 0 && make_tile_plan(M, 2 * F, d).whole : c->bf16 && gemm_swiglu_fusable(M, F);
+  const bool fuse_rope = wide ? g.head_dim == 128 && make_tile_plan(M, 3 * HD, d).whole : fuse_swiglu && gemm_rope_fusable(M, g.head_dim);
+  const bool fuse_res = wide && make_tile_plan(M, d, HD).whole;        // (the down GEMM has the same tiles)
+  OrderCheck oc(launch_order_variant({fuse_swiglu, fuse_rope, fuse_res}));
   // embedding gather fused with the first layer's attention norm
   CERB_ORDER(oc, LO_NORM_ATTN);
   { ProfScope ps(c, K_GLUE, st);
@@ -313,13 +328,16 @@ int forward_rows(cerb_ctx* c, const cerb_tree* tree, const int32_t* tok, int tok
     CERB_ORDER(oc, LO_GEMM_QKV);
     if (fuse_rope) {
       // q, k and v leave the GEMM rotated and in place: no separate kernel, no second pass over the partial sums
-      ProfScope ps(c, K_GEMM, st);
-      const int nsl = gemm_plan_split(c->sm_count, M, 3 * HD, d);
-      if ((size_t)nsl * M * 3 * HD > c->part_floats) return CERB_E_NOMEM;
       const RopeEpilogue re{c->d_len, c->d_nactive, tree->dev.depth, c->page_table, row_off, c->d_rope, c->d_q,
                             (void*)a.k_pool, (void*)a.v_pool, g.max_pages, c->max_pos, n, g.n_heads, B};
-      const GemmEpilogue epi{2, nullptr, c->d_gemm_tickets, &re};
-      CERB_TRY(launch_gemm_bf16(c, &c->tm_wqkv[l], &c->tm_xn, c->d_part, M, 3 * HD, d, nsl, c->d_status, st, &epi, gemm_clock_slot(c)));
+      const GemmEpilogue epi{2, nullptr, c->d_gemm_tickets, &re, nullptr};
+      if (wide) CERB_TRY(gemm_fused(c, &c->tm_xn, &c->tm_wqkv_rot[l], M, 3 * HD, d, epi, st));
+      else {
+        ProfScope ps(c, K_GEMM, st);
+        const int nsl = gemm_plan_split(c->sm_count, M, 3 * HD, d);
+        if ((size_t)nsl * M * 3 * HD > c->part_floats) return CERB_E_NOMEM;
+        CERB_TRY(launch_gemm_bf16(c, &c->tm_wqkv[l], &c->tm_xn, c->d_part, M, 3 * HD, d, nsl, c->d_status, st, &epi, gemm_clock_slot(c)));
+      }
     } else {
       { ProfScope ps(c, K_GEMM, st);
         CERB_TRY(gemm(c, c->d_xn, &c->tm_xn, c->wqkv[l], c->bf16 ? &c->tm_wqkv[l] : nullptr, M, 3 * HD, d, &ns, st)); }
@@ -331,20 +349,26 @@ int forward_rows(cerb_ctx* c, const cerb_tree* tree, const int32_t* tok, int tok
       CERB_TRY(launch_tree_attention(c, &a, c->bf16 ? &c->tm_kpool[l] : nullptr, c->bf16 ? &c->tm_vpool[l] : nullptr,
                                      c->sm_count, c->d_status, st, row_off, tree == c->chain)); }
     CERB_ORDER(oc, LO_GEMM_WO);
-    { ProfScope ps(c, K_GEMM, st);
+    const GemmEpilogue res{3, nullptr, c->d_gemm_tickets, nullptr, (float*)c->d_x};
+    if (fuse_res) CERB_TRY(gemm_fused(c, &c->tm_attn, &c->tm_wo[l], M, d, HD, res, st));
+    else { ProfScope ps(c, K_GEMM, st);
       CERB_TRY(gemm(c, c->d_attn, &c->tm_attn, c->wo[l], c->bf16 ? &c->tm_wo[l] : nullptr, M, d, HD, &ns, st)); }
+    if (fuse_res) ns = 0;
     // residual add fused with the MLP norm
     CERB_ORDER(oc, LO_NORM_MLP);
     { ProfScope ps(c, K_GLUE, st);
-      CERB_TRY(launch_fused_norm(c, c->d_part, ns, (size_t)M * d, nullptr, 0, 0, n, c->mlp_norm[l], c->d_xn, M, st)); }
+      CERB_TRY(launch_fused_norm(c, c->d_part, ns, (size_t)M * d, nullptr, 0, 0, n, c->mlp_norm[l], c->d_xn, M, st, nullptr, fuse_res)); }
     CERB_ORDER(oc, LO_GEMM_GU);
     if (fuse_swiglu) {
       // SwiGLU runs in the GEMM's epilogue: no separate kernel, no second pass over the partial sums
-      ProfScope ps(c, K_GEMM, st);
-      const int nsl = gemm_plan_split(c->sm_count, M, 2 * F, d);
-      if ((size_t)nsl * M * 2 * F > c->part_floats) return CERB_E_NOMEM;
-      const GemmEpilogue epi{1, c->d_act, c->d_gemm_tickets};
-      CERB_TRY(launch_gemm_bf16(c, &c->tm_wgu[l], &c->tm_xn, c->d_part, M, 2 * F, d, nsl, c->d_status, st, &epi, gemm_clock_slot(c)));
+      const GemmEpilogue epi{1, c->d_act, c->d_gemm_tickets, nullptr, nullptr};
+      if (wide) CERB_TRY(gemm_fused(c, &c->tm_xn, &c->tm_wgu_pair[l], M, 2 * F, d, epi, st));
+      else {
+        ProfScope ps(c, K_GEMM, st);
+        const int nsl = gemm_plan_split(c->sm_count, M, 2 * F, d);
+        if ((size_t)nsl * M * 2 * F > c->part_floats) return CERB_E_NOMEM;
+        CERB_TRY(launch_gemm_bf16(c, &c->tm_wgu[l], &c->tm_xn, c->d_part, M, 2 * F, d, nsl, c->d_status, st, &epi, gemm_clock_slot(c)));
+      }
     } else {
       { ProfScope ps(c, K_GEMM, st);
         CERB_TRY(gemm(c, c->d_xn, &c->tm_xn, c->wgu[l], c->bf16 ? &c->tm_wgu[l] : nullptr, M, 2 * F, d, &ns, st)); }
@@ -352,14 +376,16 @@ int forward_rows(cerb_ctx* c, const cerb_tree* tree, const int32_t* tok, int tok
       { ProfScope ps(c, K_GLUE, st); CERB_TRY(launch_swiglu(c, c->d_part, ns, (size_t)M * 2 * F, c->d_act, M, st)); }
     }
     CERB_ORDER(oc, LO_GEMM_DOWN);
-    { ProfScope ps(c, K_GEMM, st);
+    if (fuse_res) CERB_TRY(gemm_fused(c, &c->tm_act, &c->tm_wd[l], M, d, F, res, st));
+    else { ProfScope ps(c, K_GEMM, st);
       CERB_TRY(gemm(c, c->d_act, &c->tm_act, c->wd[l], c->bf16 ? &c->tm_wd[l] : nullptr, M, d, F, &ns, st)); }
+    if (fuse_res) ns = 0;
     // residual add fused with the next layer's attention norm, or with the final norm
     CERB_ORDER(oc, l + 1 == g.n_layers ? LO_NORM_FINAL : LO_NORM_ATTN);
     { ProfScope ps(c, K_GLUE, st);
       const bool last = l + 1 == g.n_layers;
       CERB_TRY(launch_fused_norm(c, c->d_part, ns, (size_t)M * d, nullptr, 0, 0, n, last ? c->final_norm : c->attn_norm[l + 1],
-                                 last ? c->d_hidden : c->d_xn, M, st)); }
+                                 last ? c->d_hidden : c->d_xn, M, st, nullptr, fuse_res)); }
   }
   return CERB_OK;
 }
@@ -368,10 +394,14 @@ int forward_rows(cerb_ctx* c, const cerb_tree* tree, const int32_t* tok, int tok
 int lm_head_argmax(cerb_ctx* c, const void* X, const ActMaps* xm, int rows, int32_t* argmax_out, float* logits_out,
                    cudaStream_t st) {
   int ns = 1;
+  // one slot: the GEMM writes the caller's logits itself, and the argmax reads them there
+  const bool direct = logits_out && c->bf16 && rows > 128 && gemm_plan_split(c->sm_count, rows, c->cfg.vocab, c->cfg.d_model) == 1;
   { ProfScope ps(c, K_GEMM, st);
-    CERB_TRY(gemm(c, X, xm, c->lm_head, c->bf16 ? &c->tm_lm_head : nullptr, rows, c->cfg.vocab, c->cfg.d_model, &ns, st)); }
+    CERB_TRY(gemm(c, X, xm, c->lm_head, c->bf16 ? &c->tm_lm_head : nullptr, rows, c->cfg.vocab, c->cfg.d_model, &ns, st,
+                  direct ? logits_out : nullptr)); }
   ProfScope ps(c, K_GLUE, st);
-  return launch_argmax_rows(c, c->d_part, ns, (size_t)rows * c->cfg.vocab, rows, c->cfg.vocab, argmax_out, logits_out, st);
+  return launch_argmax_rows(c, direct ? logits_out : c->d_part, ns, (size_t)rows * c->cfg.vocab, rows, c->cfg.vocab, argmax_out,
+                            direct ? nullptr : logits_out, st);
 }
 
 int set_active(cerb_ctx* c, const int32_t* n_active_dev, int n, cudaStream_t st) {
@@ -482,12 +512,15 @@ int cerb_load(const cerb_config* cfg, const cerb_weights* w, void* workspace_dev
     if (c->bf16) {
       const int Mr = round_up(c->Mmax, 256);
       c->tm_wqkv.resize(L); c->tm_wo.resize(L); c->tm_wgu.resize(L); c->tm_wd.resize(L);
+      c->tm_wqkv_rot.resize(L); c->tm_wgu_pair.resize(L);
       c->tm_kpool.resize(L); c->tm_vpool.resize(L);
       for (int l = 0; l < L && rc == CERB_OK; ++l) {
         if ((rc = make_weight_map(&c->tm_wqkv[l], c->wqkv[l], 3 * HD, g.d_model)) != CERB_OK) break;
         if ((rc = make_weight_map(&c->tm_wo[l], c->wo[l], g.d_model, HD)) != CERB_OK) break;
         if ((rc = make_weight_map(&c->tm_wgu[l], c->wgu[l], 2 * g.mlp_dim, g.d_model)) != CERB_OK) break;
         if ((rc = make_weight_map(&c->tm_wd[l], c->wd[l], g.d_model, g.mlp_dim)) != CERB_OK) break;
+        if (g.head_dim == 128 && (rc = make_rotation_map(&c->tm_wqkv_rot[l], c->wqkv[l], 3 * g.n_heads, g.d_model)) != CERB_OK) break;
+        if (g.mlp_dim % 16 == 0 && (rc = make_gate_up_map(&c->tm_wgu_pair[l], c->wgu[l], g.mlp_dim, g.d_model)) != CERB_OK) break;
         if ((rc = make_pool_map(&c->tm_kpool[l], c->k_pool + (size_t)l * c->pool_layer_bytes, g.n_pool_pages, g.n_heads, g.head_dim)) != CERB_OK) break;
         if ((rc = make_pool_map(&c->tm_vpool[l], c->v_pool + (size_t)l * c->pool_layer_bytes, g.n_pool_pages, g.n_heads, g.head_dim)) != CERB_OK) break;
       }
@@ -729,7 +762,7 @@ int cerb_tree_attention(const cerb_attn_args* a, void* stream) {
 
 int cerb_gemm_scratch_bytes(int32_t M, int32_t N, int32_t K, size_t* bytes_out) {
   if (!bytes_out || M < 1 || N < 1 || K < 1) return CERB_E_ARG;
-  *bytes_out = 256 + (size_t)gemm_plan_split(148, M, N, K) * M * N * sizeof(float);
+  *bytes_out = 256 + (size_t)gemm_scratch_slots(M, N, K) * M * N * sizeof(float);
   return CERB_OK;
 }
 
@@ -754,15 +787,29 @@ int cerb_gemm(int32_t dtype, const void* X_dev, const void* W_dev, float* out_de
   size_t need;
   CERB_TRY(cerb_gemm_scratch_bytes(M, N, K, &need));
   if (!scratch_dev || scratch_bytes < need || ((uintptr_t)scratch_dev & 255)) return CERB_E_NOMEM;
-  int ns = gemm_plan_split(148, M, N, K);
   CUtensorMap tw;
   ActMaps tx;
   CERB_TRY(make_weight_map(&tw, W_dev, N, K));
-  CERB_TRY(make_act_maps(&tx, X_dev, M, K));
   int32_t* status = reinterpret_cast<int32_t*>(scratch_dev);
   float* part = reinterpret_cast<float*>((char*)scratch_dev + 256);
   CERB_CUDA_OK(cudaMemsetAsync(status, 0, 4, st));
-  CERB_TRY(launch_gemm_bf16(nullptr, &tw, &tx, part, M, N, K, ns, status, st));
+  int ns;
+  if (M > 128) {
+    // behind the status word: the fix-up buffer and, after it, its tickets (one slot, which goes straight to the output),
+    // or the partial slots
+    const size_t room = (need - 256) / sizeof(float);
+    const TilePlan g = make_tile_plan(M, N, K, gemm_scratch_slots(M, N, K), room > kGemmTickets ? room - kGemmTickets : 0);
+    ns = g.nslots;
+    unsigned int* tickets = reinterpret_cast<unsigned int*>(part + g.fix_floats);
+    if (g.fix_floats) CERB_CUDA_OK(cudaMemsetAsync(tickets, 0, kGemmTickets * sizeof(unsigned int), st));
+    CERB_TRY(make_act_map(&tx, X_dev, M, K, g.n_act / 2));
+    CERB_TRY(launch_gemm_tile(nullptr, &tw, &tx, g, ns == 1 ? out_dev : part, part, tickets, M, N, status, st));
+    if (ns == 1) return CERB_OK;
+  } else {
+    ns = gemm_plan_split(148, M, N, K);
+    CERB_TRY(make_act_map(&tx, X_dev, M, K, row_bucket(M)));
+    CERB_TRY(launch_gemm_bf16(nullptr, &tw, &tx, part, M, N, K, ns, status, st));
+  }
   size_t total = (size_t)M * N;
   sum_splits_kernel<<<(unsigned)((total + 255) / 256), 256, 0, st>>>(part, ns, total, out_dev, total);
   if (cudaGetLastError() != cudaSuccess) return CERB_E_CUDA;

@@ -108,10 +108,10 @@ struct TreeDev {
 };
 constexpr size_t kTreeSlotBytes = 4 * CERB_MAX_NODES * sizeof(int32_t) + CERB_MAX_NODES * CERB_ANC_WORDS * sizeof(uint64_t);
 
-// Tensor maps for one activation buffer used as the MMA's B operand, one per row bucket.
-constexpr int kRowBuckets = 5;          // 16, 32, 64, 128, 256 rows
+// Tensor maps for one activation buffer used as the MMA's B operand, one per number of rows fetched at a time.
 struct ActMaps {
-  CUtensorMap m[kRowBuckets];
+  CUtensorMap m[8];                     // boxes of 16, 32, ... 128 rows
+  const CUtensorMap& box(int rows) const { return m[rows / 16 - 1]; }
 };
 
 }  // namespace cerb
@@ -142,6 +142,7 @@ struct cerb_ctx {
 
   // tensor maps (bf16 only)
   std::vector<CUtensorMap> tm_wqkv, tm_wo, tm_wgu, tm_wd;
+  std::vector<CUtensorMap> tm_wqkv_rot, tm_wgu_pair;   // the same rows gathered for the epilogues above 128 rows
   CUtensorMap tm_lm_head;
   cerb::ActMaps tm_xn, tm_attn, tm_act, tm_hidden, tm_hlast;
   std::vector<CUtensorMap> tm_kpool, tm_vpool;        // per layer
@@ -157,6 +158,7 @@ struct cerb_ctx {
   float* d_topk_cv;       // per-chunk top-k candidates of the heads' logits: values [B][Hc][kTopkChunks][MAX_TOPK]
   int32_t* d_topk_ci;     // ... and their token ids
   unsigned int* d_gemm_tickets;   // kGemmTickets arrival counters of the GEMM's fused epilogue (zero between launches)
+  float* d_gemm_fix;      // partial tiles of the GEMM above 128 rows
   size_t part_floats;
   float* d_hstate[2];
   float2* d_rope;
@@ -190,12 +192,12 @@ struct cerb_ctx {
 
 namespace cerb {
 
+// Rows of one pass of the single-CTA GEMM: 16, 32, 64 or 128.
 inline int row_bucket(int rows) {
-  int b = 0, r = 16;
-  while (r < rows && b < kRowBuckets - 1) { r <<= 1; ++b; }
-  return b;
+  int r = 16;
+  while (r < rows && r < 128) r <<= 1;
+  return r;
 }
-inline int bucket_rows(int b) { return 16 << b; }
 constexpr int kGemmTickets = 4096;
 constexpr int kGemmClockSlots = 4096;
 constexpr int kTopkChunks = 16;     // the vocabulary is cut into this many chunks for the heads' top-k
@@ -203,8 +205,14 @@ constexpr int kTopkChunks = 16;     // the vocabulary is cut into this many chun
 // launch_order.cu: the forward's launch sequence and what each kernel reads ahead of its dependency wait
 enum { LO_SET_ACTIVE = 0, LO_NORM_ATTN, LO_GEMM_QKV, LO_ROPE, LO_ATTN, LO_GEMM_WO, LO_NORM_MLP, LO_GEMM_GU, LO_SWIGLU,
        LO_GEMM_DOWN, LO_NORM_FINAL, LO_GEMM_LM, LO_ARGMAX };
-int launch_order_layer(int variant, const int** ids_out);     // variant 0: separate SwiGLU and RoPE kernels, 1: SwiGLU fused
-                                                               // into the gate-up GEMM, 2: RoPE + append fused into the QKV GEMM too
+// What runs in GEMM epilogues: SwiGLU in the gate-up GEMM, RoPE + cache append in the QKV GEMM, the residual add in the O
+// and down GEMMs.
+struct Fusion {
+  bool swiglu, rope, residual;
+};
+int launch_order_variant(Fusion f);
+int launch_order_layer(int variant, int* ids_out);            // the layer's launches (at most kLayerLaunches)
+constexpr int kLayerLaunches = 9;
 int launch_order_violations(int variant);
 
 // ---- launch wrappers implemented across the .cu files (all asynchronous on `st`) ----
@@ -213,7 +221,7 @@ int launch_order_violations(int variant);
 int launch_rope_table(cerb_ctx* c, cudaStream_t st);
 int launch_fused_norm(cerb_ctx* c, const float* part, int nsplit, size_t split_stride, const int32_t* tok, int tok_stride,
                       int tok_off, int n, const void* gain, void* out, int rows, cudaStream_t st,
-                      const int32_t* row_off = nullptr);
+                      const int32_t* row_off = nullptr, bool x_fresh = false);
 int launch_rope_append(cerb_ctx* c, int layer, const TreeDev& t, const float* part, int nsplit, size_t split_stride,
                        int B, int n, int rows, cudaStream_t st, const int32_t* row_off = nullptr);
 int launch_swiglu(cerb_ctx* c, const float* part, int nsplit, size_t split_stride, void* act, int rows, cudaStream_t st);
@@ -231,7 +239,9 @@ int gemm_plan_split(int sm_count, int M, int N, int K);
 // kind 2 (RoPE + cache append): W is the QKV matrix [q rows | k rows | v rows] of a model with head_dim 128; the CTA
 // that completes a 256-row tile (two heads' worth of q, k or v) last sums the tile's slots in index order, rotates q
 // and k at position len + depth and writes q dense and k, v into the paged pools -- what rope_append_kernel does,
-// with the same arithmetic in the same order.  Both pay for steps of up to 16 rows only.
+// with the same arithmetic in the same order.  In the single-CTA kernel both pay for steps of up to 16 rows only; above 128
+// rows (gemm_tile.cu) they run wherever the plan has whole tiles.
+// kind 3 (gemm_tile.cu only): the product is added to the fp32 residual stream.
 struct RopeEpilogue {
   const int32_t *len, *n_active, *depth, *page_table, *row_off;    // as for rope_append_kernel (row_off may be null)
   const float2* rope;       // rotation table [max_pos][64]
@@ -239,18 +249,35 @@ struct RopeEpilogue {
   int max_pages, max_pos, n, H, B;
 };
 struct GemmEpilogue {
-  int kind;                 // 0 none, 1 SwiGLU, 2 RoPE + cache append
+  int kind;                 // 0 none, 1 SwiGLU, 2 RoPE + cache append, 3 residual add
   void* act;                // kind 1: [M][F] bf16
   unsigned int* tickets;    // kGemmTickets counters, zero on entry and on exit
   const RopeEpilogue* rope; // kind 2
+  float* x;                 // kind 3: [M][N]
 };
+// gemm_tile.cu: more than 128 rows
+struct TilePlan {
+  int mchunks, n_act, num_kb, pairs, per, sk_tiles, nslots;
+  long long tiles;          // checked to fit 31 bits before launch
+  bool whole;               // at least as many tiles as pairs: one slot, epilogues allowed
+  size_t fix_floats;        // what the plan needs of the fix-up buffer
+};
+TilePlan make_tile_plan(int M, int N, int K, int max_slots = 1 << 30, size_t max_fix = ~(size_t)0);
+size_t gemm_fix_floats();   // of any plan
+int launch_gemm_tile(cerb_ctx* c, const CUtensorMap* tmW, const ActMaps* tmX, const TilePlan& g, float* out, float* fix, unsigned int* tickets,
+                     int M, int N, int32_t* status, cudaStream_t st, const GemmEpilogue* epi = nullptr,
+                     unsigned long long* clock_slot = nullptr);
 bool gemm_swiglu_fusable(int M, int F);
 bool gemm_rope_fusable(int M, int head_dim);
 int launch_gemm_bf16(cerb_ctx* c, const CUtensorMap* tmW, const ActMaps* tmX, float* out, int M, int N, int K,
                      int nsplit, int32_t* status, cudaStream_t st, const GemmEpilogue* epi = nullptr,
                      unsigned long long* clock_slot = nullptr);
 int make_weight_map(CUtensorMap* out, const void* W, int N, int K);
+int make_gate_up_map(CUtensorMap* out, const void* W, int F, int K);
+int make_rotation_map(CUtensorMap* out, const void* W, int heads, int K);
+int make_act_map(ActMaps* out, const void* X, int rows_alloc, int K, int box_rows);
 int make_act_maps(ActMaps* out, const void* X, int rows_alloc, int K);
+int gemm_scratch_slots(int M, int N, int K);
 int init_driver_api();
 
 // attention.cu

@@ -11,11 +11,7 @@
 // that share one activation stage), which halves the activation re-reads through L2; weight tiles
 // carry an evict-first L2 hint, activation tiles evict-last; the accumulator is double-buffered.
 //
-// More than 128 rows (batched trees, prefill chunks of a batch; gemm_bf16_pair_kernel further down):
-// two CTAs of a cluster work as one, 256 rows per pass.  More than 256 rows are cut into row chunks of
-// 256 that are not queued one after the other: the pairs are grouped, one pair per row chunk in a
-// group, and the pairs of a group walk the same weight tiles side by side, so that HBM delivers each
-// weight byte once and the other chunks find it in L2.
+// More than 128 rows: gemm_tile.cu.
 //
 // The kernel is launched programmatically dependent on its predecessor: weights do not depend on
 // the previous kernel, so the producer fills the whole stage ring with weight tiles before it
@@ -59,21 +55,16 @@ struct GemmParams {
   float* out;
   int32_t* status;
   int M, N, K;
-  int n_mma;          // activation rows per pass (16..128, power of two; 256 for CTA pairs)
+  int n_mma;          // activation rows per pass (16..128, power of two)
   int num_kb;         // ceil(K / 64)
   int tiles;          // ceil(N / 128)
   int per;            // work units per CTA
-  int total;          // work units in the list: tiles * num_kb (pairs with lock == 1: row chunks * tiles * num_kb)
-  int lock;           // CTA pairs only.  > 1: this many pairs (one per chunk of 256 rows) walk the same share of the (tile,
-                      // k block) list side by side, so a weight tile is fetched from HBM once and found in L2 by the
-                      // others; 1: row chunks are part of the list
+  int total;          // work units in the list: tiles * num_kb
   int nslots;         // partial slots per output element
   int stages;
   long long wait_cycles;   // budget of every bounded wait, SM clock cycles
   uint32_t idesc;
   uint32_t acc_cols;  // TMEM columns of one accumulator buffer
-  int acc_bufs;       // accumulator buffers in TMEM: 2 (a segment's epilogue overlaps the next segment's MMAs); 1 for CTA
-                      // pairs, whose two 256-column accumulators fill all 512 columns
   int tile_rows;      // weight rows between the starts of consecutive tiles
   int half_off;       // weight-row offset of a wide unit's second tile from its first
   int epi;            // fused epilogue (GemmEpilogue::kind)
@@ -424,261 +415,32 @@ __global__ void __launch_bounds__(224, 1) gemm_bf16_kernel(const __grid_constant
 }
 
 
-// ---------------------------------------------------------------------------------------------------------------
-// More than 128 activation rows: two CTAs of a cluster work as one (tcgen05 cta_group::2).
-//
-// With 256 activation rows per pass a single CTA's stage is half activations (32 KB of weights + 32 KB of
-// activations, three stages), so too few weight bytes are in flight per SM to cover HBM's latency, and the two
-// 256-column accumulators fill tensor memory.  A pair of CTAs shares the activation tile instead: one MMA is
-// 256 weight rows tall, 128 from each CTA's shared memory, and its 256 activation rows come half from each CTA.
-// A unit of the work list is then 512 weight rows x 64 k (two such MMA rows, hf = 0 / 1); per CTA a stage holds
-// 2 x 16 KB of weights + 16 KB of activations (four stages: 128 KB of weights in flight instead of 96), and each CTA's
-// tensor memory holds its 128 rows of both accumulators.  Every CTA fetches its own tiles (no multicast); the
-// byte counts of both CTAs' copies go to the first CTA's "landed" barrier, whose two MMA-issuing threads drive the
-// pair; their commits arrive on the "free" and "accumulator complete" barriers of both CTAs at once.  The work
-// list, the shares, the segments and the partial slots are those of the kernel above, with pairs in the place of
-// CTAs.
-// ---------------------------------------------------------------------------------------------------------------
-constexpr int PAIR_STAGES = 4;
-constexpr int PAIR_TILE = 4 * BM;                       // weight rows of a pair's unit
-constexpr uint32_t PAIR_STAGE_BYTES = 3 * A_STAGE_BYTES;  // per CTA: weights hf 0, weights hf 1, its half of the activations
-constexpr int PAIR_ACT = 2 * BM;                        // activation rows per pass (the MMA's N)
-
-__global__ void __launch_bounds__(224, 1) gemm_bf16_pair_kernel(const __grid_constant__ CUtensorMap tmW,
-                                                                const __grid_constant__ CUtensorMap tmX, const GemmParams p) {
-  extern __shared__ uint8_t smem_raw[];
-  __shared__ __align__(8) uint64_t full_bar[PAIR_STAGES];     // used in the pair's first CTA only
-  __shared__ __align__(8) uint64_t empty_bar[PAIR_STAGES];
-  __shared__ __align__(8) uint64_t acc_full, acc_empty;       // acc_empty: first CTA only, 4 epilogue warps of each CTA arrive
-  __shared__ __align__(8) uint64_t drain_bar[2];
-  __shared__ __align__(8) uint64_t meet_bar;
-  __shared__ uint32_t tmem_base_slot;
-  __shared__ int aborted_s, meet_flag_s;
-  volatile int* aborted = &aborted_s;
-  const WaitCtx wc{p.wait_cycles, aborted, p.status, p.N + 100000 * (p.M > 999 ? 999 : p.M)};
-
-  const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const uint32_t rank = cluster_ctarank();
-  const bool first = rank == 0;
-  const int pair = (int)blockIdx.x >> 1;
-  const int share = pair / p.lock;
-  const int my_chunk = pair % p.lock;
-  const int u0 = share * p.per;
-  const int u1 = (u0 + p.per < p.total) ? u0 + p.per : p.total;
-
-  if (threadIdx.x == 0) {
-    aborted_s = 0;
-    meet_flag_s = 0;
-    for (int s = 0; s < PAIR_STAGES; ++s) {
-      mbar_init(smem_u32(&full_bar[s]), 1);
-      mbar_init(smem_u32(&empty_bar[s]), 2);
-    }
-    mbar_init(smem_u32(&acc_full), 2);
-    mbar_init(smem_u32(&acc_empty), 8);
-    mbar_init(smem_u32(&drain_bar[0]), 1);
-    mbar_init(smem_u32(&drain_bar[1]), 1);
-    mbar_init(smem_u32(&meet_bar), 2);
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-  }
-  if (warp == 1) {
-    // each CTA allocates all 512 columns of its own tensor memory (so both get the same base)
-    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base_slot)), "r"(512u) : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
-  }
-  tc_fence_before();
-  __syncthreads();
-  tc_fence_after();
-  cluster_start_arrive();       // the other CTA's barriers exist before anything is signalled across
-  cluster_start_wait();
-  const uint32_t tmem_base = tmem_base_slot;
-
-  if (warp == 0) {
-    if (lane == 0) {
-      const int n_units = u1 - u0;
-      const uint64_t pol_w = l2_policy(true), pol_x = l2_policy(false);
-      int w_job = u0 / p.num_kb, w_kb = u0 - w_job * p.num_kb;
-      int x_job = w_job, x_kb = w_kb;
-      auto load_w = [&](int i) {
-        const int tile = w_job % p.tiles;
-        const int s = i % PAIR_STAGES;
-        if (first) mbar_expect_tx(smem_u32(&full_bar[s]), 2 * PAIR_STAGE_BYTES);      // both CTAs' copies of this stage
-        const uint32_t fb = mapa_u32(smem_u32(&full_bar[s]), 0);
-        const uint32_t dst = smem_base + (uint32_t)s * PAIR_STAGE_BYTES;
-        const int row = tile * PAIR_TILE + (int)rank * BM;
-        tma_load_2d_pair(dst, &tmW, w_kb * BK, row, fb, pol_w);
-        tma_load_2d_pair(dst + A_STAGE_BYTES, &tmW, w_kb * BK, row + 2 * BM, fb, pol_w);
-        if (++w_kb == p.num_kb) { w_kb = 0; ++w_job; }
-      };
-      auto load_x = [&](int i) {
-        const int mchunk = p.lock > 1 ? my_chunk : x_job / p.tiles;
-        const int s = i % PAIR_STAGES;
-        const uint32_t fb = mapa_u32(smem_u32(&full_bar[s]), 0);
-        tma_load_2d_pair(smem_base + (uint32_t)s * PAIR_STAGE_BYTES + 2 * A_STAGE_BYTES, &tmX, x_kb * BK,
-                         mchunk * PAIR_ACT + (int)rank * BM, fb, pol_x);
-        if (++x_kb == p.num_kb) { x_kb = 0; ++x_job; }
-      };
-      const int pre = n_units < PAIR_STAGES ? n_units : PAIR_STAGES;
-      for (int i = 0; i < pre; ++i) load_w(i);
-      asm volatile("prefetch.tensormap [%0];" ::"l"((uint64_t)&tmX) : "memory");
-      griddep_wait();
-      griddep_launch();
-      if (p.clk) atomicMin(p.clk, globaltimer_ns());
-      for (int i = 0; i < pre; ++i) load_x(i);
-      int issued = pre;
-      for (int i = pre; i < n_units; ++i) {
-        const int s = i % PAIR_STAGES;
-        const uint32_t ph = (uint32_t)(i / PAIR_STAGES) & 1u;
-        if (!mbar_wait_cluster(smem_u32(&empty_bar[s]), ph ^ 1u, wc, 211)) break;
-        load_w(i);
-        load_x(i);
-        issued = i + 1;
-      }
-      if (*aborted) {
-        // give-up path: this CTA's copies land in its own shared memory but are counted on the first CTA's
-        // barriers, and the two CTAs may have stopped at different units, so neither can see exactly its own
-        // copies in.  The first CTA waits for the stages it knows of (short budget); then both let the time of
-        // many memory round trips pass before they go on to the rendezvous and leave.
-        if (first)
-          for (int i = issued > PAIR_STAGES ? issued - PAIR_STAGES : 0; i < issued; ++i)
-            mbar_wait_drain(smem_u32(&full_bar[i % PAIR_STAGES]), (uint32_t)(i / PAIR_STAGES) & 1u, 2000000ll);
-        const long long t_land = clock64();
-        while (clock64() - t_land < 400000ll) __nanosleep(1000);
-      }
-    }
-  } else if (warp == 1 || warp == 6) {
-    // MMA issuers of the pair: the first CTA's warps 1 (hf 0) and 6 (hf 1)
-    const int hf = warp == 6 ? 1 : 0;
-    if (first && lane == 0) {
-      const uint32_t idesc = idesc_bf16(2 * BM, PAIR_ACT, false, false);
-      int u = u0;
-      Segment sg;
-      int i = 0, g = 0;
-      while (next_segment(u, u1, p.num_kb, sg)) {
-        if (!mbar_wait_cluster(smem_u32(&acc_empty), ((uint32_t)g & 1u) ^ 1u, wc, 212)) break;
-        tc_fence_after();
-        const uint32_t d = tmem_base + (uint32_t)(hf * PAIR_ACT);
-        for (int k = 0; k < sg.nkb; ++k, ++i) {
-          const int s = i % PAIR_STAGES;
-          const uint32_t ph = (uint32_t)(i / PAIR_STAGES) & 1u;
-          if (!mbar_wait_cluster(smem_u32(&full_bar[s]), ph, wc, 213)) break;
-          tc_fence_after();
-          const uint32_t src = smem_base + (uint32_t)s * PAIR_STAGE_BYTES;
-          const uint64_t adesc = desc_k_sw128(src + (uint32_t)hf * A_STAGE_BYTES);
-          const uint64_t bdesc = desc_k_sw128(src + 2 * A_STAGE_BYTES);
-#pragma unroll
-          for (int kk = 0; kk < BK / 16; ++kk)
-            umma_bf16_pair(d, adesc + (uint64_t)(kk * 2), bdesc + (uint64_t)(kk * 2), idesc, (k > 0 || kk > 0) ? 1u : 0u);
-          umma_commit_pair(smem_u32(&empty_bar[s]));       // the stage is free in both CTAs once these MMAs have read it
-        }
-        if (*aborted) break;
-        umma_commit_pair(smem_u32(&acc_full));
-        ++g;
-      }
-      if (*aborted) {
-        asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(&drain_bar[hf])) : "memory");
-        mbar_wait_drain(smem_u32(&drain_bar[hf]), 0, 40000000ll);
-      }
-    }
-  } else {
-    const int quarter = warp & 3;                    // TMEM lanes 32*quarter .. +31 belong to this warp
-    griddep_wait();                                  // the kernel before this one may still be reading the partial buffer
-    const uint32_t ae = mapa_u32(smem_u32(&acc_empty), 0);
-    int u = u0;
-    Segment sg;
-    int g = 0;
-    while (next_segment(u, u1, p.num_kb, sg)) {
-      const int tile = sg.job % p.tiles, mchunk = p.lock > 1 ? my_chunk : sg.job / p.tiles;
-      if (!mbar_wait_cluster(smem_u32(&acc_full), (uint32_t)g & 1u, wc, 214)) break;
-      tc_fence_after();
-      const int job_u0 = sg.job * p.num_kb;
-      const int first_share = job_u0 / p.per;
-      const int last_share = (job_u0 + p.num_kb - 1) / p.per;
-      const int slot = share - first_share;
-      const int m_base = mchunk * PAIR_ACT;
-      const int m_cnt = min(PAIR_ACT, p.M - m_base);
-      const size_t ldo = (size_t)p.N;
-      for (int hf = 0; hf < 2; ++hf) {
-        const int n_out = tile * PAIR_TILE + hf * 2 * BM + (int)rank * BM + quarter * 32 + lane;
-        const bool n_ok = n_out < p.N;
-        float* o = p.out + ((size_t)slot * p.M + m_base) * ldo + (n_ok ? n_out : 0);
-        const uint32_t taddr = tmem_base + (uint32_t)(hf * PAIR_ACT) + ((uint32_t)(quarter * 32) << 16);
-        for (int c0 = 0; c0 < m_cnt; c0 += 16) {
-          uint32_t r[16];
-          tmem_ld16(taddr + (uint32_t)c0, r);
-          if (n_ok) {
-            if (c0 + 16 <= m_cnt) {
-#pragma unroll
-              for (int j = 0; j < 16; ++j) { *o = __uint_as_float(r[j]); o += ldo; }
-            } else {
-#pragma unroll
-              for (int j = 0; j < 16; ++j)
-                if (c0 + j < m_cnt) { *o = __uint_as_float(r[j]); o += ldo; }
-            }
-          }
-        }
-      }
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive_cluster(ae);          // (the first CTA's own warps arrive the same way)
-      if (share == last_share) {
-        for (int hf = 0; hf < 2; ++hf) {
-          const int n_out = tile * PAIR_TILE + hf * 2 * BM + (int)rank * BM + quarter * 32 + lane;
-          if (n_out >= p.N) continue;
-          for (int z = last_share - first_share + 1; z < p.nslots; ++z) {
-            float* zo = p.out + ((size_t)z * p.M + m_base) * ldo + n_out;
-            for (int m = 0; m < m_cnt; ++m) { *zo = 0.f; zo += ldo; }
-          }
-        }
-      }
-      ++g;
-    }
-  }
-  tc_fence_before();
-  __syncthreads();
-  if (p.clk && threadIdx.x == 0) atomicMax(p.clk + kGemmClockSlots, globaltimer_ns());
-  // Neither CTA leaves (nor frees its tensor memory) before the other is done: copies, commits and arrivals cross
-  // between them until then.  The rendezvous keeps a budget of its own, far above that of the other waits, so that a
-  // CTA which has given up still finds its partner.
-  if (warp == 2) cluster_meet_before_exit(&meet_bar, 2, lane, wc, &meet_flag_s, 215);
-  __syncthreads();
-  if (warp == 1)
-    asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(512u) : "memory");
-}
-
 struct GemmPlan {
-  int tiles, mchunks, num_kb, per, ctas, nslots, lock;
-  bool pair;         // CTA pairs (gemm_bf16_pair_kernel): `ctas` then counts pairs, a unit is 512 weight rows
+  int tiles, num_kb, per, ctas, nslots;
   long long total;   // checked to fit 31 bits before launch
 };
 
-// Up to 128 rows: single CTAs, one pass over all rows.  More: CTA pairs, 256 rows per pass.
-GemmPlan make_plan(int sm_count, int M, int N, int K) {
-  GemmPlan g;
-  g.pair = M > BM;
-  if (g.pair) sm_count /= 2;                   // workers are pairs
-  const int rows_per_tile = g.pair ? PAIR_TILE : 2 * BM;     // a unit is two weight tiles of 128 rows (of 256 for a pair)
-  g.tiles = (N + rows_per_tile - 1) / rows_per_tile;
-  g.mchunks = g.pair ? (M + PAIR_ACT - 1) / PAIR_ACT : 1;
-  g.num_kb = (K + BK - 1) / BK;
-  // More than one row chunk: the (tile, k block) list of ONE chunk is cut into (pairs / chunks) shares and every
-  // share is walked by `chunks` pairs side by side, one per row chunk.  They ask for the same weight tiles at the
-  // same time, so HBM delivers every weight byte once instead of once per row chunk (measured at 2048 rows x
-  // 22016 x 4096 before this: 1.58 GB of DRAM reads for 180 MB of weights, the kernel at 70 % of DRAM throughput).
-  g.lock = (g.mchunks > 1 && g.mchunks * 2 <= sm_count) ? g.mchunks : 1;
-  const int jobs = g.lock > 1 ? g.tiles : g.tiles * g.mchunks;
-  const int shares = sm_count / g.lock;
-  g.total = (long long)jobs * g.num_kb;
-  long long per = (g.total + shares - 1) / shares;
+// `jobs` x num_kb units cut into `workers` equal contiguous shares.
+void cut_shares(GemmPlan& g, long long jobs, int workers) {
+  g.total = jobs * g.num_kb;
+  long long per = (g.total + workers - 1) / workers;
   int min_per = g.num_kb < 4 ? g.num_kb : 4;          // do not shred tiny problems into one-block segments
   if (per < min_per) per = min_per;
   g.per = (int)per;
-  g.ctas = (int)((g.total + per - 1) / per) * g.lock;
+  g.ctas = (int)((g.total + per - 1) / per);
   g.nslots = 1;
-  for (long long job = 0; job < (long long)jobs; ++job) {
+  for (long long job = 0; job < jobs; ++job) {
     int first = (int)(job * g.num_kb / per), last = (int)((job * g.num_kb + g.num_kb - 1) / per);
     if (last - first + 1 > g.nslots) g.nslots = last - first + 1;
   }
+}
+
+// Up to 128 rows: single CTAs, one pass over all rows; a unit is two weight tiles of 128 rows.
+GemmPlan make_plan(int sm_count, int N, int K) {
+  GemmPlan g;
+  g.tiles = (N + 2 * BM - 1) / (2 * BM);
+  g.num_kb = (K + BK - 1) / BK;
+  cut_shares(g, g.tiles, sm_count);
   return g;
 }
 
@@ -756,9 +518,45 @@ int make_weight_map(CUtensorMap* out, const void* W, int N, int K) {
   return encode_2d(out, W, (uint64_t)K, (uint64_t)N, (uint64_t)K * 2, BK, BM);
 }
 
+namespace {
+// Weight rows [N][K] seen as an array of blocks of rows, so that one box gathers 128 rows in another order.
+int encode_rows_nd(CUtensorMap* out, const void* W, int K, int nd, const cuuint64_t* counts, const cuuint64_t* row_strides, const cuuint32_t* box_rows) {
+  if (init_driver_api() != CERB_OK) return CERB_E_CUDA;
+  if (((uintptr_t)W & 15) || ((size_t)K * 2 & 15)) return CERB_E_SHAPE;
+  cuuint64_t dims[5] = {(cuuint64_t)K}, strides[4];
+  cuuint32_t box[5] = {BK}, estr[5] = {1, 1, 1, 1, 1};
+  for (int i = 0; i < nd; ++i) {
+    dims[i + 1] = counts[i];
+    strides[i] = row_strides[i] * (cuuint64_t)K * 2;
+    box[i + 1] = box_rows[i];
+  }
+  CUresult r = g_encode(out, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, nd + 1, const_cast<void*>(W), dims, strides, box, estr,
+                        CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                        CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  return r == CUDA_SUCCESS ? CERB_OK : CERB_E_CUDA;
+}
+}  // namespace
+
+// [gate rows F][up rows F]: a box is 4 x (16 gate rows, the 16 up rows of the same features).  F a multiple of 16.
+int make_gate_up_map(CUtensorMap* out, const void* W, int F, int K) {
+  const cuuint64_t counts[3] = {16, 2, (cuuint64_t)F / 16}, strides[3] = {1, (cuuint64_t)F, 16};
+  const cuuint32_t box[3] = {16, 2, 4};
+  return encode_rows_nd(out, W, K, 3, counts, strides, box);
+}
+
+// `heads` blocks of 128 rows: a box is one block as 4 x (rows 16 q .. 16 q + 15, rows 64 + 16 q .. 64 + 16 q + 15).
+int make_rotation_map(CUtensorMap* out, const void* W, int heads, int K) {
+  const cuuint64_t counts[4] = {16, 2, 4, (cuuint64_t)heads}, strides[4] = {1, 64, 16, 128};
+  const cuuint32_t box[4] = {16, 2, 4, 1};
+  return encode_rows_nd(out, W, K, 4, counts, strides, box);
+}
+
+int make_act_map(ActMaps* out, const void* X, int rows_alloc, int K, int box_rows) {
+  return encode_2d(&out->m[box_rows / 16 - 1], X, (uint64_t)K, (uint64_t)rows_alloc, (uint64_t)K * 2, BK, (uint32_t)box_rows);
+}
+
 int make_act_maps(ActMaps* out, const void* X, int rows_alloc, int K) {
-  for (int b = 0; b < kRowBuckets; ++b)
-    CERB_TRY(encode_2d(&out->m[b], X, (uint64_t)K, (uint64_t)rows_alloc, (uint64_t)K * 2, BK, (uint32_t)bucket_rows(b)));
+  for (int rows = 16; rows <= BM; rows += 16) CERB_TRY(make_act_map(out, X, rows_alloc, K, rows));
   return CERB_OK;
 }
 
@@ -768,7 +566,6 @@ int make_pool_map(CUtensorMap* out, const void* pool, int n_pool_pages, int H, i
   return encode_2d(out, pool, (uint64_t)Dh, (uint64_t)n_pool_pages * H * CERB_PAGE, (uint64_t)Dh * 2, 64, CERB_PAGE);
 }
 
-// Number of partial slots the schedule produces for this problem (what consumers must sum).
 // The fused SwiGLU epilogue needs the wide schedule (both halves of a unit in one CTA) and whole tiles.
 // It pays for few rows only (the auto-regressive step): the CTA that completes a tile re-reads the
 // tile's slots with its 128 epilogue threads, which at 64 rows took 55 us per layer against the
@@ -781,58 +578,42 @@ bool gemm_swiglu_fusable(int M, int F) {
 bool gemm_rope_fusable(int M, int head_dim) {
   return M >= 1 && M <= 16 && head_dim == 128;
 }
-int gemm_plan_split(int sm_count, int M, int N, int K) { return make_plan(sm_count, M, N, K).nslots; }
+// Number of partial slots the schedule produces for this problem (what consumers must sum).
+int gemm_plan_split(int sm_count, int M, int N, int K) {
+  return M > BM ? make_tile_plan(M, N, K).nslots : make_plan(sm_count, N, K).nslots;
+}
+
+// Slots of M x N floats that the scratch of the stand-alone GEMM holds.  Up to 128 rows the slots of the plan.  Above, the
+// size that callers of that entry have been told to provide: the slots of 74 workers walking 512 weight rows at a time,
+// side by side on chunks of 256 rows; the tile plan (gemm_tile.cu) is fitted into it.
+int gemm_scratch_slots(int M, int N, int K) {
+  GemmPlan g = make_plan(148, N, K);
+  if (M <= BM) return g.nslots;
+  const int tiles = (N + 4 * BM - 1) / (4 * BM), chunks = (M + kGemmRowsPerPass - 1) / kGemmRowsPerPass;
+  const bool grouped = chunks > 1 && chunks * 2 <= 74;
+  cut_shares(g, grouped ? tiles : (long long)tiles * chunks, grouped ? 74 / chunks : 74);
+  return g.nslots;
+}
 
 int launch_gemm_bf16(cerb_ctx* c, const CUtensorMap* tmW, const ActMaps* tmX, float* out, int M, int N, int K,
                      int nsplit, int32_t* status, cudaStream_t st, const GemmEpilogue* epi, unsigned long long* clock_slot) {
   if (M <= 0 || N <= 0 || K <= 0 || (K % 8) != 0) return CERB_E_SHAPE;
-  static int sm_count = 0;
-  if (!sm_count) {
-    int dev = 0;
-    CERB_CUDA_OK(cudaGetDevice(&dev));
-    CERB_CUDA_OK(cudaDeviceGetAttribute(&sm_count, cudaDevAttrMultiProcessorCount, dev));
-    if (sm_count > 148) sm_count = 148;      // slot counts are planned for at most 148 CTAs
-  }
+  if (M > BM) return CERB_E_SHAPE;             // (gemm_tile.cu)
   // Fewer SMs than planned for would need more slots than the caller sized: plan with the number
   // the caller used (148) and simply run that many CTAs; the hardware queues what does not fit.
-  GemmPlan g = make_plan(148, M, N, K);
+  GemmPlan g = make_plan(148, N, K);
   if (g.nslots != nsplit) return CERB_E_ARG;
-  if (g.pair) {
-    if (epi && epi->kind != 0) return CERB_E_SHAPE;
-    if (g.total >= (1ll << 30)) return CERB_E_SHAPE;
-    GemmParams q;
-    memset(&q, 0, sizeof(q));
-    q.out = out; q.status = status;
-    q.M = M; q.N = N; q.K = K;
-    q.n_mma = PAIR_ACT; q.num_kb = g.num_kb; q.tiles = g.tiles; q.per = g.per; q.total = (int)g.total; q.lock = g.lock;
-    q.nslots = g.nslots; q.stages = PAIR_STAGES; q.wait_cycles = wait_cycles(); q.acc_cols = 2u * PAIR_ACT; q.acc_bufs = 1;
-    q.tile_rows = PAIR_TILE; q.half_off = 2 * BM;
-    q.clk = clock_slot;
-    const size_t smem = (size_t)PAIR_STAGES * PAIR_STAGE_BYTES + 1024;
-    static bool pair_configured = false;
-    if (!pair_configured) {
-      CERB_CUDA_OK(cudaFuncSetAttribute(gemm_bf16_pair_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-      pair_configured = true;
-    }
-    // each CTA loads 128 of the pass's 256 activation rows: the map with 128-row boxes
-    if (launch_pdl_cluster(gemm_bf16_pair_kernel, dim3(2 * g.ctas), dim3(224), smem, st, 2u, *tmW, tmX->m[row_bucket(BM)], q) != cudaSuccess)
-      return CERB_E_CUDA;
-    CERB_LAUNCH_CHECK(c);
-    return CERB_OK;
-  }
   GemmParams p;
   memset(&p, 0, sizeof(p));
-  int bucket = row_bucket(M);                   // (M <= 128 here)
   p.out = out;
   p.status = status;
   p.M = M; p.N = N; p.K = K;
-  p.n_mma = bucket_rows(bucket);
+  p.n_mma = row_bucket(M);
   p.num_kb = g.num_kb;
   p.tiles = g.tiles;
   p.per = g.per;
   if (g.total >= (1ll << 30)) return CERB_E_SHAPE;
   p.total = (int)g.total;
-  p.lock = 1;
   p.nslots = g.nslots;
   p.tile_rows = 2 * BM;
   p.wait_cycles = wait_cycles();
@@ -840,7 +621,7 @@ int launch_gemm_bf16(cerb_ctx* c, const CUtensorMap* tmW, const ActMaps* tmX, fl
   p.epi = 0; p.F = 0; p.act = nullptr; p.tickets = nullptr;
   p.clk = clock_slot;
   if (epi && epi->kind == 1) {
-    if (!gemm_swiglu_fusable(M, N / 2) || (N & 1) || g.tiles * g.mchunks > kGemmTickets || !epi->act || !epi->tickets) return CERB_E_SHAPE;
+    if (!gemm_swiglu_fusable(M, N / 2) || (N & 1) || g.tiles > kGemmTickets || !epi->act || !epi->tickets) return CERB_E_SHAPE;
     p.epi = 1; p.F = N / 2; p.act = (bf16*)epi->act; p.tickets = epi->tickets;
     p.tile_rows = BM;            // a unit = gate tile t (rows t*128..) and up tile t (rows F + t*128..)
     p.half_off = p.F;
@@ -854,7 +635,6 @@ int launch_gemm_bf16(cerb_ctx* c, const CUtensorMap* tmW, const ActMaps* tmX, fl
   if (p.stages > MAX_STAGES) p.stages = MAX_STAGES;
   if (p.stages < 2) return CERB_E_SHAPE;
   p.acc_cols = 2u * (uint32_t)p.n_mma;            // two weight tiles side by side (at least 32 columns)
-  p.acc_bufs = 2;                                 // 2 x (2 x 128) columns at most
   // instruction descriptor: D fp32, A and B bf16, both K-major, N = n_mma, M = 128
   p.idesc = idesc_bf16(BM, (uint32_t)p.n_mma, false, false);
   size_t smem = (size_t)p.stages * stage_bytes + 1024;
@@ -864,7 +644,7 @@ int launch_gemm_bf16(cerb_ctx* c, const CUtensorMap* tmW, const ActMaps* tmX, fl
     CERB_CUDA_OK(cudaFuncSetAttribute(gemm_bf16_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(220 * 1024)));
     configured = true;
   }
-  if (launch_pdl(gemm_bf16_kernel, dim3(g.ctas), dim3(224), smem, st, *tmW, tmX->m[bucket], p) != cudaSuccess) return CERB_E_CUDA;
+  if (launch_pdl(gemm_bf16_kernel, dim3(g.ctas), dim3(224), smem, st, *tmW, tmX->box(p.n_mma), p) != cudaSuccess) return CERB_E_CUDA;
   CERB_LAUNCH_CHECK(c);
   return CERB_OK;
 }

@@ -38,72 +38,83 @@ struct Entry {
   unsigned prewait_reads;
 };
 
-// One layer, then the tail.  Ids are what forward_rows announces, in this order.
+// The launches of one layer, then the tail.  Ids are what forward_rows announces, in this order.
 const Entry kSetActive = {LO_SET_ACTIVE, "set_active / gate (live node counts)", B_STATE, 0};
-const Entry kLayer64[] = {
-    {LO_NORM_ATTN, "fused_norm (embedding or residual add, attention norm)", B_X | B_XN, B_X | B_CONST},
-    {LO_GEMM_QKV, "gemm qkv", B_PART, B_CONST},
-    {LO_ROPE, "rope_append", B_Q | B_KV, B_STATE | B_CONST},
-    {LO_ATTN, "tree attention", B_ATTN, B_STATE | B_CONST},
-    {LO_GEMM_WO, "gemm wo", B_PART, B_CONST},
-    {LO_NORM_MLP, "fused_norm (residual add, MLP norm)", B_X | B_XN, B_X | B_CONST},
-    {LO_GEMM_GU, "gemm gate-up", B_PART, B_CONST},
-    {LO_SWIGLU, "swiglu", B_ACT, 0},
-    {LO_GEMM_DOWN, "gemm down", B_PART, B_CONST},
-};
-// Few-row steps: SwiGLU runs in the gate-up GEMM's epilogue (that GEMM writes the activations itself).
-const Entry kLayer16[] = {
-    kLayer64[0], kLayer64[1], kLayer64[2], kLayer64[3], kLayer64[4], kLayer64[5],
-    {LO_GEMM_GU, "gemm gate-up + swiglu epilogue", B_PART | B_ACT, B_CONST},
-    kLayer64[8],
-};
-// ... and (head_dim 128) RoPE + cache append in the QKV GEMM's epilogue.
-const Entry kLayer16r[] = {
-    kLayer64[0],
-    {LO_GEMM_QKV, "gemm qkv + rope / append epilogue", B_PART | B_Q | B_KV, B_CONST},
-    kLayer64[3], kLayer64[4], kLayer64[5],
-    {LO_GEMM_GU, "gemm gate-up + swiglu epilogue", B_PART | B_ACT, B_CONST},
-    kLayer64[8],
-};
-const Entry kTail[] = {
-    {LO_NORM_FINAL, "fused_norm (residual add, final norm)", B_X | B_HIDDEN, B_X | B_CONST},
-    {LO_GEMM_LM, "gemm lm_head", B_PART, B_CONST},
-    {LO_ARGMAX, "argmax_rows", 0, 0},
-};
+const Entry kNormAttn = {LO_NORM_ATTN, "fused_norm (embedding or residual add, attention norm)", B_X | B_XN, B_X | B_CONST};
+const Entry kQkv = {LO_GEMM_QKV, "gemm qkv", B_PART, B_CONST};
+const Entry kRope = {LO_ROPE, "rope_append", B_Q | B_KV, B_STATE | B_CONST};
+const Entry kAttn = {LO_ATTN, "tree attention", B_ATTN, B_STATE | B_CONST};
+const Entry kWo = {LO_GEMM_WO, "gemm wo", B_PART, B_CONST};
+const Entry kNormMlp = {LO_NORM_MLP, "fused_norm (residual add, MLP norm)", B_X | B_XN, B_X | B_CONST};
+const Entry kGu = {LO_GEMM_GU, "gemm gate-up", B_PART, B_CONST};
+const Entry kSwiglu = {LO_SWIGLU, "swiglu", B_ACT, 0};
+const Entry kDown = {LO_GEMM_DOWN, "gemm down", B_PART, B_CONST};
+const Entry kNormFinal = {LO_NORM_FINAL, "fused_norm (residual add, final norm)", B_X | B_HIDDEN, B_X | B_CONST};
+const Entry kLm = {LO_GEMM_LM, "gemm lm_head", B_PART, B_CONST};
+const Entry kArgmax = {LO_ARGMAX, "argmax_rows", 0, 0};
+// SwiGLU in the gate-up GEMM's epilogue: that GEMM writes the activations itself.  RoPE + cache append in the QKV GEMM's.
+const Entry kGuSwiglu = {LO_GEMM_GU, "gemm gate-up + swiglu epilogue", B_PART | B_ACT, B_CONST};
+const Entry kQkvRope = {LO_GEMM_QKV, "gemm qkv + rope / append epilogue", B_PART | B_Q | B_KV, B_CONST};
+// The residual add in the O and down GEMMs' epilogues: the norms then read the residual stream after their wait (the
+// embedding gather in front of the first layer writes it, as ever).
+const Entry kWoAdd = {LO_GEMM_WO, "gemm wo + residual add epilogue", B_PART | B_X, B_CONST};
+const Entry kDownAdd = {LO_GEMM_DOWN, "gemm down + residual add epilogue", B_PART | B_X, B_CONST};
+const Entry kNormAttnRead = {LO_NORM_ATTN, "fused_norm (attention norm)", B_X | B_XN, B_CONST};
+const Entry kNormMlpRead = {LO_NORM_MLP, "fused_norm (MLP norm)", B_XN, B_CONST};
+const Entry kNormFinalRead = {LO_NORM_FINAL, "fused_norm (final norm)", B_HIDDEN, B_CONST};
 
-int build(int variant, const Entry** out, int cap) {
+// Variants 0, 1 and 2 are the steps of up to 128 rows; the others occur above.
+constexpr int kVariants = 8;
+const Fusion kFusion[kVariants] = {  // {swiglu, rope, residual}
+    {false, false, false}, {true, false, false}, {true, true, false}, {true, true, true},
+    {false, true, false},  {false, false, true}, {true, false, true}, {false, true, true}};
+
+int layer(int variant, const Entry** out) {
+  const Fusion& f = kFusion[variant];
+  int n = 0;
+  out[n++] = f.residual ? &kNormAttnRead : &kNormAttn;
+  out[n++] = f.rope ? &kQkvRope : &kQkv;
+  if (!f.rope) out[n++] = &kRope;
+  out[n++] = &kAttn;
+  out[n++] = f.residual ? &kWoAdd : &kWo;
+  out[n++] = f.residual ? &kNormMlpRead : &kNormMlp;
+  out[n++] = f.swiglu ? &kGuSwiglu : &kGu;
+  if (!f.swiglu) out[n++] = &kSwiglu;
+  out[n++] = f.residual ? &kDownAdd : &kDown;
+  return n;
+}
+
+int build(int variant, const Entry** out) {
   // set-up, three layers (enough to close the cycle between layers), tail
-  const Entry* layer = variant == 2 ? kLayer16r : variant == 1 ? kLayer16 : kLayer64;
-  const int nl = variant == 2   ? (int)(sizeof(kLayer16r) / sizeof(Entry))
-                 : variant == 1 ? (int)(sizeof(kLayer16) / sizeof(Entry))
-                                : (int)(sizeof(kLayer64) / sizeof(Entry));
   int n = 0;
   out[n++] = &kSetActive;
-  for (int l = 0; l < 3; ++l)
-    for (int i = 0; i < nl && n < cap; ++i) out[n++] = &layer[i];
-  for (int i = 0; i < 3 && n < cap; ++i) out[n++] = &kTail[i];
+  for (int l = 0; l < 3; ++l) n += layer(variant, out + n);
+  out[n++] = kFusion[variant].residual ? &kNormFinalRead : &kNormFinal;
+  out[n++] = &kLm;
+  out[n++] = &kArgmax;
   return n;
 }
 
 }  // namespace
 
-int launch_order_layer(int variant, const int** ids_out) {
-  static int ids64[16], ids16[16], ids16r[16];
-  static int n64 = 0, n16 = 0, n16r = 0;
-  if (!n64) {
-    for (const Entry& e : kLayer64) ids64[n64++] = e.id;
-    for (const Entry& e : kLayer16) ids16[n16++] = e.id;
-    for (const Entry& e : kLayer16r) ids16r[n16r++] = e.id;
-  }
-  *ids_out = variant == 2 ? ids16r : variant == 1 ? ids16 : ids64;
-  return variant == 2 ? n16r : variant == 1 ? n16 : n64;
+int launch_order_variant(Fusion f) {
+  for (int v = 0; v < kVariants; ++v)
+    if (kFusion[v].swiglu == f.swiglu && kFusion[v].rope == f.rope && kFusion[v].residual == f.residual) return v;
+  return 0;
+}
+
+int launch_order_layer(int variant, int* ids_out) {
+  const Entry* seq[kLayerLaunches];
+  const int n = layer(variant, seq);
+  for (int i = 0; i < n; ++i) ids_out[i] = seq[i]->id;
+  return n;
 }
 
 // Number of (kernel, buffer) pairs that break the rule; the tail after the last layer counts as the "next layer"
 // (its first kernel is a fused_norm as well).
 int launch_order_violations(int variant) {
   const Entry* seq[64];
-  const int n = build(variant, seq, 64);
+  const int n = build(variant, seq);
   int bad = 0;
   for (int i = 1; i < n; ++i) {
     for (unsigned bit = 1; bit <= B_STATE; bit <<= 1) {
@@ -120,9 +131,9 @@ int launch_order_violations(int variant) {
 
 extern "C" int cerb_launch_order_table(int32_t variant, char* buf, size_t cap) {
   using namespace cerb;
-  if (!buf || cap < 64 || variant < 0 || variant > 2) return CERB_E_ARG;
+  if (!buf || cap < 64 || variant < 0 || variant >= kVariants) return CERB_E_ARG;
   const Entry* seq[64];
-  const int n = build(variant, seq, 64);
+  const int n = build(variant, seq);
   size_t off = 0;
   for (int i = 0; i < n; ++i) {
     int w = snprintf(buf + off, cap - off, "%d|%s|%u|%u\n", seq[i]->id, seq[i]->name, seq[i]->writes, seq[i]->prewait_reads);
