@@ -105,16 +105,19 @@ size_t part_floats_needed(const cerb_config* g, int Mmax, int lm_rows, int sm_co
   const int HD = g->n_heads * g->head_dim;
   const int shapes[5][2] = {{3 * HD, g->d_model}, {g->d_model, HD}, {2 * g->mlp_dim, g->d_model},
                             {g->d_model, g->mlp_dim}, {g->vocab, g->d_model}};
+  const bool bf16 = g->dtype == CERB_BF16;
+  // GEMMs of more than 128 rows whose result an epilogue finishes leave nothing here
+  const bool finished[5] = {bf16 && g->head_dim == 128, bf16, bf16 && g->mlp_dim % 16 == 0, bf16, false};
   size_t best = 0;
-  for (int i = 0; i < 5; ++i)
-    // the plan depends on whether M exceeds 128 and on the number of 256-row chunks, so the last M of each class decides
-    for (int M = 0, top = i == 4 ? lm_rows : Mmax; M < top;) {
-      M = M == 0 ? (top < 128 ? top : 128) : M == 128 ? (top < kGemmRowsPerPass ? top : kGemmRowsPerPass)
-                                                     : (top < M + kGemmRowsPerPass ? top : M + kGemmRowsPerPass);
-      int ns = g->dtype == CERB_BF16 ? gemm_plan_split(sm_count, M, shapes[i][0], shapes[i][1]) : 1;
-      size_t f = (size_t)ns * M * shapes[i][0];
-      if (f > best) best = f;
-    }
+  for (int i = 0; i < 5; ++i) {
+    // the slots depend on M only in whether it exceeds 128, so the last M of each class decides
+    const int top = i == 4 ? lm_rows : Mmax;
+    const int narrow = top < 128 ? top : 128;
+    size_t f = (size_t)(bf16 ? gemm_plan_split(sm_count, narrow, shapes[i][0], shapes[i][1]) : 1) * narrow * shapes[i][0];
+    if (f > best) best = f;
+    f = (size_t)top * shapes[i][0];
+    if (top > 128 && !finished[i] && f > best) best = f;
+  }
   return best;
 }
 
@@ -305,11 +308,11 @@ int forward_rows(cerb_ctx* c, const cerb_tree* tree, const int32_t* tok, int tok
   }
   // Steps of up to 16 rows: SwiGLU runs in the gate-up GEMM's epilogue and (head_dim 128) RoPE + cache append in the
   // QKV GEMM's.
-  // More than 128 rows: so does whatever follows a GEMM whose plan has whole tiles, the residual adds included.
+  // More than 128 rows: so does whatever follows a GEMM, the residual adds included.
   const bool wide = c->bf16 && M > 128;
-  const bool fuse_swiglu = wide ? F % 16 == 0 && make_tile_plan(M, 2 * F, d).whole : c->bf16 && gemm_swiglu_fusable(M, F);
-  const bool fuse_rope = wide ? g.head_dim == 128 && make_tile_plan(M, 3 * HD, d).whole : fuse_swiglu && gemm_rope_fusable(M, g.head_dim);
-  const bool fuse_res = wide && make_tile_plan(M, d, HD).whole;        // (the down GEMM has the same tiles)
+  const bool fuse_swiglu = wide ? F % 16 == 0 : c->bf16 && gemm_swiglu_fusable(M, F);
+  const bool fuse_rope = wide ? g.head_dim == 128 : fuse_swiglu && gemm_rope_fusable(M, g.head_dim);
+  const bool fuse_res = wide;
   OrderCheck oc(launch_order_variant({fuse_swiglu, fuse_rope, fuse_res}));
   // embedding gather fused with the first layer's attention norm
   CERB_ORDER(oc, LO_NORM_ATTN);
@@ -395,7 +398,7 @@ int lm_head_argmax(cerb_ctx* c, const void* X, const ActMaps* xm, int rows, int3
                    cudaStream_t st) {
   int ns = 1;
   // one slot: the GEMM writes the caller's logits itself, and the argmax reads them there
-  const bool direct = logits_out && c->bf16 && rows > 128 && gemm_plan_split(c->sm_count, rows, c->cfg.vocab, c->cfg.d_model) == 1;
+  const bool direct = logits_out && c->bf16 && rows > 128;
   { ProfScope ps(c, K_GEMM, st);
     CERB_TRY(gemm(c, X, xm, c->lm_head, c->bf16 ? &c->tm_lm_head : nullptr, rows, c->cfg.vocab, c->cfg.d_model, &ns, st,
                   direct ? logits_out : nullptr)); }
@@ -793,23 +796,19 @@ int cerb_gemm(int32_t dtype, const void* X_dev, const void* W_dev, float* out_de
   int32_t* status = reinterpret_cast<int32_t*>(scratch_dev);
   float* part = reinterpret_cast<float*>((char*)scratch_dev + 256);
   CERB_CUDA_OK(cudaMemsetAsync(status, 0, 4, st));
-  int ns;
   if (M > 128) {
-    // behind the status word: the fix-up buffer and, after it, its tickets (one slot, which goes straight to the output),
-    // or the partial slots
+    // one sum, which goes straight to the output; behind the status word: the fix-up buffer and, after it, its counters
     const size_t room = (need - 256) / sizeof(float);
-    const TilePlan g = make_tile_plan(M, N, K, gemm_scratch_slots(M, N, K), room > kGemmTickets ? room - kGemmTickets : 0);
-    ns = g.nslots;
+    const TilePlan g = make_tile_plan(M, N, K, room > kGemmTickets ? room - kGemmTickets : 0);
     unsigned int* tickets = reinterpret_cast<unsigned int*>(part + g.fix_floats);
     if (g.fix_floats) CERB_CUDA_OK(cudaMemsetAsync(tickets, 0, kGemmTickets * sizeof(unsigned int), st));
     CERB_TRY(make_act_map(&tx, X_dev, M, K, g.n_act / 2));
-    CERB_TRY(launch_gemm_tile(nullptr, &tw, &tx, g, ns == 1 ? out_dev : part, part, tickets, M, N, status, st));
-    if (ns == 1) return CERB_OK;
-  } else {
-    ns = gemm_plan_split(148, M, N, K);
-    CERB_TRY(make_act_map(&tx, X_dev, M, K, row_bucket(M)));
-    CERB_TRY(launch_gemm_bf16(nullptr, &tw, &tx, part, M, N, K, ns, status, st));
+    CERB_TRY(launch_gemm_tile(nullptr, &tw, &tx, g, out_dev, part, tickets, M, N, status, st));
+    return CERB_OK;
   }
+  const int ns = gemm_plan_split(148, M, N, K);
+  CERB_TRY(make_act_map(&tx, X_dev, M, K, row_bucket(M)));
+  CERB_TRY(launch_gemm_bf16(nullptr, &tw, &tx, part, M, N, K, ns, status, st));
   size_t total = (size_t)M * N;
   sum_splits_kernel<<<(unsigned)((total + 255) / 256), 256, 0, st>>>(part, ns, total, out_dev, total);
   if (cudaGetLastError() != cudaSuccess) return CERB_E_CUDA;

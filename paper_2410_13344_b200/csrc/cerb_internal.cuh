@@ -198,7 +198,7 @@ inline int row_bucket(int rows) {
   while (r < rows && r < 128) r <<= 1;
   return r;
 }
-constexpr int kGemmTickets = 4096;
+constexpr int kGemmTickets = 8192;
 constexpr int kGemmClockSlots = 4096;
 constexpr int kTopkChunks = 16;     // the vocabulary is cut into this many chunks for the heads' top-k
 
@@ -240,7 +240,7 @@ int gemm_plan_split(int sm_count, int M, int N, int K);
 // that completes a 256-row tile (two heads' worth of q, k or v) last sums the tile's slots in index order, rotates q
 // and k at position len + depth and writes q dense and k, v into the paged pools -- what rope_append_kernel does,
 // with the same arithmetic in the same order.  In the single-CTA kernel both pay for steps of up to 16 rows only; above 128
-// rows (gemm_tile.cu) they run wherever the plan has whole tiles.
+// rows (gemm_tile.cu) they always run.
 // kind 3 (gemm_tile.cu only): the product is added to the fp32 residual stream.
 struct RopeEpilogue {
   const int32_t *len, *n_active, *depth, *page_table, *row_off;    // as for rope_append_kernel (row_off may be null)
@@ -257,12 +257,11 @@ struct GemmEpilogue {
 };
 // gemm_tile.cu: more than 128 rows
 struct TilePlan {
-  int mchunks, n_act, num_kb, pairs, per, sk_tiles, nslots;
+  int hf, chains, mchunks, n_act, num_kb, pairs, S, per, sk_tiles;
   long long tiles;          // checked to fit 31 bits before launch
-  bool whole;               // at least as many tiles as pairs: one slot, epilogues allowed
   size_t fix_floats;        // what the plan needs of the fix-up buffer
 };
-TilePlan make_tile_plan(int M, int N, int K, int max_slots = 1 << 30, size_t max_fix = ~(size_t)0);
+TilePlan make_tile_plan(int M, int N, int K, size_t max_fix = ~(size_t)0);
 size_t gemm_fix_floats();   // of any plan
 int launch_gemm_tile(cerb_ctx* c, const CUtensorMap* tmW, const ActMaps* tmX, const TilePlan& g, float* out, float* fix, unsigned int* tickets,
                      int M, int N, int32_t* status, cudaStream_t st, const GemmEpilogue* epi = nullptr,

@@ -580,7 +580,7 @@ bool gemm_rope_fusable(int M, int head_dim) {
 }
 // Number of partial slots the schedule produces for this problem (what consumers must sum).
 int gemm_plan_split(int sm_count, int M, int N, int K) {
-  return M > BM ? make_tile_plan(M, N, K).nslots : make_plan(sm_count, N, K).nslots;
+  return M > BM ? 1 : make_plan(sm_count, N, K).nslots;
 }
 
 // Slots of M x N floats that the scratch of the stand-alone GEMM holds.  Up to 128 rows the slots of the plan.  Above, the

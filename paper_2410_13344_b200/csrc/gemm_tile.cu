@@ -1,25 +1,33 @@
 // bf16 GEMM for more than 128 activation rows (batched trees, prefill): output tiles on CTA pairs (tcgen05 cta_group::2).
 //
-//   D[256 weight rows][up to 256 activation rows] per tile, fp32, in the tensor memory of two CTAs
+//   D[256 HF weight rows][up to 256 activation rows] per tile, fp32, in the tensor memory of two CTAs, HF = 1 or 2
 //
-// What bounds it: the tensor pipe from about 512 rows on, weight stream and tensor pipe alike at 256 rows.
+// What bounds it: the tensor pipe and the power limit from about 1000 rows on, L2 (11.6 TB/s measured on the way to the
+// SMs) at a few hundred rows, the weight stream at 256 rows and fewer.
 //
 // Tile.  One MMA is 256 weight rows tall, 128 from each CTA's shared memory, and its activation rows (the MMA's N, up to
-// 256) come half from each CTA; each CTA's tensor memory receives its 128 rows of D.  An accumulator takes 256 of the 512
-// columns, so there are two, and a tile's epilogue runs under the next tile's MMAs.  A stage is 64 k: 16 KB of weights and
-// up to 16 KB of activations per CTA, six or seven stages at 256 rows.  M rows are cut into ceil(M / 256) equal chunks,
-// rounded up to 32 rows: 300 rows are two passes of 160, not of 256.
+// 256) come half from each CTA; each CTA's tensor memory receives its 128 rows of D.  An accumulator takes up to 256 of the
+// 512 columns.
+//   HF = 1: one accumulator per tile, so there are two of them and a tile's epilogue runs under the next tile's MMAs.
+//           With few tiles per pair they hold the even and the odd k blocks of one tile instead (`chains`): a chain of
+//           tensor-core accumulations loses about half a unit in the last place per step, always towards zero, and 4096 k in
+//           one chain doubled the share of bf16 results that round the other way (keys of the first layer at the 13B width
+//           against the oracle, mean difference: 3.0e-6 in chains of up to 33 k blocks, 6.9e-6 in chains of 80).
+//   HF = 2: two MMA rows share one activation tile: 96 KB instead of 128 KB from L2 per 512 x 256 x 64, but the epilogue is
+//           covered only as far as the MMAs of the next tile's first accumulator run under the second one's.
+// A stage is 64 k.  M rows are cut into equal chunks of up to 256, rounded up to 32 rows.
 //
-// Schedule.  Whole tiles where there are at least as many as pairs: they are dealt out in turn (neighbouring pairs work on
-// the chunks of one weight tile, so HBM delivers it once), and what does not fill a last wave evenly, between one and two
-// tiles per pair, is cut along k into equal shares, which are done first.  A share is at least one tile long, so at most two
-// pairs meet in a tile: the one that finishes first leaves its sums in a fix-up buffer, the other adds them to its own and
-// runs the epilogue.  The result has one slot (and the same bits whoever is first).
-// Fewer tiles than pairs (a 4096-column GEMM below 1200 rows): the (tile, k block) list is cut into equal shares for all
-// pairs and every share leaves its sums in a partial slot of its own, as in gemm_bf16.cu; the kernel that consumes them
-// adds the slots.  (A fix-up by one pair would read up to five partial tiles of 256 KB through one SM.)
+// Schedule (make_tile_plan chooses by a cost model).  Every output has one sum, written once by an epilogue:
+//   - whole tiles dealt out in turn; neighbouring pairs work on the chunks of one weight tile, so HBM delivers it once;
+//   - few tiles: S pairs per tile, each a range of k.  Every pair leaves the columns that others finish in a fix-up buffer
+//     and finishes its own share of them, adding the others' sums in k order (a reduce-scatter through L2);
+//   - a last wave that would be nearly empty: between one and two tiles per pair are cut along k into equal shares, which
+//     are done first.  A share is at least one tile long, so at most two pairs meet in a tile: the one that finishes first
+//     leaves its sums in the fix-up buffer, the other adds them to its own and runs the epilogue.
+// Where pairs wait for one another they are CTAs of one launch that fits the GPU at once, and the one waited for has its
+// MMAs behind it or depends on nobody.
 //
-// Epilogues (KIND; only with one slot):
+// Epilogues (KIND; 0 writes the product):
 //   1  SwiGLU.  The weight tile is fetched with 16 gate rows and the 16 up rows of the same features in turn (a 4-D view
 //      of the matrix), so a warp's 32 accumulator lanes hold 16 (gate, up) pairs; one shuffle per two columns brings the
 //      members of a pair together, and half a warp finishes one activation row, the other half the next.
@@ -29,6 +37,8 @@
 // They replace passes of element-wise kernels over the fp32 sums.
 #include <string.h>
 
+#include <type_traits>
+
 #include "tc_common.cuh"
 
 namespace cerb {
@@ -37,7 +47,6 @@ namespace {
 
 constexpr int BK = 64;
 constexpr int MAX_STAGES = 8;
-constexpr int TILE_W = 256;                                // weight rows of a tile (128 per CTA)
 constexpr int TILE_X = kGemmRowsPerPass;                   // activation rows of a tile at most
 constexpr uint32_t A_BYTES = 128 * BK * 2;
 constexpr int kPairs = 74;
@@ -45,9 +54,9 @@ constexpr int kEpiWarps = 8;                               // two per 32 tensor-
 constexpr int kThreads = 64 + 32 * kEpiWarps;
 
 struct TileParams {
-  float* out;               // KIND 0: [slot][M][N]; KIND 3: the residual stream [M][N]
-  float* fix;               // [pair][tail, head of a split tile][CTA][column / 4][128 lanes][4]
-  unsigned int* tickets;    // [split tile][CTA][epilogue warp], zero on entry and on exit
+  float* out;               // KIND 0: [M][N]; KIND 3: the residual stream [M][N]
+  float* fix;               // [pair][tail, head of a split tile][CTA][accumulator][column / 4][128 lanes][4]; S > 1: no heads
+  unsigned int* tickets;    // [split tile][CTA][accumulator][epilogue warp], zero on entry and on exit
   bf16* act;                // KIND 1: [M][F]
   RopeEpilogue re;          // KIND 2
   int32_t* status;
@@ -55,8 +64,9 @@ struct TileParams {
   int n_act;                // activation rows per chunk
   int stages;
   int mchunks, num_kb, tiles;
-  int sk_tiles, per, sk_total;   // tiles cut along k, k blocks per share, k blocks in all of them
-  int nslots;
+  int chains;                    // 2: the two accumulators hold the even and the odd k blocks of a tile
+  int S;                         // pairs per tile
+  int sk_tiles, per, sk_total;   // tiles cut along k into equal shares, k blocks per share, k blocks in all of them
   long long wait_cycles;
   unsigned long long* clk;
 };
@@ -66,9 +76,10 @@ struct Run {
   int tile, kb0, nkb;
 };
 struct Work {
-  int u, u1, whole, step, tiles, num_kb;
+  int u, u1, whole, step, tiles, num_kb, S, part;
   __device__ __forceinline__ Work(const TileParams& p, int pair, int pairs)
-      : u(pair * p.per), u1(min(pair * p.per + p.per, p.sk_total)), whole(p.sk_tiles + pair), step(pairs), tiles(p.tiles), num_kb(p.num_kb) {}
+      : u(pair * p.per), u1(min(pair * p.per + p.per, p.sk_total)), whole(p.S > 1 ? pair / p.S : p.sk_tiles + pair), step(pairs), tiles(p.tiles),
+        num_kb(p.num_kb), S(p.S), part(pair % p.S) {}
   __device__ __forceinline__ bool next(Run& r) {
     if (u < u1) {
       r.tile = u / num_kb;
@@ -79,8 +90,8 @@ struct Work {
     }
     if (whole >= tiles) return false;
     r.tile = whole;
-    r.kb0 = 0;
-    r.nkb = num_kb;
+    r.kb0 = part * num_kb / S;
+    r.nkb = (part + 1) * num_kb / S - r.kb0;
     whole += step;
     return true;
   }
@@ -116,13 +127,13 @@ __device__ __forceinline__ void load_weights(uint32_t dst, const CUtensorMap* ma
 // stored: with the bounds checks of the stores in between, each column's chain of latencies came after the last one's
 // (QKV of the 7B shape at 512 rows: 103 us, and 58 this way with eight epilogue warps instead of four).
 template <int KIND>
-__device__ __forceinline__ void finish(const TileParams& p, const float* v, int slot, int unit, int quarter, int lane, int row0, int c0,
+__device__ __forceinline__ void finish(const TileParams& p, const float* v, int unit, int quarter, int lane, int row0, int c0,
                                        const int* pos_s, const int* kv_s) {
   const int left = min(32, min(p.n_act - c0, p.M - row0 - c0));            // live columns
   if constexpr (KIND == 0 || KIND == 3) {
     const int n_out = unit * 128 + quarter * 32 + lane;
     if (n_out >= p.N) return;
-    float* o = p.out + ((size_t)slot * p.M + row0 + c0) * p.N + n_out;     // (consecutive lanes: consecutive columns of a row)
+    float* o = p.out + (size_t)(row0 + c0) * p.N + n_out;     // (consecutive lanes: consecutive columns of a row)
     float x[32];
 #pragma unroll
     for (int j = 0; j < 32; ++j) x[j] = KIND == 3 && j < left ? o[(size_t)j * p.N] : 0.f;
@@ -189,26 +200,48 @@ __device__ __forceinline__ void finish(const TileParams& p, const float* v, int 
   }
 }
 
-// A share's half of a split tile, warp by warp: whichever of the two pairs comes first (a ticket) leaves its sums in the
-// fix-up buffer and says so; the other one waits for that (the first has finished its MMAs, so nothing but its stores is
-// waited for) and adds them to its own, which have stayed in tensor memory.
-constexpr unsigned int kFixDone = 16u;
-__device__ __forceinline__ bool wait_fix(const unsigned int* ticket, const WaitCtx& w, int site) {
+// Warp by warp, the pairs that share a tile go by one counter in global memory (bounded wait).
+//   two shares (sk): whichever comes first takes the ticket 0, leaves its sums in the fix-up buffer and adds kFixDone; the
+//     other one waits for that and adds them to its own, which have stayed in tensor memory;
+//   S pairs: each adds 1 when what it leaves is written, waits for all S, and adds kFixDone when it has read what it needs;
+//     the last one to do so puts the counter back to zero.
+constexpr unsigned int kFixDone = 256u;
+__device__ __forceinline__ unsigned int ld_acquire(const unsigned int* a) {
+  unsigned int v;
+  asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(a) : "memory");
+  return v;
+}
+__device__ __forceinline__ bool wait_fix(const unsigned int* ticket, unsigned int mask, unsigned int least, const WaitCtx& w, int site) {
   const long long t0 = clock64();
   const long long budget = *w.aborted ? kAbortedWaitCycles : w.budget;
   for (;;) {
-    for (int i = 0; i < 16; ++i) {
-      unsigned int v;
-      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(ticket) : "memory");
-      if (v & kFixDone) return true;
-    }
+    for (int i = 0; i < 16; ++i)
+      if ((ld_acquire(ticket) & mask) >= least) return true;
     if (clock64() - t0 > budget) break;
   }
   wait_ran_out(w, site);
   return false;
 }
 
-template <int KIND>
+__device__ __forceinline__ void ld_acc32(uint32_t taddr, float* v) {
+  tmem_ld16_nowait(taddr, reinterpret_cast<uint32_t*>(v));
+  tmem_ld16_nowait(taddr + 16u, reinterpret_cast<uint32_t*>(v + 16));
+  tmem_ld_wait();
+}
+__device__ __forceinline__ void put_fix(float4* at, const float* v) {
+#pragma unroll
+  for (int j = 0; j < 8; ++j) __stcg(at + j * 128, make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]));
+}
+__device__ __forceinline__ void get_fix(const float4* at, float4* o) {
+#pragma unroll
+  for (int j = 0; j < 8; ++j) o[j] = __ldcg(at + j * 128);
+}
+__device__ __forceinline__ void add(const float4* o, float* v) {
+#pragma unroll
+  for (int j = 0; j < 8; ++j) { v[4 * j] += o[j].x; v[4 * j + 1] += o[j].y; v[4 * j + 2] += o[j].z; v[4 * j + 3] += o[j].w; }
+}
+
+template <int KIND, int HF>
 __global__ void __launch_bounds__(kThreads, 1) gemm_tile_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtensorMap tmX,
                                                                 const TileParams p) {
   extern __shared__ uint8_t smem_raw[];
@@ -223,7 +256,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tile_kernel(const __grid_con
   const WaitCtx wc{p.wait_cycles, aborted, p.status, p.N + 100000 * (p.M > 999 ? 999 : p.M)};
 
   const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
-  const uint32_t stage_bytes = A_BYTES + (uint32_t)p.n_act * BK;               // (half the chunk's activation rows)
+  const uint32_t stage_bytes = HF * A_BYTES + (uint32_t)p.n_act * BK;          // (half the chunk's activation rows)
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int rank = (int)cluster_ctarank();
   const bool first = rank == 0;
@@ -268,15 +301,17 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tile_kernel(const __grid_con
       auto more_w = [&]() { return rw.nkb > 0 || ww.next(rw); };
       auto load_w = [&]() {
         if (first) mbar_expect_tx(smem_u32(&full_bar[qw.s]), tx);
-        load_weights<KIND>(smem_base + (uint32_t)qw.s * stage_bytes, &tmW, rw.kb0, (rw.tile / p.mchunks) * 2 + rank,
-                           mapa_u32(smem_u32(&full_bar[qw.s]), 0), pol_w);
+#pragma unroll
+        for (int hf = 0; hf < HF; ++hf)
+          load_weights<KIND>(smem_base + (uint32_t)qw.s * stage_bytes + hf * A_BYTES, &tmW, rw.kb0, ((rw.tile / p.mchunks) * HF + hf) * 2 + rank,
+                             mapa_u32(smem_u32(&full_bar[qw.s]), 0), pol_w);
         ++rw.kb0;
         --rw.nkb;
         qw.next(p.stages);
       };
       auto load_x = [&]() {
         if (rx.nkb == 0) wx.next(rx);
-        tma_load_2d_pair(smem_base + (uint32_t)qx.s * stage_bytes + A_BYTES, &tmX, rx.kb0 * BK, (rx.tile % p.mchunks) * p.n_act + rank * (p.n_act >> 1),
+        tma_load_2d_pair(smem_base + (uint32_t)qx.s * stage_bytes + HF * A_BYTES, &tmX, rx.kb0 * BK, (rx.tile % p.mchunks) * p.n_act + rank * (p.n_act >> 1),
                          mapa_u32(smem_u32(&full_bar[qx.s]), 0), pol_x);
         ++rx.kb0;
         --rx.nkb;
@@ -309,33 +344,71 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tile_kernel(const __grid_con
   } else if (warp == 1) {
     // MMA issuer of the pair (first CTA).  The whole warp walks the list and one elected lane issues.
     if (first) {
-      const uint32_t idesc = idesc_bf16(TILE_W, (uint32_t)p.n_act, false, false);
+      const uint32_t idesc = idesc_bf16(256, (uint32_t)p.n_act, false, false);
       Work w(p, pair, pairs);
       Run r;
-      Ring q;
+      Ring q0, q;                        // stage of the next MMAs of the first / of the last accumulator
       bool live = true;
-      for (int g = 0; live && w.next(r); ++g) {
-        const int buf = g & 1;
-        if (!mbar_wait_cluster(smem_u32(&acc_empty[buf]), ((uint32_t)(g >> 1) & 1u) ^ 1u, wc, 222)) live = false;
-        live = __all_sync(0xffffffffu, live);
+      auto wait = [&](uint64_t& bar, uint32_t parity, int site) {
+        const bool ok = mbar_wait_cluster(smem_u32(&bar), parity, wc, site);
+        live = __all_sync(0xffffffffu, ok);
         tc_fence_after();
-        const uint32_t d = tmem_base + (uint32_t)(buf * TILE_X);
-        for (int k = 0; live && k < r.nkb; ++k) {
-          if (!mbar_wait_cluster(smem_u32(&full_bar[q.s]), q.ph, wc, 223)) live = false;
-          live = __all_sync(0xffffffffu, live);
-          if (!live) break;
-          tc_fence_after();
-          const uint32_t src = smem_base + (uint32_t)q.s * stage_bytes;
-          const uint64_t adesc = desc_k_sw128(src), bdesc = desc_k_sw128(src + A_BYTES);
-          if (elect_one()) {
+        return live;
+      };
+      auto issue = [&](int stage, int hf, uint32_t d, bool fresh) {
+        const uint32_t src = smem_base + (uint32_t)stage * stage_bytes;
+        const uint64_t adesc = desc_k_sw128(src + hf * A_BYTES), bdesc = desc_k_sw128(src + HF * A_BYTES);
 #pragma unroll
-            for (int kk = 0; kk < BK / 16; ++kk)
-              umma_bf16_pair(d, adesc + (uint64_t)(kk * 2), bdesc + (uint64_t)(kk * 2), idesc, (k > 0 || kk > 0) ? 1u : 0u);
-            umma_commit_pair(smem_u32(&empty_bar[q.s]));       // the stage is free in both CTAs once these MMAs have read it
-            if (k + 1 == r.nkb) umma_commit_pair(smem_u32(&acc_full[buf]));
+        for (int kk = 0; kk < BK / 16; ++kk)
+          umma_bf16_pair(d, adesc + (uint64_t)(kk * 2), bdesc + (uint64_t)(kk * 2), idesc, (!fresh || kk > 0) ? 1u : 0u);
+      };
+      for (int g = 0; live && w.next(r); ++g) {
+        if constexpr (HF == 1) {
+          const bool two = p.chains == 2;
+          const int buf = two ? 0 : g & 1;
+          if (!wait(acc_empty[buf], ((uint32_t)(two ? g : g >> 1) & 1u) ^ 1u, 222)) break;
+          for (int k = 0; k < r.nkb; ++k) {
+            if (!wait(full_bar[q.s], q.ph, 223)) break;
+            if (elect_one()) {
+              issue(q.s, 0, tmem_base + (uint32_t)((two ? k & 1 : buf) * TILE_X), k < p.chains);
+              umma_commit_pair(smem_u32(&empty_bar[q.s]));       // the stage is free in both CTAs once these MMAs have read it
+              if (k + 1 == r.nkb) umma_commit_pair(smem_u32(&acc_full[buf]));
+            }
+            __syncwarp();
+            q.next(p.stages);
           }
-          __syncwarp();
-          q.next(p.stages);
+        } else {
+          const uint32_t free_ph = ((uint32_t)g & 1u) ^ 1u;
+          if (!wait(acc_empty[0], free_ph, 222)) break;
+          // while the second accumulator of the tile before is still being read out, the first one runs ahead
+          int n0 = 0;
+          const int ahead = min(r.nkb, p.stages);
+          while (n0 < ahead && !__all_sync(0xffffffffu, mbar_try_wait_cluster(smem_u32(&acc_empty[1]), free_ph))) {
+            if (!wait(full_bar[q0.s], q0.ph, 223)) break;
+            if (elect_one()) {
+              issue(q0.s, 0, tmem_base, n0 == 0);
+              if (n0 + 1 == r.nkb) umma_commit_pair(smem_u32(&acc_full[0]));
+            }
+            __syncwarp();
+            q0.next(p.stages);
+            ++n0;
+          }
+          if (!live || !wait(acc_empty[1], free_ph, 227)) break;
+          for (int k = 0; k < r.nkb; ++k) {
+            if (k >= n0 && !wait(full_bar[q.s], q.ph, 223)) break;
+            if (elect_one()) {
+              if (k >= n0) {
+                issue(q.s, 0, tmem_base, k == 0);
+                if (k + 1 == r.nkb) umma_commit_pair(smem_u32(&acc_full[0]));
+              }
+              issue(q.s, 1, tmem_base + TILE_X, k == 0);
+              umma_commit_pair(smem_u32(&empty_bar[q.s]));
+              if (k + 1 == r.nkb) umma_commit_pair(smem_u32(&acc_full[1]));
+            }
+            __syncwarp();
+            q.next(p.stages);
+          }
+          q0 = q;
         }
       }
       if (!live && elect_one()) {
@@ -353,19 +426,17 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tile_kernel(const __grid_con
     Run r;
     int chunk_known = -1;
     // A warp whose wait has run out writes nothing more, but goes through the remaining runs (every later wait is short
-    // then): the other epilogue warps meet it at named barriers.
+    // then): the other epilogue warps meet it at named barriers, other pairs at the counters.
     bool live = true;
     for (int g = 0; w.next(r); ++g) {
-      const int buf = g & 1;
-      const int tile_w = r.tile / p.mchunks, chunk = r.tile % p.mchunks;
-      const int unit = tile_w * 2 + rank, row0 = chunk * p.n_act;
+      const int chunk = r.tile % p.mchunks, row0 = chunk * p.n_act;
       if (KIND == 2 && chunk != chunk_known) {
         // positions and cache rows of the chunk's activation rows
         asm volatile("bar.sync 2, 256;" ::: "memory");                       // (the previous tile's readers are done)
         const RopeEpilogue& e = p.re;
-        for (int c = ew * 32 + lane; c < p.n_act; c += 32 * kEpiWarps) {
+        for (int c = ew * 32 + lane; c < TILE_X; c += 32 * kEpiWarps) {
           int pos = -1, kv = -1;
-          if (row0 + c < p.M) {
+          if (c < p.n_act && row0 + c < p.M) {
             int b, v;
             locate_row(row0 + c, e.row_off, e.B, e.n, b, v);
             const int at = e.len[b] + e.depth[v], slot = e.len[b] + v;
@@ -380,78 +451,109 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tile_kernel(const __grid_con
         asm volatile("bar.sync 2, 256;" ::: "memory");
         chunk_known = chunk;
       }
-      if (!mbar_wait_cluster(smem_u32(&acc_full[buf]), (uint32_t)(g >> 1) & 1u, wc, 224)) live = false;      // the output is undefined from here on
-      live = __all_sync(0xffffffffu, live);
-      tc_fence_after();
-      const uint32_t taddr = tmem_base + (uint32_t)(buf * TILE_X) + ((uint32_t)(quarter * 32) << 16);
       int first_share = pair, last_share = pair;
       if (r.tile < p.sk_tiles) {
         first_share = r.tile * p.num_kb / p.per;
         last_share = (r.tile * p.num_kb + p.num_kb - 1) / p.per;
       }
-      const bool split = p.nslots == 1 && last_share > first_share;         // (two pairs: the first has the tile's head)
-      // fix-up buffer: a pair has at most one tail (part 0) and one head (part 1) of a split tile
-      const size_t fix_tile = (size_t)128 * p.n_act;
-      const bool head = pair == first_share;
-      float4* mine = reinterpret_cast<float4*>(p.fix + ((size_t)(pair * 2 + (head ? 1 : 0)) * 2 + rank) * fix_tile) + et;
-      const float4* other = reinterpret_cast<const float4*>(p.fix + ((size_t)(head ? last_share * 2 : first_share * 2 + 1) * 2 + rank) * fix_tile) + et;
-      unsigned int* ticket = p.tickets + ((size_t)r.tile * 2 + rank) * kEpiWarps + ew;
-      bool leave = false;
-      if (split) {
-        unsigned int t = 0;
-        if (lane == 0) t = atomicAdd(ticket, 1u);
-        t = __shfl_sync(0xffffffffu, t, 0);
-        leave = t == 0u;
-        if (!leave && !(t & kFixDone)) {
-          if (!wait_fix(ticket, wc, 226)) live = false;
-          live = __all_sync(0xffffffffu, live);
-        }
-        if (!leave) __threadfence();
-      }
-      if (live)
-        for (int c0 = half * 32; c0 < p.n_act; c0 += 64) {
-          float v[32];
-          float4 o4[8];
-          if (split && !leave) {
+      const bool split = last_share > first_share;                          // (two pairs: the first has the tile's head)
+#pragma unroll 1
+      for (int hf = 0; hf < HF; ++hf) {
+        const bool two = HF == 1 && p.chains == 2;
+        const int acc = HF == 2 ? hf : two ? 0 : g & 1;
+        const uint32_t full_ph = (uint32_t)(HF == 2 || two ? g : g >> 1) & 1u;
+        const int unit = ((r.tile / p.mchunks) * HF + hf) * 2 + rank;
+        if (!mbar_wait_cluster(smem_u32(&acc_full[acc]), full_ph, wc, 224)) live = false;      // the output is undefined from here on
+        live = __all_sync(0xffffffffu, live);
+        tc_fence_after();
+        const uint32_t taddr = tmem_base + (uint32_t)(acc * TILE_X) + ((uint32_t)(quarter * 32) << 16);
+        auto read_acc = [&](int c0, float* v) {
+          ld_acc32(taddr + (uint32_t)c0, v);
+          if (two && r.nkb > 1) {
+            float t[32];
+            ld_acc32(taddr + (uint32_t)(TILE_X + c0), t);
 #pragma unroll
-            for (int j = 0; j < 8; ++j) o4[j] = __ldcg(other + (size_t)((c0 >> 2) + j) * 128);
+            for (int j = 0; j < 32; ++j) v[j] += t[j];
           }
-          tmem_ld16_nowait(taddr + (uint32_t)c0, reinterpret_cast<uint32_t*>(v));
-          tmem_ld16_nowait(taddr + (uint32_t)c0 + 16u, reinterpret_cast<uint32_t*>(v + 16));
-          tmem_ld_wait();
-          if (leave) {
+        };
+        unsigned int* ticket = p.tickets + (((size_t)r.tile * 2 + rank) * HF + hf) * kEpiWarps + ew;
+        constexpr size_t kFixAcc = 128 * TILE_X / 4;       // float4s of one CTA's accumulator
+        float4* fix = reinterpret_cast<float4*>(p.fix) + et;
+        auto at = [&](int who, int c0) { return fix + (((size_t)who * 2 + rank) * HF + hf) * kFixAcc + (size_t)(c0 >> 2) * 128; };
+        if (p.S > 1) {
+          const int base = r.tile * p.S, self = pair - base;
+          // 64-column groups of the tile's accumulators belong to the pairs in turn
+          auto owner = [&](int c0) { return (hf * 4 + (c0 >> 6)) % p.S; };
+          if (live)
+            for (int c0 = half * 32; c0 < p.n_act; c0 += 64)
+              if (owner(c0) != self) {
+                float v[32];
+                read_acc(c0, v);
+                put_fix(at(pair, c0), v);
+              }
+          __threadfence();
+          __syncwarp();
+          if (lane == 0) atomicAdd(ticket, 1u);
+          if (live && !wait_fix(ticket, kFixDone - 1u, (unsigned)p.S, wc, 226)) live = false;
+          live = __all_sync(0xffffffffu, live);
+          __threadfence();
+          if (live)
+            for (int c0 = half * 32; c0 < p.n_act; c0 += 64)
+              if (owner(c0) == self) {
+                float v[32];
 #pragma unroll
-            for (int j = 0; j < 8; ++j) __stcg(mine + (size_t)((c0 >> 2) + j) * 128, make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]));
-          } else {
-            if (split) {
-#pragma unroll
-              for (int j = 0; j < 8; ++j) {
-                v[4 * j] += o4[j].x; v[4 * j + 1] += o4[j].y; v[4 * j + 2] += o4[j].z; v[4 * j + 3] += o4[j].w;
+                for (int j = 0; j < 32; ++j) v[j] = 0.f;
+                for (int s = 0; s < p.S; ++s) {               // k order
+                  float4 o[8];
+                  if (s == self) read_acc(c0, reinterpret_cast<float*>(o));
+                  else get_fix(at(base + s, c0), o);
+                  add(o, v);
+                }
+                finish<KIND>(p, v, unit, quarter, lane, row0, c0, pos_s, kv_s);
+              }
+          __syncwarp();
+          if (lane == 0 && (atomicAdd(ticket, kFixDone) >> 8) == (unsigned)p.S - 1u) *ticket = 0u;       // ready for the next launch
+        } else {
+          // a pair has at most one tail (part 0) and one head (part 1) of a split tile
+          const bool head = pair == first_share;
+          const int mine = pair * 2 + (head ? 1 : 0), other = head ? last_share * 2 : first_share * 2 + 1;
+          bool leave = false;
+          if (split) {
+            unsigned int t = 0;
+            if (lane == 0) t = atomicAdd(ticket, 1u);
+            t = __shfl_sync(0xffffffffu, t, 0);
+            leave = t == 0u;
+            if (!leave && !(t & kFixDone)) {
+              if (!wait_fix(ticket, kFixDone, kFixDone, wc, 228)) live = false;
+              live = __all_sync(0xffffffffu, live);
+            }
+            if (!leave) __threadfence();
+          }
+          if (live)
+            for (int c0 = half * 32; c0 < p.n_act; c0 += 64) {
+              float v[32];
+              float4 o[8];
+              if (split && !leave) get_fix(at(other, c0), o);
+              read_acc(c0, v);
+              if (leave) {
+                put_fix(at(mine, c0), v);
+              } else {
+                if (split) add(o, v);
+                finish<KIND>(p, v, unit, quarter, lane, row0, c0, pos_s, kv_s);
               }
             }
-            finish<KIND>(p, v, p.nslots > 1 ? pair - first_share : 0, unit, quarter, lane, row0, c0, pos_s, kv_s);
+          if (split) {
+            __threadfence();
+            __syncwarp();
+            if (lane == 0) {
+              if (leave) atomicAdd(ticket, kFixDone);
+              else if (live) *ticket = 0u;                      // ready for the next launch
+            }
           }
         }
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive_cluster(ae[buf]);          // (the first CTA's own warps arrive the same way)
-      if (split) {
-        __threadfence();
+        tc_fence_before();
         __syncwarp();
-        if (lane == 0) {
-          if (leave) atomicAdd(ticket, kFixDone);
-          else if (live) *ticket = 0u;                      // ready for the next launch
-        }
-      }
-      if (KIND == 0 && p.nslots > 1 && pair == last_share) {
-        // slots this tile does not use
-        const int n_out = unit * 128 + et;
-        const int rows = min(p.n_act, p.M - row0);
-        if (half == 0 && n_out < p.N)
-          for (int z = last_share - first_share + 1; z < p.nslots; ++z) {
-            float* zo = p.out + ((size_t)z * p.M + row0) * p.N + n_out;
-            for (int m = 0; m < rows; ++m) { *zo = 0.f; zo += p.N; }
-          }
+        if (lane == 0) mbar_arrive_cluster(ae[acc]);          // (the first CTA's own warps arrive the same way)
       }
     }
   }
@@ -469,94 +571,120 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tile_kernel(const __grid_con
 
 }  // namespace
 
-// max_slots, max_fix: what the caller's scratch holds (partial slots per output, floats of fix-up buffer).
-TilePlan make_tile_plan(int M, int N, int K, int max_slots, size_t max_fix) {
-  TilePlan g;
-  g.mchunks = (M + TILE_X - 1) / TILE_X;
-  g.n_act = ((M + g.mchunks - 1) / g.mchunks + 31) / 32 * 32;
-  g.num_kb = (K + BK - 1) / BK;
-  g.tiles = (long long)((N + TILE_W - 1) / TILE_W) * g.mchunks;
-  g.whole = g.tiles >= kPairs;
-  g.pairs = kPairs;
-  g.nslots = 1;
-  g.sk_tiles = 0;
-  g.per = 0;
-  g.fix_floats = 0;
-  if (g.whole) {
-    const int rem = (int)(g.tiles % kPairs);
-    const size_t fix = (size_t)kPairs * 2 * 2 * 128 * g.n_act;
-    if (rem && fix <= max_fix) {
-      g.sk_tiles = kPairs + rem;
-      g.per = (g.sk_tiles * g.num_kb + kPairs - 1) / kPairs;
-      g.fix_floats = fix;
-    }
-    return g;
-  }
-  g.sk_tiles = (int)g.tiles;
-  const int total = g.sk_tiles * g.num_kb;
-  g.per = (total + kPairs - 1) / kPairs;
-  const int least = g.num_kb < 4 ? g.num_kb : 4;      // do not shred tiny problems into one-block shares
-  if (g.per < least) g.per = least;
-  for (;; ++g.per) {
-    g.nslots = 1;
-    for (int t = 0; t < g.sk_tiles; ++t) {
-      const int n = (t * g.num_kb + g.num_kb - 1) / g.per - t * g.num_kb / g.per + 1;
-      if (n > g.nslots) g.nslots = n;
-    }
-    if (g.nslots <= max_slots) break;                  // (a share of num_kb blocks leaves one slot)
-  }
-  g.pairs = (total + g.per - 1) / g.per;
-  return g;
+// Estimated time of a plan in us.  Measured on the way: 11.6 TB/s from L2 to all SMs together, about 56 bytes a cycle to one;
+// 6.5 TB/s from HBM; MMAs of 256 rows and less than 120 columns take no less time than those of 120 (issuing); reading out
+// an accumulator of 128 lanes x 256 columns about 2 us, and about as long again for each time it goes through the fix-up
+// buffer.
+static double tile_plan_cost(const TilePlan& g, int M, int N, int K) {
+  const double kMHz = 1750.0, n = g.n_act;
+  const double waves = g.sk_tiles ? (double)g.tiles / kPairs : (double)((g.tiles * g.S + kPairs - 1) / kPairs);
+  const double kbs = waves * ((g.num_kb + g.S - 1) / g.S);
+  const double tensor = kbs * g.hf * (2 * n > 240 ? 2 * n : 240) / kMHz;
+  const double sm = kbs * (g.hf * (double)A_BYTES + 64 * n) / (56 * kMHz);
+  const double l2 = (double)g.tiles * g.num_kb * (g.hf * 2.0 * A_BYTES + 128 * n) / 11.6e6;
+  const double hbm = (double)N * K * 2 / 6.5e6;
+  double t = tensor > sm ? tensor : sm;
+  if (l2 > t) t = l2;
+  if (hbm > t) t = hbm;
+  const double drain = 2.0 * n / 256;
+  t += g.hf == 2 || g.chains == 2 ? (waves < 1 ? 1 : waves) * 1.5 * drain : drain;
+  if (g.S > 1) t += 2 + g.hf * drain * 2 * (g.S - 1) / g.S;
+  if (g.sk_tiles) t += 3 + 1.5 * g.hf * drain;
+  return t;
 }
 
-size_t gemm_fix_floats() { return (size_t)kPairs * 2 * 2 * 128 * TILE_X; }
+// max_fix: floats of fix-up buffer that the caller has.
+TilePlan make_tile_plan(int M, int N, int K, size_t max_fix) {
+  TilePlan best;
+  double best_t = 0;
+  const int least_chunks = (M + TILE_X - 1) / TILE_X;
+  // (HF = 2 has no room for two chains: from three chunks of rows on)
+  for (int hf = 1; hf <= (least_chunks > 2 ? 2 : 1); ++hf)
+    for (int c = least_chunks; c <= least_chunks + least_chunks / 4 + 1; ++c)
+      for (int S = 1; S <= 4 * hf; ++S)
+        for (int sk = 0; sk <= (S == 1 ? 1 : 0); ++sk) {
+          TilePlan g;
+          g.hf = hf;
+          g.mchunks = c;
+          g.n_act = ((M + c - 1) / c + 31) / 32 * 32;
+          g.num_kb = (K + BK - 1) / BK;
+          g.tiles = (long long)((N + 256 * hf - 1) / (256 * hf)) * c;
+          g.S = S;
+          g.sk_tiles = g.per = 0;
+          g.fix_floats = 0;
+          g.pairs = kPairs;
+          if (S > 1) {
+            if (g.tiles * S > kPairs || g.num_kb < 4 * S) break;
+            g.fix_floats = (size_t)g.tiles * S * 2 * hf * 128 * TILE_X;
+          }
+          if (g.tiles * S < kPairs) g.pairs = (int)g.tiles * S;
+          if (sk) {
+            const int rem = (int)(g.tiles % kPairs);
+            if (g.tiles < kPairs || !rem) continue;
+            // shares walk k at their own offsets: what they read has to stay in L2 meanwhile
+            if (c > 1 && g.tiles < 3 * kPairs && ((double)M + N) * K * 2 > 64e6) continue;
+            g.sk_tiles = kPairs + rem;
+            g.per = (g.sk_tiles * g.num_kb + kPairs - 1) / kPairs;
+            g.fix_floats = (size_t)kPairs * 2 * 2 * hf * 128 * TILE_X;
+          }
+          if (g.fix_floats > max_fix) continue;
+          g.chains = hf == 1 && g.tiles * S <= 2 * kPairs ? 2 : 1;
+          const double t = tile_plan_cost(g, M, N, K);
+          if (best_t == 0 || t < best_t) {
+            best = g;
+            best_t = t;
+          }
+        }
+  return best;
+}
 
-template <int KIND>
+size_t gemm_fix_floats() { return (size_t)kPairs * 2 * 2 * 2 * 128 * TILE_X; }
+
+template <int KIND, int HF>
 static int launch_kind(const CUtensorMap& tmW, const CUtensorMap& tmX, TileParams q, int pairs, cudaStream_t st) {
   // shared memory left beside the kernel's static variables (barriers; KIND 2: positions and cache rows of a chunk)
   constexpr size_t kRing = 227 * 1024 - 1024 - (KIND == 2 ? 3072 : 512);
-  const size_t stage = A_BYTES + (size_t)q.n_act * BK;
+  const size_t stage = HF * A_BYTES + (size_t)q.n_act * BK;
   q.stages = (int)(kRing / stage);
   if (q.stages > MAX_STAGES) q.stages = MAX_STAGES;
   static bool configured = false;
   if (!configured) {
-    CERB_CUDA_OK(cudaFuncSetAttribute(gemm_tile_kernel<KIND>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(kRing + 1024)));
+    CERB_CUDA_OK(cudaFuncSetAttribute(gemm_tile_kernel<KIND, HF>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(kRing + 1024)));
     configured = true;
   }
   // (always the same request: more than half of an SM, so that a CTA may own all of its tensor memory)
-  return launch_pdl_cluster(gemm_tile_kernel<KIND>, dim3(2 * pairs), dim3(kThreads), kRing + 1024, st, 2u, tmW, tmX, q) == cudaSuccess ? CERB_OK : CERB_E_CUDA;
+  return launch_pdl_cluster(gemm_tile_kernel<KIND, HF>, dim3(2 * pairs), dim3(kThreads), kRing + 1024, st, 2u, tmW, tmX, q) == cudaSuccess ? CERB_OK : CERB_E_CUDA;
 }
 
 int launch_gemm_tile(cerb_ctx* c, const CUtensorMap* tmW, const ActMaps* tmX, const TilePlan& g, float* out, float* fix, unsigned int* tickets,
                      int M, int N, int32_t* status, cudaStream_t st, const GemmEpilogue* epi, unsigned long long* clock_slot) {
   const int kind = epi ? epi->kind : 0;
-  if (g.tiles >= (1ll << 30) || (long long)g.sk_tiles * g.num_kb >= (1ll << 30)) return CERB_E_SHAPE;
-  if (kind != 0 && !g.whole) return CERB_E_SHAPE;
-  if (g.whole && g.sk_tiles && (!fix || !tickets)) return CERB_E_ARG;
-  static_assert(2 * kPairs * 2 * kEpiWarps <= kGemmTickets, "one ticket per epilogue warp of every split tile");
+  if (g.tiles * g.num_kb >= (1ll << 30)) return CERB_E_SHAPE;
+  if (g.fix_floats && (!fix || !tickets)) return CERB_E_ARG;
+  static_assert(2 * kPairs * 2 * 2 * kEpiWarps <= kGemmTickets, "one counter per accumulator and epilogue warp of every split tile");
   TileParams q;
   memset(&q, 0, sizeof(q));
   q.out = kind == 3 ? epi->x : out;
   q.fix = fix; q.tickets = tickets; q.status = status;
   q.M = M; q.N = N;
   q.n_act = g.n_act; q.mchunks = g.mchunks; q.num_kb = g.num_kb; q.tiles = (int)g.tiles;
-  q.sk_tiles = g.sk_tiles; q.per = g.per; q.sk_total = g.sk_tiles * g.num_kb; q.nslots = g.nslots;
+  q.chains = g.chains; q.S = g.S; q.sk_tiles = g.sk_tiles; q.per = g.per; q.sk_total = g.sk_tiles * g.num_kb;
   q.wait_cycles = wait_cycles();
   q.clk = clock_slot;
   const CUtensorMap& x = tmX->box(g.n_act / 2);                      // each CTA loads half of a chunk's rows
-  int rc;
   if (kind == 1) {
     q.F = N / 2;
     q.act = (bf16*)epi->act;
-    rc = launch_kind<1>(*tmW, x, q, g.pairs, st);
-  } else if (kind == 2) {
-    q.re = *epi->rope;
-    rc = launch_kind<2>(*tmW, x, q, g.pairs, st);
-  } else if (kind == 3) {
-    rc = launch_kind<3>(*tmW, x, q, g.pairs, st);
-  } else {
-    rc = launch_kind<0>(*tmW, x, q, g.pairs, st);
   }
+  if (kind == 2) q.re = *epi->rope;
+  auto run = [&](auto hf) {
+    constexpr int HF = decltype(hf)::value;
+    return kind == 1   ? launch_kind<1, HF>(*tmW, x, q, g.pairs, st)
+           : kind == 2 ? launch_kind<2, HF>(*tmW, x, q, g.pairs, st)
+           : kind == 3 ? launch_kind<3, HF>(*tmW, x, q, g.pairs, st)
+                       : launch_kind<0, HF>(*tmW, x, q, g.pairs, st);
+  };
+  const int rc = g.hf == 2 ? run(std::integral_constant<int, 2>()) : run(std::integral_constant<int, 1>());
   if (rc != CERB_OK) return rc;
   CERB_LAUNCH_CHECK(c);
   return CERB_OK;
