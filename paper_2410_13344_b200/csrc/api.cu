@@ -160,6 +160,7 @@ size_t carve(cerb_ctx* c, char* base) {
   int Hc = g.n_cheads > 0 ? g.n_cheads : 1;
   c->d_hstate[0] = b.take<float>((size_t)MB * Hc * c->head_wmax);
   c->d_hstate[1] = b.take<float>((size_t)MB * Hc * c->head_wmax);
+  for (int i = 0; i < 2; ++i) c->d_hterms[i] = b.take<__nv_bfloat16>(c->bf16 ? (size_t)Hc * head_term_cols(g.max_batch) * c->head_wmax : 0);
   c->d_hlogits = b.take<float>((size_t)g.max_batch * Hc * g.vocab);
   c->d_rope = b.take<float2>((size_t)c->max_pos * (g.head_dim / 2));
   c->d_attn_scratch = b.take<char>(c->attn_scratch_bytes);

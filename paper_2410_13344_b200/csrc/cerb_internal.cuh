@@ -161,6 +161,7 @@ struct cerb_ctx {
   float* d_gemm_fix;      // partial tiles of the GEMM above 128 rows
   size_t part_floats;
   float* d_hstate[2];
+  __nv_bfloat16* d_hterms[2];         // bf16 models: the same states as three bf16 terms, [Hc][head_term_cols][head_wmax]
   float2* d_rope;
   char* d_attn_scratch;
   size_t attn_scratch_bytes;
@@ -289,6 +290,7 @@ int launch_tree_attention(cerb_ctx* c, const cerb_attn_args* a, const CUtensorMa
                           int sm_count, int32_t* status, cudaStream_t st, const int32_t* row_off = nullptr, bool chain = false);
 
 // heads.cu
+inline int head_term_cols(int max_batch) { return (3 * max_batch + 7) / 8 * 8; }
 int launch_heads(cerb_ctx* c, const cerb_tree* tree, int32_t* tree_tok, const int32_t* plant, int32_t* topk_out,
                  float* logits_out, cudaStream_t st);
 

@@ -3,9 +3,9 @@
 //     two-input:  h = Concat(h_i, h_{i-1});  out = SiLU((W h + b) + h)
 // followed by one FC layer to the vocabulary.  The sequential link sits inside the heads, so all
 // heads advance level by level together: one launch per level covers every head (grid.y = head),
-// the two-input block of head i reads head i-1's state as it entered the same level.  At batch 1
-// each level is a matrix-vector product: the kernel streams W once with 16-byte loads, keeps the
-// (concatenated) input vector in shared memory as fp32 and fuses bias, residual and SiLU.
+// the two-input block of head i reads head i-1's state as it entered the same level.  A level streams its
+// weights once, whatever the batch: bf16 models on the tensor cores (head_mma_kernel), fp32 models with
+// plain FMA (head_gemv_kernel); bias, residual and SiLU are fused.
 // The FC layer reuses the kernel without an epilogue; a per-head top-k (value descending, lower id
 // first among equals; per vocabulary chunk, then over the chunks' candidates) and the tree fill follow.
 #include "cerb_internal.cuh"
@@ -31,35 +31,19 @@ struct LevelParams {
   HeadJob job[CERB_MAX_HEADS];
   const float* state_in;    // [B][Hc][wmax]
   float* out;               // state_out [B][Hc][wmax] or logits [B][Hc][out_stride]
+  const bf16* terms_in;     // bf16 models: the same state as three bf16 terms, [Hc][cols][wmax], column 3 b + term
+  bf16* terms_out;
+  int cols;
   int Hc, wmax, out_stride, B, b0;
   int epilogue;             // 1: SiLU(acc + bias + input[row]); 0: plain product
 };
 
-template <typename T> struct Vec16;
-template <> struct Vec16<bf16> {
-  static constexpr int N = 8;
-  static __device__ __forceinline__ void load(const bf16* p, float* f) {
-    uint4 v;
-    // streamed once: no L1 allocation, and the memory side is asked for 256-byte pieces
-    asm volatile("ld.global.nc.L1::no_allocate.L2::256B.v4.u32 {%0, %1, %2, %3}, [%4];"
-                 : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
-    const __nv_bfloat162* h = reinterpret_cast<const __nv_bfloat162*>(&v);
-#pragma unroll
-    for (int i = 0; i < 4; ++i) { float2 t = __bfloat1622float2(h[i]); f[2 * i] = t.x; f[2 * i + 1] = t.y; }
-  }
-};
-template <> struct Vec16<float> {
-  static constexpr int N = 4;
-  static __device__ __forceinline__ void load(const float* p, float* f) {
-    float4 v = __ldg(reinterpret_cast<const float4*>(p));
-    f[0] = v.x; f[1] = v.y; f[2] = v.z; f[3] = v.w;
-  }
-};
 template <typename T> __device__ __forceinline__ float ldf(const T* p);
 template <> __device__ __forceinline__ float ldf<float>(const float* p) { return *p; }
 template <> __device__ __forceinline__ float ldf<bf16>(const bf16* p) { return __bfloat162float(*p); }
 
-template <typename T, int NB>
+// fp32 models.
+template <int NB>
 __global__ void __launch_bounds__(WARPS * 32) head_gemv_kernel(const LevelParams P) {
   extern __shared__ float su[];                       // [NB][w]
   griddep_wait();
@@ -79,24 +63,21 @@ __global__ void __launch_bounds__(WARPS * 32) head_gemv_kernel(const LevelParams
   __syncthreads();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int r0 = row_base + warp * ROWS_PER_WARP;
-  constexpr int E = Vec16<T>::N;
+  constexpr int E = 4;
   float acc[ROWS_PER_WARP][NB];
 #pragma unroll
   for (int i = 0; i < ROWS_PER_WARP; ++i)
 #pragma unroll
     for (int nb = 0; nb < NB; ++nb) acc[i][nb] = 0.f;
-  const T* Wp = reinterpret_cast<const T*>(J.W);
+  const float* Wp = reinterpret_cast<const float*>(J.W);
 #pragma unroll 2
   for (int k = lane * E; k < w; k += 32 * E) {
     float wv[ROWS_PER_WARP][E];
 #pragma unroll
     for (int i = 0; i < ROWS_PER_WARP; ++i) {
       int r = r0 + i;
-      if (r < J.rows) Vec16<T>::load(Wp + (size_t)r * w + k, wv[i]);
-      else {
-#pragma unroll
-        for (int e = 0; e < E; ++e) wv[i][e] = 0.f;
-      }
+      const float4 v = r < J.rows ? __ldg(reinterpret_cast<const float4*>(Wp + (size_t)r * w + k)) : make_float4(0.f, 0.f, 0.f, 0.f);
+      wv[i][0] = v.x; wv[i][1] = v.y; wv[i][2] = v.z; wv[i][3] = v.w;
     }
 #pragma unroll
     for (int nb = 0; nb < NB; ++nb) {
@@ -123,7 +104,7 @@ __global__ void __launch_bounds__(WARPS * 32) head_gemv_kernel(const LevelParams
         if (seq >= P.B) continue;
         float y = acc[i][nb];
         if (P.epilogue) {
-          y += ldf(reinterpret_cast<const T*>(J.bias) + r) + su[nb * w + r];
+          y += reinterpret_cast<const float*>(J.bias)[r] + su[nb * w + r];
           y = y / (1.0f + expf(-y));
         }
         P.out[((size_t)seq * P.Hc + head) * P.out_stride + r] = y;
@@ -132,13 +113,142 @@ __global__ void __launch_bounds__(WARPS * 32) head_gemv_kernel(const LevelParams
   }
 }
 
-template <typename T>
-__global__ void head_init_kernel(const T* __restrict__ h_last, float* __restrict__ state, int Hc, int wmax, int d) {
+// v = hi + mid + lo to 24 bits, a term every `stride`.
+__device__ __forceinline__ void store_terms(bf16* at, size_t stride, float v) {
+  const bf16 hi = __float2bfloat16_rn(v);
+  const float r = v - __bfloat162float(hi);
+  const bf16 mid = __float2bfloat16_rn(r);
+  at[0] = hi;
+  at[stride] = mid;
+  at[2 * stride] = __float2bfloat16_rn(r - __bfloat162float(mid));
+}
+
+__device__ __forceinline__ void mma_16816(float* c, uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1) {
+  asm volatile(
+      "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+      : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+      : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+}
+
+// One level (or the FC) of every head of a bf16 model, for the whole batch.  Bound by HBM: the weights once, 2.7 GB per
+// draft of the 7B shape.  The fp32 states enter the tensor cores as three bf16 terms each (24 bits; the products are exact
+// in fp32), so a batch is 3 B MMA columns instead of B passes of FMAs: with those, a batch of four took 1.90 ms per draft
+// (0.22 of the copy rate), bound by the FMAs and the shared-memory loads that feed them.
+// A CTA takes 16 MT 8 / KG weight rows, 16 MT to a warp; KG warps share a row group, each takes every KG-th 32-wide k block,
+// and their sums are added in shared memory.  Weights
+// go from global memory straight into the A fragments: a lane loads 16 consecutive bytes of a row, and its eight k values
+// stand for the k positions that the fragment layout gives that lane in two MMAs; the states are read in the same order.
+// The weights of the first blocks are requested before the wait for the level in front.
+constexpr int HM_WARPS = 8;
+template <int NT, int MT, int U, int KG, int MB>
+__global__ void __launch_bounds__(HM_WARPS * 32, MB) head_mma_kernel(const __grid_constant__ LevelParams P) {
+  extern __shared__ float red[];                      // [k group][rows][8 NT columns + 1]
+  constexpr int RG = HM_WARPS / KG, ROWS = 16 * MT * RG, LD = 8 * NT + 1;
+  const int head = blockIdx.y;
+  const HeadJob& J = P.job[head];
+  const int row_base = blockIdx.x * ROWS;
+  if (row_base >= J.rows) return;                     // (its dependents need not wait for it)
+  const int w = J.w0 + J.w1;
+  const int warp = (threadIdx.x >> 5) % KG, rg = (threadIdx.x >> 5) / KG, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+  const bf16* Wr[MT][2];
+#pragma unroll
+  for (int m = 0; m < MT; ++m)
+#pragma unroll
+    for (int e = 0; e < 2; ++e) Wr[m][e] = reinterpret_cast<const bf16*>(J.W) + (size_t)min(row_base + 16 * (m + MT * rg) + 8 * e + g, J.rows - 1) * w;
+  const bf16* own = P.terms_in + ((size_t)head * P.cols + g) * P.wmax;
+  const bf16* oth = P.terms_in + ((size_t)(J.src >= 0 ? J.src : head) * P.cols + g) * P.wmax - J.w0;
+  constexpr int STEP = 32 * KG;
+  auto load_w = [&](uint4 (&r)[U][MT][2], int k) {
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+#pragma unroll
+      for (int m = 0; m < MT; ++m)
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+          r[u][m][e] = make_uint4(0, 0, 0, 0);
+          if (k + u * STEP < w)
+            asm volatile("ld.global.nc.L1::no_allocate.L2::256B.v4.u32 {%0, %1, %2, %3}, [%4];"
+                         : "=r"(r[u][m][e].x), "=r"(r[u][m][e].y), "=r"(r[u][m][e].z), "=r"(r[u][m][e].w) : "l"(Wr[m][e] + k + u * STEP));
+        }
+  };
+  auto load_x = [&](uint4 (&r)[U][NT], int k) {
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+#pragma unroll
+      for (int n = 0; n < NT; ++n) {
+        const int kk = k + u * STEP;
+        r[u][n] = make_uint4(0, 0, 0, 0);
+        if (kk < w && 8 * n + g < 3 * P.B) r[u][n] = *reinterpret_cast<const uint4*>((kk < J.w0 ? own : oth) + (size_t)(8 * n) * P.wmax + kk);
+      }
+  };
+  float acc[MT][NT][4];
+#pragma unroll
+  for (int m = 0; m < MT; ++m)
+#pragma unroll
+    for (int n = 0; n < NT; ++n) acc[m][n][0] = acc[m][n][1] = acc[m][n][2] = acc[m][n][3] = 0.f;
+  auto multiply = [&](const uint4 (&a)[U][MT][2], const uint4 (&x)[U][NT]) {
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+#pragma unroll
+      for (int m = 0; m < MT; ++m)
+#pragma unroll
+        for (int n = 0; n < NT; ++n) {
+          mma_16816(acc[m][n], a[u][m][0].x, a[u][m][1].x, a[u][m][0].y, a[u][m][1].y, x[u][n].x, x[u][n].y);
+          mma_16816(acc[m][n], a[u][m][0].z, a[u][m][1].z, a[u][m][0].w, a[u][m][1].w, x[u][n].z, x[u][n].w);
+        }
+  };
+  uint4 w0[U][MT][2], w1[U][MT][2], x0[U][NT], x1[U][NT];
+  const int k0 = warp * 32 + t * 8;
+  load_w(w0, k0);
   griddep_wait();
   griddep_launch();
-  int b = blockIdx.x, h = blockIdx.y;
-  for (int k = threadIdx.x; k < d; k += blockDim.x)
-    state[((size_t)b * Hc + h) * wmax + k] = ldf(h_last + (size_t)b * d + k);
+  load_x(x0, k0);
+  for (int k = k0; k - t * 8 < w; k += 2 * U * STEP) {        // (uniform over the warp)
+    load_w(w1, k + U * STEP);
+    load_x(x1, k + U * STEP);
+    multiply(w0, x0);
+    load_w(w0, k + 2 * U * STEP);
+    load_x(x0, k + 2 * U * STEP);
+    multiply(w1, x1);
+  }
+#pragma unroll
+  for (int m = 0; m < MT; ++m)
+#pragma unroll
+    for (int n = 0; n < NT; ++n)
+#pragma unroll
+      for (int e = 0; e < 4; ++e)
+        red[(warp * ROWS + 16 * (m + MT * rg) + 8 * (e >> 1) + g) * LD + 8 * n + 2 * t + (e & 1)] = acc[m][n][e];
+  __syncthreads();
+  for (int i = threadIdx.x; i < ROWS * P.B; i += HM_WARPS * 32) {
+    const int rr = i % ROWS, b = i / ROWS, r = row_base + rr;
+    if (r >= J.rows) continue;
+    float y = 0.f;
+#pragma unroll
+    for (int q = 0; q < KG; ++q) {
+      const float* c = red + (q * ROWS + rr) * LD + 3 * b;
+      y += c[0] + c[1] + c[2];
+    }
+    if (P.epilogue) {
+      const int from = r < J.w0 ? head : J.src, at = r < J.w0 ? r : r - J.w0;
+      y += ldf(reinterpret_cast<const bf16*>(J.bias) + r) + P.state_in[((size_t)b * P.Hc + from) * P.wmax + at];
+      y = y / (1.0f + expf(-y));
+      store_terms(P.terms_out + ((size_t)head * P.cols + 3 * b) * P.wmax + r, P.wmax, y);
+    }
+    P.out[((size_t)b * P.Hc + head) * P.out_stride + r] = y;
+  }
+}
+
+// The last hidden states as the heads' first states (bf16 models: and as terms).
+template <typename T>
+__global__ void head_init_kernel(const T* __restrict__ h_last, float* __restrict__ state, int Hc, int wmax, int d, bf16* __restrict__ terms,
+                                 int cols) {
+  griddep_wait();
+  griddep_launch();
+  const int b = blockIdx.y, h = blockIdx.z, k = blockIdx.x * blockDim.x + threadIdx.x;
+  if (k >= d) return;
+  const float v = ldf(h_last + (size_t)b * d + k);
+  state[((size_t)b * Hc + h) * wmax + k] = v;
+  if (terms) store_terms(terms + ((size_t)h * cols + 3 * b) * wmax + k, wmax, v);
 }
 
 __device__ __forceinline__ bool better(float va, int ia, float vb, int ib) { return va > vb || (va == vb && ia < ib); }
@@ -172,8 +282,10 @@ __device__ __forceinline__ void block_best(float& best, int& bi, float* sv, int*
 // Per-head top-k in two steps.  Step 1: the vocabulary is cut into kTopkChunks chunks and one CTA per
 // (chunk, head, sequence) finds its chunk's k best in k rounds; round r only considers entries that come
 // strictly after the previous winner in (value descending, id ascending) order, so nothing is modified
-// in place.  The global k best are among these candidates.  Step 2: one CTA per (head, sequence) runs
-// the same k rounds over the kTopkChunks * k candidates.
+// in place.  A thread keeps its entries in registers and looks through them again only after one of them has won
+// (fetching the chunk anew in every round: 17 us for 4 heads x 32000 entries).  The global k best are among these
+// candidates.  Step 2: one CTA per (head, sequence) runs the same k rounds over the kTopkChunks * k candidates.
+constexpr int kTopkHeld = 16;             // entries a thread holds: chunks of up to 4096
 __global__ void __launch_bounds__(256) topk_part_kernel(const float* __restrict__ logits, int V, int Hc,
                                                         const int32_t* __restrict__ kper, float* __restrict__ cand_v,
                                                         int32_t* __restrict__ cand_i) {
@@ -189,15 +301,42 @@ __global__ void __launch_bounds__(256) topk_part_kernel(const float* __restrict_
   float pv = INFINITY;
   int pi = -1;
   const size_t o = (((size_t)b * Hc + h) * kTopkChunks + ch) * CERB_MAX_TOPK;
-  for (int round = 0; round < k; ++round) {
-    float best = -INFINITY;
-    int bi = 0x7fffffff;
-    for (int j = j0 + threadIdx.x; j < j1; j += blockDim.x) {
-      const float v = r[j];
-      const bool after = v < pv || (v == pv && j > pi);
-      if (after && better(v, j, best, bi)) { best = v; bi = j; }
+  const bool held = per <= kTopkHeld * (int)blockDim.x;
+  float keep[kTopkHeld];
+  if (held) {
+#pragma unroll
+    for (int e = 0; e < kTopkHeld; ++e) {
+      const int j = j0 + threadIdx.x + e * blockDim.x;
+      keep[e] = j < j1 ? r[j] : -INFINITY;
     }
+  }
+  float mine = 0.f;
+  int mi = -1;
+  bool look = true;
+  for (int round = 0; round < k; ++round) {
+    if (look) {
+      mine = -INFINITY;
+      mi = 0x7fffffff;
+      if (held) {
+#pragma unroll
+        for (int e = 0; e < kTopkHeld; ++e) {
+          const int j = j0 + threadIdx.x + e * blockDim.x;
+          const float v = keep[e];
+          const bool after = j < j1 && (v < pv || (v == pv && j > pi));
+          if (after && better(v, j, mine, mi)) { mine = v; mi = j; }
+        }
+      } else {
+        for (int j = j0 + threadIdx.x; j < j1; j += blockDim.x) {
+          const float v = r[j];
+          const bool after = v < pv || (v == pv && j > pi);
+          if (after && better(v, j, mine, mi)) { mine = v; mi = j; }
+        }
+      }
+    }
+    float best = mine;
+    int bi = mi;
     block_best(best, bi, sv, si);
+    look = bi == mi;
     pv = best;
     pi = bi;
     if (threadIdx.x == 0) {
@@ -263,26 +402,54 @@ __global__ void tree_fill_kernel(const int32_t* __restrict__ root, const int32_t
   }
 }
 
-template <typename T>
+template <int NT, int MT, int U, int KG, int MB>
+int launch_mma(cerb_ctx* c, const LevelParams& P, int max_rows, cudaStream_t st) {
+  constexpr int ROWS = 16 * MT * (HM_WARPS / KG);
+  constexpr size_t smem = (size_t)KG * ROWS * (8 * NT + 1) * sizeof(float);
+  static bool configured = false;
+  if (!configured) {
+    CERB_CUDA_OK(cudaFuncSetAttribute(head_mma_kernel<NT, MT, U, KG, MB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    configured = true;
+  }
+  if (launch_pdl(head_mma_kernel<NT, MT, U, KG, MB>, dim3((max_rows + ROWS - 1) / ROWS, P.Hc), dim3(HM_WARPS * 32), smem, st, P) != cudaSuccess)
+    return CERB_E_CUDA;
+  CERB_LAUNCH_CHECK(c);
+  return CERB_OK;
+}
+
+// bf16 models: the number of MMA column tiles decides (us per draft of the 7B shape, HBM floor 410).  Few columns want
+// small CTAs, three to an SM (batch 1: 441 against 480 with 32 rows); more columns want two warps side by side on the same k
+// blocks, whose state loads then meet in L1 (batch 4: 495 against 553; batch 8: 508 against 816), and at six tiles, where the
+// states weigh more than the weights on their way from L2, 64 rows per CTA (batch 16: 839 against 907; batch 9: 727).
+int launch_level_mma(cerb_ctx* c, const LevelParams& P, int max_rows, cudaStream_t st) {
+  switch ((3 * P.B + 7) / 8) {
+    case 1: return launch_mma<1, 1, 2, 8, 3>(c, P, max_rows, st);
+    case 2: return launch_mma<2, 1, 4, 4, 2>(c, P, max_rows, st);
+    case 3: return launch_mma<3, 2, 1, 4, 2>(c, P, max_rows, st);
+    case 4: return launch_mma<4, 2, 1, 4, 2>(c, P, max_rows, st);
+    default: return launch_mma<6, 4, 1, 8, 1>(c, P, max_rows, st);
+  }
+}
+
 int launch_level(cerb_ctx* c, const LevelParams& P, int max_rows, int max_w, cudaStream_t st) {
   dim3 grid((max_rows + ROWS_PER_BLOCK - 1) / ROWS_PER_BLOCK, P.Hc);
   size_t smem1 = (size_t)max_w * sizeof(float);
   static bool configured = false;
   if (!configured) {
-    CERB_CUDA_OK(cudaFuncSetAttribute(head_gemv_kernel<T, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
-    CERB_CUDA_OK(cudaFuncSetAttribute(head_gemv_kernel<T, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
+    CERB_CUDA_OK(cudaFuncSetAttribute(head_gemv_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
+    CERB_CUDA_OK(cudaFuncSetAttribute(head_gemv_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
     configured = true;
   }
   LevelParams Q = P;
   if (P.B == 1) {
     Q.b0 = 0;
-    launch_pdl(head_gemv_kernel<T, 1>, grid, dim3(WARPS * 32), smem1, st, Q);
+    launch_pdl(head_gemv_kernel<1>, grid, dim3(WARPS * 32), smem1, st, Q);
     CERB_LAUNCH_CHECK(c);
   } else {
     if (smem1 * 4 > 200 * 1024) return CERB_E_SHAPE;
     for (int b0 = 0; b0 < P.B; b0 += 4) {
       Q.b0 = b0;
-      launch_pdl(head_gemv_kernel<T, 4>, grid, dim3(WARPS * 32), smem1 * 4, st, Q);
+      launch_pdl(head_gemv_kernel<4>, grid, dim3(WARPS * 32), smem1 * 4, st, Q);
       CERB_LAUNCH_CHECK(c);
     }
   }
@@ -296,13 +463,14 @@ int launch_heads(cerb_ctx* c, const cerb_tree* tree, int32_t* tree_tok, const in
   const cerb_config& g = c->cfg;
   const int Hc = g.n_cheads, L = g.n_levels, d = g.d_model, B = c->B;
   if (Hc <= 0) return CERB_E_STATE;
-  if (c->bf16) launch_pdl(head_init_kernel<bf16>, dim3(B, Hc), dim3(256), 0, st, (const bf16*)c->d_hlast, c->d_hstate[0], Hc, c->head_wmax, d);
-  else launch_pdl(head_init_kernel<float>, dim3(B, Hc), dim3(256), 0, st, (const float*)c->d_hlast, c->d_hstate[0], Hc, c->head_wmax, d);
+  if (c->bf16) launch_pdl(head_init_kernel<bf16>, dim3((d + 255) / 256, B, Hc), dim3(256), 0, st, (const bf16*)c->d_hlast, c->d_hstate[0], Hc, c->head_wmax, d, c->d_hterms[0], head_term_cols(g.max_batch));
+  else launch_pdl(head_init_kernel<float>, dim3((d + 255) / 256, B, Hc), dim3(256), 0, st, (const float*)c->d_hlast, c->d_hstate[0], Hc, c->head_wmax, d, (bf16*)nullptr, 0);
   CERB_LAUNCH_CHECK(c);
   for (int j = 0; j <= L; ++j) {
     LevelParams P;
     P.state_in = c->d_hstate[j & 1];
     P.Hc = Hc; P.wmax = c->head_wmax; P.B = B; P.b0 = 0;
+    P.terms_in = c->d_hterms[j & 1]; P.terms_out = c->d_hterms[(j + 1) & 1]; P.cols = head_term_cols(g.max_batch);
     int max_rows = 0, max_w = 0;
     for (int h = 0; h < Hc; ++h) {
       HeadJob& J = P.job[h];
@@ -327,8 +495,8 @@ int launch_heads(cerb_ctx* c, const cerb_tree* tree, int32_t* tree_tok, const in
     }
     if (j < L) { P.out = c->d_hstate[(j + 1) & 1]; P.out_stride = c->head_wmax; P.epilogue = 1; }
     else { P.out = logits_out ? logits_out : c->d_hlogits; P.out_stride = g.vocab; P.epilogue = 0; }
-    if (c->bf16) CERB_TRY(launch_level<bf16>(c, P, max_rows, max_w, st));
-    else CERB_TRY(launch_level<float>(c, P, max_rows, max_w, st));
+    if (c->bf16) CERB_TRY(launch_level_mma(c, P, max_rows, st));
+    else CERB_TRY(launch_level(c, P, max_rows, max_w, st));
   }
   const float* lg = logits_out ? logits_out : c->d_hlogits;
   static_assert(kTopkChunks * CERB_MAX_TOPK <= 256, "one candidate per thread in the merge");

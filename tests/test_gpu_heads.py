@@ -1,0 +1,34 @@
+"""Decoding heads of bf16 models at every batch size class, on the tensor cores."""
+import pytest
+import torch
+
+from oracle import cerberus_oracle as orc
+from paper_2410_13344_b200 import binding as cb
+from paper_2410_13344_b200 import synth
+from tests.helpers import close
+from tests.test_gpu_model import Rig
+
+pytestmark = pytest.mark.gpu
+
+
+# one column tile, two, three, four (64 weight rows per CTA) and six; widths that are no multiple of a 32-wide k block
+# (264, concatenated 528) and shorter than a pass of all warps; a vocabulary that ends inside a CTA's rows
+@pytest.mark.parametrize("d,vocab", [(264, 1003), (64, 70), (1024, 2048)])
+@pytest.mark.parametrize("B", [1, 2, 3, 5, 8, 9, 13, 16])
+def test_draft_logits_match_oracle(B, d, vocab):
+    ms = synth.ModelShape(1, d, 2, 64, 128, vocab, "bf16")
+    rig = Rig(cb, ms, n_cheads=3, n_levels=3, topk=(5, 3, 2), concat_level=1, max_batch=B, max_tokens=32, max_nodes=16)
+    lens = [3 + b % 5 for b in range(B)]
+    tok = torch.stack([synth.make_prompt(vocab, 8, seq=50 + b) for b in range(B)]).to(torch.int32).cuda()
+    rig.eng.prefill(tok, lens)
+    _, roots, h_last = rig.eng.read_state()
+    tree = synth.best_first_tree(12, rig.topk)
+    tree_tok, topk, logits = rig.eng.draft(rig.eng.tree(tree), want_logits=True)
+    for b in range(B):
+        want = orc.heads_forward(h_last[b].double(), rig.cheads, rig.csrc)
+        for h in range(3):
+            # fp32 states, exact products, fp32 sums over at most 2048 terms: 2048 * 2^-24 per level at the worst
+            assert close(logits[b, h], want[h], 0) < 2e-4, (b, h)
+            ids = [int(t) for t in orc.topk_ids(logits[b, h].cpu().double(), rig.topk[h])]
+            assert [int(t) for t in topk[b, h, :rig.topk[h]]] == ids
+        assert [int(t) for t in tree_tok[b]] == [int(roots[b])] + [int(topk[b, tree.head[v], tree.rank[v]]) for v in range(1, tree.n)]
