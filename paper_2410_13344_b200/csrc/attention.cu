@@ -1063,20 +1063,55 @@ __global__ void __launch_bounds__(128) tree_attn_f32_kernel(const float* __restr
   const float* qp = q + ((qrow + i) * H + h) * DH;
   for (int e = 0; e < E; ++e) { qv[e] = qp[lane + 32 * e]; acc[e] = 0.f; }
   float m = -INFINITY, l = 0.f;
-  for (int kpos = warp; kpos < L + nq; kpos += 4) {
-    if (kpos >= L) {
-      int j = kpos - L;
-      if (!(((j < 64 ? a0 : j < 128 ? a1 : a2) >> (j & 63)) & 1ull)) continue;
+  // Four keys at a time, whose page entries, keys and values are all requested before the first is used: one key after the
+  // other was a chain of two round trips to memory and a reduction per key.
+  constexpr int KEYS = 4;
+  for (int base = warp * KEYS; base < L + nq; base += 4 * KEYS) {
+    size_t off[KEYS];
+    bool sees[KEYS];
+#pragma unroll
+    for (int u = 0; u < KEYS; ++u) {
+      const int kpos = base + u, j = kpos - L;
+      sees[u] = kpos < L + nq && (j < 0 || (((j < 64 ? a0 : j < 128 ? a1 : a2) >> (j & 63)) & 1ull));
+      const int page = sees[u] ? page_table[(size_t)b * max_pages + kpos / CERB_PAGE] : 0;
+      off[u] = (((size_t)page * H + h) * CERB_PAGE + kpos % CERB_PAGE) * DH;
     }
-    int page = page_table[(size_t)b * max_pages + kpos / CERB_PAGE];
-    size_t off = (((size_t)page * H + h) * CERB_PAGE + kpos % CERB_PAGE) * DH;
-    float s = 0.f;
-    for (int e = 0; e < E; ++e) s += qv[e] * kpool[off + lane + 32 * e];
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    s *= scale;
-    float mn = fmaxf(m, s), al = expf(m - mn), pw = expf(s - mn);
-    l = l * al + pw;
-    for (int e = 0; e < E; ++e) acc[e] = acc[e] * al + pw * vpool[off + lane + 32 * e];
+    float kv[KEYS][E], vv[KEYS][E], s[KEYS];
+#pragma unroll
+    for (int u = 0; u < KEYS; ++u)
+#pragma unroll
+      for (int e = 0; e < E; ++e) {
+        kv[u][e] = sees[u] ? kpool[off[u] + lane + 32 * e] : 0.f;
+        vv[u][e] = sees[u] ? vpool[off[u] + lane + 32 * e] : 0.f;
+      }
+#pragma unroll
+    for (int u = 0; u < KEYS; ++u) {
+      s[u] = 0.f;
+#pragma unroll
+      for (int e = 0; e < E; ++e) s[u] += qv[e] * kv[u][e];
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+      for (int u = 0; u < KEYS; ++u) s[u] += __shfl_xor_sync(0xffffffffu, s[u], o);
+    float mn = m;
+#pragma unroll
+    for (int u = 0; u < KEYS; ++u) {
+      s[u] = sees[u] ? s[u] * scale : -INFINITY;
+      mn = fmaxf(mn, s[u]);
+    }
+    if (mn == -INFINITY) continue;                       // (nothing seen so far; uniform over the warp)
+    const float al = expf(m - mn);
+    l *= al;
+#pragma unroll
+    for (int e = 0; e < E; ++e) acc[e] *= al;
+#pragma unroll
+    for (int u = 0; u < KEYS; ++u) {
+      const float pw = expf(s[u] - mn);
+      l += pw;
+#pragma unroll
+      for (int e = 0; e < E; ++e) acc[e] += pw * vv[u][e];
+    }
     m = mn;
   }
   for (int e = 0; e < E; ++e) s_o[warp][lane + 32 * e] = acc[e];

@@ -1,0 +1,19 @@
+"""The fp32 GEMM for few output tiles: ragged rows, columns and k, one piece of k and several."""
+import pytest
+import torch
+
+from oracle import cerberus_oracle as orc
+from paper_2410_13344_b200 import binding as cb
+from paper_2410_13344_b200 import synth
+from tests.helpers import close
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("M,N,K", [(1, 1, 1), (16, 16, 256), (17, 33, 255), (5, 700, 257), (64, 1024, 688), (3, 40, 2050),
+                                   (1024, 1184, 64)])      # 296 tiles of 64 x 64: the first size that stays on the large kernel
+def test_gemm_matches_definition(M, N, K):
+    X = synth.normal(13, 1, (M, K), 1.0, dtype=torch.float32, device="cuda")
+    W = synth.normal(13, 2, (N, K), 0.05, dtype=torch.float32, device="cuda")
+    # products and sums in fp32: sqrt(K) * 2^-24 of the terms' size
+    assert close(cb.gemm(X, W), orc.linear(X.cpu(), W.cpu()), 0) < 1e-5
