@@ -2,6 +2,8 @@
 // embedding gather, RMSNorm, RoPE + KV-page append, residual add, SwiGLU, row argmax.
 // GEMM outputs arrive as fp32 split-K partial sums [split][row][col]; every consumer here
 // adds the splits in index order, so results do not depend on scheduling.
+#include <type_traits>
+
 #include "cerb_internal.cuh"
 
 namespace cerb {
@@ -141,6 +143,61 @@ __global__ void __launch_bounds__(NORM_THREADS) fused_norm_kernel(float* __restr
       float ov[4];
 #pragma unroll
       for (int e = 0; e < 4; ++e) ov[e] = keep[it][e] * r * gv[it][e];
+      st4(o + j, ov);
+    }
+  }
+}
+
+// The same for many rows without slots (more than 128 rows: the GEMMs add to the residual stream themselves): memory-bound,
+// eight CTAs of 256 threads to an SM.  (One 1024-thread CTA per SM and row: 33 us for 2048 rows of 4096 where the bytes take 8.)
+constexpr int ROWS_THREADS = 256;
+template <typename T, int ITER>
+__global__ void __launch_bounds__(ROWS_THREADS) row_norm_kernel(float* __restrict__ x, const T* __restrict__ embed, const int32_t* __restrict__ tok,
+                                                                int tok_stride, int tok_off, const int32_t* __restrict__ n_active, int n, int V,
+                                                                const T* __restrict__ gain, T* __restrict__ out, int d, float eps,
+                                                                const int32_t* __restrict__ row_off, int B) {
+  __shared__ float red[32];
+  const int row = blockIdx.x;
+  griddep_wait();
+  griddep_launch();
+  float* xr = x + (size_t)row * d;
+  const T* src = nullptr;
+  if (embed) {
+    int b, v, t = 0;
+    locate_row(row, row_off, B, n, b, v);
+    if (v < n_active[b]) t = tok[(size_t)b * tok_stride + tok_off + v];
+    if (t < 0 || t >= V) t = 0;
+    src = embed + (size_t)t * d;
+  }
+  float v[ITER][4];
+#pragma unroll
+  for (int it = 0; it < ITER; ++it) {
+    const int j = (it * ROWS_THREADS + threadIdx.x) * 4;
+    v[it][0] = v[it][1] = v[it][2] = v[it][3] = 0.f;
+    if (j < d) {
+      if (src) ld4(src + j, v[it]);
+      else ld4(xr + j, v[it]);
+    }
+  }
+  float ss = 0.f;
+#pragma unroll
+  for (int it = 0; it < ITER; ++it) {
+    const int j = (it * ROWS_THREADS + threadIdx.x) * 4;
+    if (src && j < d) st4(xr + j, v[it]);
+#pragma unroll
+    for (int e = 0; e < 4; ++e) ss += v[it][e] * v[it][e];
+  }
+  ss = block_sum(ss, red);
+  const float r = 1.0f / sqrtf(ss / (float)d + eps);
+  T* o = out + (size_t)row * d;
+#pragma unroll
+  for (int it = 0; it < ITER; ++it) {
+    const int j = (it * ROWS_THREADS + threadIdx.x) * 4;
+    if (j < d) {
+      float g[4], ov[4];
+      ld4(gain + j, g);
+#pragma unroll
+      for (int e = 0; e < 4; ++e) ov[e] = v[it][e] * r * g[e];
       st4(o + j, ov);
     }
   }
@@ -317,7 +374,16 @@ int launch_fused_norm(cerb_ctx* c, const float* part, int nsplit, size_t split_s
   const cerb_config& g = c->cfg;
   const int d = g.d_model;
   if (d % 4 || d > NORM_THREADS * NORM_MAX_ITER * 4) return CERB_E_SHAPE;
-  if (c->bf16)
+  if (c->bf16 && nsplit == 0 && rows > 128 && out) {
+    auto wide = [&](auto iter) {
+      launch_pdl(row_norm_kernel<bf16, decltype(iter)::value>, dim3(rows), dim3(ROWS_THREADS), 0, st, (float*)c->d_x,
+                 tok ? (const bf16*)c->embed : (const bf16*)nullptr, tok, tok_stride, tok_off, (const int32_t*)c->d_nactive, n, g.vocab,
+                 (const bf16*)gain, (bf16*)out, d, g.rms_eps, row_off, c->B);
+    };
+    if (d <= 4096) wide(std::integral_constant<int, 4>());
+    else if (d <= 8192) wide(std::integral_constant<int, 8>());
+    else wide(std::integral_constant<int, 16>());
+  } else if (c->bf16)
     launch_pdl(fused_norm_kernel<bf16>, dim3(rows), dim3(NORM_THREADS), 0, st, (float*)c->d_x, part, nsplit, split_stride,
                tok ? (const bf16*)c->embed : (const bf16*)nullptr, tok, tok_stride, tok_off, (const int32_t*)c->d_nactive, n,
                g.vocab, (const bf16*)gain, (bf16*)out, d, g.rms_eps, row_off, c->B, x_fresh ? 1 : 0);

@@ -39,6 +39,8 @@ CASES = {
     "rope, swiglu, 160-row chunks": (synth.ModelShape(2, 256, 25, 128, 4752, 512, "bf16"), (170, 129)),
     "swiglu (head_dim 64)": (synth.ModelShape(1, 256, 50, 64, 4752, 512, "bf16"), (300,)),
     "rope": (synth.ModelShape(1, 256, 25, 128, 688, 512, "bf16"), (290,)),
+    "norm of 4104 columns": (synth.ModelShape(1, 4104, 2, 128, 64, 512, "bf16"), (140,)),      # beyond four pieces per thread
+    "norm of 8200 columns": (synth.ModelShape(1, 8200, 2, 128, 64, 512, "bf16"), (131,)),      # beyond eight
     "residual": (synth.ModelShape(1, 2560, 4, 128, 688, 512, "bf16"), (1800,)),
 }
 
