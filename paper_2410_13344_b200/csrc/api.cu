@@ -610,8 +610,9 @@ int cerb_prefill(cerb_ctx* c, const int32_t* tokens_dev, const int32_t* lens_hos
   CERB_CUDA_OK(cudaStreamSynchronize(st));
   for (int b = 0; b < B; ++b) c->h_stage[b] = lens_host[b];
   CERB_CUDA_OK(cudaMemcpyAsync(c->d_lens_in, c->h_stage, B * sizeof(int32_t), cudaMemcpyHostToDevice, st));
-  // Every forward takes the next C tokens of each prompt (fewer where a prompt ends), C the largest multiple of 128 whose
-  // live tokens fit a forward; only live tokens have rows.
+  // Every forward takes the next C tokens of each prompt (fewer where a prompt ends), C a multiple of 128; only live tokens
+  // have rows.  As few forwards as the rows allow, and then about equally many rows in each: a forward of few rows costs
+  // its weight stream whatever it computes.
   for (int off = 0, C; off < longest; off += C) {
     int need[CERB_MAX_BATCH], rows = 0;
     auto take = [&](int chunk) {
@@ -627,6 +628,14 @@ int cerb_prefill(cerb_ctx* c, const int32_t* tokens_dev, const int32_t* lens_hos
       take(more);
       if (rows > c->Mmax) break;
       C = more;
+    }
+    take(longest - off);
+    const int forwards = (rows + c->Mmax - 1) / c->Mmax, all = rows;
+    // (the first chunk holds the most rows: the smallest one that leaves no more than an equal share per forward to the rest)
+    for (int less = C - kPrefillQuantum; less >= kPrefillQuantum; less -= kPrefillQuantum) {
+      take(less);
+      if ((all - rows) > (long long)(forwards - 1) * c->Mmax || rows * forwards < all) break;
+      C = less;
     }
     if (C > longest - off) C = longest - off;
     take(C);

@@ -14,10 +14,10 @@ SHAPES = {"fp32": synth.tiny_shape("fp32"), "bf16 head_dim 64": synth.tiny_shape
           "bf16 head_dim 128": synth.ModelShape(2, 256, 2, 128, 512, 1024, "bf16")}
 
 
-# a window edge on both sides; one row and several forwards beside each other (the forward holds 2048 rows: 2049 tokens
-# leave one for the second, and three prompts of unequal length share it); a whole forward of 16 sequences
+# a window edge on both sides; a chunk that ends one token into a window; prompts of unequal length in one forward; a whole
+# forward of 16 sequences; two forwards of about equal size (a forward holds 4096 rows)
 @pytest.mark.parametrize("shape", list(SHAPES))
-@pytest.mark.parametrize("lens", [(127, 1, 129), (128, 256, 255), (2049,), (1300, 5, 900), tuple(range(131, 147))],
+@pytest.mark.parametrize("lens", [(127, 1, 129), (128, 256, 255), (2049,), (1300, 5, 900), tuple(range(131, 147)), (2100, 1999, 40)],
                          ids=lambda l: "-".join(map(str, l[:3])))
 def test_prefill_matches_oracle(shape, lens):
     ms = SHAPES[shape]
