@@ -50,13 +50,14 @@ constexpr int MAX_STAGES = 8;
 constexpr int TILE_X = kGemmRowsPerPass;                   // activation rows of a tile at most
 constexpr uint32_t A_BYTES = 128 * BK * 2;
 constexpr int kPairs = 74;
-constexpr int kEpiWarps = 8;                               // two per 32 tensor-memory lanes, taking 32-column blocks in turn
+constexpr int COLS = 16;                                   // columns an epilogue warp takes at a time
+constexpr int kEpiWarps = 16;                              // four per 32 tensor-memory lanes
 constexpr int kThreads = 64 + 32 * kEpiWarps;
 
 struct TileParams {
   float* out;               // KIND 0: [M][N]; KIND 3: the residual stream [M][N]
   float* fix;               // [pair][tail, head of a split tile][CTA][accumulator][column / 4][128 lanes][4]; S > 1: no heads
-  unsigned int* tickets;    // [split tile][CTA][accumulator][epilogue warp], zero on entry and on exit
+  unsigned int* tickets;    // [split tile][CTA][epilogue warp], zero on entry and on exit
   bf16* act;                // KIND 1: [M][F]
   RopeEpilogue re;          // KIND 2
   int32_t* status;
@@ -123,36 +124,38 @@ __device__ __forceinline__ void load_weights(uint32_t dst, const CUtensorMap* ma
     tma_load_2d_pair(dst, map, x, unit * 128, bar, pol);
 }
 
-// Finishes 32 columns (activation rows row0 + c0 ...) of one accumulator lane.  Everything is computed before anything is
-// stored: with the bounds checks of the stores in between, each column's chain of latencies came after the last one's
-// (QKV of the 7B shape at 512 rows: 103 us, and 58 this way with eight epilogue warps instead of four).
+// Finishes 16 columns (activation rows row0 + c0 ...) of one accumulator lane.  What an epilogue costs is latency: everything
+// is computed before anything is stored (with the bounds checks of the stores in between, each column's chain came after the
+// last one's: QKV of the 7B shape at 512 rows 103 us instead of 58), and sixteen warps with 16 columns each take turns
+// (eight with 32: 22 us for the two accumulators of a 512-row SwiGLU tile whose MMAs take 37).
 template <int KIND>
 __device__ __forceinline__ void finish(const TileParams& p, const float* v, int unit, int quarter, int lane, int row0, int c0,
                                        const int* pos_s, const int* kv_s) {
-  const int left = min(32, min(p.n_act - c0, p.M - row0 - c0));            // live columns
+  const int left = min(COLS, min(p.n_act - c0, p.M - row0 - c0));          // live columns
   if constexpr (KIND == 0 || KIND == 3) {
     const int n_out = unit * 128 + quarter * 32 + lane;
     if (n_out >= p.N) return;
     float* o = p.out + (size_t)(row0 + c0) * p.N + n_out;     // (consecutive lanes: consecutive columns of a row)
-    float x[32];
+    float x[COLS];
 #pragma unroll
-    for (int j = 0; j < 32; ++j) x[j] = KIND == 3 && j < left ? o[(size_t)j * p.N] : 0.f;
-    if (left == 32) {
+    for (int j = 0; j < COLS; ++j) x[j] = KIND == 3 && j < left ? o[(size_t)j * p.N] : 0.f;
+    if (left == COLS) {
 #pragma unroll
-      for (int j = 0; j < 32; ++j) o[(size_t)j * p.N] = KIND == 3 ? x[j] + v[j] : v[j];
+      for (int j = 0; j < COLS; ++j) o[(size_t)j * p.N] = KIND == 3 ? x[j] + v[j] : v[j];
     } else {
 #pragma unroll
-      for (int j = 0; j < 32; ++j)
+      for (int j = 0; j < COLS; ++j)
         if (j < left) o[(size_t)j * p.N] = KIND == 3 ? x[j] + v[j] : v[j];
     }
   } else {
+    constexpr int P = COLS / 2;
     const int hi = lane >> 4;
     const int i = quarter * 16 + (lane & 15);                               // feature / rotation index inside the unit
     // lanes 0-15 hold the first member of each pair (gate; element i), lanes 16-31 the second (up; element i + 64):
     // the lower half of the warp finishes column 2 j, the upper half column 2 j + 1
-    float a[16], b[16];
+    float a[P], b[P];
 #pragma unroll
-    for (int j = 0; j < 16; ++j) {
+    for (int j = 0; j < P; ++j) {
       const float got = __shfl_xor_sync(0xffffffffu, hi ? v[2 * j] : v[2 * j + 1], 16);
       a[j] = hi ? got : v[2 * j];
       b[j] = hi ? v[2 * j + 1] : got;
@@ -160,27 +163,27 @@ __device__ __forceinline__ void finish(const TileParams& p, const float* v, int 
     if constexpr (KIND == 1) {
       const int f = unit * 64 + i;
 #pragma unroll
-      for (int j = 0; j < 16; ++j) a[j] = a[j] / (1.0f + expf(-a[j])) * b[j];
+      for (int j = 0; j < P; ++j) a[j] = a[j] / (1.0f + expf(-a[j])) * b[j];
       if (f >= p.F) return;
       bf16* o = p.act + (size_t)(row0 + c0 + hi) * p.F + f;
 #pragma unroll
-      for (int j = 0; j < 16; ++j)
+      for (int j = 0; j < P; ++j)
         if (2 * j + hi < left) o[(size_t)(2 * j) * p.F] = __float2bfloat16_rn(a[j]);
     } else {
       if (unit >= 3 * p.re.H) return;
       const int which = unit / p.re.H, h = unit - which * p.re.H;
-      int kv[16];
+      int kv[P];
 #pragma unroll
-      for (int j = 0; j < 16; ++j) kv[j] = 2 * j + hi < left ? kv_s[c0 + 2 * j + hi] : -1;
+      for (int j = 0; j < P; ++j) kv[j] = 2 * j + hi < left ? kv_s[c0 + 2 * j + hi] : -1;
       if (which < 2) {
-        float2 cs[16];
+        float2 cs[P];
 #pragma unroll
-        for (int j = 0; j < 16; ++j) {
+        for (int j = 0; j < P; ++j) {
           const int pos = pos_s[c0 + 2 * j + hi];
           cs[j] = p.re.rope[(size_t)(pos < 0 ? 0 : pos) * 64 + i];
         }
 #pragma unroll
-        for (int j = 0; j < 16; ++j) {
+        for (int j = 0; j < P; ++j) {
           const float o1 = a[j] * cs[j].x - b[j] * cs[j].y;
           b[j] = b[j] * cs[j].x + a[j] * cs[j].y;
           a[j] = o1;
@@ -189,7 +192,7 @@ __device__ __forceinline__ void finish(const TileParams& p, const float* v, int 
       bf16* q = reinterpret_cast<bf16*>(p.re.q) + ((size_t)(row0 + c0 + hi) * p.re.H + h) * 128 + i;
       bf16* pool = reinterpret_cast<bf16*>(which == 1 ? p.re.kpool : p.re.vpool) + (size_t)h * CERB_PAGE * 128 + i;
 #pragma unroll
-      for (int j = 0; j < 16; ++j) {
+      for (int j = 0; j < P; ++j) {
         bf16* o = which == 0 ? q + (size_t)(2 * j) * p.re.H * 128 : pool + (size_t)kv[j] * 128;
         if (kv[j] >= 0) {
           o[0] = __float2bfloat16_rn(a[j]);
@@ -223,22 +226,21 @@ __device__ __forceinline__ bool wait_fix(const unsigned int* ticket, unsigned in
   return false;
 }
 
-__device__ __forceinline__ void ld_acc32(uint32_t taddr, float* v) {
+__device__ __forceinline__ void ld_acc(uint32_t taddr, float* v) {
   tmem_ld16_nowait(taddr, reinterpret_cast<uint32_t*>(v));
-  tmem_ld16_nowait(taddr + 16u, reinterpret_cast<uint32_t*>(v + 16));
   tmem_ld_wait();
 }
 __device__ __forceinline__ void put_fix(float4* at, const float* v) {
 #pragma unroll
-  for (int j = 0; j < 8; ++j) __stcg(at + j * 128, make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]));
+  for (int j = 0; j < COLS / 4; ++j) __stcg(at + j * 128, make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]));
 }
 __device__ __forceinline__ void get_fix(const float4* at, float4* o) {
 #pragma unroll
-  for (int j = 0; j < 8; ++j) o[j] = __ldcg(at + j * 128);
+  for (int j = 0; j < COLS / 4; ++j) o[j] = __ldcg(at + j * 128);
 }
 __device__ __forceinline__ void add(const float4* o, float* v) {
 #pragma unroll
-  for (int j = 0; j < 8; ++j) { v[4 * j] += o[j].x; v[4 * j + 1] += o[j].y; v[4 * j + 2] += o[j].z; v[4 * j + 3] += o[j].w; }
+  for (int j = 0; j < COLS / 4; ++j) { v[4 * j] += o[j].x; v[4 * j + 1] += o[j].y; v[4 * j + 2] += o[j].z; v[4 * j + 3] += o[j].w; }
 }
 
 template <int KIND, int HF>
@@ -271,7 +273,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tile_kernel(const __grid_con
     }
     for (int i = 0; i < 2; ++i) {
       mbar_init(smem_u32(&acc_full[i]), 1);
-      mbar_init(smem_u32(&acc_empty[i]), 2 * kEpiWarps);
+      mbar_init(smem_u32(&acc_empty[i]), 2 * kEpiWarps / HF);
     }
     mbar_init(smem_u32(&drain_bar), 1);
     mbar_init(smem_u32(&meet_bar), 2);
@@ -418,7 +420,11 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tile_kernel(const __grid_con
     }
   } else {
     const int quarter = warp & 3;                    // tensor-memory lanes 32 * quarter .. + 31 belong to this warp
-    const int ew = warp - 2, half = ew >> 2;         // columns: 32-column blocks half, half + 2, ...
+    const int ew = warp - 2;
+    // which blocks of columns: HF = 1: every fourth; HF = 2: of the first or of the second accumulator, every second
+    const int hf = HF == 2 ? ew >> 3 : 0;
+    const int c_first = (HF == 2 ? (ew >> 2) & 1 : ew >> 2) * COLS;
+    constexpr int C_STEP = HF == 2 ? 2 * COLS : 4 * COLS;
     const int et = quarter * 32 + lane;
     griddep_wait();                                  // the kernels before this one may still be reading what this one writes
     const uint32_t ae[2] = {mapa_u32(smem_u32(&acc_empty[0]), 0), mapa_u32(smem_u32(&acc_empty[1]), 0)};
@@ -432,7 +438,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tile_kernel(const __grid_con
       const int chunk = r.tile % p.mchunks, row0 = chunk * p.n_act;
       if (KIND == 2 && chunk != chunk_known) {
         // positions and cache rows of the chunk's activation rows
-        asm volatile("bar.sync 2, 256;" ::: "memory");                       // (the previous tile's readers are done)
+        asm volatile("bar.sync 2, 512;" ::: "memory");                       // (the previous tile's readers are done)
         const RopeEpilogue& e = p.re;
         for (int c = ew * 32 + lane; c < TILE_X; c += 32 * kEpiWarps) {
           int pos = -1, kv = -1;
@@ -448,7 +454,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tile_kernel(const __grid_con
           pos_s[c] = pos;
           kv_s[c] = kv;
         }
-        asm volatile("bar.sync 2, 256;" ::: "memory");
+        asm volatile("bar.sync 2, 512;" ::: "memory");
         chunk_known = chunk;
       }
       int first_share = pair, last_share = pair;
@@ -457,8 +463,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tile_kernel(const __grid_con
         last_share = (r.tile * p.num_kb + p.num_kb - 1) / p.per;
       }
       const bool split = last_share > first_share;                          // (two pairs: the first has the tile's head)
-#pragma unroll 1
-      for (int hf = 0; hf < HF; ++hf) {
+      {
         const bool two = HF == 1 && p.chains == 2;
         const int acc = HF == 2 ? hf : two ? 0 : g & 1;
         const uint32_t full_ph = (uint32_t)(HF == 2 || two ? g : g >> 1) & 1u;
@@ -468,15 +473,15 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tile_kernel(const __grid_con
         tc_fence_after();
         const uint32_t taddr = tmem_base + (uint32_t)(acc * TILE_X) + ((uint32_t)(quarter * 32) << 16);
         auto read_acc = [&](int c0, float* v) {
-          ld_acc32(taddr + (uint32_t)c0, v);
+          ld_acc(taddr + (uint32_t)c0, v);
           if (two && r.nkb > 1) {
-            float t[32];
-            ld_acc32(taddr + (uint32_t)(TILE_X + c0), t);
+            float t[COLS];
+            ld_acc(taddr + (uint32_t)(TILE_X + c0), t);
 #pragma unroll
-            for (int j = 0; j < 32; ++j) v[j] += t[j];
+            for (int j = 0; j < COLS; ++j) v[j] += t[j];
           }
         };
-        unsigned int* ticket = p.tickets + (((size_t)r.tile * 2 + rank) * HF + hf) * kEpiWarps + ew;
+        unsigned int* ticket = p.tickets + ((size_t)r.tile * 2 + rank) * kEpiWarps + ew;
         constexpr size_t kFixAcc = 128 * TILE_X / 4;       // float4s of one CTA's accumulator
         float4* fix = reinterpret_cast<float4*>(p.fix) + et;
         auto at = [&](int who, int c0) { return fix + (((size_t)who * 2 + rank) * HF + hf) * kFixAcc + (size_t)(c0 >> 2) * 128; };
@@ -485,9 +490,9 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tile_kernel(const __grid_con
           // 64-column groups of the tile's accumulators belong to the pairs in turn
           auto owner = [&](int c0) { return (hf * 4 + (c0 >> 6)) % p.S; };
           if (live)
-            for (int c0 = half * 32; c0 < p.n_act; c0 += 64)
+            for (int c0 = c_first; c0 < p.n_act; c0 += C_STEP)
               if (owner(c0) != self) {
-                float v[32];
+                float v[COLS];
                 read_acc(c0, v);
                 put_fix(at(pair, c0), v);
               }
@@ -498,13 +503,13 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tile_kernel(const __grid_con
           live = __all_sync(0xffffffffu, live);
           __threadfence();
           if (live)
-            for (int c0 = half * 32; c0 < p.n_act; c0 += 64)
+            for (int c0 = c_first; c0 < p.n_act; c0 += C_STEP)
               if (owner(c0) == self) {
-                float v[32];
+                float v[COLS];
 #pragma unroll
-                for (int j = 0; j < 32; ++j) v[j] = 0.f;
+                for (int j = 0; j < COLS; ++j) v[j] = 0.f;
                 for (int s = 0; s < p.S; ++s) {               // k order
-                  float4 o[8];
+                  float4 o[COLS / 4];
                   if (s == self) read_acc(c0, reinterpret_cast<float*>(o));
                   else get_fix(at(base + s, c0), o);
                   add(o, v);
@@ -530,9 +535,9 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tile_kernel(const __grid_con
             if (!leave) __threadfence();
           }
           if (live)
-            for (int c0 = half * 32; c0 < p.n_act; c0 += 64) {
-              float v[32];
-              float4 o[8];
+            for (int c0 = c_first; c0 < p.n_act; c0 += C_STEP) {
+              float v[COLS];
+              float4 o[COLS / 4];
               if (split && !leave) get_fix(at(other, c0), o);
               read_acc(c0, v);
               if (leave) {
@@ -661,7 +666,7 @@ int launch_gemm_tile(cerb_ctx* c, const CUtensorMap* tmW, const ActMaps* tmX, co
   const int kind = epi ? epi->kind : 0;
   if (g.tiles * g.num_kb >= (1ll << 30)) return CERB_E_SHAPE;
   if (g.fix_floats && (!fix || !tickets)) return CERB_E_ARG;
-  static_assert(2 * kPairs * 2 * 2 * kEpiWarps <= kGemmTickets, "one counter per accumulator and epilogue warp of every split tile");
+  static_assert(2 * kPairs * 2 * kEpiWarps <= kGemmTickets, "one counter per epilogue warp of every split tile");
   TileParams q;
   memset(&q, 0, sizeof(q));
   q.out = kind == 3 ? epi->x : out;
