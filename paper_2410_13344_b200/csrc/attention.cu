@@ -490,13 +490,13 @@ __global__ void __launch_bounds__((WQ * WK + 1) * 32) tree_attn_bf16_kernel(cons
 // Same decomposition as above (one CTA per (split, head, sequence), 64-key tiles streamed by TMA),
 // but both products run as tcgen05 MMAs with their results in tensor memory:
 //   S[128 x 64]  = Q[128 x 128] . K_tile^T      (Q staged once in shared memory, zero rows past n)
-//   O[128 x 128] += P[128 x 64] . V_tile        (P = p_hi + p_lo, two bf16 terms, staged in shared memory)
-// Warp 0 = TMA producer, warp 1 = TMEM allocator + MMA issuer, warps 2-5 and 6-9 = two softmax groups
+//   O[128 x 128] += P[128 x 64] . V_tile        (P = p_hi + p_lo, two bf16 terms, left in tensor memory as the A operand)
+// Warps 0 and 11 = TMA producers of K and V, warp 1 = TMEM allocator and QK^T issuer, warp 10 = PV issuer, warps 2-5 and 6-9 = two softmax groups
 // that take alternate key tiles.  In a group thread t owns query row t (= TMEM lane t): it reads its
 // whole S row from tensor memory with back-to-back loads and ONE wait (a dependent TMEM round trip
 // costs ~600 cycles here, measured), keeps the running maximum and sum in registers and writes its P
-// row (128-byte swizzled, the MMA's K-major A layout).  Each group has its own S buffer, its own O
-// accumulator and its own P buffers, i.e. the two groups run two independent online-softmax streams
+// row back to tensor memory (two bf16 of neighbouring keys per column: 32 columns per term).  Each group has its own S
+// buffer, its own O accumulator and its own P buffer (64 + 128 + 64 columns, twice: all 512), i.e. the two groups run two independent online-softmax streams
 // over the even and the odd tiles, merged once at the end; one group's TMEM latency and arithmetic
 // overlap the other's.  O stays in TMEM across tiles; it is only rescaled when a row's maximum grows
 // by more than 2^8 (until then the older maximum keeps being used, which is exact after the final
@@ -504,22 +504,18 @@ __global__ void __launch_bounds__((WQ * WK + 1) * 32) tree_attn_bf16_kernel(cons
 namespace {
 
 constexpr uint32_t TC_KV_BYTES = 16384;               // K (or V) of one 64-key tile, two 64-wide halves
-// K and V tiles travel through rings of 16 KB stages.  The depth of the rings, not HBM, sets the tile rate
-// up to the point where the tensor pipe is busy (a freed stage is back after a TMA round trip of ~2 us;
-// measured at 64 nodes: three K+V stages 1.36 us per 64-key tile, four or five 1.0 us).
-//  * Trees of up to 64 nodes keep only 64 rows of Q and of every P buffer in shared memory (the MMAs still
-//    read 128 rows; what they find past the 64th only reaches score and output rows nobody uses), which
-//    leaves room for five K and five V stages; K and V of a tile then share one pair of barriers (UNI).
-//  * Wider trees need all 128 rows: two K and five V stages with barriers of their own -- a K tile is
-//    free again as soon as its QK^T MMAs have retired, a V tile only after the PV MMAs one softmax later.
+// K and V tiles travel through rings of 16 KB stages with barriers of their own: a K tile is free again as soon as its QK^T
+// MMAs have retired, a V tile only after the PV MMAs one softmax later.  The depth of the rings sets the tile rate up to the
+// point where the tensor pipe is busy (a freed stage is back after a TMA round trip of ~2 us): with P in shared memory (64 KB)
+// there was room for two K and five V stages: 611 us at batch 16 x 128 nodes x 8K keys, 572 this way.
 // (One QK^T MMA set of N = 128 over two neighbouring key tiles, filling both groups' score buffers at
 // once, was tried: 24 instead of 32 MMAs per 128 keys, but the groups then run in lockstep and lose
 // their overlap -- 692 against 529 us at batch 16 x 64 nodes x 8K keys.)
-__host__ __device__ constexpr size_t tc_smem(int sk, int sv, int qrows) {
-  return (size_t)(sk + sv) * TC_KV_BYTES + 2 * (size_t)qrows * 128 + 4 * (size_t)qrows * 128 + 1024;   // rings, Q, P (2 groups x hi, lo)
-}
+constexpr int TC_SK = 5, TC_SV = 6;
+constexpr size_t TC_SMEM = (size_t)(TC_SK + TC_SV) * TC_KV_BYTES + 32768 + 1024;   // rings, Q, alignment slack
+static_assert(TC_SMEM - 1024 >= 2 * 128 * (128 + 4) * 4, "both groups' rows fit when the key loop is over");
 constexpr int TC_DH = 128, TC_ROWF = TC_DH + 4;
-constexpr int TC_THREADS = 352;                       // producer, QK^T issuer, two softmax groups of four warps, PV issuer
+constexpr int TC_THREADS = 384;                       // K producer, QK^T issuer, two softmax groups of four warps, PV issuer, V producer
 constexpr float TC_RESCALE = 8.0f;                    // log2 of the growth of a row maximum that forces a rescale
 
 __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t* r) { tmem_ld16_nowait(taddr, r); }
@@ -527,12 +523,11 @@ __device__ __forceinline__ void umma(uint32_t tmem_d, uint64_t adesc, uint64_t b
   umma_bf16(tmem_d, adesc, bdesc, idesc, acc);
 }
 
-template <int SK, int SV, int QROWS, bool UNI>
 __global__ void __launch_bounds__(TC_THREADS, 1) tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmK,
                                                                      const __grid_constant__ CUtensorMap tmV, const AttnParams p) {
   constexpr int DH = TC_DH, ROWF = TC_ROWF;
-  constexpr uint32_t QHALF = (uint32_t)QROWS * 128u, TC_Q_BYTES = 2 * QHALF;
-  constexpr uint32_t TC_P_BYTES = (uint32_t)QROWS * 128u;      // P: one term (hi or lo) of one softmax group
+  constexpr int SK = TC_SK, SV = TC_SV;
+  constexpr uint32_t QHALF = 128u * 128u, TC_Q_BYTES = 2 * QHALF;
   extern __shared__ uint8_t smem_raw[];
   __shared__ __align__(8) uint64_t full_k[SK], empty_k[SK], full_v[SV], empty_v[SV], s_full[2], s_free[2], p_ready[2], pv_done[2], q_ready, drain_bar[2];
   __shared__ int page_list[kMaxPagesPerCta];
@@ -548,11 +543,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tree_attn_tc_kernel(const __gri
   // keys.  Set-up, the page list and the first prefix tiles thus overlap the previous kernel's tail.
   const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
   uint8_t* smem_gen = smem_raw + (smem_base - smem_u32(smem_raw));
-  // Order matters: with 64-row buffers the 128-row MMAs read 8 KB past the end of a P buffer and of Q's
-  // second half; P comes first, then Q, then the rings, so that every such read stays inside this CTA's
-  // shared memory (the last P buffer runs into Q, Q into the K ring).
-  const uint32_t p_base = smem_base;                    // [group][hi, lo] x TC_P_BYTES
-  const uint32_t q_base = p_base + 4 * TC_P_BYTES;
+  const uint32_t q_base = smem_base;
   const uint32_t k_ring = q_base + TC_Q_BYTES;
   const uint32_t v_ring = k_ring + SK * TC_KV_BYTES;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -605,89 +596,54 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tree_attn_tc_kernel(const __gri
   __syncthreads();
   tc_fence_after();
   if (p.cluster) cluster_start_arrive();
-  // tensor memory: columns 0-63 / 64-127 = S of group 0 / 1, 128-255 / 256-383 = O of group 0 / 1
+  // tensor memory: columns 0-63 / 64-127 = S of group 0 / 1, 128-255 / 256-383 = O, 384-447 / 448-511 = P (hi, lo)
   const uint32_t tmem = tmem_slot;
   float* mrg = reinterpret_cast<float*>(smem_gen);   // [2][128][ROWF] over the whole buffer, once the key loop is over
 
-  if (warp == 0) {
-    // ---------------- TMA producer ----------------
+  if (warp == 0 || warp == 11) {
+    // ---------------- TMA producers: warp 0 the K tiles, warp 11 the V tiles ----------------
+    // A tile of K (or V) is 8 boxes of 2 KB (four pages, two 64-wide halves), issued by 8 lanes.  Issuing a box occupies its
+    // warp for ~88 cycles, so one warp for both made 1400 cycles and more of every tile, the kernel's pace (572 us at batch 16 x 128 nodes x 8K keys, 465 with two).
+    const bool is_v = warp == 11;
     const int32_t* pt = p.page_table + (size_t)b * p.max_pages;
     const int n_pages = T * PAGES_PER_TILE;
-    for (int i = lane; i < n_pages; i += 32) {
+    for (int i = lane + (is_v ? 32 : 0); i < n_pages; i += 64) {
       int lp = t0 * PAGES_PER_TILE + i;
       page_list[i] = (lp * CERB_PAGE < kv_total && lp < p.max_pages) ? (pt[lp] * p.H + h) * CERB_PAGE : p.oob_row;
     }
-    __syncwarp();
+    asm volatile("bar.sync 3, 64;" ::: "memory");      // the page list is complete
+    const int ring = is_v ? SV : SK;
+    uint64_t* full = is_v ? full_v : full_k;
+    uint64_t* empty = is_v ? empty_v : empty_k;
+    const uint32_t base = is_v ? v_ring : k_ring;
     // tiles of the first ring that lie wholly inside the prefix may be fetched before the wait
     int early = 0;
-    while (early < T && early < SK && (t0 + early + 1) * TILE <= L_old) ++early;
-    if constexpr (!UNI) {
-      // A tile is 16 boxes of 2 KB (K and V, four pages, two 64-wide halves).  With separate K and V rings
-      // (128 query rows) 16 lanes issue one box each: 4-7 % faster than one lane issuing them in turn
-      // (measured, 16 x 8192 and 4 x 4096 keys); with the shared ring it is 1-5 % slower, hence the other branch.
-      static_assert(PAGES_PER_TILE == 4, "the lane -> box map below assumes four pages per tile");
-      const int is_v = lane >> 3, pg = (lane >> 1) & 3, hf = lane & 1;
-      const int T_stop = *aborted ? 0 : T;         // a launch that starts after a time-out issues nothing
-      int i = 0;
-      for (; i < T_stop; ++i) {
-        if (i == early) { griddep_wait(); griddep_launch(); }
-        const int sk = i % SK, sv = i % SV;
-        const uint32_t fk = smem_u32(&full_k[sk]), fv = smem_u32(&full_v[sv]);
-        int stop = 0;
-        if (lane == 0) {
-          // (a wait that gives up says so in its return value: the consumers have stopped, nothing more is issued)
-          if (mbar_wait_polite(smem_u32(&empty_k[sk]), ((uint32_t)(i / SK) & 1u) ^ 1u, wc, 305) &&
-              mbar_wait_polite(smem_u32(&empty_v[sv]), ((uint32_t)(i / SV) & 1u) ^ 1u, wc, 306)) {
-            mbar_expect_tx(fk, TC_KV_BYTES);
-            mbar_expect_tx(fv, TC_KV_BYTES);
-          } else {
-            stop = 1;
-          }
-        }
-        if (__any_sync(0xffffffffu, stop)) break;
-        if (lane < 16) {
-          const int row = page_list[i * PAGES_PER_TILE + pg];       // out-of-range rows are zero-filled by TMA
-          const uint32_t dst = (is_v ? v_ring + (uint32_t)sv * TC_KV_BYTES : k_ring + (uint32_t)sk * TC_KV_BYTES) +
-                               (uint32_t)hf * 8192u + (uint32_t)pg * (CERB_PAGE * 128);
-          tma_load_2d(dst, is_v ? &tmV : &tmK, hf * 64, row, is_v ? fv : fk);
-        }
+    while (early < T && early < ring && (t0 + early + 1) * TILE <= L_old) ++early;
+    static_assert(PAGES_PER_TILE == 4, "the lane -> box map below assumes four pages per tile");
+    const int pg = (lane >> 1) & 3, hf = lane & 1;
+    const int T_stop = __any_sync(0xffffffffu, *aborted) ? 0 : T;         // a launch that starts after a time-out issues nothing
+    int i = 0, slot = 0;
+    uint32_t ph = 0;
+    for (; i < T_stop; ++i) {
+      if (i == early) { griddep_wait(); griddep_launch(); }
+      const uint32_t fb = smem_u32(&full[slot]);
+      int stop = 0;
+      if (lane == 0) {
+        // (a wait that gives up says so in its return value: the consumers have stopped, nothing more is issued)
+        stop = !mbar_wait_polite(smem_u32(&empty[slot]), ph ^ 1u, wc, is_v ? 306 : 305);
+        if (!stop) mbar_expect_tx(fb, TC_KV_BYTES);
       }
-      if (lane == 0 && *aborted) {
-        // give-up path: the copies already issued (tiles 0 .. i-1) still land in this CTA's shared memory; see each of them in
-        for (int j = i > SK ? i - SK : 0; j < i; ++j)
-          mbar_wait_drain(smem_u32(&full_k[j % SK]), (uint32_t)(j / SK) & 1u, 20000000ll);
-        for (int j = i > SV ? i - SV : 0; j < i; ++j)
-          mbar_wait_drain(smem_u32(&full_v[j % SV]), (uint32_t)(j / SV) & 1u, 20000000ll);
+      if (__any_sync(0xffffffffu, stop)) break;
+      if (lane < 8) {
+        const int row = page_list[i * PAGES_PER_TILE + pg];       // out-of-range rows are zero-filled by TMA
+        tma_load_2d(base + (uint32_t)slot * TC_KV_BYTES + (uint32_t)hf * 8192u + (uint32_t)pg * (CERB_PAGE * 128), is_v ? &tmV : &tmK, hf * 64, row, fb);
       }
-    } else if (lane == 0) {
-      // K and V of a tile share the V ring's barriers (SK == SV): one wait and one arrival per tile
-      const int T_stop = *aborted ? 0 : T;         // a launch that starts after a time-out issues nothing
-      int i = 0;
-      for (; i < T_stop; ++i) {
-        if (i == early) { griddep_wait(); griddep_launch(); }
-        const int sv = i % SV;
-        if (!mbar_wait_polite(smem_u32(&empty_v[sv]), ((uint32_t)(i / SV) & 1u) ^ 1u, wc, 307)) break;
-        const uint32_t fv = smem_u32(&full_v[sv]);
-        mbar_expect_tx(fv, 2 * TC_KV_BYTES);
-        const uint32_t kdst = k_ring + (uint32_t)sv * TC_KV_BYTES, vdst = v_ring + (uint32_t)sv * TC_KV_BYTES;
-#pragma unroll
-        for (int pg = 0; pg < PAGES_PER_TILE; ++pg) {
-          const int row = page_list[i * PAGES_PER_TILE + pg];       // out-of-range rows are zero-filled by TMA
-#pragma unroll
-          for (int hf = 0; hf < 2; ++hf)
-            tma_load_2d(kdst + (uint32_t)hf * 8192u + (uint32_t)pg * (CERB_PAGE * 128), &tmK, hf * 64, row, fv);
-        }
-#pragma unroll
-        for (int pg = 0; pg < PAGES_PER_TILE; ++pg) {
-          const int row = page_list[i * PAGES_PER_TILE + pg];
-#pragma unroll
-          for (int hf = 0; hf < 2; ++hf)
-            tma_load_2d(vdst + (uint32_t)hf * 8192u + (uint32_t)pg * (CERB_PAGE * 128), &tmV, hf * 64, row, fv);
-        }
-      }
-      if (*aborted)
-        for (int j = i > SV ? i - SV : 0; j < i; ++j)
-          mbar_wait_drain(smem_u32(&full_v[j % SV]), (uint32_t)(j / SV) & 1u, 20000000ll);
+      if (++slot == ring) { slot = 0; ph ^= 1u; }
+    }
+    if (lane == 0 && *aborted) {
+      // give-up path: the copies already issued (tiles 0 .. i-1) still land in this CTA's shared memory; see each of them in
+      for (int j = i > ring ? i - ring : 0; j < i; ++j)
+        mbar_wait_drain(smem_u32(&full[j % ring]), (uint32_t)(j / ring) & 1u, 20000000ll);
     }
     griddep_wait();      // (a lane that has waited already returns at once)
     griddep_launch();
@@ -697,28 +653,30 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tree_attn_tc_kernel(const __gri
     // ---------------- QK^T issuer ----------------
     // (issuing one tcgen05.mma costs this thread ~95 cycles whatever its size, measured, so the two
     // products are issued by two different warps)
-    if (lane == 0 && T > 0) {
+    if (T > 0) {
       const uint32_t idesc_s = (1u << 4) | (1u << 7) | (1u << 10) | ((64u >> 3) << 17) | ((128u >> 4) << 24);
       const uint64_t q_desc0 = desc_k_sw128(q_base), q_desc1 = desc_k_sw128(q_base + QHALF);
-      mbar_wait(smem_u32(&q_ready), 0, wc, 308);
-      const int T_stop = *aborted ? 0 : T;
+      mbar_wait_warp(smem_u32(&q_ready), 0, wc, 308);
+      const int T_stop = __any_sync(0xffffffffu, *aborted) ? 0 : T;
       for (int i = 0; i < T_stop; ++i) {
         const int g = i & 1, k = i >> 1;
-        const bool ok_kv = !UNI ? mbar_wait(smem_u32(&full_k[i % SK]), (uint32_t)(i / SK) & 1u, wc, 309)
-                                : mbar_wait(smem_u32(&full_v[i % SV]), (uint32_t)(i / SV) & 1u, wc, 310);
-        if (!mbar_wait(smem_u32(&s_free[g]), ((uint32_t)k & 1u) ^ 1u, wc, 311) || !ok_kv) break;
+        if (!mbar_wait_warp(smem_u32(&full_k[i % SK]), (uint32_t)(i / SK) & 1u, wc, 309)) break;
+        if (!mbar_wait_warp(smem_u32(&s_free[g]), ((uint32_t)k & 1u) ^ 1u, wc, 311)) break;
         tc_fence_after();
         const uint32_t kb = k_ring + (uint32_t)(i % SK) * TC_KV_BYTES;
         const uint64_t k_desc0 = desc_k_sw128(kb), k_desc1 = desc_k_sw128(kb + 8192u);
         const uint32_t d = tmem + (uint32_t)g * 64u;
+        if (elect_one()) {
 #pragma unroll
-        for (int kk = 0; kk < 4; ++kk) umma(d, q_desc0 + (uint64_t)(kk * 2), k_desc0 + (uint64_t)(kk * 2), idesc_s, kk ? 1u : 0u);
+          for (int kk = 0; kk < 4; ++kk) umma(d, q_desc0 + (uint64_t)(kk * 2), k_desc0 + (uint64_t)(kk * 2), idesc_s, kk ? 1u : 0u);
 #pragma unroll
-        for (int kk = 0; kk < 4; ++kk) umma(d, q_desc1 + (uint64_t)(kk * 2), k_desc1 + (uint64_t)(kk * 2), idesc_s, 1u);
-        if (!UNI) umma_commit(smem_u32(&empty_k[i % SK]));     // the K tile is free once these MMAs have retired
-        umma_commit(smem_u32(&s_full[g]));
+          for (int kk = 0; kk < 4; ++kk) umma(d, q_desc1 + (uint64_t)(kk * 2), k_desc1 + (uint64_t)(kk * 2), idesc_s, 1u);
+          umma_commit(smem_u32(&empty_k[i % SK]));     // the K tile is free once these MMAs have retired
+          umma_commit(smem_u32(&s_full[g]));
+        }
+        __syncwarp();
       }
-      if (*aborted) {                                // give-up path: see the MMAs already issued retire
+      if (__any_sync(0xffffffffu, *aborted) && elect_one()) {                                // give-up path: see the MMAs already issued retire
         umma_commit(smem_u32(&drain_bar[0]));
         mbar_wait_drain(smem_u32(&drain_bar[0]), 0, 20000000ll);
       }
@@ -727,28 +685,31 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tree_attn_tc_kernel(const __gri
     griddep_wait();
     griddep_launch();
     // ---------------- PV issuer ----------------
-    if (lane == 0) {
+    {
       // B operand (V) is MN-major, N = 128 (two 64-wide swizzle atoms, p.v_lbo bytes apart)
       const uint32_t idesc_pv = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 16) | ((128u >> 3) << 17) | ((128u >> 4) << 24);
-      const int T_stop = *aborted ? 0 : T;
+      const int T_stop = __any_sync(0xffffffffu, *aborted) ? 0 : T;
       for (int j = 0; j < T_stop; ++j) {
         const int g = j & 1, k = j >> 1;
-        if (!mbar_wait(smem_u32(&p_ready[g]), (uint32_t)k & 1u, wc, 312)) break;
-        if (!mbar_wait(smem_u32(&full_v[j % SV]), (uint32_t)(j / SV) & 1u, wc, 313)) break;
+        if (!mbar_wait_warp(smem_u32(&p_ready[g]), (uint32_t)k & 1u, wc, 312)) break;
+        if (!mbar_wait_warp(smem_u32(&full_v[j % SV]), (uint32_t)(j / SV) & 1u, wc, 313)) break;
         tc_fence_after();
         const uint32_t vb = v_ring + (uint32_t)(j % SV) * TC_KV_BYTES;
         const uint32_t d = tmem + 128u + (uint32_t)g * 128u;
-        const uint64_t ph = desc_k_sw128(p_base + (uint32_t)g * 2u * TC_P_BYTES), pl = desc_k_sw128(p_base + (uint32_t)g * 2u * TC_P_BYTES + TC_P_BYTES);
+        const uint32_t ph = tmem + 384u + (uint32_t)g * 64u, pl = ph + 32u;
+        if (elect_one()) {
 #pragma unroll
-        for (int ks = 0; ks < 4; ++ks) {
-          const uint64_t vd = desc_mn_sw128(vb + ks * 2048u, p.v_lbo, p.v_sbo);
-          umma(d, ph + (uint64_t)(ks * 2), vd, idesc_pv, (k == 0 && ks == 0) ? 0u : 1u);
-          umma(d, pl + (uint64_t)(ks * 2), vd, idesc_pv, 1u);
+          for (int ks = 0; ks < 4; ++ks) {
+            const uint64_t vd = desc_mn_sw128(vb + ks * 2048u, p.v_lbo, p.v_sbo);
+            umma_bf16_tmem_a(d, ph + (uint32_t)(ks * 8), vd, idesc_pv, (k == 0 && ks == 0) ? 0u : 1u);
+            umma_bf16_tmem_a(d, pl + (uint32_t)(ks * 8), vd, idesc_pv, 1u);
+          }
+          umma_commit(smem_u32(&empty_v[j % SV]));
+          umma_commit(smem_u32(&pv_done[g]));
         }
-        umma_commit(smem_u32(&empty_v[j % SV]));
-        umma_commit(smem_u32(&pv_done[g]));
+        __syncwarp();
       }
-      if (*aborted) {                                // give-up path: see the MMAs already issued retire
+      if (__any_sync(0xffffffffu, *aborted) && elect_one()) {                                // give-up path: see the MMAs already issued retire
         umma_commit(smem_u32(&drain_bar[1]));
         mbar_wait_drain(smem_u32(&drain_bar[1]), 0, 20000000ll);
       }
@@ -768,9 +729,8 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tree_attn_tc_kernel(const __gri
 #pragma unroll
       for (int c = 0; c < 16; ++c) {
         uint4 v = valid ? src[c] : make_uint4(0, 0, 0, 0);
-        if (row < QROWS)
-          *reinterpret_cast<uint4*>(smem_gen + (q_base - smem_base) + (uint32_t)(c >> 3) * QHALF + (uint32_t)row * 128u +
-                                    (uint32_t)(((c & 7) ^ (row & 7)) << 4)) = v;
+        *reinterpret_cast<uint4*>(smem_gen + (q_base - smem_base) + (uint32_t)(c >> 3) * QHALF + (uint32_t)row * 128u +
+                                  (uint32_t)(((c & 7) ^ (row & 7)) << 4)) = v;
       }
       proxy_fence();
       __syncwarp();
@@ -780,8 +740,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tree_attn_tc_kernel(const __gri
     if (valid) { anc0 = p.anc[row * CERB_ANC_WORDS]; anc1 = p.anc[row * CERB_ANC_WORDS + 1]; anc2 = p.anc[row * CERB_ANC_WORDS + 2]; }
     const uint32_t s_addr = tmem + lane_base + (uint32_t)g * 64u;
     const uint32_t o_addr = tmem + lane_base + 128u + (uint32_t)g * 128u;
-    uint8_t* ph = smem_gen + (p_base - smem_base) + (uint32_t)g * 2u * TC_P_BYTES + (uint32_t)row * 128u;
-    uint8_t* pl = ph + TC_P_BYTES;
+    const uint32_t p_addr = tmem + lane_base + 384u + (uint32_t)g * 64u;
     float m_used = -INFINITY, l = 0.f;
     int k = 0;
     for (int i = g; i < T; i += 2, ++k) {
@@ -852,25 +811,23 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tree_attn_tc_kernel(const __gri
           *reinterpret_cast<uint4*>(vgen + (size_t)(c >> 3) * 8192 + r * 128 + (c & 7) * 16) = make_uint4(0, 0, 0, 0);
         }
       }
-      // probabilities as two bf16 terms, eight keys (16 bytes) per store
+      // probabilities as two bf16 terms, two keys per column
 #pragma unroll
-      for (int c = 0; c < 8; ++c) {
-        uint32_t hi[4], lo[4];
+      for (int c0 = 0; c0 < 32; c0 += 16) {
+        uint32_t hi[16], lo[16];
 #pragma unroll
-        for (int e = 0; e < 4; ++e) {
-          const float p0 = sc[c * 8 + 2 * e], p1 = sc[c * 8 + 2 * e + 1];
+        for (int e = 0; e < 16; ++e) {
+          const float p0 = sc[2 * (c0 + e)], p1 = sc[2 * (c0 + e) + 1];
           __nv_bfloat162 hb = __floats2bfloat162_rn(p0, p1);
           float2 hf = __bfloat1622float2(hb);
           hi[e] = *reinterpret_cast<uint32_t*>(&hb);
           lo[e] = pack_bf16(p0 - hf.x, p1 - hf.y);
         }
-        const uint32_t off = (uint32_t)((c ^ (row & 7)) << 4);
-        if (row < QROWS) {
-          *reinterpret_cast<uint4*>(ph + off) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
-          *reinterpret_cast<uint4*>(pl + off) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
-        }
+        tmem_st16(p_addr + (uint32_t)c0, hi);
+        tmem_st16(p_addr + 32u + (uint32_t)c0, lo);
       }
-      proxy_fence();
+      tmem_st_wait();
+      if (key0 + TILE > kv_total) proxy_fence();      // (the zeroed rows of V)
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(smem_u32(&p_ready[g]));
@@ -1256,12 +1213,10 @@ static int launch_attn_window(const cerb_attn_args* a, int row0, int rows, const
   } else if (tensor_path) {
     static bool configured = false;
     if (!configured) {
-      CERB_CUDA_OK(cudaFuncSetAttribute(tree_attn_tc_kernel<2, 5, 128, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tc_smem(2, 5, 128)));
-      CERB_CUDA_OK(cudaFuncSetAttribute(tree_attn_tc_kernel<5, 5, 64, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tc_smem(5, 5, 64)));
+      CERB_CUDA_OK(cudaFuncSetAttribute(tree_attn_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TC_SMEM));
       configured = true;
     }
-    auto kern = rows <= 64 ? tree_attn_tc_kernel<5, 5, 64, true> : tree_attn_tc_kernel<2, 5, 128, false>;
-    const size_t TC_SMEM = rows <= 64 ? tc_smem(5, 5, 64) : tc_smem(2, 5, 128);
+    auto kern = tree_attn_tc_kernel;
     if (p.cluster)
       rc = launch_pdl_cluster(kern, dim3(p.nsplit, p.H, Bw), dim3(TC_THREADS), TC_SMEM, st, (unsigned)p.nsplit,
                               *tmK, *tmV, p) == cudaSuccess ? CERB_OK : CERB_E_CUDA;

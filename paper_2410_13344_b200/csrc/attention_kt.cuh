@@ -220,27 +220,30 @@ __global__ void __launch_bounds__(kt_threads(NCB), 1) tree_attn_kt_kernel(const 
     griddep_wait();
     griddep_launch();
     // ---------------- QK^T issuer ----------------
-    if (lane == 0 && T > 0) {
+    if (T > 0) {
       constexpr uint32_t idesc_s = idesc_bf16(128, NQ, false, false);
       const uint64_t q_desc0 = desc_k_sw128(q_base), q_desc1 = desc_k_sw128(q_base + QHALF);
-      mbar_wait(smem_u32(&q_ready), 0, wc, 102);
-      const int t_stop = *aborted ? 0 : T;
+      mbar_wait_warp(smem_u32(&q_ready), 0, wc, 102);
+      const int t_stop = __any_sync(0xffffffffu, *aborted) ? 0 : T;
       for (int t = 0; t < t_stop; ++t) {
         const int u = 2 * t, slot = u % NU, sb = t & 1;
-        if (!wait_unit(u, 103)) break;
-        if (!mbar_wait(smem_u32(&s_free[sb]), ((uint32_t)(t >> 1) & 1u) ^ 1u, wc, 104)) break;
+        if (!__all_sync(0xffffffffu, wait_unit(u, 103))) break;
+        if (!mbar_wait_warp(smem_u32(&s_free[sb]), ((uint32_t)(t >> 1) & 1u) ^ 1u, wc, 104)) break;
         tc_fence_after();
         const uint32_t kb = ring + (uint32_t)slot * KT_UNIT;
         const uint64_t k_desc0 = desc_k_sw128(kb), k_desc1 = desc_k_sw128(kb + KT_HALF);
         const uint32_t d = tmem + (uint32_t)sb * NQ;
+        if (elect_one()) {
 #pragma unroll
-        for (int kk = 0; kk < 4; ++kk) umma_bf16(d, k_desc0 + (uint64_t)(kk * 2), q_desc0 + (uint64_t)(kk * 2), idesc_s, kk ? 1u : 0u);
+          for (int kk = 0; kk < 4; ++kk) umma_bf16(d, k_desc0 + (uint64_t)(kk * 2), q_desc0 + (uint64_t)(kk * 2), idesc_s, kk ? 1u : 0u);
 #pragma unroll
-        for (int kk = 0; kk < 4; ++kk) umma_bf16(d, k_desc1 + (uint64_t)(kk * 2), q_desc1 + (uint64_t)(kk * 2), idesc_s, 1u);
-        umma_commit(smem_u32(&empty_u[slot]));       // the K unit is free once these MMAs have retired
-        umma_commit(smem_u32(&s_full[sb]));
+          for (int kk = 0; kk < 4; ++kk) umma_bf16(d, k_desc1 + (uint64_t)(kk * 2), q_desc1 + (uint64_t)(kk * 2), idesc_s, 1u);
+          umma_commit(smem_u32(&empty_u[slot]));       // the K unit is free once these MMAs have retired
+          umma_commit(smem_u32(&s_full[sb]));
+        }
+        __syncwarp();
       }
-      if (*aborted) {                                // give-up path: see the MMAs already issued retire
+      if (__any_sync(0xffffffffu, *aborted) && elect_one()) {                                // give-up path: see the MMAs already issued retire
         umma_commit(smem_u32(&drain_bar[0]));
         mbar_wait_drain(smem_u32(&drain_bar[0]), 0, 20000000ll);
       }
@@ -249,27 +252,30 @@ __global__ void __launch_bounds__(kt_threads(NCB), 1) tree_attn_kt_kernel(const 
     griddep_wait();
     griddep_launch();
     // ---------------- PV issuer ----------------
-    if (lane == 0) {
+    {
       // A = V tile read M-major (M = head_dim: two 64-wide blocks KT_HALF apart; 8-key groups 1024 bytes apart),
       // B = P^T read N-major (N = hi and lo terms side by side: 2 NQ / 64 blocks KT_HALF apart)
       constexpr uint32_t idesc_pv = idesc_bf16(128, 2 * NQ, true, true);
-      const int t_stop = *aborted ? 0 : T;
+      const int t_stop = __any_sync(0xffffffffu, *aborted) ? 0 : T;
       for (int t = 0; t < t_stop; ++t) {
         const int u = 2 * t + 1, slot = u % NU;
         const int pb = t % PB;
-        if (!mbar_wait(smem_u32(&p_ready[pb]), (uint32_t)(t / PB) & 1u, wc, 105)) break;
-        if (!wait_unit(u, 106)) break;
+        if (!mbar_wait_warp(smem_u32(&p_ready[pb]), (uint32_t)(t / PB) & 1u, wc, 105)) break;
+        if (!__all_sync(0xffffffffu, wait_unit(u, 106))) break;
         tc_fence_after();
         const uint32_t vb = ring + (uint32_t)slot * KT_UNIT;
         const uint32_t d = tmem + O_COL;
+        if (elect_one()) {
 #pragma unroll
-        for (int ks = 0; ks < 8; ++ks)
-          umma_bf16(d, desc_mn_sw128(vb + ks * 2048u, KT_HALF, 1024u), desc_mn_sw128(p_base + (uint32_t)pb * 2u * P_TERM + ks * 2048u, KT_HALF, 1024u),
-                    idesc_pv, (t == 0 && ks == 0) ? 0u : 1u);
-        umma_commit(smem_u32(&empty_u[slot]));
-        umma_commit(smem_u32(&pv_done[pb]));
+          for (int ks = 0; ks < 8; ++ks)
+            umma_bf16(d, desc_mn_sw128(vb + ks * 2048u, KT_HALF, 1024u), desc_mn_sw128(p_base + (uint32_t)pb * 2u * P_TERM + ks * 2048u, KT_HALF, 1024u),
+                      idesc_pv, (t == 0 && ks == 0) ? 0u : 1u);
+          umma_commit(smem_u32(&empty_u[slot]));
+          umma_commit(smem_u32(&pv_done[pb]));
+        }
+        __syncwarp();
       }
-      if (*aborted) {                                // give-up path: see the MMAs already issued retire
+      if (__any_sync(0xffffffffu, *aborted) && elect_one()) {                                // give-up path: see the MMAs already issued retire
         umma_commit(smem_u32(&drain_bar[1]));
         mbar_wait_drain(smem_u32(&drain_bar[1]), 0, 20000000ll);
       }

@@ -111,6 +111,11 @@ __device__ __forceinline__ bool mbar_wait_polite(uint32_t bar, uint32_t parity, 
   return false;
 }
 
+// The same wait by a whole converged warp, with one answer.
+__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, const WaitCtx& w, int site = 0) {
+  return __all_sync(0xffffffffu, mbar_wait(bar, parity, w, site));
+}
+
 // ---- TMA tile loads (no multicast anywhere) ----
 __device__ __forceinline__ uint64_t l2_policy(bool evict_first) {
   uint64_t pol;
@@ -155,6 +160,15 @@ __device__ __forceinline__ void umma_bf16(uint32_t tmem_d, uint64_t adesc, uint6
       "setp.ne.b32 p, %4, 0;\n\t"
       "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
       ::"r"(tmem_d), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(acc)
+      : "memory");
+}
+// The same with the A operand in tensor memory: row i in lane i, two neighbouring k per 32-bit column.
+__device__ __forceinline__ void umma_bf16_tmem_a(uint32_t tmem_d, uint32_t tmem_a, uint64_t bdesc, uint32_t idesc, uint32_t acc) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "setp.ne.b32 p, %4, 0;\n\t"
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
+      ::"r"(tmem_d), "r"(tmem_a), "l"(bdesc), "r"(idesc), "r"(acc)
       : "memory");
 }
 // One lane of a converged warp (always the same one); unlike "lane == 0" it tells the compiler that a single thread follows.
