@@ -79,7 +79,7 @@ struct AttnParams {
   unsigned int* counters;   // [B*H]
   int32_t* status;
   int n, H, max_pages, nsplit, oob_row;
-  int B;
+  int B, Bw;                // sequences; (sequence, window) pairs
   int win;                  // > 1: a prefill chunk of up to win * 128 consecutive tokens per sequence, one window of 128 query
                             // rows per blockIdx.z (locate_window); 1 otherwise
   int row0, rows;           // query rows row0 .. row0 + rows - 1 of the tree are this launch's (q, out, lse and anc already point
@@ -92,11 +92,10 @@ struct AttnParams {
   float scale_log2;
 };
 
-// Which sequence, and which window of 128 query rows of it, a CTA's blockIdx.z stands for.  A prefill chunk is one long
+// Which sequence, and which window of 128 query rows of it, z (blockIdx.z in most kernels) stands for.  A prefill chunk is one long
 // chain: window w is a chain of 128 nodes behind `shift` = 128 w more prefix keys, all of them in the cache before this
 // launch.  The last windows see the most keys and come first, so that the short ones fill the launch's tail.
-__device__ __forceinline__ void locate_window(const AttnParams& p, int& b, int& shift) {
-  const int z = (int)blockIdx.z;
+__device__ __forceinline__ void locate_window(const AttnParams& p, int z, int& b, int& shift) {
   b = p.win > 1 ? z % p.B : z;
   shift = p.win > 1 ? (p.win - 1 - z / p.B) * kAttnRowsPerLaunch : 0;
 }
@@ -134,7 +133,7 @@ __global__ void __launch_bounds__((WQ * WK + 1) * 32) tree_attn_bf16_kernel(cons
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int split = blockIdx.x, h = blockIdx.y;
   int b, shift;
-  locate_window(p, b, shift);
+  locate_window(p, (int)blockIdx.z, b, shift);
   const int L_old = p.len[b], L = L_old + shift;                      // keys written by earlier launches; keys every row sees
   const int nq_all = (p.n_active ? min(p.n_active[b], p.n) : p.n) - shift;   // live nodes of this sequence (from the window on)
   const size_t qrow = (p.row_off ? (size_t)p.row_off[b] : (size_t)b * p.n) + shift;   // its first row of q and out
@@ -530,7 +529,8 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tree_attn_tc_kernel(const __gri
   constexpr uint32_t QHALF = 128u * 128u, TC_Q_BYTES = 2 * QHALF;
   extern __shared__ uint8_t smem_raw[];
   __shared__ __align__(8) uint64_t full_k[SK], empty_k[SK], full_v[SV], empty_v[SV], s_full[2], s_free[2], p_ready[2], pv_done[2], q_ready, drain_bar[2];
-  __shared__ int page_list[kMaxPagesPerCta];
+  __shared__ int page_list[2][kMaxPagesPerCta];               // one per producer
+  __shared__ float2 ml_s[2][128];                             // a group's (m, l) of every row
   __shared__ uint32_t tmem_slot;
   __shared__ int aborted_s, exit_flag_s;
   __shared__ unsigned int ticket_s;
@@ -547,20 +547,42 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tree_attn_tc_kernel(const __gri
   const uint32_t k_ring = q_base + TC_Q_BYTES;
   const uint32_t v_ring = k_ring + SK * TC_KV_BYTES;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int split = blockIdx.x, h = blockIdx.y;
-  int b, shift;
-  locate_window(p, b, shift);
-  const int L_old = p.len[b], L = L_old + shift;                      // keys written by earlier launches; keys every row sees
-  const int nq_all = (p.n_active ? min(p.n_active[b], p.n) : p.n) - shift;   // live nodes of this sequence (from the window on)
-  const size_t qrow = (p.row_off ? (size_t)p.row_off[b] : (size_t)b * p.n) + shift;   // its first row of q and out
-  const int nq = min(nq_all - p.row0, p.rows);                        // live query rows of this launch
-  if (nq <= 0) return;
-  const int kv_total = L + min(nq_all, p.row0 + p.rows);
-  const int tiles = (kv_total + TILE - 1) / TILE;
-  const int per = (tiles + p.nsplit - 1) / p.nsplit;
-  const int t0 = min(tiles, split * per), t1 = min(tiles, t0 + per);
-  const bool too_long = per * PAGES_PER_TILE > kMaxPagesPerCta;
-  const int T = too_long ? 0 : t1 - t0;
+  // With one split the CTAs are persistent: (window or sequence, head) items are dealt out in turn, every second round in
+  // reverse (the items come in order of falling length where they differ).  The rings run on from item to item, so that the
+  // next item's first tiles arrive during this one's end.  (A CTA's beginning and end took 14 of the 25 us of an item of ten
+  // tiles: batch 16 x 128 nodes x 512 keys 86 -> 62 us; the 2048-token prefill's windows 108 -> 79 us per layer.)
+  const bool many = p.nsplit == 1;
+  const int items = p.Bw * p.H, ctas = many ? (int)gridDim.x : 1, rounds = many ? (items + ctas - 1) / ctas : 1;
+  const int split = many ? 0 : (int)blockIdx.x;
+  struct Item {
+    int h, b, L_old, L, nq, kv_total, t0, T, z;
+    size_t qrow;
+    bool too_long;
+  };
+  auto item_at = [&](int round) {
+    Item it;
+    int idx = many ? round * ctas + ((round & 1) ? ctas - 1 - (int)blockIdx.x : (int)blockIdx.x) : (int)(blockIdx.z * p.H + blockIdx.y);
+    it.nq = 0;
+    it.T = 0;
+    if (idx >= items) return it;
+    it.h = idx % p.H;
+    it.z = idx / p.H;
+    int shift;
+    locate_window(p, it.z, it.b, shift);
+    it.L_old = p.len[it.b];                                       // keys written by earlier launches
+    it.L = it.L_old + shift;                                      // keys every row sees
+    const int nq_all = (p.n_active ? min(p.n_active[it.b], p.n) : p.n) - shift;   // live nodes of this sequence (from the window on)
+    it.qrow = (p.row_off ? (size_t)p.row_off[it.b] : (size_t)it.b * p.n) + shift;   // its first row of q and out
+    it.nq = min(nq_all - p.row0, p.rows);                         // live query rows of this launch
+    it.kv_total = it.L + min(nq_all, p.row0 + p.rows);
+    const int tiles = (it.kv_total + TILE - 1) / TILE;
+    const int per = (tiles + p.nsplit - 1) / p.nsplit;
+    it.t0 = min(tiles, split * per);
+    it.too_long = per * PAGES_PER_TILE > kMaxPagesPerCta;
+    it.T = it.nq <= 0 || it.too_long ? 0 : min(tiles, it.t0 + per) - it.t0;
+    return it;
+  };
+  if (!many && item_at(0).nq <= 0) return;                        // (uniform over a cluster)
 
   if (threadIdx.x == 0) {
     aborted_s = (*p.status != 0);
@@ -579,13 +601,12 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tree_attn_tc_kernel(const __gri
       mbar_init(smem_u32(&p_ready[g]), 4);
       mbar_init(smem_u32(&pv_done[g]), 1);
     }
-    mbar_init(smem_u32(&q_ready), 4);
+    mbar_init(smem_u32(&q_ready), 8);
     mbar_init(smem_u32(&drain_bar[0]), 1);
     mbar_init(smem_u32(&drain_bar[1]), 1);
     mbar_init(smem_u32(&cl_bar[0]), (uint32_t)p.nsplit);
     mbar_init(smem_u32(&cl_bar[1]), (uint32_t)p.nsplit);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    if (too_long) atomicExch(p.status, CERB_E_SHAPE);
   }
   if (warp == 1) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_slot)), "r"(512u)
@@ -605,44 +626,48 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tree_attn_tc_kernel(const __gri
     // A tile of K (or V) is 8 boxes of 2 KB (four pages, two 64-wide halves), issued by 8 lanes.  Issuing a box occupies its
     // warp for ~88 cycles, so one warp for both made 1400 cycles and more of every tile, the kernel's pace (572 us at batch 16 x 128 nodes x 8K keys, 465 with two).
     const bool is_v = warp == 11;
-    const int32_t* pt = p.page_table + (size_t)b * p.max_pages;
-    const int n_pages = T * PAGES_PER_TILE;
-    for (int i = lane + (is_v ? 32 : 0); i < n_pages; i += 64) {
-      int lp = t0 * PAGES_PER_TILE + i;
-      page_list[i] = (lp * CERB_PAGE < kv_total && lp < p.max_pages) ? (pt[lp] * p.H + h) * CERB_PAGE : p.oob_row;
-    }
-    asm volatile("bar.sync 3, 64;" ::: "memory");      // the page list is complete
+    int* list = page_list[is_v ? 1 : 0];
     const int ring = is_v ? SV : SK;
     uint64_t* full = is_v ? full_v : full_k;
     uint64_t* empty = is_v ? empty_v : empty_k;
     const uint32_t base = is_v ? v_ring : k_ring;
-    // tiles of the first ring that lie wholly inside the prefix may be fetched before the wait
-    int early = 0;
-    while (early < T && early < ring && (t0 + early + 1) * TILE <= L_old) ++early;
     static_assert(PAGES_PER_TILE == 4, "the lane -> box map below assumes four pages per tile");
     const int pg = (lane >> 1) & 3, hf = lane & 1;
-    const int T_stop = __any_sync(0xffffffffu, *aborted) ? 0 : T;         // a launch that starts after a time-out issues nothing
-    int i = 0, slot = 0;
+    bool go = !__any_sync(0xffffffffu, *aborted), waited = false;         // a launch that starts after a time-out issues nothing
+    int issued = 0, slot = 0;
     uint32_t ph = 0;
-    for (; i < T_stop; ++i) {
-      if (i == early) { griddep_wait(); griddep_launch(); }
-      const uint32_t fb = smem_u32(&full[slot]);
-      int stop = 0;
-      if (lane == 0) {
-        // (a wait that gives up says so in its return value: the consumers have stopped, nothing more is issued)
-        stop = !mbar_wait_polite(smem_u32(&empty[slot]), ph ^ 1u, wc, is_v ? 306 : 305);
-        if (!stop) mbar_expect_tx(fb, TC_KV_BYTES);
+    for (int round = 0; go && round < rounds; ++round) {
+      const Item it = item_at(round);
+      if (it.T <= 0) continue;
+      const int32_t* pt = p.page_table + (size_t)it.b * p.max_pages;
+      __syncwarp();
+      for (int i = lane; i < it.T * PAGES_PER_TILE; i += 32) {
+        const int lp = it.t0 * PAGES_PER_TILE + i;
+        list[i] = (lp * CERB_PAGE < it.kv_total && lp < p.max_pages) ? (pt[lp] * p.H + it.h) * CERB_PAGE : p.oob_row;
       }
-      if (__any_sync(0xffffffffu, stop)) break;
-      if (lane < 8) {
-        const int row = page_list[i * PAGES_PER_TILE + pg];       // out-of-range rows are zero-filled by TMA
-        tma_load_2d(base + (uint32_t)slot * TC_KV_BYTES + (uint32_t)hf * 8192u + (uint32_t)pg * (CERB_PAGE * 128), is_v ? &tmV : &tmK, hf * 64, row, fb);
+      __syncwarp();
+      for (int i = 0; i < it.T; ++i) {
+        // tiles of the first ring that lie wholly inside the prefix may be fetched before the wait
+        if (!waited && (issued == ring || (it.t0 + i + 1) * TILE > it.L_old)) { griddep_wait(); griddep_launch(); waited = true; }
+        const uint32_t fb = smem_u32(&full[slot]);
+        int stop = 0;
+        if (lane == 0) {
+          // (a wait that gives up says so in its return value: the consumers have stopped, nothing more is issued)
+          stop = !mbar_wait_polite(smem_u32(&empty[slot]), ph ^ 1u, wc, is_v ? 306 : 305);
+          if (!stop) mbar_expect_tx(fb, TC_KV_BYTES);
+        }
+        if (__any_sync(0xffffffffu, stop)) { go = false; break; }
+        if (lane < 8) {
+          const int row = list[i * PAGES_PER_TILE + pg];       // out-of-range rows are zero-filled by TMA
+          tma_load_2d(base + (uint32_t)slot * TC_KV_BYTES + (uint32_t)hf * 8192u + (uint32_t)pg * (CERB_PAGE * 128), is_v ? &tmV : &tmK, hf * 64, row, fb);
+        }
+        ++issued;
+        if (++slot == ring) { slot = 0; ph ^= 1u; }
       }
-      if (++slot == ring) { slot = 0; ph ^= 1u; }
     }
     if (lane == 0 && *aborted) {
-      // give-up path: the copies already issued (tiles 0 .. i-1) still land in this CTA's shared memory; see each of them in
-      for (int j = i > ring ? i - ring : 0; j < i; ++j)
+      // give-up path: the copies already issued still land in this CTA's shared memory; see each of them in
+      for (int j = issued > ring ? issued - ring : 0; j < issued; ++j)
         mbar_wait_drain(smem_u32(&full[j % ring]), (uint32_t)(j / ring) & 1u, 20000000ll);
     }
     griddep_wait();      // (a lane that has waited already returns at once)
@@ -653,28 +678,36 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tree_attn_tc_kernel(const __gri
     // ---------------- QK^T issuer ----------------
     // (issuing one tcgen05.mma costs this thread ~95 cycles whatever its size, measured, so the two
     // products are issued by two different warps)
-    if (T > 0) {
+    {
       const uint32_t idesc_s = (1u << 4) | (1u << 7) | (1u << 10) | ((64u >> 3) << 17) | ((128u >> 4) << 24);
       const uint64_t q_desc0 = desc_k_sw128(q_base), q_desc1 = desc_k_sw128(q_base + QHALF);
-      mbar_wait_warp(smem_u32(&q_ready), 0, wc, 308);
-      const int T_stop = __any_sync(0xffffffffu, *aborted) ? 0 : T;
-      for (int i = 0; i < T_stop; ++i) {
-        const int g = i & 1, k = i >> 1;
-        if (!mbar_wait_warp(smem_u32(&full_k[i % SK]), (uint32_t)(i / SK) & 1u, wc, 309)) break;
-        if (!mbar_wait_warp(smem_u32(&s_free[g]), ((uint32_t)k & 1u) ^ 1u, wc, 311)) break;
-        tc_fence_after();
-        const uint32_t kb = k_ring + (uint32_t)(i % SK) * TC_KV_BYTES;
-        const uint64_t k_desc0 = desc_k_sw128(kb), k_desc1 = desc_k_sw128(kb + 8192u);
-        const uint32_t d = tmem + (uint32_t)g * 64u;
-        if (elect_one()) {
+      bool go = !__any_sync(0xffffffffu, *aborted);
+      int slot = 0, staged = 0;
+      uint32_t ph = 0, used[2] = {0, 0};                 // how often each group's S buffer was written
+      for (int round = 0; go && round < rounds; ++round) {
+        const int T = item_at(round).T;
+        if (T <= 0) continue;
+        if (!mbar_wait_warp(smem_u32(&q_ready), (uint32_t)staged & 1u, wc, 308)) break;
+        ++staged;
+        for (int i = 0; i < T; ++i) {
+          const int g = i & 1;
+          if (!mbar_wait_warp(smem_u32(&full_k[slot]), ph, wc, 309) || !mbar_wait_warp(smem_u32(&s_free[g]), (used[g] & 1u) ^ 1u, wc, 311)) { go = false; break; }
+          ++used[g];
+          tc_fence_after();
+          const uint32_t kb = k_ring + (uint32_t)slot * TC_KV_BYTES;
+          const uint64_t k_desc0 = desc_k_sw128(kb), k_desc1 = desc_k_sw128(kb + 8192u);
+          const uint32_t d = tmem + (uint32_t)g * 64u;
+          if (elect_one()) {
 #pragma unroll
-          for (int kk = 0; kk < 4; ++kk) umma(d, q_desc0 + (uint64_t)(kk * 2), k_desc0 + (uint64_t)(kk * 2), idesc_s, kk ? 1u : 0u);
+            for (int kk = 0; kk < 4; ++kk) umma(d, q_desc0 + (uint64_t)(kk * 2), k_desc0 + (uint64_t)(kk * 2), idesc_s, kk ? 1u : 0u);
 #pragma unroll
-          for (int kk = 0; kk < 4; ++kk) umma(d, q_desc1 + (uint64_t)(kk * 2), k_desc1 + (uint64_t)(kk * 2), idesc_s, 1u);
-          umma_commit(smem_u32(&empty_k[i % SK]));     // the K tile is free once these MMAs have retired
-          umma_commit(smem_u32(&s_full[g]));
+            for (int kk = 0; kk < 4; ++kk) umma(d, q_desc1 + (uint64_t)(kk * 2), k_desc1 + (uint64_t)(kk * 2), idesc_s, 1u);
+            umma_commit(smem_u32(&empty_k[slot]));     // the K tile is free once these MMAs have retired
+            umma_commit(smem_u32(&s_full[g]));
+          }
+          __syncwarp();
+          if (++slot == SK) { slot = 0; ph ^= 1u; }
         }
-        __syncwarp();
       }
       if (__any_sync(0xffffffffu, *aborted) && elect_one()) {                                // give-up path: see the MMAs already issued retire
         umma_commit(smem_u32(&drain_bar[0]));
@@ -688,26 +721,32 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tree_attn_tc_kernel(const __gri
     {
       // B operand (V) is MN-major, N = 128 (two 64-wide swizzle atoms, p.v_lbo bytes apart)
       const uint32_t idesc_pv = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 16) | ((128u >> 3) << 17) | ((128u >> 4) << 24);
-      const int T_stop = __any_sync(0xffffffffu, *aborted) ? 0 : T;
-      for (int j = 0; j < T_stop; ++j) {
-        const int g = j & 1, k = j >> 1;
-        if (!mbar_wait_warp(smem_u32(&p_ready[g]), (uint32_t)k & 1u, wc, 312)) break;
-        if (!mbar_wait_warp(smem_u32(&full_v[j % SV]), (uint32_t)(j / SV) & 1u, wc, 313)) break;
-        tc_fence_after();
-        const uint32_t vb = v_ring + (uint32_t)(j % SV) * TC_KV_BYTES;
-        const uint32_t d = tmem + 128u + (uint32_t)g * 128u;
-        const uint32_t ph = tmem + 384u + (uint32_t)g * 64u, pl = ph + 32u;
-        if (elect_one()) {
+      bool go = !__any_sync(0xffffffffu, *aborted);
+      int slot = 0;
+      uint32_t vph = 0, used[2] = {0, 0};
+      for (int round = 0; go && round < rounds; ++round) {
+        const int T = item_at(round).T;
+        for (int j = 0; j < T; ++j) {
+          const int g = j & 1;
+          if (!mbar_wait_warp(smem_u32(&p_ready[g]), used[g] & 1u, wc, 312) || !mbar_wait_warp(smem_u32(&full_v[slot]), vph, wc, 313)) { go = false; break; }
+          ++used[g];
+          tc_fence_after();
+          const uint32_t vb = v_ring + (uint32_t)slot * TC_KV_BYTES;
+          const uint32_t d = tmem + 128u + (uint32_t)g * 128u;
+          const uint32_t ph = tmem + 384u + (uint32_t)g * 64u, pl = ph + 32u;
+          if (elect_one()) {
 #pragma unroll
-          for (int ks = 0; ks < 4; ++ks) {
-            const uint64_t vd = desc_mn_sw128(vb + ks * 2048u, p.v_lbo, p.v_sbo);
-            umma_bf16_tmem_a(d, ph + (uint32_t)(ks * 8), vd, idesc_pv, (k == 0 && ks == 0) ? 0u : 1u);
-            umma_bf16_tmem_a(d, pl + (uint32_t)(ks * 8), vd, idesc_pv, 1u);
+            for (int ks = 0; ks < 4; ++ks) {
+              const uint64_t vd = desc_mn_sw128(vb + ks * 2048u, p.v_lbo, p.v_sbo);
+              umma_bf16_tmem_a(d, ph + (uint32_t)(ks * 8), vd, idesc_pv, (j < 2 && ks == 0) ? 0u : 1u);
+              umma_bf16_tmem_a(d, pl + (uint32_t)(ks * 8), vd, idesc_pv, 1u);
+            }
+            umma_commit(smem_u32(&empty_v[slot]));
+            umma_commit(smem_u32(&pv_done[g]));
           }
-          umma_commit(smem_u32(&empty_v[j % SV]));
-          umma_commit(smem_u32(&pv_done[g]));
+          __syncwarp();
+          if (++slot == SV) { slot = 0; vph ^= 1u; }
         }
-        __syncwarp();
       }
       if (__any_sync(0xffffffffu, *aborted) && elect_one()) {                                // give-up path: see the MMAs already issued retire
         umma_commit(smem_u32(&drain_bar[1]));
@@ -720,17 +759,32 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tree_attn_tc_kernel(const __gri
     const int gt = (int)threadIdx.x - 64 - g * 128;           // thread index inside the group
     const int row = (warp & 3) * 32 + lane;                    // = TMEM lane
     const uint32_t lane_base = (uint32_t)((warp & 3) * 32) << 16;
-    const bool valid = row < nq;
+    const int st = (int)threadIdx.x - 64;
+    const float LN2 = 0.6931471805599453f;
     griddep_wait();
     griddep_launch();
-    if (g == 0) {
-      // stage this row of Q (zeros past the last node) in the swizzled K-major layout
-      const uint4* src = reinterpret_cast<const uint4*>(p.q + ((qrow + (valid ? row : 0)) * p.H + h) * DH);
+    int nv = 0;                                                // V tiles of the rounds before
+    uint32_t n = 0;                                            // tiles this group has taken in all
+    for (int round = 0; round < rounds; ++round) {
+    const Item it = item_at(round);
+    if (it.nq <= 0) continue;
+    const int h = it.h, b = it.b, L = it.L, nq = it.nq, kv_total = it.kv_total, t0 = it.t0, T = it.T;
+    const size_t qrow = it.qrow;
+    const bool valid = row < nq;
+    if (it.too_long && st == 0) atomicExch(p.status, CERB_E_SHAPE);
+    if (T > 0) {
+      // stage Q (zeros past the last node) in the swizzled K-major layout, 16-byte pieces spread over both groups
+      uint4 v[8];
 #pragma unroll
-      for (int c = 0; c < 16; ++c) {
-        uint4 v = valid ? src[c] : make_uint4(0, 0, 0, 0);
-        *reinterpret_cast<uint4*>(smem_gen + (q_base - smem_base) + (uint32_t)(c >> 3) * QHALF + (uint32_t)row * 128u +
-                                  (uint32_t)(((c & 7) ^ (row & 7)) << 4)) = v;
+      for (int i = 0; i < 8; ++i) {
+        const int piece = st + i * 256, r = piece >> 4, c = piece & 15;
+        v[i] = r < nq ? reinterpret_cast<const uint4*>(p.q + ((qrow + r) * p.H + h) * DH)[c] : make_uint4(0, 0, 0, 0);
+      }
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        const int piece = st + i * 256, r = piece >> 4, c = piece & 15;
+        *reinterpret_cast<uint4*>(smem_gen + (q_base - smem_base) + (uint32_t)(c >> 3) * QHALF + (uint32_t)r * 128u +
+                                  (uint32_t)(((c & 7) ^ (r & 7)) << 4)) = v[i];
       }
       proxy_fence();
       __syncwarp();
@@ -743,8 +797,8 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tree_attn_tc_kernel(const __gri
     const uint32_t p_addr = tmem + lane_base + 384u + (uint32_t)g * 64u;
     float m_used = -INFINITY, l = 0.f;
     int k = 0;
-    for (int i = g; i < T; i += 2, ++k) {
-      mbar_wait(smem_u32(&s_full[g]), (uint32_t)k & 1u, wc, 314);
+    for (int i = g; i < T; i += 2, ++k, ++n) {
+      mbar_wait(smem_u32(&s_full[g]), n & 1u, wc, 314);
       tc_fence_after();
       float sc[64];
 #pragma unroll
@@ -782,7 +836,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tree_attn_tc_kernel(const __gri
       for (int j = 0; j < 64; ++j) { sc[j] = ex2(sc[j] - mu); rs4[j & 3] += sc[j]; }
       l = l * alpha + ((rs4[0] + rs4[1]) + (rs4[2] + rs4[3]));
       if (k > 0) {
-        mbar_wait(smem_u32(&pv_done[g]), (uint32_t)(k - 1) & 1u, wc, 315);   // P buffers free, O at rest
+        mbar_wait(smem_u32(&pv_done[g]), (n - 1u) & 1u, wc, 315);   // P buffers free, O at rest
         tc_fence_after();
         if (__any_sync(0xffffffffu, rescale)) {
 #pragma unroll 1
@@ -803,9 +857,10 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tree_attn_tc_kernel(const __gri
         // last, partial tile: rows past the end may hold anything (stale pool memory); zero V there so
         // that a zero probability times a non-finite value cannot poison the sum.  V travels apart
         // from K, so wait until it has landed.
-        mbar_wait(smem_u32(&full_v[i % SV]), (uint32_t)(i / SV) & 1u, wc, 316);
+        const int vt = nv + i;
+        mbar_wait(smem_u32(&full_v[vt % SV]), (uint32_t)(vt / SV) & 1u, wc, 316);
         const int first_bad = kv_total - key0;
-        uint8_t* vgen = smem_gen + (v_ring - smem_base) + (size_t)(i % SV) * TC_KV_BYTES;
+        uint8_t* vgen = smem_gen + (v_ring - smem_base) + (size_t)(vt % SV) * TC_KV_BYTES;
         for (int idx = gt; idx < (TILE - first_bad) * 16; idx += 128) {
           const int r = first_bad + (idx >> 4), c = idx & 15;
           *reinterpret_cast<uint4*>(vgen + (size_t)(c >> 3) * 8192 + r * 128 + (c & 7) * 16) = make_uint4(0, 0, 0, 0);
@@ -832,11 +887,50 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tree_attn_tc_kernel(const __gri
       __syncwarp();
       if (lane == 0) mbar_arrive(smem_u32(&p_ready[g]));
     }
-    // ---- this group's (m, l, O) rows into shared memory ----
+    nv += T;
     if (k > 0) {
-      mbar_wait(smem_u32(&pv_done[g]), (uint32_t)(k - 1) & 1u, wc, 317);
+      mbar_wait(smem_u32(&pv_done[g]), (n - 1u) & 1u, wc, 317);
       tc_fence_after();
     }
+    if (many) {
+      // ---- output: a row's thread of group g finishes columns 64 g .. 64 g + 63 from both groups' accumulators ----
+      ml_s[g][row] = make_float2(m_used, l);
+      tc_fence_before();
+      compute_bar(256);
+      tc_fence_after();
+      const float2 x0 = ml_s[0][row], x1 = ml_s[1][row];
+      const float M = fmaxf(x0.x, x1.x), u = M == -INFINITY ? 0.f : M;
+      const float w0 = ex2(x0.x - u), w1 = ex2(x1.x - u), Lsum = x0.y * w0 + x1.y * w1, inv = 1.0f / Lsum;
+      const float f0 = w0 * inv, f1 = w1 * inv;
+      bf16* o = p.out + ((qrow + (valid ? row : 0)) * p.H + h) * DH + g * 64;
+#pragma unroll 1
+      for (int c0 = 0; c0 < 64; c0 += 16) {
+        uint32_t r0[16], r1[16];
+        tmem_ld16(tmem + lane_base + 128u + (uint32_t)(g * 64 + c0), r0);
+        tmem_ld16(tmem + lane_base + 256u + (uint32_t)(g * 64 + c0), r1);
+        tmem_ld_wait();
+        uint32_t w[8];
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+          float a = __uint_as_float(r0[2 * e]) * f0, c = __uint_as_float(r0[2 * e + 1]) * f0;
+          if (T > 1) {                                  // (with one tile the second group has accumulated nothing)
+            a += __uint_as_float(r1[2 * e]) * f1;
+            c += __uint_as_float(r1[2 * e + 1]) * f1;
+          }
+          w[e] = pack_bf16(a, c);
+        }
+        if (valid) {
+          reinterpret_cast<uint4*>(o + c0)[0] = make_uint4(w[0], w[1], w[2], w[3]);
+          reinterpret_cast<uint4*>(o + c0)[1] = make_uint4(w[4], w[5], w[6], w[7]);
+        }
+      }
+      if (g == 0 && valid && p.lse) p.lse[((size_t)b * p.H + h) * p.n + row] = (M + log2f(Lsum)) * LN2;
+      tc_fence_before();
+      compute_bar(256);                                 // Q, the accumulators and ml_s may be written again
+      tc_fence_after();
+      continue;
+    }
+    // ---- this group's (m, l, O) rows into shared memory ----
     compute_bar(256);                               // every MMA has retired: all of shared memory can be reused
     {
       float* mr = mrg + ((size_t)g * 128 + row) * ROWF;
@@ -882,27 +976,14 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tree_attn_tc_kernel(const __gri
 
     // ---- output: final, or partial + fixed-order merge by the last CTA of this (sequence, head) ----
     const int ct = threadIdx.x - 64, nct = 256, RP = p.rows_pad;
-    const float LN2 = 0.6931471805599453f;
-    if (p.cluster) {
-      // merged after the role branches, where every thread of the cluster meets
-    } else if (p.nsplit == 1) {
-      for (int idx = ct; idx < nq * (DH / 4); idx += nct) {
-        const int r = idx / (DH / 4), c4 = idx % (DH / 4);
-        const float inv = 1.0f / mrg[(size_t)r * ROWF + DH + 1];
-        const float4 v = *reinterpret_cast<const float4*>(mrg + (size_t)r * ROWF + c4 * 4);
-        *reinterpret_cast<uint2*>(p.out + ((qrow + r) * p.H + h) * DH + c4 * 4) =
-            make_uint2(pack_bf16(v.x * inv, v.y * inv), pack_bf16(v.z * inv, v.w * inv));
-      }
-      if (p.lse)
-        for (int r = ct; r < nq; r += nct)
-          p.lse[((size_t)b * p.H + h) * p.n + r] = (mrg[(size_t)r * ROWF + DH] + log2f(mrg[(size_t)r * ROWF + DH + 1])) * LN2;
-    } else {
-      float* part = p.partial + (((size_t)blockIdx.z * p.H + h) * p.nsplit) * (size_t)(RP * ROWF);
+    // (with a cluster the merge follows the role branches, where every thread of the cluster meets)
+    if (!p.cluster) {
+      float* part = p.partial + (((size_t)it.z * p.H + h) * p.nsplit) * (size_t)(RP * ROWF);
       float* mine = part + (size_t)split * (RP * ROWF);
       for (int idx = ct; idx < nq * ROWF; idx += nct) __stcg(mine + idx, mrg[idx]);
       __threadfence();
       compute_bar(256);
-      if (ct == 0) ticket_s = atomicAdd(&p.counters[blockIdx.z * p.H + h], 1u);
+      if (ct == 0) ticket_s = atomicAdd(&p.counters[it.z * p.H + h], 1u);
       compute_bar(256);
       if (ticket_s == (unsigned)p.nsplit - 1) {
         __threadfence();
@@ -935,8 +1016,9 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tree_attn_tc_kernel(const __gri
           *reinterpret_cast<uint2*>(p.out + ((qrow + r) * p.H + h) * DH + c4 * 4) =
               make_uint2(pack_bf16(acc.x, acc.y), pack_bf16(acc.z, acc.w));
         }
-        if (ct == 0) p.counters[blockIdx.z * p.H + h] = 0u;          // ready for the next launch
+        if (ct == 0) p.counters[it.z * p.H + h] = 0u;          // ready for the next launch
       }
+    }
     }
   }
   if (p.cluster) {
@@ -945,6 +1027,9 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tree_attn_tc_kernel(const __gri
     // those rows from every member in split order, weighs them and writes the final output.  Nobody leaves
     // before the second meeting, so no shared memory is read after its CTA has gone.
     cluster_start_wait();
+    const Item it = item_at(0);
+    const int h = it.h, b = it.b, nq = it.nq;
+    const size_t qrow = it.qrow;
     if (warp >= 2 && warp < 10) {
       cluster_meet(&cl_bar[0], p.nsplit, (int)threadIdx.x - 64, wc, 318);  // every member's rows are in place
       const int ct = threadIdx.x - 64;
@@ -1136,6 +1221,7 @@ static int launch_attn_window(const cerb_attn_args* a, int row0, int rows, const
   AttnParams p;
   const int Bw = a->B * win;             // (sequence, window) pairs
   p.B = a->B;
+  p.Bw = Bw;
   p.win = win;
   const size_t row_elems = (size_t)a->n_heads * a->head_dim;
   p.q = (const bf16*)a->q + (size_t)row0 * row_elems;
@@ -1221,8 +1307,11 @@ static int launch_attn_window(const cerb_attn_args* a, int row0, int rows, const
       rc = launch_pdl_cluster(kern, dim3(p.nsplit, p.H, Bw), dim3(TC_THREADS), TC_SMEM, st, (unsigned)p.nsplit,
                               *tmK, *tmV, p) == cudaSuccess ? CERB_OK : CERB_E_CUDA;
     else
-      rc = launch_pdl(kern, dim3(p.nsplit, p.H, Bw), dim3(TC_THREADS), TC_SMEM, st, *tmK, *tmV, p) == cudaSuccess
-               ? CERB_OK : CERB_E_CUDA;
+    {
+      // one split: persistent CTAs over the (window or sequence, head) items
+      const dim3 grid = p.nsplit == 1 ? dim3(Bw * p.H < 148 ? Bw * p.H : 148) : dim3(p.nsplit, p.H, Bw);
+      rc = launch_pdl(kern, grid, dim3(TC_THREADS), TC_SMEM, st, *tmK, *tmV, p) == cudaSuccess ? CERB_OK : CERB_E_CUDA;
+    }
   } else if (a->head_dim == 128) {
     if (np == 16) rc = launch_cfg<128, 1, 4, 3>(p, tmK, tmV, Bw, st);
     else if (np == 32) rc = launch_cfg<128, 2, 4, 3>(p, tmK, tmV, Bw, st);

@@ -103,7 +103,7 @@ __global__ void __launch_bounds__(kt_threads(NCB), 1) tree_attn_kt_kernel(const 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int split = blockIdx.x, h = blockIdx.y;
   int b, shift;
-  locate_window(p, b, shift);
+  locate_window(p, (int)blockIdx.z, b, shift);
   // Lengths, live node counts, the page table, the tree and the prefix keys are at least two kernels old:
   // everything up to the first use of Q or of this step's tree keys runs before griddep_wait().
   const int L_old = p.len[b], L = L_old + shift;                      // keys written by earlier launches; keys every row sees

@@ -607,7 +607,7 @@ TilePlan make_tile_plan(int M, int N, int K, size_t max_fix) {
   for (int hf = 1; hf <= (least_chunks > 2 ? 2 : 1); ++hf)
     for (int c = least_chunks; c <= least_chunks + least_chunks / 4 + 1; ++c)
       for (int S = 1; S <= 4 * hf; ++S)
-        for (int sk = 0; sk <= (S == 1 ? 1 : 0); ++sk) {
+        for (int sk = 0; sk <= (S == 1 && hf == 1 ? 1 : 0); ++sk) {      // (two accumulators per share: never the fastest)
           TilePlan g;
           g.hf = hf;
           g.mchunks = c;
@@ -643,7 +643,7 @@ TilePlan make_tile_plan(int M, int N, int K, size_t max_fix) {
   return best;
 }
 
-size_t gemm_fix_floats() { return (size_t)kPairs * 2 * 2 * 2 * 128 * TILE_X; }
+size_t gemm_fix_floats() { return (size_t)kPairs * 2 * 2 * 128 * TILE_X; }
 
 template <int KIND, int HF>
 static int launch_kind(const CUtensorMap& tmW, const CUtensorMap& tmX, TileParams q, int pairs, cudaStream_t st) {
