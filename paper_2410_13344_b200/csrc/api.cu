@@ -699,11 +699,9 @@ int cerb_step(cerb_ctx* c, const cerb_tree* tree, float T, const int32_t* plant_
   cudaStream_t st = (cudaStream_t)stream;
   const int B = c->B;
   // gate; it also writes each sequence's live node count (1 for an auto-regressive sequence)
-  { ProfScope ps(c, K_GATE, st); CERB_TRY(launch_gate(c, T, out->S_dev, out->mode_dev, c->d_nactive, tree->n, st)); }
+  // (the gate writes them itself: with three copies of a few words behind it a step took 5 to 10 us more)
   int32_t* hs = c->h_stage;
-  CERB_CUDA_OK(cudaMemcpyAsync(hs, out->mode_dev, B * sizeof(int32_t), cudaMemcpyDeviceToHost, st));
-  CERB_CUDA_OK(cudaMemcpyAsync(hs + CERB_MAX_BATCH, c->d_len, B * sizeof(int32_t), cudaMemcpyDeviceToHost, st));
-  CERB_CUDA_OK(cudaMemcpyAsync(hs + 2 * CERB_MAX_BATCH, out->S_dev, B * sizeof(float), cudaMemcpyDeviceToHost, st));
+  { ProfScope ps(c, K_GATE, st); CERB_TRY(launch_gate(c, T, out->S_dev, out->mode_dev, c->d_nactive, tree->n, st, hs)); }
   CERB_CUDA_OK(cudaStreamSynchronize(st));
   bool any_par = false;
   for (int b = 0; b < B; ++b) {

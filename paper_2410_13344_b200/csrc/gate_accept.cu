@@ -28,7 +28,8 @@ __device__ __forceinline__ float block_reduce(float v, float* red, bool is_max) 
 // mode = S > T ? auto-regressive : parallel (Algorithm 1).
 template <typename T>
 __global__ void __launch_bounds__(256) gate_kernel(const T* __restrict__ h_last, int d, float thr, float* __restrict__ S,
-                                                   int32_t* __restrict__ mode, int32_t* __restrict__ n_active, int n_par) {
+                                                   int32_t* __restrict__ mode, int32_t* __restrict__ n_active, int n_par,
+                                                   const int32_t* __restrict__ len, int32_t* __restrict__ host) {
   __shared__ float red[32];
   griddep_wait();
   griddep_launch();
@@ -50,6 +51,13 @@ __global__ void __launch_bounds__(256) gate_kernel(const T* __restrict__ h_last,
     S[blockIdx.x] = s;
     mode[blockIdx.x] = md;
     if (n_active) n_active[blockIdx.x] = md == CERB_MODE_AR ? 1 : n_par;
+    if (host) {
+      // the step's one read-back, written to pinned host memory here: mode, length and S
+      host[blockIdx.x] = md;
+      host[CERB_MAX_BATCH + blockIdx.x] = len[blockIdx.x];
+      host[2 * CERB_MAX_BATCH + blockIdx.x] = __float_as_int(s);
+      __threadfence_system();
+    }
   }
 }
 
@@ -167,10 +175,10 @@ __global__ void kv_compact_kernel(char* __restrict__ kpool, char* __restrict__ v
 
 }  // namespace
 
-int launch_gate(cerb_ctx* c, float T, float* S, int32_t* mode, int32_t* nactive_or_null, int n_par, cudaStream_t st) {
+int launch_gate(cerb_ctx* c, float T, float* S, int32_t* mode, int32_t* nactive_or_null, int n_par, cudaStream_t st, int32_t* host) {
   int d = c->cfg.d_model;
-  if (c->bf16) gate_kernel<bf16><<<c->B, 256, 0, st>>>((const bf16*)c->d_hlast, d, T, S, mode, nactive_or_null, n_par);
-  else gate_kernel<float><<<c->B, 256, 0, st>>>((const float*)c->d_hlast, d, T, S, mode, nactive_or_null, n_par);
+  if (c->bf16) gate_kernel<bf16><<<c->B, 256, 0, st>>>((const bf16*)c->d_hlast, d, T, S, mode, nactive_or_null, n_par, c->d_len, host);
+  else gate_kernel<float><<<c->B, 256, 0, st>>>((const float*)c->d_hlast, d, T, S, mode, nactive_or_null, n_par, c->d_len, host);
   CERB_LAUNCH_CHECK(c);
   return CERB_OK;
 }
