@@ -253,149 +253,135 @@ __global__ void head_init_kernel(const T* __restrict__ h_last, float* __restrict
 
 __device__ __forceinline__ bool better(float va, int ia, float vb, int ib) { return va > vb || (va == vb && ia < ib); }
 
-// Block-wide arg-best over (value, id) pairs in (value descending, id ascending) order.
-__device__ __forceinline__ void block_best(float& best, int& bi, float* sv, int* si) {
-  for (int o = 16; o > 0; o >>= 1) {
-    float ov = __shfl_xor_sync(0xffffffffu, best, o);
-    int oi = __shfl_xor_sync(0xffffffffu, bi, o);
-    if (better(ov, oi, best, bi)) { best = ov; bi = oi; }
-  }
-  const int w = threadIdx.x >> 5, l = threadIdx.x & 31, nw = blockDim.x >> 5;
-  if (l == 0) { sv[w] = best; si[w] = bi; }
-  __syncthreads();
-  if (w == 0) {
-    best = l < nw ? sv[l] : -INFINITY;
-    bi = l < nw ? si[l] : 0x7fffffff;
-    for (int o = 16; o > 0; o >>= 1) {
-      float ov = __shfl_xor_sync(0xffffffffu, best, o);
-      int oi = __shfl_xor_sync(0xffffffffu, bi, o);
-      if (better(ov, oi, best, bi)) { best = ov; bi = oi; }
-    }
-    if (l == 0) { sv[0] = best; si[0] = bi; }
-  }
-  __syncthreads();
-  best = sv[0];
-  bi = si[0];
-  __syncthreads();
-}
-
-// Per-head top-k in two steps.  Step 1: the vocabulary is cut into kTopkChunks chunks and one CTA per
-// (chunk, head, sequence) finds its chunk's k best in k rounds; round r only considers entries that come
-// strictly after the previous winner in (value descending, id ascending) order, so nothing is modified
-// in place.  A thread keeps its entries in registers and looks through them again only after one of them has won
-// (fetching the chunk anew in every round: 17 us for 4 heads x 32000 entries).  The global k best are among these
-// candidates.  Step 2: one CTA per (head, sequence) runs the same k rounds over the kTopkChunks * k candidates.
-constexpr int kTopkHeld = 16;             // entries a thread holds: chunks of up to 4096
-__global__ void __launch_bounds__(256) topk_part_kernel(const float* __restrict__ logits, int V, int Hc,
-                                                        const int32_t* __restrict__ kper, float* __restrict__ cand_v,
-                                                        int32_t* __restrict__ cand_i) {
-  __shared__ float sv[32];
-  __shared__ int si[32];
-  griddep_wait();
-  griddep_launch();
-  const int ch = blockIdx.x, h = blockIdx.y, b = blockIdx.z;
-  const float* r = logits + ((size_t)b * Hc + h) * V;
-  const int k = kper[h];
-  const int per = (V + kTopkChunks - 1) / kTopkChunks;
-  const int j0 = ch * per, j1 = min(V, j0 + per);
-  float pv = INFINITY;
-  int pi = -1;
-  const size_t o = (((size_t)b * Hc + h) * kTopkChunks + ch) * CERB_MAX_TOPK;
-  const bool held = per <= kTopkHeld * (int)blockDim.x;
-  float keep[kTopkHeld];
-  if (held) {
-#pragma unroll
-    for (int e = 0; e < kTopkHeld; ++e) {
-      const int j = j0 + threadIdx.x + e * blockDim.x;
-      keep[e] = j < j1 ? r[j] : -INFINITY;
-    }
-  }
-  float mine = 0.f;
-  int mi = -1;
+// The k best of the entries that a warp's lanes hold (N each, in registers), in (value descending, id ascending) order: in
+// every round the lanes' own best meet in two warp-wide reductions, and the lane whose entry has won looks through its others again.  Entries
+// without an id (0x7fffffff) never win against others.  emit(round, value, id) is called by every lane.
+template <int N, typename Emit>
+__device__ __forceinline__ void warp_topk(const float (&v)[N], const int (&id)[N], int k, Emit emit) {
+  float pv = INFINITY, mine = -INFINITY;
+  int pi = -1, mi = 0x7fffffff;
   bool look = true;
   for (int round = 0; round < k; ++round) {
     if (look) {
       mine = -INFINITY;
       mi = 0x7fffffff;
-      if (held) {
 #pragma unroll
-        for (int e = 0; e < kTopkHeld; ++e) {
-          const int j = j0 + threadIdx.x + e * blockDim.x;
-          const float v = keep[e];
-          const bool after = j < j1 && (v < pv || (v == pv && j > pi));
-          if (after && better(v, j, mine, mi)) { mine = v; mi = j; }
-        }
-      } else {
-        for (int j = j0 + threadIdx.x; j < j1; j += blockDim.x) {
-          const float v = r[j];
-          const bool after = v < pv || (v == pv && j > pi);
-          if (after && better(v, j, mine, mi)) { mine = v; mi = j; }
-        }
+      for (int e = 0; e < N; ++e) {
+        const bool after = id[e] != 0x7fffffff && (v[e] < pv || (v[e] == pv && id[e] > pi));
+        if (after && better(v[e], id[e], mine, mi)) { mine = v[e]; mi = id[e]; }
       }
     }
-    float best = mine;
-    int bi = mi;
-    block_best(best, bi, sv, si);
-    look = bi == mi;
-    pv = best;
-    pi = bi;
-    if (threadIdx.x == 0) {
-      cand_v[o + round] = best;
-      cand_i[o + round] = bi == 0x7fffffff ? -1 : bi;
-    }
+    // unsigned in the order of the values (+ 0.f: both zeros are one value)
+    const unsigned bits = __float_as_uint(mine + 0.f), key = bits & 0x80000000u ? ~bits : bits | 0x80000000u;
+    const unsigned top = __reduce_max_sync(0xffffffffu, key);
+    pi = __reduce_min_sync(0xffffffffu, key == top ? mi : 0x7fffffff);
+    pv = __uint_as_float(top & 0x80000000u ? top & 0x7fffffffu : ~top);
+    look = pi == mi;
+    emit(round, pv, pi);
   }
 }
 
-__global__ void __launch_bounds__(256) topk_merge_kernel(const float* __restrict__ cand_v, const int32_t* __restrict__ cand_i,
-                                                         int Hc, const int32_t* __restrict__ kper, int32_t* __restrict__ topk,
-                                                         int32_t* __restrict__ topk_copy) {
-  __shared__ float sv[32];
-  __shared__ int si[32];
+// Per-head top-k in two steps, bound by their chains of loads and rounds and not by the 0.5 MB they read.  Step 1: the
+// vocabulary is cut into kTopkChunks chunks, one CTA per (chunk, head, sequence); each warp finds the k best of its eighth of
+// the chunk, 512 entries at a time against the k best so far, and the first warp the k best of the eight lists.  Step 2: one
+// warp per (head, sequence) does the same with the chunks' candidates, among which the global k best are, and one CTA per
+// sequence then fills the tree.  4 heads x 32000 entries, k = 10: 10.6 and 11.8 us with cold caches; with block-wide rounds
+// and the tree filled by a launch of its own 13, 8 and 3 us (a draft of the 7B shape, batch 4: 536 -> 531 us).
+constexpr int TK_WARPS = 8, TK_HELD = 16;
+__global__ void __launch_bounds__(TK_WARPS * 32) topk_part_kernel(const float* __restrict__ logits, int V, int Hc,
+                                                                  const int32_t* __restrict__ kper, float* __restrict__ cand_v,
+                                                                  int32_t* __restrict__ cand_i) {
+  __shared__ float lv[TK_WARPS][CERB_MAX_TOPK];
+  __shared__ int li[TK_WARPS][CERB_MAX_TOPK];
   griddep_wait();
   griddep_launch();
-  const int h = blockIdx.x, b = blockIdx.y;
+  const int ch = blockIdx.x, h = blockIdx.y, b = blockIdx.z, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const float* r = logits + ((size_t)b * Hc + h) * V;
   const int k = kper[h];
-  const size_t base = ((size_t)b * Hc + h) * kTopkChunks * CERB_MAX_TOPK;
-  // candidate of this thread: (chunk, round) = (t / MAX_TOPK, t % MAX_TOPK)
-  float cv = -INFINITY;
-  int ci = 0x7fffffff;
-  const int t = threadIdx.x;
-  if (t < kTopkChunks * CERB_MAX_TOPK && (t % CERB_MAX_TOPK) < k) {
-    const int id = cand_i[base + t];
-    if (id >= 0) { cv = cand_v[base + t]; ci = id; }
+  const int per = (V + kTopkChunks - 1) / kTopkChunks;
+  const int c1 = min(V, (ch + 1) * per), part = (per + TK_WARPS - 1) / TK_WARPS;
+  const int j0 = min(c1, ch * per + warp * part), j1 = min(c1, j0 + part);
+  if (lane < CERB_MAX_TOPK) { lv[warp][lane] = -INFINITY; li[warp][lane] = 0x7fffffff; }
+  for (int base = j0; base < j1; base += 32 * TK_HELD) {
+    float v[TK_HELD + 1];
+    int id[TK_HELD + 1];
+#pragma unroll
+    for (int e = 0; e < TK_HELD; ++e) {
+      const int j = base + e * 32 + lane;
+      v[e] = j < j1 ? r[j] : -INFINITY;
+      id[e] = j < j1 ? j : 0x7fffffff;
+    }
+    __syncwarp();
+    v[TK_HELD] = lane < CERB_MAX_TOPK ? lv[warp][lane] : -INFINITY;       // the best so far
+    id[TK_HELD] = lane < CERB_MAX_TOPK ? li[warp][lane] : 0x7fffffff;
+    __syncwarp();
+    warp_topk(v, id, k, [&](int round, float bv, int bi) {
+      if (lane == 0) { lv[warp][round] = bv; li[warp][round] = bi; }
+    });
   }
-  float pv = INFINITY;
-  int pi = -1;
-  for (int round = 0; round < CERB_MAX_TOPK; ++round) {
-    int32_t res = -1;
-    if (round < k) {
-      const bool after = ci != 0x7fffffff && (cv < pv || (cv == pv && ci > pi));
-      float best = after ? cv : -INFINITY;
-      int bi = after ? ci : 0x7fffffff;
-      block_best(best, bi, sv, si);
-      pv = best;
-      pi = bi;
-      res = pi == 0x7fffffff ? -1 : pi;
+  __syncthreads();
+  if (warp == 0) {
+    constexpr int N = TK_WARPS * CERB_MAX_TOPK / 32;
+    float v[N];
+    int id[N];
+#pragma unroll
+    for (int e = 0; e < N; ++e) {
+      v[e] = (&lv[0][0])[e * 32 + lane];
+      id[e] = (&li[0][0])[e * 32 + lane];
     }
-    if (threadIdx.x == 0) {
-      const size_t o = ((size_t)b * Hc + h) * CERB_MAX_TOPK + round;
-      topk[o] = res;
-      if (topk_copy) topk_copy[o] = res;
-    }
+    const size_t o = (((size_t)b * Hc + h) * kTopkChunks + ch) * CERB_MAX_TOPK;
+    warp_topk(v, id, k, [&](int round, float bv, int bi) {
+      if (lane == 0) {
+        cand_v[o + round] = bv;
+        cand_i[o + round] = bi == 0x7fffffff ? -1 : bi;
+      }
+    });
   }
 }
 
-__global__ void tree_fill_kernel(const int32_t* __restrict__ root, const int32_t* __restrict__ topk,
-                                 const int32_t* __restrict__ head_of, const int32_t* __restrict__ rank_of,
-                                 const int32_t* __restrict__ plant, int Hc, int n, int32_t* __restrict__ tree_tok) {
+// One CTA per sequence, one warp per head: the merge, then the tree's tokens.
+__global__ void __launch_bounds__(CERB_MAX_HEADS * 32) topk_merge_kernel(const float* __restrict__ cand_v, const int32_t* __restrict__ cand_i,
+                                                                         int Hc, const int32_t* __restrict__ kper, int32_t* __restrict__ topk,
+                                                                         int32_t* __restrict__ topk_copy, const int32_t* __restrict__ root,
+                                                                         const int32_t* __restrict__ head_of, const int32_t* __restrict__ rank_of,
+                                                                         const int32_t* __restrict__ plant, int n, int32_t* __restrict__ tree_tok) {
+  __shared__ int best_s[CERB_MAX_HEADS][CERB_MAX_TOPK];
   griddep_wait();
   griddep_launch();
-  int b = blockIdx.x;
+  const int b = blockIdx.x, h = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (h < Hc) {
+    const int k = kper[h];
+    const size_t base = ((size_t)b * Hc + h) * kTopkChunks * CERB_MAX_TOPK;
+    constexpr int N = kTopkChunks * CERB_MAX_TOPK / 32;
+    float v[N];
+    int id[N];
+#pragma unroll
+    for (int e = 0; e < N; ++e) {
+      // candidate (chunk, round) = (t / MAX_TOPK, t % MAX_TOPK)
+      const int t = e * 32 + lane;
+      const int c = (t % CERB_MAX_TOPK) < k ? cand_i[base + t] : -1;
+      v[e] = c >= 0 ? cand_v[base + t] : -INFINITY;
+      id[e] = c >= 0 ? c : 0x7fffffff;
+    }
+    if (lane < CERB_MAX_TOPK) best_s[h][lane] = -1;
+    __syncwarp();
+    warp_topk(v, id, k, [&](int round, float, int bi) {
+      if (lane == 0) best_s[h][round] = bi == 0x7fffffff ? -1 : bi;
+    });
+    __syncwarp();
+    if (lane < CERB_MAX_TOPK) {
+      const size_t o = ((size_t)b * Hc + h) * CERB_MAX_TOPK + lane;
+      topk[o] = best_s[h][lane];
+      if (topk_copy) topk_copy[o] = best_s[h][lane];
+    }
+  }
+  __syncthreads();
+  if (!tree_tok) return;
   for (int v = threadIdx.x; v < n; v += blockDim.x) {
     int t;
     if (v == 0) t = root[b];
     else {
-      t = topk[((size_t)b * Hc + head_of[v]) * CERB_MAX_TOPK + rank_of[v]];
+      t = best_s[head_of[v]][rank_of[v]];
       if (plant && plant[(size_t)b * n + v] >= 0) t = plant[(size_t)b * n + v];
     }
     tree_tok[(size_t)b * n + v] = t;
@@ -499,16 +485,13 @@ int launch_heads(cerb_ctx* c, const cerb_tree* tree, int32_t* tree_tok, const in
     else CERB_TRY(launch_level(c, P, max_rows, max_w, st));
   }
   const float* lg = logits_out ? logits_out : c->d_hlogits;
-  static_assert(kTopkChunks * CERB_MAX_TOPK <= 256, "one candidate per thread in the merge");
-  launch_pdl(topk_part_kernel, dim3(kTopkChunks, Hc, B), dim3(256), 0, st, lg, g.vocab, Hc, (const int32_t*)c->d_kper, c->d_topk_cv, c->d_topk_ci);
+  static_assert(kTopkChunks * CERB_MAX_TOPK % 32 == 0, "whole warps of candidates in the merge");
+  launch_pdl(topk_part_kernel, dim3(kTopkChunks, Hc, B), dim3(TK_WARPS * 32), 0, st, lg, g.vocab, Hc, (const int32_t*)c->d_kper, c->d_topk_cv, c->d_topk_ci);
   CERB_LAUNCH_CHECK(c);
-  launch_pdl(topk_merge_kernel, dim3(Hc, B), dim3(256), 0, st, (const float*)c->d_topk_cv, (const int32_t*)c->d_topk_ci, Hc, (const int32_t*)c->d_kper, c->d_topk, topk_out);
+  launch_pdl(topk_merge_kernel, dim3(B), dim3(CERB_MAX_HEADS * 32), 0, st, (const float*)c->d_topk_cv, (const int32_t*)c->d_topk_ci, Hc,
+             (const int32_t*)c->d_kper, c->d_topk, topk_out, (const int32_t*)c->d_root, tree ? (const int32_t*)tree->dev.head_of : (const int32_t*)nullptr,
+             tree ? (const int32_t*)tree->dev.rank_of : (const int32_t*)nullptr, plant, tree ? tree->n : 0, tree_tok);
   CERB_LAUNCH_CHECK(c);
-  if (tree_tok) {
-    launch_pdl(tree_fill_kernel, dim3(B), dim3(128), 0, st, (const int32_t*)c->d_root, (const int32_t*)c->d_topk,
-               (const int32_t*)tree->dev.head_of, (const int32_t*)tree->dev.rank_of, plant, Hc, tree->n, tree_tok);
-    CERB_LAUNCH_CHECK(c);
-  }
   return CERB_OK;
 }
 

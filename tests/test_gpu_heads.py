@@ -13,7 +13,8 @@ pytestmark = pytest.mark.gpu
 
 # one column tile, two, three, four (64 weight rows per CTA) and six; widths that are no multiple of a 32-wide k block
 # (264, concatenated 528) and shorter than a pass of all warps; a vocabulary that ends inside a CTA's rows
-@pytest.mark.parametrize("d,vocab", [(264, 1003), (64, 70), (1024, 2048)])
+# (and top-k chunks of less than a warp's lanes, of several lists and, at 140000, of more than the 512 entries a warp holds)
+@pytest.mark.parametrize("d,vocab", [(264, 1003), (64, 70), (1024, 2048), (64, 140000)])
 @pytest.mark.parametrize("B", [1, 2, 3, 5, 8, 9, 13, 16])
 def test_draft_logits_match_oracle(B, d, vocab):
     ms = synth.ModelShape(1, d, 2, 64, 128, vocab, "bf16")
