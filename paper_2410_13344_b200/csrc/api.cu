@@ -237,27 +237,33 @@ unsigned long long* gemm_clock_slot(cerb_ctx* c) {
   return c->d_gemm_clock + c->gemm_clock_used++;
 }
 
-// X . W^T as fp32 split partials in d_part; returns the split count.  A caller that knows there is one slot (more than 128
-// rows) may have it elsewhere (out).
+// X . W^T as fp32 split partials in d_part; returns the split count.  A caller that knows there is one slot (up to kFewRows
+// rows, more than 128) may have it elsewhere (out).
 int gemm(cerb_ctx* c, const void* X, const ActMaps* xm, const void* W, const CUtensorMap* wm, int M, int N, int K,
          int* nsplit, cudaStream_t st, float* out = nullptr) {
   if (c->bf16) {
+    if (M <= kFewRows) {
+      *nsplit = 1;
+      return launch_gemm_few(X, W, out ? out : c->d_part, M, N, K, st, nullptr, nullptr, gemm_clock_slot(c));
+    }
     int ns = gemm_plan_split(c->sm_count, M, N, K);
     if ((size_t)ns * M * N > c->part_floats) return CERB_E_NOMEM;
     *nsplit = ns;
     if (M > 128)
       return launch_gemm_tile(c, wm, xm, make_tile_plan(M, N, K), out ? out : c->d_part, c->d_gemm_fix, c->d_gemm_tickets, M, N, c->d_status, st,
                               nullptr, gemm_clock_slot(c));
-    return launch_gemm_bf16(c, wm, xm, c->d_part, M, N, K, ns, c->d_status, st, nullptr, gemm_clock_slot(c));
+    return launch_gemm_bf16(c, wm, xm, c->d_part, M, N, K, ns, c->d_status, st, gemm_clock_slot(c));
   }
   if ((size_t)M * N > c->part_floats) return CERB_E_NOMEM;
   *nsplit = 1;
   return launch_gemm_f32(c, (const float*)X, (const float*)W, c->d_part, M, N, K, st);
 }
 
-// The same for a GEMM of more than 128 rows that ends in a fused epilogue.
-int gemm_fused(cerb_ctx* c, const ActMaps* xm, const CUtensorMap* wm, int M, int N, int K, const GemmEpilogue& epi, cudaStream_t st) {
+// The same for a GEMM that ends in a fused epilogue.
+int gemm_fused(cerb_ctx* c, const void* X, const ActMaps* xm, const void* W, const CUtensorMap* wm, int M, int N, int K,
+               const GemmEpilogue& epi, cudaStream_t st, const GemmNorm* norm = nullptr) {
   ProfScope ps(c, K_GEMM, st);
+  if (M <= kFewRows) return launch_gemm_few(X, W, nullptr, M, N, K, st, &epi, norm, gemm_clock_slot(c));
   return launch_gemm_tile(c, wm, xm, make_tile_plan(M, N, K), nullptr, c->d_gemm_fix, c->d_gemm_tickets, M, N, c->d_status, st, &epi,
                           gemm_clock_slot(c));
 }
@@ -267,9 +273,11 @@ int gemm_fused(cerb_ctx* c, const ActMaps* xm, const CUtensorMap* wm, int M, int
 struct OrderCheck {
   int ids[kLayerLaunches];
   int n, pos;
+  bool fresh = true;
   explicit OrderCheck(int variant) : pos(0) { n = launch_order_layer(variant, ids); }
   bool next(int id) {
     if (id == LO_NORM_FINAL) return pos == 0;
+    if (id == LO_NORM_ATTN && ids[0] != id && fresh) { fresh = false; return pos == 0; }       // the embedding, in front of the layers
     const bool ok = ids[pos] == id;
     pos = (pos + 1) % n;
     return ok;
@@ -307,14 +315,15 @@ int forward_rows(cerb_ctx* c, const cerb_tree* tree, const int32_t* tok, int tok
     if (c->h_len[b] + nb > c->max_pos) return CERB_E_STATE;
     if (c->h_len[b] + nb > max_len) max_len = c->h_len[b] + nb;
   }
-  // Steps of up to 16 rows: SwiGLU runs in the gate-up GEMM's epilogue and (head_dim 128) RoPE + cache append in the
-  // QKV GEMM's.
-  // More than 128 rows: so does whatever follows a GEMM, the residual adds included.
-  const bool wide = c->bf16 && M > 128;
-  const bool fuse_swiglu = wide ? F % 16 == 0 : c->bf16 && gemm_swiglu_fusable(M, F);
-  const bool fuse_rope = wide ? g.head_dim == 128 : fuse_swiglu && gemm_rope_fusable(M, g.head_dim);
+  // Up to 16 rows and above 128, whatever follows a GEMM runs in its epilogue: SwiGLU, (head_dim 128) RoPE + cache append,
+  // the residual adds.
+  const bool wide = c->bf16 && (M > 128 || M <= kFewRows);
+  const bool fuse_swiglu = wide && (M <= kFewRows || F % 16 == 0);
+  const bool fuse_rope = wide && g.head_dim == 128;
   const bool fuse_res = wide;
-  OrderCheck oc(launch_order_variant({fuse_swiglu, fuse_rope, fuse_res}));
+  // Very few rows: the gate-up and QKV GEMMs normalise their rows themselves (the first layer's QKV GEMM excepted).
+  const bool fuse_norm = fuse_swiglu && fuse_rope && M <= kFewRows && gemm_few_normalises(M, d);
+  OrderCheck oc(launch_order_variant({fuse_swiglu, fuse_rope, fuse_res, fuse_norm}));
   // embedding gather fused with the first layer's attention norm
   CERB_ORDER(oc, LO_NORM_ATTN);
   { ProfScope ps(c, K_GLUE, st);
@@ -335,13 +344,8 @@ int forward_rows(cerb_ctx* c, const cerb_tree* tree, const int32_t* tok, int tok
       const RopeEpilogue re{c->d_len, c->d_nactive, tree->dev.depth, c->page_table, row_off, c->d_rope, c->d_q,
                             (void*)a.k_pool, (void*)a.v_pool, g.max_pages, c->max_pos, n, g.n_heads, B};
       const GemmEpilogue epi{2, nullptr, c->d_gemm_tickets, &re, nullptr};
-      if (wide) CERB_TRY(gemm_fused(c, &c->tm_xn, &c->tm_wqkv_rot[l], M, 3 * HD, d, epi, st));
-      else {
-        ProfScope ps(c, K_GEMM, st);
-        const int nsl = gemm_plan_split(c->sm_count, M, 3 * HD, d);
-        if ((size_t)nsl * M * 3 * HD > c->part_floats) return CERB_E_NOMEM;
-        CERB_TRY(launch_gemm_bf16(c, &c->tm_wqkv[l], &c->tm_xn, c->d_part, M, 3 * HD, d, nsl, c->d_status, st, &epi, gemm_clock_slot(c)));
-      }
+      const GemmNorm nm{(const float*)c->d_x, c->attn_norm[l], g.rms_eps};
+      CERB_TRY(gemm_fused(c, c->d_xn, &c->tm_xn, c->wqkv[l], &c->tm_wqkv_rot[l], M, 3 * HD, d, epi, st, fuse_norm && l ? &nm : nullptr));
     } else {
       { ProfScope ps(c, K_GEMM, st);
         CERB_TRY(gemm(c, c->d_xn, &c->tm_xn, c->wqkv[l], c->bf16 ? &c->tm_wqkv[l] : nullptr, M, 3 * HD, d, &ns, st)); }
@@ -354,25 +358,21 @@ int forward_rows(cerb_ctx* c, const cerb_tree* tree, const int32_t* tok, int tok
                                      c->sm_count, c->d_status, st, row_off, tree == c->chain)); }
     CERB_ORDER(oc, LO_GEMM_WO);
     const GemmEpilogue res{3, nullptr, c->d_gemm_tickets, nullptr, (float*)c->d_x};
-    if (fuse_res) CERB_TRY(gemm_fused(c, &c->tm_attn, &c->tm_wo[l], M, d, HD, res, st));
+    if (fuse_res) CERB_TRY(gemm_fused(c, c->d_attn, &c->tm_attn, c->wo[l], &c->tm_wo[l], M, d, HD, res, st));
     else { ProfScope ps(c, K_GEMM, st);
       CERB_TRY(gemm(c, c->d_attn, &c->tm_attn, c->wo[l], c->bf16 ? &c->tm_wo[l] : nullptr, M, d, HD, &ns, st)); }
     if (fuse_res) ns = 0;
     // residual add fused with the MLP norm
-    CERB_ORDER(oc, LO_NORM_MLP);
-    { ProfScope ps(c, K_GLUE, st);
+    if (!fuse_norm) {
+      CERB_ORDER(oc, LO_NORM_MLP);
+      ProfScope ps(c, K_GLUE, st);
       CERB_TRY(launch_fused_norm(c, c->d_part, ns, (size_t)M * d, nullptr, 0, 0, n, c->mlp_norm[l], c->d_xn, M, st, nullptr, fuse_res)); }
     CERB_ORDER(oc, LO_GEMM_GU);
     if (fuse_swiglu) {
       // SwiGLU runs in the GEMM's epilogue: no separate kernel, no second pass over the partial sums
       const GemmEpilogue epi{1, c->d_act, c->d_gemm_tickets, nullptr, nullptr};
-      if (wide) CERB_TRY(gemm_fused(c, &c->tm_xn, &c->tm_wgu_pair[l], M, 2 * F, d, epi, st));
-      else {
-        ProfScope ps(c, K_GEMM, st);
-        const int nsl = gemm_plan_split(c->sm_count, M, 2 * F, d);
-        if ((size_t)nsl * M * 2 * F > c->part_floats) return CERB_E_NOMEM;
-        CERB_TRY(launch_gemm_bf16(c, &c->tm_wgu[l], &c->tm_xn, c->d_part, M, 2 * F, d, nsl, c->d_status, st, &epi, gemm_clock_slot(c)));
-      }
+      const GemmNorm nm{(const float*)c->d_x, c->mlp_norm[l], g.rms_eps};
+      CERB_TRY(gemm_fused(c, c->d_xn, &c->tm_xn, c->wgu[l], &c->tm_wgu_pair[l], M, 2 * F, d, epi, st, fuse_norm ? &nm : nullptr));
     } else {
       { ProfScope ps(c, K_GEMM, st);
         CERB_TRY(gemm(c, c->d_xn, &c->tm_xn, c->wgu[l], c->bf16 ? &c->tm_wgu[l] : nullptr, M, 2 * F, d, &ns, st)); }
@@ -380,11 +380,12 @@ int forward_rows(cerb_ctx* c, const cerb_tree* tree, const int32_t* tok, int tok
       { ProfScope ps(c, K_GLUE, st); CERB_TRY(launch_swiglu(c, c->d_part, ns, (size_t)M * 2 * F, c->d_act, M, st)); }
     }
     CERB_ORDER(oc, LO_GEMM_DOWN);
-    if (fuse_res) CERB_TRY(gemm_fused(c, &c->tm_act, &c->tm_wd[l], M, d, F, res, st));
+    if (fuse_res) CERB_TRY(gemm_fused(c, c->d_act, &c->tm_act, c->wd[l], &c->tm_wd[l], M, d, F, res, st));
     else { ProfScope ps(c, K_GEMM, st);
       CERB_TRY(gemm(c, c->d_act, &c->tm_act, c->wd[l], c->bf16 ? &c->tm_wd[l] : nullptr, M, d, F, &ns, st)); }
     if (fuse_res) ns = 0;
     // residual add fused with the next layer's attention norm, or with the final norm
+    if (fuse_norm && l + 1 < g.n_layers) continue;
     CERB_ORDER(oc, l + 1 == g.n_layers ? LO_NORM_FINAL : LO_NORM_ATTN);
     { ProfScope ps(c, K_GLUE, st);
       const bool last = l + 1 == g.n_layers;
@@ -399,7 +400,7 @@ int lm_head_argmax(cerb_ctx* c, const void* X, const ActMaps* xm, int rows, int3
                    cudaStream_t st) {
   int ns = 1;
   // one slot: the GEMM writes the caller's logits itself, and the argmax reads them there
-  const bool direct = logits_out && c->bf16 && rows > 128;
+  const bool direct = logits_out && c->bf16 && (rows > 128 || rows <= kFewRows);
   { ProfScope ps(c, K_GEMM, st);
     CERB_TRY(gemm(c, X, xm, c->lm_head, c->bf16 ? &c->tm_lm_head : nullptr, rows, c->cfg.vocab, c->cfg.d_model, &ns, st,
                   direct ? logits_out : nullptr)); }
@@ -814,6 +815,7 @@ int cerb_gemm(int32_t dtype, const void* X_dev, const void* W_dev, float* out_de
     CERB_TRY(launch_gemm_tile(nullptr, &tw, &tx, g, out_dev, part, tickets, M, N, status, st));
     return CERB_OK;
   }
+  if (M <= kFewRows) return launch_gemm_few(X_dev, W_dev, out_dev, M, N, K, st);
   const int ns = gemm_plan_split(148, M, N, K);
   CERB_TRY(make_act_map(&tx, X_dev, M, K, row_bucket(M)));
   CERB_TRY(launch_gemm_bf16(nullptr, &tw, &tx, part, M, N, K, ns, status, st));

@@ -194,9 +194,9 @@ struct cerb_ctx {
 
 namespace cerb {
 
-// Rows of one pass of the single-CTA GEMM: 16, 32, 64 or 128.
+// Rows of one pass of the single-CTA GEMM: 32, 64 or 128.
 inline int row_bucket(int rows) {
-  int r = 16;
+  int r = 32;
   while (r < rows && r < 128) r <<= 1;
   return r;
 }
@@ -210,7 +210,7 @@ enum { LO_SET_ACTIVE = 0, LO_NORM_ATTN, LO_GEMM_QKV, LO_ROPE, LO_ATTN, LO_GEMM_W
 // What runs in GEMM epilogues: SwiGLU in the gate-up GEMM, RoPE + cache append in the QKV GEMM, the residual add in the O
 // and down GEMMs.
 struct Fusion {
-  bool swiglu, rope, residual;
+  bool swiglu, rope, residual, norm;
 };
 int launch_order_variant(Fusion f);
 int launch_order_layer(int variant, int* ids_out);            // the layer's launches (at most kLayerLaunches)
@@ -235,15 +235,13 @@ int launch_prefill_commit(cerb_ctx* c, cudaStream_t st);
 // gemm_f32.cu / gemm_bf16.cu : out[split][M][N] fp32 partial sums of X[M][K] . W[N][K]^T
 int launch_gemm_f32(cerb_ctx* c, const float* X, const float* W, float* out, int M, int N, int K, cudaStream_t st);
 int gemm_plan_split(int sm_count, int M, int N, int K);
-// Optional fused epilogue of the bf16 GEMM.  kind 1 (SwiGLU): W is [gate rows F][up rows F]; the GEMM
-// pairs gate tile t with up tile t in one unit and the CTA that completes a tile last writes
-// act[row][f] = SiLU(gate) * up (bf16) instead of leaving the partial slots to a separate kernel.
-// kind 2 (RoPE + cache append): W is the QKV matrix [q rows | k rows | v rows] of a model with head_dim 128; the CTA
-// that completes a 256-row tile (two heads' worth of q, k or v) last sums the tile's slots in index order, rotates q
-// and k at position len + depth and writes q dense and k, v into the paged pools -- what rope_append_kernel does,
-// with the same arithmetic in the same order.  In the single-CTA kernel both pay for steps of up to 16 rows only; above 128
-// rows (gemm_tile.cu) they always run.
-// kind 3 (gemm_tile.cu only): the product is added to the fp32 residual stream.
+// What may follow a bf16 GEMM in its epilogue (gemm_few.cu, up to kFewRows rows; gemm_tile.cu, above 128 rows).
+// kind 1 (SwiGLU): W is [gate rows F][up rows F]; act[row][f] = SiLU(gate) * up (bf16).
+// kind 2 (RoPE + cache append): W is the QKV matrix [q rows | k rows | v rows] of a model with head_dim 128; q and k are
+// rotated at position len + depth, q is written dense and k, v into the paged pools -- what rope_append_kernel does, with the
+// same arithmetic in the same order.
+// kind 3: the product is added to the fp32 residual stream.
+// In between (17 to 128 rows) separate kernels do this work: the GEMM leaves partial sums there.
 struct RopeEpilogue {
   const int32_t *len, *n_active, *depth, *page_table, *row_off;    // as for rope_append_kernel (row_off may be null)
   const float2* rope;       // rotation table [max_pos][64]
@@ -268,11 +266,18 @@ size_t gemm_fix_floats();   // of any plan
 int launch_gemm_tile(cerb_ctx* c, const CUtensorMap* tmW, const ActMaps* tmX, const TilePlan& g, float* out, float* fix, unsigned int* tickets,
                      int M, int N, int32_t* status, cudaStream_t st, const GemmEpilogue* epi = nullptr,
                      unsigned long long* clock_slot = nullptr);
-bool gemm_swiglu_fusable(int M, int F);
-bool gemm_rope_fusable(int M, int head_dim);
+// gemm_few.cu: few rows
+constexpr int kFewRows = 16;
+struct GemmNorm {           // the GEMM's X is RMSNorm(x) * gain of the residual stream x [M][K]
+  const float* x;
+  const void* gain;
+  float eps;
+};
+int launch_gemm_few(const void* X, const void* W, float* out, int M, int N, int K, cudaStream_t st, const GemmEpilogue* epi = nullptr,
+                    const GemmNorm* norm = nullptr, unsigned long long* clock_slot = nullptr);
+bool gemm_few_normalises(int M, int K);
 int launch_gemm_bf16(cerb_ctx* c, const CUtensorMap* tmW, const ActMaps* tmX, float* out, int M, int N, int K,
-                     int nsplit, int32_t* status, cudaStream_t st, const GemmEpilogue* epi = nullptr,
-                     unsigned long long* clock_slot = nullptr);
+                     int nsplit, int32_t* status, cudaStream_t st, unsigned long long* clock_slot = nullptr);
 int make_weight_map(CUtensorMap* out, const void* W, int N, int K);
 int make_gate_up_map(CUtensorMap* out, const void* W, int F, int K);
 int make_rotation_map(CUtensorMap* out, const void* W, int heads, int K);

@@ -55,7 +55,7 @@ struct GemmParams {
   float* out;
   int32_t* status;
   int M, N, K;
-  int n_mma;          // activation rows per pass (16..128, power of two)
+  int n_mma;          // activation rows per pass (32..128, power of two)
   int num_kb;         // ceil(K / 64)
   int tiles;          // ceil(N / 128)
   int per;            // work units per CTA
@@ -67,11 +67,6 @@ struct GemmParams {
   uint32_t acc_cols;  // TMEM columns of one accumulator buffer
   int tile_rows;      // weight rows between the starts of consecutive tiles
   int half_off;       // weight-row offset of a wide unit's second tile from its first
-  int epi;            // fused epilogue (GemmEpilogue::kind)
-  int F;              // SwiGLU: width of the gate (and of the up) block
-  bf16* act;          // SwiGLU: output [M][F]
-  unsigned int* tickets;
-  RopeEpilogue re;    // RoPE + cache append (epi == 2)
   unsigned long long* clk;   // measurement only: clk[0] <- min over CTAs of the time the dependency wait returned,
                              // clk[kGemmClockSlots] <- max over CTAs of the time the CTA finished (globaltimer, ns); or null
 };
@@ -101,7 +96,6 @@ __global__ void __launch_bounds__(224, 1) gemm_bf16_kernel(const __grid_constant
   __shared__ __align__(8) uint64_t drain_bar[2];       // one per MMA issuer: "everything I issued has retired" (give-up path only)
   __shared__ uint32_t tmem_base_slot;
   __shared__ int aborted_s;
-  __shared__ unsigned int ticket_s;
   volatile int* aborted = &aborted_s;
   const WaitCtx wc{p.wait_cycles, aborted, p.status, p.N + 100000 * (p.M > 999 ? 999 : p.M)};
 
@@ -249,29 +243,6 @@ __global__ void __launch_bounds__(224, 1) gemm_bf16_kernel(const __grid_constant
       const int m_base = 0;                            // (all rows in one pass: this kernel takes up to 128)
       const int m_cnt = p.M;
       const size_t ldo = (size_t)p.N;
-      const int cnt = last_cta - first_cta + 1;        // CTAs that share this job = slots it uses
-      if (p.epi == 1 && cnt == 1) {
-        // SwiGLU, whole tile in this CTA: gate in the first accumulator half, up in the second
-        const int f = tile * p.tile_rows + quarter * 32 + lane;
-        bf16* a = p.act + (size_t)m_base * p.F + f;
-        const uint32_t tg = tmem_base + (uint32_t)buf * p.acc_cols + ((uint32_t)(quarter * 32) << 16);
-        for (int c0 = 0; c0 < m_cnt; c0 += 16) {
-          uint32_t rg[16], ru[16];
-          tmem_ld16(tg + (uint32_t)c0, rg);
-          tmem_ld16(tg + (uint32_t)p.n_mma + (uint32_t)c0, ru);
-#pragma unroll
-          for (int j = 0; j < 16; ++j)
-            if (c0 + j < m_cnt) {
-              const float gv = __uint_as_float(rg[j]), uv = __uint_as_float(ru[j]);
-              a[(size_t)(c0 + j) * p.F] = __float2bfloat16_rn(gv / (1.0f + expf(-gv)) * uv);
-            }
-        }
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(smem_u32(&acc_empty[buf]));
-        ++g;
-        continue;
-      }
       for (int hf = 0; hf < 2; ++hf) {
         const int n_out = tile * p.tile_rows + hf * p.half_off + quarter * 32 + lane;
         const bool n_ok = n_out < p.N;
@@ -296,7 +267,7 @@ __global__ void __launch_bounds__(224, 1) gemm_bf16_kernel(const __grid_constant
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(smem_u32(&acc_empty[buf]));
-      if (p.epi == 0 && share == last_cta) {
+      if (share == last_cta) {
         for (int hf = 0; hf < 2; ++hf) {
           const int n_out = tile * p.tile_rows + hf * p.half_off + quarter * 32 + lane;
           if (n_out >= p.N) continue;
@@ -304,103 +275,6 @@ __global__ void __launch_bounds__(224, 1) gemm_bf16_kernel(const __grid_constant
             float* zo = p.out + ((size_t)z * p.M + m_base) * ldo + n_out;
             for (int m = 0; m < m_cnt; ++m) { *zo = 0.f; zo += ldo; }
           }
-        }
-      }
-      if (p.epi == 1) {
-        // The CTA that finishes this tile last (by ticket) adds the tile's slots in index order and applies SwiGLU.
-        __threadfence();
-        asm volatile("bar.sync 2, 128;" ::: "memory");
-        if (warp == 2 && lane == 0) ticket_s = atomicAdd(&p.tickets[sg.job], 1u);
-        asm volatile("bar.sync 2, 128;" ::: "memory");
-        if (ticket_s == (unsigned)cnt - 1u) {
-          __threadfence();
-          const int f = tile * p.tile_rows + quarter * 32 + lane;
-          const float* src = p.out + (size_t)m_base * ldo + f;
-          bf16* a = p.act + (size_t)m_base * p.F + f;
-          const size_t sstride = (size_t)p.M * ldo;
-#pragma unroll 4
-          for (int m = 0; m < m_cnt; ++m) {
-            float gv = 0.f, uv = 0.f;
-            for (int z = 0; z < cnt; ++z) {
-              gv += __ldcg(src + z * sstride + (size_t)m * ldo);
-              uv += __ldcg(src + z * sstride + (size_t)m * ldo + p.F);
-            }
-            a[(size_t)m * p.F] = __float2bfloat16_rn(gv / (1.0f + expf(-gv)) * uv);
-          }
-          if (warp == 2 && lane == 0) p.tickets[sg.job] = 0u;      // ready for the next launch
-        }
-      }
-      if (p.epi == 2) {
-        // The CTA that finishes this tile last (by ticket) adds the tile's slots in index order, rotates q and k and
-        // stores q, k and v where the attention kernel expects them.  A thread owns one output column (= weight row)
-        // of each half of the unit; the other element of its rotation pair is 64 columns away in the same head.
-        __threadfence();
-        asm volatile("bar.sync 2, 128;" ::: "memory");
-        if (warp == 2 && lane == 0) ticket_s = atomicAdd(&p.tickets[sg.job], 1u);
-        asm volatile("bar.sync 2, 128;" ::: "memory");
-        if (ticket_s == (unsigned)cnt - 1u) {
-          __threadfence();
-          const RopeEpilogue& e = p.re;
-          const int HD = e.H * 128;
-          const size_t sstride = (size_t)p.M * ldo;
-          // this thread's two output columns (one per half of the unit) and their rotation partners
-          int col[2], which[2], hd[2];
-          bool col_ok[2];
-#pragma unroll
-          for (int hf = 0; hf < 2; ++hf) {
-            col[hf] = tile * p.tile_rows + hf * p.half_off + quarter * 32 + lane;
-            col_ok[hf] = col[hf] < 3 * HD;
-            which[hf] = col_ok[hf] ? col[hf] / HD : 2;
-            hd[hf] = col[hf] - which[hf] * HD;
-          }
-          for (int m = 0; m < m_cnt; ++m) {
-            int b, v;
-            locate_row(m, e.row_off, e.B, e.n, b, v);
-            const int na = e.n_active[b], L = e.len[b], dep = e.depth[v];
-            // every slot value this thread needs, requested before any of them is used (one round trip to L2)
-            constexpr int ZMAX = 6;
-            float own[2][ZMAX], oth[2][ZMAX];
-            const float* src = p.out + (size_t)m * ldo;
-#pragma unroll
-            for (int hf = 0; hf < 2; ++hf) {
-              const int i = hd[hf] & 127;
-              const int partner = i < 64 ? col[hf] + 64 : col[hf] - 64;
-#pragma unroll
-              for (int z = 0; z < ZMAX; ++z) {
-                const bool take = col_ok[hf] && z < cnt;
-                own[hf][z] = take ? __ldcg(src + z * sstride + col[hf]) : 0.f;
-                oth[hf][z] = take && which[hf] < 2 ? __ldcg(src + z * sstride + partner) : 0.f;
-              }
-            }
-            const int pos = L + dep, slot = L + v;
-            const bool ok = v < na && pos < e.max_pos && slot < e.max_pos;
-            const int page = ok ? e.page_table[(size_t)b * e.max_pages + slot / CERB_PAGE] : 0;
-            float2 cs[2];
-#pragma unroll
-            for (int hf = 0; hf < 2; ++hf) cs[hf] = ok && which[hf] < 2 ? e.rope[(size_t)pos * 64 + (hd[hf] & 63)] : make_float2(1.f, 0.f);
-#pragma unroll
-            for (int hf = 0; hf < 2; ++hf) {
-              if (!col_ok[hf] || !ok) continue;
-              const int i = hd[hf] & 127, h = hd[hf] >> 7;
-              float a = 0.f, o2 = 0.f;
-#pragma unroll
-              for (int z = 0; z < ZMAX; ++z) { a += own[hf][z]; o2 += oth[hf][z]; }        // slots in index order
-              for (int z = ZMAX; z < cnt; ++z) {                                          // (more slots than usual)
-                const int partner = i < 64 ? col[hf] + 64 : col[hf] - 64;
-                a += __ldcg(src + z * sstride + col[hf]);
-                if (which[hf] < 2) o2 += __ldcg(src + z * sstride + partner);
-              }
-              float val = a;
-              if (which[hf] < 2) val = i < 64 ? a * cs[hf].x - o2 * cs[hf].y : a * cs[hf].x + o2 * cs[hf].y;
-              if (which[hf] == 0) {
-                reinterpret_cast<bf16*>(e.q)[(size_t)m * HD + hd[hf]] = __float2bfloat16_rn(val);
-              } else {
-                bf16* pool = reinterpret_cast<bf16*>(which[hf] == 1 ? e.kpool : e.vpool);
-                pool[(((size_t)page * e.H + h) * CERB_PAGE + (size_t)(slot % CERB_PAGE)) * 128 + i] = __float2bfloat16_rn(val);
-              }
-            }
-          }
-          if (warp == 2 && lane == 0) p.tickets[sg.job] = 0u;      // ready for the next launch
         }
       }
       ++g;
@@ -566,18 +440,6 @@ int make_pool_map(CUtensorMap* out, const void* pool, int n_pool_pages, int H, i
   return encode_2d(out, pool, (uint64_t)Dh, (uint64_t)n_pool_pages * H * CERB_PAGE, (uint64_t)Dh * 2, 64, CERB_PAGE);
 }
 
-// The fused SwiGLU epilogue needs the wide schedule (both halves of a unit in one CTA) and whole tiles.
-// It pays for few rows only (the auto-regressive step): the CTA that completes a tile re-reads the
-// tile's slots with its 128 epilogue threads, which at 64 rows took 55 us per layer against the
-// 6.6 us of the separate kernel that spreads the same bytes over every SM (measured).
-bool gemm_swiglu_fusable(int M, int F) {
-  return M >= 1 && M <= 16 && F % BM == 0;
-}
-// The same reasoning for the RoPE + cache-append epilogue of the QKV GEMM (head_dim 128: a 128-row weight tile is one
-// head, so both elements of every rotation pair lie in the tile that the finishing CTA owns).
-bool gemm_rope_fusable(int M, int head_dim) {
-  return M >= 1 && M <= 16 && head_dim == 128;
-}
 // Number of partial slots the schedule produces for this problem (what consumers must sum).
 int gemm_plan_split(int sm_count, int M, int N, int K) {
   return M > BM ? 1 : make_plan(sm_count, N, K).nslots;
@@ -596,7 +458,7 @@ int gemm_scratch_slots(int M, int N, int K) {
 }
 
 int launch_gemm_bf16(cerb_ctx* c, const CUtensorMap* tmW, const ActMaps* tmX, float* out, int M, int N, int K,
-                     int nsplit, int32_t* status, cudaStream_t st, const GemmEpilogue* epi, unsigned long long* clock_slot) {
+                     int nsplit, int32_t* status, cudaStream_t st, unsigned long long* clock_slot) {
   if (M <= 0 || N <= 0 || K <= 0 || (K % 8) != 0) return CERB_E_SHAPE;
   if (M > BM) return CERB_E_SHAPE;             // (gemm_tile.cu)
   // Fewer SMs than planned for would need more slots than the caller sized: plan with the number
@@ -618,18 +480,7 @@ int launch_gemm_bf16(cerb_ctx* c, const CUtensorMap* tmW, const ActMaps* tmX, fl
   p.tile_rows = 2 * BM;
   p.wait_cycles = wait_cycles();
   p.half_off = BM;
-  p.epi = 0; p.F = 0; p.act = nullptr; p.tickets = nullptr;
   p.clk = clock_slot;
-  if (epi && epi->kind == 1) {
-    if (!gemm_swiglu_fusable(M, N / 2) || (N & 1) || g.tiles > kGemmTickets || !epi->act || !epi->tickets) return CERB_E_SHAPE;
-    p.epi = 1; p.F = N / 2; p.act = (bf16*)epi->act; p.tickets = epi->tickets;
-    p.tile_rows = BM;            // a unit = gate tile t (rows t*128..) and up tile t (rows F + t*128..)
-    p.half_off = p.F;
-  }
-  if (epi && epi->kind == 2) {
-    if (!epi->rope || !gemm_rope_fusable(M, 128) || N != 3 * epi->rope->H * 128 || g.tiles > kGemmTickets || !epi->tickets) return CERB_E_SHAPE;
-    p.epi = 2; p.tickets = epi->tickets; p.re = *epi->rope;
-  }
   uint32_t stage_bytes = 2 * A_STAGE_BYTES + (uint32_t)p.n_mma * BK * 2;
   p.stages = (int)((216u * 1024u) / stage_bytes);
   if (p.stages > MAX_STAGES) p.stages = MAX_STAGES;

@@ -374,7 +374,7 @@ int launch_fused_norm(cerb_ctx* c, const float* part, int nsplit, size_t split_s
   const cerb_config& g = c->cfg;
   const int d = g.d_model;
   if (d % 4 || d > NORM_THREADS * NORM_MAX_ITER * 4) return CERB_E_SHAPE;
-  if (c->bf16 && nsplit == 0 && rows > 128 && out) {
+  if (c->bf16 && nsplit == 0 && (rows > 128 || rows <= kFewRows) && out) {
     auto wide = [&](auto iter) {
       launch_pdl(row_norm_kernel<bf16, decltype(iter)::value>, dim3(rows), dim3(ROWS_THREADS), 0, st, (float*)c->d_x,
                  tok ? (const bf16*)c->embed : (const bf16*)nullptr, tok, tok_stride, tok_off, (const int32_t*)c->d_nactive, n, g.vocab,

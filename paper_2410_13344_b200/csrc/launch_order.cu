@@ -63,22 +63,29 @@ const Entry kNormAttnRead = {LO_NORM_ATTN, "fused_norm (attention norm)", B_X | 
 const Entry kNormMlpRead = {LO_NORM_MLP, "fused_norm (MLP norm)", B_XN, B_CONST};
 const Entry kNormFinalRead = {LO_NORM_FINAL, "fused_norm (final norm)", B_HIDDEN, B_CONST};
 
-// Variants 0, 1 and 2 are the steps of up to 128 rows; the others occur above.
-constexpr int kVariants = 8;
-const Fusion kFusion[kVariants] = {  // {swiglu, rope, residual}
+// The norms in the GEMMs that read them, which then read the residual stream after their wait; the embedding gather with the
+// first attention norm stays, in front of the layers.
+const Entry kNormEmbed = {LO_NORM_ATTN, "fused_norm (embedding, attention norm)", B_X | B_XN, B_CONST};
+const Entry kQkvNorm = {LO_GEMM_QKV, "gemm norm + qkv + rope / append epilogue", B_Q | B_KV, B_CONST};
+const Entry kGuNorm = {LO_GEMM_GU, "gemm norm + gate-up + swiglu epilogue", B_ACT, B_CONST};
+
+// Variant 0 is the steps of 17 to 128 rows; those with a residual add in the GEMMs occur above and up to 16 rows, the norms in
+// the GEMMs (8) with one or two.
+constexpr int kVariants = 9;
+const Fusion kFusion[kVariants] = {  // {swiglu, rope, residual, norm}
     {false, false, false}, {true, false, false}, {true, true, false}, {true, true, true},
-    {false, true, false},  {false, false, true}, {true, false, true}, {false, true, true}};
+    {false, true, false},  {false, false, true}, {true, false, true}, {false, true, true}, {true, true, true, true}};
 
 int layer(int variant, const Entry** out) {
   const Fusion& f = kFusion[variant];
   int n = 0;
-  out[n++] = f.residual ? &kNormAttnRead : &kNormAttn;
-  out[n++] = f.rope ? &kQkvRope : &kQkv;
+  if (!f.norm) out[n++] = f.residual ? &kNormAttnRead : &kNormAttn;
+  out[n++] = f.norm ? &kQkvNorm : f.rope ? &kQkvRope : &kQkv;
   if (!f.rope) out[n++] = &kRope;
   out[n++] = &kAttn;
   out[n++] = f.residual ? &kWoAdd : &kWo;
-  out[n++] = f.residual ? &kNormMlpRead : &kNormMlp;
-  out[n++] = f.swiglu ? &kGuSwiglu : &kGu;
+  if (!f.norm) out[n++] = f.residual ? &kNormMlpRead : &kNormMlp;
+  out[n++] = f.norm ? &kGuNorm : f.swiglu ? &kGuSwiglu : &kGu;
   if (!f.swiglu) out[n++] = &kSwiglu;
   out[n++] = f.residual ? &kDownAdd : &kDown;
   return n;
@@ -88,6 +95,7 @@ int build(int variant, const Entry** out) {
   // set-up, three layers (enough to close the cycle between layers), tail
   int n = 0;
   out[n++] = &kSetActive;
+  if (kFusion[variant].norm) out[n++] = &kNormEmbed;
   for (int l = 0; l < 3; ++l) n += layer(variant, out + n);
   out[n++] = kFusion[variant].residual ? &kNormFinalRead : &kNormFinal;
   out[n++] = &kLm;
@@ -99,7 +107,7 @@ int build(int variant, const Entry** out) {
 
 int launch_order_variant(Fusion f) {
   for (int v = 0; v < kVariants; ++v)
-    if (kFusion[v].swiglu == f.swiglu && kFusion[v].rope == f.rope && kFusion[v].residual == f.residual) return v;
+    if (kFusion[v].swiglu == f.swiglu && kFusion[v].rope == f.rope && kFusion[v].residual == f.residual && kFusion[v].norm == f.norm) return v;
   return 0;
 }
 
