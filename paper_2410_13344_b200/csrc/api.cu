@@ -315,7 +315,7 @@ int forward_rows(cerb_ctx* c, const cerb_tree* tree, const int32_t* tok, int tok
     if (c->h_len[b] + nb > c->max_pos) return CERB_E_STATE;
     if (c->h_len[b] + nb > max_len) max_len = c->h_len[b] + nb;
   }
-  // Up to 16 rows and above 128, whatever follows a GEMM runs in its epilogue: SwiGLU, (head_dim 128) RoPE + cache append,
+  // Up to 8 rows and above 128, whatever follows a GEMM runs in its epilogue: SwiGLU, (head_dim 128) RoPE + cache append,
   // the residual adds.
   const bool wide = c->bf16 && (M > 128 || M <= kFewRows);
   const bool fuse_swiglu = wide && (M <= kFewRows || F % 16 == 0);

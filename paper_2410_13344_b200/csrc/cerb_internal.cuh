@@ -241,7 +241,7 @@ int gemm_plan_split(int sm_count, int M, int N, int K);
 // rotated at position len + depth, q is written dense and k, v into the paged pools -- what rope_append_kernel does, with the
 // same arithmetic in the same order.
 // kind 3: the product is added to the fp32 residual stream.
-// In between (17 to 128 rows) separate kernels do this work: the GEMM leaves partial sums there.
+// In between (9 to 128 rows) separate kernels do this work: the GEMM leaves partial sums there.
 struct RopeEpilogue {
   const int32_t *len, *n_active, *depth, *page_table, *row_off;    // as for rope_append_kernel (row_off may be null)
   const float2* rope;       // rotation table [max_pos][64]
@@ -267,7 +267,7 @@ int launch_gemm_tile(cerb_ctx* c, const CUtensorMap* tmW, const ActMaps* tmX, co
                      int M, int N, int32_t* status, cudaStream_t st, const GemmEpilogue* epi = nullptr,
                      unsigned long long* clock_slot = nullptr);
 // gemm_few.cu: few rows
-constexpr int kFewRows = 16;
+constexpr int kFewRows = 8;
 struct GemmNorm {           // the GEMM's X is RMSNorm(x) * gain of the residual stream x [M][K]
   const float* x;
   const void* gain;

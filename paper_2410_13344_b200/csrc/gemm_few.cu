@@ -12,9 +12,10 @@
 // next one, and at the start ahead of the wait for the kernel in front.  Loads in flight occupy the L1, so the kernel asks for
 // no more shared memory than it needs: with the largest share of it a step took 1.6 times as long.
 //
-// 7B shape, 16 layers and LM head, 1000 tokens before, us per forward of 1 / 2 / 4 / 8 / 12 rows: 1410 / 1381 / 1551 / 1797 /
-// 1881; with tensor-memory tiles of 256 weight rows, partial sums in slots and a norm kernel of its own 1664 / 1654 / 1815 /
-// 2138 / 2149.  Warps that take k blocks in turn instead of an eighth each: 1436 with one row.
+// 7B shape, 16 layers and LM head, 1000 tokens before, us per forward of 1 / 2 / 4 / 8 rows: 1410 / 1381 / 1551 / 1597; with the
+// tensor-memory tiles of gemm_bf16.cu, whose partial sums then meet in separate kernels, 1664 / 1623 / 1648 / 1643 (4 and 8 rows
+// as one tree).  From nine rows on, a second column tile per MMA row and twice the activation reads cost more than that: 12
+// rows 1868 against 1657.
 #include <string.h>
 
 #include "cerb_internal.cuh"
@@ -24,6 +25,9 @@ namespace cerb {
 namespace {
 
 constexpr int WARPS = 8;
+constexpr int U = 4;                 // 32-wide k blocks of a round
+constexpr int ROWS = 16, LD = kFewRows + 1, ROUND = 32 * U;
+constexpr int CTAS = 2 * 148;
 
 struct FewParams {
   const bf16* X;
@@ -52,25 +56,23 @@ __device__ __forceinline__ void mma_16816(float* c, uint32_t a0, uint32_t a1, ui
       : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
 }
 
-// KIND as in GemmEpilogue.  NT: column tiles of eight activation rows; KG warps to a row group; U: k blocks of a round; MB CTAs
-// to an SM.  The 16 rows of a group are 16 neighbours (0, 3), or eight and the eight that belong to them (1: gate, up; 2:
+// KIND as in GemmEpilogue.  A tile's 16 rows are neighbours (0, 3), or eight and the eight that belong to them (1: gate, up; 2:
 // elements i and i + 64 of a head).
-template <int KIND, int NT, int KG, int U, int MB, bool XB, bool NORM>
-__global__ void __launch_bounds__(WARPS * 32, MB) gemm_few_kernel(const __grid_constant__ FewParams p) {
+template <int KIND, bool NORM>
+__global__ void __launch_bounds__(WARPS * 32, 2) gemm_few_kernel(const __grid_constant__ FewParams p) {
   constexpr bool PAIRS = KIND == 1 || KIND == 2;
-  constexpr int RG = WARPS / KG, ROWS = 16 * RG, LD = 8 * NT + 1, ROUND = 32 * U;
-  constexpr int OUTS = PAIRS ? ROWS / 2 : ROWS, ITEMS = (OUTS * 8 * NT + WARPS * 32 - 1) / (WARPS * 32);
-  __shared__ float red_s[2][KG * ROWS * LD];                 // [tile's parity][k group][row][column + 1]
+  constexpr int OUTS = PAIRS ? ROWS / 2 : ROWS;
+  __shared__ float red_s[2][WARPS * ROWS * LD];              // [tile's parity][warp][row][column + 1]
   extern __shared__ __align__(16) bf16 xs[];                 // NORM: the normalised rows, then the gains; [.][K + 32]
-  const int kg = (threadIdx.x >> 5) % KG, rg = (threadIdx.x >> 5) / KG, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
   const int K = p.K;
   // a tile's first row (of a pair: its first member)
   auto first_row = [](int tile) { return KIND == 2 ? (tile / (64 / OUTS)) * 128 + (tile % (64 / OUTS)) * OUTS : tile * OUTS; };
   const bf16* Wr[2];
-  const int k0 = kg * p.range + t * 8, k1 = min(K, (kg + 1) * p.range);     // this warp's part of k
+  const int k0 = warp * p.range + t * 8, k1 = min(K, (warp + 1) * p.range);     // this warp's part of k
   int load_tile = blockIdx.x, load_k = k0;                   // what the next load_w fetches
   auto set_rows = [&]() {
-    const int r0 = first_row(load_tile) + (PAIRS ? 8 : 16) * rg + g;
+    const int r0 = first_row(load_tile) + g;
     const int r1 = KIND == 1 ? min(r0, p.F - 1) + p.F : KIND == 2 ? r0 + 64 : r0 + 8;
     Wr[0] = p.W + (size_t)min(r0, (KIND == 1 ? p.F : p.N) - 1) * K;
     Wr[1] = p.W + (size_t)min(r1, p.N - 1) * K;
@@ -87,30 +89,24 @@ __global__ void __launch_bounds__(WARPS * 32, MB) gemm_few_kernel(const __grid_c
                        : "=r"(r[u][e].x), "=r"(r[u][e].y), "=r"(r[u][e].z), "=r"(r[u][e].w) : "l"(Wr[e] + load_k + u * 32));
       }
   };
-  auto load_x = [&](uint4 (&r)[U][NT], int k) {
+  auto load_x = [&](uint4 (&r)[U], int k) {
 #pragma unroll
-    for (int u = 0; u < U; ++u)
-#pragma unroll
-      for (int n = 0; n < NT; ++n) {
-        r[u][n] = make_uint4(0, 0, 0, 0);
-        if (k + u * 32 < k1 && 8 * n + g < p.M)
-          r[u][n] = NORM ? *reinterpret_cast<const uint4*>(xs + (8 * n + g) * (K + 32) + k + u * 32)
-                         : *reinterpret_cast<const uint4*>(p.X + (size_t)(8 * n + g) * K + k + u * 32);
-      }
+    for (int u = 0; u < U; ++u) {
+      r[u] = make_uint4(0, 0, 0, 0);
+      if (k + u * 32 < k1 && g < p.M)
+        r[u] = *reinterpret_cast<const uint4*>(NORM ? xs + g * (K + 32) + k + u * 32 : p.X + (size_t)g * K + k + u * 32);
+    }
   };
   // (two accumulators in turn: the tensor cores cut the sum off at every step, so half the steps is half the error)
-  float acc[2][NT][4];
-  auto multiply = [&](const uint4 (&a)[U][2], const uint4 (&x)[U][NT]) {
+  float acc[2][4];
+  auto multiply = [&](const uint4 (&a)[U][2], const uint4 (&x)[U]) {
 #pragma unroll
-    for (int u = 0; u < U; ++u)
-#pragma unroll
-      for (int n = 0; n < NT; ++n) {
-        mma_16816(acc[0][n], a[u][0].x, a[u][1].x, a[u][0].y, a[u][1].y, x[u][n].x, x[u][n].y);
-        mma_16816(acc[1][n], a[u][0].z, a[u][1].z, a[u][0].w, a[u][1].w, x[u][n].z, x[u][n].w);
-      }
+    for (int u = 0; u < U; ++u) {
+      mma_16816(acc[0], a[u][0].x, a[u][1].x, a[u][0].y, a[u][1].y, x[u].x, x[u].y);
+      mma_16816(acc[1], a[u][0].z, a[u][1].z, a[u][0].w, a[u][1].w, x[u].z, x[u].w);
+    }
   };
-  // (XB: X is fetched along with the weights.  Sixteen rows of it leave no registers for that; it comes from L1 or L2 then.)
-  uint4 w0[U][2], w1[U][2], x0[U][NT], x1[U][NT];
+  uint4 w0[U][2], w1[U][2], x0[U], x1[U];
   set_rows();
   load_w(w0);
   load_k += ROUND;
@@ -123,7 +119,7 @@ __global__ void __launch_bounds__(WARPS * 32, MB) gemm_few_kernel(const __grid_c
   griddep_launch();
   if constexpr (NORM) {
     // every CTA normalises the rows for itself, while its first weights are on their way
-    __shared__ float ss_s[8 * NT][WARPS];
+    __shared__ float ss_s[kFewRows][WARPS];
     for (int m = 0; m < p.M; ++m) {
       const float* xr = p.x + (size_t)m * K;
       float ss = 0.f;
@@ -134,7 +130,7 @@ __global__ void __launch_bounds__(WARPS * 32, MB) gemm_few_kernel(const __grid_c
       }
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
-      if (lane == 0) ss_s[m][threadIdx.x >> 5] = ss;
+      if (lane == 0) ss_s[m][warp] = ss;
     }
     asm volatile("cp.async.wait_all;" ::: "memory");
     __syncthreads();
@@ -156,106 +152,75 @@ __global__ void __launch_bounds__(WARPS * 32, MB) gemm_few_kernel(const __grid_c
     }
     __syncthreads();
   }
-  if (XB) {
-    load_x(x0, k0);
-    load_x(x1, k0 + ROUND);
-  }
-  int pos[ITEMS], kv[ITEMS];
-  if constexpr (KIND == 2) {
-#pragma unroll
-    for (int it = 0; it < ITEMS; ++it) {
-      const int m = (it * WARPS * 32 + threadIdx.x) / OUTS;
-      pos[it] = kv[it] = -1;
-      if (m < p.M) {
-        const RopeEpilogue& e = p.re;
-        int b, v;
-        locate_row(m, e.row_off, e.B, e.n, b, v);
-        const int at = e.len[b] + e.depth[v], slot = e.len[b] + v;
-        if (v < e.n_active[b] && at < e.max_pos && slot < e.max_pos) {
-          pos[it] = at;
-          kv[it] = e.page_table[(size_t)b * e.max_pages + slot / CERB_PAGE] * e.H * CERB_PAGE + slot % CERB_PAGE;
-        }
-      }
+  load_x(x0, k0);
+  load_x(x1, k0 + ROUND);
+  // thread: row threadIdx.x % OUTS of the tile (of a pair: its first member), activation row threadIdx.x / OUTS
+  const int m = threadIdx.x / OUTS, rr = threadIdx.x % OUTS;
+  int pos = -1, kv = -1;
+  if (KIND == 2 && m < p.M) {
+    const RopeEpilogue& e = p.re;
+    int b, v;
+    locate_row(m, e.row_off, e.B, e.n, b, v);
+    const int at = e.len[b] + e.depth[v], slot = e.len[b] + v;
+    if (v < e.n_active[b] && at < e.max_pos && slot < e.max_pos) {
+      pos = at;
+      kv = e.page_table[(size_t)b * e.max_pages + slot / CERB_PAGE] * e.H * CERB_PAGE + slot % CERB_PAGE;
     }
   }
   int parity = 0;
   for (int tile = blockIdx.x; tile < p.tiles; tile += gridDim.x, parity ^= 1) {
     const int first = first_row(tile);
-    float old[ITEMS];
-    if constexpr (KIND == 3) {
+    const float old = KIND == 3 && m < p.M && first + rr < p.N ? p.out[(size_t)m * p.N + first + rr] : 0.f;
 #pragma unroll
-      for (int it = 0; it < ITEMS; ++it) {
-        const int i = it * WARPS * 32 + threadIdx.x, m = i / OUTS, rr = i % OUTS;
-        old[it] = m < p.M && first + rr < p.N ? p.out[(size_t)m * p.N + first + rr] : 0.f;
-      }
-    }
-#pragma unroll
-    for (int n = 0; n < NT; ++n)
-#pragma unroll
-      for (int e = 0; e < 4; ++e) acc[0][n][e] = acc[1][n][e] = 0.f;
+    for (int e = 0; e < 4; ++e) acc[0][e] = acc[1][e] = 0.f;
     // rounds in pairs (p.rounds of them); the loads run two rounds ahead, over the end of the tile into the next
     for (int q = 0; q < p.rounds; q += 2) {
-      const bool last = q + 2 >= p.rounds;
-      if (last) {
+      multiply(w0, x0);
+      if (q + 2 < p.rounds) {
+        load_k = k0 + (q + 2) * ROUND;
+      } else {
         load_tile += gridDim.x;
         load_k = k0;
-        if (!XB) load_x(x0, k0 + q * ROUND);
-        multiply(w0, x0);
         set_rows();
-      } else {
-        load_k = k0 + (q + 2) * ROUND;
-        if (!XB) load_x(x0, k0 + q * ROUND);
-        multiply(w0, x0);
       }
       load_w(w0);
-      if (XB) load_x(x0, load_k);
+      load_x(x0, load_k);
       load_k += ROUND;
-      if (!XB) load_x(x1, k0 + (q + 1) * ROUND);
       multiply(w1, x1);
       load_w(w1);
-      if (XB) load_x(x1, load_k);
+      load_x(x1, load_k);
     }
     float* red = red_s[parity];
 #pragma unroll
-    for (int n = 0; n < NT; ++n)
-#pragma unroll
-      for (int e = 0; e < 4; ++e)
-        red[(kg * ROWS + 16 * rg + 8 * (e >> 1) + g) * LD + 8 * n + 2 * t + (e & 1)] = acc[0][n][e] + acc[1][n][e];
+    for (int e = 0; e < 4; ++e) red[(warp * ROWS + 8 * (e >> 1) + g) * LD + 2 * t + (e & 1)] = acc[0][e] + acc[1][e];
     __syncthreads();
+    if (m >= p.M) continue;
+    auto sum = [&](int row) {
+      float s = 0.f;
 #pragma unroll
-    for (int it = 0; it < ITEMS; ++it) {
-      const int i = it * WARPS * 32 + threadIdx.x, m = i / OUTS, rr = i % OUTS;
-      if (m >= p.M) continue;
-      auto sum = [&](int row) {
-        float s = 0.f;
-#pragma unroll
-        for (int q = 0; q < KG; ++q) s += red[(q * ROWS + row) * LD + m];
-        return s;
-      };
-      if constexpr (!PAIRS) {
-        if (first + rr >= p.N) continue;
-        const float s = sum(rr);
-        p.out[(size_t)m * p.N + first + rr] = KIND == 3 ? old[it] + s : s;
+      for (int q = 0; q < WARPS; ++q) s += red[(q * ROWS + row) * LD + m];
+      return s;
+    };
+    if constexpr (!PAIRS) {
+      if (first + rr < p.N) p.out[(size_t)m * p.N + first + rr] = KIND == 3 ? old + sum(rr) : sum(rr);
+    } else {
+      float a = sum(rr), b = sum(rr + 8);
+      if constexpr (KIND == 1) {
+        if (first + rr < p.F) p.act[(size_t)m * p.F + first + rr] = __float2bfloat16_rn(a / (1.0f + expf(-a)) * b);
       } else {
-        const int row = 16 * (rr >> 3) + (rr & 7);
-        float a = sum(row), b = sum(row + 8);
-        if constexpr (KIND == 1) {
-          if (first + rr < p.F) p.act[(size_t)m * p.F + first + rr] = __float2bfloat16_rn(a / (1.0f + expf(-a)) * b);
-        } else {
-          if (kv[it] < 0) continue;
-          const RopeEpilogue& e = p.re;
-          const int unit = first >> 7, el = (first & 127) + rr, which = unit / e.H, h = unit - which * e.H;
-          if (which < 2) {
-            const float2 cs = e.rope[(size_t)pos[it] * 64 + el];
-            const float o1 = a * cs.x - b * cs.y;
-            b = b * cs.x + a * cs.y;
-            a = o1;
-          }
-          bf16* o = which == 0 ? reinterpret_cast<bf16*>(e.q) + ((size_t)m * e.H + h) * 128 + el
-                               : reinterpret_cast<bf16*>(which == 1 ? e.kpool : e.vpool) + ((size_t)kv[it] + (size_t)h * CERB_PAGE) * 128 + el;
-          o[0] = __float2bfloat16_rn(a);
-          o[64] = __float2bfloat16_rn(b);
+        if (kv < 0) continue;
+        const RopeEpilogue& e = p.re;
+        const int unit = first >> 7, el = (first & 127) + rr, which = unit / e.H, h = unit - which * e.H;
+        if (which < 2) {
+          const float2 cs = e.rope[(size_t)pos * 64 + el];
+          const float o1 = a * cs.x - b * cs.y;
+          b = b * cs.x + a * cs.y;
+          a = o1;
         }
+        bf16* o = which == 0 ? reinterpret_cast<bf16*>(e.q) + ((size_t)m * e.H + h) * 128 + el
+                             : reinterpret_cast<bf16*>(which == 1 ? e.kpool : e.vpool) + ((size_t)kv + (size_t)h * CERB_PAGE) * 128 + el;
+        o[0] = __float2bfloat16_rn(a);
+        o[64] = __float2bfloat16_rn(b);
       }
     }
   }
@@ -268,39 +233,29 @@ __global__ void __launch_bounds__(WARPS * 32, MB) gemm_few_kernel(const __grid_c
 constexpr size_t kNormSmem = 25 * 1024;
 size_t norm_smem(int M, int K) { return (size_t)(M + 1) * (K + 32) * sizeof(bf16); }
 
-template <int KIND, int NT, int KG, int U, int MB, bool XB, bool NORM>
+template <int KIND, bool NORM>
 int launch(FewParams p, cudaStream_t st) {
-  constexpr int ROWS = 16 * (WARPS / KG), OUTS = KIND == 1 || KIND == 2 ? ROWS / 2 : ROWS, ROUND = 32 * U;
+  constexpr int OUTS = KIND == 1 || KIND == 2 ? ROWS / 2 : ROWS;
   p.tiles = ((KIND == 1 ? p.F : KIND == 2 ? p.N / 2 : p.N) + OUTS - 1) / OUTS;
-  p.rounds = (p.K + KG * ROUND - 1) / (KG * ROUND);
-  p.range = p.rounds * ROUND;
-  p.rounds = (p.rounds + 1) & ~1;
-  const int grid = p.tiles < 148 * MB ? p.tiles : 148 * MB;
-  auto kern = gemm_few_kernel<KIND, NT, KG, U, MB, XB, NORM>;
-  const size_t smem = NORM ? norm_smem(p.M, p.K) : 0;
+  const int rounds = (p.K + WARPS * ROUND - 1) / (WARPS * ROUND);
+  p.range = rounds * ROUND;
+  p.rounds = (rounds + 1) & ~1;
+  auto kern = gemm_few_kernel<KIND, NORM>;
   static bool configured = false;
   if (!configured) {
-    // the share of the SM's memory that MB CTAs need as shared memory; the rest is L1
-    constexpr size_t most = NORM ? kNormSmem : 0;
-    const int share = (int)((MB * (2 * KG * ROWS * (8 * NT + 1) * sizeof(float) + most + 1024) * 100 + 228 * 1024 - 1) / (228 * 1024));
+    // the share of the SM's memory that two CTAs need as shared memory; the rest is L1
+    constexpr size_t need = 2 * (2 * WARPS * ROWS * LD * sizeof(float) + (NORM ? kNormSmem : 0) + 1024), all = 228 * 1024;
     if (NORM) CERB_CUDA_OK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kNormSmem));
-    CERB_CUDA_OK(cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, share));
+    CERB_CUDA_OK(cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, (int)((need * 100 + all - 1) / all)));
     configured = true;
   }
-  return launch_pdl(kern, dim3(grid), dim3(WARPS * 32), smem, st, p) == cudaSuccess ? CERB_OK : CERB_E_CUDA;
-}
-
-template <int KIND>
-int pick(const FewParams& p, cudaStream_t st) {
-  if constexpr (KIND == 1 || KIND == 2) {
-    if (p.x) return launch<KIND, 1, 8, 4, 2, true, true>(p, st);
-  }
-  return p.M <= 8 ? launch<KIND, 1, 8, 4, 2, true, false>(p, st) : launch<KIND, 2, 8, 4, 2, false, false>(p, st);
+  return launch_pdl(kern, dim3(p.tiles < CTAS ? p.tiles : CTAS), dim3(WARPS * 32), NORM ? norm_smem(p.M, p.K) : 0, st, p) == cudaSuccess
+             ? CERB_OK : CERB_E_CUDA;
 }
 
 }  // namespace
 
-bool gemm_few_normalises(int M, int K) { return M <= 8 && norm_smem(M, K) <= kNormSmem; }
+bool gemm_few_normalises(int M, int K) { return M <= kFewRows && norm_smem(M, K) <= kNormSmem; }
 
 int launch_gemm_few(const void* X, const void* W, float* out, int M, int N, int K, cudaStream_t st, const GemmEpilogue* epi,
                     const GemmNorm* norm, unsigned long long* clock_slot) {
@@ -319,20 +274,20 @@ int launch_gemm_few(const void* X, const void* W, float* out, int M, int N, int 
     p.eps = norm->eps;
   }
   switch (epi ? epi->kind : 0) {
-    case 0: return pick<0>(p, st);
+    case 0: return launch<0, false>(p, st);
     case 1:
       if ((N & 1) || !epi->act) return CERB_E_SHAPE;
       p.F = N / 2;
       p.act = (bf16*)epi->act;
-      return pick<1>(p, st);
+      return norm ? launch<1, true>(p, st) : launch<1, false>(p, st);
     case 2:
       if (!epi->rope || N != 3 * epi->rope->H * 128) return CERB_E_SHAPE;
       p.re = *epi->rope;
-      return pick<2>(p, st);
+      return norm ? launch<2, true>(p, st) : launch<2, false>(p, st);
     case 3:
       if (!epi->x) return CERB_E_SHAPE;
       p.out = epi->x;
-      return pick<3>(p, st);
+      return launch<3, false>(p, st);
   }
   return CERB_E_SHAPE;
 }

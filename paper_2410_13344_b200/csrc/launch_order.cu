@@ -69,7 +69,7 @@ const Entry kNormEmbed = {LO_NORM_ATTN, "fused_norm (embedding, attention norm)"
 const Entry kQkvNorm = {LO_GEMM_QKV, "gemm norm + qkv + rope / append epilogue", B_Q | B_KV, B_CONST};
 const Entry kGuNorm = {LO_GEMM_GU, "gemm norm + gate-up + swiglu epilogue", B_ACT, B_CONST};
 
-// Variant 0 is the steps of 17 to 128 rows; those with a residual add in the GEMMs occur above and up to 16 rows, the norms in
+// Variant 0 is the steps of 9 to 128 rows; those with a residual add in the GEMMs occur above and up to 8 rows, the norms in
 // the GEMMs (8) with one or two.
 constexpr int kVariants = 9;
 const Fusion kFusion[kVariants] = {  // {swiglu, rope, residual, norm}
