@@ -1077,6 +1077,152 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tree_attn_tc_kernel(const __gri
 #include "attention_kt.cuh"
 
 // ---------------------------------------------------------------------------------------------
+// bf16, one query row per sequence (auto-regressive steps)
+// ---------------------------------------------------------------------------------------------
+// One CTA per (split, head, sequence), a page of 16 keys to a warp at a time, both products as plain FMA: with one row there is
+// nothing for the tensor cores.  What such a launch costs at a few thousand keys is its start and its end, so it has no ring,
+// no barriers and little shared memory: a lane holds 16 bytes of eight keys and eight values in registers, the first page's
+// from before the wait for the kernel in front.  DH / 8 lanes share a key, the 256 / DH keys of a load are separate online
+// softmaxes until the end.  The splits of a (sequence, head) are a cluster and meet in the shared memory of its first CTA.
+// 32 heads of 128, against the warp-MMA kernel's 16-row layout: 16 sequences of 500 / 2000 / 8192 keys 20.9 / 75 / 299 us
+// (25.9 / 82 / 308), one of 16000 39.5 (42.0); a 16-layer one-node forward of the 7B shape with 1000 keys 1270 us (1413), its
+// neighbours' loads no longer waiting for an SM to be divided anew between L1 and shared memory.
+constexpr int ONE_WARPS = 8;
+template <int DH>
+__global__ void __launch_bounds__(ONE_WARPS * 32, 2) tree_attn_one_kernel(const AttnParams p, const bf16* kpool, const bf16* vpool) {
+  constexpr int LPK = DH / 8, KPL = 32 / LPK, NL = CERB_PAGE / KPL;       // lanes per key, keys per load, loads per page
+  __shared__ float s_o[ONE_WARPS][DH], s_m[ONE_WARPS], s_l[ONE_WARPS];
+  __shared__ float c_o[8][DH], c_m[8], c_l[8];                           // first CTA of the cluster: what every split has found
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, sub = lane / LPK, d0 = (lane % LPK) * 8;
+  const int split = blockIdx.x, h = blockIdx.y, b = blockIdx.z;
+  const int L = p.len[b];
+  if (p.n_active && p.n_active[b] < 1) return;                           // (every CTA of the cluster does)
+  const size_t row = p.row_off ? (size_t)p.row_off[b] : (size_t)b;
+  if (p.nsplit > 1) cluster_start_arrive();
+  const int pages = min((L + 1 + CERB_PAGE - 1) / CERB_PAGE, p.max_pages), per = (pages + p.nsplit - 1) / p.nsplit;
+  const int pg1 = min(pages, (split + 1) * per);
+  const int32_t* pt = p.page_table + (size_t)b * p.max_pages;
+  int pg = split * per + warp;
+  auto load = [&](uint4 (&r)[NL], const bf16* pool, int at) {
+    const bf16* src = pool + ((size_t)pt[at] * p.H + h) * CERB_PAGE * DH + sub * DH + d0;
+#pragma unroll
+    for (int i = 0; i < NL; ++i)
+      asm volatile("ld.global.L1::no_allocate.v4.u32 {%0, %1, %2, %3}, [%4];"
+                   : "=r"(r[i].x), "=r"(r[i].y), "=r"(r[i].z), "=r"(r[i].w) : "l"(src + i * KPL * DH) : "memory");
+  };
+  uint4 k[NL], v[NL];
+  const bool early = pg < pg1 && (pg + 1) * CERB_PAGE <= L;              // a page without this step's key
+  if (early) {
+    load(k, kpool, pg);
+    load(v, vpool, pg);
+  }
+  griddep_wait();
+  griddep_launch();
+  if (!early && pg < pg1) {
+    load(k, kpool, pg);
+    load(v, vpool, pg);
+  }
+  auto unpack = [](const uint4& r, float* f) {
+    const uint32_t w[4] = {r.x, r.y, r.z, r.w};
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      f[2 * e] = __uint_as_float(w[e] << 16);
+      f[2 * e + 1] = __uint_as_float(w[e] & 0xffff0000u);
+    }
+  };
+  float q[8], o[8], m = -INFINITY, l = 0.f;
+  unpack(*reinterpret_cast<const uint4*>(p.q + (row * p.H + h) * DH + d0), q);
+#pragma unroll
+  for (int e = 0; e < 8; ++e) { q[e] *= p.scale_log2; o[e] = 0.f; }
+  for (; pg < pg1; pg += ONE_WARPS) {
+    float s[NL], mx = m;
+#pragma unroll
+    for (int i = 0; i < NL; ++i) {
+      float f[8];
+      unpack(k[i], f);
+      s[i] = 0.f;
+#pragma unroll
+      for (int e = 0; e < 8; ++e) s[i] = fmaf(q[e], f[e], s[i]);
+    }
+    const bool more = pg + ONE_WARPS < pg1;
+    if (more) load(k, kpool, pg + ONE_WARPS);
+#pragma unroll
+    for (int i = 0; i < NL; ++i) {
+#pragma unroll
+      for (int w = 1; w < LPK; w <<= 1) s[i] += __shfl_xor_sync(0xffffffffu, s[i], w);
+      if (pg * CERB_PAGE + i * KPL + sub > L) {                          // past the end: whatever the pool holds
+        s[i] = -INFINITY;
+        v[i] = make_uint4(0, 0, 0, 0);
+      }
+      mx = fmaxf(mx, s[i]);
+    }
+    const float u = mx == -INFINITY ? 0.f : mx, a = exp2f(m - u);
+    m = mx;
+    l *= a;
+#pragma unroll
+    for (int e = 0; e < 8; ++e) o[e] *= a;
+#pragma unroll
+    for (int i = 0; i < NL; ++i) {
+      const float w = exp2f(s[i] - u);
+      float f[8];
+      unpack(v[i], f);
+      l += w;
+#pragma unroll
+      for (int e = 0; e < 8; ++e) o[e] = fmaf(w, f[e], o[e]);
+    }
+    if (more) load(v, vpool, pg + ONE_WARPS);
+  }
+#pragma unroll
+  for (int w = LPK; w < 32; w <<= 1) {
+    const float mo = __shfl_xor_sync(0xffffffffu, m, w), lo = __shfl_xor_sync(0xffffffffu, l, w), mn = fmaxf(m, mo);
+    const float u = mn == -INFINITY ? 0.f : mn, wa = exp2f(m - u), wb = exp2f(mo - u);
+    l = l * wa + lo * wb;
+#pragma unroll
+    for (int e = 0; e < 8; ++e) o[e] = o[e] * wa + __shfl_xor_sync(0xffffffffu, o[e], w) * wb;
+    m = mn;
+  }
+  if (lane < LPK) {
+#pragma unroll
+    for (int e = 0; e < 8; ++e) s_o[warp][d0 + e] = o[e];
+  }
+  if (lane == 0) { s_m[warp] = m; s_l[warp] = l; }
+  __syncthreads();
+  const int c = threadIdx.x;
+  // the parts of one output (its column c, the running maxima, the sums) as one
+  auto merge = [&](int parts, const float* po, const float* pm, const float* pl, float& M, float& sum) {
+    M = -INFINITY;
+    for (int w = 0; w < parts; ++w) M = fmaxf(M, pm[w]);
+    const float u = M == -INFINITY ? 0.f : M;
+    float acc = 0.f;
+    sum = 0.f;
+    for (int w = 0; w < parts; ++w) {
+      const float f = exp2f(pm[w] - u);
+      sum += pl[w] * f;
+      acc += po[w * DH + c] * f;
+    }
+    return acc;
+  };
+  float acc = 0.f, M = 0.f, sum = 1.f;
+  if (c < DH) acc = merge(ONE_WARPS, &s_o[0][0], s_m, s_l, M, sum);
+  if (p.nsplit > 1) {
+    cluster_start_wait();                                                // every CTA of the cluster runs
+    if (c < DH) {
+      auto put = [](float* at, float x) {
+        asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(mapa_u32(smem_u32(at), 0)), "f"(x) : "memory");
+      };
+      put(&c_o[split][c], acc);
+      if (c == 0) { put(&c_m[split], M); put(&c_l[split], sum); }
+    }
+    cluster_start_arrive();
+    cluster_start_wait();                                                // ... and has left its part
+    if (split != 0) return;
+    if (c < DH) acc = merge(p.nsplit, &c_o[0][0], c_m, c_l, M, sum);
+  }
+  if (c < DH) p.out[(row * p.H + h) * DH + c] = __float2bfloat16_rn(acc / sum);
+  if (c == 0 && p.lse) p.lse[((size_t)b * p.H + h) * p.n] = (M + log2f(sum)) * 0.6931471805599453f;
+}
+
+// ---------------------------------------------------------------------------------------------
 // fp32 path
 // ---------------------------------------------------------------------------------------------
 // A CTA per (node, head), whose warps take four keys each in turn.  A launch is bound by the rounds of memory latency that one
@@ -1247,7 +1393,7 @@ static int launch_attn_window(const cerb_attn_args* a, int row0, int rows, const
   p.H = a->n_heads;
   p.max_pages = a->max_pages;
   // Which kernel: windows of 65 .. 128 rows take the tcgen05 kernel whose MMAs are 128 query rows tall; 17 .. 64 rows
-  // the keys-on-M kernel (below); up to 16 rows and one-node steps the warp-MMA kernel, whose 16-row layout wastes
+  // the keys-on-M kernel (below); one row the kernel of its own; up to 16 rows the warp-MMA kernel, whose 16-row layout wastes
   // no tensor work and streams at 7.0 TB/s at batch 16 x 8K keys.  Short caches and head_dim 64 stay on the
   // warp-MMA kernel too.  CERB_ATTN_TC=0 / 1 forces the warp-MMA / the query-rows-on-M tcgen05 kernel (tests).
   static const int force_tc = getenv("CERB_ATTN_TC") ? atoi(getenv("CERB_ATTN_TC")) : -1;
@@ -1277,6 +1423,19 @@ static int launch_attn_window(const cerb_attn_args* a, int row0, int rows, const
   // 128-query form, not built any more) 654 / 572 us.  CERB_ATTN_KT=0 / 1 keeps it off / uses it for every launch of
   // up to 64 rows (tests).
   static const int force_kt = getenv("CERB_ATTN_KT") ? atoi(getenv("CERB_ATTN_KT")) : -1;
+  // One row per sequence: the kernel without tensor cores, at every length (figures there); the switches for tests keep it off.
+  if (a->n == 1 && win == 1 && use_cluster && force_tc < 0 && force_kt < 0) {
+    // two CTAs to an SM, at least a page to a warp
+    int want = 2 * 148 / (a->B * a->n_heads);
+    const int pages = (a->max_len + CERB_PAGE - 1) / CERB_PAGE;
+    if (want > (pages + ONE_WARPS - 1) / ONE_WARPS) want = (pages + ONE_WARPS - 1) / ONE_WARPS;
+    p.nsplit = want < 1 ? 1 : want > 8 ? 8 : want;
+    auto kern = a->head_dim == 128 ? tree_attn_one_kernel<128> : tree_attn_one_kernel<64>;
+    const dim3 grid(p.nsplit, p.H, Bw), block(ONE_WARPS * 32);
+    const bf16 *kp = (const bf16*)a->k_pool, *vp = (const bf16*)a->v_pool;
+    if (p.nsplit > 1) return launch_pdl_cluster(kern, grid, block, 0, st, (unsigned)p.nsplit, p, kp, vp) == cudaSuccess ? CERB_OK : CERB_E_CUDA;
+    return launch_pdl(kern, grid, block, 0, st, p, kp, vp) == cudaSuccess ? CERB_OK : CERB_E_CUDA;
+  }
   const bool kt_path = a->head_dim == 128 && force_tc < 0 && rows <= 64 && (force_kt < 0 ? rows > 16 : force_kt != 0);
   if (kt_path) {
     const int tiles = (a->max_len + KT_TILE - 1) / KT_TILE;
