@@ -1133,7 +1133,7 @@ __global__ void __launch_bounds__(ONE_WARPS * 32, 2) tree_attn_one_kernel(const 
   float q[8], o[8], m = -INFINITY, l = 0.f;
   unpack(*reinterpret_cast<const uint4*>(p.q + (row * p.H + h) * DH + d0), q);
 #pragma unroll
-  for (int e = 0; e < 8; ++e) { q[e] *= p.scale_log2; o[e] = 0.f; }
+  for (int e = 0; e < 8; ++e) o[e] = 0.f;
   for (; pg < pg1; pg += ONE_WARPS) {
     float s[NL], mx = m;
 #pragma unroll
@@ -1150,6 +1150,7 @@ __global__ void __launch_bounds__(ONE_WARPS * 32, 2) tree_attn_one_kernel(const 
     for (int i = 0; i < NL; ++i) {
 #pragma unroll
       for (int w = 1; w < LPK; w <<= 1) s[i] += __shfl_xor_sync(0xffffffffu, s[i], w);
+      s[i] *= p.scale_log2;                                              // (the exact dot product first, as in the other kernels)
       if (pg * CERB_PAGE + i * KPL + sub > L) {                          // past the end: whatever the pool holds
         s[i] = -INFINITY;
         v[i] = make_uint4(0, 0, 0, 0);
