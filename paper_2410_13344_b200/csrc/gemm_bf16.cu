@@ -7,11 +7,11 @@
 // W is the MMA's A operand (M = 128), the activation rows are the B operand (N = rows), and
 // D[128][rows] accumulates in tensor memory and is written out transposed.
 //
-// Up to 128 activation rows (gemm_bf16_kernel): a CTA takes 256 weight rows at a time (two MMA tiles
+// 9 to 128 activation rows (gemm_bf16_kernel): a CTA takes 256 weight rows at a time (two MMA tiles
 // that share one activation stage), which halves the activation re-reads through L2; weight tiles
 // carry an evict-first L2 hint, activation tiles evict-last; the accumulator is double-buffered.
 //
-// More than 128 rows: gemm_tile.cu.
+// Fewer rows: gemm_few.cu.  More: gemm_tile.cu.
 //
 // The kernel is launched programmatically dependent on its predecessor: weights do not depend on
 // the previous kernel, so the producer fills the whole stage ring with weight tiles before it
