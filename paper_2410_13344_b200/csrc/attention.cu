@@ -1497,14 +1497,14 @@ int launch_tree_attention(cerb_ctx* c, const cerb_attn_args* a, const CUtensorMa
   const int win = chain ? (a->n + kAttnRowsPerLaunch - 1) / kAttnRowsPerLaunch : 1;
   if (a->dtype == CERB_F32) {
     dim3 grid(win > 1 ? kAttnRowsPerLaunch : a->n, a->n_heads, a->B * win);
+    auto go = [&](auto kern) {
+      launch_pdl(kern, grid, dim3(F32_WARPS * 32), 0, st, (const float*)a->q, (const float*)a->k_pool, (const float*)a->v_pool, a->page_table, a->len,
+                 a->n_active, a->anc, (float*)a->out, a->lse, a->n, a->n_heads, a->max_pages, a->scale, row_off, win);
+    };
     if (a->head_dim == 64)
-      tree_attn_f32_kernel<64><<<grid, F32_WARPS * 32, 0, st>>>((const float*)a->q, (const float*)a->k_pool, (const float*)a->v_pool,
-                                                     a->page_table, a->len, a->n_active, a->anc, (float*)a->out, a->lse,
-                                                     a->n, a->n_heads, a->max_pages, a->scale, row_off, win);
+      go(tree_attn_f32_kernel<64>);
     else if (a->head_dim == 128)
-      tree_attn_f32_kernel<128><<<grid, F32_WARPS * 32, 0, st>>>((const float*)a->q, (const float*)a->k_pool, (const float*)a->v_pool,
-                                                      a->page_table, a->len, a->n_active, a->anc, (float*)a->out, a->lse,
-                                                      a->n, a->n_heads, a->max_pages, a->scale, row_off, win);
+      go(tree_attn_f32_kernel<128>);
     else
       return CERB_E_SHAPE;
     CERB_LAUNCH_CHECK(c);
