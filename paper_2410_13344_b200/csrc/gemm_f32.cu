@@ -49,8 +49,9 @@ __global__ void __launch_bounds__(256) gemm_f32_kernel(const float* __restrict__
 
 // The same for few output tiles (the small models this path is for: 16 rows x 768 columns x 256).  Such a GEMM is pure
 // latency: with the kernel above it was 12 CTAs going through 16 load - wait - multiply rounds one after the other, 16 us for
-// 6 MFLOP (a request to the tiny fp32 model: 11.1 ms, 2.8 with this kernel and the attention in fours).  Here a CTA takes 16 x 16 outputs, fetches 256 k of both operands in one round, the next 256 while it multiplies,
-// and its eight warps take 32 k each; their sums meet in shared memory at the end.
+// 6 MFLOP (a request to the tiny fp32 model: 11.1 ms, 2.8 with this kernel and the attention in fours).  Here a CTA takes
+// 16 x 16 outputs, fetches 256 k of both operands in one round, the next 256 while it multiplies, and its eight warps take 32 k
+// each; their sums meet in shared memory at the end.
 constexpr int SM_T = 16, SM_K = 256, SM_LD = SM_K + 4;
 __global__ void __launch_bounds__(256) gemm_f32_small_kernel(const float* __restrict__ X, const float* __restrict__ W,
                                                              float* __restrict__ out, int M, int N, int K) {
@@ -129,7 +130,9 @@ int launch_gemm_f32(cerb_ctx* c, const float* X, const float* W, float* out, int
   // 1024 x 1024 x 256 with 256 tiles 38 / 39).
   if ((long long)((N + TN - 1) / TN) * ((M + TM - 1) / TM) < kFewTiles) {
     dim3 small((N + SM_T - 1) / SM_T, (M + SM_T - 1) / SM_T);
-    launch_pdl(gemm_f32_small_kernel, small, dim3(256), 0, st, X, W, out, M, N, K);
+    // (a caller without a model may hand over as weights what the kernel in front is still writing)
+    if (c) launch_pdl(gemm_f32_small_kernel, small, dim3(256), 0, st, X, W, out, M, N, K);
+    else gemm_f32_small_kernel<<<small, 256, 0, st>>>(X, W, out, M, N, K);
     CERB_LAUNCH_CHECK(c);
     return CERB_OK;
   }

@@ -17,3 +17,12 @@ def test_gemm_matches_definition(M, N, K):
     W = synth.normal(13, 2, (N, K), 0.05, dtype=torch.float32, device="cuda")
     # products and sums in fp32: sqrt(K) * 2^-24 of the terms' size
     assert close(cb.gemm(X, W), orc.linear(X.cpu(), W.cpu()), 0) < 1e-5
+
+
+def test_weights_may_be_what_the_previous_call_wrote():
+    X = synth.normal(13, 3, (48, 1 << 16), 1.0, dtype=torch.float32, device="cuda")
+    V = synth.normal(13, 4, (256, 1 << 16), 1e-4, dtype=torch.float32, device="cuda")
+    Y = synth.normal(13, 5, (16, 256), 1.0, dtype=torch.float32, device="cuda")
+    W = cb.gemm(X, V)                                        # a long launch (65536 deep) ...
+    out = cb.gemm(Y, W)                                      # ... whose output (0.03 in size) is the next one's weights
+    assert close(out, orc.linear(Y.cpu(), W.cpu()), 0) < 1e-5
