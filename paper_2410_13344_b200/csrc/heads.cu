@@ -31,7 +31,7 @@ struct LevelParams {
   HeadJob job[CERB_MAX_HEADS];
   const float* state_in;    // [B][Hc][wmax]
   float* out;               // state_out [B][Hc][wmax] or logits [B][Hc][out_stride]
-  const bf16* terms_in;     // bf16 models: the same state as three bf16 terms, [Hc][cols][wmax], column 3 b + term
+  const bf16* terms_in;     // bf16 models: the same state as three bf16 terms, [Hc][cols][wmax], column B term + b
   bf16* terms_out;
   int cols;
   int Hc, wmax, out_stride, B, b0;
@@ -132,8 +132,13 @@ __device__ __forceinline__ void mma_16816(float* c, uint32_t a0, uint32_t a1, ui
 
 // One level (or the FC) of every head of a bf16 model, for the whole batch.  Bound by HBM: the weights once, 2.7 GB per
 // draft of the 7B shape.  The fp32 states enter the tensor cores as three bf16 terms each (24 bits; the products are exact
-// in fp32), so a batch is 3 B MMA columns instead of B passes of FMAs: with those, a batch of four took 1.90 ms per draft
-// (0.22 of the copy rate), bound by the FMAs and the shared-memory loads that feed them.
+// in fp32), so a batch is 3 B MMA columns (all leading terms, then all middle ones, then all last ones) instead of B passes of
+// FMAs: with those, a batch of four took 1.90 ms per draft (0.22 of the copy rate), bound by the FMAs and the shared-memory
+// loads that feed them.
+// The tensor cores cut a sum off, towards zero, at every step, which FMAs do not: with the leading terms of the whole k in one
+// chain the logits of the 7B shape were 0.7e-6 to 3.8e-6 (relative, 2-norm) away from float64, FMAs 1.6e-7.  So each pair of
+// MMAs of a column tile with leading terms starts from zero and is added to the sum in fp32: 1.2e-7 to 1.4e-7.  The other
+// terms are at most 2^-8 of the first; their sums stay in the tensor cores.
 // A CTA takes 16 MT 8 / KG weight rows, 16 MT to a warp; KG warps share a row group, each takes every KG-th 32-wide k block,
 // and their sums are added in shared memory.  Weights
 // go from global memory straight into the A fragments: a lane loads 16 consecutive bytes of a row, and its eight k values
@@ -144,6 +149,7 @@ template <int NT, int MT, int U, int KG, int MB>
 __global__ void __launch_bounds__(HM_WARPS * 32, MB) head_mma_kernel(const __grid_constant__ LevelParams P) {
   extern __shared__ float red[];                      // [k group][rows][8 NT columns + 1]
   constexpr int RG = HM_WARPS / KG, ROWS = 16 * MT * RG, LD = 8 * NT + 1;
+  constexpr int FT = NT <= 3 ? 1 : 2;                 // column tiles with leading terms: B columns, NT = ceil(3 B / 8)
   const int head = blockIdx.y;
   const HeadJob& J = P.job[head];
   const int row_base = blockIdx.x * ROWS;
@@ -187,14 +193,24 @@ __global__ void __launch_bounds__(HM_WARPS * 32, MB) head_mma_kernel(const __gri
 #pragma unroll
     for (int n = 0; n < NT; ++n) acc[m][n][0] = acc[m][n][1] = acc[m][n][2] = acc[m][n][3] = 0.f;
   auto multiply = [&](const uint4 (&a)[U][MT][2], const uint4 (&x)[U][NT]) {
+    auto step = [&](float* c, int u, int m, int n) {
+      mma_16816(c, a[u][m][0].x, a[u][m][1].x, a[u][m][0].y, a[u][m][1].y, x[u][n].x, x[u][n].y);
+      mma_16816(c, a[u][m][0].z, a[u][m][1].z, a[u][m][0].w, a[u][m][1].w, x[u][n].z, x[u][n].w);
+    };
 #pragma unroll
     for (int u = 0; u < U; ++u)
 #pragma unroll
       for (int m = 0; m < MT; ++m)
 #pragma unroll
         for (int n = 0; n < NT; ++n) {
-          mma_16816(acc[m][n], a[u][m][0].x, a[u][m][1].x, a[u][m][0].y, a[u][m][1].y, x[u][n].x, x[u][n].y);
-          mma_16816(acc[m][n], a[u][m][0].z, a[u][m][1].z, a[u][m][0].w, a[u][m][1].w, x[u][n].z, x[u][n].w);
+          if (n >= FT) {
+            step(acc[m][n], u, m, n);
+            continue;
+          }
+          float c[4] = {0.f, 0.f, 0.f, 0.f};
+          step(c, u, m, n);
+#pragma unroll
+          for (int e = 0; e < 4; ++e) acc[m][n][e] += c[e];
         }
   };
   uint4 w0[U][MT][2], w1[U][MT][2], x0[U][NT], x1[U][NT];
@@ -225,14 +241,14 @@ __global__ void __launch_bounds__(HM_WARPS * 32, MB) head_mma_kernel(const __gri
     float y = 0.f;
 #pragma unroll
     for (int q = 0; q < KG; ++q) {
-      const float* c = red + (q * ROWS + rr) * LD + 3 * b;
-      y += c[0] + c[1] + c[2];
+      const float* c = red + (q * ROWS + rr) * LD + b;
+      y += c[0] + c[P.B] + c[2 * P.B];
     }
     if (P.epilogue) {
       const int from = r < J.w0 ? head : J.src, at = r < J.w0 ? r : r - J.w0;
       y += ldf(reinterpret_cast<const bf16*>(J.bias) + r) + P.state_in[((size_t)b * P.Hc + from) * P.wmax + at];
       y = y / (1.0f + expf(-y));
-      store_terms(P.terms_out + ((size_t)head * P.cols + 3 * b) * P.wmax + r, P.wmax, y);
+      store_terms(P.terms_out + ((size_t)head * P.cols + b) * P.wmax + r, (size_t)P.B * P.wmax, y);
     }
     P.out[((size_t)b * P.Hc + head) * P.out_stride + r] = y;
   }
@@ -248,7 +264,7 @@ __global__ void head_init_kernel(const T* __restrict__ h_last, float* __restrict
   if (k >= d) return;
   const float v = ldf(h_last + (size_t)b * d + k);
   state[((size_t)b * Hc + h) * wmax + k] = v;
-  if (terms) store_terms(terms + ((size_t)h * cols + 3 * b) * wmax + k, wmax, v);
+  if (terms) store_terms(terms + ((size_t)h * cols + b) * wmax + k, (size_t)gridDim.y * wmax, v);
 }
 
 __device__ __forceinline__ bool better(float va, int ia, float vb, int ib) { return va > vb || (va == vb && ia < ib); }
@@ -404,16 +420,19 @@ int launch_mma(cerb_ctx* c, const LevelParams& P, int max_rows, cudaStream_t st)
 }
 
 // bf16 models: the number of MMA column tiles decides (us per draft of the 7B shape, HBM floor 410).  Few columns want
-// small CTAs, three to an SM (batch 1: 441 against 480 with 32 rows); more columns want two warps side by side on the same k
-// blocks, whose state loads then meet in L1 (batch 4: 495 against 553; batch 8: 508 against 816), and at six tiles, where the
-// states weigh more than the weights on their way from L2, 64 rows per CTA (batch 16: 839 against 907; batch 9: 727).
+// small CTAs, three to an SM (batch 1: 449 against 492 with 32 rows); more columns want two row tiles to a warp, which share
+// its state loads (batch 4: 489 against 520), two warps side by side on the same k blocks, whose state loads meet in L1 (batch
+// 8: 519 against 524; batch 9: 687 against 712), and from five tiles on, where the states weigh more than the weights on their
+// way from L2, three row tiles (batch 11: 782 against 810 with two and 848 with four, which do not fit the registers; batch
+// 16: 846, 976, 1130).
 int launch_level_mma(cerb_ctx* c, const LevelParams& P, int max_rows, cudaStream_t st) {
   switch ((3 * P.B + 7) / 8) {
     case 1: return launch_mma<1, 1, 2, 8, 3>(c, P, max_rows, st);
-    case 2: return launch_mma<2, 1, 4, 4, 2>(c, P, max_rows, st);
+    case 2: return launch_mma<2, 2, 1, 8, 2>(c, P, max_rows, st);
     case 3: return launch_mma<3, 2, 1, 4, 2>(c, P, max_rows, st);
-    case 4: return launch_mma<4, 2, 1, 4, 2>(c, P, max_rows, st);
-    default: return launch_mma<6, 4, 1, 8, 1>(c, P, max_rows, st);
+    case 4: return launch_mma<4, 2, 2, 4, 1>(c, P, max_rows, st);
+    case 5: return launch_mma<5, 3, 1, 8, 1>(c, P, max_rows, st);
+    default: return launch_mma<6, 3, 1, 8, 1>(c, P, max_rows, st);
   }
 }
 

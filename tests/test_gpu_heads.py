@@ -33,3 +33,20 @@ def test_draft_logits_match_oracle(B, d, vocab):
             ids = [int(t) for t in orc.topk_ids(logits[b, h].cpu().double(), rig.topk[h])]
             assert [int(t) for t in topk[b, h, :rig.topk[h]]] == ids
         assert [int(t) for t in tree_tok[b]] == [int(roots[b])] + [int(topk[b, tree.head[v], tree.rank[v]]) for v in range(1, tree.n)]
+
+
+# A sum of w products in fp32 is off by about sqrt(w / 2) * 2^-25 at most when every addition rounds (w = 8192: 1.9e-6), and by
+# less where partial sums meet in a tree: FMAs with 32 lanes to a row are 1.6e-7 away.  Sums left in the tensor cores,
+# which cut off towards zero at every step, are 7e-7 and more away at these widths.
+@pytest.mark.parametrize("B", [1, 3, 8, 9, 11, 16])
+def test_draft_logits_are_fp32_sums(B):
+    ms = synth.ModelShape(1, 4096, 2, 64, 128, 1024, "bf16")
+    rig = Rig(cb, ms, n_cheads=2, n_levels=2, topk=(5, 3), concat_level=1, max_batch=B, max_tokens=32, max_nodes=16)
+    tok = torch.stack([synth.make_prompt(1024, 8, seq=60 + b) for b in range(B)]).to(torch.int32).cuda()
+    rig.eng.prefill(tok, [3 + b % 5 for b in range(B)])
+    _, _, h_last = rig.eng.read_state()
+    _, _, logits = rig.eng.draft(rig.eng.tree(synth.best_first_tree(12, rig.topk)), want_logits=True)
+    for b in {0, B - 1}:
+        for h, want in enumerate(orc.heads_forward(h_last[b].double(), rig.cheads, rig.csrc)):
+            got, want = logits[b, h].double().cpu(), want.double()
+            assert float((got - want).norm() / want.norm()) < 3e-7, (b, h)
