@@ -138,7 +138,10 @@ __global__ void __launch_bounds__((WQ * WK + 1) * 32) tree_attn_bf16_kernel(cons
   const int nq_all = (p.n_active ? min(p.n_active[b], p.n) : p.n) - shift;   // live nodes of this sequence (from the window on)
   const size_t qrow = (p.row_off ? (size_t)p.row_off[b] : (size_t)b * p.n) + shift;   // its first row of q and out
   const int nq = min(nq_all - p.row0, p.rows);                        // live query rows of this launch
-  if (nq <= 0) return;
+  if (nq <= 0) {
+    griddep_wait();      // (no CTA leaves ahead of the kernel in front: this launch would count as complete while that one runs)
+    return;
+  }
   const int kv_total = L + min(nq_all, p.row0 + p.rows);
   const int tiles = (kv_total + TILE - 1) / TILE;
   const int per = (tiles + p.nsplit - 1) / p.nsplit;
@@ -582,7 +585,10 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tree_attn_tc_kernel(const __gri
     it.T = it.nq <= 0 || it.too_long ? 0 : min(tiles, it.t0 + per) - it.t0;
     return it;
   };
-  if (!many && item_at(0).nq <= 0) return;                        // (uniform over a cluster)
+  if (!many && item_at(0).nq <= 0) {                              // (uniform over a cluster)
+    griddep_wait();
+    return;
+  }
 
   if (threadIdx.x == 0) {
     aborted_s = (*p.status != 0);
@@ -1096,7 +1102,10 @@ __global__ void __launch_bounds__(ONE_WARPS * 32, 2) tree_attn_one_kernel(const 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, sub = lane / LPK, d0 = (lane % LPK) * 8;
   const int split = blockIdx.x, h = blockIdx.y, b = blockIdx.z;
   const int L = p.len[b];
-  if (p.n_active && p.n_active[b] < 1) return;                           // (every CTA of the cluster does)
+  if (p.n_active && p.n_active[b] < 1) {                                 // (every CTA of the cluster does)
+    griddep_wait();
+    return;
+  }
   const size_t row = p.row_off ? (size_t)p.row_off[b] : (size_t)b;
   if (p.nsplit > 1) cluster_start_arrive();
   const int pages = min((L + 1 + CERB_PAGE - 1) / CERB_PAGE, p.max_pages), per = (pages + p.nsplit - 1) / p.nsplit;

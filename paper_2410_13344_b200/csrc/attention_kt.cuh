@@ -110,7 +110,10 @@ __global__ void __launch_bounds__(kt_threads(NCB), 1) tree_attn_kt_kernel(const 
   const int nq_all = (p.n_active ? min(p.n_active[b], p.n) : p.n) - shift;   // live nodes of this sequence (from the window on)
   const size_t qrow = (p.row_off ? (size_t)p.row_off[b] : (size_t)b * p.n) + shift;   // its first row of q and out
   const int nq = min(nq_all - p.row0, p.rows);                        // live query rows of this launch
-  if (nq <= 0) return;                                                // (uniform over a cluster)
+  if (nq <= 0) {                                                      // (uniform over a cluster)
+    griddep_wait();
+    return;
+  }
   const int n_tree = min(nq_all, p.row0 + p.rows);                    // tree keys these rows can see
   const int kv_total = L + n_tree;
   const int tiles = (kv_total + KT_TILE - 1) / KT_TILE;

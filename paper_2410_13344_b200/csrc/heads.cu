@@ -153,7 +153,10 @@ __global__ void __launch_bounds__(HM_WARPS * 32, MB) head_mma_kernel(const __gri
   const int head = blockIdx.y;
   const HeadJob& J = P.job[head];
   const int row_base = blockIdx.x * ROWS;
-  if (row_base >= J.rows) return;                     // (its dependents need not wait for it)
+  if (row_base >= J.rows) {
+    griddep_wait();
+    return;
+  }
   const int w = J.w0 + J.w1;
   const int warp = (threadIdx.x >> 5) % KG, rg = (threadIdx.x >> 5) / KG, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
   const bf16* Wr[MT][2];

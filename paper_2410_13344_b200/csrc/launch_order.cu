@@ -2,7 +2,8 @@
 //
 // Every kernel of the forward is launched programmatically dependent on its predecessor: it may start while the
 // kernel in front is still running, and it executes griddepcontrol.wait before it touches what that kernel writes.
-// Every kernel also releases its own dependents only AFTER its own wait.  So when kernel i runs, kernel i - 2 and
+// Every kernel also releases its own dependents only AFTER its own wait, and no CTA leaves without having waited (a launch whose
+// CTAs all had would be complete while the kernel in front runs).  So when kernel i runs, kernel i - 2 and
 // everything older is complete, and kernel i may read, ahead of its wait, any buffer whose youngest writer is at
 // least two launches older.  This file states, per kernel, what it writes and what it reads ahead of its wait;
 // launch_order_violations() checks the rule over the cyclic layer sequence, and the host controller steps

@@ -135,3 +135,22 @@ def test_every_forward_kernel_releases_its_dependents_after_its_own_wait():
                 seen += 1
                 assert 0 <= w < t, (fn, body[:80])
     assert seen >= 8
+
+
+def test_no_forward_kernel_leaves_ahead_of_its_wait():
+    """... and on no CTA leaving before it has waited: a launch whose CTAs all find nothing to do (the second window of a tree
+    of more than 128 nodes with no live rows) would be complete while the kernel in front still runs, and the launch
+    behind it would no longer wait for that one."""
+    src = os.path.join(ROOT, "paper_2410_13344_b200", "csrc")
+    seen = 0
+    for fn in sorted(os.listdir(src)):
+        if not fn.endswith((".cu", ".cuh")) or fn == "cerb_internal.cuh":
+            continue
+        text = re.sub(r"//[^\n]*", "", open(os.path.join(src, fn)).read())
+        for body in re.split(r"__global__", text)[1:]:
+            w = body.find("griddep_wait()")
+            if w < 0:
+                continue
+            seen += 1
+            assert not re.search(r"\breturn\s*;", body[:w]), (fn, body[:80])
+    assert seen >= 12

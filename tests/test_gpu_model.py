@@ -565,3 +565,28 @@ def test_error_codes(cb):
     with pytest.raises(cb.CerbError) as e:            # prompt longer than the page table allows
         eng.prefill(torch.zeros(1, 4000, dtype=torch.int32, device="cuda"), [4000])
     assert e.value.code == cb.E_STATE
+
+
+@pytest.mark.parametrize("head_dim", [64, 128])
+def test_wide_tree_with_no_live_node_in_its_second_window(cb, head_dim):
+    """A tree of more than 128 nodes takes two attention launches per layer; with at most 128 live nodes in every sequence
+    the second one has nothing to do and must still wait for the first."""
+    ms = synth.ModelShape(2, 256, 4, head_dim, 512, 1024, "bf16")
+    rig = Rig(cb, ms, max_tokens=700, max_batch=2, max_nodes=151)
+    tree = synth.random_parent_tree(151, 4, tree_id=8, n_heads=4, kmax=1)
+    lens, live = [600, 333], [128, 77]
+    prompts = [[int(t) for t in synth.make_prompt(ms.vocab, n, seq=80 + b)] for b, n in enumerate(lens)]
+    tok = torch.zeros(2, max(lens), dtype=torch.int32, device="cuda")
+    for b, p in enumerate(prompts):
+        tok[b, :len(p)] = torch.tensor(p, dtype=torch.int32)
+    rig.eng.prefill(tok, lens)
+    tt = torch.stack([synth.make_prompt(ms.vocab, 151, seq=90 + b).to(torch.int32) for b in range(2)]).cuda().contiguous()
+    th = rig.eng.tree(tree)
+    na = torch.tensor(live, dtype=torch.int32, device="cuda")
+    outs = [rig.eng.verify(th, tt, n_active=na, want_hidden=True)[2] for _ in range(5)]
+    assert rig.eng.device_status() == 0
+    for b in range(2):
+        st = orc.prefill(rig.cmodel, rig.sh, prompts[b], 760)
+        want, _ = orc.verify_tree(rig.cmodel, rig.sh, st, [int(t) for t in tt[b, :live[b]]], tree.parent[:live[b]])
+        for hidden in outs:
+            assert close(hidden[b, :live[b]], want, 0) < TOL["bf16"], b
