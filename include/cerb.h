@@ -288,6 +288,12 @@ int cerb_tree_ancestors(const int32_t* parent, int32_t n, uint64_t* anc_out);
  * when few weight tiles exist); scratch holds the split-K partial sums,
  * cerb_gemm_scratch_bytes().  K must be a multiple of 8. */
 int cerb_gemm_scratch_bytes(int32_t M, int32_t N, int32_t K, size_t* bytes_out);
+/* How the bf16 GEMM of more than 128 rows cuts this problem up (host only, for tests and measurement; the paper has no
+ * counterpart): as cerb_gemm runs it (fused = 0, with the scratch that cerb_gemm_scratch_bytes asks for), or inside the
+ * forward with an epilogue (fused = 1).  out8_host: [0] weight tiles of 256 rows that share an activation tile, [1] chunks of
+ * rows, [2] rows of a chunk, [3] tiles, [4] CTA pairs per tile, [5] tiles cut along k into equal shares, [6] CTA pairs,
+ * [7] chains of accumulations per output of a run (fused = 0: fills of an accumulator). */
+int cerb_gemm_plan(int32_t M, int32_t N, int32_t K, int32_t fused, int32_t* out8_host);
 int cerb_gemm(int32_t dtype, const void* X_dev, const void* W_dev, float* out_dev, int32_t M, int32_t N, int32_t K,
               void* scratch_dev, size_t scratch_bytes, void* stream);
 

@@ -8,7 +8,7 @@ from __future__ import annotations
 
 import ctypes as C
 import os
-from typing import Dict, List, Optional, Sequence
+from typing import Dict, List, NamedTuple, Optional, Sequence
 
 import numpy as np
 import torch
@@ -32,6 +32,7 @@ EXPORTS = [
     "cerb_attn_scratch_bytes", "cerb_tree_attention", "cerb_tree_ancestors", "cerb_gemm_scratch_bytes", "cerb_gemm",
     "cerb_read_state", "cerb_device_status", "cerb_launch_count", "cerb_strerror", "cerb_profile_enable",
     "cerb_profile_read", "cerb_tree_attention_noalloc", "cerb_set_wait_cycles", "cerb_wait_diagnosis", "cerb_tree_attention_noalloc_status", "cerb_launch_order_table", "cerb_last_forward_rows",
+    "cerb_gemm_plan",
 ]
 
 
@@ -115,6 +116,7 @@ def lib():
         L.cerb_gemm_scratch_bytes.argtypes = [C.c_int32] * 3 + [C.POINTER(C.c_size_t)]
         L.cerb_gemm.argtypes = [C.c_int32, C.c_void_p, C.c_void_p, C.c_void_p, C.c_int32, C.c_int32, C.c_int32,
                                 C.c_void_p, C.c_size_t, C.c_void_p]
+        L.cerb_gemm_plan.argtypes = [C.c_int32] * 4 + [C.c_void_p]
         L.cerb_read_state.argtypes = [C.c_void_p] * 5
         L.cerb_device_status.argtypes = [C.c_void_p, C.c_void_p]
         L.cerb_profile_enable.argtypes = [C.c_void_p, C.c_int32]
@@ -422,6 +424,24 @@ def tree_attention_noalloc(q: torch.Tensor, k_pool: torch.Tensor, v_pool: torch.
 def tree_attention_noalloc_status() -> int:
     """Device-side status of the calls made through tree_attention_noalloc since the last read (synchronises)."""
     return lib().cerb_tree_attention_noalloc_status(_stream())
+
+
+class GemmPlan(NamedTuple):
+    halves: int
+    chunks: int
+    chunk_rows: int
+    tiles: int
+    pairs_per_tile: int
+    cut_tiles: int
+    pairs: int
+    chains: int
+
+
+def gemm_plan(M: int, N: int, K: int, fused: bool = False) -> GemmPlan:
+    """How the bf16 GEMM of more than 128 rows cuts a problem up (see cerb_gemm_plan)."""
+    out = (C.c_int32 * 8)()
+    _check(lib().cerb_gemm_plan(M, N, K, int(fused), out), "cerb_gemm_plan")
+    return GemmPlan(*out)
 
 
 def gemm(X: torch.Tensor, W: torch.Tensor, scratch: Optional[torch.Tensor] = None) -> torch.Tensor:

@@ -250,7 +250,7 @@ int gemm(cerb_ctx* c, const void* X, const ActMaps* xm, const void* W, const CUt
     if ((size_t)ns * M * N > c->part_floats) return CERB_E_NOMEM;
     *nsplit = ns;
     if (M > 128)
-      return launch_gemm_tile(c, wm, xm, make_tile_plan(M, N, K), out ? out : c->d_part, c->d_gemm_fix, c->d_gemm_tickets, M, N, c->d_status, st,
+      return launch_gemm_tile(c, wm, xm, make_tile_plan(M, N, K, true), out ? out : c->d_part, c->d_gemm_fix, c->d_gemm_tickets, M, N, c->d_status, st,
                               nullptr, gemm_clock_slot(c));
     return launch_gemm_bf16(c, wm, xm, c->d_part, M, N, K, ns, c->d_status, st, gemm_clock_slot(c));
   }
@@ -264,7 +264,7 @@ int gemm_fused(cerb_ctx* c, const void* X, const ActMaps* xm, const void* W, con
                const GemmEpilogue& epi, cudaStream_t st, const GemmNorm* norm = nullptr) {
   ProfScope ps(c, K_GEMM, st);
   if (M <= kFewRows) return launch_gemm_few(X, W, nullptr, M, N, K, st, &epi, norm, gemm_clock_slot(c));
-  return launch_gemm_tile(c, wm, xm, make_tile_plan(M, N, K), nullptr, c->d_gemm_fix, c->d_gemm_tickets, M, N, c->d_status, st, &epi,
+  return launch_gemm_tile(c, wm, xm, make_tile_plan(M, N, K, false), nullptr, c->d_gemm_fix, c->d_gemm_tickets, M, N, c->d_status, st, &epi,
                           gemm_clock_slot(c));
 }
 
@@ -778,6 +778,21 @@ int cerb_gemm_scratch_bytes(int32_t M, int32_t N, int32_t K, size_t* bytes_out) 
   return CERB_OK;
 }
 
+// The stand-alone GEMM's plan above 128 rows.  Its scratch: the status word, and, where pairs add their sums up, 256 bytes further on
+// the counters and the fix-up buffer; what the caller was told to provide decides which plans there is room for.
+static TilePlan standalone_plan(int M, int N, int K) {
+  const size_t room = (size_t)gemm_scratch_slots(M, N, K) * M * N;
+  return make_tile_plan(M, N, K, true, room > kGemmTickets ? room - kGemmTickets : 0);
+}
+
+int cerb_gemm_plan(int32_t M, int32_t N, int32_t K, int32_t fused, int32_t* o) {
+  if (!o || M <= 128 || N < 1 || K < 1) return CERB_E_ARG;
+  const TilePlan g = fused ? make_tile_plan(M, N, K, false) : standalone_plan(M, N, K);
+  const int32_t v[8] = {g.hf, g.mchunks, g.n_act, (int32_t)g.tiles, g.S, g.sk_tiles, g.pairs, fused ? g.chains : g.fills};
+  memcpy(o, v, sizeof(v));
+  return CERB_OK;
+}
+
 // Sums split partials into the output (used only by the stand-alone GEMM entry point).
 __global__ void sum_splits_kernel(const float* __restrict__ part, int nsplit, size_t stride, float* __restrict__ out,
                                   size_t total) {
@@ -804,17 +819,15 @@ int cerb_gemm(int32_t dtype, const void* X_dev, const void* W_dev, float* out_de
   CERB_TRY(make_weight_map(&tw, W_dev, N, K));
   int32_t* status = reinterpret_cast<int32_t*>(scratch_dev);
   float* part = reinterpret_cast<float*>((char*)scratch_dev + 256);
-  CERB_CUDA_OK(cudaMemsetAsync(status, 0, 4, st));
   if (M > 128) {
-    // one sum, which goes straight to the output; behind the status word: the fix-up buffer and, after it, its counters
-    const size_t room = (need - 256) / sizeof(float);
-    const TilePlan g = make_tile_plan(M, N, K, room > kGemmTickets ? room - kGemmTickets : 0);
-    unsigned int* tickets = reinterpret_cast<unsigned int*>(part + g.fix_floats);
-    if (g.fix_floats) CERB_CUDA_OK(cudaMemsetAsync(tickets, 0, kGemmTickets * sizeof(unsigned int), st));
+    // one sum, which goes straight to the output
+    const TilePlan g = standalone_plan(M, N, K);
+    CERB_CUDA_OK(cudaMemsetAsync(status, 0, g.fix_floats ? 256 + kGemmTickets * sizeof(unsigned int) : 4, st));
     CERB_TRY(make_act_map(&tx, X_dev, M, K, g.n_act / 2));
-    CERB_TRY(launch_gemm_tile(nullptr, &tw, &tx, g, out_dev, part, tickets, M, N, status, st));
+    CERB_TRY(launch_gemm_tile(nullptr, &tw, &tx, g, out_dev, part + kGemmTickets, reinterpret_cast<unsigned int*>(part), M, N, status, st));
     return CERB_OK;
   }
+  CERB_CUDA_OK(cudaMemsetAsync(status, 0, 4, st));
   if (M <= kFewRows) return launch_gemm_few(X_dev, W_dev, out_dev, M, N, K, st);
   const int ns = gemm_plan_split(148, M, N, K);
   CERB_TRY(make_act_map(&tx, X_dev, M, K, row_bucket(M)));

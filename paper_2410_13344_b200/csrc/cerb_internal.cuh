@@ -257,11 +257,11 @@ struct GemmEpilogue {
 };
 // gemm_tile.cu: more than 128 rows
 struct TilePlan {
-  int hf, chains, mchunks, n_act, num_kb, pairs, S, per, sk_tiles;
+  int hf, chains, fill, fills, mchunks, n_act, num_kb, pairs, S, per, sk_tiles;
   long long tiles;          // checked to fit 31 bits before launch
   size_t fix_floats;        // what the plan needs of the fix-up buffer
 };
-TilePlan make_tile_plan(int M, int N, int K, size_t max_fix = ~(size_t)0);
+TilePlan make_tile_plan(int M, int N, int K, bool plain, size_t max_fix = ~(size_t)0);
 size_t gemm_fix_floats();   // of any plan
 int launch_gemm_tile(cerb_ctx* c, const CUtensorMap* tmW, const ActMaps* tmX, const TilePlan& g, float* out, float* fix, unsigned int* tickets,
                      int M, int N, int32_t* status, cudaStream_t st, const GemmEpilogue* epi = nullptr,

@@ -13,6 +13,10 @@
 //           tensor-core accumulations loses about half a unit in the last place per step, always towards zero, and 4096 k in
 //           one chain doubled the share of bf16 results that round the other way (keys of the first layer at the 13B width
 //           against the oracle, mean difference: 3.0e-6 in chains of up to 33 k blocks, 6.9e-6 in chains of 80).
+//           Where the fp32 product itself is the result (KIND 0) a chain is `fill` k blocks long: then the other accumulator
+//           goes on, and the epilogue warps add what is there to their registers.  Relative error (2-norm, against float64)
+//           of 4096 k: 4.4e-6 in one chain, 2.1e-6 in two, 1.0e-6 in fills of 16 and 0.5e-6 of 8.  Taking a fill over costs
+//           the warps 3.4 us, of which the last one shows (256 x 12288 x 4096: 36 us in one chain, 40 in fills of 16, 46 of 8).
 //   HF = 2: two MMA rows share one activation tile: 96 KB instead of 128 KB from L2 per 512 x 256 x 64, but the epilogue is
 //           covered only as far as the MMAs of the next tile's first accumulator run under the second one's.
 // A stage is 64 k.  M rows are cut into equal chunks of up to 256, rounded up to 32 rows.
@@ -21,11 +25,13 @@
 //   - whole tiles dealt out in turn; neighbouring pairs work on the chunks of one weight tile, so HBM delivers it once;
 //   - few tiles: S pairs per tile, each a range of k.  Every pair leaves the columns that others finish in a fix-up buffer
 //     and finishes its own share of them, adding the others' sums in k order (a reduce-scatter through L2);
-//   - a last wave that would be nearly empty: between one and two tiles per pair are cut along k into equal shares, which
-//     are done first.  A share is at least one tile long, so at most two pairs meet in a tile: the one that finishes first
-//     leaves its sums in the fix-up buffer, the other adds them to its own and runs the epilogue.
-// Where pairs wait for one another they are CTAs of one launch that fits the GPU at once, and the one waited for has its
-// MMAs behind it or depends on nobody.
+//   - a last wave that would be nearly empty, or fewer tiles than pairs: up to two tiles per pair are cut along k into equal
+//     shares, which are done first.  Of the pairs that meet in a tile the last one to finish its run adds up what the others
+//     have left in the fix-up buffer, in k order, and runs the epilogue.
+// Pairs that wait for one another get on whatever else holds SMs.  With shares, the one that waits is the last: the others are
+// already writing what it waits for.  With S pairs to a tile they have neighbouring block indices and no other tile, so of
+// those resident at any time only the ones of the last tile begun can be waiting for pairs that are not.  (A pair must not
+// be given a second tile there, nor the pairs of a tile be spread out.)
 //
 // Epilogues (KIND; 0 writes the product):
 //   1  SwiGLU.  The weight tile is fetched with 16 gate rows and the 16 up rows of the same features in turn (a 4-D view
@@ -35,6 +41,7 @@
 //      and i + 64 of a rotation pair sit 16 lanes apart (a 5-D view).  Arithmetic and order as in rope_append_kernel.
 //   3  Residual add: the tile is added to the fp32 residual stream.
 // They replace passes of element-wise kernels over the fp32 sums.
+#include <math.h>
 #include <string.h>
 
 #include <type_traits>
@@ -56,7 +63,7 @@ constexpr int kThreads = 64 + 32 * kEpiWarps;
 
 struct TileParams {
   float* out;               // KIND 0: [M][N]; KIND 3: the residual stream [M][N]
-  float* fix;               // [pair][tail, head of a split tile][CTA][accumulator][column / 4][128 lanes][4]; S > 1: no heads
+  float* fix;               // [pair][its first, its last run in a cut tile][CTA][accumulator][column / 4][128 lanes][4]; S > 1: no heads
   unsigned int* tickets;    // [split tile][CTA][epilogue warp], zero on entry and on exit
   bf16* act;                // KIND 1: [M][F]
   RopeEpilogue re;          // KIND 2
@@ -65,7 +72,8 @@ struct TileParams {
   int n_act;                // activation rows per chunk
   int stages;
   int mchunks, num_kb, tiles;
-  int chains;                    // 2: the two accumulators hold the even and the odd k blocks of a tile
+  int chains;                    // 2 (HF = 1): the two accumulators hold the even and the odd k blocks of a tile
+  int fill;                      // KIND 0: k blocks that an accumulator takes before its sums move to registers
   int S;                         // pairs per tile
   int sk_tiles, per, sk_total;   // tiles cut along k into equal shares, k blocks per share, k blocks in all of them
   long long wait_cycles;
@@ -204,8 +212,8 @@ __device__ __forceinline__ void finish(const TileParams& p, const float* v, int 
 }
 
 // Warp by warp, the pairs that share a tile go by one counter in global memory (bounded wait).
-//   two shares (sk): whichever comes first takes the ticket 0, leaves its sums in the fix-up buffer and adds kFixDone; the
-//     other one waits for that and adds them to its own, which have stayed in tensor memory;
+//   shares: each takes a number; all but the last leave their sums in the fix-up buffer and add kFixDone, the last one waits for
+//     that and adds them to its own, which have stayed in tensor memory;
 //   S pairs: each adds 1 when what it leaves is written, waits for all S, and adds kFixDone when it has read what it needs;
 //     the last one to do so puts the counter back to zero.
 constexpr unsigned int kFixDone = 256u;
@@ -364,20 +372,23 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tile_kernel(const __grid_con
         for (int kk = 0; kk < BK / 16; ++kk)
           umma_bf16_pair(d, adesc + (uint64_t)(kk * 2), bdesc + (uint64_t)(kk * 2), idesc, (!fresh || kk > 0) ? 1u : 0u);
       };
-      for (int g = 0; live && w.next(r); ++g) {
+      for (int g = 0; live && w.next(r);) {
         if constexpr (HF == 1) {
           const bool two = p.chains == 2;
-          const int buf = two ? 0 : g & 1;
-          if (!wait(acc_empty[buf], ((uint32_t)(two ? g : g >> 1) & 1u) ^ 1u, 222)) break;
-          for (int k = 0; k < r.nkb; ++k) {
-            if (!wait(full_bar[q.s], q.ph, 223)) break;
-            if (elect_one()) {
-              issue(q.s, 0, tmem_base + (uint32_t)((two ? k & 1 : buf) * TILE_X), k < p.chains);
-              umma_commit_pair(smem_u32(&empty_bar[q.s]));       // the stage is free in both CTAs once these MMAs have read it
-              if (k + 1 == r.nkb) umma_commit_pair(smem_u32(&acc_full[buf]));
+          const int fill = KIND == 0 ? p.fill : r.nkb;
+          for (int left = r.nkb; live && left > 0; left -= fill, ++g) {
+            const int buf = two ? 0 : g & 1, n = min(fill, left);
+            if (!wait(acc_empty[buf], ((uint32_t)(two ? g : g >> 1) & 1u) ^ 1u, 222)) break;
+            for (int k = 0; k < n; ++k) {
+              if (!wait(full_bar[q.s], q.ph, 223)) break;
+              if (elect_one()) {
+                issue(q.s, 0, tmem_base + (uint32_t)((two ? k & 1 : buf) * TILE_X), k < p.chains);
+                umma_commit_pair(smem_u32(&empty_bar[q.s]));       // the stage is free in both CTAs once these MMAs have read it
+                if (k + 1 == n) umma_commit_pair(smem_u32(&acc_full[buf]));
+              }
+              __syncwarp();
+              q.next(p.stages);
             }
-            __syncwarp();
-            q.next(p.stages);
           }
         } else {
           const uint32_t free_ph = ((uint32_t)g & 1u) ^ 1u;
@@ -411,6 +422,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tile_kernel(const __grid_con
             q.next(p.stages);
           }
           q0 = q;
+          ++g;
         }
       }
       if (!live && elect_one()) {
@@ -434,7 +446,8 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tile_kernel(const __grid_con
     // A warp whose wait has run out writes nothing more, but goes through the remaining runs (every later wait is short
     // then): the other epilogue warps meet it at named barriers, other pairs at the counters.
     bool live = true;
-    for (int g = 0; w.next(r); ++g) {
+    int g = 0;                                       // accumulator fills so far
+    while (w.next(r)) {
       const int chunk = r.tile % p.mchunks, row0 = chunk * p.n_act;
       if (KIND == 2 && chunk != chunk_known) {
         // positions and cache rows of the chunk's activation rows
@@ -462,104 +475,143 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tile_kernel(const __grid_con
         first_share = r.tile * p.num_kb / p.per;
         last_share = (r.tile * p.num_kb + p.num_kb - 1) / p.per;
       }
-      const bool split = last_share > first_share;                          // (two pairs: the first has the tile's head)
-      {
-        const bool two = HF == 1 && p.chains == 2;
-        const int acc = HF == 2 ? hf : two ? 0 : g & 1;
-        const uint32_t full_ph = (uint32_t)(HF == 2 || two ? g : g >> 1) & 1u;
-        const int unit = ((r.tile / p.mchunks) * HF + hf) * 2 + rank;
-        if (!mbar_wait_cluster(smem_u32(&acc_full[acc]), full_ph, wc, 224)) live = false;      // the output is undefined from here on
+      const int parts = last_share - first_share + 1;
+      const int unit = ((r.tile / p.mchunks) * HF + hf) * 2 + rank;
+      const bool two = HF == 1 && p.chains == 2;
+      int acc = hf;                                                          // the accumulator that ends up with the run's sums
+      auto filled = [&](int i, uint32_t parity) {
+        if (!mbar_wait_cluster(smem_u32(&acc_full[i]), parity, wc, 224)) live = false;      // the output is undefined from here on
         live = __all_sync(0xffffffffu, live);
         tc_fence_after();
-        const uint32_t taddr = tmem_base + (uint32_t)(acc * TILE_X) + ((uint32_t)(quarter * 32) << 16);
-        auto read_acc = [&](int c0, float* v) {
-          ld_acc(taddr + (uint32_t)c0, v);
-          if (two && r.nkb > 1) {
-            float t[COLS];
-            ld_acc(taddr + (uint32_t)(TILE_X + c0), t);
+      };
+      auto release = [&](int i) {
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive_cluster(ae[i]);          // (the first CTA's own warps arrive the same way)
+      };
+      const uint32_t lanes = tmem_base + ((uint32_t)(quarter * 32) << 16);
+      if constexpr (HF == 2) {
+        filled(hf, (uint32_t)g & 1u);
+        ++g;
+      } else if (KIND != 0 || r.nkb <= p.fill) {
+        acc = two ? 0 : g & 1;
+        filled(acc, (uint32_t)(two ? g : g >> 1) & 1u);
+        ++g;
+      } else {
+        // several fills: this warp's columns wait in registers, the last fill's accumulator receives their sum
+        constexpr int BLOCKS = TILE_X / C_STEP;
+        float held[BLOCKS][COLS];
+        for (int left = r.nkb;; left -= p.fill) {
+          acc = g & 1;
+          filled(acc, (uint32_t)(g >> 1) & 1u);
+          ++g;
+          const uint32_t from = lanes + (uint32_t)(acc * TILE_X + c_first);
 #pragma unroll
-            for (int j = 0; j < COLS; ++j) v[j] += t[j];
-          }
-        };
-        unsigned int* ticket = p.tickets + ((size_t)r.tile * 2 + rank) * kEpiWarps + ew;
-        constexpr size_t kFixAcc = 128 * TILE_X / 4;       // float4s of one CTA's accumulator
-        float4* fix = reinterpret_cast<float4*>(p.fix) + et;
-        auto at = [&](int who, int c0) { return fix + (((size_t)who * 2 + rank) * HF + hf) * kFixAcc + (size_t)(c0 >> 2) * 128; };
-        if (p.S > 1) {
-          const int base = r.tile * p.S, self = pair - base;
-          // 64-column groups of the tile's accumulators belong to the pairs in turn
-          auto owner = [&](int c0) { return (hf * 4 + (c0 >> 6)) % p.S; };
-          if (live)
-            for (int c0 = c_first; c0 < p.n_act; c0 += C_STEP)
-              if (owner(c0) != self) {
-                float v[COLS];
-                read_acc(c0, v);
-                put_fix(at(pair, c0), v);
-              }
-          __threadfence();
-          __syncwarp();
-          if (lane == 0) atomicAdd(ticket, 1u);
-          if (live && !wait_fix(ticket, kFixDone - 1u, (unsigned)p.S, wc, 226)) live = false;
-          live = __all_sync(0xffffffffu, live);
-          __threadfence();
-          if (live)
-            for (int c0 = c_first; c0 < p.n_act; c0 += C_STEP)
-              if (owner(c0) == self) {
-                float v[COLS];
+          for (int i = 0; i < BLOCKS; ++i)
+            if (c_first + i * C_STEP < p.n_act) {
+              float v[COLS];
+              ld_acc(from + (uint32_t)(i * C_STEP), v);
 #pragma unroll
-                for (int j = 0; j < COLS; ++j) v[j] = 0.f;
-                for (int s = 0; s < p.S; ++s) {               // k order
-                  float4 o[COLS / 4];
-                  if (s == self) read_acc(c0, reinterpret_cast<float*>(o));
-                  else get_fix(at(base + s, c0), o);
-                  add(o, v);
-                }
-                finish<KIND>(p, v, unit, quarter, lane, row0, c0, pos_s, kv_s);
-              }
-          __syncwarp();
-          if (lane == 0 && (atomicAdd(ticket, kFixDone) >> 8) == (unsigned)p.S - 1u) *ticket = 0u;       // ready for the next launch
-        } else {
-          // a pair has at most one tail (part 0) and one head (part 1) of a split tile
-          const bool head = pair == first_share;
-          const int mine = pair * 2 + (head ? 1 : 0), other = head ? last_share * 2 : first_share * 2 + 1;
-          bool leave = false;
-          if (split) {
-            unsigned int t = 0;
-            if (lane == 0) t = atomicAdd(ticket, 1u);
-            t = __shfl_sync(0xffffffffu, t, 0);
-            leave = t == 0u;
-            if (!leave && !(t & kFixDone)) {
-              if (!wait_fix(ticket, kFixDone, kFixDone, wc, 228)) live = false;
-              live = __all_sync(0xffffffffu, live);
+              for (int j = 0; j < COLS; ++j) held[i][j] = left == r.nkb ? v[j] : held[i][j] + v[j];
+              if (left <= p.fill) tmem_st16(from + (uint32_t)(i * C_STEP), reinterpret_cast<const uint32_t*>(held[i]));
             }
-            if (!leave) __threadfence();
-          }
+          if (left <= p.fill) break;
+          release(acc);
+        }
+        tmem_st_wait();
+      }
+      const uint32_t taddr = lanes + (uint32_t)(acc * TILE_X);
+      auto read_acc = [&](int c0, float* v) {
+        ld_acc(taddr + (uint32_t)c0, v);
+        if (two && r.nkb > 1) {
+          float t[COLS];
+          ld_acc(taddr + (uint32_t)(TILE_X + c0), t);
+#pragma unroll
+          for (int j = 0; j < COLS; ++j) v[j] += t[j];
+        }
+      };
+      unsigned int* ticket = p.tickets + ((size_t)r.tile * 2 + rank) * kEpiWarps + ew;
+      const size_t fix_acc = 32 * (size_t)p.n_act;            // float4s of one CTA's accumulator
+      float4* fix = reinterpret_cast<float4*>(p.fix) + et;
+      auto at = [&](int who, int c0) { return fix + (((size_t)who * 2 + rank) * HF + hf) * fix_acc + (size_t)(c0 >> 2) * 128; };
+      if (p.S > 1) {
+        const int base = r.tile * p.S, self = pair - base;
+        // 64-column groups of the tile's accumulators belong to the pairs in turn
+        auto owner = [&](int c0) { return (hf * 4 + (c0 >> 6)) % p.S; };
+        if (live)
+          for (int c0 = c_first; c0 < p.n_act; c0 += C_STEP)
+            if (owner(c0) != self) {
+              float v[COLS];
+              read_acc(c0, v);
+              put_fix(at(pair, c0), v);
+            }
+        __threadfence();
+        __syncwarp();
+        if (lane == 0) atomicAdd(ticket, 1u);
+        if (live && !wait_fix(ticket, kFixDone - 1u, (unsigned)p.S, wc, 226)) live = false;
+        live = __all_sync(0xffffffffu, live);
+        __threadfence();
+        if (live)
+          for (int c0 = c_first; c0 < p.n_act; c0 += C_STEP)
+            if (owner(c0) == self) {
+              float v[COLS];
+#pragma unroll
+              for (int j = 0; j < COLS; ++j) v[j] = 0.f;
+              for (int s = 0; s < p.S; ++s) {               // k order
+                float4 o[COLS / 4];
+                if (s == self) read_acc(c0, reinterpret_cast<float*>(o));
+                else get_fix(at(base + s, c0), o);
+                add(o, v);
+              }
+              finish<KIND>(p, v, unit, quarter, lane, row0, c0, pos_s, kv_s);
+            }
+        __syncwarp();
+        if (lane == 0 && (atomicAdd(ticket, kFixDone) >> 8) == (unsigned)p.S - 1u) *ticket = 0u;       // ready for the next launch
+      } else if (parts > 1) {
+        // a share's first run goes to part 0 of its pair's place in the buffer, its last one to part 1
+        auto place = [&](int share) { return share * 2 + (share * p.per / p.num_kb == r.tile ? 0 : 1); };
+        unsigned int t = 0;
+        if (lane == 0) t = atomicAdd(ticket, 1u);
+        t = __shfl_sync(0xffffffffu, t, 0);
+        const bool leave = (int)(t & (kFixDone - 1u)) + 1 < parts;
+        if (leave) {
           if (live)
             for (int c0 = c_first; c0 < p.n_act; c0 += C_STEP) {
               float v[COLS];
-              float4 o[COLS / 4];
-              if (split && !leave) get_fix(at(other, c0), o);
               read_acc(c0, v);
-              if (leave) {
-                put_fix(at(mine, c0), v);
-              } else {
-                if (split) add(o, v);
-                finish<KIND>(p, v, unit, quarter, lane, row0, c0, pos_s, kv_s);
+              put_fix(at(place(pair), c0), v);
+            }
+          __threadfence();
+          __syncwarp();
+          if (lane == 0) atomicAdd(ticket, kFixDone);
+        } else {
+          if (!wait_fix(ticket, ~(kFixDone - 1u), (unsigned)(parts - 1) * kFixDone, wc, 228)) live = false;
+          live = __all_sync(0xffffffffu, live);
+          __threadfence();
+          if (live)
+            for (int c0 = c_first; c0 < p.n_act; c0 += C_STEP) {
+              float v[COLS];
+#pragma unroll
+              for (int j = 0; j < COLS; ++j) v[j] = 0.f;
+              for (int s = first_share; s <= last_share; ++s) {               // k order
+                float4 o[COLS / 4];
+                if (s == pair) read_acc(c0, reinterpret_cast<float*>(o));
+                else get_fix(at(place(s), c0), o);
+                add(o, v);
               }
+              finish<KIND>(p, v, unit, quarter, lane, row0, c0, pos_s, kv_s);
             }
-          if (split) {
-            __threadfence();
-            __syncwarp();
-            if (lane == 0) {
-              if (leave) atomicAdd(ticket, kFixDone);
-              else if (live) *ticket = 0u;                      // ready for the next launch
-            }
-          }
+          __syncwarp();
+          if (lane == 0 && live) *ticket = 0u;                      // ready for the next launch
         }
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive_cluster(ae[acc]);          // (the first CTA's own warps arrive the same way)
+      } else if (live) {
+        for (int c0 = c_first; c0 < p.n_act; c0 += C_STEP) {
+          float v[COLS];
+          read_acc(c0, v);
+          finish<KIND>(p, v, unit, quarter, lane, row0, c0, pos_s, kv_s);
+        }
       }
+      release(acc);
     }
   }
   tc_fence_before();
@@ -576,36 +628,43 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tile_kernel(const __grid_con
 
 }  // namespace
 
-// Estimated time of a plan in us.  Measured on the way: 11.6 TB/s from L2 to all SMs together, about 56 bytes a cycle to one;
-// 6.5 TB/s from HBM; MMAs of 256 rows and less than 120 columns take no less time than those of 120 (issuing); reading out
-// an accumulator of 128 lanes x 256 columns about 2 us, and about as long again for each time it goes through the fix-up
-// buffer.
-static double tile_plan_cost(const TilePlan& g, int M, int N, int K) {
-  const double kMHz = 1750.0, n = g.n_act;
+// Estimated time of a plan in us, launch included.  Fitted to 600 measured plans (129 .. 4096 rows of the 7B and 13B matrices):
+// 11.2 TB/s from L2 to all SMs together, 54 bytes a cycle to one; 6.5 TB/s from HBM, as long as 70 pairs take part; MMAs
+// of 256 rows and less than 120 columns take no less time than those of 120 (issuing); reading out an accumulator of 128 lanes
+// x 256 columns about 1.5 us, and about as long again for each time it goes through the fix-up buffer.  Over 123 measured shapes
+// what it picks is 1 % slower than the fastest plan in the mean, 21 % at the worst (2048 x 5120 x 5120).
+static double tile_plan_cost(const TilePlan& g, int N, int K) {
+  const double kMHz = 1576.0, n = g.n_act;
   const double waves = g.sk_tiles ? (double)g.tiles / kPairs : (double)((g.tiles * g.S + kPairs - 1) / kPairs);
-  const double kbs = waves * ((g.num_kb + g.S - 1) / g.S);
+  const double kbs = !g.sk_tiles ? waves * ((g.num_kb + g.S - 1) / g.S) : g.tiles < kPairs ? (double)g.per : waves * g.num_kb;
   const double tensor = kbs * g.hf * (2 * n > 240 ? 2 * n : 240) / kMHz;
-  const double sm = kbs * (g.hf * (double)A_BYTES + 64 * n) / (56 * kMHz);
-  const double l2 = (double)g.tiles * g.num_kb * (g.hf * 2.0 * A_BYTES + 128 * n) / 11.6e6;
-  const double hbm = (double)N * K * 2 / 6.5e6;
+  const double sm = kbs * (g.hf * (double)A_BYTES + 64 * n) / (53.5 * kMHz);
+  const double l2 = (double)g.tiles * g.num_kb * (g.hf * 2.0 * A_BYTES + 128 * n) / 11.2e6;
+  const double hbm = (double)N * K * 2 / 6.5e6 * (g.pairs < 70 ? 70.0 / g.pairs : 1.0);
   double t = tensor > sm ? tensor : sm;
   if (l2 > t) t = l2;
   if (hbm > t) t = hbm;
-  const double drain = 2.0 * n / 256;
-  t += g.hf == 2 || g.chains == 2 ? (waves < 1 ? 1 : waves) * 1.5 * drain : drain;
-  if (g.S > 1) t += 2 + g.hf * drain * 2 * (g.S - 1) / g.S;
-  if (g.sk_tiles) t += 3 + 1.5 * g.hf * drain;
+  if (g.sk_tiles && g.mchunks > 2) t *= 1.12;               // (shares walk k at their own offsets: L2 serves fewer of them)
+  const double drain = 1.45 * n / 256;
+  t += 13 + (g.hf == 2 || g.chains == 2 ? (waves < 1 ? 1 : waves) * 1.7 * drain : drain);
+  if (g.S > 1) t += 1.7 + 0.95 * g.hf * drain * (g.S - 1) / g.S + (g.hf == 2 ? 1.75 * (g.S - 1) : 0.0);
+  if (g.fills > 1) {
+    const double over = (waves < 1 ? 1 : waves) * g.fills;              // fills taken over, one after the other
+    t += (3 + over) * n / 256;
+    if (t < 13 + 3.4 * over * n / 256) t = 13 + 3.4 * over * n / 256;
+  }
+  if (g.sk_tiles) t += 5.8 + drain * (g.tiles < kPairs ? (g.num_kb + g.per - 1) / g.per - 1 : 1);
   return t;
 }
 
-// max_fix: floats of fix-up buffer that the caller has.
-TilePlan make_tile_plan(int M, int N, int K, size_t max_fix) {
+// plain: the fp32 product itself is the result.  max_fix: floats of fix-up buffer that the caller has.
+TilePlan make_tile_plan(int M, int N, int K, bool plain, size_t max_fix) {
   TilePlan best;
   double best_t = 0;
   const int least_chunks = (M + TILE_X - 1) / TILE_X;
   // (HF = 2 has no room for two chains: from three chunks of rows on)
-  for (int hf = 1; hf <= (least_chunks > 2 ? 2 : 1); ++hf)
-    for (int c = least_chunks; c <= least_chunks + least_chunks / 4 + 1; ++c)
+  for (int hf = 1; hf <= (least_chunks > 2 && !plain ? 2 : 1); ++hf)
+    for (int c = least_chunks; c <= least_chunks + least_chunks / 4 + 2; ++c)
       for (int S = 1; S <= 4 * hf; ++S)
         for (int sk = 0; sk <= (S == 1 && hf == 1 ? 1 : 0); ++sk) {      // (two accumulators per share: never the fastest)
           TilePlan g;
@@ -620,21 +679,29 @@ TilePlan make_tile_plan(int M, int N, int K, size_t max_fix) {
           g.pairs = kPairs;
           if (S > 1) {
             if (g.tiles * S > kPairs || g.num_kb < 4 * S) break;
-            g.fix_floats = (size_t)g.tiles * S * 2 * hf * 128 * TILE_X;
+            g.fix_floats = (size_t)g.tiles * S * 2 * hf * 128 * g.n_act;
           }
           if (g.tiles * S < kPairs) g.pairs = (int)g.tiles * S;
           if (sk) {
             const int rem = (int)(g.tiles % kPairs);
-            if (g.tiles < kPairs || !rem) continue;
-            // shares walk k at their own offsets: what they read has to stay in L2 meanwhile
-            if (c > 1 && g.tiles < 3 * kPairs && ((double)M + N) * K * 2 > 64e6) continue;
-            g.sk_tiles = kPairs + rem;
+            if (!rem) continue;
+            g.sk_tiles = g.tiles < kPairs ? rem : kPairs + rem;
             g.per = (g.sk_tiles * g.num_kb + kPairs - 1) / kPairs;
-            g.fix_floats = (size_t)kPairs * 2 * 2 * hf * 128 * TILE_X;
+            if (g.tiles < kPairs && g.per < 4) g.per = 4;
+            if (g.tiles < kPairs && g.per >= g.num_kb) continue;          // (as good as whole tiles)
+            g.pairs = (g.sk_tiles * g.num_kb + g.per - 1) / g.per;
+            g.fix_floats = (size_t)g.pairs * 2 * 2 * hf * 128 * g.n_act;
           }
           if (g.fix_floats > max_fix) continue;
-          g.chains = hf == 1 && g.tiles * S <= 2 * kPairs ? 2 : 1;
-          const double t = tile_plan_cost(g, M, N, K);
+          // a chain is no longer than the product cut evenly over all pairs would make it (in pieces of 4 k blocks at least), nor
+          // than half a run
+          const int run = sk && g.tiles < kPairs ? g.per : (g.num_kb + S - 1) / S;
+          const double piece = 0.9 * ((N + 511) / 512) * g.num_kb * least_chunks / kPairs;
+          g.fills = !plain ? 1 : (int)ceil(run / (piece < 4 ? 4 : piece));
+          if (plain && g.fills < 2 && run >= 8) g.fills = 2;
+          g.fill = (run + g.fills - 1) / g.fills;
+          g.chains = !plain && hf == 1 && g.tiles * S <= 2 * kPairs ? 2 : 1;
+          const double t = tile_plan_cost(g, N, K);
           if (best_t == 0 || t < best_t) {
             best = g;
             best_t = t;
@@ -673,7 +740,7 @@ int launch_gemm_tile(cerb_ctx* c, const CUtensorMap* tmW, const ActMaps* tmX, co
   q.fix = fix; q.tickets = tickets; q.status = status;
   q.M = M; q.N = N;
   q.n_act = g.n_act; q.mchunks = g.mchunks; q.num_kb = g.num_kb; q.tiles = (int)g.tiles;
-  q.chains = g.chains; q.S = g.S; q.sk_tiles = g.sk_tiles; q.per = g.per; q.sk_total = g.sk_tiles * g.num_kb;
+  q.chains = g.chains; q.fill = g.fill; q.S = g.S; q.sk_tiles = g.sk_tiles; q.per = g.per; q.sk_total = g.sk_tiles * g.num_kb;
   q.wait_cycles = wait_cycles();
   q.clk = clock_slot;
   const CUtensorMap& x = tmX->box(g.n_act / 2);                      // each CTA loads half of a chunk's rows
@@ -687,8 +754,9 @@ int launch_gemm_tile(cerb_ctx* c, const CUtensorMap* tmW, const ActMaps* tmX, co
     return kind == 1   ? launch_kind<1, HF>(*tmW, x, q, g.pairs, st)
            : kind == 2 ? launch_kind<2, HF>(*tmW, x, q, g.pairs, st)
            : kind == 3 ? launch_kind<3, HF>(*tmW, x, q, g.pairs, st)
-                       : launch_kind<0, HF>(*tmW, x, q, g.pairs, st);
+                       : launch_kind<0, 1>(*tmW, x, q, g.pairs, st);
   };
+  if (g.hf == 2 && kind == 0) return CERB_E_ARG;
   const int rc = g.hf == 2 ? run(std::integral_constant<int, 2>()) : run(std::integral_constant<int, 1>());
   if (rc != CERB_OK) return rc;
   CERB_LAUNCH_CHECK(c);
