@@ -80,8 +80,8 @@ struct AttnParams {
   int32_t* status;
   int n, H, max_pages, nsplit, oob_row;
   int B, Bw;                // sequences; (sequence, window) pairs
-  int win;                  // > 1: a prefill chunk of up to win * 128 consecutive tokens per sequence, one window of 128 query
-                            // rows per blockIdx.z (locate_window); 1 otherwise
+  int win, win0;            // a prefill chunk of consecutive tokens per sequence: its windows of 128 query rows win0 .. win0 + win - 1, one
+                            // per blockIdx.z (locate_window); 1 and 0 otherwise
   int row0, rows;           // query rows row0 .. row0 + rows - 1 of the tree are this launch's (q, out, lse and anc already point
                             // at row0); a tree of more than 128 nodes takes two launches.  n stays the tree's node count
                             // (the row stride between sequences); only keys below row0 + rows can be ancestors of these rows.
@@ -97,7 +97,7 @@ struct AttnParams {
 // launch.  The last windows see the most keys and come first, so that the short ones fill the launch's tail.
 __device__ __forceinline__ void locate_window(const AttnParams& p, int z, int& b, int& shift) {
   b = p.win > 1 ? z % p.B : z;
-  shift = p.win > 1 ? (p.win - 1 - z / p.B) * kAttnRowsPerLaunch : 0;
+  shift = (p.win0 + (p.win > 1 ? p.win - 1 - z / p.B : 0)) * kAttnRowsPerLaunch;
 }
 
 template <int DH, int WQ, int WK, int STAGES>
@@ -1375,15 +1375,24 @@ size_t attn_scratch_bytes(int B, int n, int H, int Dh) {
   return kCounterBytes + rows * (size_t)nq_pad(n) * (size_t)(Dh + 4) * sizeof(float);
 }
 
+// With clusters the splits of a (sequence, head) merge through distributed shared memory: at most 8 of them
+// (the portable cluster size).  CERB_ATTN_CLUSTER=0 keeps the merge through global partials (up to 32 splits).
+static bool attn_use_cluster() {
+  static const int v = getenv("CERB_ATTN_CLUSTER") ? atoi(getenv("CERB_ATTN_CLUSTER")) : 1;
+  return v != 0;
+}
+static int attn_max_split() { return attn_use_cluster() ? 8 : kMaxSplit; }
+
 // One launch of the bf16 kernels over query rows row0 .. row0 + rows - 1 (rows <= 128) of every sequence's tree.
-// win > 1: `rows` is 128 and the launch covers that many windows of a prefill chunk per sequence side by side.
+// A prefill chunk: `rows` is 128 and the launch covers its windows win0 .. win0 + win - 1 of every sequence side by side.
 static int launch_attn_window(const cerb_attn_args* a, int row0, int rows, const CUtensorMap* tmK, const CUtensorMap* tmV,
-                              int32_t* status, cudaStream_t st, const int32_t* row_off, int win = 1) {
+                              int32_t* status, cudaStream_t st, const int32_t* row_off, int win = 1, int win0 = 0) {
   AttnParams p;
   const int Bw = a->B * win;             // (sequence, window) pairs
   p.B = a->B;
   p.Bw = Bw;
   p.win = win;
+  p.win0 = win0;
   const size_t row_elems = (size_t)a->n_heads * a->head_dim;
   p.q = (const bf16*)a->q + (size_t)row0 * row_elems;
   p.page_table = a->page_table;
@@ -1410,13 +1419,11 @@ static int launch_attn_window(const cerb_attn_args* a, int row0, int rows, const
   const int np_ = nq_pad(rows);
   const bool auto_tc = np_ == 128;
   const bool tensor_path = a->head_dim == 128 && (force_tc < 0 ? auto_tc : force_tc != 0);
-  // With clusters the splits of a (sequence, head) merge through distributed shared memory: at most 8 of them
-  // (the portable cluster size).  CERB_ATTN_CLUSTER=0 keeps the merge through global partials (up to 32 splits).
-  static const int use_cluster = getenv("CERB_ATTN_CLUSTER") ? atoi(getenv("CERB_ATTN_CLUSTER")) : 1;
+  const bool use_cluster = attn_use_cluster();
   // CTAs that fit at once: one per SM for the tensor-core kernel and for the warp-MMA layouts of 32 rows and more
   // (288 threads x 168 registers), two per SM for the 16-row layout (160 threads); the grid is planned to fit one wave
   const int resident = (tensor_path || np_ > 16) ? 148 : kTargetCtas;
-  p.nsplit = plan_nsplit(Bw, a->n_heads, nq_pad(rows), a->max_len, resident, true, use_cluster ? 8 : kMaxSplit);
+  p.nsplit = plan_nsplit(Bw, a->n_heads, nq_pad(rows), a->max_len, resident, true, attn_max_split());
   if (p.nsplit < 1) return CERB_E_SHAPE;
   p.oob_row = a->n_pool_pages * a->n_heads * CERB_PAGE;
   p.scale_log2 = a->scale * 1.4426950408889634f;
@@ -1450,8 +1457,7 @@ static int launch_attn_window(const cerb_attn_args* a, int row0, int rows, const
   if (kt_path) {
     const int tiles = (a->max_len + KT_TILE - 1) / KT_TILE;
     int want = 148 / (Bw * a->n_heads);
-    const int max_split = use_cluster ? 8 : kMaxSplit;
-    if (want > max_split) want = max_split;
+    if (want > attn_max_split()) want = attn_max_split();
     if (want > tiles) want = tiles;
     if (want < 1) want = 1;
     const int per = (tiles + want - 1) / want;
@@ -1523,8 +1529,15 @@ int launch_tree_attention(cerb_ctx* c, const cerb_attn_args* a, const CUtensorMa
   if (win > 1) {
     // a prefill chunk of more than 128 tokens per sequence: its windows are CTAs of one launch
     if (a->scratch_bytes < attn_scratch_bytes(a->B, kAttnRowsPerLaunch, a->n_heads, a->head_dim)) return CERB_E_NOMEM;
-    CERB_TRY(launch_attn_window(a, 0, kAttnRowsPerLaunch, tmK, tmV, status, st, row_off, win));
-    CERB_LAUNCH_CHECK(c);
+    // ... of as few as there is a plan for: with many windows no keys are split, and a CTA's page list ends at 16384 keys
+    int per = win;
+    while (per > 1 && plan_nsplit(a->B * per, a->n_heads, kAttnRowsPerLaunch, a->max_len, 148, true, attn_max_split()) < 1) --per;
+    const int launches = (win + per - 1) / per;
+    per = (win + launches - 1) / launches;
+    for (int win0 = 0; win0 < win; win0 += per) {
+      CERB_TRY(launch_attn_window(a, 0, kAttnRowsPerLaunch, tmK, tmV, status, st, row_off, win - win0 < per ? win - win0 : per, win0));
+      CERB_LAUNCH_CHECK(c);
+    }
     return CERB_OK;
   }
   if (a->scratch_bytes < attn_scratch_bytes(a->B, a->n, a->n_heads, a->head_dim)) return CERB_E_NOMEM;
