@@ -52,7 +52,10 @@ __global__ void __launch_bounds__(256) gemm_f32_kernel(const float* __restrict__
 // 6 MFLOP (a request to the tiny fp32 model: 11.1 ms, 2.8 with this kernel and the attention in fours).  Here a CTA takes
 // 16 x 16 outputs, fetches 256 k of both operands in one round, the next 256 while it multiplies, and its eight warps take 32 k
 // each; their sums meet in shared memory at the end.
+// VEC: the rows of both operands start on 16-byte boundaries (K a multiple of 4, aligned pointers) and come in 16-byte loads;
+// otherwise value by value.
 constexpr int SM_T = 16, SM_K = 256, SM_LD = SM_K + 4;
+template <bool VEC>
 __global__ void __launch_bounds__(256) gemm_f32_small_kernel(const float* __restrict__ X, const float* __restrict__ W,
                                                              float* __restrict__ out, int M, int N, int K) {
   __shared__ __align__(16) float sx[SM_T][SM_LD], sw[SM_T][SM_LD];
@@ -64,7 +67,7 @@ __global__ void __launch_bounds__(256) gemm_f32_small_kernel(const float* __rest
   auto piece = [&](const float* P, int rows, int row, int k) {
     if (row >= rows || k >= K) return make_float4(0.f, 0.f, 0.f, 0.f);
     const float* at = P + (size_t)row * K + k;
-    if ((K & 3) == 0) return *reinterpret_cast<const float4*>(at);
+    if constexpr (VEC) return *reinterpret_cast<const float4*>(at);
     return make_float4(at[0], k + 1 < K ? at[1] : 0.f, k + 2 < K ? at[2] : 0.f, k + 3 < K ? at[3] : 0.f);
   };
   auto fetch_w = [&](int k0) {
@@ -131,8 +134,10 @@ int launch_gemm_f32(cerb_ctx* c, const float* X, const float* W, float* out, int
   if ((long long)((N + TN - 1) / TN) * ((M + TM - 1) / TM) < kFewTiles) {
     dim3 small((N + SM_T - 1) / SM_T, (M + SM_T - 1) / SM_T);
     // (a caller without a model may hand over as weights what the kernel in front is still writing)
-    if (c) launch_pdl(gemm_f32_small_kernel, small, dim3(256), 0, st, X, W, out, M, N, K);
-    else gemm_f32_small_kernel<<<small, 256, 0, st>>>(X, W, out, M, N, K);
+    const bool vec = K % 4 == 0 && (((uintptr_t)X | (uintptr_t)W) & 15) == 0;
+    auto kern = vec ? gemm_f32_small_kernel<true> : gemm_f32_small_kernel<false>;
+    if (c) launch_pdl(kern, small, dim3(256), 0, st, X, W, out, M, N, K);
+    else kern<<<small, 256, 0, st>>>(X, W, out, M, N, K);
     CERB_LAUNCH_CHECK(c);
     return CERB_OK;
   }

@@ -26,3 +26,13 @@ def test_weights_may_be_what_the_previous_call_wrote():
     W = cb.gemm(X, V)                                        # a long launch (65536 deep) ...
     out = cb.gemm(Y, W)                                      # ... whose output (0.03 in size) is the next one's weights
     assert close(out, orc.linear(Y.cpu(), W.cpu()), 0) < 1e-5
+
+
+# Operands that start one, two or three values into a buffer: nothing but 4-byte alignment is asked for.
+@pytest.mark.parametrize("M,N,K", [(16, 768, 256), (5, 33, 260), (3, 40, 255), (1024, 1184, 64)])
+@pytest.mark.parametrize("dx,dw", [(1, 0), (0, 2), (3, 3)])
+def test_gemm_takes_operands_at_any_offset(M, N, K, dx, dw):
+    fx = synth.normal(13, 6, (M * K + 4,), 1.0, dtype=torch.float32, device="cuda")
+    fw = synth.normal(13, 7, (N * K + 4,), 0.05, dtype=torch.float32, device="cuda")
+    X, W = fx[dx:dx + M * K].view(M, K), fw[dw:dw + N * K].view(N, K)
+    assert close(cb.gemm(X, W), orc.linear(X.cpu(), W.cpu()), 0) < 1e-5
