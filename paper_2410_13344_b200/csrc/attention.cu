@@ -909,6 +909,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tree_attn_tc_kernel(const __gri
       const float w0 = ex2(x0.x - u), w1 = ex2(x1.x - u), Lsum = x0.y * w0 + x1.y * w1, inv = 1.0f / Lsum;
       const float f0 = w0 * inv, f1 = w1 * inv;
       bf16* o = p.out + ((qrow + (valid ? row : 0)) * p.H + h) * DH + g * 64;
+      const bool wide = (reinterpret_cast<uintptr_t>(p.out) & 15) == 0;      // (8-byte alignment is all that the other routes ask for)
 #pragma unroll 1
       for (int c0 = 0; c0 < 64; c0 += 16) {
         uint32_t r0[16], r1[16];
@@ -925,9 +926,12 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tree_attn_tc_kernel(const __gri
           }
           w[e] = pack_bf16(a, c);
         }
-        if (valid) {
+        if (valid && wide) {
           reinterpret_cast<uint4*>(o + c0)[0] = make_uint4(w[0], w[1], w[2], w[3]);
           reinterpret_cast<uint4*>(o + c0)[1] = make_uint4(w[4], w[5], w[6], w[7]);
+        } else if (valid) {
+#pragma unroll
+          for (int e = 0; e < 4; ++e) reinterpret_cast<uint2*>(o + c0)[e] = make_uint2(w[2 * e], w[2 * e + 1]);
         }
       }
       if (g == 0 && valid && p.lse) p.lse[((size_t)b * p.H + h) * p.n + row] = (M + log2f(Lsum)) * LN2;
@@ -1140,7 +1144,8 @@ __global__ void __launch_bounds__(ONE_WARPS * 32, 2) tree_attn_one_kernel(const 
     }
   };
   float q[8], o[8], m = -INFINITY, l = 0.f;
-  unpack(*reinterpret_cast<const uint4*>(p.q + (row * p.H + h) * DH + d0), q);
+  const uint32_t* qw = reinterpret_cast<const uint32_t*>(p.q + (row * p.H + h) * DH + d0);      // (q: 4-byte alignment, as for any up to 16 rows)
+  unpack(make_uint4(qw[0], qw[1], qw[2], qw[3]), q);
 #pragma unroll
   for (int e = 0; e < 8; ++e) o[e] = 0.f;
   for (; pg < pg1; pg += ONE_WARPS) {
