@@ -6,6 +6,7 @@ from oracle import cerberus_oracle as orc
 from paper_2410_13344_b200 import binding as cb
 from paper_2410_13344_b200 import synth
 from tests.helpers import close
+from tests.test_gpu_kernels import _attention_case
 
 pytestmark = pytest.mark.gpu
 
@@ -36,3 +37,13 @@ def test_gemm_takes_operands_at_any_offset(M, N, K, dx, dw):
     fw = synth.normal(13, 7, (N * K + 4,), 0.05, dtype=torch.float32, device="cuda")
     X, W = fx[dx:dx + M * K].view(M, K), fw[dw:dw + N * K].view(N, K)
     assert close(cb.gemm(X, W), orc.linear(X.cpu(), W.cpu()), 0) < 1e-5
+
+
+# The list of a node's live ancestors: words of the bitmask full and cut by the number of live nodes, none but the node itself,
+# more ancestors than a round of all warps (a chain), no prefix
+@pytest.mark.parametrize("n,depth,n_active,lens", [(1, 1, None, [0, 37]), (64, 6, [64, 63], [16, 0]), (65, 6, [65, 64], [5, 300]), (128, 127, [128, 127], [3, 50]),
+                                                   (192, 8, [129, 192], [16, 100]), (192, 191, [192, 1], [0, 7])])
+@pytest.mark.parametrize("head_dim", [64, 128])
+def test_attention_over_listed_ancestors(n, depth, n_active, lens, head_dim):
+    for got_o, got_l, O, l in _attention_case(cb, "fp32", 2, n, 2, head_dim, lens, depth, seed_id=170, n_active=n_active):
+        assert close(got_o, O, 0) < 1e-5 and close(got_l, l, 0) < 1e-5
