@@ -318,7 +318,9 @@ __global__ void __launch_bounds__(TK_WARPS * 32) topk_part_kernel(const float* _
   const float* r = logits + ((size_t)b * Hc + h) * V;
   const int k = kper[h];
   const int per = (V + kTopkChunks - 1) / kTopkChunks;
-  const int c1 = min(V, (ch + 1) * per), part = (per + TK_WARPS - 1) / TK_WARPS;
+  // (what one warp holds at once goes to one warp: its list is the chunk's)
+  const bool one = per <= 32 * TK_HELD;
+  const int c1 = min(V, (ch + 1) * per), part = one ? per : (per + TK_WARPS - 1) / TK_WARPS;
   const int j0 = min(c1, ch * per + warp * part), j1 = min(c1, j0 + part);
   if (lane < CERB_MAX_TOPK) { lv[warp][lane] = -INFINITY; li[warp][lane] = 0x7fffffff; }
   for (int base = j0; base < j1; base += 32 * TK_HELD) {
@@ -338,6 +340,15 @@ __global__ void __launch_bounds__(TK_WARPS * 32) topk_part_kernel(const float* _
       if (lane == 0) { lv[warp][round] = bv; li[warp][round] = bi; }
     });
   }
+  const size_t o = (((size_t)b * Hc + h) * kTopkChunks + ch) * CERB_MAX_TOPK;
+  if (one) {
+    __syncwarp();
+    if (warp == 0 && lane < k) {
+      cand_v[o + lane] = lv[0][lane];
+      cand_i[o + lane] = li[0][lane] == 0x7fffffff ? -1 : li[0][lane];
+    }
+    return;
+  }
   __syncthreads();
   if (warp == 0) {
     constexpr int N = TK_WARPS * CERB_MAX_TOPK / 32;
@@ -348,7 +359,6 @@ __global__ void __launch_bounds__(TK_WARPS * 32) topk_part_kernel(const float* _
       v[e] = (&lv[0][0])[e * 32 + lane];
       id[e] = (&li[0][0])[e * 32 + lane];
     }
-    const size_t o = (((size_t)b * Hc + h) * kTopkChunks + ch) * CERB_MAX_TOPK;
     warp_topk(v, id, k, [&](int round, float bv, int bi) {
       if (lane == 0) {
         cand_v[o + round] = bv;
