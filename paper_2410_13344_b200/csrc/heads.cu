@@ -113,11 +113,12 @@ __global__ void __launch_bounds__(WARPS * 32) head_gemv_kernel(const LevelParams
   }
 }
 
-// v = hi + mid + lo to 24 bits, a term every `stride`.
+// v = hi + mid + lo, all 24 bits, a term every `stride`.  Cut off, not rounded: the largest values would round to infinity.  An
+// infinity is its own first term (inf - inf would make the others, and with them every product, NaN).
 __device__ __forceinline__ void store_terms(bf16* at, size_t stride, float v) {
-  const bf16 hi = __float2bfloat16_rn(v);
-  const float r = v - __bfloat162float(hi);
-  const bf16 mid = __float2bfloat16_rn(r);
+  const bf16 hi = __float2bfloat16_rz(v);
+  const float r = isinf(v) ? 0.f : v - __bfloat162float(hi);
+  const bf16 mid = __float2bfloat16_rz(r);
   at[0] = hi;
   at[stride] = mid;
   at[2 * stride] = __float2bfloat16_rn(r - __bfloat162float(mid));

@@ -50,3 +50,22 @@ def test_draft_logits_are_fp32_sums(B):
         for h, want in enumerate(orc.heads_forward(h_last[b].double(), rig.cheads, rig.csrc)):
             got, want = logits[b, h].double().cpu(), want.double()
             assert float((got - want).norm() / want.norm()) < 3e-7, (b, h)
+
+
+@pytest.mark.parametrize("B", [1, 4])
+def test_infinite_states_stay_infinite(B):
+    """One infinite component in the last hidden state and weights without a sign: every logit is +inf, and the lowest ids win."""
+    ms = synth.ModelShape(1, 64, 2, 64, 128, 300, "bf16")
+    rig = Rig(cb, ms, n_cheads=2, n_levels=2, topk=(5, 3), concat_level=1, max_batch=B, max_tokens=32, max_nodes=16)
+    tok = synth.make_prompt(300, 8, seq=61).to(torch.int32).cuda().repeat(B, 1)
+    rig.eng.prefill(tok, [6] * B)
+    c = int(torch.argmax(rig.eng.read_state()[2][0].float()))
+    rig.model["final_norm"][c] = float("inf")
+    for w in rig.heads.values():
+        w.copy_(w.abs() + 0.01)
+    rig.eng.prefill(tok, [6] * B)
+    assert bool(torch.isinf(rig.eng.read_state()[2][:, c]).all())
+    _, topk, logits = rig.eng.draft(rig.eng.tree(synth.best_first_tree(12, rig.topk)), want_logits=True)
+    assert bool((logits == float("inf")).all())
+    for h in range(2):
+        assert topk[:, h, :rig.topk[h]].tolist() == [list(range(rig.topk[h]))] * B
