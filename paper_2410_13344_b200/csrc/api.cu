@@ -244,7 +244,7 @@ int gemm(cerb_ctx* c, const void* X, const ActMaps* xm, const void* W, const CUt
   if (c->bf16) {
     if (M <= kFewRows) {
       *nsplit = 1;
-      return launch_gemm_few(X, W, out ? out : c->d_part, M, N, K, st, nullptr, nullptr, gemm_clock_slot(c));
+      return launch_gemm_few(c, X, W, out ? out : c->d_part, M, N, K, st, nullptr, nullptr, gemm_clock_slot(c));
     }
     int ns = gemm_plan_split(c->sm_count, M, N, K);
     if ((size_t)ns * M * N > c->part_floats) return CERB_E_NOMEM;
@@ -263,7 +263,7 @@ int gemm(cerb_ctx* c, const void* X, const ActMaps* xm, const void* W, const CUt
 int gemm_fused(cerb_ctx* c, const void* X, const ActMaps* xm, const void* W, const CUtensorMap* wm, int M, int N, int K,
                const GemmEpilogue& epi, cudaStream_t st, const GemmNorm* norm = nullptr) {
   ProfScope ps(c, K_GEMM, st);
-  if (M <= kFewRows) return launch_gemm_few(X, W, nullptr, M, N, K, st, &epi, norm, gemm_clock_slot(c));
+  if (M <= kFewRows) return launch_gemm_few(c, X, W, nullptr, M, N, K, st, &epi, norm, gemm_clock_slot(c));
   return launch_gemm_tile(c, wm, xm, make_tile_plan(M, N, K, false), nullptr, c->d_gemm_fix, c->d_gemm_tickets, M, N, c->d_status, st, &epi,
                           gemm_clock_slot(c));
 }
@@ -828,7 +828,7 @@ int cerb_gemm(int32_t dtype, const void* X_dev, const void* W_dev, float* out_de
     return CERB_OK;
   }
   CERB_CUDA_OK(cudaMemsetAsync(status, 0, 4, st));
-  if (M <= kFewRows) return launch_gemm_few(X_dev, W_dev, out_dev, M, N, K, st);
+  if (M <= kFewRows) return launch_gemm_few(nullptr, X_dev, W_dev, out_dev, M, N, K, st);
   const int ns = gemm_plan_split(148, M, N, K);
   CERB_TRY(make_act_map(&tx, X_dev, M, K, row_bucket(M)));
   CERB_TRY(launch_gemm_bf16(nullptr, &tw, &tx, part, M, N, K, ns, status, st));

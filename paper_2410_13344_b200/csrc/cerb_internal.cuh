@@ -273,7 +273,7 @@ struct GemmNorm {           // the GEMM's X is RMSNorm(x) * gain of the residual
   const void* gain;
   float eps;
 };
-int launch_gemm_few(const void* X, const void* W, float* out, int M, int N, int K, cudaStream_t st, const GemmEpilogue* epi = nullptr,
+int launch_gemm_few(cerb_ctx* c, const void* X, const void* W, float* out, int M, int N, int K, cudaStream_t st, const GemmEpilogue* epi = nullptr,
                     const GemmNorm* norm = nullptr, unsigned long long* clock_slot = nullptr);
 bool gemm_few_normalises(int M, int K);
 int launch_gemm_bf16(cerb_ctx* c, const CUtensorMap* tmW, const ActMaps* tmX, float* out, int M, int N, int K,

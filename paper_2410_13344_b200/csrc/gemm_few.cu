@@ -257,7 +257,7 @@ int launch(FewParams p, cudaStream_t st) {
 
 bool gemm_few_normalises(int M, int K) { return M <= kFewRows && norm_smem(M, K) <= kNormSmem; }
 
-int launch_gemm_few(const void* X, const void* W, float* out, int M, int N, int K, cudaStream_t st, const GemmEpilogue* epi,
+int launch_gemm_few(cerb_ctx* c, const void* X, const void* W, float* out, int M, int N, int K, cudaStream_t st, const GemmEpilogue* epi,
                     const GemmNorm* norm, unsigned long long* clock_slot) {
   if (M < 1 || M > kFewRows || N < 1 || K < 1 || K % 8 || (((uintptr_t)X | (uintptr_t)W) & 15)) return CERB_E_SHAPE;
   FewParams p;
@@ -273,23 +273,29 @@ int launch_gemm_few(const void* X, const void* W, float* out, int M, int N, int 
     p.gain = (const bf16*)norm->gain;
     p.eps = norm->eps;
   }
+  int rc = CERB_E_SHAPE;
   switch (epi ? epi->kind : 0) {
-    case 0: return launch<0, false>(p, st);
+    case 0: rc = launch<0, false>(p, st); break;
     case 1:
       if ((N & 1) || !epi->act) return CERB_E_SHAPE;
       p.F = N / 2;
       p.act = (bf16*)epi->act;
-      return norm ? launch<1, true>(p, st) : launch<1, false>(p, st);
+      rc = norm ? launch<1, true>(p, st) : launch<1, false>(p, st);
+      break;
     case 2:
       if (!epi->rope || N != 3 * epi->rope->H * 128) return CERB_E_SHAPE;
       p.re = *epi->rope;
-      return norm ? launch<2, true>(p, st) : launch<2, false>(p, st);
+      rc = norm ? launch<2, true>(p, st) : launch<2, false>(p, st);
+      break;
     case 3:
       if (!epi->x) return CERB_E_SHAPE;
       p.out = epi->x;
-      return launch<3, false>(p, st);
+      rc = launch<3, false>(p, st);
+      break;
   }
-  return CERB_E_SHAPE;
+  if (rc != CERB_OK) return rc;
+  CERB_LAUNCH_CHECK(c);
+  return CERB_OK;
 }
 
 }  // namespace cerb

@@ -590,3 +590,20 @@ def test_wide_tree_with_no_live_node_in_its_second_window(cb, head_dim):
         want, _ = orc.verify_tree(rig.cmodel, rig.sh, st, [int(t) for t in tt[b, :live[b]]], tree.parent[:live[b]])
         for hidden in outs:
             assert close(hidden[b, :live[b]], want, 0) < TOL["bf16"], b
+
+
+# (nodes, batch, head_dim, mlp_dim) -> the variant of the launch sequence that such a forward takes
+@pytest.mark.parametrize("n,B,head_dim,mlp,variant", [(1, 1, 128, 368, 8), (2, 4, 128, 360, 8), (2, 4, 64, 360, 6), (9, 1, 128, 368, 0), (64, 2, 64, 368, 0),
+                                                      (80, 2, 128, 368, 3), (80, 2, 128, 360, 7), (80, 2, 64, 368, 6), (80, 2, 64, 360, 5)])
+def test_every_launch_is_counted(cb, n, B, head_dim, mlp, variant):
+    """The launch count over a forward of three layers against the exported launch sequence (set-up, three layers, tail)."""
+    import ctypes as C
+    ms = synth.ModelShape(3, 256, 2, head_dim, mlp, 512, "bf16")
+    rig = Rig(cb, ms, max_tokens=64, max_batch=B, max_nodes=n)
+    rig.eng.prefill(torch.zeros(B, 4, dtype=torch.int32, device="cuda"), [4] * B)
+    th = rig.eng.tree(synth.random_parent_tree(n, 4, tree_id=3, n_heads=4, kmax=1) if n > 1 else synth.single_node_tree())
+    before = rig.eng.launch_count()
+    rig.eng.verify(th, torch.zeros(B, n, dtype=torch.int32, device="cuda"))
+    buf = C.create_string_buffer(1 << 14)
+    assert cb.lib().cerb_launch_order_table(variant, buf, len(buf)) == cb.OK
+    assert rig.eng.launch_count() - before == len(buf.value.decode().strip().split("\n"))
