@@ -323,7 +323,9 @@ int forward_rows(cerb_ctx* c, const cerb_tree* tree, const int32_t* tok, int tok
   const bool fuse_res = wide;
   // Very few rows: the gate-up and QKV GEMMs normalise their rows themselves (the first layer's QKV GEMM excepted).
   const bool fuse_norm = fuse_swiglu && fuse_rope && M <= kFewRows && gemm_few_normalises(M, d);
-  OrderCheck oc(launch_order_variant({fuse_swiglu, fuse_rope, fuse_res, fuse_norm}));
+  const int variant = launch_order_variant({fuse_swiglu, fuse_rope, fuse_res, fuse_norm});
+  if (variant < 0) return CERB_E_STATE;                     // (a combination that the launch-order table does not describe)
+  OrderCheck oc(variant);
   // embedding gather fused with the first layer's attention norm
   CERB_ORDER(oc, LO_NORM_ATTN);
   { ProfScope ps(c, K_GLUE, st);

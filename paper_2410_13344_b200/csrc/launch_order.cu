@@ -56,22 +56,23 @@ const Entry kArgmax = {LO_ARGMAX, "argmax_rows", 0, 0};
 // SwiGLU in the gate-up GEMM's epilogue: that GEMM writes the activations itself.  RoPE + cache append in the QKV GEMM's.
 const Entry kGuSwiglu = {LO_GEMM_GU, "gemm gate-up + swiglu epilogue", B_PART | B_ACT, B_CONST};
 const Entry kQkvRope = {LO_GEMM_QKV, "gemm qkv + rope / append epilogue", B_PART | B_Q | B_KV, B_CONST};
-// The residual add in the O and down GEMMs' epilogues: the norms then read the residual stream after their wait (the
+// The residual add in the O and down GEMMs' epilogues: the norms then read nothing ahead of their wait (the
 // embedding gather in front of the first layer writes it, as ever).
 const Entry kWoAdd = {LO_GEMM_WO, "gemm wo + residual add epilogue", B_PART | B_X, B_CONST};
 const Entry kDownAdd = {LO_GEMM_DOWN, "gemm down + residual add epilogue", B_PART | B_X, B_CONST};
-const Entry kNormAttnRead = {LO_NORM_ATTN, "fused_norm (attention norm)", B_X | B_XN, B_CONST};
-const Entry kNormMlpRead = {LO_NORM_MLP, "fused_norm (MLP norm)", B_XN, B_CONST};
-const Entry kNormFinalRead = {LO_NORM_FINAL, "fused_norm (final norm)", B_HIDDEN, B_CONST};
+const Entry kNormAttnRead = {LO_NORM_ATTN, "row_norm (embedding; attention norm)", B_X | B_XN, 0};
+const Entry kNormMlpRead = {LO_NORM_MLP, "row_norm (MLP norm)", B_XN, 0};
+const Entry kNormFinalRead = {LO_NORM_FINAL, "row_norm (final norm)", B_HIDDEN, 0};
 
 // The norms in the GEMMs that read them, which then read the residual stream after their wait; the embedding gather with the
 // first attention norm stays, in front of the layers.
-const Entry kNormEmbed = {LO_NORM_ATTN, "fused_norm (embedding, attention norm)", B_X | B_XN, B_CONST};
+const Entry kNormEmbed = {LO_NORM_ATTN, "row_norm (embedding, attention norm)", B_X | B_XN, 0};
 const Entry kQkvNorm = {LO_GEMM_QKV, "gemm norm + qkv + rope / append epilogue", B_Q | B_KV, B_CONST};
 const Entry kGuNorm = {LO_GEMM_GU, "gemm norm + gate-up + swiglu epilogue", B_ACT, B_CONST};
 
 // Variant 0 is the steps of 9 to 128 rows; those with a residual add in the GEMMs occur above and up to 8 rows, the norms in
-// the GEMMs (8) with one or two.
+// the GEMMs (8) with as many of those as gemm_few_normalises allows.  1, 2 and 4 (a fusion without the residual add) are no forward's;
+// their tables stay for callers of the entry below.
 constexpr int kVariants = 9;
 const Fusion kFusion[kVariants] = {  // {swiglu, rope, residual, norm}
     {false, false, false}, {true, false, false}, {true, true, false}, {true, true, true},
@@ -109,7 +110,7 @@ int build(int variant, const Entry** out) {
 int launch_order_variant(Fusion f) {
   for (int v = 0; v < kVariants; ++v)
     if (kFusion[v].swiglu == f.swiglu && kFusion[v].rope == f.rope && kFusion[v].residual == f.residual && kFusion[v].norm == f.norm) return v;
-  return 0;
+  return -1;
 }
 
 int launch_order_layer(int variant, int* ids_out) {

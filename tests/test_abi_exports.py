@@ -154,3 +154,27 @@ def test_no_forward_kernel_leaves_ahead_of_its_wait():
             seen += 1
             assert not re.search(r"\breturn\s*;", body[:w]), (fn, body[:80])
     assert seen >= 12
+
+
+def test_the_read_before_wait_rule_holds_in_every_variant():
+    """The rule of test_no_kernel_reads_before_its_wait_what_the_kernel_in_front_writes over all exported launch sequences, those of
+    the forwards (0, 3, 5, 6, 7, 8) among them."""
+    from paper_2410_13344_b200 import binding
+    # variant: SwiGLU in a GEMM, RoPE in a GEMM, residual add in the GEMMs, norms in the GEMMs
+    fused = {0: (0, 0, 0, 0), 1: (1, 0, 0, 0), 2: (1, 1, 0, 0), 3: (1, 1, 1, 0), 4: (0, 1, 0, 0), 5: (0, 0, 1, 0), 6: (1, 0, 1, 0), 7: (0, 1, 1, 0), 8: (1, 1, 1, 1)}
+    for variant, (swiglu, rope, residual, norm) in fused.items():
+        rc, rows = _launch_table(variant)
+        assert rc == binding.OK
+        names = [r[1] for r in rows]
+        # four GEMMs and the attention; a norm in front of QKV and gate-up, RoPE and SwiGLU, unless a GEMM does it; set-up and tail
+        assert len(rows) == 1 + 3 * (5 + 2 * (not norm) + (not rope) + (not swiglu)) + norm + 3, (variant, names)
+        assert sum("residual add epilogue" in n for n in names) == 6 * residual
+        assert sum(n.startswith("row_norm" if residual else "fused_norm") for n in names) == (2 if norm else 7)
+        for i, (_, name, _, reads) in enumerate(rows):
+            for bit in range(9):
+                writers = [j for j in range(i) if rows[j][2] >> bit & 1]
+                if reads >> bit & 1 and writers:
+                    assert i - writers[-1] >= 2, (variant, name, bit, rows[writers[-1]][1])
+    buf = ctypes.create_string_buffer(1 << 14)
+    for variant in (-1, len(fused)):
+        assert binding.lib().cerb_launch_order_table(variant, buf, len(buf)) == binding.E_ARG
