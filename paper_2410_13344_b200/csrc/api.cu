@@ -345,7 +345,7 @@ int forward_rows(cerb_ctx* c, const cerb_tree* tree, const int32_t* tok, int tok
       // q, k and v leave the GEMM rotated and in place: no separate kernel, no second pass over the partial sums
       const RopeEpilogue re{c->d_len, c->d_nactive, tree->dev.depth, c->page_table, row_off, c->d_rope, c->d_q,
                             (void*)a.k_pool, (void*)a.v_pool, g.max_pages, c->max_pos, n, g.n_heads, B};
-      const GemmEpilogue epi{2, nullptr, c->d_gemm_tickets, &re, nullptr};
+      const GemmEpilogue epi{2, nullptr, &re, nullptr};
       const GemmNorm nm{(const float*)c->d_x, c->attn_norm[l], g.rms_eps};
       CERB_TRY(gemm_fused(c, c->d_xn, &c->tm_xn, c->wqkv[l], &c->tm_wqkv_rot[l], M, 3 * HD, d, epi, st, fuse_norm && l ? &nm : nullptr));
     } else {
@@ -359,7 +359,7 @@ int forward_rows(cerb_ctx* c, const cerb_tree* tree, const int32_t* tok, int tok
       CERB_TRY(launch_tree_attention(c, &a, c->bf16 ? &c->tm_kpool[l] : nullptr, c->bf16 ? &c->tm_vpool[l] : nullptr,
                                      c->sm_count, c->d_status, st, row_off, tree == c->chain)); }
     CERB_ORDER(oc, LO_GEMM_WO);
-    const GemmEpilogue res{3, nullptr, c->d_gemm_tickets, nullptr, (float*)c->d_x};
+    const GemmEpilogue res{3, nullptr, nullptr, (float*)c->d_x};
     if (fuse_res) CERB_TRY(gemm_fused(c, c->d_attn, &c->tm_attn, c->wo[l], &c->tm_wo[l], M, d, HD, res, st));
     else { ProfScope ps(c, K_GEMM, st);
       CERB_TRY(gemm(c, c->d_attn, &c->tm_attn, c->wo[l], c->bf16 ? &c->tm_wo[l] : nullptr, M, d, HD, &ns, st)); }
@@ -368,11 +368,11 @@ int forward_rows(cerb_ctx* c, const cerb_tree* tree, const int32_t* tok, int tok
     if (!fuse_norm) {
       CERB_ORDER(oc, LO_NORM_MLP);
       ProfScope ps(c, K_GLUE, st);
-      CERB_TRY(launch_fused_norm(c, c->d_part, ns, (size_t)M * d, nullptr, 0, 0, n, c->mlp_norm[l], c->d_xn, M, st, nullptr, fuse_res)); }
+      CERB_TRY(launch_fused_norm(c, c->d_part, ns, (size_t)M * d, nullptr, 0, 0, n, c->mlp_norm[l], c->d_xn, M, st)); }
     CERB_ORDER(oc, LO_GEMM_GU);
     if (fuse_swiglu) {
       // SwiGLU runs in the GEMM's epilogue: no separate kernel, no second pass over the partial sums
-      const GemmEpilogue epi{1, c->d_act, c->d_gemm_tickets, nullptr, nullptr};
+      const GemmEpilogue epi{1, c->d_act, nullptr, nullptr};
       const GemmNorm nm{(const float*)c->d_x, c->mlp_norm[l], g.rms_eps};
       CERB_TRY(gemm_fused(c, c->d_xn, &c->tm_xn, c->wgu[l], &c->tm_wgu_pair[l], M, 2 * F, d, epi, st, fuse_norm ? &nm : nullptr));
     } else {
@@ -392,7 +392,7 @@ int forward_rows(cerb_ctx* c, const cerb_tree* tree, const int32_t* tok, int tok
     { ProfScope ps(c, K_GLUE, st);
       const bool last = l + 1 == g.n_layers;
       CERB_TRY(launch_fused_norm(c, c->d_part, ns, (size_t)M * d, nullptr, 0, 0, n, last ? c->final_norm : c->attn_norm[l + 1],
-                                 last ? c->d_hidden : c->d_xn, M, st, nullptr, fuse_res)); }
+                                 last ? c->d_hidden : c->d_xn, M, st)); }
   }
   return CERB_OK;
 }
@@ -863,7 +863,7 @@ int cerb_device_status(cerb_ctx* c, void* stream) {
   int32_t s = 0;
   CERB_CUDA_OK(cudaMemcpy(&s, c->d_status, sizeof(s), cudaMemcpyDeviceToHost));
   if (s != 0) {
-    // a launch that gave up may have left the arrival counters of the GEMM's fused epilogue half-way
+    // a launch that gave up may have left the GEMM's counters half-way
     CERB_CUDA_OK(cudaMemset(c->d_status, 0, 4 * sizeof(int32_t)));
     CERB_CUDA_OK(cudaMemset(c->d_gemm_tickets, 0, kGemmTickets * sizeof(unsigned int)));
   }

@@ -101,14 +101,12 @@ __global__ void __launch_bounds__(kt_threads(NCB), 1) tree_attn_kt_kernel(const 
   const uint32_t q_base = p_base + PB * 2 * P_TERM;                       // [half of head_dim][NQ rows][128 B]
   const uint32_t ring = q_base + 2 * QHALF;                          // NU units
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int split = blockIdx.x, h = blockIdx.y;
-  int b, shift;
-  locate_window(p, (int)blockIdx.z, b, shift);
+  const int split = blockIdx.x, h = blockIdx.y, b = blockIdx.z;
   // Lengths, live node counts, the page table, the tree and the prefix keys are at least two kernels old:
   // everything up to the first use of Q or of this step's tree keys runs before griddep_wait().
-  const int L_old = p.len[b], L = L_old + shift;                      // keys written by earlier launches; keys every row sees
-  const int nq_all = (p.n_active ? min(p.n_active[b], p.n) : p.n) - shift;   // live nodes of this sequence (from the window on)
-  const size_t qrow = (p.row_off ? (size_t)p.row_off[b] : (size_t)b * p.n) + shift;   // its first row of q and out
+  const int L = p.len[b];
+  const int nq_all = p.n_active ? min(p.n_active[b], p.n) : p.n;      // live nodes of this sequence
+  const size_t qrow = p.row_off ? (size_t)p.row_off[b] : (size_t)b * p.n;   // this sequence's first row of q and out
   const int nq = min(nq_all - p.row0, p.rows);                        // live query rows of this launch
   if (nq <= 0) {                                                      // (uniform over a cluster)
     griddep_wait();
@@ -184,7 +182,7 @@ __global__ void __launch_bounds__(kt_threads(NCB), 1) tree_attn_kt_kernel(const 
     asm volatile("bar.sync 3, %0;" ::"r"(32 * NPROD) : "memory");      // the page list is complete
     // units (K and V) of tiles that lie wholly inside the prefix may be fetched before the wait
     int early = 0;
-    while (early < T && 2 * early < NU && (t0 + early + 1) * KT_TILE <= L_old) ++early;
+    while (early < T && 2 * early < NU && (t0 + early + 1) * KT_TILE <= L) ++early;
     const int early_units = min(2 * early, NU);
     static_assert(KT_PAGES == 8, "the lane -> box map below assumes eight pages per tile");
     const int box = pw + NPROD * lane;               // lanes 0 .. BOXES-1

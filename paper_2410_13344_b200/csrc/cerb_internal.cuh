@@ -48,6 +48,18 @@ __device__ __forceinline__ void locate_row(int row, const int32_t* __restrict__ 
 }
 __device__ __forceinline__ void griddep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void griddep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ unsigned long long globaltimer_ns() {
+  unsigned long long t;
+  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+  return t;
+}
+// Warp MMA, 16 x 8 x 16, bf16 operands, fp32 sums.
+__device__ __forceinline__ void mma_16816(float* c, uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1) {
+  asm volatile(
+      "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+      : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+      : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+}
 #endif
 bool pdl_enabled();
 // Budget of every bounded device-side wait, in SM clock cycles (cerb_set_wait_cycles; about 2 s by default).
@@ -158,7 +170,7 @@ struct cerb_ctx {
   float *d_part, *d_logits, *d_hlogits;
   float* d_topk_cv;       // per-chunk top-k candidates of the heads' logits: values [B][Hc][kTopkChunks][MAX_TOPK]
   int32_t* d_topk_ci;     // ... and their token ids
-  unsigned int* d_gemm_tickets;   // kGemmTickets arrival counters of the GEMM's fused epilogue (zero between launches)
+  unsigned int* d_gemm_tickets;   // kGemmTickets counters of the GEMM above 128 rows (zero between launches)
   float* d_gemm_fix;      // partial tiles of the GEMM above 128 rows
   size_t part_floats;
   float* d_hstate[2];
@@ -223,7 +235,7 @@ int launch_order_violations(int variant);
 int launch_rope_table(cerb_ctx* c, cudaStream_t st);
 int launch_fused_norm(cerb_ctx* c, const float* part, int nsplit, size_t split_stride, const int32_t* tok, int tok_stride,
                       int tok_off, int n, const void* gain, void* out, int rows, cudaStream_t st,
-                      const int32_t* row_off = nullptr, bool x_fresh = false);
+                      const int32_t* row_off = nullptr);
 int launch_rope_append(cerb_ctx* c, int layer, const TreeDev& t, const float* part, int nsplit, size_t split_stride,
                        int B, int n, int rows, cudaStream_t st, const int32_t* row_off = nullptr);
 int launch_swiglu(cerb_ctx* c, const float* part, int nsplit, size_t split_stride, void* act, int rows, cudaStream_t st);
@@ -251,7 +263,6 @@ struct RopeEpilogue {
 struct GemmEpilogue {
   int kind;                 // 0 none, 1 SwiGLU, 2 RoPE + cache append, 3 residual add
   void* act;                // kind 1: [M][F] bf16
-  unsigned int* tickets;    // kGemmTickets counters, zero on entry and on exit
   const RopeEpilogue* rope; // kind 2
   float* x;                 // kind 3: [M][N]
 };

@@ -43,19 +43,6 @@ struct FewParams {
   unsigned long long* clk;
 };
 
-__device__ __forceinline__ unsigned long long now_ns() {
-  unsigned long long t;
-  asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
-  return t;
-}
-
-__device__ __forceinline__ void mma_16816(float* c, uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1) {
-  asm volatile(
-      "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
-      : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
-      : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
-}
-
 // KIND as in GemmEpilogue.  A tile's 16 rows are neighbours (0, 3), or eight and the eight that belong to them (1: gate, up; 2:
 // elements i and i + 64 of a head).
 template <int KIND, bool NORM>
@@ -115,7 +102,7 @@ __global__ void __launch_bounds__(WARPS * 32, 2) gemm_few_kernel(const __grid_co
     for (int j = threadIdx.x * 4; j < K; j += WARPS * 32 * 4)
       asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"((uint32_t)__cvta_generic_to_shared(xs + p.M * (K + 32) + j)), "l"(p.gain + j) : "memory");
   griddep_wait();
-  if (p.clk && threadIdx.x == 0) atomicMin(p.clk, now_ns());
+  if (p.clk && threadIdx.x == 0) atomicMin(p.clk, globaltimer_ns());
   griddep_launch();
   if constexpr (NORM) {
     // every CTA normalises the rows for itself, while its first weights are on their way
@@ -224,7 +211,7 @@ __global__ void __launch_bounds__(WARPS * 32, 2) gemm_few_kernel(const __grid_co
       }
     }
   }
-  if (p.clk && threadIdx.x == 0) atomicMax(p.clk + kGemmClockSlots, now_ns());
+  if (p.clk && threadIdx.x == 0) atomicMax(p.clk + kGemmClockSlots, globaltimer_ns());
 }
 
 // Rows whose norm a GEMM computes itself: as many as fit 25 KB of shared memory with the gains, two of 4096 columns.  (One

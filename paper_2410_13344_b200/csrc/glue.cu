@@ -72,32 +72,24 @@ __global__ void __launch_bounds__(NORM_THREADS) fused_norm_kernel(float* __restr
                                                                    const int32_t* __restrict__ tok, int tok_stride, int tok_off,
                                                                    const int32_t* __restrict__ n_active, int n, int V,
                                                                    const T* __restrict__ gain, T* __restrict__ out, int d, float eps,
-                                                                   const int32_t* __restrict__ row_off, int B, int x_fresh) {
+                                                                   const int32_t* __restrict__ row_off, int B) {
   __shared__ float red[32];
   const int row = blockIdx.x;
   float* xr = x + (size_t)row * d;
   // The residual stream was last written by the previous norm (at least two kernels ago) and the gains
   // never change: both are fetched before waiting for the kernel in front (a GEMM, or whatever produced
-  // the token ids), so that after the wait only that kernel's output remains to be read.  (x_fresh: the GEMM in front
-  // has added to the residual stream itself; then it is read after the wait.)
+  // the token ids), so that after the wait only that kernel's output remains to be read.
   float keep[NORM_MAX_ITER][4], gv[NORM_MAX_ITER][4];
 #pragma unroll
   for (int it = 0; it < NORM_MAX_ITER; ++it) {
     const int j = (it * NORM_THREADS + threadIdx.x) * 4;
     if (j < d) {
-      if (!embed && !x_fresh) ld4(xr + j, keep[it]);
+      if (!embed) ld4(xr + j, keep[it]);
       if (out) ld4(gain + j, gv[it]);
     }
   }
   griddep_wait();
   griddep_launch();
-  if (x_fresh) {
-#pragma unroll
-    for (int it = 0; it < NORM_MAX_ITER; ++it) {
-      const int j = (it * NORM_THREADS + threadIdx.x) * 4;
-      if (j < d) ld4(xr + j, keep[it]);
-    }
-  }
   const T* src = nullptr;
   if (embed) {
     int b, v, t = 0;
@@ -148,8 +140,8 @@ __global__ void __launch_bounds__(NORM_THREADS) fused_norm_kernel(float* __restr
   }
 }
 
-// The same for many rows without slots (more than 128 rows: the GEMMs add to the residual stream themselves): memory-bound,
-// eight CTAs of 256 threads to an SM.  (One 1024-thread CTA per SM and row: 33 us for 2048 rows of 4096 where the bytes take 8.)
+// The same without slots (more than 128 rows and up to 8: the GEMMs add to the residual stream themselves, so it is read after the
+// wait).  Many rows are memory-bound: eight CTAs of 256 threads to an SM.  (One 1024-thread CTA per SM and row: 33 us for 2048 rows of 4096 where the bytes take 8.)
 constexpr int ROWS_THREADS = 256;
 template <typename T, int ITER>
 __global__ void __launch_bounds__(ROWS_THREADS) row_norm_kernel(float* __restrict__ x, const T* __restrict__ embed, const int32_t* __restrict__ tok,
@@ -370,7 +362,7 @@ int launch_rope_table(cerb_ctx* c, cudaStream_t st) {
 
 // x <- embedding rows (tok != null) | x + partials (nsplit > 0) | x;  out <- RMSNorm(x) * gain (out may be null).
 int launch_fused_norm(cerb_ctx* c, const float* part, int nsplit, size_t split_stride, const int32_t* tok, int tok_stride,
-                      int tok_off, int n, const void* gain, void* out, int rows, cudaStream_t st, const int32_t* row_off, bool x_fresh) {
+                      int tok_off, int n, const void* gain, void* out, int rows, cudaStream_t st, const int32_t* row_off) {
   const cerb_config& g = c->cfg;
   const int d = g.d_model;
   if (d % 4 || d > NORM_THREADS * NORM_MAX_ITER * 4) return CERB_E_SHAPE;
@@ -386,11 +378,11 @@ int launch_fused_norm(cerb_ctx* c, const float* part, int nsplit, size_t split_s
   } else if (c->bf16)
     launch_pdl(fused_norm_kernel<bf16>, dim3(rows), dim3(NORM_THREADS), 0, st, (float*)c->d_x, part, nsplit, split_stride,
                tok ? (const bf16*)c->embed : (const bf16*)nullptr, tok, tok_stride, tok_off, (const int32_t*)c->d_nactive, n,
-               g.vocab, (const bf16*)gain, (bf16*)out, d, g.rms_eps, row_off, c->B, x_fresh ? 1 : 0);
+               g.vocab, (const bf16*)gain, (bf16*)out, d, g.rms_eps, row_off, c->B);
   else
     launch_pdl(fused_norm_kernel<float>, dim3(rows), dim3(NORM_THREADS), 0, st, (float*)c->d_x, part, nsplit, split_stride,
                tok ? (const float*)c->embed : (const float*)nullptr, tok, tok_stride, tok_off, (const int32_t*)c->d_nactive, n,
-               g.vocab, (const float*)gain, (float*)out, d, g.rms_eps, row_off, c->B, x_fresh ? 1 : 0);
+               g.vocab, (const float*)gain, (float*)out, d, g.rms_eps, row_off, c->B);
   CERB_LAUNCH_CHECK(c);
   return CERB_OK;
 }

@@ -124,13 +124,6 @@ __device__ __forceinline__ void store_terms(bf16* at, size_t stride, float v) {
   at[2 * stride] = __float2bfloat16_rn(r - __bfloat162float(mid));
 }
 
-__device__ __forceinline__ void mma_16816(float* c, uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1) {
-  asm volatile(
-      "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
-      : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
-      : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
-}
-
 // One level (or the FC) of every head of a bf16 model, for the whole batch.  Bound by HBM: the weights once, 2.7 GB per
 // draft of the 7B shape.  The fp32 states enter the tensor cores as three bf16 terms each (24 bits; the products are exact
 // in fp32), so a batch is 3 B MMA columns (all leading terms, then all middle ones, then all last ones) instead of B passes of
