@@ -145,7 +145,9 @@ int cerb_reset(cerb_ctx* ctx, void* stream);
  * Runs the base model over the prompt in chain-shaped chunks (a chain tree is
  * ordinary causal attention), fills the KV cache, sets len, the last hidden state
  * (final-norm output at the last position) and the root token
- * argmax LH(h_last) (Algorithm 1, LH).  Sets the batch size B for later calls. */
+ * argmax LH(h_last) (Algorithm 1, LH).  Sets the batch size B for later calls.
+ * bf16: a prompt may be 16384 tokens long for every key split that its attention gets, 148 / (B * n_heads) of them, one at least
+ * and eight at most; CERB_E_SHAPE, with the caches filled in part, beyond that. */
 int cerb_prefill(cerb_ctx* ctx, const int32_t* tokens_dev, const int32_t* lens_host, int32_t B, int32_t max_len,
                  void* stream);
 
@@ -284,9 +286,9 @@ int cerb_tree_ancestors(const int32_t* parent, int32_t n, uint64_t* anc_out);
 
 /* Stand-alone dense GEMM as the verification forward runs it (Algorithm 1, TL_i / LH):
  * out[M][N] (fp32) = X[M][K] . W[N][K]^T, X and W in `dtype`, fp32 accumulation.
- * bf16 runs on the tcgen05 tensor-core path (weights streamed once, split along K
- * when few weight tiles exist); scratch holds the split-K partial sums,
- * cerb_gemm_scratch_bytes().  K must be a multiple of 8. */
+ * bf16: X and W 16-byte aligned, K a multiple of 8, weights streamed once; up to 8 rows warp MMAs fed from global
+ * memory, up to 128 rows tcgen05 with the split-K partial sums in scratch, above that output tiles on CTA pairs, which use
+ * scratch where pairs add their sums up; cerb_gemm_scratch_bytes() in every case.  fp32: any 4-byte alignment, no scratch. */
 int cerb_gemm_scratch_bytes(int32_t M, int32_t N, int32_t K, size_t* bytes_out);
 /* How the bf16 GEMM of more than 128 rows cuts this problem up (host only, for tests and measurement; the paper has no
  * counterpart): as cerb_gemm runs it (fused = 0, with the scratch that cerb_gemm_scratch_bytes asks for), or inside the

@@ -12,13 +12,13 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("M,N,K", [
-    (256, 74 * 256, 72),      # exactly one whole tile per pair, ragged last k block
-    (129, 74 * 256 + 1, 64),  # one k block; one tile more than pairs: 75 tiles cut along k; 160-row chunk
-    (300, 37 * 256 + 130, 320),   # two chunks of 160, 76 tiles, the last one half empty
-    (2047, 2400, 136),        # eight chunks, 80 tiles
-    (513, 50 * 256, 1000),    # three chunks of 192, 150 tiles: whole tiles after the split ones
-    (1100, 1000, 2048),       # fewer tiles than pairs: partial slots
-    (131, 40, 4096),          # one tile for all pairs
+    (256, 74 * 256, 72),      # every pair has the same number of whole tiles, ragged last k block
+    (129, 74 * 256 + 1, 64),  # one k block; a last weight tile of one row
+    (300, 37 * 256 + 130, 320),   # a last weight tile that is half empty
+    (2047, 2400, 136),        # ragged chunks of rows, ragged last k block
+    (513, 50 * 256, 1000),    # more tiles than two per pair
+    (1100, 1000, 2048),       # fewer tiles than pairs: several pairs per tile
+    (131, 40, 4096),          # one weight tile of 40 rows, sixteen fills
 ])
 def test_gemm_matches_definition(M, N, K):
     X = synth.normal(12, 1, (M, K), 1.0, dtype=torch.bfloat16, device="cuda")
@@ -32,7 +32,8 @@ def test_gemm_matches_definition(M, N, K):
     assert close(out.double().sum(0) / M, orc.linear(X.double().mean(0, keepdim=True).cpu(), W.cpu())[0], 0) < 2e-4
 
 
-# which epilogues run depends on how many tiles the matrices have: (model, prompt lengths)
+# (model, prompt lengths); every epilogue runs above 128 rows: the residual add always, RoPE at head_dim 128, SwiGLU with mlp_dim a
+# multiple of 16, as in all of these
 CASES = {
     "rope, swiglu, residual": (synth.ModelShape(2, 2560, 8, 128, 1168, 512, "bf16"), (1900,)),
     "rope, swiglu, residual, two sequences": (synth.ModelShape(1, 2560, 8, 128, 1168, 512, "bf16"), (1500, 431)),
