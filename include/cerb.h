@@ -345,7 +345,8 @@ int cerb_set_wait_cycles(int64_t cycles);
  * launch, three layers and the tail, into buf (host).  variant 0: separate SwiGLU and RoPE kernels (steps of 9
  * to 128 rows).  With the residual add inside the O and down GEMMs (steps above 128 rows and of up to 8): 3 with SwiGLU inside the
  * gate-up GEMM and RoPE + cache append inside the QKV GEMM, 5 without either, 6 with SwiGLU, 7 with RoPE; 8: variant 3 with
- * the norms inside the QKV and gate-up GEMMs (up to 8 rows, as far as they fit: two of 4096 columns).  1 (SwiGLU alone), 2 (SwiGLU
+ * the norms inside the QKV and gate-up GEMMs (up to 8 rows, as far as they fit: two of 4096 columns).  fp32 models: 8 with up to 256
+ * columns, else 3, while the GEMMs have few output tiles; 0 above.  1 (SwiGLU alone), 2 (SwiGLU
  * and RoPE) and 4 (RoPE alone) describe no forward any more.  Returns CERB_OK when no kernel reads, ahead of its wait, a buffer
  * that the kernel right in front of it writes, CERB_E_STATE otherwise, CERB_E_NOMEM when buf is too small. */
 int cerb_launch_order_table(int32_t variant, char* buf_host, size_t cap);

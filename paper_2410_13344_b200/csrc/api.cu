@@ -263,6 +263,7 @@ int gemm(cerb_ctx* c, const void* X, const ActMaps* xm, const void* W, const CUt
 int gemm_fused(cerb_ctx* c, const void* X, const ActMaps* xm, const void* W, const CUtensorMap* wm, int M, int N, int K,
                const GemmEpilogue& epi, cudaStream_t st, const GemmNorm* norm = nullptr) {
   ProfScope ps(c, K_GEMM, st);
+  if (!c->bf16) return launch_gemm_f32_fused(c, (const float*)X, (const float*)W, M, N, K, epi, norm, st);
   if (M <= kFewRows) return launch_gemm_few(c, X, W, nullptr, M, N, K, st, &epi, norm, gemm_clock_slot(c));
   return launch_gemm_tile(c, wm, xm, make_tile_plan(M, N, K, false), nullptr, c->d_gemm_fix, c->d_gemm_tickets, M, N, c->d_status, st, &epi,
                           gemm_clock_slot(c));
@@ -317,19 +318,21 @@ int forward_rows(cerb_ctx* c, const cerb_tree* tree, const int32_t* tok, int tok
   }
   // Up to 8 rows and above 128, whatever follows a GEMM runs in its epilogue: SwiGLU, (head_dim 128) RoPE + cache append,
   // the residual adds.
-  const bool wide = c->bf16 && (M > 128 || M <= kFewRows);
-  const bool fuse_swiglu = wide && (M <= kFewRows || F % 16 == 0);
-  const bool fuse_rope = wide && g.head_dim == 128;
+  // fp32: the same as long as the GEMMs have few output tiles.
+  const bool small = !c->bf16 && c->f32_aligned && gemm_f32_small(M, 2 * F) && gemm_f32_small(M, 3 * HD) && gemm_f32_small(M, d);
+  const bool wide = small || (c->bf16 && (M > 128 || M <= kFewRows));
+  const bool fuse_swiglu = small || (wide && (M <= kFewRows || F % 16 == 0));
+  const bool fuse_rope = small || (wide && g.head_dim == 128);
   const bool fuse_res = wide;
   // Very few rows: the gate-up and QKV GEMMs normalise their rows themselves (the first layer's QKV GEMM excepted).
-  const bool fuse_norm = fuse_swiglu && fuse_rope && M <= kFewRows && gemm_few_normalises(M, d);
+  const bool fuse_norm = small ? d <= kF32NormMax : fuse_swiglu && fuse_rope && M <= kFewRows && gemm_few_normalises(M, d);
   const int variant = launch_order_variant({fuse_swiglu, fuse_rope, fuse_res, fuse_norm});
   if (variant < 0) return CERB_E_STATE;                     // (a combination that the launch-order table does not describe)
   OrderCheck oc(variant);
   // embedding gather fused with the first layer's attention norm
   CERB_ORDER(oc, LO_NORM_ATTN);
   { ProfScope ps(c, K_GLUE, st);
-    CERB_TRY(launch_fused_norm(c, nullptr, 0, 0, tok, tok_stride, tok_off, n, c->attn_norm[0], c->d_xn, M, st, row_off)); }
+    CERB_TRY(launch_fused_norm(c, nullptr, 0, 0, tok, tok_stride, tok_off, n, c->attn_norm[0], c->d_xn, M, st, row_off, wide)); }
   cerb_attn_args a;
   memset(&a, 0, sizeof(a));
   a.dtype = g.dtype; a.B = B; a.n = n; a.n_heads = g.n_heads; a.head_dim = g.head_dim; a.max_pages = g.max_pages;
@@ -347,7 +350,7 @@ int forward_rows(cerb_ctx* c, const cerb_tree* tree, const int32_t* tok, int tok
                             (void*)a.k_pool, (void*)a.v_pool, g.max_pages, c->max_pos, n, g.n_heads, B};
       const GemmEpilogue epi{2, nullptr, &re, nullptr};
       const GemmNorm nm{(const float*)c->d_x, c->attn_norm[l], g.rms_eps};
-      CERB_TRY(gemm_fused(c, c->d_xn, &c->tm_xn, c->wqkv[l], &c->tm_wqkv_rot[l], M, 3 * HD, d, epi, st, fuse_norm && l ? &nm : nullptr));
+      CERB_TRY(gemm_fused(c, c->d_xn, &c->tm_xn, c->wqkv[l], c->bf16 ? &c->tm_wqkv_rot[l] : nullptr, M, 3 * HD, d, epi, st, fuse_norm && l ? &nm : nullptr));
     } else {
       { ProfScope ps(c, K_GEMM, st);
         CERB_TRY(gemm(c, c->d_xn, &c->tm_xn, c->wqkv[l], c->bf16 ? &c->tm_wqkv[l] : nullptr, M, 3 * HD, d, &ns, st)); }
@@ -360,7 +363,7 @@ int forward_rows(cerb_ctx* c, const cerb_tree* tree, const int32_t* tok, int tok
                                      c->sm_count, c->d_status, st, row_off, tree == c->chain)); }
     CERB_ORDER(oc, LO_GEMM_WO);
     const GemmEpilogue res{3, nullptr, nullptr, (float*)c->d_x};
-    if (fuse_res) CERB_TRY(gemm_fused(c, c->d_attn, &c->tm_attn, c->wo[l], &c->tm_wo[l], M, d, HD, res, st));
+    if (fuse_res) CERB_TRY(gemm_fused(c, c->d_attn, &c->tm_attn, c->wo[l], c->bf16 ? &c->tm_wo[l] : nullptr, M, d, HD, res, st));
     else { ProfScope ps(c, K_GEMM, st);
       CERB_TRY(gemm(c, c->d_attn, &c->tm_attn, c->wo[l], c->bf16 ? &c->tm_wo[l] : nullptr, M, d, HD, &ns, st)); }
     if (fuse_res) ns = 0;
@@ -368,13 +371,13 @@ int forward_rows(cerb_ctx* c, const cerb_tree* tree, const int32_t* tok, int tok
     if (!fuse_norm) {
       CERB_ORDER(oc, LO_NORM_MLP);
       ProfScope ps(c, K_GLUE, st);
-      CERB_TRY(launch_fused_norm(c, c->d_part, ns, (size_t)M * d, nullptr, 0, 0, n, c->mlp_norm[l], c->d_xn, M, st)); }
+      CERB_TRY(launch_fused_norm(c, c->d_part, ns, (size_t)M * d, nullptr, 0, 0, n, c->mlp_norm[l], c->d_xn, M, st, nullptr, wide)); }
     CERB_ORDER(oc, LO_GEMM_GU);
     if (fuse_swiglu) {
       // SwiGLU runs in the GEMM's epilogue: no separate kernel, no second pass over the partial sums
       const GemmEpilogue epi{1, c->d_act, nullptr, nullptr};
       const GemmNorm nm{(const float*)c->d_x, c->mlp_norm[l], g.rms_eps};
-      CERB_TRY(gemm_fused(c, c->d_xn, &c->tm_xn, c->wgu[l], &c->tm_wgu_pair[l], M, 2 * F, d, epi, st, fuse_norm ? &nm : nullptr));
+      CERB_TRY(gemm_fused(c, c->d_xn, &c->tm_xn, c->wgu[l], c->bf16 ? &c->tm_wgu_pair[l] : nullptr, M, 2 * F, d, epi, st, fuse_norm ? &nm : nullptr));
     } else {
       { ProfScope ps(c, K_GEMM, st);
         CERB_TRY(gemm(c, c->d_xn, &c->tm_xn, c->wgu[l], c->bf16 ? &c->tm_wgu[l] : nullptr, M, 2 * F, d, &ns, st)); }
@@ -382,7 +385,7 @@ int forward_rows(cerb_ctx* c, const cerb_tree* tree, const int32_t* tok, int tok
       { ProfScope ps(c, K_GLUE, st); CERB_TRY(launch_swiglu(c, c->d_part, ns, (size_t)M * 2 * F, c->d_act, M, st)); }
     }
     CERB_ORDER(oc, LO_GEMM_DOWN);
-    if (fuse_res) CERB_TRY(gemm_fused(c, c->d_act, &c->tm_act, c->wd[l], &c->tm_wd[l], M, d, F, res, st));
+    if (fuse_res) CERB_TRY(gemm_fused(c, c->d_act, &c->tm_act, c->wd[l], c->bf16 ? &c->tm_wd[l] : nullptr, M, d, F, res, st));
     else { ProfScope ps(c, K_GEMM, st);
       CERB_TRY(gemm(c, c->d_act, &c->tm_act, c->wd[l], c->bf16 ? &c->tm_wd[l] : nullptr, M, d, F, &ns, st)); }
     if (fuse_res) ns = 0;
@@ -392,7 +395,7 @@ int forward_rows(cerb_ctx* c, const cerb_tree* tree, const int32_t* tok, int tok
     { ProfScope ps(c, K_GLUE, st);
       const bool last = l + 1 == g.n_layers;
       CERB_TRY(launch_fused_norm(c, c->d_part, ns, (size_t)M * d, nullptr, 0, 0, n, last ? c->final_norm : c->attn_norm[l + 1],
-                                 last ? c->d_hidden : c->d_xn, M, st)); }
+                                 last ? c->d_hidden : c->d_xn, M, st, nullptr, wide)); }
   }
   return CERB_OK;
 }
@@ -489,6 +492,10 @@ int cerb_load(const cerb_config* cfg, const cerb_weights* w, void* workspace_dev
   c->mlp_norm.assign(w->mlp_norm, w->mlp_norm + L);
   c->wgu.assign(w->wgu, w->wgu + L);
   c->wd.assign(w->wd, w->wd + L);
+  c->f32_aligned = !c->bf16;
+  for (int l = 0; l < L; ++l)
+    for (const void* w_l : {c->attn_norm[l], c->wqkv[l], c->wo[l], c->mlp_norm[l], c->wgu[l], c->wd[l]})
+      if ((uintptr_t)w_l & 15) c->f32_aligned = false;
   if (g.n_cheads > 0) {
     c->head_W.assign(w->head_W, w->head_W + g.n_cheads * g.n_levels);
     c->head_b.assign(w->head_b, w->head_b + g.n_cheads * g.n_levels);

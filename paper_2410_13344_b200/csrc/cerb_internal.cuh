@@ -148,6 +148,7 @@ struct cerb_ctx {
 
   // weights (device pointers, host arrays)
   const void *embed, *final_norm, *lm_head;
+  bool f32_aligned;                   // fp32: every matrix and gain of the layers starts on a 16-byte boundary
   std::vector<const void*> attn_norm, wqkv, wo, mlp_norm, wgu, wd, head_W, head_b, head_fc;
   char *k_pool, *v_pool;
   size_t pool_layer_bytes;
@@ -235,7 +236,7 @@ int launch_order_violations(int variant);
 int launch_rope_table(cerb_ctx* c, cudaStream_t st);
 int launch_fused_norm(cerb_ctx* c, const float* part, int nsplit, size_t split_stride, const int32_t* tok, int tok_stride,
                       int tok_off, int n, const void* gain, void* out, int rows, cudaStream_t st,
-                      const int32_t* row_off = nullptr);
+                      const int32_t* row_off = nullptr, bool complete = false);
 int launch_rope_append(cerb_ctx* c, int layer, const TreeDev& t, const float* part, int nsplit, size_t split_stride,
                        int B, int n, int rows, cudaStream_t st, const int32_t* row_off = nullptr);
 int launch_swiglu(cerb_ctx* c, const float* part, int nsplit, size_t split_stride, void* act, int rows, cudaStream_t st);
@@ -284,6 +285,11 @@ struct GemmNorm {           // the GEMM's X is RMSNorm(x) * gain of the residual
   const void* gain;
   float eps;
 };
+// gemm_f32.cu: fp32, a forward's GEMMs with what stands before and behind them (few output tiles, operands on 16-byte boundaries; norm: K up to 256)
+constexpr int kF32NormMax = 256;
+bool gemm_f32_small(int M, int N);
+int launch_gemm_f32_fused(cerb_ctx* c, const float* X, const float* W, int M, int N, int K, const GemmEpilogue& epi, const GemmNorm* norm,
+                          cudaStream_t st);
 int launch_gemm_few(cerb_ctx* c, const void* X, const void* W, float* out, int M, int N, int K, cudaStream_t st, const GemmEpilogue* epi = nullptr,
                     const GemmNorm* norm = nullptr, unsigned long long* clock_slot = nullptr);
 bool gemm_few_normalises(int M, int K);

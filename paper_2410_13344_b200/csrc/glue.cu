@@ -140,8 +140,7 @@ __global__ void __launch_bounds__(NORM_THREADS) fused_norm_kernel(float* __restr
   }
 }
 
-// The same without slots (more than 128 rows and up to 8: the GEMMs add to the residual stream themselves, so it is read after the
-// wait).  Many rows are memory-bound: eight CTAs of 256 threads to an SM.  (One 1024-thread CTA per SM and row: 33 us for 2048 rows of 4096 where the bytes take 8.)
+// The same without slots (the GEMMs add to the residual stream themselves, so it is read after the wait).  Many rows are memory-bound: eight CTAs of 256 threads to an SM.  (One 1024-thread CTA per SM and row: 33 us for 2048 rows of 4096 where the bytes take 8.)
 constexpr int ROWS_THREADS = 256;
 template <typename T, int ITER>
 __global__ void __launch_bounds__(ROWS_THREADS) row_norm_kernel(float* __restrict__ x, const T* __restrict__ embed, const int32_t* __restrict__ tok,
@@ -361,17 +360,21 @@ int launch_rope_table(cerb_ctx* c, cudaStream_t st) {
 }
 
 // x <- embedding rows (tok != null) | x + partials (nsplit > 0) | x;  out <- RMSNorm(x) * gain (out may be null).
+// complete: the forward's GEMMs add to the residual stream themselves.
 int launch_fused_norm(cerb_ctx* c, const float* part, int nsplit, size_t split_stride, const int32_t* tok, int tok_stride,
-                      int tok_off, int n, const void* gain, void* out, int rows, cudaStream_t st, const int32_t* row_off) {
+                      int tok_off, int n, const void* gain, void* out, int rows, cudaStream_t st, const int32_t* row_off,
+                      bool complete) {
   const cerb_config& g = c->cfg;
   const int d = g.d_model;
   if (d % 4 || d > NORM_THREADS * NORM_MAX_ITER * 4) return CERB_E_SHAPE;
-  if (c->bf16 && nsplit == 0 && (rows > 128 || rows <= kFewRows) && out) {
-    auto wide = [&](auto iter) {
-      launch_pdl(row_norm_kernel<bf16, decltype(iter)::value>, dim3(rows), dim3(ROWS_THREADS), 0, st, (float*)c->d_x,
-                 tok ? (const bf16*)c->embed : (const bf16*)nullptr, tok, tok_stride, tok_off, (const int32_t*)c->d_nactive, n, g.vocab,
-                 (const bf16*)gain, (bf16*)out, d, g.rms_eps, row_off, c->B);
+  if (complete && nsplit == 0 && out) {
+    auto rows_of = [&](auto type, auto iter) {
+      typedef decltype(type) T;
+      launch_pdl(row_norm_kernel<T, decltype(iter)::value>, dim3(rows), dim3(ROWS_THREADS), 0, st, (float*)c->d_x,
+                 tok ? (const T*)c->embed : (const T*)nullptr, tok, tok_stride, tok_off, (const int32_t*)c->d_nactive, n, g.vocab,
+                 (const T*)gain, (T*)out, d, g.rms_eps, row_off, c->B);
     };
+    auto wide = [&](auto iter) { c->bf16 ? rows_of(bf16(), iter) : rows_of(float(), iter); };
     if (d <= 4096) wide(std::integral_constant<int, 4>());
     else if (d <= 8192) wide(std::integral_constant<int, 8>());
     else wide(std::integral_constant<int, 16>());

@@ -47,3 +47,30 @@ def test_gemm_takes_operands_at_any_offset(M, N, K, dx, dw):
 def test_attention_over_listed_ancestors(n, depth, n_active, lens, head_dim):
     for got_o, got_l, O, l in _attention_case(cb, "fp32", 2, n, 2, head_dim, lens, depth, seed_id=170, n_active=n_active):
         assert close(got_o, O, 0) < 1e-5 and close(got_l, l, 0) < 1e-5
+
+
+# Forwards whose GEMMs take the norm, RoPE, SwiGLU and the residual add in: rows and columns that leave a tile part empty, k below, at and
+# above the one round that the norm inside takes, both head sizes, and matrices off the 16-byte boundaries (separate kernels).  Sums of
+# up to 688 terms in fp32, 2^-24 each, through three layers: 1e-5 of states of size one.
+@pytest.mark.parametrize("d,heads,head_dim,mlp,n,off", [(256, 4, 64, 688, 16, 0), (256, 2, 128, 360, 17, 0), (248, 3, 64, 88, 33, 0), (264, 1, 128, 96, 1, 0),
+                                                        (512, 4, 64, 8, 64, 0), (8, 1, 64, 8, 5, 0), (256, 4, 64, 688, 16, 1)])
+def test_forward_with_fused_gemms(d, heads, head_dim, mlp, n, off):
+    ms = synth.ModelShape(3, d, heads, head_dim, mlp, 512, "fp32")
+    model = synth.make_model(ms, device="cuda", std=0.05)
+    cmodel = {k: v.cpu() for k, v in model.items()}
+    if off:
+        model = {k: torch.cat([v.new_zeros(off), v.flatten()])[off:].view(v.shape) if k[0] == "w" else v for k, v in model.items()}
+    eng = cb.Cerberus(ms, model, None, None, [], max_tokens=64, max_batch=2, max_nodes=n)
+    prompts = [[int(t) for t in synth.make_prompt(512, k, seq=300 + k)] for k in (19, 6)]
+    tok = torch.zeros(2, 19, dtype=torch.int32, device="cuda")
+    for b, p in enumerate(prompts):
+        tok[b, :len(p)] = torch.tensor(p, dtype=torch.int32)
+    eng.prefill(tok, [19, 6])
+    tree = synth.random_parent_tree(n, 4, tree_id=9) if n > 1 else synth.single_node_tree()
+    tt = torch.stack([synth.make_prompt(512, n, seq=310 + b).to(torch.int32) for b in range(2)]).cuda().contiguous()
+    hidden = eng.verify(eng.tree(tree), tt, want_hidden=True)[2]
+    sh = orc.Shape(3, d, heads, head_dim, mlp, 512, "fp32")
+    for b, p in enumerate(prompts):
+        st = orc.prefill(cmodel, sh, p, 64 + n)
+        want, _ = orc.verify_tree(cmodel, sh, st, [int(t) for t in tt[b]], tree.parent)
+        assert close(hidden[b], want, 0) < 1e-5, b
