@@ -43,9 +43,18 @@ __global__ void __launch_bounds__(256) gate_kernel(const T* __restrict__ h_last,
     z += e;
     a += e * t;
   }
-  z = block_reduce(z, red, false);
-  a = block_reduce(a, red, false);
+  // (both sums in one go; the order of each is that of block_reduce)
+  for (int o = 16; o > 0; o >>= 1) {
+    z += __shfl_xor_sync(0xffffffffu, z, o);
+    a += __shfl_xor_sync(0xffffffffu, a, o);
+  }
+  __shared__ float2 both[32];
+  if ((threadIdx.x & 31) == 0) both[threadIdx.x >> 5] = make_float2(z, a);
+  __syncthreads();
   if (threadIdx.x == 0) {
+    z = both[0].x;
+    a = both[0].y;
+    for (int i = 1; i < (int)blockDim.x >> 5; ++i) { z += both[i].x; a += both[i].y; }
     float s = (logf(z) - a / z) * 1.4426950408889634f;
     int md = s > thr ? CERB_MODE_AR : CERB_MODE_PAR;
     S[blockIdx.x] = s;
@@ -78,14 +87,22 @@ __global__ void __launch_bounds__(CERB_MAX_NODES) accept_kernel(const int32_t* _
   __shared__ uint32_t mword[NWARP];
   __shared__ int skey[NWARP];
   __shared__ int best_s;
+  __shared__ int tok_s[CERB_MAX_NODES], am_s[CERB_MAX_NODES];
+  const int b = blockIdx.x, v = threadIdx.x;
+  // ahead of the wait: the tree.  The lengths are not: of two calls for trees of one node the second follows the kernel that writes them.
+  const size_t row0 = row_off ? (size_t)row_off[b] : (size_t)b * n;      // this sequence's first row of argmax / hidden
+  const int at = v < n ? v : 0;
+  const int up = at ? parent[at] : 0, level = depth[at];
+  uint64_t see[CERB_ANC_WORDS];
+#pragma unroll
+  for (int w = 0; w < CERB_ANC_WORDS; ++w) see[w] = anc[at * CERB_ANC_WORDS + w];
   griddep_wait();
   griddep_launch();
-  const int b = blockIdx.x, v = threadIdx.x;
-  const int na = min(n_active[b], n);
-  const int32_t* tk = tok + (size_t)b * n;
-  const size_t row0 = row_off ? (size_t)row_off[b] : (size_t)b * n;      // this sequence's first row of argmax / hidden
-  const int32_t* am = argmax + row0;
-  bool match = v < na && (v == 0 || tk[v] == am[parent[v]]);
+  // (all of these on their way together; the rows of nodes that are not live lie inside the buffers)
+  const int na = min(n_active[b], n), mine = tok[(size_t)b * n + at], above = argmax[row0 + up], own = argmax[row0 + at], L = len[b];
+  tok_s[v] = mine;
+  am_s[v] = own;
+  bool match = v < na && (v == 0 || mine == above);
   uint32_t bal = __ballot_sync(0xffffffffu, match);
   if ((v & 31) == 0) mword[v >> 5] = bal;
   __syncthreads();
@@ -96,33 +113,33 @@ __global__ void __launch_bounds__(CERB_MAX_NODES) accept_kernel(const int32_t* _
   if (v < na) {
     bool reach = true;
 #pragma unroll
-    for (int w = 0; w < CERB_ANC_WORDS; ++w) reach = reach && (anc[v * CERB_ANC_WORDS + w] & ~mm[w]) == 0;
-    if (reach) key = depth[v] * 256 + (255 - v);
+    for (int w = 0; w < CERB_ANC_WORDS; ++w) reach = reach && (see[w] & ~mm[w]) == 0;
+    if (reach) key = level * 256 + (255 - v);
   }
   for (int o = 16; o > 0; o >>= 1) key = max(key, __shfl_xor_sync(0xffffffffu, key, o));
   if ((v & 31) == 0) skey[v >> 5] = key;
   __syncthreads();
-  if (v == 0) {
-    int k = skey[0];
+  int k = skey[0];
 #pragma unroll
-    for (int w = 1; w < NWARP; ++w) k = max(k, skey[w]);
-    int best = k < 0 ? 0 : 255 - (k & 255);
+  for (int w = 1; w < NWARP; ++w) k = max(k, skey[w]);
+  const int best = k < 0 ? 0 : 255 - (k & 255);
+  if (v == best) {
     best_s = best;
     int cnt = 0;
+#pragma unroll
     for (int w = 0; w < CERB_ANC_WORDS; ++w) {
-      uint64_t bits = anc[best * CERB_ANC_WORDS + w];
+      uint64_t bits = see[w];
       while (bits && cnt < kPathMax) {
         int j = __ffsll((long long)bits) - 1;
         bits &= bits - 1;
         path[(size_t)b * kPathMax + cnt] = w * 64 + j;
-        out_tok[(size_t)b * kPathMax + cnt] = tk[w * 64 + j];
+        out_tok[(size_t)b * kPathMax + cnt] = tok_s[w * 64 + j];
         ++cnt;
       }
     }
     for (int j = cnt; j < kPathMax; ++j) { path[(size_t)b * kPathMax + j] = -1; out_tok[(size_t)b * kPathMax + j] = -1; }
     n_accept[b] = cnt;
-    root[b] = am[best];
-    int L = len[b];
+    root[b] = am_s[best];
     len_old[b] = L;
     len[b] = L + cnt;
   }

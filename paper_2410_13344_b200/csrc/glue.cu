@@ -305,10 +305,15 @@ __global__ void argmax_rows_kernel(const float* __restrict__ part, int nsplit, s
   int w = threadIdx.x >> 5, l = threadIdx.x & 31, nw = blockDim.x >> 5;
   if (l == 0) { sv[w] = best; si[w] = bi; }
   __syncthreads();
-  if (threadIdx.x == 0) {
-    for (int i = 1; i < nw; ++i)
-      if (sv[i] > best || (sv[i] == best && si[i] < bi)) { best = sv[i]; bi = si[i]; }
-    out[blockIdx.x] = (bi == 0x7fffffff) ? 0 : bi;
+  if (w == 0) {
+    best = l < nw ? sv[l] : -INFINITY;
+    bi = l < nw ? si[l] : 0x7fffffff;
+    for (int o = 16; o > 0; o >>= 1) {
+      const float ov = __shfl_xor_sync(0xffffffffu, best, o);
+      const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
+      if (ov > best || (ov == best && oi < bi)) { best = ov; bi = oi; }
+    }
+    if (l == 0) out[blockIdx.x] = (bi == 0x7fffffff) ? 0 : bi;
   }
 }
 

@@ -45,13 +45,28 @@ template <> __device__ __forceinline__ float ldf<bf16>(const bf16* p) { return _
 // fp32 models.
 template <int NB>
 __global__ void __launch_bounds__(WARPS * 32) head_gemv_kernel(const LevelParams P) {
-  extern __shared__ float su[];                       // [NB][w]
-  griddep_wait();
-  griddep_launch();
+  extern __shared__ __align__(16) float su[];         // [NB][w]
   const int head = blockIdx.y;
   const HeadJob J = P.job[head];
   const int w = J.w0 + J.w1;
   const int row_base = blockIdx.x * ROWS_PER_BLOCK;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int r0 = row_base + warp * ROWS_PER_WARP;
+  constexpr int E = 4, AHEAD = 2;
+  const float* Wp = reinterpret_cast<const float*>(J.W);
+  // the weights' first pieces and the bias come while the kernel in front ends (a level of 4 heads of 256: 4.06 -> 2.64 us)
+  float4 wv[AHEAD][ROWS_PER_WARP];
+  auto fetch = [&](float4 (&to)[ROWS_PER_WARP], int k) {
+#pragma unroll
+    for (int i = 0; i < ROWS_PER_WARP; ++i)
+      to[i] = r0 + i < J.rows && k < w ? __ldg(reinterpret_cast<const float4*>(Wp + (size_t)(r0 + i) * w + k)) : make_float4(0.f, 0.f, 0.f, 0.f);
+  };
+#pragma unroll
+  for (int a = 0; a < AHEAD; ++a) fetch(wv[a], (a * 32 + lane) * E);
+  const int my_row = r0 + lane;                       // lanes 0 .. ROWS_PER_WARP - 1 finish a row each
+  const float bias = P.epilogue && lane < ROWS_PER_WARP && my_row < J.rows ? __ldg(reinterpret_cast<const float*>(J.bias) + my_row) : 0.f;
+  griddep_wait();
+  griddep_launch();
   if (row_base >= J.rows) return;
   for (int nb = 0; nb < NB; ++nb) {
     int seq = P.b0 + nb;
@@ -61,54 +76,46 @@ __global__ void __launch_bounds__(WARPS * 32) head_gemv_kernel(const LevelParams
       su[nb * w + k] = seq < P.B ? (k < J.w0 ? own[k] : oth[k - J.w0]) : 0.f;
   }
   __syncthreads();
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int r0 = row_base + warp * ROWS_PER_WARP;
-  constexpr int E = 4;
   float acc[ROWS_PER_WARP][NB];
 #pragma unroll
   for (int i = 0; i < ROWS_PER_WARP; ++i)
 #pragma unroll
     for (int nb = 0; nb < NB; ++nb) acc[i][nb] = 0.f;
-  const float* Wp = reinterpret_cast<const float*>(J.W);
-#pragma unroll 2
-  for (int k = lane * E; k < w; k += 32 * E) {
-    float wv[ROWS_PER_WARP][E];
+  for (int k0 = lane * E; k0 < w; k0 += 32 * E * AHEAD) {
 #pragma unroll
-    for (int i = 0; i < ROWS_PER_WARP; ++i) {
-      int r = r0 + i;
-      const float4 v = r < J.rows ? __ldg(reinterpret_cast<const float4*>(Wp + (size_t)r * w + k)) : make_float4(0.f, 0.f, 0.f, 0.f);
-      wv[i][0] = v.x; wv[i][1] = v.y; wv[i][2] = v.z; wv[i][3] = v.w;
-    }
+    for (int a = 0; a < AHEAD; ++a) {
+      const int k = k0 + a * 32 * E;
+      if (k >= w) break;
 #pragma unroll
-    for (int nb = 0; nb < NB; ++nb) {
-      float x[E];
+      for (int nb = 0; nb < NB; ++nb) {
+        const float4 x = *reinterpret_cast<const float4*>(su + nb * w + k);
 #pragma unroll
-      for (int e = 0; e < E; ++e) x[e] = su[nb * w + k + e];
-#pragma unroll
-      for (int i = 0; i < ROWS_PER_WARP; ++i)
-#pragma unroll
-        for (int e = 0; e < E; ++e) acc[i][nb] = fmaf(wv[i][e], x[e], acc[i][nb]);
+        for (int i = 0; i < ROWS_PER_WARP; ++i) {
+          acc[i][nb] = fmaf(wv[a][i].x, x.x, acc[i][nb]);
+          acc[i][nb] = fmaf(wv[a][i].y, x.y, acc[i][nb]);
+          acc[i][nb] = fmaf(wv[a][i].z, x.z, acc[i][nb]);
+          acc[i][nb] = fmaf(wv[a][i].w, x.w, acc[i][nb]);
+        }
+      }
+      fetch(wv[a], k + 32 * E * AHEAD);
     }
   }
 #pragma unroll
-  for (int i = 0; i < ROWS_PER_WARP; ++i)
+  for (int nb = 0; nb < NB; ++nb) {
+    float mine = 0.f;
 #pragma unroll
-    for (int nb = 0; nb < NB; ++nb)
-      for (int o = 16; o > 0; o >>= 1) acc[i][nb] += __shfl_xor_sync(0xffffffffu, acc[i][nb], o);
-  if (lane == 0) {
     for (int i = 0; i < ROWS_PER_WARP; ++i) {
-      int r = r0 + i;
-      if (r >= J.rows) continue;
-      for (int nb = 0; nb < NB; ++nb) {
-        int seq = P.b0 + nb;
-        if (seq >= P.B) continue;
-        float y = acc[i][nb];
-        if (P.epilogue) {
-          y += reinterpret_cast<const float*>(J.bias)[r] + su[nb * w + r];
-          y = y / (1.0f + expf(-y));
-        }
-        P.out[((size_t)seq * P.Hc + head) * P.out_stride + r] = y;
+      for (int o = 16; o > 0; o >>= 1) acc[i][nb] += __shfl_xor_sync(0xffffffffu, acc[i][nb], o);
+      if (lane == i) mine = acc[i][nb];
+    }
+    const int seq = P.b0 + nb;
+    if (lane < ROWS_PER_WARP && my_row < J.rows && seq < P.B) {
+      float y = mine;
+      if (P.epilogue) {
+        y += bias + su[nb * w + my_row];
+        y = y / (1.0f + expf(-y));
       }
+      P.out[((size_t)seq * P.Hc + head) * P.out_stride + my_row] = y;
     }
   }
 }
@@ -306,11 +313,11 @@ __global__ void __launch_bounds__(TK_WARPS * 32) topk_part_kernel(const float* _
                                                                   int32_t* __restrict__ cand_i) {
   __shared__ float lv[TK_WARPS][CERB_MAX_TOPK];
   __shared__ int li[TK_WARPS][CERB_MAX_TOPK];
-  griddep_wait();
-  griddep_launch();
   const int ch = blockIdx.x, h = blockIdx.y, b = blockIdx.z, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const float* r = logits + ((size_t)b * Hc + h) * V;
   const int k = kper[h];
+  griddep_wait();
+  griddep_launch();
   const int per = (V + kTopkChunks - 1) / kTopkChunks;
   // (what one warp holds at once goes to one warp: its list is the chunk's)
   const bool one = per <= 32 * TK_HELD;
@@ -369,11 +376,20 @@ __global__ void __launch_bounds__(CERB_MAX_HEADS * 32) topk_merge_kernel(const f
                                                                          const int32_t* __restrict__ head_of, const int32_t* __restrict__ rank_of,
                                                                          const int32_t* __restrict__ plant, int n, int32_t* __restrict__ tree_tok) {
   __shared__ int best_s[CERB_MAX_HEADS][CERB_MAX_TOPK];
+  const int b = blockIdx.x, h = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  // (what the tree is filled from beside the candidates is older than the heads' launches)
+  static_assert(CERB_MAX_HEADS * 32 >= CERB_MAX_NODES, "a thread per node");
+  const int v_node = threadIdx.x;
+  int from_head = 0, from_rank = 0, planted = -1, root_tok = 0;
+  if (tree_tok && v_node < n) {
+    if (v_node == 0) root_tok = root[b];
+    else { from_head = head_of[v_node]; from_rank = rank_of[v_node]; }
+    if (plant) planted = plant[(size_t)b * n + v_node];
+  }
+  const int k = h < Hc ? kper[h] : 0;
   griddep_wait();
   griddep_launch();
-  const int b = blockIdx.x, h = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (h < Hc) {
-    const int k = kper[h];
     const size_t base = ((size_t)b * Hc + h) * kTopkChunks * CERB_MAX_TOPK;
     constexpr int N = kTopkChunks * CERB_MAX_TOPK / 32;
     float v[N];
@@ -382,8 +398,10 @@ __global__ void __launch_bounds__(CERB_MAX_HEADS * 32) topk_merge_kernel(const f
     for (int e = 0; e < N; ++e) {
       // candidate (chunk, round) = (t / MAX_TOPK, t % MAX_TOPK)
       const int t = e * 32 + lane;
-      const int c = (t % CERB_MAX_TOPK) < k ? cand_i[base + t] : -1;
-      v[e] = c >= 0 ? cand_v[base + t] : -INFINITY;
+      const bool in = (t % CERB_MAX_TOPK) < k;
+      const int c = in ? cand_i[base + t] : -1;
+      const float val = in ? cand_v[base + t] : 0.f;
+      v[e] = c >= 0 ? val : -INFINITY;
       id[e] = c >= 0 ? c : 0x7fffffff;
     }
     if (lane < CERB_MAX_TOPK) best_s[h][lane] = -1;
@@ -399,16 +417,8 @@ __global__ void __launch_bounds__(CERB_MAX_HEADS * 32) topk_merge_kernel(const f
     }
   }
   __syncthreads();
-  if (!tree_tok) return;
-  for (int v = threadIdx.x; v < n; v += blockDim.x) {
-    int t;
-    if (v == 0) t = root[b];
-    else {
-      t = best_s[head_of[v]][rank_of[v]];
-      if (plant && plant[(size_t)b * n + v] >= 0) t = plant[(size_t)b * n + v];
-    }
-    tree_tok[(size_t)b * n + v] = t;
-  }
+  if (!tree_tok || v_node >= n) return;
+  tree_tok[(size_t)b * n + v_node] = v_node == 0 ? root_tok : planted >= 0 ? planted : best_s[from_head][from_rank];
 }
 
 template <int NT, int MT, int U, int KG, int MB>
