@@ -1485,18 +1485,17 @@ static int launch_attn_window(const cerb_attn_args* a, int row0, int rows, const
     if (per * KT_PAGES > kMaxPagesPerCta) return CERB_E_SHAPE;
     p.nsplit = (tiles + per - 1) / per;
     p.cluster = (use_cluster && p.nsplit >= 2 && p.nsplit <= 8) ? 1 : 0;
-    constexpr int ncb = 2;             // two blocks of 32 queries: the MMAs are 64 queries wide
     static bool kt_configured = false;
     if (!kt_configured) {
-      CERB_CUDA_OK(cudaFuncSetAttribute(tree_attn_kt_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kt_smem(2)));
+      CERB_CUDA_OK(cudaFuncSetAttribute(tree_attn_kt_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)KT_SMEM));
       kt_configured = true;
     }
-    auto kern = tree_attn_kt_kernel<2>;
-    const dim3 grid(p.nsplit, p.H, Bw), block(kt_threads(ncb));
+    auto kern = tree_attn_kt_kernel;
+    const dim3 grid(p.nsplit, p.H, Bw), block(KT_THREADS);
     if (p.cluster)
-      rc = launch_pdl_cluster(kern, grid, block, kt_smem(ncb), st, (unsigned)p.nsplit, *tmK, *tmV, p) == cudaSuccess ? CERB_OK : CERB_E_CUDA;
+      rc = launch_pdl_cluster(kern, grid, block, KT_SMEM, st, (unsigned)p.nsplit, *tmK, *tmV, p) == cudaSuccess ? CERB_OK : CERB_E_CUDA;
     else
-      rc = launch_pdl(kern, grid, block, kt_smem(ncb), st, *tmK, *tmV, p) == cudaSuccess ? CERB_OK : CERB_E_CUDA;
+      rc = launch_pdl(kern, grid, block, KT_SMEM, st, *tmK, *tmV, p) == cudaSuccess ? CERB_OK : CERB_E_CUDA;
   } else if (tensor_path) {
     static bool configured = false;
     if (!configured) {

@@ -5,10 +5,11 @@
 //   S^T[128 keys x N queries]   = K_tile[128 x 128] . Q^T          (A = K tile as TMA delivers it, B = Q)
 //   O^T[128 dh   x N queries]  += V_tile^T[128 dh x 128 keys] . P^T (A = V tile, read M-major; B = P^T in shared memory)
 //
-// with N = 64 (trees of up to 64 nodes) or 128 query columns.  Every one of the 128 accumulator lanes is a key
+// with N = 64 query columns (trees of up to 64 nodes).  Every one of the 128 accumulator lanes is a key
 // (for S^T) or a head-dim element (for O^T), so no tensor-core row is wasted on a narrow tree, a tile is 128
 // keys (half as many MMAs, barriers and tensor-memory round trips per key as with 64-key tiles), and the
-// element-wise work of a tile is spread over 128 x N/32 threads: thread (key lane, block of 32 queries).
+// element-wise work of a tile is spread over 128 x 4 threads: thread (key lane, block of 16 queries).  (That work is a chain of latencies;
+// with blocks of 32 queries, two softmax warps per scheduler, a tile took 2200 cycles whatever the memory did.)
 //
 // Softmax.  Thread = key means a row maximum would be a reduction across threads, so none is taken per tile:
 // every query keeps a reference exponent m[q] in shared memory and p = 2^(s - m[q]) is used as long as no
@@ -23,7 +24,7 @@
 // O^T_hi | O^T_lo in neighbouring accumulator columns, added when the accumulator is read out: the second term
 // costs no extra instruction issue (issuing, not multiplying, is what limits MMAs this small).
 //
-// Roles: warps 0 .. 4 N/32 - 1 = softmax (warp & 3 = lane quarter, warp / 4 = query block); then the TMA producer
+// Roles: warps 0 .. 15 = softmax (warp & 3 = lane quarter, warp / 4 = query block); then the TMA producer
 // warps (one ring of 32 KB units, K and V tiles alternating; a K unit is free again as soon as its QK^T MMAs
 // have retired, a V unit after its PV MMAs); then the tensor-memory allocator and QK^T issuer; then the PV
 // issuer.  A tile of one head arrives as 32 boxes of 2 KB (a 16-token page is 16 rows of two 128-byte swizzle
@@ -31,8 +32,10 @@
 // 16 lanes of one warp takes 1400 cycles, which alone would cap an SM at 64 KB per 2800 cycles), so several
 // warps issue the boxes of a unit side by side.
 // S^T is double-buffered in tensor memory so that QK^T of the next tile runs during the softmax of this one.
-// Split-KV, the cluster merge through distributed shared memory, bounded waits and the pre-wait set-up are the
-// same as in the other bf16 kernels of this file.
+// Split-KV, bounded waits and the pre-wait set-up are the same as in the other bf16 kernels of this file; the members of a cluster send
+// each other their rows instead of reading them.  Producers per kind of unit, 16-query blocks and the sent rows together: verify step of
+// 64 nodes behind 2048 keys 3622 -> 3560 us (32 layers), of 8 x 32 nodes behind 2000 keys 6913 -> 6850; alone, 64 nodes behind 1024 keys,
+// no change (13.9 us: set-up, first round trip, exit).  A fifth ring slot in place of the second P^T buffer: 3570.
 #pragma once
 
 namespace {
@@ -48,15 +51,14 @@ constexpr int KT_DH = 128, KT_ROWF = KT_DH + 4;
 constexpr float KT_RAISE = 30.0f;
 constexpr float KT_UNSET = -1.0e30f;               // reference of a query that has seen no key yet: any real score exceeds it
 
-__host__ __device__ constexpr int kt_nq(int ncb) { return ncb <= 2 ? 64 : 128; }           // query columns of the MMAs
-__host__ __device__ constexpr int kt_units(int ncb) { return ncb <= 2 ? 4 : 3; }           // ring depth in 32 KB units
-__host__ __device__ constexpr int kt_pbufs(int ncb) { return ncb <= 2 ? 2 : 1; }           // P^T buffers
-__host__ __device__ constexpr int kt_producers(int ncb) { return ncb <= 2 ? 4 : 2; }      // TMA-issuing warps
-__host__ __device__ constexpr int kt_threads(int ncb) { return 128 * ncb + 32 * (kt_producers(ncb) + 2); }
-__host__ __device__ constexpr size_t kt_smem(int ncb) {
-  // P^T (hi | lo), Q, ring, alignment slack
-  return (size_t)kt_pbufs(ncb) * 2 * kt_nq(ncb) * 256 + (size_t)kt_nq(ncb) * 256 + (size_t)kt_units(ncb) * KT_UNIT + 1024;
-}
+constexpr int KT_NQ = 64;                          // query columns of the MMAs
+constexpr int KT_QB = 16;                          // queries per softmax thread (a query block)
+constexpr int KT_NU = 4;                           // ring depth in 32 KB units
+constexpr int KT_PB = 2;                           // P^T buffers
+constexpr int KT_PRODUCERS = 4;                    // TMA-issuing warps
+constexpr int KT_THREADS = 128 * (KT_NQ / KT_QB) + 32 * (KT_PRODUCERS + 2);
+// P^T (hi | lo), Q, ring, alignment slack
+constexpr size_t KT_SMEM = (size_t)KT_PB * 2 * KT_NQ * 256 + (size_t)KT_NQ * 256 + (size_t)KT_NU * KT_UNIT + 1024;
 
 // Order-preserving map float -> int (for integer atomicMax on floats) and back.
 __device__ __forceinline__ int f2ord(float f) {
@@ -65,24 +67,23 @@ __device__ __forceinline__ int f2ord(float f) {
 }
 __device__ __forceinline__ float ord2f(int i) { return __int_as_float(i >= 0 ? i : i ^ 0x7fffffff); }
 
-template <int NCB>
-__global__ void __launch_bounds__(kt_threads(NCB), 1) tree_attn_kt_kernel(const __grid_constant__ CUtensorMap tmK,
-                                                                          const __grid_constant__ CUtensorMap tmV,
-                                                                          const AttnParams p) {
+__global__ void __launch_bounds__(KT_THREADS, 1) tree_attn_kt_kernel(const __grid_constant__ CUtensorMap tmK,
+                                                                     const __grid_constant__ CUtensorMap tmV,
+                                                                     const AttnParams p) {
   constexpr int DH = KT_DH, ROWF = KT_ROWF;
-  constexpr int NQ = kt_nq(NCB);                   // query columns of S^T; O^T has 2 * NQ (hi | lo)
-  constexpr int NU = kt_units(NCB);
-  constexpr int PB = kt_pbufs(NCB);                // P^T buffers: with two, the stores of tile t need not wait for PV of tile t - 1
+  constexpr int NQ = KT_NQ, QB = KT_QB, NCB = NQ / QB;     // O^T has 2 * NQ columns (hi | lo)
+  constexpr int NU = KT_NU;
+  constexpr int PB = KT_PB;                        // with two, the stores of tile t need not wait for PV of tile t - 1
   constexpr int NSW = 4 * NCB;                     // softmax warps
-  constexpr int NPROD = kt_producers(NCB);         // producer warps NSW .. NSW + NPROD - 1; then QK^T issuer, PV issuer
+  constexpr int NPROD = KT_PRODUCERS;              // producer warps NSW .. NSW + NPROD - 1; then QK^T issuer, PV issuer
   constexpr int W_QK = NSW + NPROD, W_PV = W_QK + 1;
   constexpr uint32_t QHALF = (uint32_t)NQ * 128u;
-  constexpr uint32_t P_TERM = (uint32_t)(NQ / 64) * KT_HALF;        // bytes of one term (hi or lo) of P^T
-  constexpr uint32_t TMEM_COLS = NQ == 64 ? 256u : 512u;           // S^T x 2 buffers, then O^T hi | lo
+  constexpr uint32_t P_TERM = KT_HALF;                              // bytes of one term (hi or lo) of P^T
+  constexpr uint32_t TMEM_COLS = 4u * NQ;                          // S^T x 2 buffers, then O^T hi | lo
   constexpr uint32_t O_COL = 2u * NQ;
   extern __shared__ uint8_t smem_raw[];
   __shared__ __align__(8) uint64_t full_u[2][NU], empty_u[NU], s_full[2], s_free[2], p_ready[PB], pv_done[PB], q_ready, drain_bar[2];
-  __shared__ __align__(8) uint64_t cl_bar[2];
+  __shared__ __align__(8) uint64_t cl_bar[2], rx_bar;
   __shared__ int page_list[kMaxPagesPerCta];
   __shared__ uint32_t desc_t[CERB_MAX_NODES][4];   // per tree key: which queries of this launch see it, 32 per word
   __shared__ __align__(16) float m_ref[128];       // reference exponent per query (KT_UNSET until a key is seen)
@@ -119,13 +120,15 @@ __global__ void __launch_bounds__(kt_threads(NCB), 1) tree_attn_kt_kernel(const 
   const int t0 = min(tiles, split * per), t1 = min(tiles, t0 + per);
   const bool too_long = per * KT_PAGES > kMaxPagesPerCta;
   const int T = too_long ? 0 : t1 - t0;
+  // a cluster's members each finish rows_each neighbouring rows; the others' shares of these come into rx
+  const int rows_each = (nq + p.nsplit - 1) / p.nsplit, my_lo = min(nq, split * rows_each), my_hi = min(nq, my_lo + rows_each);
 
   if (threadIdx.x == 0) {
     aborted_s = (*p.status != 0);
     exit_flag_s = 0;
     for (int s = 0; s < NU; ++s) {
-      mbar_init(smem_u32(&full_u[0][s]), NPROD);
-      mbar_init(smem_u32(&full_u[1][s]), NPROD);
+      mbar_init(smem_u32(&full_u[0][s]), NPROD / 2);
+      mbar_init(smem_u32(&full_u[1][s]), NPROD / 2);
       mbar_init(smem_u32(&empty_u[s]), 1);
     }
     for (int g = 0; g < 2; ++g) {
@@ -141,7 +144,9 @@ __global__ void __launch_bounds__(kt_threads(NCB), 1) tree_attn_kt_kernel(const 
     mbar_init(smem_u32(&drain_bar[1]), 1);
     mbar_init(smem_u32(&cl_bar[0]), (uint32_t)p.nsplit);
     mbar_init(smem_u32(&cl_bar[1]), (uint32_t)p.nsplit);
+    mbar_init(smem_u32(&rx_bar), 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    if (p.cluster) mbar_expect_tx(smem_u32(&rx_bar), (uint32_t)((my_hi - my_lo) * ROWF * 4 * (p.nsplit - 1)));
     if (too_long) atomicExch(p.status, CERB_E_SHAPE);
   }
   // queries that do not exist keep reference 0: their score columns are zero and never ask for a new one
@@ -157,7 +162,9 @@ __global__ void __launch_bounds__(kt_threads(NCB), 1) tree_attn_kt_kernel(const 
   tc_fence_after();
   if (p.cluster) cluster_start_arrive();
   const uint32_t tmem = tmem_slot;                   // columns [0, 2 NQ): S^T buffers 0 / 1; [2 NQ, 4 NQ): O^T hi | lo
-  float* mrg = reinterpret_cast<float*>(smem_gen);   // [NQ][ROWF] over the operand buffers, once the key loop is over
+  float* mrg = reinterpret_cast<float*>(smem_gen);   // [NQ][ROWF] over P^T and Q, once the key loop is over; behind it
+  float* rx = mrg + NQ * ROWF;                       // [member][rows_each][ROWF], up to 8 members
+  static_assert((2 * NQ + 7) * ROWF * 4 <= (int)(PB * 2 * P_TERM + 2 * QHALF), "both fit there");
 
   // Waiting for unit u (K units are even, V units odd) to have landed.  A parity wait only tells "the phase before
   // the current one is complete", so every barrier needs ONE waiter that sees each of its phases in turn.  With
@@ -169,9 +176,13 @@ __global__ void __launch_bounds__(kt_threads(NCB), 1) tree_attn_kt_kernel(const 
   auto wait_unit = [&](int u, int site) { return mbar_wait(smem_u32(&full_u[u & 1][u % NU]), unit_parity(u), wc, site); };
   if (warp >= NSW && warp < NSW + NPROD) {
     // ---------------- TMA producers ----------------
-    // producer w issues boxes w, w + NPROD, ... of every unit (box = page * 2 + half of head_dim), one per lane
-    const int pw = warp - NSW;
-    constexpr int BOXES = 16 / NPROD;                // boxes of a unit per producer warp
+    // One half of the producers fetches K units, the other V units (neighbouring slots of an even ring belong to one kind each): a
+    // K unit's slot is free a softmax and its PV MMAs ahead of the V unit's in front of it, and queued behind that the K unit of
+    // every other tile came 1500 cycles late (2200 and 3800 cycles from tile to tile in turn).  Producer w of its half issues boxes
+    // w, w + NPROD / 2, ... of every unit (box = page * 2 + half of head_dim), one per lane.
+    const int pw = warp - NSW, kind = pw & 1;
+    static_assert(NU % 2 == 0 && NPROD % 2 == 0, "slots and producers of one kind");
+    constexpr int BOXES = 32 / NPROD;                // boxes of a unit per producer warp
     const int32_t* pt = p.page_table + (size_t)b * p.max_pages;
     const int n_pages = T * KT_PAGES;
     if (pw == 0)
@@ -183,37 +194,36 @@ __global__ void __launch_bounds__(kt_threads(NCB), 1) tree_attn_kt_kernel(const 
     // units (K and V) of tiles that lie wholly inside the prefix may be fetched before the wait
     int early = 0;
     while (early < T && 2 * early < NU && (t0 + early + 1) * KT_TILE <= L) ++early;
-    const int early_units = min(2 * early, NU);
     static_assert(KT_PAGES == 8, "the lane -> box map below assumes eight pages per tile");
-    const int box = pw + NPROD * lane;               // lanes 0 .. BOXES-1
+    const int box = (pw >> 1) + (NPROD / 2) * lane;  // lanes 0 .. BOXES-1
     const int pg = box >> 1, hf = box & 1;
     const uint64_t pol = l2_policy(true);            // K/V are read once per step
     int issued = 0;
     // (the abort flag itself is looked at once, for a launch that starts after a time-out: nothing is issued then;
     // later a wait that gives up says so in its return value, which costs the loop nothing)
-    const int u_stop = *aborted ? 0 : 2 * T;
-    for (int u = 0; u < u_stop; ++u) {
-      if (u == early_units) { griddep_wait(); griddep_launch(); }
-      const int slot = u % NU, t = u >> 1;
-      const uint32_t fb = smem_u32(&full_u[u & 1][slot]);
+    const int t_stop = *aborted ? 0 : T;
+    for (int t = 0; t < t_stop; ++t) {
+      if (t == early) { griddep_wait(); griddep_launch(); }
+      const int u = 2 * t + kind, slot = u % NU;
+      const uint32_t fb = smem_u32(&full_u[kind][slot]);
       int stop = 0;
       if (lane == 0) {
         stop = !mbar_wait_polite(smem_u32(&empty_u[slot]), ((uint32_t)(u / NU) & 1u) ^ 1u, wc, 101);
-        if (!stop) mbar_expect_tx(fb, KT_UNIT / NPROD);
+        if (!stop) mbar_expect_tx(fb, KT_UNIT / (NPROD / 2));
       }
       if (__shfl_sync(0xffffffffu, stop, 0)) break;            // this wait ran out (the consumers have stopped): issue nothing more
       if (lane < BOXES) {
         const int row = page_list[t * KT_PAGES + pg];          // out-of-range rows are zero-filled by TMA
         const uint32_t dst = ring + (uint32_t)slot * KT_UNIT + (uint32_t)hf * KT_HALF + (uint32_t)pg * (CERB_PAGE * 128);
-        tma_load_2d_hint(dst, (u & 1) ? &tmV : &tmK, hf * 64, row, fb, pol);
+        tma_load_2d_hint(dst, kind ? &tmV : &tmK, hf * 64, row, fb, pol);
       }
-      issued = u + 1;
+      issued = t + 1;
     }
     if (lane == 0 && *aborted) {
       // give-up path: the copies this warp has issued still land in the CTA's shared memory; see them in (the
       // phase also needs the other producers' shares, hence a limit of its own: 10 ms)
-      for (int u = issued > NU ? issued - NU : 0; u < issued; ++u)
-        mbar_wait_drain(smem_u32(&full_u[u & 1][u % NU]), unit_parity(u), 20000000ll);
+      for (int t = issued > NU / 2 ? issued - NU / 2 : 0; t < issued; ++t)
+        mbar_wait_drain(smem_u32(&full_u[kind][(2 * t + kind) % NU]), unit_parity(2 * t + kind), 20000000ll);
     }
     griddep_wait();      // (a lane that has waited already returns at once)
     griddep_launch();
@@ -280,9 +290,17 @@ __global__ void __launch_bounds__(kt_threads(NCB), 1) tree_attn_kt_kernel(const 
         umma_commit(smem_u32(&drain_bar[1]));
         mbar_wait_drain(smem_u32(&drain_bar[1]), 0, 20000000ll);
       }
+      if (p.cluster) {
+        // Q is staged and every MMA has retired: this CTA's rx may be written.  (Said from here the release costs the softmax warps nothing.)
+        __syncwarp();
+        mbar_wait_warp(smem_u32(&q_ready), 0, wc, 115);
+        if (T > 0) mbar_wait_warp(smem_u32(&pv_done[(T - 1) % PB]), (uint32_t)((T - 1) / PB) & 1u, wc, 111);
+        cluster_start_wait();
+        if (lane < p.nsplit) mbar_arrive_cluster(mapa_u32(smem_u32(&cl_bar[0]), (uint32_t)lane));
+      }
     }
   } else {
-    // ---------------- softmax: thread = (key lane of the tile, block of 32 queries) ----------------
+    // ---------------- softmax: thread = (key lane of the tile, block of QB queries) ----------------
     const int lq = warp & 3, cb = warp >> 2;
     const int r = lq * 32 + lane;                               // key row of the tile = tensor-memory lane
     const int st = (int)threadIdx.x, nst = 128 * NCB;           // index among the softmax threads
@@ -304,6 +322,7 @@ __global__ void __launch_bounds__(kt_threads(NCB), 1) tree_attn_kt_kernel(const 
         }
       }
     }
+    asm volatile("bar.sync 2, %0;" ::"r"(nst) : "memory");      // desc_t is complete
     griddep_wait();
     griddep_launch();
     {
@@ -327,34 +346,33 @@ __global__ void __launch_bounds__(kt_threads(NCB), 1) tree_attn_kt_kernel(const 
       __syncwarp();
       if (lane == 0) mbar_arrive(smem_u32(&q_ready));
     }
-    asm volatile("bar.sync 2, %0;" ::"r"(nst) : "memory");      // desc_t is complete
+    if (p.cluster) cluster_start_wait();                        // (well ahead of the first arrival at another member's barriers)
     // queries of this block that exist
-    const int qn = nq - cb * 32;
-    const uint32_t qmask = qn >= 32 ? 0xffffffffu : qn <= 0 ? 0u : ((1u << qn) - 1u);
-    float* mr = m_ref + cb * 32;
-    int* pend = m_pending + cb * 32;
-    float l_acc[32];
+    const int qn = nq - cb * QB;
+    const uint32_t qmask = qn >= QB ? (1u << QB) - 1u : qn <= 0 ? 0u : ((1u << qn) - 1u);
+    float* mr = m_ref + cb * QB;
+    int* pend = m_pending + cb * QB;
+    float l_acc[QB];
 #pragma unroll
-    for (int j = 0; j < 32; ++j) l_acc[j] = 0.f;
-    uint8_t* prow0 = smem_gen + (p_base - smem_base) + (uint32_t)(cb >> 1) * KT_HALF + (uint32_t)r * 128u;
+    for (int j = 0; j < QB; ++j) l_acc[j] = 0.f;
+    uint8_t* prow0 = smem_gen + (p_base - smem_base) + (uint32_t)r * 128u;
     for (int t = 0; t < T; ++t) {
       const int sb = t & 1;
       mbar_wait(smem_u32(&s_full[sb]), (uint32_t)(t >> 1) & 1u, wc, 107);
       tc_fence_after();
-      float sc[32];
-      const uint32_t s_addr = tmem + lane_base + (uint32_t)sb * NQ + (uint32_t)cb * 32u;
+      float sc[QB];
+      const uint32_t s_addr = tmem + lane_base + (uint32_t)sb * NQ + (uint32_t)(cb * QB);
       tmem_ld16_nowait(s_addr, reinterpret_cast<uint32_t*>(sc));
-      tmem_ld16_nowait(s_addr + 16u, reinterpret_cast<uint32_t*>(sc + 16));
       tmem_ld_wait();
       const int kpos = (t0 + t) * KT_TILE + r;
       const bool masked = (t0 + t + 1) * KT_TILE > L;           // the tile reaches past the prefix (uniform over the CTA)
-      const uint32_t vis = !masked ? 0xffffffffu : kpos < L ? qmask : kpos < kv_total ? (desc_t[kpos - L][cb] & qmask) : 0u;
+      const uint32_t vis = !masked ? 0xffffffffu : kpos < L ? qmask : kpos < kv_total ? ((desc_t[kpos - L][cb * QB / 32] >> (cb * QB % 32)) & qmask) : 0u;
       if (t == 0 && !masked) {
         // First tile, all keys visible: the scores of its first key serve as the reference (any value within the
         // exponent range of the true maximum does; whatever exceeds it by 2^8 later raises it the usual way).
         if (r == 0) {
 #pragma unroll
-          for (int j = 0; j < 32; ++j)
+          for (int j = 0; j < QB; ++j)
             if ((qmask >> j) & 1u) mr[j] = sc[j] * p.scale_log2;
         }
         asm volatile("bar.sync %0, 128;" ::"r"(4 + cb) : "memory");
@@ -363,7 +381,7 @@ __global__ void __launch_bounds__(kt_threads(NCB), 1) tree_attn_kt_kernel(const 
       float tmax = -INFINITY;
       if (!masked) {
 #pragma unroll
-        for (int j4 = 0; j4 < 32; j4 += 4) {
+        for (int j4 = 0; j4 < QB; j4 += 4) {
           const float4 m4 = *reinterpret_cast<const float4*>(mr + j4);
           sc[j4] = fmaf(sc[j4], p.scale_log2, -m4.x);
           sc[j4 + 1] = fmaf(sc[j4 + 1], p.scale_log2, -m4.y);
@@ -373,7 +391,7 @@ __global__ void __launch_bounds__(kt_threads(NCB), 1) tree_attn_kt_kernel(const 
         }
       } else {
 #pragma unroll
-        for (int j = 0; j < 32; ++j) {
+        for (int j = 0; j < QB; ++j) {
           sc[j] = ((vis >> j) & 1u) ? fmaf(sc[j], p.scale_log2, -mr[j]) : -INFINITY;
           tmax = fmaxf(tmax, sc[j]);
         }
@@ -381,18 +399,17 @@ __global__ void __launch_bounds__(kt_threads(NCB), 1) tree_attn_kt_kernel(const 
       if (__any_sync(0xffffffffu, tmax > KT_RAISE)) {
         // Rare: a score of this warp's keys calls for a higher reference.  Report, per query, the largest visible
         // score of these 32 keys (one warp reduction each; lane j then files query j's).
-        uint32_t raw[32];
+        uint32_t raw[QB];
         tmem_ld16_nowait(s_addr, raw);
-        tmem_ld16_nowait(s_addr + 16u, raw + 16);
         tmem_ld_wait();
         int mine = f2ord(-INFINITY);
 #pragma unroll
-        for (int j = 0; j < 32; ++j) {
+        for (int j = 0; j < QB; ++j) {
           const float v = ((vis >> j) & 1u) ? __uint_as_float(raw[j]) * p.scale_log2 : -INFINITY;
           const int red = __reduce_max_sync(0xffffffffu, f2ord(v));
           if (lane == j) mine = red;
         }
-        atomicMax(&pend[lane], mine);
+        if (lane < QB) atomicMax(&pend[lane], mine);
         if (lane == 0) raise_at[t & 1][cb] = t + 1;
       }
       asm volatile("bar.sync %0, 128;" ::"r"(4 + cb) : "memory");     // the four warps of this query block agree
@@ -403,7 +420,7 @@ __global__ void __launch_bounds__(kt_threads(NCB), 1) tree_attn_kt_kernel(const 
         auto alpha_of = [&](int j) { return ex2(mr[j] - fmaxf(mr[j], ord2f(pend[j]))); };
         bool any_change = false;
 #pragma unroll
-        for (int j = 0; j < 32; ++j) {
+        for (int j = 0; j < QB; ++j) {
           const float mo = mr[j], mn = fmaxf(mo, ord2f(pend[j]));
           if (mn != mo) {
             any_change = true;
@@ -416,28 +433,27 @@ __global__ void __launch_bounds__(kt_threads(NCB), 1) tree_attn_kt_kernel(const 
           waited_pv = true;
           // rows of O^T = head-dim lanes of this warp's quarter; columns of this query block, both terms
 #pragma unroll 1
-          for (int c0 = 0; c0 < 4; ++c0) {
-            const uint32_t o_addr = tmem + lane_base + O_COL + (uint32_t)(c0 >> 1) * NQ + (uint32_t)cb * 32u + (uint32_t)(c0 & 1) * 16u;
-            uint32_t o[16];
+          for (int term = 0; term < 2; ++term) {
+            const uint32_t o_addr = tmem + lane_base + O_COL + (uint32_t)term * NQ + (uint32_t)(cb * QB);
+            uint32_t o[QB];
             tmem_ld16_nowait(o_addr, o);
             tmem_ld_wait();
 #pragma unroll
-            for (int j = 0; j < 16; ++j) o[j] = __float_as_uint(__uint_as_float(o[j]) * alpha_of((c0 & 1) * 16 + j));
+            for (int j = 0; j < QB; ++j) o[j] = __float_as_uint(__uint_as_float(o[j]) * alpha_of(j));
             tmem_st16(o_addr, o);
           }
           tmem_st_wait();
         }
         {
-          uint32_t raw[32];
+          uint32_t raw[QB];
           tmem_ld16_nowait(s_addr, raw);
-          tmem_ld16_nowait(s_addr + 16u, raw + 16);
-          tmem_ld_wait();
+            tmem_ld_wait();
 #pragma unroll
-          for (int j = 0; j < 32; ++j)
+          for (int j = 0; j < QB; ++j)
             sc[j] = ((vis >> j) & 1u) ? fmaf(__uint_as_float(raw[j]), p.scale_log2, -fmaxf(mr[j], ord2f(pend[j]))) : -INFINITY;
         }
         asm volatile("bar.sync %0, 128;" ::"r"(4 + cb) : "memory");   // everyone has read the old reference
-        if (lq == 0) mr[lane] = fmaxf(mr[lane], ord2f(pend[lane]));
+        if (lq == 0 && lane < QB) mr[lane] = fmaxf(mr[lane], ord2f(pend[lane]));
         asm volatile("bar.sync %0, 128;" ::"r"(4 + cb) : "memory");   // the new reference is in place
       }
       tc_fence_before();
@@ -445,9 +461,9 @@ __global__ void __launch_bounds__(kt_threads(NCB), 1) tree_attn_kt_kernel(const 
       if (lane == 0) mbar_arrive(smem_u32(&s_free[sb]));        // S^T is no longer needed: its buffer may be overwritten
       // probabilities, running sums, and the two bf16 terms p = hi + lo: hi is p cut to its upper 16 bits, lo the
       // (exact) remainder cut the same way -- integer operations only, the conversion unit stays free for exp2
-      uint32_t hi[16], lo[16];
+      uint32_t hi[QB / 2], lo[QB / 2];
 #pragma unroll
-      for (int j = 0; j < 32; j += 2) {
+      for (int j = 0; j < QB; j += 2) {
         const float p0 = ex2(sc[j]), p1 = ex2(sc[j + 1]);
         l_acc[j] += p0;
         l_acc[j + 1] += p1;
@@ -470,10 +486,10 @@ __global__ void __launch_bounds__(kt_threads(NCB), 1) tree_attn_kt_kernel(const 
 #pragma unroll
         for (int c = 0; c < 16; ++c) *reinterpret_cast<uint4*>(vrow + (size_t)(c >> 3) * KT_HALF + (c & 7) * 16) = make_uint4(0, 0, 0, 0);
       }
-      // P^T row of this key: 32 queries = four 16-byte pieces per term
+      // P^T row of this key: 16 queries = two 16-byte pieces per term
 #pragma unroll
-      for (int c = 0; c < 4; ++c) {
-        const uint32_t off = (uint32_t)((((cb & 1) * 4 + c) ^ (r & 7)) << 4);
+      for (int c = 0; c < QB / 8; ++c) {
+        const uint32_t off = (uint32_t)(((cb * (QB / 8) + c) ^ (r & 7)) << 4);
         *reinterpret_cast<uint4*>(prow + off) = make_uint4(hi[4 * c], hi[4 * c + 1], hi[4 * c + 2], hi[4 * c + 3]);
         *reinterpret_cast<uint4*>(prow + P_TERM + off) = make_uint4(lo[4 * c], lo[4 * c + 1], lo[4 * c + 2], lo[4 * c + 3]);
       }
@@ -483,14 +499,12 @@ __global__ void __launch_bounds__(kt_threads(NCB), 1) tree_attn_kt_kernel(const 
       if (lane == 0) mbar_arrive(smem_u32(&p_ready[t % PB]));
     }
     // ---- this CTA's rows (O, m, l) into shared memory ----
-    if (T > 0) {
-      mbar_wait(smem_u32(&pv_done[(T - 1) % PB]), (uint32_t)((T - 1) / PB) & 1u, wc, 111);
-      tc_fence_after();
-    }
-    // row sums: transpose-reduce the 32 partials of a warp (lane q ends up with the sum for query q)
+    // row sums, while the last products run: transpose-reduce the partials of a warp (lanes q and q + 16 end up with the sum for query q)
     {
 #pragma unroll
-      for (int w = 16; w >= 1; w >>= 1) {
+      for (int j = 0; j < QB; ++j) l_acc[j] += __shfl_xor_sync(0xffffffffu, l_acc[j], 16);
+#pragma unroll
+      for (int w = QB / 2; w >= 1; w >>= 1) {
 #pragma unroll
         for (int j = 0; j < w; ++j) {
           const bool upper = (lane & w) != 0;
@@ -500,39 +514,84 @@ __global__ void __launch_bounds__(kt_threads(NCB), 1) tree_attn_kt_kernel(const 
         }
       }
       // lane's bit pattern now selects the query: bit w of the lane chose the upper half at step w
-      l_part[lq][cb * 32 + lane] = l_acc[0];
+      if (lane < QB) l_part[lq][cb * QB + lane] = l_acc[0];
+    }
+    if (T > 0) {
+      mbar_wait(smem_u32(&pv_done[(T - 1) % PB]), (uint32_t)((T - 1) / PB) & 1u, wc, 111);
+      tc_fence_after();
     }
     asm volatile("bar.sync 2, %0;" ::"r"(nst) : "memory");      // every MMA has retired: shared memory can be reused
     {
-      // thread = head-dim element r of this warp's quarter, 32 queries of its block
-      uint32_t oh[32], ol[32];
+      // thread = head-dim element r of this warp's quarter, the queries of its block
+      uint32_t oh[QB], ol[QB];
       if (T > 0) {
-        const uint32_t o_addr = tmem + lane_base + O_COL + (uint32_t)cb * 32u;
+        const uint32_t o_addr = tmem + lane_base + O_COL + (uint32_t)(cb * QB);
         tmem_ld16_nowait(o_addr, oh);
-        tmem_ld16_nowait(o_addr + 16u, oh + 16);
         tmem_ld16_nowait(o_addr + NQ, ol);
-        tmem_ld16_nowait(o_addr + NQ + 16u, ol + 16);
         tmem_ld_wait();
       } else {
 #pragma unroll
-        for (int j = 0; j < 32; ++j) oh[j] = ol[j] = 0u;
+        for (int j = 0; j < QB; ++j) oh[j] = ol[j] = 0u;
       }
 #pragma unroll
-      for (int j = 0; j < 32; ++j) mrg[(size_t)(cb * 32 + j) * ROWF + r] = __uint_as_float(oh[j]) + __uint_as_float(ol[j]);
-      if (lq == 0) {
-        const int q = cb * 32 + lane;
+      for (int j = 0; j < QB; ++j) mrg[(size_t)(cb * QB + j) * ROWF + r] = __uint_as_float(oh[j]) + __uint_as_float(ol[j]);
+      if (lq == 0 && lane < QB) {
+        const int q = cb * QB + lane;
         mrg[(size_t)q * ROWF + DH] = m_ref[q];
         mrg[(size_t)q * ROWF + DH + 1] = (l_part[0][q] + l_part[1][q]) + (l_part[2][q] + l_part[3][q]);
       }
     }
     tc_fence_before();
+    if (p.cluster) proxy_fence();
     asm volatile("bar.sync 2, %0;" ::"r"(nst) : "memory");
 
     // ---- output: final, or partial + fixed-order merge by the last CTA of this (sequence, head) ----
     const int ct = st, nct = nst, RP = p.rows_pad;
     const float LN2 = 0.6931471805599453f;
     if (p.cluster) {
-      // merged after the role branches, where every thread of the cluster meets
+      // The splits of this (sequence, head) are the CTAs of one cluster (rank = split).  Each sends every other member that member's
+      // rows (O, m, l) as one bulk copy and finishes its own from what it has received, in split order.  (Read out of the others'
+      // shared memory by loads instead, the rows took 3900 of the 27500 cycles of a launch of 64 rows over 2048 keys, and another
+      // 1200 went by until everyone had seen that everyone had read.)
+      if (warp == 0) {
+        mbar_wait_cluster(smem_u32(&cl_bar[0]), 0, wc, 112);     // every member's rx may be written
+        proxy_fence();
+        const int lo = min(nq, lane * rows_each), rows = min(nq, lo + rows_each) - lo;
+        if (lane < p.nsplit && lane != split && rows > 0)
+          bulk_to_member(mapa_u32(smem_u32(rx + split * rows_each * ROWF), (uint32_t)lane), smem_u32(mrg + lo * ROWF), (uint32_t)(rows * ROWF * 4),
+                         mapa_u32(smem_u32(&rx_bar), (uint32_t)lane));
+        __syncwarp();
+      }
+      if (!mbar_wait(smem_u32(&rx_bar), 0, wc, 113)) mbar_wait_drain(smem_u32(&rx_bar), 0, 20000000ll);      // (given up: the copies still land here)
+      if (st < p.nsplit) mbar_arrive_cluster(mapa_u32(smem_u32(&cl_bar[1]), (uint32_t)st));        // this CTA has received all it needs
+      // half a warp finishes a row; its lane s2 looks after member s2's weight.  (Short code: what runs once comes from far away.)
+      const int half = lane >> 4, hl = lane & 15;
+      for (int r0 = my_lo + 2 * warp; r0 < my_hi; r0 += 2 * NSW) {
+        const int rr = min(r0 + half, my_hi - 1);
+        auto row_of = [&](int s2) { return s2 == split ? mrg + rr * ROWF : rx + (s2 * rows_each + rr - my_lo) * ROWF; };
+        const float m = hl < p.nsplit ? row_of(hl)[DH] : -INFINITY, lm = hl < p.nsplit ? row_of(hl)[DH + 1] : 0.f;
+        float M = m;
+#pragma unroll
+        for (int o = 4; o > 0; o >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, o));
+        M = __shfl_sync(0xffffffffu, M, 0, 16);
+        const float wm = ex2(m - M);
+        float Lsum = 0.f;
+        float4 a0 = make_float4(0.f, 0.f, 0.f, 0.f), a1 = a0;
+#pragma unroll 2
+        for (int s2 = 0; s2 < p.nsplit; ++s2) {          // split order: the sum does not depend on timing
+          const float* row = row_of(s2) + hl * 4;
+          const float4 v0 = *reinterpret_cast<const float4*>(row), v1 = *reinterpret_cast<const float4*>(row + 64);
+          const float w = __shfl_sync(0xffffffffu, wm, s2, 16);
+          Lsum += __shfl_sync(0xffffffffu, lm, s2, 16) * w;
+          a0.x += v0.x * w; a0.y += v0.y * w; a0.z += v0.z * w; a0.w += v0.w * w;
+          a1.x += v1.x * w; a1.y += v1.y * w; a1.z += v1.z * w; a1.w += v1.w * w;
+        }
+        const float inv = 1.0f / Lsum;
+        bf16* o = p.out + ((qrow + rr) * p.H + h) * DH + hl * 4;
+        *reinterpret_cast<uint2*>(o) = make_uint2(pack_bf16(a0.x * inv, a0.y * inv), pack_bf16(a0.z * inv, a0.w * inv));
+        *reinterpret_cast<uint2*>(o + 64) = make_uint2(pack_bf16(a1.x * inv, a1.y * inv), pack_bf16(a1.z * inv, a1.w * inv));
+        if (hl == 0 && p.lse) p.lse[((size_t)b * p.H + h) * p.n + rr] = (M + log2f(Lsum)) * LN2;
+      }
     } else if (p.nsplit == 1) {
       for (int idx = ct; idx < nq * (DH / 4); idx += nct) {
         const int rr = idx / (DH / 4), c4 = idx % (DH / 4);
@@ -590,53 +649,9 @@ __global__ void __launch_bounds__(kt_threads(NCB), 1) tree_attn_kt_kernel(const 
     }
   }
   if (p.cluster) {
-    // The splits of this (sequence, head) are the CTAs of one cluster (rank = split).  Each holds its rows
-    // (O, m, l) in shared memory; once all have arrived, CTA r finishes rows r, r + nsplit, ...: it reads those
-    // rows from every member in split order, weighs them and writes the final output.  Nobody leaves before
-    // the second meeting, so no shared memory is read after its CTA has gone.
-    cluster_start_wait();
-    if (warp < NSW) {
-      const int ct = (int)threadIdx.x, nwarps = NSW;
-      cluster_meet(&cl_bar[0], p.nsplit, ct, wc, 112);              // every member's rows are in place
-      const float LN2 = 0.6931471805599453f;
-      const uint32_t mine = smem_u32(smem_gen);
-      const int c4 = ct & 31;
-      for (int rr = split + p.nsplit * (ct >> 5); rr < nq; rr += p.nsplit * nwarps) {
-        const uint32_t row_off = (uint32_t)rr * (ROWF * 4);
-        // every member's (m, l) and this thread's four output columns, all loads in flight at once (a cluster
-        // has at most 8 members)
-        float ms[8], ls[8];
-        float4 vs[8];
-#pragma unroll
-        for (int s2 = 0; s2 < 8; ++s2) {
-          if (s2 < p.nsplit) {
-            const uint32_t base = mapa_u32(mine, (uint32_t)s2) + row_off;
-            ms[s2] = ld_cluster_f32(base + DH * 4);
-            ls[s2] = ld_cluster_f32(base + DH * 4 + 4);
-            vs[s2] = ld_cluster_v4(base + (uint32_t)c4 * 16u);
-          } else {
-            ms[s2] = -INFINITY; ls[s2] = 0.f; vs[s2] = make_float4(0.f, 0.f, 0.f, 0.f);
-          }
-        }
-        float M = -INFINITY;
-#pragma unroll
-        for (int s2 = 0; s2 < 8; ++s2) M = fmaxf(M, ms[s2]);
-        float Lsum = 0.f;
-        float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-        for (int s2 = 0; s2 < 8; ++s2) {          // split order: the sum does not depend on timing
-          const float w = ex2(ms[s2] - M);
-          Lsum += ls[s2] * w;
-          acc.x += vs[s2].x * w; acc.y += vs[s2].y * w; acc.z += vs[s2].z * w; acc.w += vs[s2].w * w;
-        }
-        const float inv = 1.0f / Lsum;
-        *reinterpret_cast<uint2*>(p.out + ((qrow + rr) * p.H + h) * DH + c4 * 4) =
-            make_uint2(pack_bf16(acc.x * inv, acc.y * inv), pack_bf16(acc.z * inv, acc.w * inv));
-        if (c4 == 0 && p.lse) p.lse[((size_t)b * p.H + h) * p.n + rr] = (M + log2f(Lsum)) * LN2;
-      }
-      asm volatile("bar.sync 2, %0;" ::"r"(128 * NCB) : "memory");            // this CTA has read all it needs
-      if (warp == 0) cluster_meet_before_exit(&cl_bar[1], p.nsplit, lane, wc, &exit_flag_s, 113);
-    }
+    // Nobody leaves before every member has received its rows: what this CTA has sent leaves from its shared memory until then.
+    if (warp >= NSW && warp != W_PV) cluster_start_wait();
+    else if (warp == 0) cluster_wait_before_exit(&cl_bar[1], wc, &exit_flag_s, 114);
   }
   tc_fence_before();
   __syncthreads();                             // nobody exits before warp 0 has seen every member done

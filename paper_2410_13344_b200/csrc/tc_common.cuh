@@ -313,6 +313,19 @@ __device__ __forceinline__ bool mbar_wait_cluster(uint32_t bar, uint32_t parity,
   wait_ran_out(w, site);
   return false;
 }
+// The waiting half of cluster_meet_before_exit, for members that have arrived earlier.
+__device__ __forceinline__ void cluster_wait_before_exit(uint64_t* bar, const WaitCtx& w, int* flag, int site) {
+  const long long budget = w.budget * 4 > 40000000ll ? w.budget * 4 : 40000000ll;
+  const WaitCtx wx{budget, flag, w.status, w.tag};
+  mbar_wait_cluster((uint32_t)__cvta_generic_to_shared(bar), 0, wx, site);
+}
+// Shared memory of this CTA -> shared memory of a CTA of the cluster (dst and bar: shared::cluster addresses there); its bytes count
+// on `bar`.  Addresses and size are multiples of 16.
+__device__ __forceinline__ void bulk_to_member(uint32_t dst, uint32_t src, uint32_t bytes, uint32_t bar) {
+  asm volatile("cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst), "r"(src), "r"(bytes),
+               "r"(bar)
+               : "memory");
+}
 __device__ __forceinline__ uint32_t mapa_u32(uint32_t saddr, uint32_t rank) {
   uint32_t r;
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(saddr), "r"(rank));
