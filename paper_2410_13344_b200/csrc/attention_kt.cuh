@@ -553,17 +553,22 @@ __global__ void __launch_bounds__(KT_THREADS, 1) tree_attn_kt_kernel(const __gri
       // rows (O, m, l) as one bulk copy and finishes its own from what it has received, in split order.  (Read out of the others'
       // shared memory by loads instead, the rows took 3900 of the 27500 cycles of a launch of 64 rows over 2048 keys, and another
       // 1200 went by until everyone had seen that everyone had read.)
+      //
+      // A copy must neither reach a CTA that has left nor leave from one, whoever has given up.  So a member sends only once all have
+      // said that their rx may be written, says that it has received only once all has landed, and leaves only when all have said
+      // that; if it has given up, it waits for each of these as long as a member that has not may take.
       if (warp == 0) {
-        mbar_wait_cluster(smem_u32(&cl_bar[0]), 0, wc, 112);     // every member's rx may be written
+        const bool ready = __all_sync(0xffffffffu, mbar_wait_cluster(smem_u32(&cl_bar[0]), 0, wc, 112) ||
+                                                       mbar_wait_drain(smem_u32(&cl_bar[0]), 0, partner_cycles(wc)));
         proxy_fence();
         const int lo = min(nq, lane * rows_each), rows = min(nq, lo + rows_each) - lo;
-        if (lane < p.nsplit && lane != split && rows > 0)
+        if (ready && lane < p.nsplit && lane != split && rows > 0)
           bulk_to_member(mapa_u32(smem_u32(rx + split * rows_each * ROWF), (uint32_t)lane), smem_u32(mrg + lo * ROWF), (uint32_t)(rows * ROWF * 4),
                          mapa_u32(smem_u32(&rx_bar), (uint32_t)lane));
         __syncwarp();
       }
-      if (!mbar_wait(smem_u32(&rx_bar), 0, wc, 113)) mbar_wait_drain(smem_u32(&rx_bar), 0, 20000000ll);      // (given up: the copies still land here)
-      if (st < p.nsplit) mbar_arrive_cluster(mapa_u32(smem_u32(&cl_bar[1]), (uint32_t)st));        // this CTA has received all it needs
+      const bool landed = mbar_wait(smem_u32(&rx_bar), 0, wc, 113) || mbar_wait_drain(smem_u32(&rx_bar), 0, partner_cycles(wc));
+      if (landed && st < p.nsplit) mbar_arrive_cluster(mapa_u32(smem_u32(&cl_bar[1]), (uint32_t)st));        // this CTA has received all it needs
       // half a warp finishes a row; its lane s2 looks after member s2's weight.  (Short code: what runs once comes from far away.)
       const int half = lane >> 4, hl = lane & 15;
       for (int r0 = my_lo + 2 * warp; r0 < my_hi; r0 += 2 * NSW) {

@@ -86,12 +86,12 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, const W
 // none of them outlives the CTA's shared and tensor memory.  It keeps a budget of its own (what it waits for
 // was issued and will complete; the limit only guards against the unforeseen) and reports nothing.
 constexpr long long kDrainCycles = 4000000000ll;
-__device__ __forceinline__ void mbar_wait_drain(uint32_t bar, uint32_t parity, long long cycles = kDrainCycles) {
+__device__ __forceinline__ bool mbar_wait_drain(uint32_t bar, uint32_t parity, long long cycles = kDrainCycles) {
   const long long t0 = clock64();
   for (;;) {
     for (int i = 0; i < 256; ++i)
-      if (mbar_try_wait(bar, parity)) return;
-    if (clock64() - t0 > cycles) return;
+      if (mbar_try_wait(bar, parity)) return true;
+    if (clock64() - t0 > cycles) return false;
   }
 }
 // Same bounded wait for a lane whose warp shares an issue port with busy warps: back off between polls.
@@ -282,12 +282,14 @@ __device__ __forceinline__ void cluster_meet(uint64_t* bar, int members, int idx
   }
   wait_ran_out(w, site);
 }
+// How long a CTA that has given up still waits for the other members of its cluster: longer than one of them can take that has
+// not given up (a whole budget, then kAbortedWaitCycles per wait).
+__device__ __forceinline__ long long partner_cycles(const WaitCtx& w) { return w.budget * 4 > 40000000ll ? w.budget * 4 : 40000000ll; }
 // Last rendezvous before a CTA of a cluster leaves: the others may still be reading this CTA's shared memory or about to
 // arrive on its barriers, so this wait keeps a budget of its own, far above that of the other waits (which shrink to
 // microseconds once a wait has run out): a CTA that has given up still waits for its partners here.
 __device__ __forceinline__ void cluster_meet_before_exit(uint64_t* bar, int members, int idx, const WaitCtx& w, int* flag, int site) {
-  const long long budget = w.budget * 4 > 40000000ll ? w.budget * 4 : 40000000ll;
-  const WaitCtx wx{budget, flag, w.status, w.tag};
+  const WaitCtx wx{partner_cycles(w), flag, w.status, w.tag};
   cluster_meet(bar, members, idx, wx, site);
 }
 __device__ __forceinline__ uint32_t cluster_ctarank() {
@@ -315,8 +317,7 @@ __device__ __forceinline__ bool mbar_wait_cluster(uint32_t bar, uint32_t parity,
 }
 // The waiting half of cluster_meet_before_exit, for members that have arrived earlier.
 __device__ __forceinline__ void cluster_wait_before_exit(uint64_t* bar, const WaitCtx& w, int* flag, int site) {
-  const long long budget = w.budget * 4 > 40000000ll ? w.budget * 4 : 40000000ll;
-  const WaitCtx wx{budget, flag, w.status, w.tag};
+  const WaitCtx wx{partner_cycles(w), flag, w.status, w.tag};
   mbar_wait_cluster((uint32_t)__cvta_generic_to_shared(bar), 0, wx, site);
 }
 // Shared memory of this CTA -> shared memory of a CTA of the cluster (dst and bar: shared::cluster addresses there); its bytes count

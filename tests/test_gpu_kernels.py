@@ -278,6 +278,37 @@ def test_attention_after_a_timeout_comes_back_and_the_next_call_is_correct(cb, B
     assert close(out[b], O, 0) < TOL_BF16 and close(lse[b], l, 0) < 2e-3
 
 
+@pytest.mark.parametrize("n,H,lens", [(64, 8, [7232]), (20, 2, [40000, 300]), (33, 16, [2500])])
+def test_clusters_that_give_up_come_back(cb, n, H, lens):
+    """The members of a cluster send each other their rows also when they have given up (here because the status word is set before the
+    launch): members with eight tiles of keys and with one, members without keys or without rows of their own.  The launch comes back
+    with the word still set, and the same call after the word has been cleared matches the oracle."""
+    B, Dh = len(lens), 128
+    max_len = max(lens) + n
+    mp = (max_len + 15) // 16
+    tree = synth.random_parent_tree(n, 5, tree_id=78)
+    q = synth.normal(synth.SEED_ATTN, 811, (B, n, H, Dh), 1.0, dtype=torch.bfloat16, device="cuda")
+    kp, vp = (synth.normal(synth.SEED_ATTN, 812 + i, (B * mp, H, 16, Dh), 1.0, dtype=torch.bfloat16, device="cuda") for i in (0, 1))
+    pt = torch.arange(B * mp, dtype=torch.int32, device="cuda").view(B, mp)
+    anc = torch.from_numpy(cb.tree_ancestors(tree.parent).view(np.int64)).cuda()
+    lens_t = torch.tensor(lens, dtype=torch.int32, device="cuda")
+    scale = 1.0 / math.sqrt(Dh)
+    _, _, scratch = cb.tree_attention(q, kp, vp, pt, lens_t, anc, scale, max_len)
+    status = scratch[4096 - 16:4096].view(torch.int32)
+    status[0] = cb.E_TIMEOUT
+    cb.tree_attention(q, kp, vp, pt, lens_t, anc, scale, max_len, scratch=scratch)
+    torch.cuda.synchronize()
+    assert int(status[0].item()) == cb.E_TIMEOUT
+    status.zero_()
+    out, lse, _ = cb.tree_attention(q, kp, vp, pt, lens_t, anc, scale, max_len, scratch=scratch)
+    torch.cuda.synchronize()
+    assert int(status[0].item()) == 0
+    for b in range(B):
+        kc, vc = (x[b * mp:(b + 1) * mp].cpu().permute(0, 2, 1, 3).reshape(-1, H, Dh).double() for x in (kp, vp))
+        O, l = orc.tree_attention(q[b].cpu().double(), kc[:lens[b]], vc[:lens[b]], kc[lens[b]:lens[b] + n], vc[lens[b]:lens[b] + n], tree.parent, scale)
+        assert close(out[b], O, 0) < TOL_BF16 and close(lse[b], l, 0) < 2e-3
+
+
 def test_abi_rejects_bad_arguments(cb):
     L = cb.lib()
     assert L.cerb_tree_attention(None, None) == cb.E_ARG
