@@ -803,7 +803,7 @@ int cerb_gemm_plan(int32_t M, int32_t N, int32_t K, int32_t fused, int32_t* o) {
 }
 
 // Sums split partials into the output (used only by the stand-alone GEMM entry point).
-__global__ void sum_splits_kernel(const float* __restrict__ part, int nsplit, size_t stride, float* __restrict__ out,
+__global__ void sum_splits_kernel(const float* part, int nsplit, size_t stride, float* __restrict__ out,
                                   size_t total) {
   griddep_wait();
   size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;

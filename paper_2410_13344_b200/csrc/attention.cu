@@ -1246,14 +1246,13 @@ __global__ void __launch_bounds__(ONE_WARPS * 32, 2) tree_attn_one_kernel(const 
 // (2 x 192 nodes x 4 heads behind 16 keys: 9.8 us; 37.0 with fours of neighbouring keys, 18.5 with single ones that skip).
 constexpr int F32_WARPS = 8;
 template <int DH>
-__global__ void __launch_bounds__(F32_WARPS * 32) tree_attn_f32_kernel(const float* __restrict__ q, const float* __restrict__ kpool,
-                                                            const float* __restrict__ vpool,
+__global__ void __launch_bounds__(F32_WARPS * 32) tree_attn_f32_kernel(const float* q, const float* kpool,
+                                                            const float* vpool,
                                                             const int32_t* __restrict__ page_table,
-                                                            const int32_t* __restrict__ len,
-                                                            const int32_t* __restrict__ n_active,
+                                                            const int32_t* len, const int32_t* n_active,
                                                             const uint64_t* __restrict__ anc, float* __restrict__ out,
                                                             float* __restrict__ lse, int n, int H, int max_pages,
-                                                            float scale, const int32_t* __restrict__ row_off, int win) {
+                                                            float scale, const int32_t* row_off, int win) {
   constexpr int E = DH / 32;
   __shared__ float s_o[F32_WARPS][DH];
   __shared__ float s_m[F32_WARPS], s_l[F32_WARPS];

@@ -36,11 +36,14 @@ typedef __nv_bfloat16 bf16;
 // predecessor in the stream is still running; it must execute griddep_wait() before it touches
 // anything the predecessor writes (or anything the predecessor may still be reading and this
 // kernel overwrites).  griddep_launch() lets the next kernel in the stream be scheduled early.
+// What another kernel of the stream writes while this one waits is not const __restrict__ here: the compiler may fetch such data through
+// the read-only path, which the wait does not order.  (Products of a small fp32 model, compiled for three CTAs to an SM, read the
+// residual stream of a layer before.)  Constants (weights, gains, trees, rotations) and what is at least two kernels old may be.
 #ifdef __CUDACC__
 // Which sequence and which node a row of the step's activation buffers belongs to: with ragged rows (sequences that
 // verify a one-node tree next to sequences that verify the whole tree) sequence b starts at row_off[b], otherwise at
 // b * n.
-__device__ __forceinline__ void locate_row(int row, const int32_t* __restrict__ row_off, int B, int n, int& b, int& v) {
+__device__ __forceinline__ void locate_row(int row, const int32_t* row_off, int B, int n, int& b, int& v) {
   if (!row_off) { b = row / n; v = row - b * n; return; }
   b = 0;
   while (b + 1 < B && row_off[b + 1] <= row) ++b;

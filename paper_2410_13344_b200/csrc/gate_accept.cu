@@ -27,9 +27,9 @@ __device__ __forceinline__ float block_reduce(float v, float* red, bool is_max) 
 // With m = max h, Z = sum e^(h-m), A = sum e^(h-m) (h-m):  S = (ln Z - A / Z) / ln 2.
 // mode = S > T ? auto-regressive : parallel (Algorithm 1).
 template <typename T>
-__global__ void __launch_bounds__(256) gate_kernel(const T* __restrict__ h_last, int d, float thr, float* __restrict__ S,
+__global__ void __launch_bounds__(256) gate_kernel(const T* h_last, int d, float thr, float* __restrict__ S,
                                                    int32_t* __restrict__ mode, int32_t* __restrict__ n_active, int n_par,
-                                                   const int32_t* __restrict__ len, int32_t* __restrict__ host) {
+                                                   const int32_t* len, int32_t* __restrict__ host) {
   __shared__ float red[32];
   griddep_wait();
   griddep_launch();
@@ -75,14 +75,13 @@ __global__ void __launch_bounds__(256) gate_kernel(const T* __restrict__ h_last,
 //   v is accepted-reachable iff every node on its root path matches: (anc[v] & ~match) == 0
 //   winner = deepest reachable node, lowest index among equals; its ancestors, ascending, are the path.
 template <typename T>
-__global__ void __launch_bounds__(CERB_MAX_NODES) accept_kernel(const int32_t* __restrict__ tok, const int32_t* __restrict__ argmax,
-                                                     const int32_t* __restrict__ n_active,
+__global__ void __launch_bounds__(CERB_MAX_NODES) accept_kernel(const int32_t* tok, const int32_t* argmax, const int32_t* n_active,
                                                      const int32_t* __restrict__ parent, const int32_t* __restrict__ depth,
-                                                     const uint64_t* __restrict__ anc, int n, int32_t* __restrict__ len,
+                                                     const uint64_t* __restrict__ anc, int n, int32_t* len,
                                                      int32_t* __restrict__ len_old, int32_t* __restrict__ root,
-                                                     const T* __restrict__ hidden, T* __restrict__ h_last, int d,
+                                                     const T* hidden, T* __restrict__ h_last, int d,
                                                      int32_t* __restrict__ n_accept, int32_t* __restrict__ path,
-                                                     int32_t* __restrict__ out_tok, const int32_t* __restrict__ row_off) {
+                                                     int32_t* __restrict__ out_tok, const int32_t* row_off) {
   constexpr int NWARP = CERB_MAX_NODES / 32;
   __shared__ uint32_t mword[NWARP];
   __shared__ int skey[NWARP];
@@ -151,10 +150,9 @@ __global__ void __launch_bounds__(CERB_MAX_NODES) accept_kernel(const int32_t* _
 // Move the accepted nodes' K/V from slot L + path[j] to slot L + j in every layer.  One thread owns
 // one 16-byte column chunk of one (layer, K|V, head) and loads all path rows before storing any:
 // path[j] >= j, so a destination may be a later source.
-__global__ void kv_compact_kernel(char* __restrict__ kpool, char* __restrict__ vpool, size_t layer_bytes,
+__global__ void kv_compact_kernel(char* kpool, char* vpool, size_t layer_bytes,
                                   const int32_t* __restrict__ page_table, int max_pages,
-                                  const int32_t* __restrict__ len_old, const int32_t* __restrict__ n_accept,
-                                  const int32_t* __restrict__ path, int H, int row_bytes) {
+                                  const int32_t* len_old, const int32_t* n_accept, const int32_t* path, int H, int row_bytes) {
   griddep_wait();
   griddep_launch();
   const int b = blockIdx.z, layer = blockIdx.y >> 1;

@@ -7,7 +7,7 @@ namespace cerb {
 constexpr int TM = 64, TN = 64, TK = 16;
 constexpr int kFewTiles = 296;          // 64 x 64 tiles below which the small kernel runs
 
-__global__ void __launch_bounds__(256) gemm_f32_kernel(const float* __restrict__ X, const float* __restrict__ W,
+__global__ void __launch_bounds__(256) gemm_f32_kernel(const float* X, const float* __restrict__ W,
                                                        float* __restrict__ out, int M, int N, int K) {
   __shared__ float sx[TK][TM + 4];
   __shared__ float sw[TK][TN + 4];
@@ -68,8 +68,8 @@ struct F32Fused {
   float eps;
 };
 template <bool VEC, int KIND, bool NORM>
-__global__ void __launch_bounds__(256) gemm_f32_small_kernel(const float* __restrict__ X, const float* __restrict__ W,
-                                                             float* __restrict__ out, int M, int N, int K, const F32Fused f) {
+__global__ void __launch_bounds__(256, KIND == 0 ? 3 : 0) gemm_f32_small_kernel(const float* X, const float* __restrict__ W,
+                                                             float* out, int M, int N, int K, const F32Fused f) {
   constexpr bool PAIRS = KIND == 1 || KIND == 2;
   __shared__ __align__(16) float sx[SM_T][SM_LD], sw[SM_T][SM_LD];
   __shared__ float red[8][SM_T * SM_T];

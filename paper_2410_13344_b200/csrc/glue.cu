@@ -90,12 +90,12 @@ __device__ __forceinline__ void add_slots(float4 (&sum)[COLS], const float* p, c
 constexpr int NORM_THREADS = 1024;
 constexpr int NORM_MAX_ITER = 4;          // d_model up to 16384
 template <typename T, int ITER, int AHEAD, bool EXACT>
-__global__ void __launch_bounds__(NORM_THREADS, 1) fused_norm_kernel(float* __restrict__ x, const float* __restrict__ part, int nsplit,
+__global__ void __launch_bounds__(NORM_THREADS, 1) fused_norm_kernel(float* __restrict__ x, const float* part, int nsplit,
                                                                    size_t split_stride, const T* __restrict__ embed,
-                                                                   const int32_t* __restrict__ tok, int tok_stride, int tok_off,
-                                                                   const int32_t* __restrict__ n_active, int n, int V,
+                                                                   const int32_t* tok, int tok_stride, int tok_off,
+                                                                   const int32_t* n_active, int n, int V,
                                                                    const T* __restrict__ gain, T* __restrict__ out, int d, float eps,
-                                                                   const int32_t* __restrict__ row_off, int B) {
+                                                                   const int32_t* row_off, int B) {
   __shared__ __align__(16) float red[32];
   const int row = blockIdx.x;
   float* xr = x + (size_t)row * d;
@@ -170,10 +170,10 @@ __global__ void __launch_bounds__(NORM_THREADS, 1) fused_norm_kernel(float* __re
 // The same without slots (the GEMMs add to the residual stream themselves, so it is read after the wait).  Many rows are memory-bound: eight CTAs of 256 threads to an SM.  (One 1024-thread CTA per SM and row: 33 us for 2048 rows of 4096 where the bytes take 8.)
 constexpr int ROWS_THREADS = 256;
 template <typename T, int ITER>
-__global__ void __launch_bounds__(ROWS_THREADS) row_norm_kernel(float* __restrict__ x, const T* __restrict__ embed, const int32_t* __restrict__ tok,
-                                                                int tok_stride, int tok_off, const int32_t* __restrict__ n_active, int n, int V,
+__global__ void __launch_bounds__(ROWS_THREADS) row_norm_kernel(float* x, const T* __restrict__ embed, const int32_t* tok,
+                                                                int tok_stride, int tok_off, const int32_t* n_active, int n, int V,
                                                                 const T* __restrict__ gain, T* __restrict__ out, int d, float eps,
-                                                                const int32_t* __restrict__ row_off, int B) {
+                                                                const int32_t* row_off, int B) {
   __shared__ float red[32];
   const int row = blockIdx.x;
   griddep_wait();
@@ -224,7 +224,7 @@ __global__ void __launch_bounds__(ROWS_THREADS) row_norm_kernel(float* __restric
 // q,k rotated at position len + depth; k,v stored at slot len + node of the paged pools; q kept dense.
 // One CTA per (row, head), one thread per rotation pair.
 template <typename T>
-__global__ void rope_append_kernel(const float* __restrict__ part, int nsplit, size_t split_stride,
+__global__ void rope_append_kernel(const float* part, int nsplit, size_t split_stride,
                                    const int32_t* __restrict__ len, const int32_t* __restrict__ n_active,
                                    const int32_t* __restrict__ depth, const int32_t* __restrict__ page_table,
                                    int max_pages, const float2* __restrict__ rope, int max_pos, int n, int H, int Dh,
@@ -278,7 +278,7 @@ __global__ void rope_append_kernel(const float* __restrict__ part, int nsplit, s
 }
 
 template <typename T>
-__global__ void swiglu_kernel(const float* __restrict__ part, int nsplit, size_t split_stride, T* __restrict__ act, int F) {
+__global__ void swiglu_kernel(const float* part, int nsplit, size_t split_stride, T* __restrict__ act, int F) {
   const size_t row = blockIdx.x;
   const int j = (blockIdx.y * blockDim.x + threadIdx.x) * 4;
   griddep_wait();
@@ -298,7 +298,7 @@ __global__ void swiglu_kernel(const float* __restrict__ part, int nsplit, size_t
 // `summed` is not null the summed logits are also written there ([rows][V]).
 // A thread has U groups of four columns in S slots each on their way at once.
 template <int U, int S>
-__global__ void __launch_bounds__(1024) argmax_rows_kernel(const float* __restrict__ part, int nsplit, size_t split_stride, int V,
+__global__ void __launch_bounds__(1024) argmax_rows_kernel(const float* part, int nsplit, size_t split_stride, int V,
                                    int32_t* __restrict__ out, float* __restrict__ summed) {
   __shared__ float sv[32];
   __shared__ int si[32];
@@ -385,9 +385,7 @@ __global__ void set_nactive_kernel(int32_t* n_active, const int32_t* lens_in, in
 
 // After a chain-shaped prefill chunk: everything is accepted in place.
 template <typename T>
-__global__ void prefill_commit_kernel(const int32_t* __restrict__ n_active, int32_t* __restrict__ len,
-                                      const T* __restrict__ hidden, T* __restrict__ h_last,
-                                      const int32_t* __restrict__ row_off, int d) {
+__global__ void prefill_commit_kernel(const int32_t* n_active, int32_t* len, const T* hidden, T* __restrict__ h_last, const int32_t* row_off, int d) {
   griddep_wait();
   griddep_launch();
   int b = blockIdx.x, na = n_active[b];

@@ -260,7 +260,7 @@ __global__ void __launch_bounds__(HM_WARPS * 32, MB) head_mma_kernel(const __gri
 
 // The last hidden states as the heads' first states (bf16 models: and as terms).
 template <typename T>
-__global__ void head_init_kernel(const T* __restrict__ h_last, float* __restrict__ state, int Hc, int wmax, int d, bf16* __restrict__ terms,
+__global__ void head_init_kernel(const T* h_last, float* __restrict__ state, int Hc, int wmax, int d, bf16* __restrict__ terms,
                                  int cols) {
   griddep_wait();
   griddep_launch();
@@ -308,7 +308,7 @@ __device__ __forceinline__ void warp_topk(const float (&v)[N], const int (&id)[N
 // sequence then fills the tree.  4 heads x 32000 entries, k = 10: 10.6 and 11.8 us with cold caches; with block-wide rounds
 // and the tree filled by a launch of its own 13, 8 and 3 us (a draft of the 7B shape, batch 4: 536 -> 531 us).
 constexpr int TK_WARPS = 8, TK_HELD = 16;
-__global__ void __launch_bounds__(TK_WARPS * 32) topk_part_kernel(const float* __restrict__ logits, int V, int Hc,
+__global__ void __launch_bounds__(TK_WARPS * 32) topk_part_kernel(const float* logits, int V, int Hc,
                                                                   const int32_t* __restrict__ kper, float* __restrict__ cand_v,
                                                                   int32_t* __restrict__ cand_i) {
   __shared__ float lv[TK_WARPS][CERB_MAX_TOPK];
@@ -370,7 +370,7 @@ __global__ void __launch_bounds__(TK_WARPS * 32) topk_part_kernel(const float* _
 }
 
 // One CTA per sequence, one warp per head: the merge, then the tree's tokens.
-__global__ void __launch_bounds__(CERB_MAX_HEADS * 32) topk_merge_kernel(const float* __restrict__ cand_v, const int32_t* __restrict__ cand_i,
+__global__ void __launch_bounds__(CERB_MAX_HEADS * 32) topk_merge_kernel(const float* cand_v, const int32_t* cand_i,
                                                                          int Hc, const int32_t* __restrict__ kper, int32_t* __restrict__ topk,
                                                                          int32_t* __restrict__ topk_copy, const int32_t* __restrict__ root,
                                                                          const int32_t* __restrict__ head_of, const int32_t* __restrict__ rank_of,
