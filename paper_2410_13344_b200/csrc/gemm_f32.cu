@@ -59,6 +59,10 @@ __global__ void __launch_bounds__(256) gemm_f32_kernel(const float* X, const flo
 // its way to shared memory), SwiGLU, RoPE and cache append, the residual add behind.  For KIND 1 and 2 a CTA's 16 weight rows are 8 and
 // the 8 that belong to them, so that the members of a pair sit 8 lanes apart.  Five launches per layer instead of nine: a 16-node
 // verification of four layers of 256 columns 125 -> 90 us, a request of 12 steps 2445 -> 2075; 320 rows 378 -> 353.
+// What such a launch needs beside its sum comes behind the rounds, and the kernel behind it is let go there: held through them it took
+// the third CTA of an SM, and the next launch's CTAs, with their own fetches, the places and the bandwidth of this one's (four layers of
+// 2048 columns, one row: 488 us with separate kernels, 585 so, 475 now; 768 columns, 128 rows 571, 615, 556; 1024 columns, 64 rows 567,
+// 499, 506).  (KIND 2 with the norm has 80 registers by itself; held to them it spills.)
 constexpr int SM_T = 16, SM_K = 256, SM_LD = SM_K + 4;
 struct F32Fused {
   float* act;               // KIND 1: [M][N / 2]
@@ -68,8 +72,8 @@ struct F32Fused {
   float eps;
 };
 template <bool VEC, int KIND, bool NORM>
-__global__ void __launch_bounds__(256, KIND == 0 ? 3 : 0) gemm_f32_small_kernel(const float* X, const float* __restrict__ W,
-                                                             float* out, int M, int N, int K, const F32Fused f) {
+__global__ void __launch_bounds__(256, KIND == 2 && NORM ? 0 : 3) gemm_f32_small_kernel(const float* X, const float* __restrict__ W,
+                                                                                         float* out, int M, int N, int K, const F32Fused f) {
   constexpr bool PAIRS = KIND == 1 || KIND == 2;
   __shared__ __align__(16) float sx[SM_T][SM_LD], sw[SM_T][SM_LD];
   __shared__ float red[8][SM_T * SM_T];
@@ -106,29 +110,30 @@ __global__ void __launch_bounds__(256, KIND == 0 ? 3 : 0) gemm_f32_small_kernel(
     for (int i = 0; i < 4; ++i) pg[i] = c4 + 64 * i < K ? *reinterpret_cast<const float4*>(f.gain + c4 + 64 * i) : make_float4(0.f, 0.f, 0.f, 0.f);
   }
   griddep_wait();
-  griddep_launch();
+  if constexpr (KIND == 0) griddep_launch();
   fetch_x(0);
   // this thread's output, and what it needs beside the sum
   const int m = m0 + (threadIdx.x >> 4), n = n0 + (threadIdx.x & 15);
   float old = 0.f;
-  if (KIND == 3 && m < M && n < N) old = out[(size_t)m * N + n];
-  int kv = -1, head = 0, el = 0;
+  int kv = -1;
   float2 cs = make_float2(1.f, 0.f);
-  if constexpr (KIND == 2) {
-    const int e = blockIdx.x * 8 + (threadIdx.x & 7);
-    head = e / f.half;
-    el = e % f.half;
-    if (m < M && e < N / 2) {
-      int b, v;
-      locate_row(m, f.re.row_off, f.re.B, f.re.n, b, v);
-      const int at = f.re.len[b] + f.re.depth[v], slot = f.re.len[b] + v;
-      if (v < f.re.n_active[b] && at < f.re.max_pos && slot < f.re.max_pos) {
-        kv = f.re.page_table[(size_t)b * f.re.max_pages + slot / CERB_PAGE] * f.re.H * CERB_PAGE + slot % CERB_PAGE;
-        cs = f.re.rope[(size_t)at * f.half + el];
+  auto fetch_rest = [&]() {
+    if (KIND == 3 && m < M && n < N) old = out[(size_t)m * N + n];
+    if constexpr (KIND == 2) {
+      const int e = blockIdx.x * 8 + (threadIdx.x & 7);
+      if (m < M && e < N / 2) {
+        int b, v;
+        locate_row(m, f.re.row_off, f.re.B, f.re.n, b, v);
+        const int at = f.re.len[b] + f.re.depth[v], slot = f.re.len[b] + v;
+        if (v < f.re.n_active[b] && at < f.re.max_pos && slot < f.re.max_pos) {
+          kv = f.re.page_table[(size_t)b * f.re.max_pages + slot / CERB_PAGE] * f.re.H * CERB_PAGE + slot % CERB_PAGE;
+          cs = f.re.rope[(size_t)at * f.half + e % f.half];
+        }
       }
     }
-  }
+  };
   if constexpr (NORM) {
+    fetch_rest();
     // (K is at most one round: 16 threads hold a row)
     float ss = 0.f;
 #pragma unroll
@@ -178,6 +183,8 @@ __global__ void __launch_bounds__(256, KIND == 0 ? 3 : 0) gemm_f32_small_kernel(
     }
     __syncthreads();
   }
+  if constexpr (!NORM) fetch_rest();
+  if constexpr (KIND != 0) griddep_launch();
 #pragma unroll
   for (int i = 0; i < 2; ++i)
 #pragma unroll
@@ -195,6 +202,7 @@ __global__ void __launch_bounds__(256, KIND == 0 ? 3 : 0) gemm_f32_small_kernel(
       const int e = blockIdx.x * 8 + (threadIdx.x & 7);
       if (!second && m < M && e < N / 2) f.act[(size_t)m * (N / 2) + e] = v / (1.0f + expf(-v)) * other;
     } else if (kv >= 0) {
+      const int e = blockIdx.x * 8 + (threadIdx.x & 7), head = e / f.half, el = e % f.half;
       const int which = head / f.re.H, h = head - which * f.re.H, Dh = 2 * f.half;
       const float o = which == 2 ? v : second ? v * cs.x + other * cs.y : v * cs.x - other * cs.y;
       float* at = which == 0 ? reinterpret_cast<float*>(f.re.q) + ((size_t)m * f.re.H + h) * Dh
