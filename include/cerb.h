@@ -98,7 +98,9 @@ typedef struct cerb_config {
 } cerb_config;
 
 /* Caller-owned device tensors, row-major [out][in], dtype as in the config.
- * The arrays of pointers themselves are HOST arrays and are copied at load. */
+ * The arrays of pointers themselves are HOST arrays and are copied at load.
+ * embed and the gains start on a boundary of four elements (cerb_load: CERB_E_ARG otherwise).  fp32: layers whose matrices do not all
+ * start on 16-byte boundaries run with separate kernels around their products. */
 typedef struct cerb_weights {
   const void* embed;             /* dev [vocab][d_model]  */
   const void* final_norm;        /* dev [d_model]         */
@@ -346,7 +348,8 @@ int cerb_set_wait_cycles(int64_t cycles);
  * to 128 rows).  With the residual add inside the O and down GEMMs (steps above 128 rows and of up to 8): 3 with SwiGLU inside the
  * gate-up GEMM and RoPE + cache append inside the QKV GEMM, 5 without either, 6 with SwiGLU, 7 with RoPE; 8: variant 3 with
  * the norms inside the QKV and gate-up GEMMs (up to 8 rows, as far as they fit: two of 4096 columns).  fp32 models: 8 with up to 256
- * columns, else 3, while the GEMMs have few output tiles; 0 above.  1 (SwiGLU alone), 2 (SwiGLU
+ * columns, else 3, while the layers' matrices start on 16-byte boundaries and each of their products has fewer than 296 tiles of 64 x 64
+ * outputs; else 0.  1 (SwiGLU alone), 2 (SwiGLU
  * and RoPE) and 4 (RoPE alone) describe no forward any more.  Returns CERB_OK when no kernel reads, ahead of its wait, a buffer
  * that the kernel right in front of it writes, CERB_E_STATE otherwise, CERB_E_NOMEM when buf is too small. */
 int cerb_launch_order_table(int32_t variant, char* buf_host, size_t cap);

@@ -475,6 +475,11 @@ int cerb_load(const cerb_config* cfg, const cerb_weights* w, void* workspace_dev
     return CERB_E_ARG;
   if (cfg->n_cheads > 0 && (!w->head_W || !w->head_b || !w->head_fc)) return CERB_E_ARG;
   if ((uintptr_t)workspace_dev & 255) return CERB_E_ARG;
+  // (every forward reads these four elements at a time; a load off their boundary would fault)
+  const uintptr_t four = (cfg->dtype == CERB_BF16 ? 4 * sizeof(bf16) : 4 * sizeof(float)) - 1;
+  uintptr_t odd = (uintptr_t)w->embed | (uintptr_t)w->final_norm;
+  for (int l = 0; l < cfg->n_layers; ++l) odd |= (uintptr_t)w->attn_norm[l] | (uintptr_t)w->mlp_norm[l];
+  if (odd & four) return CERB_E_ARG;
   cerb_ctx* c = new (std::nothrow) cerb_ctx();
   if (!c) return CERB_E_NOMEM;
   // The split plan (and with it the workspace size) is fixed for a 148-SM part so that
@@ -494,7 +499,7 @@ int cerb_load(const cerb_config* cfg, const cerb_weights* w, void* workspace_dev
   c->wd.assign(w->wd, w->wd + L);
   c->f32_aligned = !c->bf16;
   for (int l = 0; l < L; ++l)
-    for (const void* w_l : {c->attn_norm[l], c->wqkv[l], c->wo[l], c->mlp_norm[l], c->wgu[l], c->wd[l]})
+    for (const void* w_l : {c->wqkv[l], c->wo[l], c->wgu[l], c->wd[l]})
       if ((uintptr_t)w_l & 15) c->f32_aligned = false;
   if (g.n_cheads > 0) {
     c->head_W.assign(w->head_W, w->head_W + g.n_cheads * g.n_levels);

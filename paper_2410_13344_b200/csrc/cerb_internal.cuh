@@ -151,7 +151,7 @@ struct cerb_ctx {
 
   // weights (device pointers, host arrays)
   const void *embed, *final_norm, *lm_head;
-  bool f32_aligned;                   // fp32: every matrix and gain of the layers starts on a 16-byte boundary
+  bool f32_aligned;                   // fp32: every matrix of the layers starts on a 16-byte boundary (gains always do)
   std::vector<const void*> attn_norm, wqkv, wo, mlp_norm, wgu, wd, head_W, head_b, head_fc;
   char *k_pool, *v_pool;
   size_t pool_layer_bytes;

@@ -178,3 +178,30 @@ def test_the_read_before_wait_rule_holds_in_every_variant():
     buf = ctypes.create_string_buffer(1 << 14)
     for variant in (-1, len(fused)):
         assert binding.lib().cerb_launch_order_table(variant, buf, len(buf)) == binding.E_ARG
+
+
+def test_load_refuses_gains_and_embeddings_off_their_boundary():
+    """The norms read gains and embedding rows four elements at a time, which off a boundary of four elements is a fault on the GPU.  The
+    check comes before anything is launched (the addresses here belong to nobody)."""
+    import ctypes as C
+    from paper_2410_13344_b200 import binding, synth
+    for dtype, step in (("fp32", 16), ("bf16", 8)):
+        cfg = binding.make_config(synth.tiny_shape(dtype), None, [], 4, 4, 1, 16)
+
+        def load(**moved):
+            w = binding.Weights()
+            for name, kind in binding.Weights._fields_:
+                if kind is C.c_void_p:
+                    setattr(w, name, (1 << 20) + moved.get(name, 0))
+                else:
+                    at = [(1 << 20) + (moved.get(name, 0) if l == cfg.n_layers - 1 else 0) for l in range(cfg.n_layers)]
+                    setattr(w, name, (C.c_void_p * cfg.n_layers)(*at))
+            ctx = C.c_void_p()
+            return binding.lib().cerb_load(C.byref(cfg), C.byref(w), 1 << 20, 0, C.byref(ctx))
+
+        assert load() == binding.E_NOMEM                       # (past the pointers, at the workspace of no bytes)
+        for name in ("embed", "final_norm", "attn_norm", "mlp_norm"):
+            assert load(**{name: step}) == binding.E_NOMEM, name
+            for off in (4, step // 2, step - 2):
+                assert load(**{name: off}) == binding.E_ARG, (name, off)
+        assert load(wqkv=4, wd=4) == binding.E_NOMEM
