@@ -85,11 +85,11 @@ __global__ void __launch_bounds__(KT_THREADS, 1) tree_attn_kt_kernel(const __gri
   __shared__ __align__(8) uint64_t full_u[2][NU], empty_u[NU], s_full[2], s_free[2], p_ready[PB], pv_done[PB], q_ready, drain_bar[2];
   __shared__ __align__(8) uint64_t cl_bar[2], rx_bar;
   __shared__ int page_list[kMaxPagesPerCta];
-  __shared__ uint32_t desc_t[CERB_MAX_NODES][4];   // per tree key: which queries of this launch see it, 32 per word
-  __shared__ __align__(16) float m_ref[128];       // reference exponent per query (KT_UNSET until a key is seen)
-  __shared__ int m_pending[128];                   // largest visible score reported since the last raise (ordered int)
-  __shared__ int raise_at[2][4];                   // [tile parity][query block]: 1 + the last tile at which a raise was requested
-  __shared__ float l_part[4][128];                 // per lane quarter: partial row sums, added at the end
+  __shared__ uint32_t desc_t[CERB_MAX_NODES][NQ / 32];   // per tree key: which queries of this launch see it, 32 per word
+  __shared__ __align__(16) float m_ref[NQ];        // reference exponent per query (KT_UNSET until a key is seen)
+  __shared__ int m_pending[NQ];                    // largest visible score reported since the last raise (ordered int)
+  __shared__ int raise_at[2][NCB];                 // [tile parity][query block]: 1 + the last tile at which a raise was requested
+  __shared__ float l_part[4][NQ];                  // per lane quarter: partial row sums, added at the end
   __shared__ uint32_t tmem_slot;
   __shared__ int aborted_s, exit_flag_s;
   __shared__ unsigned int ticket_s;
@@ -98,7 +98,7 @@ __global__ void __launch_bounds__(KT_THREADS, 1) tree_attn_kt_kernel(const __gri
 
   const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
   uint8_t* smem_gen = smem_raw + (smem_base - smem_u32(smem_raw));
-  const uint32_t p_base = smem_base;                                 // [buffer][hi, lo][64-query block][128 keys][128 B]
+  const uint32_t p_base = smem_base;                                 // [buffer][hi, lo][128 keys][128 B]
   const uint32_t q_base = p_base + PB * 2 * P_TERM;                       // [half of head_dim][NQ rows][128 B]
   const uint32_t ring = q_base + 2 * QHALF;                          // NU units
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -150,8 +150,8 @@ __global__ void __launch_bounds__(KT_THREADS, 1) tree_attn_kt_kernel(const __gri
     if (too_long) atomicExch(p.status, CERB_E_SHAPE);
   }
   // queries that do not exist keep reference 0: their score columns are zero and never ask for a new one
-  if (threadIdx.x < 128) { m_ref[threadIdx.x] = (int)threadIdx.x < nq ? KT_UNSET : 0.f; m_pending[threadIdx.x] = f2ord(-INFINITY); }
-  if (threadIdx.x < 8) raise_at[threadIdx.x >> 2][threadIdx.x & 3] = 0;
+  if (threadIdx.x < NQ) { m_ref[threadIdx.x] = (int)threadIdx.x < nq ? KT_UNSET : 0.f; m_pending[threadIdx.x] = f2ord(-INFINITY); }
+  if (threadIdx.x < 2 * NCB) raise_at[threadIdx.x / NCB][threadIdx.x % NCB] = 0;
   if (warp == W_QK) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_slot)), "r"(TMEM_COLS)
                  : "memory");
@@ -166,13 +166,11 @@ __global__ void __launch_bounds__(KT_THREADS, 1) tree_attn_kt_kernel(const __gri
   float* rx = mrg + NQ * ROWF;                       // [member][rows_each][ROWF], up to 8 members
   static_assert((2 * NQ + 7) * ROWF * 4 <= (int)(PB * 2 * P_TERM + 2 * QHALF), "both fit there");
 
-  // Waiting for unit u (K units are even, V units odd) to have landed.  A parity wait only tells "the phase before
-  // the current one is complete", so every barrier needs ONE waiter that sees each of its phases in turn.  With
-  // an odd ring depth a slot holds K and V units alternately, and a K consumer looking at every other phase of a
-  // shared barrier returned at once when its wait began before the V unit in between had landed (a rare
-  // dead-lock, measured).  Hence one "landed" barrier per slot and per kind of unit: full_u[kind][slot], whose
-  // phases the one consumer of that kind sees in order.
-  auto unit_parity = [](int u) { return (uint32_t)((NU & 1) ? (u / NU) >> 1 : u / NU) & 1u; };
+  // Waiting for unit u (K units are even, V units odd) to have landed.  A parity wait only tells "the phase before the current one is
+  // complete", so a barrier's phases have to be seen in turn: one "landed" barrier per slot and kind of unit, whose one consumer sees
+  // all of them.
+  static_assert(NU % 2 == 0, "a slot holds units of one kind");
+  auto unit_parity = [](int u) { return (uint32_t)(u / NU) & 1u; };
   auto wait_unit = [&](int u, int site) { return mbar_wait(smem_u32(&full_u[u & 1][u % NU]), unit_parity(u), wc, site); };
   if (warp >= NSW && warp < NSW + NPROD) {
     // ---------------- TMA producers ----------------
@@ -181,7 +179,7 @@ __global__ void __launch_bounds__(KT_THREADS, 1) tree_attn_kt_kernel(const __gri
     // every other tile came 1500 cycles late (2200 and 3800 cycles from tile to tile in turn).  Producer w of its half issues boxes
     // w, w + NPROD / 2, ... of every unit (box = page * 2 + half of head_dim), one per lane.
     const int pw = warp - NSW, kind = pw & 1;
-    static_assert(NU % 2 == 0 && NPROD % 2 == 0, "slots and producers of one kind");
+    static_assert(NPROD % 2 == 0, "producers of one kind");
     constexpr int BOXES = 32 / NPROD;                // boxes of a unit per producer warp
     const int32_t* pt = p.page_table + (size_t)b * p.max_pages;
     const int n_pages = T * KT_PAGES;
@@ -369,7 +367,7 @@ __global__ void __launch_bounds__(KT_THREADS, 1) tree_attn_kt_kernel(const __gri
       const uint32_t vis = !masked ? 0xffffffffu : kpos < L ? qmask : kpos < kv_total ? ((desc_t[kpos - L][cb * QB / 32] >> (cb * QB % 32)) & qmask) : 0u;
       if (t == 0 && !masked) {
         // First tile, all keys visible: the scores of its first key serve as the reference (any value within the
-        // exponent range of the true maximum does; whatever exceeds it by 2^8 later raises it the usual way).
+        // exponent range of the true maximum does; whatever exceeds it by 2^30 later raises it the usual way).
         if (r == 0) {
 #pragma unroll
           for (int j = 0; j < QB; ++j)
@@ -413,7 +411,6 @@ __global__ void __launch_bounds__(KT_THREADS, 1) tree_attn_kt_kernel(const __gri
         if (lane == 0) raise_at[t & 1][cb] = t + 1;
       }
       asm volatile("bar.sync %0, 128;" ::"r"(4 + cb) : "memory");     // the four warps of this query block agree
-      bool waited_pv = false;
       if (raise_at[t & 1][cb] == t + 1) {
         // New reference m' = max(m, reported) for this block's queries: what was accumulated under m shrinks by
         // 2^(m - m'), this tile's scores are taken again relative to m'.
@@ -430,7 +427,6 @@ __global__ void __launch_bounds__(KT_THREADS, 1) tree_attn_kt_kernel(const __gri
         if (t > 0 && any_change) {
           mbar_wait(smem_u32(&pv_done[(t - 1) % PB]), (uint32_t)((t - 1) / PB) & 1u, wc, 108);      // O^T at rest (PV retires in order)
           tc_fence_after();
-          waited_pv = true;
           // rows of O^T = head-dim lanes of this warp's quarter; columns of this query block, both terms
 #pragma unroll 1
           for (int term = 0; term < 2; ++term) {
@@ -447,7 +443,7 @@ __global__ void __launch_bounds__(KT_THREADS, 1) tree_attn_kt_kernel(const __gri
         {
           uint32_t raw[QB];
           tmem_ld16_nowait(s_addr, raw);
-            tmem_ld_wait();
+          tmem_ld_wait();
 #pragma unroll
           for (int j = 0; j < QB; ++j)
             sc[j] = ((vis >> j) & 1u) ? fmaf(__uint_as_float(raw[j]), p.scale_log2, -fmaxf(mr[j], ord2f(pend[j]))) : -INFINITY;
@@ -472,7 +468,7 @@ __global__ void __launch_bounds__(KT_THREADS, 1) tree_attn_kt_kernel(const __gri
         const float r0 = p0 - __uint_as_float(b0 & 0xffff0000u), r1 = p1 - __uint_as_float(b1 & 0xffff0000u);
         lo[j >> 1] = __byte_perm(__float_as_uint(r0), __float_as_uint(r1), 0x7632);
       }
-      if (t >= PB && !(PB == 1 && waited_pv)) {
+      if (t >= PB) {
         mbar_wait(smem_u32(&pv_done[t % PB]), (uint32_t)(t / PB - 1) & 1u, wc, 109);        // this tile's P^T buffer is free
         tc_fence_after();
       }
