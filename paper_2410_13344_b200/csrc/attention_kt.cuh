@@ -192,7 +192,7 @@ __global__ void __launch_bounds__(KT_THREADS, 1) tree_attn_kt_kernel(const __gri
     // units (K and V) of tiles that lie wholly inside the prefix may be fetched before the wait
     int early = 0;
     while (early < T && 2 * early < NU && (t0 + early + 1) * KT_TILE <= L) ++early;
-    static_assert(KT_PAGES == 8, "the lane -> box map below assumes eight pages per tile");
+    static_assert(KT_PAGES == 8 && BOXES == 8, "the lane -> box map below assumes eight pages per tile and two producers of a kind");
     const int box = (pw >> 1) + (NPROD / 2) * lane;  // lanes 0 .. BOXES-1
     const int pg = box >> 1, hf = box & 1;
     const uint64_t pol = l2_policy(true);            // K/V are read once per step
@@ -200,7 +200,18 @@ __global__ void __launch_bounds__(KT_THREADS, 1) tree_attn_kt_kernel(const __gri
     // (the abort flag itself is looked at once, for a launch that starts after a time-out: nothing is issued then;
     // later a wait that gives up says so in its return value, which costs the loop nothing)
     const int t_stop = *aborted ? 0 : T;
-    for (int t = 0; t < t_stop; ++t) {
+    // All producers fetch the first K unit, which everything waits for; its bytes are expected by those of its kind.  (Cold caches, by its
+    // own two producers / by all: 192 items of 60 keys, 64 nodes, 18.8 / 18.4 us; 512 of 100 keys, 24 nodes, 33.6 / 32.8; 96 of 1000 keys,
+    // 64 nodes, 20.4 / 20.2; a verification step of 64 nodes behind 2048 keys 3509 / 3494.)
+    if (t_stop > 0) {
+      if (early == 0) { griddep_wait(); griddep_launch(); }
+      if (!kind && lane == 0) mbar_expect_tx(smem_u32(&full_u[0][0]), KT_UNIT / (NPROD / 2));
+      __syncwarp();
+      if (lane >> 2 == kind)
+        tma_load_2d_hint(ring + (uint32_t)hf * KT_HALF + (uint32_t)pg * (CERB_PAGE * 128), &tmK, hf * 64, page_list[pg], smem_u32(&full_u[0][0]), pol);
+      issued = 1 - kind;
+    }
+    for (int t = issued; t < t_stop; ++t) {
       if (t == early) { griddep_wait(); griddep_launch(); }
       const int u = 2 * t + kind, slot = u % NU;
       const uint32_t fb = smem_u32(&full_u[kind][slot]);
@@ -220,6 +231,7 @@ __global__ void __launch_bounds__(KT_THREADS, 1) tree_attn_kt_kernel(const __gri
     if (lane == 0 && *aborted) {
       // give-up path: the copies this warp has issued still land in the CTA's shared memory; see them in (the
       // phase also needs the other producers' shares, hence a limit of its own: 10 ms)
+      if (kind && t_stop > 0) mbar_wait_drain(smem_u32(&full_u[0][0]), 0, 20000000ll);
       for (int t = issued > NU / 2 ? issued - NU / 2 : 0; t < issued; ++t)
         mbar_wait_drain(smem_u32(&full_u[kind][(2 * t + kind) % NU]), unit_parity(2 * t + kind), 20000000ll);
     }
