@@ -85,8 +85,9 @@ __device__ __forceinline__ void add_slots(float4 (&sum)[COLS], const float* p, c
 //   x <- (embedding row | x | x + sum of GEMM partial slots), kept in fp32 (the residual stream is never rounded);
 //   out <- RMSNorm(x) * gain, in the model's storage type.
 // Fusing the residual add (and the first layer's embedding gather) with the norm that always follows
-// it halves the element-wise launches; all slots of a thread's columns (ten after a 4096-column product of 64 rows) are on their way
-// at once, and the sums of the warps are read back four at a time.
+// it halves the element-wise launches.  Of up to 4096 columns, all of up to eleven slots of a thread's columns are on their way at once
+// (ten after a 4096-column product of 64 rows); up to 8192 columns eight at a time, above that two.  The sums of the warps are read back
+// four at a time.
 constexpr int NORM_THREADS = 1024;
 constexpr int NORM_MAX_ITER = 4;          // d_model up to 16384
 template <typename T, int ITER, int AHEAD, bool EXACT>
@@ -429,7 +430,10 @@ int launch_fused_norm(cerb_ctx* c, const float* part, int nsplit, size_t split_s
                  tok ? (const T*)c->embed : (const T*)nullptr, tok, tok_stride, tok_off, (const int32_t*)c->d_nactive, n, g.vocab,
                  (const T*)gain, (T*)out, d, g.rms_eps, row_off, c->B);
     };
-    // Up to eight slots are one trip to L2; nine to eleven are with code for just that many (their tests would cost spills).
+    // Up to 4096 columns: up to eight slots are one trip to L2; nine to eleven (O products of 2560 to 4096 columns, down products of 1024 and
+    // 4096) are with code for just that many, whose tests would cost spills; 12 to 19 (2048 to 3200 columns) take two trips and three.
+    // Wider rows have at most nine slots.  Whole forwards of 64 rows against four slots at a time, unrolled by the compiler: 1024 columns
+    // 1.08 x, 2048 to 3200 1.05 x, 4096 1.055 x, 5120 1.03 x, 8192 1.01 x, 12288 1.00 to 1.015 x (with all sums of slots).
     const bool one = d <= NORM_THREADS * 4;
     if (c->bf16 && one && nsplit == 9) go(fused_norm_kernel<bf16, 1, 9, true>, bf16());
     else if (c->bf16 && one && nsplit == 10) go(fused_norm_kernel<bf16, 1, 10, true>, bf16());
@@ -479,7 +483,7 @@ int launch_argmax_rows(cerb_ctx* c, const float* part, int nsplit, size_t split_
   // four rows to an SM, the loads of one beside the reduction of another (2048 rows: 97 -> 67 us; 256 rows 9.0 -> 6.3; one row 4.4 -> 3.5, 64 rows of three
   // slots 8.2 -> 7.4).
   auto go = [&](auto kern, int threads) { launch_pdl(kern, dim3(rows), dim3(threads), 0, st, part, nsplit, split_stride, V, out, summed); };
-  if (nsplit == 1) go(argmax_rows_kernel<8, 1>, rows <= 148 ? 1024 : rows <= 2 * 148 ? 512 : 256);
+  if (nsplit == 1) go(argmax_rows_kernel<8, 1>, rows <= c->sm_count ? 1024 : rows <= 2 * c->sm_count ? 512 : 256);
   else if (nsplit == 2) go(argmax_rows_kernel<4, 2>, 1024);
   else go(argmax_rows_kernel<2, 3>, 1024);
   CERB_LAUNCH_CHECK(c);
