@@ -67,6 +67,14 @@ __device__ __forceinline__ int f2ord(float f) {
 }
 __device__ __forceinline__ float ord2f(int i) { return __int_as_float(i >= 0 ? i : i ^ 0x7fffffff); }
 
+// The first phase of a barrier of the exchange, for a CTA that has given up.  (Out of line, and the end of a launch without splits right
+// behind the key loop: what runs once comes from far away, and with both waits inside, in front of that end, a launch of one tile per CTA
+// took 0.65 us longer; 0.2 so.)
+__device__ __noinline__ bool wait_for_partner(uint32_t bar, long long budget) {
+  const WaitCtx w{budget, nullptr, nullptr};
+  return mbar_wait_drain(bar, 0, partner_cycles(w));
+}
+
 __global__ void __launch_bounds__(KT_THREADS, 1) tree_attn_kt_kernel(const __grid_constant__ CUtensorMap tmK,
                                                                      const __grid_constant__ CUtensorMap tmV,
                                                                      const AttnParams p) {
@@ -556,7 +564,18 @@ __global__ void __launch_bounds__(KT_THREADS, 1) tree_attn_kt_kernel(const __gri
     // ---- output: final, or partial + fixed-order merge by the last CTA of this (sequence, head) ----
     const int ct = st, nct = nst, RP = p.rows_pad;
     const float LN2 = 0.6931471805599453f;
-    if (p.cluster) {
+    if (p.nsplit == 1) {
+      for (int idx = ct; idx < nq * (DH / 4); idx += nct) {
+        const int rr = idx / (DH / 4), c4 = idx % (DH / 4);
+        const float inv = 1.0f / mrg[(size_t)rr * ROWF + DH + 1];
+        const float4 v = *reinterpret_cast<const float4*>(mrg + (size_t)rr * ROWF + c4 * 4);
+        *reinterpret_cast<uint2*>(p.out + ((qrow + rr) * p.H + h) * DH + c4 * 4) =
+            make_uint2(pack_bf16(v.x * inv, v.y * inv), pack_bf16(v.z * inv, v.w * inv));
+      }
+      if (p.lse)
+        for (int rr = ct; rr < nq; rr += nct)
+          p.lse[((size_t)b * p.H + h) * p.n + rr] = (mrg[(size_t)rr * ROWF + DH] + log2f(mrg[(size_t)rr * ROWF + DH + 1])) * LN2;
+    } else if (p.cluster) {
       // The splits of this (sequence, head) are the CTAs of one cluster (rank = split).  Each sends every other member that member's
       // rows (O, m, l) as one bulk copy and finishes its own from what it has received, in split order.  (Read out of the others'
       // shared memory by loads instead, the rows took 3900 of the 27500 cycles of a launch of 64 rows over 2048 keys, and another
@@ -567,7 +586,7 @@ __global__ void __launch_bounds__(KT_THREADS, 1) tree_attn_kt_kernel(const __gri
       // that; if it has given up, it waits for each of these as long as a member that has not may take.
       if (warp == 0) {
         const bool ready = __all_sync(0xffffffffu, mbar_wait_cluster(smem_u32(&cl_bar[0]), 0, wc, 112) ||
-                                                       mbar_wait_drain(smem_u32(&cl_bar[0]), 0, partner_cycles(wc)));
+                                                       wait_for_partner(smem_u32(&cl_bar[0]), wc.budget));
         proxy_fence();
         const int lo = min(nq, lane * rows_each), rows = min(nq, lo + rows_each) - lo;
         if (ready && lane < p.nsplit && lane != split && rows > 0)
@@ -575,7 +594,7 @@ __global__ void __launch_bounds__(KT_THREADS, 1) tree_attn_kt_kernel(const __gri
                          mapa_u32(smem_u32(&rx_bar), (uint32_t)lane));
         __syncwarp();
       }
-      const bool landed = mbar_wait(smem_u32(&rx_bar), 0, wc, 113) || mbar_wait_drain(smem_u32(&rx_bar), 0, partner_cycles(wc));
+      const bool landed = mbar_wait(smem_u32(&rx_bar), 0, wc, 113) || wait_for_partner(smem_u32(&rx_bar), wc.budget);
       if (landed && st < p.nsplit) mbar_arrive_cluster(mapa_u32(smem_u32(&cl_bar[1]), (uint32_t)st));        // this CTA has received all it needs
       // half a warp finishes a row; its lane s2 looks after member s2's weight.  (Short code: what runs once comes from far away.)
       const int half = lane >> 4, hl = lane & 15;
@@ -605,17 +624,6 @@ __global__ void __launch_bounds__(KT_THREADS, 1) tree_attn_kt_kernel(const __gri
         *reinterpret_cast<uint2*>(o + 64) = make_uint2(pack_bf16(a1.x * inv, a1.y * inv), pack_bf16(a1.z * inv, a1.w * inv));
         if (hl == 0 && p.lse) p.lse[((size_t)b * p.H + h) * p.n + rr] = (M + log2f(Lsum)) * LN2;
       }
-    } else if (p.nsplit == 1) {
-      for (int idx = ct; idx < nq * (DH / 4); idx += nct) {
-        const int rr = idx / (DH / 4), c4 = idx % (DH / 4);
-        const float inv = 1.0f / mrg[(size_t)rr * ROWF + DH + 1];
-        const float4 v = *reinterpret_cast<const float4*>(mrg + (size_t)rr * ROWF + c4 * 4);
-        *reinterpret_cast<uint2*>(p.out + ((qrow + rr) * p.H + h) * DH + c4 * 4) =
-            make_uint2(pack_bf16(v.x * inv, v.y * inv), pack_bf16(v.z * inv, v.w * inv));
-      }
-      if (p.lse)
-        for (int rr = ct; rr < nq; rr += nct)
-          p.lse[((size_t)b * p.H + h) * p.n + rr] = (mrg[(size_t)rr * ROWF + DH] + log2f(mrg[(size_t)rr * ROWF + DH + 1])) * LN2;
     } else {
       float* part = p.partial + (((size_t)blockIdx.z * p.H + h) * p.nsplit) * (size_t)(RP * ROWF);
       float* mine = part + (size_t)split * (RP * ROWF);
