@@ -261,10 +261,11 @@ int gemm(cerb_ctx* c, const void* X, const ActMaps* xm, const void* W, const CUt
 
 // The same for a GEMM that ends in a fused epilogue.
 int gemm_fused(cerb_ctx* c, const void* X, const ActMaps* xm, const void* W, const CUtensorMap* wm, int M, int N, int K,
-               const GemmEpilogue& epi, cudaStream_t st, const GemmNorm* norm = nullptr) {
+               const GemmEpilogue& epi, cudaStream_t st, const GemmNorm* norm = nullptr, const RowsPlan* rows = nullptr) {
   ProfScope ps(c, K_GEMM, st);
   if (!c->bf16) return launch_gemm_f32_fused(c, (const float*)X, (const float*)W, M, N, K, epi, norm, st);
   if (M <= kFewRows) return launch_gemm_few(c, X, W, nullptr, M, N, K, st, &epi, norm, gemm_clock_slot(c));
+  if (rows) return launch_gemm_rows(c, wm, xm, *rows, M, N, K, c->d_status, st, &epi, gemm_clock_slot(c));
   return launch_gemm_tile(c, wm, xm, make_tile_plan(M, N, K, false), nullptr, c->d_gemm_fix, c->d_gemm_tickets, M, N, c->d_status, st, &epi,
                           gemm_clock_slot(c));
 }
@@ -321,8 +322,11 @@ int forward_rows(cerb_ctx* c, const cerb_tree* tree, const int32_t* tok, int tok
   // fp32: the same as long as the GEMMs have few output tiles.
   const bool small = !c->bf16 && c->f32_aligned && gemm_f32_small(M, 2 * F) && gemm_f32_small(M, 3 * HD) && gemm_f32_small(M, d);
   const bool wide = small || (c->bf16 && (M > 128 || M <= kFewRows));
-  const bool fuse_swiglu = small || (wide && (M <= kFewRows || F % 16 == 0));
-  const bool fuse_rope = small || (wide && g.head_dim == 128);
+  // 9 to 128 rows: SwiGLU and RoPE + cache append only, where the matrix is for gemm_rows.cu (which takes some of these up to 256 rows, too).
+  const RowsPlan* rows_gu = c->bf16 && gemm_rows_takes(c->rows_gu, M, 2 * F, d) ? &c->rows_gu : nullptr;
+  const RowsPlan* rows_qkv = c->bf16 && gemm_rows_takes(c->rows_qkv, M, 3 * HD, d) ? &c->rows_qkv : nullptr;
+  const bool fuse_swiglu = small || rows_gu || (wide && (M <= kFewRows || F % 16 == 0));
+  const bool fuse_rope = small || rows_qkv || (wide && g.head_dim == 128);
   const bool fuse_res = wide;
   // Very few rows: the gate-up and QKV GEMMs normalise their rows themselves (the first layer's QKV GEMM excepted).
   const bool fuse_norm = small ? d <= kF32NormMax : fuse_swiglu && fuse_rope && M <= kFewRows && gemm_few_normalises(M, d);
@@ -350,7 +354,7 @@ int forward_rows(cerb_ctx* c, const cerb_tree* tree, const int32_t* tok, int tok
                             (void*)a.k_pool, (void*)a.v_pool, g.max_pages, c->max_pos, n, g.n_heads, B};
       const GemmEpilogue epi{2, nullptr, &re, nullptr};
       const GemmNorm nm{(const float*)c->d_x, c->attn_norm[l], g.rms_eps};
-      CERB_TRY(gemm_fused(c, c->d_xn, &c->tm_xn, c->wqkv[l], c->bf16 ? &c->tm_wqkv_rot[l] : nullptr, M, 3 * HD, d, epi, st, fuse_norm && l ? &nm : nullptr));
+      CERB_TRY(gemm_fused(c, c->d_xn, &c->tm_xn, c->wqkv[l], c->bf16 ? (rows_qkv ? &c->tm_wqkv_rows[l] : &c->tm_wqkv_rot[l]) : nullptr, M, 3 * HD, d, epi, st, fuse_norm && l ? &nm : nullptr, rows_qkv));
     } else {
       { ProfScope ps(c, K_GEMM, st);
         CERB_TRY(gemm(c, c->d_xn, &c->tm_xn, c->wqkv[l], c->bf16 ? &c->tm_wqkv[l] : nullptr, M, 3 * HD, d, &ns, st)); }
@@ -377,7 +381,7 @@ int forward_rows(cerb_ctx* c, const cerb_tree* tree, const int32_t* tok, int tok
       // SwiGLU runs in the GEMM's epilogue: no separate kernel, no second pass over the partial sums
       const GemmEpilogue epi{1, c->d_act, nullptr, nullptr};
       const GemmNorm nm{(const float*)c->d_x, c->mlp_norm[l], g.rms_eps};
-      CERB_TRY(gemm_fused(c, c->d_xn, &c->tm_xn, c->wgu[l], c->bf16 ? &c->tm_wgu_pair[l] : nullptr, M, 2 * F, d, epi, st, fuse_norm ? &nm : nullptr));
+      CERB_TRY(gemm_fused(c, c->d_xn, &c->tm_xn, c->wgu[l], c->bf16 ? (rows_gu ? &c->tm_wgu_rows[l] : &c->tm_wgu_pair[l]) : nullptr, M, 2 * F, d, epi, st, fuse_norm ? &nm : nullptr, rows_gu));
     } else {
       { ProfScope ps(c, K_GEMM, st);
         CERB_TRY(gemm(c, c->d_xn, &c->tm_xn, c->wgu[l], c->bf16 ? &c->tm_wgu[l] : nullptr, M, 2 * F, d, &ns, st)); }
@@ -532,6 +536,9 @@ int cerb_load(const cerb_config* cfg, const cerb_weights* w, void* workspace_dev
       const int Mr = round_up(c->Mmax, 256);
       c->tm_wqkv.resize(L); c->tm_wo.resize(L); c->tm_wgu.resize(L); c->tm_wd.resize(L);
       c->tm_wqkv_rot.resize(L); c->tm_wgu_pair.resize(L);
+      c->rows_qkv = plan_rows_rope(g.n_heads, g.head_dim);
+      c->rows_gu = plan_rows_swiglu(g.mlp_dim);
+      c->tm_wqkv_rows.resize(L); c->tm_wgu_rows.resize(L);
       c->tm_kpool.resize(L); c->tm_vpool.resize(L);
       for (int l = 0; l < L && rc == CERB_OK; ++l) {
         if ((rc = make_weight_map(&c->tm_wqkv[l], c->wqkv[l], 3 * HD, g.d_model)) != CERB_OK) break;
@@ -540,6 +547,8 @@ int cerb_load(const cerb_config* cfg, const cerb_weights* w, void* workspace_dev
         if ((rc = make_weight_map(&c->tm_wd[l], c->wd[l], g.d_model, g.mlp_dim)) != CERB_OK) break;
         if (g.head_dim == 128 && (rc = make_rotation_map(&c->tm_wqkv_rot[l], c->wqkv[l], 3 * g.n_heads, g.d_model)) != CERB_OK) break;
         if (g.mlp_dim % 16 == 0 && (rc = make_gate_up_map(&c->tm_wgu_pair[l], c->wgu[l], g.mlp_dim, g.d_model)) != CERB_OK) break;
+        if (c->rows_qkv.tiles && (rc = make_rotation_groups(&c->tm_wqkv_rows[l], c->wqkv[l], 3 * g.n_heads, g.d_model, c->rows_qkv.groups)) != CERB_OK) break;
+        if (c->rows_gu.tiles && (rc = make_gate_up_groups(&c->tm_wgu_rows[l], c->wgu[l], g.mlp_dim, g.d_model, c->rows_gu.groups)) != CERB_OK) break;
         if ((rc = make_pool_map(&c->tm_kpool[l], c->k_pool + (size_t)l * c->pool_layer_bytes, g.n_pool_pages, g.n_heads, g.head_dim)) != CERB_OK) break;
         if ((rc = make_pool_map(&c->tm_vpool[l], c->v_pool + (size_t)l * c->pool_layer_bytes, g.n_pool_pages, g.n_heads, g.head_dim)) != CERB_OK) break;
       }

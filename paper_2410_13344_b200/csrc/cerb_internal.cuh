@@ -130,6 +130,12 @@ struct ActMaps {
   const CUtensorMap& box(int rows) const { return m[rows / 16 - 1]; }
 };
 
+// gemm_rows.cu: how a matrix is cut into one tile per SM; no tiles = it is not for that kernel
+struct RowsPlan {
+  int groups, tiles;
+  bool heads;               // cut by heads (RoPE)
+};
+
 }  // namespace cerb
 
 struct cerb_tree {
@@ -160,6 +166,8 @@ struct cerb_ctx {
   // tensor maps (bf16 only)
   std::vector<CUtensorMap> tm_wqkv, tm_wo, tm_wgu, tm_wd;
   std::vector<CUtensorMap> tm_wqkv_rot, tm_wgu_pair;   // the same rows gathered for the epilogues above 128 rows
+  std::vector<CUtensorMap> tm_wqkv_rows, tm_wgu_rows;  // ... and for those of gemm_rows.cu, where there is a plan
+  cerb::RowsPlan rows_qkv, rows_gu;
   CUtensorMap tm_lm_head;
   cerb::ActMaps tm_xn, tm_attn, tm_act, tm_hidden, tm_hlast;
   std::vector<CUtensorMap> tm_kpool, tm_vpool;        // per layer
@@ -251,13 +259,14 @@ int launch_prefill_commit(cerb_ctx* c, cudaStream_t st);
 // gemm_f32.cu / gemm_bf16.cu : out[split][M][N] fp32 partial sums of X[M][K] . W[N][K]^T
 int launch_gemm_f32(cerb_ctx* c, const float* X, const float* W, float* out, int M, int N, int K, cudaStream_t st);
 int gemm_plan_split(int sm_count, int M, int N, int K);
-// What may follow a bf16 GEMM in its epilogue (gemm_few.cu, up to kFewRows rows; gemm_tile.cu, above 128 rows).
+// What may follow a bf16 GEMM in its epilogue (gemm_few.cu, up to kFewRows rows; gemm_rows.cu, 9 to 256 rows, kinds 1 and 2; gemm_tile.cu, above 128
+// rows).
 // kind 1 (SwiGLU): W is [gate rows F][up rows F]; act[row][f] = SiLU(gate) * up (bf16).
 // kind 2 (RoPE + cache append): W is the QKV matrix [q rows | k rows | v rows] of a model with head_dim 128; q and k are
 // rotated at position len + depth, q is written dense and k, v into the paged pools -- what rope_append_kernel does, with the
 // same arithmetic in the same order.
 // kind 3: the product is added to the fp32 residual stream.
-// In between (9 to 128 rows) separate kernels do this work: the GEMM leaves partial sums there.
+// From 9 to 128 rows separate kernels add the residual (and do the rest where the matrix is not for gemm_rows.cu): the GEMM leaves partial sums there.
 struct RopeEpilogue {
   const int32_t *len, *n_active, *depth, *page_table, *row_off;    // as for rope_append_kernel (row_off may be null)
   const float2* rope;       // rotation table [max_pos][64]
@@ -296,11 +305,19 @@ int launch_gemm_f32_fused(cerb_ctx* c, const float* X, const float* W, int M, in
 int launch_gemm_few(cerb_ctx* c, const void* X, const void* W, float* out, int M, int N, int K, cudaStream_t st, const GemmEpilogue* epi = nullptr,
                     const GemmNorm* norm = nullptr, unsigned long long* clock_slot = nullptr);
 bool gemm_few_normalises(int M, int K);
+// gemm_rows.cu: 9 to 256 rows, kinds 1 and 2
+bool gemm_rows_takes(const RowsPlan& g, int M, int N, int K);
+RowsPlan plan_rows_swiglu(int F);
+RowsPlan plan_rows_rope(int n_heads, int head_dim);
+int launch_gemm_rows(cerb_ctx* c, const CUtensorMap* tmW, const ActMaps* tmX, const RowsPlan& g, int M, int N, int K, int32_t* status, cudaStream_t st,
+                     const GemmEpilogue* epi, unsigned long long* clock_slot = nullptr);
 int launch_gemm_bf16(cerb_ctx* c, const CUtensorMap* tmW, const ActMaps* tmX, float* out, int M, int N, int K,
                      int nsplit, int32_t* status, cudaStream_t st, unsigned long long* clock_slot = nullptr);
 int make_weight_map(CUtensorMap* out, const void* W, int N, int K);
 int make_gate_up_map(CUtensorMap* out, const void* W, int F, int K);
 int make_rotation_map(CUtensorMap* out, const void* W, int heads, int K);
+int make_gate_up_groups(CUtensorMap* out, const void* W, int F, int K, int groups);
+int make_rotation_groups(CUtensorMap* out, const void* W, int heads, int K, int groups);
 int make_act_map(ActMaps* out, const void* X, int rows_alloc, int K, int box_rows);
 int make_act_maps(ActMaps* out, const void* X, int rows_alloc, int K);
 int gemm_scratch_slots(int M, int N, int K);

@@ -425,6 +425,20 @@ int make_rotation_map(CUtensorMap* out, const void* W, int heads, int K) {
   return encode_rows_nd(out, W, K, 4, counts, strides, box);
 }
 
+// The same matrices as tiles of gemm_rows.cu: boxes of `groups` x (4 gate rows, the 4 up rows of the same features) ...
+int make_gate_up_groups(CUtensorMap* out, const void* W, int F, int K, int groups) {
+  const cuuint64_t counts[3] = {4, 2, (cuuint64_t)F / 4}, strides[3] = {1, (cuuint64_t)F, 4};
+  const cuuint32_t box[3] = {4, 2, (cuuint32_t)groups};
+  return encode_rows_nd(out, W, K, 3, counts, strides, box);
+}
+
+// ... and of `groups` heads x (4 rows of the first half of the head, the same of its second half).
+int make_rotation_groups(CUtensorMap* out, const void* W, int heads, int K, int groups) {
+  const cuuint64_t counts[3] = {64, 2, (cuuint64_t)heads}, strides[3] = {1, 64, 128};
+  const cuuint32_t box[3] = {4, 2, (cuuint32_t)groups};
+  return encode_rows_nd(out, W, K, 3, counts, strides, box);
+}
+
 int make_act_map(ActMaps* out, const void* X, int rows_alloc, int K, int box_rows) {
   return encode_2d(&out->m[box_rows / 16 - 1], X, (uint64_t)K, (uint64_t)rows_alloc, (uint64_t)K * 2, BK, (uint32_t)box_rows);
 }

@@ -1,0 +1,551 @@
+// bf16 GEMM of 9 to 256 activation rows whose outputs are finished where they are summed: gate-up with SwiGLU, QKV with RoPE and
+// cache append.
+//
+//   CG = 1:  D[128 activation rows][w weight rows] per CTA
+//   CG = 2:  D[256 activation rows][2 w weight rows] per pair of CTAs (cta_group::2), fp32, in tensor memory; one tile, all of k
+//
+// What bounds it: the weight stream up to 64 rows, then L2 on its way to the SMs.  The activation rows are the MMA's M side (rows that do not exist
+// are whatever lies behind them in shared memory; they only reach accumulator rows that nobody reads), the weight rows its N side, which comes
+// in steps of 16: so a matrix is cut into as many equal tiles as there are SMs, every output has one sum in one place, and no partial
+// sums, no exchange and no kernel behind the product are needed.  (Weights on the M side come in steps of 128 or 256 rows: 86 tiles of a
+// 22016-row matrix for 148 SMs or 74 pairs had to be cut along k.)
+//
+// Weight tile of a CTA.  Groups of eight rows, one 8 x 128-byte swizzle atom each:
+//   SwiGLU: the gate rows of four neighbouring features, then their up rows (4-D view of the matrix);
+//   RoPE (head_dim 128): elements i .. i + 3 of a head, then i + 64 .. i + 67; a tile has the same four rotations of `groups` heads, so that a
+//   thread (one activation row) keeps its angles in registers (4-D view; 16 tiles per block of heads).
+// An epilogue thread thus finds both members of every pair among its own columns.
+// A pair's MMA takes half of the activation rows and half of the weight rows from each CTA: each CTA's accumulator has its half of the
+// rows and the columns of both.  That halves the activations that each SM fetches.
+//
+// Issuers and chains.  One thread waits for a stage, issues four MMAs and commits them in 600 to 670 cycles, whatever the MMAs' size up to 160 columns
+// (80 cycles each are possible); it issues nothing while it waits, and two accumulators of its own change nothing.  Two warps that take the
+// stages in turn need 320 to 340 per stage, three 225.  Each has an accumulator of its own, or two in turn where there is room: the tensor cores
+// cut a running sum off towards zero at every step, so a sum is made of several short chains (at most as long as the partial sums were:
+// keys of the first 7B layer against float64, mean error of 64 rows 3.1e-6 with two chains of 32 k blocks, 2.5e-6 with partial sums of 21).
+// A pair's tile of more than 256 columns is two MMAs wide (and one issuer keeps the tensor cores busy: 712 cycles of 640 per stage); there is
+// room for three accumulators then, and each half of the columns goes over to another one near the middle: the first half to the third, the
+// second to the first, which the epilogue warps have taken to registers by then.
+//
+// Roles (512 threads): warp 0 = TMA producer (one lane), which fills the ring with weights ahead of the dependency wait; warps 1 to 3 = MMA
+// issuers (of a pair's first CTA); warps 4 to 15 = epilogue, three per 32 accumulator rows.
+#include <string.h>
+
+#include <type_traits>
+
+#include "tc_common.cuh"
+
+namespace cerb {
+
+namespace {
+
+constexpr int BK = 64;
+constexpr int MAX_STAGES = 18;
+constexpr int ROWS = 128;                                  // accumulator rows of a CTA
+constexpr int kSms = 148;
+constexpr int kIssuers = 3;                                // at most
+constexpr int kParts = 3;                                  // epilogue warps per 32 accumulator rows
+constexpr int kThreads = 128 + 128 * kParts;
+constexpr int COLS = 16;                                   // columns an epilogue warp takes at a time (two groups)
+constexpr int HELD = 4;                                    // blocks of columns that an epilogue thread can hold
+constexpr size_t kRing = 226 * 1024;                       // shared memory of the ring, with what the last stage's missing rows need
+
+struct RowsParams {
+  bf16* act;                // KIND 1: [M][F]
+  RopeEpilogue re;          // KIND 2
+  int32_t* status;
+  int M, F, num_kb;
+  int groups;               // groups of eight weight rows of a CTA
+  int groups0;              // ... of them in the first MMA (CG = 2; the rest in the second)
+  int x_rows;               // activation rows fetched by a CTA
+  int stages, issuers, chains;
+  int turn0, turn1;         // two MMAs: k blocks after which each goes over to its second accumulator
+  uint32_t acc_cols, tmem_cols;
+  long long wait_cycles;
+  unsigned long long* clk;
+};
+
+template <int CG>
+__device__ __forceinline__ void load_groups(uint32_t dst, const CUtensorMap* map, int x, int row, int group, uint32_t bar, uint64_t pol) {
+  if constexpr (CG == 1)
+    asm volatile(
+        "cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1, {%2, %3, %4, %5}], [%6], %7;"
+        ::"r"(dst), "l"((uint64_t)map), "r"(x), "r"(row), "r"(0), "r"(group), "r"(bar), "l"(pol)
+        : "memory");
+  else
+    asm volatile(
+        "cp.async.bulk.tensor.4d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1, {%2, %3, %4, %5}], [%6], %7;"
+        ::"r"(dst), "l"((uint64_t)map), "r"(x), "r"(row), "r"(0), "r"(group), "r"(bar), "l"(pol)
+        : "memory");
+}
+
+template <int KIND, int CG>
+__global__ void __launch_bounds__(kThreads, 1) gemm_rows_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtensorMap tmX,
+                                                                const RowsParams p) {
+  extern __shared__ uint8_t smem_raw[];
+  __shared__ __align__(8) uint64_t full_bar[MAX_STAGES];      // CG = 2: used in the pair's first CTA only
+  __shared__ __align__(8) uint64_t empty_bar[MAX_STAGES];
+  __shared__ __align__(8) uint64_t acc_full, drain_bar[kIssuers];
+  __shared__ __align__(8) uint64_t turn_full, turn_done, meet_bar;       // turn_done: first CTA only, all epilogue warps of the pair arrive
+  __shared__ uint32_t tmem_base_slot;
+  __shared__ int aborted_s, meet_flag_s;
+  volatile int* aborted = &aborted_s;
+  const WaitCtx wc{p.wait_cycles, aborted, p.status, KIND + 10 * p.num_kb + 100000 * p.M};
+
+  const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
+  const uint32_t w_bytes = (uint32_t)p.groups * 1024u;
+  const uint32_t stage_bytes = w_bytes + (uint32_t)p.x_rows * 128u;
+  const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;       // (one value per warp, as the compiler sees)
+  const int rank = CG == 2 ? (int)cluster_ctarank() : 0;
+  const bool first = rank == 0;
+  const bool two = KIND == 1 && CG == 2 && p.groups0 < p.groups;           // two MMAs per 16 k
+  // SwiGLU: consecutive groups.  RoPE: four rotations of a block of heads.
+  const int row0 = KIND == 2 ? ((int)blockIdx.x & 15) * 4 : 0;
+  const int group0 = (KIND == 2 ? (int)blockIdx.x >> 4 : (int)blockIdx.x) * p.groups;
+
+  if (threadIdx.x == 0) {
+    aborted_s = 0;
+    meet_flag_s = 0;
+    for (int s = 0; s < p.stages; ++s) {
+      mbar_init(smem_u32(&full_bar[s]), 1);
+      mbar_init(smem_u32(&empty_bar[s]), 1);
+    }
+    mbar_init(smem_u32(&acc_full), (uint32_t)p.issuers);
+    for (int i = 0; i < kIssuers; ++i) mbar_init(smem_u32(&drain_bar[i]), 1);
+    if constexpr (CG == 2) {
+      mbar_init(smem_u32(&turn_full), 1);
+      mbar_init(smem_u32(&turn_done), 2 * 4 * kParts);
+      mbar_init(smem_u32(&meet_bar), 2);
+    }
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == 1) {
+    if constexpr (CG == 1) {
+      asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base_slot)), "r"(p.tmem_cols) : "memory");
+      asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    } else {
+      asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base_slot)), "r"(p.tmem_cols) : "memory");
+      asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+    }
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  if constexpr (CG == 2) {
+    cluster_start_arrive();       // the other CTA's barriers exist before anything is signalled across
+    cluster_start_wait();
+  }
+  const uint32_t tmem_base = tmem_base_slot;
+  auto wait = [&](uint64_t& bar, uint32_t parity, int site) {
+    return CG == 2 ? mbar_wait_cluster(smem_u32(&bar), parity, wc, site) : mbar_wait(smem_u32(&bar), parity, wc, site);
+  };
+
+  if (warp == 0) {
+    if (lane == 0) {
+      const uint64_t pol_w = l2_policy(true), pol_x = l2_policy(false);
+      auto full = [&](int s) { return CG == 2 ? mapa_u32(smem_u32(&full_bar[s]), 0) : smem_u32(&full_bar[s]); };
+      auto load_w = [&](int kb, int s) {
+        if (first) mbar_expect_tx(smem_u32(&full_bar[s]), CG * stage_bytes);               // (a pair's first CTA counts both CTAs' copies)
+        load_groups<CG>(smem_base + (uint32_t)s * stage_bytes, &tmW, kb * BK, row0, group0, full(s), pol_w);
+      };
+      auto load_x = [&](int kb, int s) {
+        const uint32_t dst = smem_base + (uint32_t)s * stage_bytes + w_bytes;
+        if constexpr (CG == 2) tma_load_2d_pair(dst, &tmX, kb * BK, rank * p.x_rows, full(s), pol_x);
+        else tma_load_2d_hint(dst, &tmX, kb * BK, 0, full(s), pol_x);
+      };
+      const int pre = min(p.num_kb, p.stages);
+      for (int i = 0; i < pre; ++i) load_w(i, i);
+      asm volatile("prefetch.tensormap [%0];" ::"l"((uint64_t)&tmX) : "memory");
+      griddep_wait();
+      griddep_launch();                                    // (only now: see launch_order.cu)
+      if (p.clk) atomicMin(p.clk, globaltimer_ns());
+      for (int i = 0; i < pre; ++i) load_x(i, i);
+      int issued = pre, s = 0;
+      uint32_t ph = 0;
+      for (int i = pre; i < p.num_kb; ++i) {
+        if (!wait(empty_bar[s], ph, 241)) break;
+        load_w(i, s);
+        load_x(i, s);
+        issued = i + 1;
+        if (++s == p.stages) { s = 0; ph ^= 1u; }
+      }
+      if (*aborted) {
+        // give-up path: the copies already issued still land in this CTA's shared memory; see each of them in.  (A pair's are counted on
+        // the first CTA's barriers, and the CTAs may have stopped at different stages: both let the time of many round trips pass, too.)
+        if (first)
+          for (int i = issued > p.stages ? issued - p.stages : 0; i < issued; ++i)
+            mbar_wait_drain(smem_u32(&full_bar[i % p.stages]), (uint32_t)(i / p.stages) & 1u, CG == 2 ? 2000000ll : kDrainCycles);
+        const long long t_land = clock64();
+        while (CG == 2 && clock64() - t_land < 400000ll) __nanosleep(1000);
+      }
+    }
+  } else if (warp <= kIssuers) {
+    const int self = warp - 1;
+    if (first && self < p.issuers) {
+      bool live = true;
+      auto commit = [&](uint64_t& bar) {
+        if constexpr (CG == 2) umma_commit_pair(smem_u32(&bar));
+        else umma_commit(smem_u32(&bar));
+      };
+      auto issue = [&](int s, int groups_at, uint32_t idesc, uint32_t d, bool fresh) {
+        const uint32_t src = smem_base + (uint32_t)s * stage_bytes;
+        const uint64_t adesc = desc_k_sw128(src + w_bytes), bdesc = desc_k_sw128(src + (uint32_t)groups_at * 1024u);
+#pragma unroll
+        for (int kk = 0; kk < BK / 16; ++kk) {
+          const uint32_t acc = (!fresh || kk > 0) ? 1u : 0u;
+          if constexpr (CG == 2) umma_bf16_pair(d, adesc + (uint64_t)(kk * 2), bdesc + (uint64_t)(kk * 2), idesc, acc);
+          else umma_bf16(d, adesc + (uint64_t)(kk * 2), bdesc + (uint64_t)(kk * 2), idesc, acc);
+        }
+      };
+      if (!two) {
+        const uint32_t idesc = idesc_bf16(CG * ROWS, p.acc_cols, false, false);
+        uint32_t d = tmem_base + (uint32_t)self * p.acc_cols, other = d + (p.chains > p.issuers ? (uint32_t)p.issuers * p.acc_cols : 0u), ph = 0;
+        int s = self;
+        for (int i = self; i < p.num_kb; i += p.issuers) {
+          live = __all_sync(0xffffffffu, wait(full_bar[s], ph, 242));
+          if (!live) break;
+          tc_fence_after();
+          if (elect_one()) {
+            issue(s, 0, idesc, d, i < p.chains);
+            commit(empty_bar[s]);                              // the stage is free once the MMAs have read it
+          }
+          __syncwarp();
+          const uint32_t t = d;
+          d = other;
+          other = t;
+          if ((s += p.issuers) >= p.stages) { s = self; ph ^= 1u; }
+        }
+      } else {
+        const uint32_t n0 = 16u * (uint32_t)p.groups0, n1 = 16u * (uint32_t)p.groups - n0;
+        const uint32_t idesc0 = idesc_bf16(2 * ROWS, n0, false, false), idesc1 = idesc_bf16(2 * ROWS, n1, false, false);
+        uint32_t d0 = tmem_base, d1 = tmem_base + n0;
+        uint32_t ph = 0;
+        for (int i = 0, s = 0; i < p.num_kb; ++i) {
+          // to the second accumulators: the third one's columns; the first one's, when they have been taken from there
+          if (i == p.turn0) d0 = tmem_base + n0 + n1;
+          if (i == p.turn1) {
+            live = __all_sync(0xffffffffu, wait(turn_done, 0, 244));
+            if (!live) break;
+            d1 = tmem_base;
+          }
+          live = __all_sync(0xffffffffu, wait(full_bar[s], ph, 242));
+          if (!live) break;
+          tc_fence_after();
+          if (elect_one()) {
+            issue(s, 0, idesc0, d0, i == 0 || i == p.turn0);
+            if (i + 1 == p.turn0) commit(turn_full);
+            issue(s, p.groups0, idesc1, d1, i == 0 || i == p.turn1);
+            commit(empty_bar[s]);
+          }
+          __syncwarp();
+          if (++s == p.stages) { s = 0; ph ^= 1u; }
+        }
+      }
+      if (elect_one()) {
+        if (!live) {
+          // give-up path: the MMAs already issued still read shared memory and write tensor memory; see them retire
+          if constexpr (CG == 2)
+            asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(&drain_bar[self])) : "memory");
+          else umma_commit(smem_u32(&drain_bar[self]));
+          mbar_wait_drain(smem_u32(&drain_bar[self]), 0, CG == 2 ? 40000000ll : kDrainCycles);
+        } else {
+          commit(acc_full);
+        }
+      }
+    }
+  } else if (warp >= 4) {
+    const int quarter = warp & 3, part = (warp >> 2) - 1;
+    const int own = quarter * 32 + lane, row = rank * p.x_rows + own;
+    griddep_wait();
+    bool ok = own < p.x_rows && row < p.M;
+    float cs[CG][4], sn[CG][4];
+    size_t kv = 0;
+    if constexpr (KIND == 2) {
+      // where the row's key goes, and its rotations: on the way while the products run
+      const RopeEpilogue& e = p.re;
+      if (ok) {
+        int b, v;
+        locate_row(row, e.row_off, e.B, e.n, b, v);
+        const int len = e.len[b], pos = len + e.depth[v], slot = len + v;
+        ok = v < e.n_active[b] && pos < e.max_pos && slot < e.max_pos;
+        if (ok) {
+          kv = (size_t)e.page_table[(size_t)b * e.max_pages + slot / CERB_PAGE] * e.H * CERB_PAGE + slot % CERB_PAGE;
+#pragma unroll
+          for (int r = 0; r < CG; ++r) {
+            const float4* rot = reinterpret_cast<const float4*>(e.rope + (size_t)pos * 64 + row0 + (r - rank) * 4);
+            const float4 r0 = rot[0], r1 = rot[1];
+            cs[r][0] = r0.x; sn[r][0] = r0.y; cs[r][1] = r0.z; sn[r][1] = r0.w;
+            cs[r][2] = r1.x; sn[r][2] = r1.y; cs[r][3] = r1.z; sn[r][3] = r1.w;
+          }
+        }
+      }
+    }
+    const uint32_t lanes = tmem_base + ((uint32_t)(quarter * 32) << 16);
+    const uint32_t n0 = 16u * (uint32_t)p.groups0;
+    bool live = rank * p.x_rows + quarter * 32 < p.M && quarter * 32 < p.x_rows;      // (a warp none of whose rows exist reads no accumulator)
+    float held[CG == 2 ? HELD : 1][COLS];
+    if (CG == 2 && two) {
+      if (live) live = __all_sync(0xffffffffu, wait(turn_full, 0, 245));
+      if (live) {
+        tc_fence_after();
+#pragma unroll
+        for (int i = 0; i < HELD; ++i)
+          if ((part + i * kParts) * COLS < (int)n0) tmem_ld16_nowait(lanes + (uint32_t)((part + i * kParts) * COLS), reinterpret_cast<uint32_t*>(held[CG == 2 ? i : 0]));
+        tmem_ld_wait();
+        tc_fence_before();
+      }
+      __syncwarp();
+      if (lane == 0) mbar_arrive_cluster(mapa_u32(smem_u32(&turn_done), 0));
+    }
+    if (live && __all_sync(0xffffffffu, wait(acc_full, 0, 243))) {
+      tc_fence_after();
+      // two blocks of eight columns of all chains
+      auto load = [&](uint32_t c0, uint32_t c1, float* v) {
+        float t[COLS];
+        tmem_ld8_nowait(lanes + c0, reinterpret_cast<uint32_t*>(v));
+        tmem_ld8_nowait(lanes + c1, reinterpret_cast<uint32_t*>(v + 8));
+        auto next = [&](int chain, float* t) {
+          tmem_ld8_nowait(lanes + (uint32_t)chain * p.acc_cols + c0, reinterpret_cast<uint32_t*>(t));
+          tmem_ld8_nowait(lanes + (uint32_t)chain * p.acc_cols + c1, reinterpret_cast<uint32_t*>(t + 8));
+        };
+        float u[COLS];
+        if (p.chains > 1) next(1, t);
+        if (p.chains > 2) next(2, u);
+        tmem_ld_wait();
+#pragma unroll
+        for (int j = 0; j < COLS; ++j) v[j] += (p.chains > 1 ? t[j] : 0.f) + (p.chains > 2 ? u[j] : 0.f);
+        if (p.chains > 3) {
+          next(3, t);
+          tmem_ld_wait();
+#pragma unroll
+          for (int j = 0; j < COLS; ++j) v[j] += t[j];
+        }
+      };
+      if constexpr (KIND == 1) {
+        auto finish = [&](int c, float* v) {
+          int g[2];
+#pragma unroll
+          for (int half = 0; half < 2; ++half) {
+            int lg = 2 * c + half, r = 0;                    // the column group's place among its CTA's, and which CTA that is
+            if constexpr (CG == 2) {
+              const int base = lg < 2 * p.groups0 ? 0 : p.groups0, here = base ? p.groups - base : p.groups0;
+              lg -= 2 * base;
+              r = lg >= here ? 1 : 0;
+              lg += base - r * here;
+            }
+            g[half] = 2 * c + half < CG * p.groups ? group0 + lg + (r - rank) * p.groups : p.F;
+          }
+          uint2 o[2];
+#pragma unroll
+          for (int half = 0; half < 2; ++half) {
+            float* a = v + 8 * half;
+            float x[4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) x[j] = a[j] / (1.0f + expf(-a[j])) * a[4 + j];
+            o[half] = make_uint2(pack_bf16(x[0], x[1]), pack_bf16(x[2], x[3]));
+          }
+          if (!ok) return;
+          bf16* at = p.act + (size_t)row * p.F;
+          // (a store instruction costs the lines it touches, and every lane has a row of its own: the fewer the better)
+          if (g[1] == g[0] + 1 && !(g[0] & 1) && 4 * g[1] < p.F) {
+            *reinterpret_cast<uint4*>(at + 4 * g[0]) = make_uint4(o[0].x, o[0].y, o[1].x, o[1].y);
+          } else {
+            if (4 * g[0] < p.F) *reinterpret_cast<uint2*>(at + 4 * g[0]) = o[0];
+            if (4 * g[1] < p.F) *reinterpret_cast<uint2*>(at + 4 * g[1]) = o[1];
+          }
+        };
+        if (CG == 2 && two) {
+          const uint32_t n = 16u * (uint32_t)p.groups;
+#pragma unroll
+          for (int i = 0; i < HELD; ++i) {
+            const int c = part + i * kParts;
+            if (c * COLS < (int)n0) {
+              float v[COLS];
+              tmem_ld16_nowait(lanes + n + (uint32_t)(c * COLS), reinterpret_cast<uint32_t*>(v));
+              tmem_ld_wait();
+#pragma unroll
+              for (int j = 0; j < COLS; ++j) v[j] += held[CG == 2 ? i : 0][j];
+              finish(c, v);
+            }
+          }
+          for (int c = (int)n0 / COLS + part; c < p.groups; c += kParts) {
+            float v[COLS], t[COLS];
+            tmem_ld16_nowait(lanes + (uint32_t)(c * COLS), reinterpret_cast<uint32_t*>(v));
+            tmem_ld16_nowait(lanes + (uint32_t)(c * COLS) - n0, reinterpret_cast<uint32_t*>(t));
+            tmem_ld_wait();
+#pragma unroll
+            for (int j = 0; j < COLS; ++j) v[j] += t[j];
+            finish(c, v);
+          }
+        } else {
+          for (int c = part; 2 * c < CG * p.groups; c += kParts) {
+            float v[COLS];
+            load((uint32_t)(c * COLS), (uint32_t)(c * COLS + 8), v);
+            finish(c, v);
+          }
+        }
+      } else {
+        // a step: two heads of this CTA, or a head's rotations of both CTAs (next to each other)
+        const RopeEpilogue& e = p.re;
+        for (int c = part; CG == 2 ? c < p.groups : 2 * c < p.groups; c += kParts) {
+          float v[COLS];
+          if constexpr (CG == 2) load((uint32_t)(c * 8), (uint32_t)((p.groups + c) * 8), v);
+          else load((uint32_t)(c * COLS), (uint32_t)(c * COLS + 8), v);
+          uint2 lo[2], hi[2];
+          bf16* o[2];
+#pragma unroll
+          for (int half = 0; half < 2; ++half) {
+            const int lg = CG == 2 ? c : 2 * c + half, r = CG == 2 ? half : 0, g = group0 + lg;
+            const int which = g / e.H, h = g - which * e.H;
+            float* a = v + 8 * half;
+            float* b = a + 4;
+            if (which < 2)
+#pragma unroll
+              for (int j = 0; j < 4; ++j) {
+                const float o1 = a[j] * cs[r][j] - b[j] * sn[r][j];
+                b[j] = b[j] * cs[r][j] + a[j] * sn[r][j];
+                a[j] = o1;
+              }
+            lo[half] = make_uint2(pack_bf16(a[0], a[1]), pack_bf16(a[2], a[3]));
+            hi[half] = make_uint2(pack_bf16(b[0], b[1]), pack_bf16(b[2], b[3]));
+            o[half] = !ok || lg >= p.groups || which > 2 ? nullptr
+                      : which == 0 ? reinterpret_cast<bf16*>(e.q) + ((size_t)row * e.H + h) * 128
+                                   : reinterpret_cast<bf16*>(which == 1 ? e.kpool : e.vpool) + (kv + (size_t)h * CERB_PAGE) * 128;
+          }
+          if constexpr (CG == 2) {
+            if (o[0]) {
+              bf16* at = o[0] + (row0 & ~7);
+              *reinterpret_cast<uint4*>(at) = make_uint4(lo[0].x, lo[0].y, lo[1].x, lo[1].y);
+              *reinterpret_cast<uint4*>(at + 64) = make_uint4(hi[0].x, hi[0].y, hi[1].x, hi[1].y);
+            }
+          } else {
+#pragma unroll
+            for (int half = 0; half < 2; ++half)
+              if (o[half]) {
+                *reinterpret_cast<uint2*>(o[half] + row0) = lo[half];
+                *reinterpret_cast<uint2*>(o[half] + row0 + 64) = hi[half];
+              }
+          }
+        }
+      }
+    }
+  }
+  tc_fence_before();
+  __syncthreads();
+  if (p.clk && threadIdx.x == 0) atomicMax(p.clk + kGemmClockSlots, globaltimer_ns());
+  if constexpr (CG == 2) {
+    // Neither CTA leaves (nor frees its tensor memory) before the other is done: copies, commits and arrivals cross between them until then.
+    if (warp == 2) cluster_meet_before_exit(&meet_bar, 2, lane, wc, &meet_flag_s, 246);
+    __syncthreads();
+    if (warp == 1) asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(p.tmem_cols) : "memory");
+  } else {
+    if (warp == 1) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(p.tmem_cols) : "memory");
+  }
+}
+
+template <int KIND, int CG>
+int launch_kind(const CUtensorMap& tmW, const CUtensorMap& tmX, const RowsParams& p, int tiles, cudaStream_t st) {
+  static bool configured = false;
+  if (!configured) {
+    CERB_CUDA_OK(cudaFuncSetAttribute(gemm_rows_kernel<KIND, CG>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRing));
+    configured = true;
+  }
+  // (always the same request, more than half of an SM: one CTA there, which may own all of its tensor memory)
+  const cudaError_t e = CG == 2 ? launch_pdl_cluster(gemm_rows_kernel<KIND, CG>, dim3((tiles + 1) / 2 * 2), dim3(kThreads), kRing, st, 2u, tmW, tmX, p)
+                                : launch_pdl(gemm_rows_kernel<KIND, CG>, dim3(tiles), dim3(kThreads), kRing, st, tmW, tmX, p);
+  return e == cudaSuccess ? CERB_OK : CERB_E_CUDA;
+}
+
+}  // namespace
+
+RowsPlan plan_rows_swiglu(int F) {
+  RowsPlan g{0, 0, false};
+  const int groups = F / 4, per = (groups + kSms - 1) / kSms;
+  if (F % 4 || per < 2 || per > 32) return g;
+  g.groups = per;
+  g.tiles = (groups + per - 1) / per;
+  return g;
+}
+
+RowsPlan plan_rows_rope(int n_heads, int head_dim) {
+  RowsPlan g{0, 0, true};
+  const int heads = 3 * n_heads, per = (heads + kSms / 16 - 1) / (kSms / 16);
+  if (head_dim != 128 || per < 2 || per > 32) return g;
+  g.groups = per;
+  g.tiles = 16 * ((heads + per - 1) / per);
+  return g;
+}
+
+// A pair's tile is up to 256 columns wide in one MMA, or has room for three accumulators.
+// Which products come here, from 9 rows on.
+//   Up to 128 rows, against partial sums and kernels behind them: matrices of at least 16 rows per SM (an MMA's N is no less) and at most 256.  From
+//   more than 160 rows per SM on, the ring is 6 or 7 stages of 24 KB and more, where units of 256 weight rows put a third more weights on their
+//   way: these from 49 rows on (13B width, 9 rows 0.985 x, 40 rows 0.995 x, 64 rows 1.03 x).  RoPE from 65 rows on: below, the separate kernel and its
+//   sums of up to four slots cost little more than the epilogue (1.01 to 1.015 x).
+//   Forwards: 7B width 9 / 64 / 96 / 128 rows 1.02 / 1.02 / 1.075 / 1.10 x, 13B 64 / 96 / 128 rows 1.01 / 1.09 / 1.10 x, 3200 columns 1.02 to 1.17 x.
+//   129 to 256 rows, in pairs, against output tiles of 256 weight rows (gemm_tile.cu): a pair's tile has to fit one MMA, or (SwiGLU, 16 k
+//   blocks and more) three accumulators.  Tiles of 256 rows leave SMs idle or have to be cut along k: 7B width, 129 / 192 / 256 rows, 8 layers 1317 /
+//   1368 / 1457 -> 1224 / 1319 / 1311 us.  Where the tiles of QKV occupy more than 0.7 of the pairs, there is something to gain from 192 rows on
+//   only (13B, QKV alone: 129 rows 0.98 x, 192 1.01, 256 1.02).
+bool gemm_rows_takes(const RowsPlan& g, int M, int N, int K) {
+  if (M <= kFewRows || M > 2 * ROWS || g.tiles < 1) return false;
+  if (M <= ROWS) return g.heads ? M > 64 : g.groups <= 20 || M > 48;
+  if (g.groups > 16) return !g.heads && (g.groups + (g.groups + 1) / 2) * 16 <= 512 && K >= 16 * BK;
+  return !g.heads || M >= 192 || (N + 255) / 256 <= 0.7 * (kSms / 2);
+}
+
+int launch_gemm_rows(cerb_ctx* c, const CUtensorMap* tmW, const ActMaps* tmX, const RowsPlan& g, int M, int N, int K, int32_t* status, cudaStream_t st,
+                     const GemmEpilogue* epi, unsigned long long* clock_slot) {
+  if (!gemm_rows_takes(g, M, N, K)) return CERB_E_SHAPE;
+  const bool pairs = M > ROWS;            // (7B width, 96 and 128 rows: 1062 and 1082 us in pairs, 926 and 974 in single CTAs)
+  RowsParams p;
+  memset(&p, 0, sizeof(p));
+  p.status = status;
+  p.M = M;
+  p.F = N / 2;
+  p.num_kb = (K + BK - 1) / BK;
+  p.groups = p.groups0 = g.groups;
+  // (activation tiles of 16 or 48 rows: forwards 2 % slower than with 32 and 64)
+  p.x_rows = ((pairs ? (M + 1) / 2 : M) + 31) / 32 * 32;
+  const size_t stage = (size_t)p.groups * 1024 + (size_t)p.x_rows * 128;
+  // (the MMAs read 128 rows of the last stage, too; 1 KB for the alignment of the ring)
+  p.stages = (int)((kRing - 1024 - (size_t)(ROWS - p.x_rows) * 128) / stage);
+  if (p.stages > MAX_STAGES) p.stages = MAX_STAGES;
+  const int cols = (g.groups * 8 * (pairs ? 2 : 1) + 15) / 16 * 16;
+  if (pairs && g.groups > 16) {
+    p.groups0 = (g.groups + 1) / 2;
+    p.issuers = 1;
+    p.turn0 = p.num_kb * 30 / 64;
+    p.turn1 = p.num_kb * 34 / 64;
+    p.tmem_cols = 512;
+  } else {
+    // A stage belongs to one issuer, which waits for its phases in turn.  (Issuers that took turns at a stage could be a round apart when copies
+    // land out of order, and a parity tells neighbouring phases apart only.)  Three issuers or two where the ring loses no stage by it; one
+    // where it would and the weights of a stage take as long to come as one issuer needs.
+    p.issuers = p.stages % 3 == 0 && 3 * cols <= 512 ? 3 : p.stages % 2 == 0 ? 2 : p.groups >= 16 ? 1 : 2;
+    p.stages -= p.stages % p.issuers;
+    if (p.issuers > p.num_kb) p.issuers = p.num_kb;
+    p.chains = p.issuers < 3 && p.num_kb >= 2 * p.issuers && 2 * p.issuers * cols <= 512 ? 2 * p.issuers : p.issuers;
+    p.acc_cols = (uint32_t)cols;
+    for (p.tmem_cols = 32; p.tmem_cols < p.chains * p.acc_cols; p.tmem_cols *= 2) {}
+  }
+  p.wait_cycles = wait_cycles();
+  p.clk = clock_slot;
+  auto run = [&](auto kind, const CUtensorMap& x) {
+    constexpr int KIND = decltype(kind)::value;
+    return pairs ? launch_kind<KIND, 2>(*tmW, x, p, g.tiles, st) : launch_kind<KIND, 1>(*tmW, x, p, g.tiles, st);
+  };
+  int rc;
+  if (epi->kind == 1) {
+    p.act = (bf16*)epi->act;
+    rc = run(std::integral_constant<int, 1>(), tmX->box(p.x_rows));
+  } else {
+    p.re = *epi->rope;
+    rc = run(std::integral_constant<int, 2>(), tmX->box(p.x_rows));
+  }
+  if (rc != CERB_OK) return rc;
+  CERB_LAUNCH_CHECK(c);
+  return CERB_OK;
+}
+
+}  // namespace cerb

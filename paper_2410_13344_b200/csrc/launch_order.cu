@@ -70,10 +70,10 @@ const Entry kNormEmbed = {LO_NORM_ATTN, "row_norm (embedding, attention norm)", 
 const Entry kQkvNorm = {LO_GEMM_QKV, "gemm norm + qkv + rope / append epilogue", B_Q | B_KV, B_CONST};
 const Entry kGuNorm = {LO_GEMM_GU, "gemm norm + gate-up + swiglu epilogue", B_ACT, B_CONST};
 
-// Variant 0 is the steps of 9 to 128 rows (bf16); those with a residual add in the GEMMs occur above and up to 8 rows, the norms in
+// Variants 0, 1, 2 and 4 are the steps of 9 to 128 rows (bf16): a tile per SM finishes SwiGLU, RoPE + cache append or both, where the matrix has the size
+// for it (gemm_rows.cu).  Those with a residual add in the GEMMs occur above and up to 8 rows, the norms in
 // the GEMMs (8) with as many of those as gemm_few_normalises allows.  fp32 models take 8 or, above kF32NormMax columns, 3 as long as their
-// GEMMs have few output tiles, 0 otherwise.  1, 2 and 4 (a fusion without the residual add) are no forward's;
-// their tables stay for callers of the entry below.
+// GEMMs have few output tiles, 0 otherwise.
 constexpr int kVariants = 9;
 const Fusion kFusion[kVariants] = {  // {swiglu, rope, residual, norm}
     {false, false, false}, {true, false, false}, {true, true, false}, {true, true, true},

@@ -1,0 +1,85 @@
+"""Gate-up and QKV products of 9 to 256 rows in one tile per SM (or pair of SMs): edges of rows, of weight tiles, of k."""
+import ctypes as C
+
+import pytest
+import torch
+
+from oracle import cerberus_oracle as orc
+from paper_2410_13344_b200 import binding as cb
+from paper_2410_13344_b200 import synth
+from tests.helpers import close
+from tests.test_gpu_model import TOL, Rig
+
+pytestmark = pytest.mark.gpu
+
+# (d_model, heads, mlp_dim): weight rows per SM, k blocks
+SHAPES = {
+    "16 and 16 rows, one k block": (64, 4, 1184),                # the least of both plans
+    "16 and 24 rows, ragged k block": (200, 4, 1192),            # one feature group more than two per SM
+    "32 and 152 rows, two MMAs per pair": (1096, 10, 11000),     # odd number of groups; the last tile of SwiGLU half empty
+    "112 and 168 rows": (1024, 40, 12432),                       # the widest pair of MMAs
+}
+# prompt lengths: rows of one accumulator quarter, its edges, all of them; pairs: one row in the second CTA's half and all
+CASES = [(n, m) for n in SHAPES for m in (9, 33, 64, 65, 128, 129, 256)]
+
+
+@pytest.mark.parametrize("name,M", CASES)
+def test_prompts_match_oracle(name, M):
+    d, H, F = SHAPES[name]
+    ms = synth.ModelShape(1, d, H, 128, F, 512, "bf16")
+    rig = Rig(cb, ms, max_tokens=M + 16, max_nodes=16)
+    prompt = [int(t) for t in synth.make_prompt(ms.vocab, M, seq=140 + M)]
+    tok = torch.tensor([prompt], dtype=torch.int32, device="cuda")
+    st = orc.prefill(rig.cmodel, rig.sh, prompt, M + 16)
+    for _ in range(2):
+        before = rig.eng.launch_count()
+        rig.eng.prefill(tok, [M])
+        launches = rig.eng.launch_count() - before
+        _, _, h_last = rig.eng.read_state()
+        assert rig.eng.device_status() == 0 and rig.eng.last_forward_rows() == M
+        assert close(h_last[0], st.h_last, 0) < TOL["bf16"]
+        k, v = rig.eng.gather_kv(0, 0, M)
+        assert close(k, st.k[0][:M], 0) < TOL["bf16"] and close(v, st.v[0][:M], 0) < TOL["bf16"]
+    # live rows, first norm, the layer (seven launches, separate RoPE up to 64 rows, separate SwiGLU of wide tiles up to 48), commit, LM head, argmax
+    if M <= 128:
+        assert launches == 1 + 1 + 7 + (M <= 64) + (M <= 48 and "168" in name) + 3
+
+
+@pytest.mark.parametrize("n,live", [(40, (40, 17, 1)), (70, (1, 70, 33))])
+def test_trees_with_dead_nodes_match_oracle(n, live):
+    """Three sequences (120 and 210 rows): rows of nodes that are not live write nothing."""
+    d, H, F = SHAPES["32 and 152 rows, two MMAs per pair"]
+    ms = synth.ModelShape(1, d, H, 128, F, 512, "bf16")
+    rig = Rig(cb, ms, max_tokens=128, max_batch=3, max_nodes=n)
+    lens = [29, 16, 5]
+    prompts = [[int(t) for t in synth.make_prompt(ms.vocab, k, seq=160 + k)] for k in lens]
+    tok = torch.zeros(3, max(lens), dtype=torch.int32, device="cuda")
+    for b, p in enumerate(prompts):
+        tok[b, :len(p)] = torch.tensor(p, dtype=torch.int32)
+    rig.eng.prefill(tok, lens)
+    tree = synth.random_parent_tree(n, 4, tree_id=6, n_heads=4, kmax=1)
+    tt = torch.stack([synth.make_prompt(ms.vocab, n, seq=170 + b).to(torch.int32) for b in range(3)]).cuda().contiguous()
+    before = rig.eng.k_pool.clone()
+    hidden = rig.eng.verify(rig.eng.tree(tree), tt, n_active=torch.tensor(live, dtype=torch.int32, device="cuda"), want_hidden=True)[2]
+    assert rig.eng.device_status() == 0
+    for b in range(3):
+        st = orc.prefill(rig.cmodel, rig.sh, prompts[b], 200)
+        want, _ = orc.verify_tree(rig.cmodel, rig.sh, st, [int(t) for t in tt[b, :live[b]]], tree.parent[:live[b]])
+        assert close(hidden[b, :live[b]], want, 0) < TOL["bf16"], b
+    # cache slots written: the live nodes' only
+    changed = (rig.eng.k_pool != before).any(dim=-1).any(dim=2).sum().item()        # (page, slot) pairs with any head changed
+    assert changed <= sum(live)
+
+
+def test_launches_of_a_forward_are_the_table():
+    d, H, F = SHAPES["16 and 24 rows, ragged k block"]
+    ms = synth.ModelShape(3, d, H, 128, F, 512, "bf16")
+    for n, B, variant in ((9, 1, 1), (64, 2, 2), (65, 2, 3)):
+        rig = Rig(cb, ms, max_tokens=64, max_batch=B, max_nodes=n)
+        rig.eng.prefill(torch.zeros(B, 4, dtype=torch.int32, device="cuda"), [4] * B)
+        th = rig.eng.tree(synth.random_parent_tree(n, 4, tree_id=3, n_heads=4, kmax=1))
+        before = rig.eng.launch_count()
+        rig.eng.verify(th, torch.zeros(B, n, dtype=torch.int32, device="cuda"))
+        buf = C.create_string_buffer(1 << 14)
+        assert cb.lib().cerb_launch_order_table(variant, buf, len(buf)) == cb.OK
+        assert rig.eng.launch_count() - before == len(buf.value.decode().strip().split("\n"))
