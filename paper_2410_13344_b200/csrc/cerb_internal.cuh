@@ -134,6 +134,13 @@ struct ActMaps {
 struct RowsPlan {
   int groups, tiles;
   bool heads;               // cut by heads (RoPE)
+  int parts;                // plain sums: pieces that k is cut into, each a slot of the output
+};
+
+// ... and the plain products of up to 32, 64, 96 and 128 rows: a plan each, with the maps of all layers.
+struct RowsSums {
+  RowsPlan plan[4];
+  std::vector<CUtensorMap> map[4];
 };
 
 }  // namespace cerb
@@ -168,6 +175,7 @@ struct cerb_ctx {
   std::vector<CUtensorMap> tm_wqkv_rot, tm_wgu_pair;   // the same rows gathered for the epilogues above 128 rows
   std::vector<CUtensorMap> tm_wqkv_rows, tm_wgu_rows;  // ... and for those of gemm_rows.cu, where there is a plan
   cerb::RowsPlan rows_qkv, rows_gu;
+  cerb::RowsSums rows_wo, rows_wd, rows_lm;
   CUtensorMap tm_lm_head;
   cerb::ActMaps tm_xn, tm_attn, tm_act, tm_hidden, tm_hlast;
   std::vector<CUtensorMap> tm_kpool, tm_vpool;        // per layer
@@ -310,12 +318,14 @@ bool gemm_rows_takes(const RowsPlan& g, int M, int N, int K);
 RowsPlan plan_rows_swiglu(int F);
 RowsPlan plan_rows_rope(int n_heads, int head_dim);
 int launch_gemm_rows(cerb_ctx* c, const CUtensorMap* tmW, const ActMaps* tmX, const RowsPlan& g, int M, int N, int K, int32_t* status, cudaStream_t st,
-                     const GemmEpilogue* epi, unsigned long long* clock_slot = nullptr);
+                     const GemmEpilogue* epi, float* out = nullptr, unsigned long long* clock_slot = nullptr);
+RowsPlan plan_rows_sums(int M, int N, int K, int max_parts);
 int launch_gemm_bf16(cerb_ctx* c, const CUtensorMap* tmW, const ActMaps* tmX, float* out, int M, int N, int K,
                      int nsplit, int32_t* status, cudaStream_t st, unsigned long long* clock_slot = nullptr);
 int make_weight_map(CUtensorMap* out, const void* W, int N, int K);
 int make_gate_up_map(CUtensorMap* out, const void* W, int F, int K);
 int make_rotation_map(CUtensorMap* out, const void* W, int heads, int K);
+int make_rows_map(CUtensorMap* out, const void* W, int N, int K, int rows);
 int make_gate_up_groups(CUtensorMap* out, const void* W, int F, int K, int groups);
 int make_rotation_groups(CUtensorMap* out, const void* W, int heads, int K, int groups);
 int make_act_map(ActMaps* out, const void* X, int rows_alloc, int K, int box_rows);

@@ -425,6 +425,10 @@ int make_rotation_map(CUtensorMap* out, const void* W, int heads, int K) {
   return encode_rows_nd(out, W, K, 4, counts, strides, box);
 }
 
+int make_rows_map(CUtensorMap* out, const void* W, int N, int K, int rows) {
+  return encode_2d(out, W, (uint64_t)K, (uint64_t)N, (uint64_t)K * 2, BK, (uint32_t)rows);
+}
+
 // The same matrices as tiles of gemm_rows.cu: boxes of `groups` x (4 gate rows, the 4 up rows of the same features) ...
 int make_gate_up_groups(CUtensorMap* out, const void* W, int F, int K, int groups) {
   const cuuint64_t counts[3] = {4, 2, (cuuint64_t)F / 4}, strides[3] = {1, (cuuint64_t)F, 4};

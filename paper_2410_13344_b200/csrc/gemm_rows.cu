@@ -1,5 +1,5 @@
-// bf16 GEMM of 9 to 256 activation rows whose outputs are finished where they are summed: gate-up with SwiGLU, QKV with RoPE and
-// cache append.
+// bf16 GEMM of 9 to 256 activation rows in tiles as wide as an SM's share: gate-up with SwiGLU, QKV with RoPE and cache append, whose outputs are
+// finished where they are summed, and up to 128 rows plain sums (O, down, LM head) in few parts of k.
 //
 //   CG = 1:  D[128 activation rows][w weight rows] per CTA
 //   CG = 2:  D[256 activation rows][2 w weight rows] per pair of CTAs (cta_group::2), fp32, in tensor memory; one tile, all of k
@@ -12,6 +12,7 @@
 //
 // Weight tile of a CTA.  Groups of eight rows, one 8 x 128-byte swizzle atom each:
 //   SwiGLU: the gate rows of four neighbouring features, then their up rows (4-D view of the matrix);
+//   plain sums: neighbouring rows;
 //   RoPE (head_dim 128): elements i .. i + 3 of a head, then i + 64 .. i + 67; a tile has the same four rotations of `groups` heads, so that a
 //   thread (one activation row) keeps its angles in registers (4-D view; 16 tiles per block of heads).
 // An epilogue thread thus finds both members of every pair among its own columns.
@@ -51,6 +52,8 @@ constexpr int HELD = 4;                                    // blocks of columns 
 constexpr size_t kRing = 226 * 1024;                       // shared memory of the ring, with what the last stage's missing rows need
 
 struct RowsParams {
+  float* out;               // KIND 0: [part][M][N]
+  int N, parts;             // KIND 0: columns of the output, pieces that k is cut into
   bf16* act;                // KIND 1: [M][F]
   RopeEpilogue re;          // KIND 2
   int32_t* status;
@@ -58,6 +61,7 @@ struct RowsParams {
   int groups;               // groups of eight weight rows of a CTA
   int groups0;              // ... of them in the first MMA (CG = 2; the rest in the second)
   int x_rows;               // activation rows fetched by a CTA
+  int m_rows;               // rows of a CTA's accumulator: 128, or (CG = 1) 64, of which each warp quarter has 16
   int stages, issuers, chains;
   int turn0, turn1;         // two MMAs: k blocks after which each goes over to its second accumulator
   uint32_t acc_cols, tmem_cols;
@@ -99,9 +103,11 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_rows_kernel(const __grid_con
   const int rank = CG == 2 ? (int)cluster_ctarank() : 0;
   const bool first = rank == 0;
   const bool two = KIND == 1 && CG == 2 && p.groups0 < p.groups;           // two MMAs per 16 k
-  // SwiGLU: consecutive groups.  RoPE: four rotations of a block of heads.
+  // Consecutive groups; RoPE: four rotations of a block of heads.  Plain sums: the parts of a tile are neighbours.
   const int row0 = KIND == 2 ? ((int)blockIdx.x & 15) * 4 : 0;
-  const int group0 = (KIND == 2 ? (int)blockIdx.x >> 4 : (int)blockIdx.x) * p.groups;
+  const int tile = KIND == 2 ? (int)blockIdx.x >> 4 : KIND == 0 ? (int)blockIdx.x / p.parts : (int)blockIdx.x;
+  const int group0 = tile * p.groups, slot = KIND == 0 ? (int)blockIdx.x - tile * p.parts : 0;
+  const int kb0 = KIND == 0 ? slot * p.num_kb / p.parts : 0, num_kb = KIND == 0 ? (slot + 1) * p.num_kb / p.parts - kb0 : p.num_kb;
 
   if (threadIdx.x == 0) {
     aborted_s = 0;
@@ -146,14 +152,15 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_rows_kernel(const __grid_con
       auto full = [&](int s) { return CG == 2 ? mapa_u32(smem_u32(&full_bar[s]), 0) : smem_u32(&full_bar[s]); };
       auto load_w = [&](int kb, int s) {
         if (first) mbar_expect_tx(smem_u32(&full_bar[s]), CG * stage_bytes);               // (a pair's first CTA counts both CTAs' copies)
-        load_groups<CG>(smem_base + (uint32_t)s * stage_bytes, &tmW, kb * BK, row0, group0, full(s), pol_w);
+        if constexpr (KIND == 0) tma_load_2d_hint(smem_base + (uint32_t)s * stage_bytes, &tmW, (kb0 + kb) * BK, group0 * 8, full(s), pol_w);
+        else load_groups<CG>(smem_base + (uint32_t)s * stage_bytes, &tmW, kb * BK, row0, group0, full(s), pol_w);
       };
       auto load_x = [&](int kb, int s) {
         const uint32_t dst = smem_base + (uint32_t)s * stage_bytes + w_bytes;
         if constexpr (CG == 2) tma_load_2d_pair(dst, &tmX, kb * BK, rank * p.x_rows, full(s), pol_x);
-        else tma_load_2d_hint(dst, &tmX, kb * BK, 0, full(s), pol_x);
+        else tma_load_2d_hint(dst, &tmX, (kb0 + kb) * BK, 0, full(s), pol_x);
       };
-      const int pre = min(p.num_kb, p.stages);
+      const int pre = min(num_kb, p.stages);
       for (int i = 0; i < pre; ++i) load_w(i, i);
       asm volatile("prefetch.tensormap [%0];" ::"l"((uint64_t)&tmX) : "memory");
       griddep_wait();
@@ -162,7 +169,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_rows_kernel(const __grid_con
       for (int i = 0; i < pre; ++i) load_x(i, i);
       int issued = pre, s = 0;
       uint32_t ph = 0;
-      for (int i = pre; i < p.num_kb; ++i) {
+      for (int i = pre; i < num_kb; ++i) {
         if (!wait(empty_bar[s], ph, 241)) break;
         load_w(i, s);
         load_x(i, s);
@@ -198,10 +205,10 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_rows_kernel(const __grid_con
         }
       };
       if (!two) {
-        const uint32_t idesc = idesc_bf16(CG * ROWS, p.acc_cols, false, false);
+        const uint32_t idesc = idesc_bf16(CG * (uint32_t)p.m_rows, p.acc_cols, false, false);
         uint32_t d = tmem_base + (uint32_t)self * p.acc_cols, other = d + (p.chains > p.issuers ? (uint32_t)p.issuers * p.acc_cols : 0u), ph = 0;
         int s = self;
-        for (int i = self; i < p.num_kb; i += p.issuers) {
+        for (int i = self; i < num_kb; i += p.issuers) {
           live = __all_sync(0xffffffffu, wait(full_bar[s], ph, 242));
           if (!live) break;
           tc_fence_after();
@@ -220,7 +227,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_rows_kernel(const __grid_con
         const uint32_t idesc0 = idesc_bf16(2 * ROWS, n0, false, false), idesc1 = idesc_bf16(2 * ROWS, n1, false, false);
         uint32_t d0 = tmem_base, d1 = tmem_base + n0;
         uint32_t ph = 0;
-        for (int i = 0, s = 0; i < p.num_kb; ++i) {
+        for (int i = 0, s = 0; i < num_kb; ++i) {
           // to the second accumulators: the third one's columns; the first one's, when they have been taken from there
           if (i == p.turn0) d0 = tmem_base + n0 + n1;
           if (i == p.turn1) {
@@ -255,9 +262,9 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_rows_kernel(const __grid_con
     }
   } else if (warp >= 4) {
     const int quarter = warp & 3, part = (warp >> 2) - 1;
-    const int own = quarter * 32 + lane, row = rank * p.x_rows + own;
+    const int per_quarter = p.m_rows / 4, own = quarter * per_quarter + lane, row = rank * p.x_rows + own;
     griddep_wait();
-    bool ok = own < p.x_rows && row < p.M;
+    bool ok = lane < per_quarter && own < p.x_rows && row < p.M;
     float cs[CG][4], sn[CG][4];
     size_t kv = 0;
     if constexpr (KIND == 2) {
@@ -282,7 +289,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_rows_kernel(const __grid_con
     }
     const uint32_t lanes = tmem_base + ((uint32_t)(quarter * 32) << 16);
     const uint32_t n0 = 16u * (uint32_t)p.groups0;
-    bool live = rank * p.x_rows + quarter * 32 < p.M && quarter * 32 < p.x_rows;      // (a warp none of whose rows exist reads no accumulator)
+    bool live = rank * p.x_rows + quarter * per_quarter < p.M && quarter * per_quarter < p.x_rows;      // (a warp none of whose rows exist reads no accumulator)
     float held[CG == 2 ? HELD : 1][COLS];
     if (CG == 2 && two) {
       if (live) live = __all_sync(0xffffffffu, wait(turn_full, 0, 245));
@@ -384,6 +391,23 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_rows_kernel(const __grid_con
             finish(c, v);
           }
         }
+      } else if constexpr (KIND == 0) {
+        for (int c = part; 2 * c < p.groups; c += kParts) {
+          float v[COLS];
+          load((uint32_t)(c * COLS), (uint32_t)(c * COLS + 8), v);
+          const int n = group0 * 8 + c * COLS, cols = min(2 * c + 2 <= p.groups ? 16 : 8, p.N - n);
+          float* o = p.out + ((size_t)slot * p.M + row) * p.N + n;
+          if (!ok) continue;
+          if (!(p.N & 3)) {
+#pragma unroll
+            for (int j = 0; j < COLS; j += 4)
+              if (j < cols) *reinterpret_cast<float4*>(o + j) = make_float4(v[j], v[j + 1], v[j + 2], v[j + 3]);
+          } else {
+#pragma unroll
+            for (int j = 0; j < COLS; ++j)
+              if (j < cols) o[j] = v[j];
+          }
+        }
       } else {
         // a step: two heads of this CTA, or a head's rotations of both CTAs (next to each other)
         const RopeEpilogue& e = p.re;
@@ -459,7 +483,7 @@ int launch_kind(const CUtensorMap& tmW, const CUtensorMap& tmX, const RowsParams
 }  // namespace
 
 RowsPlan plan_rows_swiglu(int F) {
-  RowsPlan g{0, 0, false};
+  RowsPlan g{0, 0, false, 0};
   const int groups = F / 4, per = (groups + kSms - 1) / kSms;
   if (F % 4 || per < 2 || per > 32) return g;
   g.groups = per;
@@ -468,7 +492,7 @@ RowsPlan plan_rows_swiglu(int F) {
 }
 
 RowsPlan plan_rows_rope(int n_heads, int head_dim) {
-  RowsPlan g{0, 0, true};
+  RowsPlan g{0, 0, true, 0};
   const int heads = 3 * n_heads, per = (heads + kSms / 16 - 1) / (kSms / 16);
   if (head_dim != 128 || per < 2 || per > 32) return g;
   g.groups = per;
@@ -478,25 +502,47 @@ RowsPlan plan_rows_rope(int n_heads, int head_dim) {
 
 // A pair's tile is up to 256 columns wide in one MMA, or has room for three accumulators.
 // Which products come here, from 9 rows on.
-//   Up to 128 rows, against partial sums and kernels behind them: matrices of at least 16 rows per SM (an MMA's N is no less) and at most 256.  From
-//   more than 160 rows per SM on, the ring is 6 or 7 stages of 24 KB and more, where units of 256 weight rows put a third more weights on their
-//   way: these from 49 rows on (13B width, 9 rows 0.985 x, 40 rows 0.995 x, 64 rows 1.03 x).  RoPE from 65 rows on: below, the separate kernel and its
-//   sums of up to four slots cost little more than the epilogue (1.01 to 1.015 x).
-//   Forwards: 7B width 9 / 64 / 96 / 128 rows 1.02 / 1.02 / 1.075 / 1.10 x, 13B 64 / 96 / 128 rows 1.01 / 1.09 / 1.10 x, 3200 columns 1.02 to 1.17 x.
+//   Up to 128 rows, against partial sums and kernels behind them: matrices of at least 16 rows per SM (an MMA's N is no less) and at most 256.
+//   Forwards, plain sums (below) included: 7B width 9 / 64 / 128 rows 1.06 / 1.06 / 1.12 x, 13B 1.02 / 1.09 / 1.13 x, 1024 to 3200 columns 1.04 to 1.25 x.
 //   129 to 256 rows, in pairs, against output tiles of 256 weight rows (gemm_tile.cu): a pair's tile has to fit one MMA, or (SwiGLU, 16 k
 //   blocks and more) three accumulators.  Tiles of 256 rows leave SMs idle or have to be cut along k: 7B width, 129 / 192 / 256 rows, 8 layers 1317 /
 //   1368 / 1457 -> 1224 / 1319 / 1311 us.  Where the tiles of QKV occupy more than 0.7 of the pairs, there is something to gain from 192 rows on
 //   only (13B, QKV alone: 129 rows 0.98 x, 192 1.01, 256 1.02).
 bool gemm_rows_takes(const RowsPlan& g, int M, int N, int K) {
   if (M <= kFewRows || M > 2 * ROWS || g.tiles < 1) return false;
-  if (M <= ROWS) return g.heads ? M > 64 : g.groups <= 20 || M > 48;
+  if (M <= ROWS) return true;
   if (g.groups > 16) return !g.heads && (g.groups + (g.groups + 1) / 2) * 16 <= 512 && K >= 16 * BK;
   return !g.heads || M >= 192 || (N + 255) / 256 <= 0.7 * (kSms / 2);
 }
 
+// Plain sums of up to 128 rows (O, down, LM head): k is cut into parts, each a sum of its own (a slot) for the kernel behind to add, so that tiles are wide
+// enough.  A CTA takes in its weights (8 x groups rows) at 44 bytes a ns, its share of the HBM rate, and everything, activations included, at
+// 85; a k block takes 0.34 us, however narrow the tile.  7B width, 64 rows, 8 layers: down in 2 / 4 / 5 / 8 parts 872 / 847 / 845 / 859 us, O in 4 / 5 / 8
+// 847 / 845 / 856.  (Units of 256 weight rows left ten slots after both, 10 MB that the norm read back; slots of the same plan, 64 rows: norm 4.65 ->
+// 4.0 us, O 9.8 -> 8.8, down 17.6 -> 16.5.)
+RowsPlan plan_rows_sums(int M, int N, int K, int max_parts) {
+  RowsPlan best{0, 0, false, 0};
+  double best_t = 0;
+  const int groups = (N + 7) / 8, num_kb = (K + BK - 1) / BK, x = (M + 31) / 32 * 32 / 8;
+  if (M <= kFewRows || M > ROWS) return best;
+  for (int parts = 1; parts <= max_parts && parts <= 8 && parts * 4 <= num_kb; ++parts) {
+    const int tiles = kSms / parts, per = (groups + tiles - 1) / tiles;
+    if (per > 32 || per < 2) continue;
+    const double kb = (num_kb + parts - 1) / parts;
+    const double hbm = kb * per / 44.0, sm = kb * (per + x) / 85.0;
+    const double least = kb * 0.34;                      // a stage's copies, waits and MMAs
+    const double in = hbm > sm ? hbm : sm, t = (in > least ? in : least) + parts * (0.05 + 0.001 * M);
+    if (!best_t || t < best_t) {
+      best_t = t;
+      best = RowsPlan{per, (groups + per - 1) / per * parts, false, parts};
+    }
+  }
+  return best;
+}
+
 int launch_gemm_rows(cerb_ctx* c, const CUtensorMap* tmW, const ActMaps* tmX, const RowsPlan& g, int M, int N, int K, int32_t* status, cudaStream_t st,
-                     const GemmEpilogue* epi, unsigned long long* clock_slot) {
-  if (!gemm_rows_takes(g, M, N, K)) return CERB_E_SHAPE;
+                     const GemmEpilogue* epi, float* out, unsigned long long* clock_slot) {
+  if (epi ? !gemm_rows_takes(g, M, N, K) : M < 1 || M > ROWS || g.parts < 1) return CERB_E_SHAPE;
   const bool pairs = M > ROWS;            // (7B width, 96 and 128 rows: 1062 and 1082 us in pairs, 926 and 974 in single CTAs)
   RowsParams p;
   memset(&p, 0, sizeof(p));
@@ -504,14 +550,21 @@ int launch_gemm_rows(cerb_ctx* c, const CUtensorMap* tmW, const ActMaps* tmX, co
   p.M = M;
   p.F = N / 2;
   p.num_kb = (K + BK - 1) / BK;
+  p.out = out;
+  p.N = N;
+  p.parts = g.parts;
+  const int least_kb = epi ? p.num_kb : p.num_kb / g.parts;
   p.groups = p.groups0 = g.groups;
   // (activation tiles of 16 or 48 rows: forwards 2 % slower than with 32 and 64)
   p.x_rows = ((pairs ? (M + 1) / 2 : M) + 31) / 32 * 32;
   const size_t stage = (size_t)p.groups * 1024 + (size_t)p.x_rows * 128;
-  // (the MMAs read 128 rows of the last stage, too; 1 KB for the alignment of the ring)
-  p.stages = (int)((kRing - 1024 - (size_t)(ROWS - p.x_rows) * 128) / stage);
+  // Up to 64 rows: MMAs of 64 rows.  A stream of weights at the HBM rate and half-empty MMAs run into the power limit together: 64-node forwards of the 7B
+  // shape, one after the other, 3511 us with MMAs of 128 rows and 3358 with 64; the first ones on an idle GPU take 3280 either way.
+  p.m_rows = !pairs && M <= 64 ? 64 : ROWS;
+  // (the MMAs read all rows of the last stage, too; 1 KB for the alignment of the ring)
+  p.stages = (int)((kRing - 1024 - (size_t)(p.m_rows - p.x_rows) * 128) / stage);
   if (p.stages > MAX_STAGES) p.stages = MAX_STAGES;
-  const int cols = (g.groups * 8 * (pairs ? 2 : 1) + 15) / 16 * 16;
+  const int step = p.m_rows == 64 ? 8 : 16, cols = (g.groups * 8 * (pairs ? 2 : 1) + step - 1) / step * step;
   if (pairs && g.groups > 16) {
     p.groups0 = (g.groups + 1) / 2;
     p.issuers = 1;
@@ -524,8 +577,8 @@ int launch_gemm_rows(cerb_ctx* c, const CUtensorMap* tmW, const ActMaps* tmX, co
     // where it would and the weights of a stage take as long to come as one issuer needs.
     p.issuers = p.stages % 3 == 0 && 3 * cols <= 512 ? 3 : p.stages % 2 == 0 ? 2 : p.groups >= 16 ? 1 : 2;
     p.stages -= p.stages % p.issuers;
-    if (p.issuers > p.num_kb) p.issuers = p.num_kb;
-    p.chains = p.issuers < 3 && p.num_kb >= 2 * p.issuers && 2 * p.issuers * cols <= 512 ? 2 * p.issuers : p.issuers;
+    if (p.issuers > least_kb) p.issuers = least_kb;
+    p.chains = p.issuers < 3 && least_kb >= 2 * p.issuers && 2 * p.issuers * cols <= 512 ? 2 * p.issuers : p.issuers;
     p.acc_cols = (uint32_t)cols;
     for (p.tmem_cols = 32; p.tmem_cols < p.chains * p.acc_cols; p.tmem_cols *= 2) {}
   }
@@ -536,7 +589,9 @@ int launch_gemm_rows(cerb_ctx* c, const CUtensorMap* tmW, const ActMaps* tmX, co
     return pairs ? launch_kind<KIND, 2>(*tmW, x, p, g.tiles, st) : launch_kind<KIND, 1>(*tmW, x, p, g.tiles, st);
   };
   int rc;
-  if (epi->kind == 1) {
+  if (!epi) {
+    rc = launch_kind<0, 1>(*tmW, tmX->box(p.x_rows), p, g.tiles, st);
+  } else if (epi->kind == 1) {
     p.act = (bf16*)epi->act;
     rc = run(std::integral_constant<int, 1>(), tmX->box(p.x_rows));
   } else {

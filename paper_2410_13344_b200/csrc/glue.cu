@@ -60,23 +60,21 @@ template <> __device__ __forceinline__ void st4<bf16>(bf16* p, const float* f) {
   *reinterpret_cast<uint2*>(p) = v;
 }
 // sum += p[s * stride] over all s, in index order: up to AHEAD slots are requested before the first is added.  (Left to the
-// compiler's unrolling by four, the three slots of a gate-up product, or the last two of ten of a down product, were a round trip to
-// L2 each.  64 rows of a 4096-wide model, behind the kernel in front: norm 6.1 -> 4.7 us, RoPE 5.5 -> 4.5, SwiGLU 4.8 -> 3.7; what is
-// left is 10 to 17 MB through the L2 and the launch itself.  A spilled register costs more than a round trip gains.)  p is the same for all threads of a block, so that only `col` (in floats) takes registers.
-// EXACT: there are AHEAD of them.
-template <int AHEAD, bool EXACT = false, int COLS>
+// compiler's unrolling by four, slots beyond a multiple of four were a round trip to L2 each.  64 rows of a 4096-wide model, behind the kernel in front:
+// norm of ten slots 6.1 -> 4.7 us, of five 4.0.  A spilled register costs more than a round trip gains.)  p is the same for all threads of a block, so that only `col` (in floats) takes registers.
+template <int AHEAD, int COLS>
 __device__ __forceinline__ void add_slots(float4 (&sum)[COLS], const float* p, const uint32_t (&col)[COLS], int nsplit, size_t stride) {
 #pragma unroll 1
-  for (int s0 = 0; EXACT ? s0 == 0 : s0 < nsplit; s0 += AHEAD) {
+  for (int s0 = 0; s0 < nsplit; s0 += AHEAD) {
     float4 t[AHEAD][COLS];
 #pragma unroll
     for (int u = 0; u < AHEAD; ++u, p += stride)
-      if (EXACT || s0 + u < nsplit)
+      if (s0 + u < nsplit)
 #pragma unroll
         for (int c = 0; c < COLS; ++c) t[u][c] = *reinterpret_cast<const float4*>(p + col[c]);
 #pragma unroll
     for (int u = 0; u < AHEAD; ++u)
-      if (EXACT || s0 + u < nsplit)
+      if (s0 + u < nsplit)
 #pragma unroll
         for (int c = 0; c < COLS; ++c) { sum[c].x += t[u][c].x; sum[c].y += t[u][c].y; sum[c].z += t[u][c].z; sum[c].w += t[u][c].w; }
   }
@@ -85,12 +83,11 @@ __device__ __forceinline__ void add_slots(float4 (&sum)[COLS], const float* p, c
 //   x <- (embedding row | x | x + sum of GEMM partial slots), kept in fp32 (the residual stream is never rounded);
 //   out <- RMSNorm(x) * gain, in the model's storage type.
 // Fusing the residual add (and the first layer's embedding gather) with the norm that always follows
-// it halves the element-wise launches.  Of up to 4096 columns, all of up to eleven slots of a thread's columns are on their way at once
-// (ten after a 4096-column product of 64 rows); up to 8192 columns eight at a time, above that two.  The sums of the warps are read back
-// four at a time.
+// it halves the element-wise launches.  Of up to 8192 columns, all of up to eight slots of a thread's columns are on their way at once
+// (four or five after a product of 64 rows), above that two.  The sums of the warps are read back four at a time.
 constexpr int NORM_THREADS = 1024;
 constexpr int NORM_MAX_ITER = 4;          // d_model up to 16384
-template <typename T, int ITER, int AHEAD, bool EXACT>
+template <typename T, int ITER, int AHEAD>
 __global__ void __launch_bounds__(NORM_THREADS, 1) fused_norm_kernel(float* __restrict__ x, const float* part, int nsplit,
                                                                    size_t split_stride, const T* __restrict__ embed,
                                                                    const int32_t* tok, int tok_stride, int tok_off,
@@ -135,7 +132,7 @@ __global__ void __launch_bounds__(NORM_THREADS, 1) fused_norm_kernel(float* __re
       }
       if (nsplit > 0) {
         float4 sum[1] = {make_float4(0.f, 0.f, 0.f, 0.f)};
-        add_slots<AHEAD, EXACT>(sum, part + (size_t)row * d, {(uint32_t)j}, nsplit, split_stride);
+        add_slots<AHEAD>(sum, part + (size_t)row * d, {(uint32_t)j}, nsplit, split_stride);
         const float4 a = sum[0];
         v[0] += a.x; v[1] += a.y; v[2] += a.z; v[3] += a.w;
       }
@@ -430,19 +427,13 @@ int launch_fused_norm(cerb_ctx* c, const float* part, int nsplit, size_t split_s
                  tok ? (const T*)c->embed : (const T*)nullptr, tok, tok_stride, tok_off, (const int32_t*)c->d_nactive, n, g.vocab,
                  (const T*)gain, (T*)out, d, g.rms_eps, row_off, c->B);
     };
-    // Up to 4096 columns: up to eight slots are one trip to L2; nine to eleven (O products of 2560 to 4096 columns, down products of 1024 and
-    // 4096) are with code for just that many, whose tests would cost spills; 12 to 19 (2048 to 3200 columns) take two trips and three.
-    // Wider rows have at most nine slots.  Whole forwards of 64 rows against four slots at a time, unrolled by the compiler: 1024 columns
-    // 1.08 x, 2048 to 3200 1.05 x, 4096 1.055 x, 5120 1.03 x, 8192 1.01 x, 12288 1.00 to 1.015 x (with all sums of slots).
+    // A product leaves at most eight slots: of up to 8192 columns they are one trip to L2; wider rows take two at a time.
     const bool one = d <= NORM_THREADS * 4;
-    if (c->bf16 && one && nsplit == 9) go(fused_norm_kernel<bf16, 1, 9, true>, bf16());
-    else if (c->bf16 && one && nsplit == 10) go(fused_norm_kernel<bf16, 1, 10, true>, bf16());
-    else if (c->bf16 && one && nsplit == 11) go(fused_norm_kernel<bf16, 1, 11, true>, bf16());
-    else if (c->bf16 && one) go(fused_norm_kernel<bf16, 1, 8, false>, bf16());
-    else if (c->bf16 && d <= NORM_THREADS * 8) go(fused_norm_kernel<bf16, 2, 8, false>, bf16());
-    else if (c->bf16) go(fused_norm_kernel<bf16, NORM_MAX_ITER, 2, false>, bf16());
-    else if (one) go(fused_norm_kernel<float, 1, 8, false>, float());
-    else go(fused_norm_kernel<float, NORM_MAX_ITER, 2, false>, float());
+    if (c->bf16 && one) go(fused_norm_kernel<bf16, 1, 8>, bf16());
+    else if (c->bf16 && d <= NORM_THREADS * 8) go(fused_norm_kernel<bf16, 2, 8>, bf16());
+    else if (c->bf16) go(fused_norm_kernel<bf16, NORM_MAX_ITER, 2>, bf16());
+    else if (one) go(fused_norm_kernel<float, 1, 8>, float());
+    else go(fused_norm_kernel<float, NORM_MAX_ITER, 2>, float());
   }
   CERB_LAUNCH_CHECK(c);
   return CERB_OK;
