@@ -90,6 +90,9 @@ struct AttnParams {
   long long wait_cycles;    // budget of every bounded wait, SM clock cycles
   int cluster;              // tensor-core path: the splits of a (sequence, head) form one cluster and merge through shared memory
   float scale_log2;
+  int items, item0;         // tensor-core kernels, PART: the launch's (sequence or window, head) items, and the first of them
+  int follows;              // ... the launch in front is of the same call: it writes nothing that this one reads and reads nothing that this one
+                            // writes.  What that one waited for is complete, so this one waits (and lets its own dependents go) only at its end.
 };
 
 // Which sequence, and which window of 128 query rows of it, z (blockIdx.z in most kernels) stands for.  A prefill chunk is one long
@@ -525,6 +528,7 @@ __device__ __forceinline__ void umma(uint32_t tmem_d, uint64_t adesc, uint64_t b
   umma_bf16(tmem_d, adesc, bdesc, idesc, acc);
 }
 
+template <bool PART>
 __global__ void __launch_bounds__(TC_THREADS, 1) tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmK,
                                                                      const __grid_constant__ CUtensorMap tmV, const AttnParams p) {
   constexpr int DH = TC_DH, ROWF = TC_ROWF;
@@ -555,7 +559,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tree_attn_tc_kernel(const __gri
   // next item's first tiles arrive during this one's end.  (A CTA's beginning and end took 14 of the 25 us of an item of ten
   // tiles: batch 16 x 128 nodes x 512 keys 86 -> 62 us; the 2048-token prefill's windows 108 -> 79 us per layer.)
   const bool many = p.nsplit == 1;
-  const int items = p.Bw * p.H, ctas = many ? (int)gridDim.x : 1, rounds = many ? (items + ctas - 1) / ctas : 1;
+  const int items = PART ? p.items : p.Bw * p.H, ctas = many ? (int)gridDim.x : 1, rounds = many ? (items + ctas - 1) / ctas : 1;
   const int split = many ? 0 : (int)blockIdx.x;
   struct Item {
     int h, b, L_old, L, nq, kv_total, t0, T, z;
@@ -564,10 +568,11 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tree_attn_tc_kernel(const __gri
   };
   auto item_at = [&](int round) {
     Item it;
-    int idx = many ? round * ctas + ((round & 1) ? ctas - 1 - (int)blockIdx.x : (int)blockIdx.x) : (int)(blockIdx.z * p.H + blockIdx.y);
+    int idx = many ? round * ctas + ((round & 1) ? ctas - 1 - (int)blockIdx.x : (int)blockIdx.x) : PART ? (int)blockIdx.y : (int)(blockIdx.z * p.H + blockIdx.y);
     it.nq = 0;
     it.T = 0;
     if (idx >= items) return it;
+    if (PART) idx += p.item0;
     it.h = idx % p.H;
     it.z = idx / p.H;
     int shift;
@@ -589,6 +594,11 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tree_attn_tc_kernel(const __gri
     griddep_wait();
     return;
   }
+  auto enter = [&]() {                                            // (see AttnParams::follows)
+    if (PART && p.follows) return;
+    griddep_wait();
+    griddep_launch();
+  };
 
   if (threadIdx.x == 0) {
     aborted_s = (*p.status != 0);
@@ -654,7 +664,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tree_attn_tc_kernel(const __gri
       __syncwarp();
       for (int i = 0; i < it.T; ++i) {
         // tiles of the first ring that lie wholly inside the prefix may be fetched before the wait
-        if (!waited && (issued == ring || (it.t0 + i + 1) * TILE > it.L_old)) { griddep_wait(); griddep_launch(); waited = true; }
+        if (!waited && (issued == ring || (it.t0 + i + 1) * TILE > it.L_old)) { enter(); waited = true; }
         const uint32_t fb = smem_u32(&full[slot]);
         int stop = 0;
         if (lane == 0) {
@@ -676,11 +686,9 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tree_attn_tc_kernel(const __gri
       for (int j = issued > ring ? issued - ring : 0; j < issued; ++j)
         mbar_wait_drain(smem_u32(&full[j % ring]), (uint32_t)(j / ring) & 1u, 20000000ll);
     }
-    griddep_wait();      // (a lane that has waited already returns at once)
-    griddep_launch();
+    enter();             // (a lane that has waited already returns at once)
   } else if (warp == 1) {
-    griddep_wait();
-    griddep_launch();
+    enter();
     // ---------------- QK^T issuer ----------------
     // (issuing one tcgen05.mma costs this thread ~95 cycles whatever its size, measured, so the two
     // products are issued by two different warps)
@@ -721,8 +729,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tree_attn_tc_kernel(const __gri
       }
     }
   } else if (warp == 10) {
-    griddep_wait();
-    griddep_launch();
+    enter();
     // ---------------- PV issuer ----------------
     {
       // B operand (V) is MN-major, N = 128 (two 64-wide swizzle atoms, p.v_lbo bytes apart)
@@ -767,8 +774,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tree_attn_tc_kernel(const __gri
     const uint32_t lane_base = (uint32_t)((warp & 3) * 32) << 16;
     const int st = (int)threadIdx.x - 64;
     const float LN2 = 0.6931471805599453f;
-    griddep_wait();
-    griddep_launch();
+    enter();
     int nv = 0;                                                // V tiles of the rounds before
     uint32_t n = 0;                                            // tiles this group has taken in all
     for (int round = 0; round < rounds; ++round) {
@@ -1077,6 +1083,10 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tree_attn_tc_kernel(const __gri
       if (warp == 2) cluster_meet_before_exit(&cl_bar[1], p.nsplit, lane, wc, &exit_flag_s, 319);
     }
   }
+  if (PART && p.follows) {
+    griddep_wait();
+    griddep_launch();
+  }
   tc_fence_before();
   __syncthreads();                             // nobody exits before warp 2 has seen every member done
   if (warp == 1) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512u) : "memory");
@@ -1368,16 +1378,64 @@ int plan_nsplit(int B, int H, int n, int max_len, int target_ctas, bool one_wave
   return (tiles + per - 1) / per;
 }
 
+// How many clusters of `size` CTAs of a kernel the GPU holds at once.  A cluster lives in one GPC, so this is less than the CTAs that fit divided by
+// the size: of one CTA to an SM 16 clusters of eight, and fewer than 20 of seven or 24 of six.
+template <auto KERNEL>
+int clusters_at_once(int threads, size_t smem, int size, int per_sm) {
+  static int known[9];                           // (per kernel; every call would store the same)
+  if (size < 2 || size > 8) return 148 * per_sm / (size < 1 ? 1 : size);
+  if (!known[size]) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(size);
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = (unsigned)size;
+    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    int n = 0;
+    if (cudaOccupancyMaxActiveClusters(&n, KERNEL, &cfg) != cudaSuccess) {
+      cudaGetLastError();
+      n = 148 * per_sm / size;
+    }
+    known[size] = n < 1 ? 1 : n;
+  }
+  return known[size];
+}
+
+// The most splits, `want` at most, whose clusters are all there at once (those of a second round cost a whole round: 24 heads of 4000 keys and 64
+// nodes in six splits 29.8 us, in four 18.4; 48 heads of 700 keys in three 21.0, in two 12.0).
+template <typename Fits>
+int splits_at_once(int tiles, int want, int items, Fits fits) {
+  for (int s = want; s > 1; --s) {
+    const int per = (tiles + s - 1) / s, n = (tiles + per - 1) / per;
+    if (n > 1 && items <= fits(n)) return n;
+  }
+  return 1;
+}
+
 inline int nq_pad(int n) { return n <= 16 ? 16 : n <= 32 ? 32 : n <= 64 ? 64 : 128; }
 
 template <int DH, int WQ, int WK, int STAGES>
-int launch_cfg(const AttnParams& p, const CUtensorMap* tmK, const CUtensorMap* tmV, int B, cudaStream_t st) {
+int launch_cfg(AttnParams p, const CUtensorMap* tmK, const CUtensorMap* tmV, int B, int max_len, cudaStream_t st) {
+  const int planned = p.nsplit;
   constexpr size_t smem = (size_t)STAGES * 2 * (DH / 64) * TILE * 128 + 1024;
   static bool configured = false;
   if (!configured) {
     CERB_CUDA_OK(cudaFuncSetAttribute(tree_attn_bf16_kernel<DH, WQ, WK, STAGES>,
                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     configured = true;
+  }
+  if (p.cluster) {
+    const int tiles = (max_len + TILE - 1) / TILE;
+    p.nsplit = splits_at_once(tiles, p.nsplit, B * p.H, [&](int n) {
+      return clusters_at_once<tree_attn_bf16_kernel<DH, WQ, WK, STAGES>>((WQ * WK + 1) * 32, smem, n, WQ == 1 ? 2 : 1);
+    });
+    // (fewer splits are longer ones)
+    if ((tiles + p.nsplit - 1) / p.nsplit * PAGES_PER_TILE > kMaxPagesPerCta) p.nsplit = planned;
+    p.cluster = p.nsplit > 1 ? 1 : 0;
   }
   dim3 grid(p.nsplit, p.H, B);
   if (p.cluster)
@@ -1405,10 +1463,12 @@ static int attn_max_split() { return attn_use_cluster() ? 8 : kMaxSplit; }
 
 // One launch of the bf16 kernels over query rows row0 .. row0 + rows - 1 (rows <= 128) of every sequence's tree.
 // A prefill chunk: `rows` is 128 and the launch covers its windows win0 .. win0 + win - 1 of every sequence side by side.
-static int launch_attn_window(const cerb_attn_args* a, int row0, int rows, const CUtensorMap* tmK, const CUtensorMap* tmV,
+static int launch_attn_window(cerb_ctx* c, const cerb_attn_args* a, int row0, int rows, const CUtensorMap* tmK, const CUtensorMap* tmV,
                               int32_t* status, cudaStream_t st, const int32_t* row_off, int win = 1, int win0 = 0) {
   AttnParams p;
   const int Bw = a->B * win;             // (sequence, window) pairs
+  p.items = Bw * a->n_heads;
+  p.item0 = p.follows = 0;
   p.B = a->B;
   p.Bw = Bw;
   p.win = win;
@@ -1443,7 +1503,7 @@ static int launch_attn_window(const cerb_attn_args* a, int row0, int rows, const
   // CTAs that fit at once: one per SM for the tensor-core kernel and for the warp-MMA layouts of 32 rows and more
   // (288 threads x 168 registers), two per SM for the 16-row layout (160 threads); the grid is planned to fit one wave
   const int resident = (tensor_path || np_ > 16) ? 148 : kTargetCtas;
-  p.nsplit = plan_nsplit(Bw, a->n_heads, nq_pad(rows), a->max_len, resident, true, attn_max_split());
+  p.nsplit = plan_nsplit(Bw, a->n_heads, np_, a->max_len, resident, true, attn_max_split());
   if (p.nsplit < 1) return CERB_E_SHAPE;
   p.oob_row = a->n_pool_pages * a->n_heads * CERB_PAGE;
   p.scale_log2 = a->scale * 1.4426950408889634f;
@@ -1466,7 +1526,11 @@ static int launch_attn_window(const cerb_attn_args* a, int row0, int rows, const
     int want = 2 * 148 / (a->B * a->n_heads);
     const int pages = (a->max_len + CERB_PAGE - 1) / CERB_PAGE;
     if (want > (pages + ONE_WARPS - 1) / ONE_WARPS) want = (pages + ONE_WARPS - 1) / ONE_WARPS;
-    p.nsplit = want < 1 ? 1 : want > 8 ? 8 : want;
+    want = want < 1 ? 1 : want > 8 ? 8 : want;
+    while (want > 1 && a->B * a->n_heads > (a->head_dim == 128 ? clusters_at_once<tree_attn_one_kernel<128>>(ONE_WARPS * 32, 0, want, 2)
+                                                                : clusters_at_once<tree_attn_one_kernel<64>>(ONE_WARPS * 32, 0, want, 2)))
+      --want;
+    p.nsplit = want;
     auto kern = a->head_dim == 128 ? tree_attn_one_kernel<128> : tree_attn_one_kernel<64>;
     const dim3 grid(p.nsplit, p.H, Bw), block(ONE_WARPS * 32);
     const bf16 *kp = (const bf16*)a->k_pool, *vp = (const bf16*)a->v_pool;
@@ -1474,53 +1538,83 @@ static int launch_attn_window(const cerb_attn_args* a, int row0, int rows, const
     return launch_pdl(kern, grid, block, 0, st, p, kp, vp) == cudaSuccess ? CERB_OK : CERB_E_CUDA;
   }
   const bool kt_path = a->head_dim == 128 && force_tc < 0 && rows <= 64 && (force_kt < 0 ? rows > 16 : force_kt != 0);
-  if (kt_path) {
-    const int tiles = (a->max_len + KT_TILE - 1) / KT_TILE;
-    int want = 148 / (Bw * a->n_heads);
-    if (want > attn_max_split()) want = attn_max_split();
-    if (want > tiles) want = tiles;
-    if (want < 1) want = 1;
-    const int per = (tiles + want - 1) / want;
-    if (per * KT_PAGES > kMaxPagesPerCta) return CERB_E_SHAPE;
-    p.nsplit = (tiles + per - 1) / per;
-    p.cluster = (use_cluster && p.nsplit >= 2 && p.nsplit <= 8) ? 1 : 0;
-    static bool kt_configured = false;
-    if (!kt_configured) {
-      CERB_CUDA_OK(cudaFuncSetAttribute(tree_attn_kt_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)KT_SMEM));
-      kt_configured = true;
-    }
-    auto kern = tree_attn_kt_kernel;
-    const dim3 grid(p.nsplit, p.H, Bw), block(KT_THREADS);
-    if (p.cluster)
-      rc = launch_pdl_cluster(kern, grid, block, KT_SMEM, st, (unsigned)p.nsplit, *tmK, *tmV, p) == cudaSuccess ? CERB_OK : CERB_E_CUDA;
-    else
-      rc = launch_pdl(kern, grid, block, KT_SMEM, st, *tmK, *tmV, p) == cudaSuccess ? CERB_OK : CERB_E_CUDA;
-  } else if (tensor_path) {
+  if (kt_path || tensor_path) {
     static bool configured = false;
     if (!configured) {
-      CERB_CUDA_OK(cudaFuncSetAttribute(tree_attn_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TC_SMEM));
+      for (auto kern : {tree_attn_kt_kernel<false>, tree_attn_kt_kernel<true>})
+        CERB_CUDA_OK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)KT_SMEM));
+      for (auto kern : {tree_attn_tc_kernel<false>, tree_attn_tc_kernel<true>})
+        CERB_CUDA_OK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TC_SMEM));
       configured = true;
     }
-    auto kern = tree_attn_tc_kernel;
-    if (p.cluster)
-      rc = launch_pdl_cluster(kern, dim3(p.nsplit, p.H, Bw), dim3(TC_THREADS), TC_SMEM, st, (unsigned)p.nsplit,
-                              *tmK, *tmV, p) == cudaSuccess ? CERB_OK : CERB_E_CUDA;
-    else
-    {
-      // one split: persistent CTAs over the (window or sequence, head) items
-      const dim3 grid = p.nsplit == 1 ? dim3(Bw * p.H < 148 ? Bw * p.H : 148) : dim3(p.nsplit, p.H, Bw);
-      rc = launch_pdl(kern, grid, dim3(TC_THREADS), TC_SMEM, st, *tmK, *tmV, p) == cudaSuccess ? CERB_OK : CERB_E_CUDA;
+    const int items = p.items, tile = kt_path ? KT_TILE : TILE, tiles = (a->max_len + tile - 1) / tile;
+    // A launch over `n_items` of the (sequence or window, head) pairs, whose keys are cut into `nsplit` splits.  The kernels' forms for a part of
+    // the items or for a launch that follows are instances of their own: with the tests in the others these took 0.6 us more.
+    auto launch = [&](int n_items, int nsplit) {
+      p.items = n_items;
+      p.nsplit = nsplit;
+      p.cluster = (use_cluster && nsplit >= 2 && nsplit <= 8) ? 1 : 0;
+      const bool part = n_items != items || p.follows;
+      auto go = [&](auto kern, dim3 grid, int threads, size_t smem) {
+        return (p.cluster ? launch_pdl_cluster(kern, grid, dim3(threads), smem, st, (unsigned)nsplit, *tmK, *tmV, p)
+                          : launch_pdl(kern, grid, dim3(threads), smem, st, *tmK, *tmV, p)) == cudaSuccess ? CERB_OK : CERB_E_CUDA;
+      };
+      const dim3 grid = part ? dim3(nsplit, n_items) : dim3(nsplit, p.H, Bw);
+      if (kt_path) return go(part ? tree_attn_kt_kernel<true> : tree_attn_kt_kernel<false>, grid, KT_THREADS, KT_SMEM);
+      // one split: persistent CTAs over the items
+      return go(part ? tree_attn_tc_kernel<true> : tree_attn_tc_kernel<false>, nsplit == 1 ? dim3(n_items < 148 ? n_items : 148) : grid, TC_THREADS, TC_SMEM);
+    };
+    auto splits = [&](int n_items) {
+      int planned;
+      if (kt_path) {
+        int want = 148 / n_items;
+        if (want > attn_max_split()) want = attn_max_split();
+        if (want > tiles) want = tiles;
+        if (want < 1) want = 1;
+        const int per = (tiles + want - 1) / want;
+        planned = (tiles + per - 1) / per;
+      } else {
+        planned = plan_nsplit(n_items, 1, np_, a->max_len, resident, true, attn_max_split());
+      }
+      int ns = planned;
+      if (use_cluster && ns > 1)
+        ns = splits_at_once(tiles, ns, n_items, [&](int n) {
+          return kt_path ? clusters_at_once<tree_attn_kt_kernel<false>>(KT_THREADS, KT_SMEM, n, 1) : clusters_at_once<tree_attn_tc_kernel<false>>(TC_THREADS, TC_SMEM, n, 1);
+        });
+      const int pages = kt_path ? KT_PAGES : PAGES_PER_TILE;
+      auto too_long = [&](int n) { return (tiles + n - 1) / n * pages > kMaxPagesPerCta; };      // (fewer splits are longer ones)
+      if (ns > 0 && too_long(ns)) ns = planned;
+      return ns < 1 || too_long(ns) ? -1 : ns;
+    };
+    p.follows = row0 > 0 && use_cluster ? 1 : 0;                     // the second window of a wide tree (150 nodes behind 600 keys 28.4 -> 20.2 us)
+    // More items than SMs: where the last round leaves half of the SMs and more without one, its items' keys are split over them in a launch of its
+    // own, which needs nothing from the first one.  160 heads of 800 / 1564 / 4096 keys, 64 nodes: 30.7 / 44.9 / 94.9 us in one launch, 26.9 / 35.9 / 65.4 in two;
+    // 512: 65.6 / 95.4 / 217 and 66.1 / 91.8 / 201; below 768 keys the second launch costs as much as it gives (300 keys: 0.88 to 0.97 x).
+    const int rest = items % 148;
+    if (win == 1 && use_cluster && items > 148 && rest > 0 && rest <= 74 && tiles * tile >= 768) {
+      const int ns = splits(rest);
+      if (ns > 1 && splits(items) == 1) {
+        rc = launch(items - rest, 1);
+        if (rc != CERB_OK) return rc;
+        CERB_LAUNCH_CHECK(c);
+        p.item0 = items - rest;
+        p.follows = 1;
+        return launch(rest, ns);
+      }
     }
+    const int ns = splits(items);
+    if (ns < 1) return CERB_E_SHAPE;
+    rc = launch(items, ns);
   } else if (a->head_dim == 128) {
-    if (np == 16) rc = launch_cfg<128, 1, 4, 3>(p, tmK, tmV, Bw, st);
-    else if (np == 32) rc = launch_cfg<128, 2, 4, 3>(p, tmK, tmV, Bw, st);
-    else if (np == 64) rc = launch_cfg<128, 4, 2, 3>(p, tmK, tmV, Bw, st);
-    else rc = launch_cfg<128, 8, 1, 3>(p, tmK, tmV, Bw, st);
+    if (np == 16) rc = launch_cfg<128, 1, 4, 3>(p, tmK, tmV, Bw, a->max_len, st);
+    else if (np == 32) rc = launch_cfg<128, 2, 4, 3>(p, tmK, tmV, Bw, a->max_len, st);
+    else if (np == 64) rc = launch_cfg<128, 4, 2, 3>(p, tmK, tmV, Bw, a->max_len, st);
+    else rc = launch_cfg<128, 8, 1, 3>(p, tmK, tmV, Bw, a->max_len, st);
   } else if (a->head_dim == 64) {
-    if (np == 16) rc = launch_cfg<64, 1, 4, 4>(p, tmK, tmV, Bw, st);
-    else if (np == 32) rc = launch_cfg<64, 2, 4, 4>(p, tmK, tmV, Bw, st);
-    else if (np == 64) rc = launch_cfg<64, 4, 2, 4>(p, tmK, tmV, Bw, st);
-    else rc = launch_cfg<64, 8, 1, 4>(p, tmK, tmV, Bw, st);
+    if (np == 16) rc = launch_cfg<64, 1, 4, 4>(p, tmK, tmV, Bw, a->max_len, st);
+    else if (np == 32) rc = launch_cfg<64, 2, 4, 4>(p, tmK, tmV, Bw, a->max_len, st);
+    else if (np == 64) rc = launch_cfg<64, 4, 2, 4>(p, tmK, tmV, Bw, a->max_len, st);
+    else rc = launch_cfg<64, 8, 1, 4>(p, tmK, tmV, Bw, a->max_len, st);
   }
   return rc;
 }
@@ -1554,7 +1648,7 @@ int launch_tree_attention(cerb_ctx* c, const cerb_attn_args* a, const CUtensorMa
     const int launches = (win + per - 1) / per;
     per = (win + launches - 1) / launches;
     for (int win0 = 0; win0 < win; win0 += per) {
-      CERB_TRY(launch_attn_window(a, 0, kAttnRowsPerLaunch, tmK, tmV, status, st, row_off, win - win0 < per ? win - win0 : per, win0));
+      CERB_TRY(launch_attn_window(c, a, 0, kAttnRowsPerLaunch, tmK, tmV, status, st, row_off, win - win0 < per ? win - win0 : per, win0));
       CERB_LAUNCH_CHECK(c);
     }
     return CERB_OK;
@@ -1566,7 +1660,7 @@ int launch_tree_attention(cerb_ctx* c, const cerb_attn_args* a, const CUtensorMa
   // whole tree, rows of the first only nodes below 128 (an ancestor has a lower index than its descendant).
   for (int row0 = 0; row0 < a->n; row0 += kAttnRowsPerLaunch) {
     const int rows = a->n - row0 < kAttnRowsPerLaunch ? a->n - row0 : kAttnRowsPerLaunch;
-    CERB_TRY(launch_attn_window(a, row0, rows, tmK, tmV, status, st, row_off));
+    CERB_TRY(launch_attn_window(c, a, row0, rows, tmK, tmV, status, st, row_off));
     CERB_LAUNCH_CHECK(c);
   }
   return CERB_OK;

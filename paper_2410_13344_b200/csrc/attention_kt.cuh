@@ -75,6 +75,7 @@ __device__ __noinline__ bool wait_for_partner(uint32_t bar, long long budget) {
   return mbar_wait_drain(bar, 0, partner_cycles(w));
 }
 
+template <bool PART>
 __global__ void __launch_bounds__(KT_THREADS, 1) tree_attn_kt_kernel(const __grid_constant__ CUtensorMap tmK,
                                                                      const __grid_constant__ CUtensorMap tmV,
                                                                      const AttnParams p) {
@@ -110,7 +111,8 @@ __global__ void __launch_bounds__(KT_THREADS, 1) tree_attn_kt_kernel(const __gri
   const uint32_t q_base = p_base + PB * 2 * P_TERM;                       // [half of head_dim][NQ rows][128 B]
   const uint32_t ring = q_base + 2 * QHALF;                          // NU units
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int split = blockIdx.x, h = blockIdx.y, b = blockIdx.z;
+  const int split = blockIdx.x, item = PART ? p.item0 + (int)blockIdx.y : (int)(blockIdx.z * p.H + blockIdx.y);
+  const int b = PART ? item / p.H : (int)blockIdx.z, h = PART ? item - b * p.H : (int)blockIdx.y;
   // Lengths, live node counts, the page table, the tree and the prefix keys are at least two kernels old:
   // everything up to the first use of Q or of this step's tree keys runs before griddep_wait().
   const int L = p.len[b];
@@ -121,6 +123,12 @@ __global__ void __launch_bounds__(KT_THREADS, 1) tree_attn_kt_kernel(const __gri
     griddep_wait();
     return;
   }
+  // (a launch that follows another one of the same call waits for it at the end only: see AttnParams)
+  auto enter = [&]() {
+    if (PART && p.follows) return;
+    griddep_wait();
+    griddep_launch();
+  };
   const int n_tree = min(nq_all, p.row0 + p.rows);                    // tree keys these rows can see
   const int kv_total = L + n_tree;
   const int tiles = (kv_total + KT_TILE - 1) / KT_TILE;
@@ -212,7 +220,7 @@ __global__ void __launch_bounds__(KT_THREADS, 1) tree_attn_kt_kernel(const __gri
     // own two producers / by all: 192 items of 60 keys, 64 nodes, 18.8 / 18.4 us; 512 of 100 keys, 24 nodes, 33.6 / 32.8; 96 of 1000 keys,
     // 64 nodes, 20.4 / 20.2; a verification step of 64 nodes behind 2048 keys 3509 / 3494.)
     if (t_stop > 0) {
-      if (early == 0) { griddep_wait(); griddep_launch(); }
+      if (early == 0) enter();
       if (!kind && lane == 0) mbar_expect_tx(smem_u32(&full_u[0][0]), KT_UNIT / (NPROD / 2));
       __syncwarp();
       if (lane >> 2 == kind)
@@ -220,7 +228,7 @@ __global__ void __launch_bounds__(KT_THREADS, 1) tree_attn_kt_kernel(const __gri
       issued = 1 - kind;
     }
     for (int t = issued; t < t_stop; ++t) {
-      if (t == early) { griddep_wait(); griddep_launch(); }
+      if (t == early) enter();
       const int u = 2 * t + kind, slot = u % NU;
       const uint32_t fb = smem_u32(&full_u[kind][slot]);
       int stop = 0;
@@ -243,11 +251,9 @@ __global__ void __launch_bounds__(KT_THREADS, 1) tree_attn_kt_kernel(const __gri
       for (int t = issued > NU / 2 ? issued - NU / 2 : 0; t < issued; ++t)
         mbar_wait_drain(smem_u32(&full_u[kind][(2 * t + kind) % NU]), unit_parity(2 * t + kind), 20000000ll);
     }
-    griddep_wait();      // (a lane that has waited already returns at once)
-    griddep_launch();
+    enter();             // (a lane that has waited already returns at once)
   } else if (warp == W_QK) {
-    griddep_wait();
-    griddep_launch();
+    enter();
     // ---------------- QK^T issuer ----------------
     if (T > 0) {
       constexpr uint32_t idesc_s = idesc_bf16(128, NQ, false, false);
@@ -278,8 +284,7 @@ __global__ void __launch_bounds__(KT_THREADS, 1) tree_attn_kt_kernel(const __gri
       }
     }
   } else if (warp == W_PV) {
-    griddep_wait();
-    griddep_launch();
+    enter();
     // ---------------- PV issuer ----------------
     {
       // A = V tile read M-major (M = head_dim: two 64-wide blocks KT_HALF apart; 8-key groups 1024 bytes apart),
@@ -341,8 +346,7 @@ __global__ void __launch_bounds__(KT_THREADS, 1) tree_attn_kt_kernel(const __gri
       }
     }
     asm volatile("bar.sync 2, %0;" ::"r"(nst) : "memory");      // desc_t is complete
-    griddep_wait();
-    griddep_launch();
+    enter();
     {
       // stage Q (zeros past the last live node) in the swizzled K-major layout: 16-byte pieces, NQ * 16 of them,
       // spread over all softmax threads so that every thread has its loads in flight at once
@@ -625,12 +629,12 @@ __global__ void __launch_bounds__(KT_THREADS, 1) tree_attn_kt_kernel(const __gri
         if (hl == 0 && p.lse) p.lse[((size_t)b * p.H + h) * p.n + rr] = (M + log2f(Lsum)) * LN2;
       }
     } else {
-      float* part = p.partial + (((size_t)blockIdx.z * p.H + h) * p.nsplit) * (size_t)(RP * ROWF);
+      float* part = p.partial + ((size_t)item * p.nsplit) * (size_t)(RP * ROWF);
       float* mine = part + (size_t)split * (RP * ROWF);
       for (int idx = ct; idx < nq * ROWF; idx += nct) __stcg(mine + idx, mrg[idx]);
       __threadfence();
       asm volatile("bar.sync 2, %0;" ::"r"(nst) : "memory");
-      if (ct == 0) ticket_s = atomicAdd(&p.counters[blockIdx.z * p.H + h], 1u);
+      if (ct == 0) ticket_s = atomicAdd(&p.counters[item], 1u);
       asm volatile("bar.sync 2, %0;" ::"r"(nst) : "memory");
       if (ticket_s == (unsigned)p.nsplit - 1) {
         __threadfence();
@@ -665,7 +669,7 @@ __global__ void __launch_bounds__(KT_THREADS, 1) tree_attn_kt_kernel(const __gri
           *reinterpret_cast<uint2*>(p.out + ((qrow + rr) * p.H + h) * DH + c4 * 4) =
               make_uint2(pack_bf16(acc.x, acc.y), pack_bf16(acc.z, acc.w));
         }
-        if (ct == 0) p.counters[blockIdx.z * p.H + h] = 0u;          // ready for the next launch
+        if (ct == 0) p.counters[item] = 0u;          // ready for the next launch
       }
     }
   }
@@ -673,6 +677,10 @@ __global__ void __launch_bounds__(KT_THREADS, 1) tree_attn_kt_kernel(const __gri
     // Nobody leaves before every member has received its rows: what this CTA has sent leaves from its shared memory until then.
     if (warp >= NSW && warp != W_PV) cluster_start_wait();
     else if (warp == 0) cluster_wait_before_exit(&cl_bar[1], wc, &exit_flag_s, 114);
+  }
+  if (PART && p.follows) {
+    griddep_wait();
+    griddep_launch();
   }
   tc_fence_before();
   __syncthreads();                             // nobody exits before warp 0 has seen every member done
