@@ -117,6 +117,11 @@ size_t part_floats_needed(const cerb_config* g, int Mmax, int lm_rows, int sm_co
     if (f > best) best = f;
     f = (size_t)top * shapes[i][0];
     if (top > 128 && !finished[i] && f > best) best = f;
+    if (bf16 && top > 128 && (i == 1 || i == 3))             // O and down in parts
+      for (int M : {192, 256}) {
+        f = (size_t)plan_rows_sums(M, shapes[i][0], shapes[i][1], 8).parts * M * shapes[i][0];
+        if (f > best) best = f;
+      }
   }
   return best;
 }
@@ -231,10 +236,15 @@ int tree_build(cerb_ctx* c, const int32_t* parent, const int32_t* head_of, const
   return CERB_OK;
 }
 
-// Plans and maps of the plain products of 9 to 128 rows; in no more slots than the workspace has for them.
-int make_rows_sums(RowsSums* s, const void* const* W, int layers, int N, int K) {
-  for (int b = 0; b < 4; ++b) {
-    s->plan[b] = plan_rows_sums(32 * (b + 1), N, K, gemm_plan_split(148, 32 * (b + 1), N, K));
+// Plans and maps of the plain products of 9 to `rows` rows; in no more slots than the workspace has for them.
+int rows_sums_parts(int M, int N, int K) { return M > 128 ? 8 : gemm_plan_split(148, M, N, K); }
+int make_rows_sums(RowsSums* s, const void* const* W, int layers, int N, int K, int rows) {
+  for (int b = 0; b < kRowsSums && rows_sums_limit(b) <= rows; ++b) {
+    // Above 128 rows, against output tiles that pairs add up through a fix-up buffer (8-layer forwards of 129 / 192 / 256 rows): 1024 columns 1.26 / 1.28 / 1.29 x,
+    // 2048 1.17 / 1.19 / 1.18 x, 4096 1.03 / 1.02 / 1.035 x, 5120 0.98 / 1.00 / 1.012 x, 8192 0.99 / 1.00 / 0.955 x.  (The wider the output, the fewer
+    // parts and the less there was to add up; and the MMAs of output tiles follow the rows, a pair's are 256 high.)
+    if (rows_sums_limit(b) > 128 && N > (rows_sums_limit(b) == 192 ? 4096 : 6144)) continue;
+    s->plan[b] = plan_rows_sums(rows_sums_limit(b), N, K, rows_sums_parts(rows_sums_limit(b), N, K));
     if (!s->plan[b].tiles) continue;
     s->map[b].resize(layers);
     for (int l = 0; l < layers; ++l) CERB_TRY(make_rows_map(&s->map[b][l], W[l], N, K, s->plan[b].groups * 8));
@@ -253,11 +263,11 @@ unsigned long long* gemm_clock_slot(cerb_ctx* c) {
 int gemm(cerb_ctx* c, const void* X, const ActMaps* xm, const void* W, const CUtensorMap* wm, int M, int N, int K,
          int* nsplit, cudaStream_t st, float* out = nullptr, const RowsSums* sums = nullptr, int layer = 0) {
   if (c->bf16) {
-    if (sums && M > kFewRows && M <= 128 && sums->plan[(M - 1) / 32].tiles) {
-      const RowsPlan& g = sums->plan[(M - 1) / 32];
+    if (const int i = sums ? sums->at(M) : -1; i >= 0) {
+      const RowsPlan& g = sums->plan[i];
       *nsplit = g.parts;
       if ((size_t)g.parts * M * N > c->part_floats) return CERB_E_NOMEM;
-      return launch_gemm_rows(c, &sums->map[(M - 1) / 32][layer], xm, g, M, N, K, c->d_status, st, nullptr, out && g.parts == 1 ? out : c->d_part,
+      return launch_gemm_rows(c, &sums->map[i][layer], xm, g, M, N, K, c->d_status, st, nullptr, out && g.parts == 1 ? out : c->d_part,
                               gemm_clock_slot(c));
     }
     if (M <= kFewRows) {
@@ -345,7 +355,8 @@ int forward_rows(cerb_ctx* c, const cerb_tree* tree, const int32_t* tok, int tok
   const RowsPlan* rows_qkv = c->bf16 && gemm_rows_takes(c->rows_qkv, M, 3 * HD, d) ? &c->rows_qkv : nullptr;
   const bool fuse_swiglu = small || rows_gu || (wide && (M <= kFewRows || F % 16 == 0));
   const bool fuse_rope = small || rows_qkv || (wide && g.head_dim == 128);
-  const bool fuse_res = wide;
+  // (129 to 256 rows: O and down leave parts of k for the norm to add where both are for gemm_rows.cu)
+  const bool fuse_res = wide && !(M > 128 && c->rows_wo.at(M) >= 0 && c->rows_wd.at(M) >= 0);
   // Very few rows: the gate-up and QKV GEMMs normalise their rows themselves (the first layer's QKV GEMM excepted).
   const bool fuse_norm = small ? d <= kF32NormMax : fuse_swiglu && fuse_rope && M <= kFewRows && gemm_few_normalises(M, d);
   const int variant = launch_order_variant({fuse_swiglu, fuse_rope, fuse_res, fuse_norm});
@@ -427,7 +438,8 @@ int lm_head_argmax(cerb_ctx* c, const void* X, const ActMaps* xm, int rows, int3
                    cudaStream_t st) {
   int ns = 1;
   // one slot: the GEMM writes the caller's logits itself, and the argmax reads them there
-  const bool one_slot = rows > 128 || rows <= kFewRows || (c->rows_lm.plan[(rows - 1) / 32].tiles && c->rows_lm.plan[(rows - 1) / 32].parts == 1);
+  const int own = c->rows_lm.at(rows);
+  const bool one_slot = rows > 128 || rows <= kFewRows || (own >= 0 && c->rows_lm.plan[own].parts == 1);
   const bool direct = logits_out && c->bf16 && one_slot;
   { ProfScope ps(c, K_GEMM, st);
     CERB_TRY(gemm(c, X, xm, c->lm_head, c->bf16 ? &c->tm_lm_head : nullptr, rows, c->cfg.vocab, c->cfg.d_model, &ns, st,
@@ -573,10 +585,10 @@ int cerb_load(const cerb_config* cfg, const cerb_weights* w, void* workspace_dev
       }
       if (rc != CERB_OK) break;
       if ((rc = make_weight_map(&c->tm_lm_head, c->lm_head, g.vocab, g.d_model)) != CERB_OK) break;
-      if ((rc = make_rows_sums(&c->rows_wo, c->wo.data(), L, g.d_model, HD)) != CERB_OK) break;
-      if ((rc = make_rows_sums(&c->rows_wd, c->wd.data(), L, g.d_model, g.mlp_dim)) != CERB_OK) break;
+      if ((rc = make_rows_sums(&c->rows_wo, c->wo.data(), L, g.d_model, HD, 256)) != CERB_OK) break;
+      if ((rc = make_rows_sums(&c->rows_wd, c->wd.data(), L, g.d_model, g.mlp_dim, 256)) != CERB_OK) break;
       // (one part: the LM head's sums go straight to the logits.  4096 columns and more: 13B forwards 1.005 to 1.015 x; 1024 columns 0.98 x)
-      if (g.d_model >= 4096 && (rc = make_rows_sums(&c->rows_lm, &c->lm_head, 1, g.vocab, g.d_model)) != CERB_OK) break;
+      if (g.d_model >= 4096 && (rc = make_rows_sums(&c->rows_lm, &c->lm_head, 1, g.vocab, g.d_model, 128)) != CERB_OK) break;
       if ((rc = make_act_maps(&c->tm_xn, c->d_xn, Mr, g.d_model)) != CERB_OK) break;
       if ((rc = make_act_maps(&c->tm_hidden, c->d_hidden, Mr, g.d_model)) != CERB_OK) break;
       if ((rc = make_act_maps(&c->tm_attn, c->d_attn, Mr, HD)) != CERB_OK) break;

@@ -137,10 +137,17 @@ struct RowsPlan {
   int parts;                // plain sums: pieces that k is cut into, each a slot of the output
 };
 
-// ... and the plain products of up to 32, 64, 96 and 128 rows: a plan each, with the maps of all layers.
+// ... and the plain products of up to 32, 64, 96, 128, 192 and 256 rows: a plan each, with the maps of all layers.
+constexpr int kRowsSums = 6;
+inline int rows_sums_limit(int i) { return i < 4 ? 32 * (i + 1) : 64 * (i - 1); }
 struct RowsSums {
-  RowsPlan plan[4];
-  std::vector<CUtensorMap> map[4];
+  RowsPlan plan[kRowsSums];
+  std::vector<CUtensorMap> map[kRowsSums];
+  // which of them is for M rows, or -1
+  int at(int M) const {
+    const int i = M <= 8 || M > 256 ? -1 : M <= 128 ? (M - 1) / 32 : (M - 1) / 64 + 2;
+    return i >= 0 && plan[i].tiles ? i : -1;
+  }
 };
 
 }  // namespace cerb

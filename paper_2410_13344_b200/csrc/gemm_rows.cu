@@ -1,5 +1,5 @@
 // bf16 GEMM of 9 to 256 activation rows in tiles as wide as an SM's share: gate-up with SwiGLU, QKV with RoPE and cache append, whose outputs are
-// finished where they are summed, and up to 128 rows plain sums (O, down, LM head) in few parts of k.
+// finished where they are summed, and plain sums (O, down, up to 128 rows the LM head) in few parts of k.
 //
 //   CG = 1:  D[128 activation rows][w weight rows] per CTA
 //   CG = 2:  D[256 activation rows][2 w weight rows] per pair of CTAs (cta_group::2), fp32, in tensor memory; one tile, all of k
@@ -105,8 +105,9 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_rows_kernel(const __grid_con
   const bool two = KIND == 1 && CG == 2 && p.groups0 < p.groups;           // two MMAs per 16 k
   // Consecutive groups; RoPE: four rotations of a block of heads.  Plain sums: the parts of a tile are neighbours.
   const int row0 = KIND == 2 ? ((int)blockIdx.x & 15) * 4 : 0;
-  const int tile = KIND == 2 ? (int)blockIdx.x >> 4 : KIND == 0 ? (int)blockIdx.x / p.parts : (int)blockIdx.x;
-  const int group0 = tile * p.groups, slot = KIND == 0 ? (int)blockIdx.x - tile * p.parts : 0;
+  const int tile = KIND == 2 ? (int)blockIdx.x >> 4 : KIND == 0 ? (int)blockIdx.x / CG / p.parts : (int)blockIdx.x;
+  const int slot = KIND == 0 ? (int)blockIdx.x / CG - tile * p.parts : 0;
+  const int group0 = (KIND == 0 ? tile * CG + rank : tile) * p.groups;
   const int kb0 = KIND == 0 ? slot * p.num_kb / p.parts : 0, num_kb = KIND == 0 ? (slot + 1) * p.num_kb / p.parts - kb0 : p.num_kb;
 
   if (threadIdx.x == 0) {
@@ -152,12 +153,13 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_rows_kernel(const __grid_con
       auto full = [&](int s) { return CG == 2 ? mapa_u32(smem_u32(&full_bar[s]), 0) : smem_u32(&full_bar[s]); };
       auto load_w = [&](int kb, int s) {
         if (first) mbar_expect_tx(smem_u32(&full_bar[s]), CG * stage_bytes);               // (a pair's first CTA counts both CTAs' copies)
-        if constexpr (KIND == 0) tma_load_2d_hint(smem_base + (uint32_t)s * stage_bytes, &tmW, (kb0 + kb) * BK, group0 * 8, full(s), pol_w);
+        if constexpr (KIND == 0 && CG == 2) tma_load_2d_pair(smem_base + (uint32_t)s * stage_bytes, &tmW, (kb0 + kb) * BK, group0 * 8, full(s), pol_w);
+        else if constexpr (KIND == 0) tma_load_2d_hint(smem_base + (uint32_t)s * stage_bytes, &tmW, (kb0 + kb) * BK, group0 * 8, full(s), pol_w);
         else load_groups<CG>(smem_base + (uint32_t)s * stage_bytes, &tmW, kb * BK, row0, group0, full(s), pol_w);
       };
       auto load_x = [&](int kb, int s) {
         const uint32_t dst = smem_base + (uint32_t)s * stage_bytes + w_bytes;
-        if constexpr (CG == 2) tma_load_2d_pair(dst, &tmX, kb * BK, rank * p.x_rows, full(s), pol_x);
+        if constexpr (CG == 2) tma_load_2d_pair(dst, &tmX, (kb0 + kb) * BK, rank * p.x_rows, full(s), pol_x);
         else tma_load_2d_hint(dst, &tmX, (kb0 + kb) * BK, 0, full(s), pol_x);
       };
       const int pre = min(num_kb, p.stages);
@@ -392,10 +394,10 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_rows_kernel(const __grid_con
           }
         }
       } else if constexpr (KIND == 0) {
-        for (int c = part; 2 * c < p.groups; c += kParts) {
+        for (int c = part; 2 * c < CG * p.groups; c += kParts) {
           float v[COLS];
           load((uint32_t)(c * COLS), (uint32_t)(c * COLS + 8), v);
-          const int n = group0 * 8 + c * COLS, cols = min(2 * c + 2 <= p.groups ? 16 : 8, p.N - n);
+          const int n = (tile * CG * p.groups + 2 * c) * 8, cols = min(2 * c + 2 <= CG * p.groups ? 16 : 8, p.N - n);
           float* o = p.out + ((size_t)slot * p.M + row) * p.N + n;
           if (!ok) continue;
           if (!(p.N & 3)) {
@@ -520,21 +522,22 @@ bool gemm_rows_takes(const RowsPlan& g, int M, int N, int K) {
 // 85; a k block takes 0.34 us, however narrow the tile.  7B width, 64 rows, 8 layers: down in 2 / 4 / 5 / 8 parts 872 / 847 / 845 / 859 us, O in 4 / 5 / 8
 // 847 / 845 / 856.  (Units of 256 weight rows left ten slots after both, 10 MB that the norm read back; slots of the same plan, 64 rows: norm 4.65 ->
 // 4.0 us, O 9.8 -> 8.8, down 17.6 -> 16.5.)
+// 129 to 256 rows, in pairs: the same, a part costing more (4 MB to write and to read back at 256 rows and 4096 columns).
 RowsPlan plan_rows_sums(int M, int N, int K, int max_parts) {
   RowsPlan best{0, 0, false, 0};
   double best_t = 0;
-  const int groups = (N + 7) / 8, num_kb = (K + BK - 1) / BK, x = (M + 31) / 32 * 32 / 8;
-  if (M <= kFewRows || M > ROWS) return best;
+  const int pair = M > ROWS ? 2 : 1, groups = (N + 7) / 8, num_kb = (K + BK - 1) / BK, x = ((M + pair - 1) / pair + 31) / 32 * 32 / 8;
+  if (M <= kFewRows || M > 2 * ROWS) return best;
   for (int parts = 1; parts <= max_parts && parts <= 8 && parts * 4 <= num_kb; ++parts) {
-    const int tiles = kSms / parts, per = (groups + tiles - 1) / tiles;
-    if (per > 32 || per < 2) continue;
+    const int tiles = kSms / pair / parts, per = (groups + pair * tiles - 1) / (pair * tiles);
+    if (per > 32 / pair || per < 2) continue;
     const double kb = (num_kb + parts - 1) / parts;
     const double hbm = kb * per / 44.0, sm = kb * (per + x) / 85.0;
     const double least = kb * 0.34;                      // a stage's copies, waits and MMAs
-    const double in = hbm > sm ? hbm : sm, t = (in > least ? in : least) + parts * (0.05 + 0.001 * M);
+    const double in = hbm > sm ? hbm : sm, t = (in > least ? in : least) + parts * (pair == 2 ? 0.004 * M : 0.05 + 0.001 * M);
     if (!best_t || t < best_t) {
       best_t = t;
-      best = RowsPlan{per, (groups + per - 1) / per * parts, false, parts};
+      best = RowsPlan{per, (groups + pair * per - 1) / (pair * per) * parts * pair, false, parts};
     }
   }
   return best;
@@ -542,7 +545,7 @@ RowsPlan plan_rows_sums(int M, int N, int K, int max_parts) {
 
 int launch_gemm_rows(cerb_ctx* c, const CUtensorMap* tmW, const ActMaps* tmX, const RowsPlan& g, int M, int N, int K, int32_t* status, cudaStream_t st,
                      const GemmEpilogue* epi, float* out, unsigned long long* clock_slot) {
-  if (epi ? !gemm_rows_takes(g, M, N, K) : M < 1 || M > ROWS || g.parts < 1) return CERB_E_SHAPE;
+  if (epi ? !gemm_rows_takes(g, M, N, K) : M < 1 || M > 2 * ROWS || g.parts < 1) return CERB_E_SHAPE;
   const bool pairs = M > ROWS;            // (7B width, 96 and 128 rows: 1062 and 1082 us in pairs, 926 and 974 in single CTAs)
   RowsParams p;
   memset(&p, 0, sizeof(p));
@@ -590,7 +593,7 @@ int launch_gemm_rows(cerb_ctx* c, const CUtensorMap* tmW, const ActMaps* tmX, co
   };
   int rc;
   if (!epi) {
-    rc = launch_kind<0, 1>(*tmW, tmX->box(p.x_rows), p, g.tiles, st);
+    rc = run(std::integral_constant<int, 0>(), tmX->box(p.x_rows));
   } else if (epi->kind == 1) {
     p.act = (bf16*)epi->act;
     rc = run(std::integral_constant<int, 1>(), tmX->box(p.x_rows));

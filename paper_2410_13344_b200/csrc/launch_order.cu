@@ -8,6 +8,8 @@
 // least two launches older.  This file states, per kernel, what it writes and what it reads ahead of its wait;
 // launch_order_violations() checks the rule over the cyclic layer sequence, and the host controller steps
 // through the same table while it launches (forward_rows), so that the table cannot drift from the code.
+// An attention that takes two launches (a rest of items, the second window of a wide tree) is one entry: the second one reads what is complete when
+// the first one runs, and waits for that one at its end.
 #include <stdio.h>
 #include <string.h>
 
