@@ -351,8 +351,8 @@ int forward_rows(cerb_ctx* c, const cerb_tree* tree, const int32_t* tok, int tok
   const bool small = !c->bf16 && c->f32_aligned && gemm_f32_small(M, 2 * F) && gemm_f32_small(M, 3 * HD) && gemm_f32_small(M, d);
   const bool wide = small || (c->bf16 && (M > 128 || M <= kFewRows));
   // 9 to 128 rows: SwiGLU and RoPE + cache append only, where the matrix is for gemm_rows.cu (which takes some of these up to 256 rows, too).
-  const RowsPlan* rows_gu = c->bf16 && gemm_rows_takes(c->rows_gu, M, 2 * F, d) ? &c->rows_gu : nullptr;
-  const RowsPlan* rows_qkv = c->bf16 && gemm_rows_takes(c->rows_qkv, M, 3 * HD, d) ? &c->rows_qkv : nullptr;
+  const RowsPlan* rows_gu = c->bf16 && gemm_rows_takes(c->rows_gu, M, d) ? &c->rows_gu : nullptr;
+  const RowsPlan* rows_qkv = c->bf16 && gemm_rows_takes(c->rows_qkv, M, d) ? &c->rows_qkv : nullptr;
   const bool fuse_swiglu = small || rows_gu || (wide && (M <= kFewRows || F % 16 == 0));
   const bool fuse_rope = small || rows_qkv || (wide && g.head_dim == 128);
   // (129 to 256 rows: O and down leave parts of k for the norm to add where both are for gemm_rows.cu)

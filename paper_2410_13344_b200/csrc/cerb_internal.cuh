@@ -321,7 +321,7 @@ int launch_gemm_few(cerb_ctx* c, const void* X, const void* W, float* out, int M
                     const GemmNorm* norm = nullptr, unsigned long long* clock_slot = nullptr);
 bool gemm_few_normalises(int M, int K);
 // gemm_rows.cu: 9 to 256 rows, kinds 1 and 2
-bool gemm_rows_takes(const RowsPlan& g, int M, int N, int K);
+bool gemm_rows_takes(const RowsPlan& g, int M, int K);
 RowsPlan plan_rows_swiglu(int F);
 RowsPlan plan_rows_rope(int n_heads, int head_dim);
 int launch_gemm_rows(cerb_ctx* c, const CUtensorMap* tmW, const ActMaps* tmX, const RowsPlan& g, int M, int N, int K, int32_t* status, cudaStream_t st,

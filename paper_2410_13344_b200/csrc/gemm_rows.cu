@@ -507,14 +507,14 @@ RowsPlan plan_rows_rope(int n_heads, int head_dim) {
 //   Up to 128 rows, against partial sums and kernels behind them: matrices of at least 16 rows per SM (an MMA's N is no less) and at most 256.
 //   Forwards, plain sums (below) included: 7B width 9 / 64 / 128 rows 1.06 / 1.06 / 1.12 x, 13B 1.02 / 1.09 / 1.13 x, 1024 to 3200 columns 1.04 to 1.25 x.
 //   129 to 256 rows, in pairs, against output tiles of 256 weight rows (gemm_tile.cu): a pair's tile has to fit one MMA, or (SwiGLU, 16 k
-//   blocks and more) three accumulators.  Tiles of 256 rows leave SMs idle or have to be cut along k: 7B width, 129 / 192 / 256 rows, 8 layers 1317 /
-//   1368 / 1457 -> 1224 / 1319 / 1311 us.  Where the tiles of QKV occupy more than 0.7 of the pairs, there is something to gain from 192 rows on
-//   only (13B, QKV alone: 129 rows 0.98 x, 192 1.01, 256 1.02).
-bool gemm_rows_takes(const RowsPlan& g, int M, int N, int K) {
+//   blocks and more) three accumulators.  Tiles of 256 rows leave SMs idle or have to be cut along k: 7B width, gate-up of 129 / 256 rows 46 / 53 -> 41 /
+//   43 us.  RoPE from 193 rows on: below, the output tiles are cut and sum shorter chains than the two that fit here (keys of 130 to 180 rows against float64
+//   1.10e-4 to 1.32e-4 there, 1.32e-4 to 1.52e-4 here; from 193 rows on the bits are the same; QKV of 256 rows 32.5 -> 27 us).
+bool gemm_rows_takes(const RowsPlan& g, int M, int K) {
   if (M <= kFewRows || M > 2 * ROWS || g.tiles < 1) return false;
   if (M <= ROWS) return true;
   if (g.groups > 16) return !g.heads && (g.groups + (g.groups + 1) / 2) * 16 <= 512 && K >= 16 * BK;
-  return !g.heads || M >= 192 || (N + 255) / 256 <= 0.7 * (kSms / 2);
+  return !g.heads || M > 192;
 }
 
 // Plain sums of up to 128 rows (O, down, LM head): k is cut into parts, each a sum of its own (a slot) for the kernel behind to add, so that tiles are wide
@@ -545,7 +545,7 @@ RowsPlan plan_rows_sums(int M, int N, int K, int max_parts) {
 
 int launch_gemm_rows(cerb_ctx* c, const CUtensorMap* tmW, const ActMaps* tmX, const RowsPlan& g, int M, int N, int K, int32_t* status, cudaStream_t st,
                      const GemmEpilogue* epi, float* out, unsigned long long* clock_slot) {
-  if (epi ? !gemm_rows_takes(g, M, N, K) : M < 1 || M > 2 * ROWS || g.parts < 1) return CERB_E_SHAPE;
+  if (epi ? !gemm_rows_takes(g, M, K) : M < 1 || M > 2 * ROWS || g.parts < 1) return CERB_E_SHAPE;
   const bool pairs = M > ROWS;            // (7B width, 96 and 128 rows: 1062 and 1082 us in pairs, 926 and 974 in single CTAs)
   RowsParams p;
   memset(&p, 0, sizeof(p));
