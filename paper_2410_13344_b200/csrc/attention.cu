@@ -1382,9 +1382,10 @@ int plan_nsplit(int B, int H, int n, int max_len, int target_ctas, bool one_wave
 // the size: of one CTA to an SM 16 clusters of eight, and fewer than 20 of seven or 24 of six.
 template <auto KERNEL>
 int clusters_at_once(int threads, size_t smem, int size, int per_sm) {
-  static int known[9];                           // (per kernel; every call would store the same)
+  static std::atomic<int> known[9];              // (per kernel; every call would store the same)
   if (size < 2 || size > 8) return 148 * per_sm / (size < 1 ? 1 : size);
-  if (!known[size]) {
+  int n = known[size].load(std::memory_order_relaxed);
+  if (!n) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(size);
     cfg.blockDim = dim3(threads);
@@ -1395,14 +1396,14 @@ int clusters_at_once(int threads, size_t smem, int size, int per_sm) {
     attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    int n = 0;
     if (cudaOccupancyMaxActiveClusters(&n, KERNEL, &cfg) != cudaSuccess) {
       cudaGetLastError();
       n = 148 * per_sm / size;
     }
-    known[size] = n < 1 ? 1 : n;
+    n = n < 1 ? 1 : n;
+    known[size].store(n, std::memory_order_relaxed);
   }
-  return known[size];
+  return n;
 }
 
 // The most splits, `want` at most, whose clusters are all there at once (those of a second round cost a whole round: 24 heads of 4000 keys and 64
