@@ -750,6 +750,19 @@ int cerb_accept(cerb_ctx* c, const cerb_tree* tree, const int32_t* tree_tok_dev,
   return CERB_OK;
 }
 
+// The device's address of `words` words of the caller's host memory, or null where kernels cannot write all of them (pageable, registered in part).
+// Asked on every call: memory may have been freed and come back as another kind.
+static int32_t* pinned_words(int32_t* p, size_t words) {
+  if (!p) return nullptr;
+  cudaPointerAttributes a, z;
+  if (cudaPointerGetAttributes(&a, p) != cudaSuccess || cudaPointerGetAttributes(&z, p + words - 1) != cudaSuccess) {
+    cudaGetLastError();
+    return nullptr;
+  }
+  int32_t* d = (int32_t*)a.devicePointer;
+  return a.type == cudaMemoryTypeHost && z.type == cudaMemoryTypeHost && d && (int32_t*)z.devicePointer == d + (words - 1) ? d : nullptr;
+}
+
 int cerb_step(cerb_ctx* c, const cerb_tree* tree, float T, const int32_t* plant_tok_dev, cerb_step_out* out,
               void* stream) {
   if (!c || !tree || !out || !out->S_dev || !out->mode_dev || !out->n_accept_dev || !out->tokens_dev) return CERB_E_ARG;
@@ -797,12 +810,15 @@ int cerb_step(cerb_ctx* c, const cerb_tree* tree, float T, const int32_t* plant_
   }
   CERB_TRY(forward_rows(c, used, tok, n, 0, n, st, M, row_off));
   CERB_TRY(lm_head_argmax(c, c->d_hidden, &c->tm_hidden, M, c->d_argmax, nullptr, st));
+  // (the two results for the host: from the kernel where it can reach them, two copies of a few words otherwise)
+  int32_t* host_n = pinned_words(out->n_accept_host, B);
+  int32_t* host_tok = pinned_words(out->tokens_host, (size_t)B * kPathMax);
   { ProfScope ps(c, K_ACCEPT, st);
-    CERB_TRY(launch_accept(c, used, tok, c->d_nactive, c->d_argmax, out->n_accept_dev, c->d_path, out->tokens_dev, st, row_off)); }
+    CERB_TRY(launch_accept(c, used, tok, c->d_nactive, c->d_argmax, out->n_accept_dev, c->d_path, out->tokens_dev, st, row_off, host_n, host_tok)); }
   for (int b = 0; b < B; ++b) c->h_len[b] += used->max_depth + 1;
-  if (out->n_accept_host)
+  if (out->n_accept_host && !host_n)
     CERB_CUDA_OK(cudaMemcpyAsync(out->n_accept_host, out->n_accept_dev, B * sizeof(int32_t), cudaMemcpyDeviceToHost, st));
-  if (out->tokens_host)
+  if (out->tokens_host && !host_tok)
     CERB_CUDA_OK(cudaMemcpyAsync(out->tokens_host, out->tokens_dev, (size_t)B * kPathMax * sizeof(int32_t),
                                  cudaMemcpyDeviceToHost, st));
   c->verified_tree = nullptr;

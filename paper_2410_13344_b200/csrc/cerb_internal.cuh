@@ -355,10 +355,11 @@ int launch_heads(cerb_ctx* c, const cerb_tree* tree, int32_t* tree_tok, const in
                  float* logits_out, cudaStream_t st);
 
 // gate_accept.cu
-// host: pinned staging that receives [mode | len | S], CERB_MAX_BATCH words each, or null
+// host: pinned staging that receives [mode | len | S], CERB_MAX_BATCH words each, or null; host_n, host_tok: device addresses of pinned copies of n_accept
+// and out_tok, or null
 int launch_gate(cerb_ctx* c, float T, float* S, int32_t* mode, int32_t* nactive_or_null, int n_par, cudaStream_t st, int32_t* host = nullptr);
 int launch_accept(cerb_ctx* c, const cerb_tree* tree, const int32_t* tree_tok, const int32_t* n_active,
                   const int32_t* node_argmax, int32_t* n_accept, int32_t* path, int32_t* out_tok, cudaStream_t st,
-                  const int32_t* row_off = nullptr);
+                  const int32_t* row_off = nullptr, int32_t* host_n = nullptr, int32_t* host_tok = nullptr);
 
 }  // namespace cerb
