@@ -1252,30 +1252,40 @@ __global__ void __launch_bounds__(ONE_WARPS * 32, 2) tree_attn_one_kernel(const 
 // ---------------------------------------------------------------------------------------------
 // A CTA per (node, head), whose warps take four keys each in turn.  A launch is bound by the rounds of memory latency that one
 // warp goes through, hence eight warps and not four: twelve steps and the prefill of the 4-layer fp32 model over a 64-token prompt, 2857 -> 2690 us.
+// In a forward (`ahead`) the lists and (TWO) the first two fours of every warp, where they are committed keys, come ahead of the dependency
+// wait, and the next four is under way while one is used: verification forwards of 4 layers with 4 heads, head_dim 64 behind 64 keys / 128 behind 500,
+// 16 nodes 142.9 / 346.8 -> 139.0 / 309.1 us, 64 nodes 202.6 / 480.1 -> 195.9 / 443.9; 4 x 64 nodes behind 2000 keys (1024 CTAs) 1125 -> 1076.  More CTAs
+// hide each other's latency and want the registers (72 and 108, 48 and 64 with one four): 2 x 192 nodes (1536 CTAs) 592.1 / 1606 against 596.2 / 1617.
+constexpr int F32_TWO_CTAS = 1024;
 // Of the tree's keys a node sees only its ancestors: their indices are laid out in shared memory first, so that the fours are full
 // (2 x 192 nodes x 4 heads behind 16 keys: 9.8 us; 37.0 with fours of neighbouring keys, 18.5 with single ones that skip).
 constexpr int F32_WARPS = 8;
-template <int DH>
+template <int DH, bool TWO>
 __global__ void __launch_bounds__(F32_WARPS * 32) tree_attn_f32_kernel(const float* q, const float* kpool,
                                                             const float* vpool,
                                                             const int32_t* __restrict__ page_table,
                                                             const int32_t* len, const int32_t* n_active,
                                                             const uint64_t* __restrict__ anc, float* __restrict__ out,
                                                             float* __restrict__ lse, int n, int H, int max_pages,
-                                                            float scale, const int32_t* row_off, int win) {
+                                                            float scale, const int32_t* row_off, int win, int ahead) {
   constexpr int E = DH / 32;
   __shared__ float s_o[F32_WARPS][DH];
   __shared__ float s_m[F32_WARPS], s_l[F32_WARPS];
   __shared__ short s_key[CERB_MAX_NODES];
   static_assert(F32_WARPS * 32 >= CERB_MAX_NODES, "a thread per tree key");
-  griddep_wait();
-  griddep_launch();
+  if (!ahead) {
+    griddep_wait();
+    griddep_launch();
+  }
   // (windows of 128 rows of a prefill chunk: see locate_window)
   const int i = blockIdx.x, h = blockIdx.y, b = blockIdx.z / win, shift = (blockIdx.z % win) * kAttnRowsPerLaunch;
   const int nq_all = (n_active ? min(n_active[b], n) : n) - shift;
   const int nq = win > 1 ? min(nq_all, kAttnRowsPerLaunch) : nq_all;
-  if (i >= nq) return;
-  const int L = len[b] + shift, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (i >= nq) {
+    griddep_wait();      // (no CTA leaves ahead of the kernel in front; at once where it has waited already)
+    return;
+  }
+  const int settled = len[b], L = settled + shift, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   // the live tree keys that this node sees, in order
   uint64_t see[CERB_ANC_WORDS];
   int seen = 0, mine = -1;                             // how many there are; the place of key threadIdx.x among them
@@ -1291,23 +1301,22 @@ __global__ void __launch_bounds__(F32_WARPS * 32) tree_attn_f32_kernel(const flo
   float qv[E], acc[E];
   const size_t qrow = (row_off ? (size_t)row_off[b] : (size_t)b * n) + shift;
   const float* qp = q + ((qrow + i) * H + h) * DH;
-  for (int e = 0; e < E; ++e) { qv[e] = qp[lane + 32 * e]; acc[e] = 0.f; }
   float m = -INFINITY, l = 0.f;
   // Four keys at a time, whose page entries, keys and values are all requested before the first is used: one key after the
   // other was a chain of two round trips to memory and a reduction per key.
-  constexpr int KEYS = 4;
-  for (int base = warp * KEYS; base < L + seen; base += F32_WARPS * KEYS) {
+  constexpr int KEYS = 4, ROUND = F32_WARPS * KEYS;
+  const int first = warp * KEYS, end = L + seen;
+  auto fetch = [&](int base, float (&kv)[KEYS][E], float (&vv)[KEYS][E]) {
     size_t off[KEYS];
     bool sees[KEYS];
 #pragma unroll
     for (int u = 0; u < KEYS; ++u) {
       int kpos = base + u;
-      sees[u] = kpos < L + seen;
+      sees[u] = kpos < end;
       if (sees[u] && kpos >= L) kpos = L + s_key[kpos - L];
       const int page = sees[u] ? page_table[(size_t)b * max_pages + kpos / CERB_PAGE] : 0;
       off[u] = (((size_t)page * H + h) * CERB_PAGE + kpos % CERB_PAGE) * DH;
     }
-    float kv[KEYS][E], vv[KEYS][E], s[KEYS];
 #pragma unroll
     for (int u = 0; u < KEYS; ++u)
 #pragma unroll
@@ -1315,6 +1324,9 @@ __global__ void __launch_bounds__(F32_WARPS * 32) tree_attn_f32_kernel(const flo
         kv[u][e] = sees[u] ? kpool[off[u] + lane + 32 * e] : 0.f;
         vv[u][e] = sees[u] ? vpool[off[u] + lane + 32 * e] : 0.f;
       }
+  };
+  auto take = [&](int base, const float (&kv)[KEYS][E], const float (&vv)[KEYS][E]) {
+    float s[KEYS];
 #pragma unroll
     for (int u = 0; u < KEYS; ++u) {
       s[u] = 0.f;
@@ -1328,10 +1340,10 @@ __global__ void __launch_bounds__(F32_WARPS * 32) tree_attn_f32_kernel(const flo
     float mn = m;
 #pragma unroll
     for (int u = 0; u < KEYS; ++u) {
-      s[u] = sees[u] ? s[u] * scale : -INFINITY;
+      s[u] = base + u < end ? s[u] * scale : -INFINITY;
       mn = fmaxf(mn, s[u]);
     }
-    if (mn == -INFINITY) continue;                       // (nothing seen so far; uniform over the warp)
+    if (mn == -INFINITY) return;                         // (nothing seen so far; uniform over the warp)
     const float al = expf(m - mn);
     l *= al;
 #pragma unroll
@@ -1344,6 +1356,28 @@ __global__ void __launch_bounds__(F32_WARPS * 32) tree_attn_f32_kernel(const flo
       for (int e = 0; e < E; ++e) acc[e] += pw * vv[u][e];
     }
     m = mn;
+  };
+  float ka[KEYS][E], va[KEYS][E], kb[KEYS][E], vb[KEYS][E];              // TWO: two fours in turn
+  const bool early_a = TWO && ahead && first + KEYS <= settled, early_b = TWO && ahead && first + ROUND + KEYS <= settled;
+  if (early_a) fetch(first, ka, va);
+  if (early_b) fetch(first + ROUND, kb, vb);
+  if (ahead) {
+    griddep_wait();
+    griddep_launch();
+  }
+#pragma unroll
+  for (int e = 0; e < E; ++e) { qv[e] = qp[lane + 32 * e]; acc[e] = 0.f; }
+  if (!TWO) {
+    for (int base = first; base < end; base += ROUND) { fetch(base, ka, va); take(base, ka, va); }
+  } else if (!early_a) {
+    fetch(first, ka, va);
+  }
+  for (int base = first; TWO && base < end; base += 2 * ROUND) {
+    if (base + ROUND < end && !(early_b && base == first)) fetch(base + ROUND, kb, vb);
+    take(base, ka, va);
+    if (base + ROUND >= end) break;
+    if (base + 2 * ROUND < end) fetch(base + 2 * ROUND, ka, va);
+    take(base + ROUND, kb, vb);
   }
   for (int e = 0; e < E; ++e) s_o[warp][lane + 32 * e] = acc[e];
   if (lane == 0) { s_m[warp] = m; s_l[warp] = l; }
@@ -1626,14 +1660,15 @@ int launch_tree_attention(cerb_ctx* c, const cerb_attn_args* a, const CUtensorMa
   const int win = chain ? (a->n + kAttnRowsPerLaunch - 1) / kAttnRowsPerLaunch : 1;
   if (a->dtype == CERB_F32) {
     dim3 grid(win > 1 ? kAttnRowsPerLaunch : a->n, a->n_heads, a->B * win);
+    const bool two = (long long)grid.x * grid.y * grid.z <= F32_TWO_CTAS;
     auto go = [&](auto kern) {
       launch_pdl(kern, grid, dim3(F32_WARPS * 32), 0, st, (const float*)a->q, (const float*)a->k_pool, (const float*)a->v_pool, a->page_table, a->len,
-                 a->n_active, a->anc, (float*)a->out, a->lse, a->n, a->n_heads, a->max_pages, a->scale, row_off, win);
+                 a->n_active, a->anc, (float*)a->out, a->lse, a->n, a->n_heads, a->max_pages, a->scale, row_off, win, c ? 1 : 0);
     };
     if (a->head_dim == 64)
-      go(tree_attn_f32_kernel<64>);
+      two ? go(tree_attn_f32_kernel<64, true>) : go(tree_attn_f32_kernel<64, false>);
     else if (a->head_dim == 128)
-      go(tree_attn_f32_kernel<128>);
+      two ? go(tree_attn_f32_kernel<128, true>) : go(tree_attn_f32_kernel<128, false>);
     else
       return CERB_E_SHAPE;
     CERB_LAUNCH_CHECK(c);
