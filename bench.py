@@ -35,10 +35,10 @@ N_NODES = 64
 TOPK = [10, 10, 10, 10]
 PROMPT_LEN = 2048
 HBM_NOMINAL_GBS = 8000.0
-# dram__bytes_read.sum + dram__bytes_write.sum of one gemm_bf16_kernel launch (ncu --set full, M=64 N=22016 K=4096:
-# profiles/gemm_bf16_kernel_M64_N22016_K4096.md); algorithmic bytes of that launch: 183.7 MB.
-GEMM_TRAFFIC = 186.0e6
-GEMM_TRAFFIC_NOTE = {"launch": "M=64 N=22016 K=4096", "algorithmic_bytes_per_launch": 183.7e6}
+# dram__bytes_read.sum + dram__bytes_write.sum of one gemm_rows_kernel launch (ncu, M=64 N=22016 K=4096 with SwiGLU behind:
+# profiles/gemm_rows_kernel.md); algorithmic bytes of that launch: weights, activations in, M x 11008 activations out.
+GEMM_TRAFFIC = 181.1e6
+GEMM_TRAFFIC_NOTE = {"launch": "M=64 N=22016 K=4096", "algorithmic_bytes_per_launch": 182.3e6}
 
 
 def draft_setup(name: str):
@@ -361,7 +361,7 @@ def run_cerb(args, rank, world):
         "planted": {"value": agg(tok_d) / (ms_d / 1e3), "unit": UNIT, "mean_accepted_per_step": tok_d / max(1, len(acc_d)),
                     "note": "synthetic acceptance: one tree path overwritten with the greedy continuation (lengths 1..5 requested), every step parallel; only the steps are timed"},
         "prefill_ms": prefill_ms,
-        "roofline": {"bound": "hbm", "kernel": "gemm_bf16_kernel (tcgen05 weight-streaming GEMM)",
+        "roofline": {"bound": "hbm", "kernel": "gemm_rows_kernel (tcgen05 weight-streaming GEMM)",
                      "achieved": gemm_gbs, "peak": hbm_peak, "unit": "GB/s", "frac": (gemm_gbs / hbm_peak) if gemm_gbs else None,
                      "peak_kind": peak_kind + " copy bandwidth", "frac_of_nominal_8TBs": (gemm_gbs / HBM_NOMINAL_GBS) if gemm_gbs else None,
                      "traffic": GEMM_TRAFFIC, "traffic_of": GEMM_TRAFFIC_NOTE, "launch_groups": gemm_groups, "ms_per_step": gemm_ms / prof_steps,
