@@ -1255,8 +1255,9 @@ __global__ void __launch_bounds__(ONE_WARPS * 32, 2) tree_attn_one_kernel(const 
 // In a forward (`ahead`) the lists and (TWO) the first two fours of every warp, where they are committed keys, come ahead of the dependency
 // wait, and the next four is under way while one is used: verification forwards of 4 layers with 4 heads, head_dim 64 behind 64 keys / 128 behind 500,
 // 16 nodes 142.9 / 346.8 -> 139.0 / 309.1 us, 64 nodes 202.6 / 480.1 -> 195.9 / 443.9; 4 x 64 nodes behind 2000 keys (1024 CTAs) 1125 -> 1076.  More CTAs
-// hide each other's latency and want the registers (72 and 108, 48 and 64 with one four): 2 x 192 nodes (1536 CTAs) 592.1 / 1606 against 596.2 / 1617.
-constexpr int F32_TWO_CTAS = 1024;
+// hide each other's latency and want the registers (80 and 114, 48 and 64 with one four): 2 x 192 nodes (1536 CTAs) 592.1 / 1606 against 596.2 / 1617;
+// head_dim 128, 512 CTAs (8 x 16 nodes behind 500 keys) 666 -> 651, 1024 (a prompt of 256) 714 -> 721.
+constexpr int F32_TWO_CTAS = 1024;      // (of head_dim 64)
 // Of the tree's keys a node sees only its ancestors: their indices are laid out in shared memory first, so that the fours are full
 // (2 x 192 nodes x 4 heads behind 16 keys: 9.8 us; 37.0 with fours of neighbouring keys, 18.5 with single ones that skip).
 constexpr int F32_WARPS = 8;
@@ -1273,7 +1274,8 @@ __global__ void __launch_bounds__(F32_WARPS * 32) tree_attn_f32_kernel(const flo
   __shared__ float s_m[F32_WARPS], s_l[F32_WARPS];
   __shared__ short s_key[CERB_MAX_NODES];
   static_assert(F32_WARPS * 32 >= CERB_MAX_NODES, "a thread per tree key");
-  if (!ahead) {
+  const bool late = !TWO || !ahead;
+  if (late) {
     griddep_wait();
     griddep_launch();
   }
@@ -1282,7 +1284,7 @@ __global__ void __launch_bounds__(F32_WARPS * 32) tree_attn_f32_kernel(const flo
   const int nq_all = (n_active ? min(n_active[b], n) : n) - shift;
   const int nq = win > 1 ? min(nq_all, kAttnRowsPerLaunch) : nq_all;
   if (i >= nq) {
-    griddep_wait();      // (no CTA leaves ahead of the kernel in front; at once where it has waited already)
+    if (!late) griddep_wait();      // (no CTA leaves ahead of the kernel in front)
     return;
   }
   const int settled = len[b], L = settled + shift, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -1306,9 +1308,8 @@ __global__ void __launch_bounds__(F32_WARPS * 32) tree_attn_f32_kernel(const flo
   // other was a chain of two round trips to memory and a reduction per key.
   constexpr int KEYS = 4, ROUND = F32_WARPS * KEYS;
   const int first = warp * KEYS, end = L + seen;
-  auto fetch = [&](int base, float (&kv)[KEYS][E], float (&vv)[KEYS][E]) {
+  auto fetch = [&](int base, float (&kv)[KEYS][E], float (&vv)[KEYS][E], bool (&sees)[KEYS]) {
     size_t off[KEYS];
-    bool sees[KEYS];
 #pragma unroll
     for (int u = 0; u < KEYS; ++u) {
       int kpos = base + u;
@@ -1325,7 +1326,7 @@ __global__ void __launch_bounds__(F32_WARPS * 32) tree_attn_f32_kernel(const flo
         vv[u][e] = sees[u] ? vpool[off[u] + lane + 32 * e] : 0.f;
       }
   };
-  auto take = [&](int base, const float (&kv)[KEYS][E], const float (&vv)[KEYS][E]) {
+  auto take = [&](const float (&kv)[KEYS][E], const float (&vv)[KEYS][E], const bool (&sees)[KEYS]) {
     float s[KEYS];
 #pragma unroll
     for (int u = 0; u < KEYS; ++u) {
@@ -1340,7 +1341,7 @@ __global__ void __launch_bounds__(F32_WARPS * 32) tree_attn_f32_kernel(const flo
     float mn = m;
 #pragma unroll
     for (int u = 0; u < KEYS; ++u) {
-      s[u] = base + u < end ? s[u] * scale : -INFINITY;
+      s[u] = sees[u] ? s[u] * scale : -INFINITY;
       mn = fmaxf(mn, s[u]);
     }
     if (mn == -INFINITY) return;                         // (nothing seen so far; uniform over the warp)
@@ -1358,26 +1359,27 @@ __global__ void __launch_bounds__(F32_WARPS * 32) tree_attn_f32_kernel(const flo
     m = mn;
   };
   float ka[KEYS][E], va[KEYS][E], kb[KEYS][E], vb[KEYS][E];              // TWO: two fours in turn
-  const bool early_a = TWO && ahead && first + KEYS <= settled, early_b = TWO && ahead && first + ROUND + KEYS <= settled;
-  if (early_a) fetch(first, ka, va);
-  if (early_b) fetch(first + ROUND, kb, vb);
-  if (ahead) {
+  bool sa[KEYS], sb[KEYS];
+  const bool early_a = !late && first + KEYS <= settled, early_b = !late && first + ROUND + KEYS <= settled;
+  if (early_a) fetch(first, ka, va, sa);
+  if (early_b) fetch(first + ROUND, kb, vb, sb);
+  if (!late) {
     griddep_wait();
     griddep_launch();
   }
 #pragma unroll
   for (int e = 0; e < E; ++e) { qv[e] = qp[lane + 32 * e]; acc[e] = 0.f; }
   if (!TWO) {
-    for (int base = first; base < end; base += ROUND) { fetch(base, ka, va); take(base, ka, va); }
+    for (int base = first; base < end; base += ROUND) { fetch(base, ka, va, sa); take(ka, va, sa); }
   } else if (!early_a) {
-    fetch(first, ka, va);
+    fetch(first, ka, va, sa);
   }
   for (int base = first; TWO && base < end; base += 2 * ROUND) {
-    if (base + ROUND < end && !(early_b && base == first)) fetch(base + ROUND, kb, vb);
-    take(base, ka, va);
+    if (base + ROUND < end && !(early_b && base == first)) fetch(base + ROUND, kb, vb, sb);
+    take(ka, va, sa);
     if (base + ROUND >= end) break;
-    if (base + 2 * ROUND < end) fetch(base + 2 * ROUND, ka, va);
-    take(base + ROUND, kb, vb);
+    if (base + 2 * ROUND < end) fetch(base + 2 * ROUND, ka, va, sa);
+    take(kb, vb, sb);
   }
   for (int e = 0; e < E; ++e) s_o[warp][lane + 32 * e] = acc[e];
   if (lane == 0) { s_m[warp] = m; s_l[warp] = l; }
@@ -1660,10 +1662,10 @@ int launch_tree_attention(cerb_ctx* c, const cerb_attn_args* a, const CUtensorMa
   const int win = chain ? (a->n + kAttnRowsPerLaunch - 1) / kAttnRowsPerLaunch : 1;
   if (a->dtype == CERB_F32) {
     dim3 grid(win > 1 ? kAttnRowsPerLaunch : a->n, a->n_heads, a->B * win);
-    const bool two = (long long)grid.x * grid.y * grid.z <= F32_TWO_CTAS;
+    const bool two = (long long)grid.x * grid.y * grid.z * a->head_dim <= F32_TWO_CTAS * 64;
     auto go = [&](auto kern) {
       launch_pdl(kern, grid, dim3(F32_WARPS * 32), 0, st, (const float*)a->q, (const float*)a->k_pool, (const float*)a->v_pool, a->page_table, a->len,
-                 a->n_active, a->anc, (float*)a->out, a->lse, a->n, a->n_heads, a->max_pages, a->scale, row_off, win, c ? 1 : 0);
+                 a->n_active, a->anc, (float*)a->out, a->lse, a->n, a->n_heads, a->max_pages, a->scale, row_off, win, c && two ? 1 : 0);
     };
     if (a->head_dim == 64)
       two ? go(tree_attn_f32_kernel<64, true>) : go(tree_attn_f32_kernel<64, false>);

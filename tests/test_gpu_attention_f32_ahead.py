@@ -13,7 +13,7 @@ pytestmark = pytest.mark.gpu
 CHAIN = 6        # nodes of the longest path; the tree's other nodes hang on the root
 
 
-# up to 1024 (node, head) pairs two rounds in turn, above one
+# up to 1024 (node, head) pairs, 512 at head_dim 128, two rounds in turn; above one
 @pytest.mark.parametrize("head_dim", [64, 128])
 @pytest.mark.parametrize("B,n", [(1, CHAIN), (3, 20), (16, 17)])
 def test_verified_chain_is_the_prompt_it_spells(B, n, head_dim):
