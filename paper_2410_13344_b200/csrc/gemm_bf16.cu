@@ -132,6 +132,7 @@ __global__ void __launch_bounds__(224, 1) gemm_bf16_kernel(const __grid_constant
   tc_fence_after();
   const uint32_t tmem_base = tmem_base_slot;
 
+  int issued = 0;                                      // warp 0, lane 0: units whose copies it has issued
   if (warp == 0) {
     if (lane == 0) {
       const int n_units = u1 - u0;
@@ -169,7 +170,7 @@ __global__ void __launch_bounds__(224, 1) gemm_bf16_kernel(const __grid_constant
       griddep_launch();
       if (p.clk) atomicMin(p.clk, globaltimer_ns());
       for (int i = 0; i < pre; ++i) load_x(i);
-      int issued = pre;
+      issued = pre;
       for (int i = pre; i < n_units; ++i) {
         const int s = i % p.stages;
         const uint32_t ph = (uint32_t)(i / p.stages) & 1u;
@@ -177,11 +178,6 @@ __global__ void __launch_bounds__(224, 1) gemm_bf16_kernel(const __grid_constant
         load_w(i);
         load_x(i);
         issued = i + 1;
-      }
-      if (*aborted) {
-        // give-up path: the copies already issued still land in this CTA's shared memory; see each of them in
-        for (int i = issued > p.stages ? issued - p.stages : 0; i < issued; ++i)
-          mbar_wait_drain(smem_u32(&full_bar[i % p.stages]), (uint32_t)(i / p.stages) & 1u);
       }
     }
   } else if (warp == 1 || warp == 6) {
@@ -217,11 +213,6 @@ __global__ void __launch_bounds__(224, 1) gemm_bf16_kernel(const __grid_constant
         if (*aborted) break;
         umma_commit(smem_u32(&acc_full[buf]));       // this thread's part of the segment's accumulator is complete
         ++g;
-      }
-      if (*aborted) {
-        // give-up path: the MMAs already issued still read shared memory and write tensor memory; see them retire
-        umma_commit(smem_u32(&drain_bar[hf]));
-        mbar_wait_drain(smem_u32(&drain_bar[hf]), 0);
       }
     }
   } else {
@@ -281,7 +272,20 @@ __global__ void __launch_bounds__(224, 1) gemm_bf16_kernel(const __grid_constant
     }
   }
   tc_fence_before();
-  __syncthreads();
+  if (__syncthreads_or(*aborted)) {
+    // Give-up path: whichever role's wait ran out, what the others have begun is seen in here, where all of them have stopped.
+    if ((warp == 1 || warp == 6) && lane == 0) {
+      // the MMAs issued still read shared memory and write tensor memory
+      const uint32_t bar = smem_u32(&drain_bar[warp == 6 ? 1 : 0]);
+      umma_commit(bar);
+      mbar_wait_drain(bar, 0);
+    } else if (warp == 0 && lane == 0) {
+      // the copies issued still land in this CTA's shared memory
+      for (int i = issued > p.stages ? issued - p.stages : 0; i < issued; ++i)
+        mbar_wait_drain(smem_u32(&full_bar[i % p.stages]), (uint32_t)(i / p.stages) & 1u);
+    }
+    __syncthreads();
+  }
   if (p.clk && threadIdx.x == 0) atomicMax(p.clk + kGemmClockSlots, globaltimer_ns());
   if (warp == 1) {
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(2u * p.acc_cols) : "memory");

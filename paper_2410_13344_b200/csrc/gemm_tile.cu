@@ -299,6 +299,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tile_kernel(const __grid_con
   cluster_start_wait();
   const uint32_t tmem_base = tmem_base_slot;
 
+  int issued = 0;                  // warp 0, lane 0: stages whose copies it has issued
   if (warp == 0) {
     if (lane == 0) {
       // weights that several row chunks read, at different times where tiles are cut along k, stay in L2 like anything else
@@ -327,7 +328,6 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tile_kernel(const __grid_con
         --rx.nkb;
         qx.next(p.stages);
       };
-      int issued = 0;
       for (; issued < p.stages && more_w(); ++issued) load_w();
       asm volatile("prefetch.tensormap [%0];" ::"l"((uint64_t)&tmX) : "memory");
       griddep_wait();
@@ -338,17 +338,6 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tile_kernel(const __grid_con
         if (!mbar_wait_cluster(smem_u32(&empty_bar[qw.s]), qw.ph ^ 1u, wc, 221)) break;
         load_w();
         load_x();
-      }
-      if (*aborted) {
-        // give-up path: this CTA's copies land in its own shared memory but are counted on the first CTA's
-        // barriers, and the two CTAs may have stopped at different stages, so neither can see exactly its own
-        // copies in.  The first CTA waits for the stages it knows of (short budget); then both let the time of
-        // many memory round trips pass before they go on to the rendezvous and leave.
-        if (first)
-          for (int i = issued > p.stages ? issued - p.stages : 0; i < issued; ++i)
-            mbar_wait_drain(smem_u32(&full_bar[i % p.stages]), (uint32_t)(i / p.stages) & 1u, 2000000ll);
-        const long long t_land = clock64();
-        while (clock64() - t_land < 400000ll) __nanosleep(1000);
       }
     }
   } else if (warp == 1) {
@@ -424,10 +413,6 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tile_kernel(const __grid_con
           q0 = q;
           ++g;
         }
-      }
-      if (!live && elect_one()) {
-        asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(&drain_bar)) : "memory");
-        mbar_wait_drain(smem_u32(&drain_bar), 0, 40000000ll);
       }
     }
   } else {
@@ -615,7 +600,25 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tile_kernel(const __grid_con
     }
   }
   tc_fence_before();
-  __syncthreads();
+  if (__syncthreads_or(*aborted)) {
+    // Give-up path: whichever role's wait ran out, what the others have begun is seen in here, where all of them have stopped.
+    if (warp == 1 && first && elect_one()) {
+      // the MMAs issued still read shared memory and write tensor memory
+      asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(&drain_bar)) : "memory");
+      mbar_wait_drain(smem_u32(&drain_bar), 0, 40000000ll);
+    } else if (warp == 0 && lane == 0) {
+      // This CTA's copies land in its own shared memory but are counted on the first CTA's
+      // barriers, and the two CTAs may have stopped at different stages, so neither can see exactly its own
+      // copies in.  The first CTA waits for the stages it knows of (short budget); then both let the time of
+      // many memory round trips pass before they go on to the rendezvous and leave.
+      if (first)
+        for (int i = issued > p.stages ? issued - p.stages : 0; i < issued; ++i)
+          mbar_wait_drain(smem_u32(&full_bar[i % p.stages]), (uint32_t)(i / p.stages) & 1u, 2000000ll);
+      const long long t_land = clock64();
+      while (clock64() - t_land < 400000ll) __nanosleep(1000);
+    }
+    __syncthreads();
+  }
   if (p.clk && threadIdx.x == 0) atomicMax(p.clk + kGemmClockSlots, globaltimer_ns());
   // Neither CTA leaves (nor frees its tensor memory) before the other is done: copies, commits and arrivals cross
   // between them until then.  The rendezvous keeps a budget of its own, far above that of the other waits, so that a

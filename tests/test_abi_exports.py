@@ -156,6 +156,26 @@ def test_no_forward_kernel_leaves_ahead_of_its_wait():
     assert seen >= 12
 
 
+def test_what_is_in_flight_is_seen_in_after_every_role_has_stopped():
+    """A kernel that gives up must not let a copy outlive its shared memory, nor an MMA its tensor memory.  Any role's wait may be the one that
+    runs out, when the others have already done all of theirs: so copies and MMAs are waited for behind the point where all threads of the CTA
+    meet and learn whether one of them gave up, and not inside the roles."""
+    src = os.path.join(ROOT, "paper_2410_13344_b200", "csrc")
+    seen = 0
+    for fn in ("gemm_bf16.cu", "gemm_tile.cu"):
+        text = re.sub(r"//[^\n]*", "", open(os.path.join(src, fn)).read())
+        for body in re.split(r"__global__", text)[1:]:
+            body = body[:body.index("\n}\n")]
+            if "WaitCtx wc" not in body:
+                continue
+            seen += 1
+            assert body.count("__syncthreads_or(*aborted)") == 1, (fn, body[:80])
+            met = body.index("__syncthreads_or(*aborted)")
+            assert "mbar_wait_drain(" in body[met:] and "mbar_wait_drain(" not in body[:met], (fn, body[:80])
+            assert "tcgen05.dealloc" not in body[:met], (fn, body[:80])
+    assert seen == 2
+
+
 def test_the_read_before_wait_rule_holds_in_every_variant():
     """The rule of test_no_kernel_reads_before_its_wait_what_the_kernel_in_front_writes over all exported launch sequences, those of
     the forwards (0, 3, 5, 6, 7, 8) among them."""
