@@ -188,6 +188,7 @@ __global__ void __launch_bounds__(KT_THREADS, 1) tree_attn_kt_kernel(const __gri
   static_assert(NU % 2 == 0, "a slot holds units of one kind");
   auto unit_parity = [](int u) { return (uint32_t)(u / NU) & 1u; };
   auto wait_unit = [&](int u, int site) { return mbar_wait(smem_u32(&full_u[u & 1][u % NU]), unit_parity(u), wc, site); };
+  int issued = -1;                                   // producers: units of this warp's kind whose copies it has issued, -1: none of any kind
   if (warp >= NSW && warp < NSW + NPROD) {
     // ---------------- TMA producers ----------------
     // One half of the producers fetches K units, the other V units (neighbouring slots of an even ring belong to one kind each): a
@@ -212,7 +213,6 @@ __global__ void __launch_bounds__(KT_THREADS, 1) tree_attn_kt_kernel(const __gri
     const int box = (pw >> 1) + (NPROD / 2) * lane;  // lanes 0 .. BOXES-1
     const int pg = box >> 1, hf = box & 1;
     const uint64_t pol = l2_policy(true);            // K/V are read once per step
-    int issued = 0;
     // (the abort flag itself is looked at once, for a launch that starts after a time-out: nothing is issued then;
     // later a wait that gives up says so in its return value, which costs the loop nothing)
     const int t_stop = *aborted ? 0 : T;
@@ -227,7 +227,7 @@ __global__ void __launch_bounds__(KT_THREADS, 1) tree_attn_kt_kernel(const __gri
         tma_load_2d_hint(ring + (uint32_t)hf * KT_HALF + (uint32_t)pg * (CERB_PAGE * 128), &tmK, hf * 64, page_list[pg], smem_u32(&full_u[0][0]), pol);
       issued = 1 - kind;
     }
-    for (int t = issued; t < t_stop; ++t) {
+    for (int t = max(issued, 0); t < t_stop; ++t) {
       if (t == early) enter();
       const int u = 2 * t + kind, slot = u % NU;
       const uint32_t fb = smem_u32(&full_u[kind][slot]);
@@ -243,13 +243,6 @@ __global__ void __launch_bounds__(KT_THREADS, 1) tree_attn_kt_kernel(const __gri
         tma_load_2d_hint(dst, kind ? &tmV : &tmK, hf * 64, row, fb, pol);
       }
       issued = t + 1;
-    }
-    if (lane == 0 && *aborted) {
-      // give-up path: the copies this warp has issued still land in the CTA's shared memory; see them in (the
-      // phase also needs the other producers' shares, hence a limit of its own: 10 ms)
-      if (kind && t_stop > 0) mbar_wait_drain(smem_u32(&full_u[0][0]), 0, 20000000ll);
-      for (int t = issued > NU / 2 ? issued - NU / 2 : 0; t < issued; ++t)
-        mbar_wait_drain(smem_u32(&full_u[kind][(2 * t + kind) % NU]), unit_parity(2 * t + kind), 20000000ll);
     }
     enter();             // (a lane that has waited already returns at once)
   } else if (warp == W_QK) {
@@ -278,10 +271,6 @@ __global__ void __launch_bounds__(KT_THREADS, 1) tree_attn_kt_kernel(const __gri
         }
         __syncwarp();
       }
-      if (__any_sync(0xffffffffu, *aborted) && elect_one()) {                                // give-up path: see the MMAs already issued retire
-        umma_commit(smem_u32(&drain_bar[0]));
-        mbar_wait_drain(smem_u32(&drain_bar[0]), 0, 20000000ll);
-      }
     }
   } else if (warp == W_PV) {
     enter();
@@ -308,10 +297,6 @@ __global__ void __launch_bounds__(KT_THREADS, 1) tree_attn_kt_kernel(const __gri
           umma_commit(smem_u32(&pv_done[pb]));
         }
         __syncwarp();
-      }
-      if (__any_sync(0xffffffffu, *aborted) && elect_one()) {                                // give-up path: see the MMAs already issued retire
-        umma_commit(smem_u32(&drain_bar[1]));
-        mbar_wait_drain(smem_u32(&drain_bar[1]), 0, 20000000ll);
       }
       if (p.cluster) {
         // Q is staged and every MMA has retired: this CTA's rx may be written.  (Said from here the release costs the softmax warps nothing.)
@@ -683,7 +668,23 @@ __global__ void __launch_bounds__(KT_THREADS, 1) tree_attn_kt_kernel(const __gri
     griddep_launch();
   }
   tc_fence_before();
-  __syncthreads();                             // nobody exits before warp 0 has seen every member done
+  if (__syncthreads_or(*aborted)) {            // (nobody exits before warp 0 has seen every member done)
+    // Give-up path, where every role has stopped (see tree_attn_tc_kernel)
+    if (warp >= NSW && warp < NSW + NPROD) {
+      // (a phase also needs the other producers' shares, hence a limit of its own: 10 ms)
+      if (lane == 0) {
+        const int kind = (warp - NSW) & 1;
+        if (kind && issued >= 0) mbar_wait_drain(smem_u32(&full_u[0][0]), 0, 20000000ll);
+        for (int t = issued > NU / 2 ? issued - NU / 2 : 0; t < issued; ++t)
+          mbar_wait_drain(smem_u32(&full_u[kind][(2 * t + kind) % NU]), unit_parity(2 * t + kind), 20000000ll);
+      }
+    } else if ((warp == W_QK || warp == W_PV) && elect_one()) {
+      const uint32_t bar = smem_u32(&drain_bar[warp == W_PV ? 1 : 0]);
+      umma_commit(bar);
+      mbar_wait_drain(bar, 0, 20000000ll);
+    }
+    __syncthreads();
+  }
   if (warp == W_QK) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TMEM_COLS) : "memory");
 }
 
