@@ -147,6 +147,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_rows_kernel(const __grid_con
     return CG == 2 ? mbar_wait_cluster(smem_u32(&bar), parity, wc, site) : mbar_wait(smem_u32(&bar), parity, wc, site);
   };
 
+  int issued = 0;                 // warp 0, lane 0: k blocks whose copies it has issued
   if (warp == 0) {
     if (lane == 0) {
       const uint64_t pol_w = l2_policy(true), pol_x = l2_policy(false);
@@ -169,7 +170,8 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_rows_kernel(const __grid_con
       griddep_launch();                                    // (only now: see launch_order.cu)
       if (p.clk) atomicMin(p.clk, globaltimer_ns());
       for (int i = 0; i < pre; ++i) load_x(i, i);
-      int issued = pre, s = 0;
+      issued = pre;
+      int s = 0;
       uint32_t ph = 0;
       for (int i = pre; i < num_kb; ++i) {
         if (!wait(empty_bar[s], ph, 241)) break;
@@ -177,15 +179,6 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_rows_kernel(const __grid_con
         load_x(i, s);
         issued = i + 1;
         if (++s == p.stages) { s = 0; ph ^= 1u; }
-      }
-      if (*aborted) {
-        // give-up path: the copies already issued still land in this CTA's shared memory; see each of them in.  (A pair's are counted on
-        // the first CTA's barriers, and the CTAs may have stopped at different stages: both let the time of many round trips pass, too.)
-        if (first)
-          for (int i = issued > p.stages ? issued - p.stages : 0; i < issued; ++i)
-            mbar_wait_drain(smem_u32(&full_bar[i % p.stages]), (uint32_t)(i / p.stages) & 1u, CG == 2 ? 2000000ll : kDrainCycles);
-        const long long t_land = clock64();
-        while (CG == 2 && clock64() - t_land < 400000ll) __nanosleep(1000);
       }
     }
   } else if (warp <= kIssuers) {
@@ -250,17 +243,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_rows_kernel(const __grid_con
           if (++s == p.stages) { s = 0; ph ^= 1u; }
         }
       }
-      if (elect_one()) {
-        if (!live) {
-          // give-up path: the MMAs already issued still read shared memory and write tensor memory; see them retire
-          if constexpr (CG == 2)
-            asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(&drain_bar[self])) : "memory");
-          else umma_commit(smem_u32(&drain_bar[self]));
-          mbar_wait_drain(smem_u32(&drain_bar[self]), 0, CG == 2 ? 40000000ll : kDrainCycles);
-        } else {
-          commit(acc_full);
-        }
-      }
+      if (live && elect_one()) commit(acc_full);
     }
   } else if (warp >= 4) {
     const int quarter = warp & 3, part = (warp >> 2) - 1;
@@ -457,7 +440,29 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_rows_kernel(const __grid_con
     }
   }
   tc_fence_before();
-  __syncthreads();
+  if (__syncthreads_or(*aborted)) {
+    // Give-up path.  Which role's wait runs out first is open, and the others may have done all of theirs by then: so what is in flight is seen
+    // in here, where every role has stopped, by the threads that have begun it.
+    if (warp >= 1 && warp <= kIssuers) {
+      // the MMAs issued still read shared memory and write tensor memory
+      const int self = warp - 1;
+      if (first && self < p.issuers && elect_one()) {
+        if constexpr (CG == 2)
+          asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(&drain_bar[self])) : "memory");
+        else umma_commit(smem_u32(&drain_bar[self]));
+        mbar_wait_drain(smem_u32(&drain_bar[self]), 0, CG == 2 ? 40000000ll : kDrainCycles);
+      }
+    } else if (warp == 0 && lane == 0) {
+      // The copies still land in this CTA's shared memory.  (A pair's are counted on the first CTA's barriers, and the CTAs may have stopped at
+      // different stages: both let the time of many round trips pass, too.)
+      if (first)
+        for (int i = issued > p.stages ? issued - p.stages : 0; i < issued; ++i)
+          mbar_wait_drain(smem_u32(&full_bar[i % p.stages]), (uint32_t)(i / p.stages) & 1u, CG == 2 ? 2000000ll : kDrainCycles);
+      const long long t_land = clock64();
+      while (CG == 2 && clock64() - t_land < 400000ll) __nanosleep(1000);
+    }
+    __syncthreads();
+  }
   if (p.clk && threadIdx.x == 0) atomicMax(p.clk + kGemmClockSlots, globaltimer_ns());
   if constexpr (CG == 2) {
     // Neither CTA leaves (nor frees its tensor memory) before the other is done: copies, commits and arrivals cross between them until then.

@@ -162,7 +162,9 @@ def test_what_is_in_flight_is_seen_in_after_every_role_has_stopped():
     meet and learn whether one of them gave up, and not inside the roles."""
     src = os.path.join(ROOT, "paper_2410_13344_b200", "csrc")
     seen = 0
-    for fn in ("gemm_bf16.cu", "gemm_tile.cu", "attention.cu", "attention_kt.cuh"):
+    for fn in sorted(os.listdir(src)):
+        if not fn.endswith((".cu", ".cuh")):
+            continue
         text = re.sub(r"//[^\n]*", "", open(os.path.join(src, fn)).read())
         for body in re.split(r"__global__", text)[1:]:
             body = body[:body.index("\n}\n")]
@@ -173,7 +175,7 @@ def test_what_is_in_flight_is_seen_in_after_every_role_has_stopped():
             met = body.index("__syncthreads_or(*aborted)")
             assert "mbar_wait_drain(" in body[met:] and "mbar_wait_drain(" not in body[:met], (fn, body[:80])
             assert "tcgen05.dealloc" not in body[:met], (fn, body[:80])
-    assert seen == 5
+    assert seen == 6
 
 
 def test_the_read_before_wait_rule_holds_in_every_variant():

@@ -98,3 +98,28 @@ def test_lm_head_sums(vocab, n):
     assert eng.device_status() == 0
     assert close(logits[0], orc.linear(hidden[0].cpu(), model["lm_head"].cpu()), 0) < 1e-4
     assert torch.equal(top[0].long(), logits[0].argmax(-1)) and torch.equal(eng.verify(eng.tree(tree), tt)[0], top)
+
+
+@pytest.mark.parametrize("M", [64, 256])
+def test_a_forward_whose_waits_run_out_comes_back_and_the_next_one_is_correct(M):
+    """With the budget of every wait at a thousand cycles the epilogue warps of the gate-up product (11008 features of 16384 columns: over 100 us
+    of weights) run out of it by the limit alone, in single CTAs and in pairs, while copies and MMAs are in flight.  The forward must come back
+    with CERB_E_TIMEOUT from a wait of this kernel, and the same forward with the default budget must give the bits it gave before."""
+    ms = synth.ModelShape(1, 16384, 4, 128, 11008, 512, "bf16")
+    eng = cb.Cerberus(ms, synth.make_model(ms, device="cuda", std=0.01), None, None, [], max_tokens=M + 16, max_batch=1, max_nodes=16)
+    tok = torch.tensor([[int(t) for t in synth.make_prompt(ms.vocab, M, seq=180)]], dtype=torch.int32, device="cuda")
+
+    def forward():
+        eng.prefill(tok, [M])
+        return eng.wait_diagnosis(), eng.device_status(), eng.read_state()[2].clone()
+
+    _, status, want = forward()
+    assert status == cb.OK
+    assert cb.lib().cerb_set_wait_cycles(1000) == cb.OK
+    try:
+        words, status, _ = forward()
+    finally:
+        assert cb.lib().cerb_set_wait_cycles(4_000_000_000) == cb.OK
+    assert status == cb.E_TIMEOUT and 241 <= words[1] <= 246, words
+    _, status, got = forward()
+    assert status == cb.OK and torch.equal(got, want)
