@@ -169,8 +169,8 @@ __global__ void __launch_bounds__((WQ * WK + 1) * 32) tree_attn_bf16_kernel(cons
 
   float* mrg = reinterpret_cast<float*>(smem_gen);   // [NQ][ROWF], used after the key loop
 
-  int issued = 0;                                    // producer: tiles whose copies it has issued
   if (warp == NW) {
+    int issued = 0;                                    // (lane 0: tiles whose copies it has issued)
     // ---------------- producer warp ----------------
     const int32_t* pt = p.page_table + (size_t)b * p.max_pages;
     const int n_pages = (t_end - t0) * PAGES_PER_TILE;
@@ -208,6 +208,7 @@ __global__ void __launch_bounds__((WQ * WK + 1) * 32) tree_attn_bf16_kernel(cons
     }
     griddep_wait();      // (a lane that has waited already returns at once)
     griddep_launch();
+    see_own_copies_in(smem_u32(&full_bar[0]), STAGES, issued, lane, 20000000ll);
   } else {
     // ---------------- compute warps ----------------
     griddep_wait();
@@ -481,12 +482,7 @@ __global__ void __launch_bounds__((WQ * WK + 1) * 32) tree_attn_bf16_kernel(cons
       compute_bar(NW * 32);                                                          // this CTA has read all it needs
       if (warp == 0) cluster_meet_before_exit(&cl_bar[1], p.nsplit, lane, wc, &exit_flag_s, 304);
     }
-  }
-  // (nobody exits before warp 0 has seen every member done)
-  if (__syncthreads_or(*aborted) && warp == NW && lane == 0) {
-    // give-up path: whoever's wait ran out, the copies issued (units 0 .. issued - 1) still land in this CTA's shared memory; see each of them in
-    for (int j = issued > STAGES ? issued - STAGES : 0; j < issued; ++j)
-      mbar_wait_drain(smem_u32(&full_bar[j % STAGES]), (uint32_t)(j / STAGES) & 1u, 20000000ll);
+    __syncthreads();                           // nobody exits before warp 0 has seen every member done
   }
 }
 
@@ -638,7 +634,6 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tree_attn_tc_kernel(const __gri
   const uint32_t tmem = tmem_slot;
   float* mrg = reinterpret_cast<float*>(smem_gen);   // [2][128][ROWF] over the whole buffer, once the key loop is over
 
-  int issued = 0;                                  // producers: tiles whose copies this warp has issued
   if (warp == 0 || warp == 11) {
     // ---------------- TMA producers: warp 0 the K tiles, warp 11 the V tiles ----------------
     // A tile of K (or V) is 8 boxes of 2 KB (four pages, two 64-wide halves), issued by 8 lanes.  Issuing a box occupies its
@@ -652,7 +647,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tree_attn_tc_kernel(const __gri
     static_assert(PAGES_PER_TILE == 4, "the lane -> box map below assumes four pages per tile");
     const int pg = (lane >> 1) & 3, hf = lane & 1;
     bool go = !__any_sync(0xffffffffu, *aborted), waited = false;         // a launch that starts after a time-out issues nothing
-    int slot = 0;
+    int issued = 0, slot = 0;
     uint32_t ph = 0;
     for (int round = 0; go && round < rounds; ++round) {
       const Item it = item_at(round);
@@ -684,6 +679,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tree_attn_tc_kernel(const __gri
       }
     }
     enter();             // (a lane that has waited already returns at once)
+    see_own_copies_in(smem_u32(full), ring, issued, lane, 20000000ll);
   } else if (warp == 1) {
     enter();
     // ---------------- QK^T issuer ----------------
@@ -720,6 +716,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tree_attn_tc_kernel(const __gri
           if (++slot == SK) { slot = 0; ph ^= 1u; }
         }
       }
+      if (elect_one()) see_mmas_retire<1>(smem_u32(&drain_bar[0]), 20000000ll);
     }
   } else if (warp == 10) {
     enter();
@@ -754,6 +751,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tree_attn_tc_kernel(const __gri
           if (++slot == SV) { slot = 0; vph ^= 1u; }
         }
       }
+      if (elect_one()) see_mmas_retire<1>(smem_u32(&drain_bar[1]), 20000000ll);
     }
   } else {
     // ---------------- softmax groups: thread <-> query row, group g takes tiles g, g+2, ... ----------------
@@ -1077,21 +1075,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tree_attn_tc_kernel(const __gri
     griddep_launch();
   }
   tc_fence_before();
-  if (__syncthreads_or(*aborted)) {            // (nobody exits before warp 2 has seen every member done)
-    // Give-up path: whichever role's wait ran out, what the others have begun is seen in here, where all of them have stopped: copies still
-    // land in this CTA's shared memory, MMAs still read it and write tensor memory.
-    if ((warp == 0 || warp == 11) && lane == 0) {
-      const int ring = warp == 11 ? SV : SK;
-      uint64_t* full = warp == 11 ? full_v : full_k;
-      for (int j = issued > ring ? issued - ring : 0; j < issued; ++j)
-        mbar_wait_drain(smem_u32(&full[j % ring]), (uint32_t)(j / ring) & 1u, 20000000ll);
-    } else if ((warp == 1 || warp == 10) && elect_one()) {
-      const uint32_t bar = smem_u32(&drain_bar[warp == 10 ? 1 : 0]);
-      umma_commit(bar);
-      mbar_wait_drain(bar, 0, 20000000ll);
-    }
-    __syncthreads();
-  }
+  __syncthreads();                             // nobody exits before warp 2 has seen every member done
   if (warp == 1) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512u) : "memory");
 }
 

@@ -75,6 +75,16 @@ __device__ __noinline__ bool wait_for_partner(uint32_t bar, long long budget) {
   return mbar_wait_drain(bar, 0, partner_cycles(w));
 }
 
+// What see_own_copies_in is for, of the units of one kind (t-th: unit 2 t + kind, in slot u % nu) that a producer has issued, and of its boxes of the first K unit (of
+// more units than slots the last ones go out only when the first have been used).  A phase also needs the other producers' shares.
+static __device__ __noinline__ void see_units_in(uint32_t first_unit, uint32_t full, int kind, int issued, int nu) {
+  if (kind && issued >= 0 && issued <= nu / 2) mbar_wait_drain(first_unit, 0, 20000000ll);
+  for (int t = issued > nu / 2 ? issued - nu / 2 : 0; t < issued; ++t) {
+    const int u = 2 * t + kind;
+    mbar_wait_drain(full + 8u * (uint32_t)(u % nu), (uint32_t)(u / nu) & 1u, 20000000ll);
+  }
+}
+
 template <bool PART>
 __global__ void __launch_bounds__(KT_THREADS, 1) tree_attn_kt_kernel(const __grid_constant__ CUtensorMap tmK,
                                                                      const __grid_constant__ CUtensorMap tmV,
@@ -188,7 +198,6 @@ __global__ void __launch_bounds__(KT_THREADS, 1) tree_attn_kt_kernel(const __gri
   static_assert(NU % 2 == 0, "a slot holds units of one kind");
   auto unit_parity = [](int u) { return (uint32_t)(u / NU) & 1u; };
   auto wait_unit = [&](int u, int site) { return mbar_wait(smem_u32(&full_u[u & 1][u % NU]), unit_parity(u), wc, site); };
-  int issued = -1;                                   // producers: units of this warp's kind whose copies it has issued, -1: none of any kind
   if (warp >= NSW && warp < NSW + NPROD) {
     // ---------------- TMA producers ----------------
     // One half of the producers fetches K units, the other V units (neighbouring slots of an even ring belong to one kind each): a
@@ -213,6 +222,7 @@ __global__ void __launch_bounds__(KT_THREADS, 1) tree_attn_kt_kernel(const __gri
     const int box = (pw >> 1) + (NPROD / 2) * lane;  // lanes 0 .. BOXES-1
     const int pg = box >> 1, hf = box & 1;
     const uint64_t pol = l2_policy(true);            // K/V are read once per step
+    int issued = -1;                                 // units of this warp's kind whose copies it has issued, -1: none of any kind
     // (the abort flag itself is looked at once, for a launch that starts after a time-out: nothing is issued then;
     // later a wait that gives up says so in its return value, which costs the loop nothing)
     const int t_stop = *aborted ? 0 : T;
@@ -245,6 +255,7 @@ __global__ void __launch_bounds__(KT_THREADS, 1) tree_attn_kt_kernel(const __gri
       issued = t + 1;
     }
     enter();             // (a lane that has waited already returns at once)
+    if (lane == 0) see_units_in(smem_u32(&full_u[0][0]), smem_u32(&full_u[kind][0]), kind, issued, NU);
   } else if (warp == W_QK) {
     enter();
     // ---------------- QK^T issuer ----------------
@@ -271,6 +282,7 @@ __global__ void __launch_bounds__(KT_THREADS, 1) tree_attn_kt_kernel(const __gri
         }
         __syncwarp();
       }
+      if (elect_one()) see_mmas_retire<1>(smem_u32(&drain_bar[0]), 20000000ll);
     }
   } else if (warp == W_PV) {
     enter();
@@ -306,6 +318,7 @@ __global__ void __launch_bounds__(KT_THREADS, 1) tree_attn_kt_kernel(const __gri
         cluster_start_wait();
         if (lane < p.nsplit) mbar_arrive_cluster(mapa_u32(smem_u32(&cl_bar[0]), (uint32_t)lane));
       }
+      if (elect_one()) see_mmas_retire<1>(smem_u32(&drain_bar[1]), 20000000ll);
     }
   } else {
     // ---------------- softmax: thread = (key lane of the tile, block of QB queries) ----------------
@@ -668,23 +681,7 @@ __global__ void __launch_bounds__(KT_THREADS, 1) tree_attn_kt_kernel(const __gri
     griddep_launch();
   }
   tc_fence_before();
-  if (__syncthreads_or(*aborted)) {            // (nobody exits before warp 0 has seen every member done)
-    // Give-up path, where every role has stopped (see tree_attn_tc_kernel)
-    if (warp >= NSW && warp < NSW + NPROD) {
-      // (a phase also needs the other producers' shares, hence a limit of its own: 10 ms)
-      if (lane == 0) {
-        const int kind = (warp - NSW) & 1;
-        if (kind && issued >= 0) mbar_wait_drain(smem_u32(&full_u[0][0]), 0, 20000000ll);
-        for (int t = issued > NU / 2 ? issued - NU / 2 : 0; t < issued; ++t)
-          mbar_wait_drain(smem_u32(&full_u[kind][(2 * t + kind) % NU]), unit_parity(2 * t + kind), 20000000ll);
-      }
-    } else if ((warp == W_QK || warp == W_PV) && elect_one()) {
-      const uint32_t bar = smem_u32(&drain_bar[warp == W_PV ? 1 : 0]);
-      umma_commit(bar);
-      mbar_wait_drain(bar, 0, 20000000ll);
-    }
-    __syncthreads();
-  }
+  __syncthreads();                             // nobody exits before warp 0 has seen every member done
   if (warp == W_QK) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TMEM_COLS) : "memory");
 }
 

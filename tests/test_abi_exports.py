@@ -156,12 +156,16 @@ def test_no_forward_kernel_leaves_ahead_of_its_wait():
     assert seen >= 12
 
 
-def test_what_is_in_flight_is_seen_in_after_every_role_has_stopped():
+def test_every_role_sees_in_what_it_has_begun():
     """A kernel that gives up must not let a copy outlive its shared memory, nor an MMA its tensor memory.  Any role's wait may be the one that
-    runs out, when the others have already done all of theirs: so copies and MMAs are waited for behind the point where all threads of the CTA
-    meet and learn whether one of them gave up, and not inside the roles."""
+    runs out, when the others have already done all of theirs: so an issuer waits for its MMAs at its end in every launch, and copies are waited for in
+    every launch by their producer (attention) or by the issuers, of which one that leaves early sees in all that the producer has issued.  (Of a
+    pair's copies the second CTA cannot see its own: a CTA that has given up also lets them land before the two meet.)"""
     src = os.path.join(ROOT, "paper_2410_13344_b200", "csrc")
-    seen = 0
+    always, leaving = r"see_(own_copies|units)_in\(", r"if \(!(live|__shfl_sync\(0xffffffffu, live, 0\))\) see_copies_in\("
+    # copies; MMAs; pairs
+    roles = {"gemm_bf16_kernel": (leaving, 1, 0), "gemm_tile_kernel": (leaving, 1, 1), "gemm_rows_kernel": (leaving, 1, 1),
+             "tree_attn_bf16_kernel": (always, 0, 0), "tree_attn_tc_kernel": (always, 2, 0), "tree_attn_kt_kernel": (always, 2, 0)}
     for fn in sorted(os.listdir(src)):
         if not fn.endswith((".cu", ".cuh")):
             continue
@@ -170,12 +174,14 @@ def test_what_is_in_flight_is_seen_in_after_every_role_has_stopped():
             body = body[:body.index("\n}\n")]
             if "WaitCtx wc" not in body:
                 continue
-            seen += 1
-            assert body.count("__syncthreads_or(*aborted)") == 1, (fn, body[:80])
-            met = body.index("__syncthreads_or(*aborted)")
-            assert "mbar_wait_drain(" in body[met:] and "mbar_wait_drain(" not in body[:met], (fn, body[:80])
-            assert "tcgen05.dealloc" not in body[:met], (fn, body[:80])
-    assert seen == 6
+            copies, mmas, pair = roles.pop(re.search(r"\b(\w+_kernel)\(", body).group(1))
+            assert len(re.findall(copies, body)) == 1 and len(re.findall(r"see_(own_copies|copies|units)_in\(", body)) == 1, fn
+            retire = [s for s in body.split("\n") if "see_mmas_retire" in s]
+            assert len(retire) == mmas and not any(w in s for s in retire for w in ("aborted", "live")), (fn, retire)
+            assert len(re.findall(r"if \(\*aborted\) let_pair_copies_land\(\);\s*cluster_meet_before_exit", body)) == pair, fn
+            if copies == leaving:                        # an issuer that leaves its loop early says so, whatever made it
+                assert not re.search(r"\*aborted\) break", body) and body.count("*(volatile int*)&issued_s = issued;") == 1, fn
+    assert not roles
 
 
 def test_the_read_before_wait_rule_holds_in_every_variant():
