@@ -298,6 +298,12 @@ int cerb_gemm_scratch_bytes(int32_t M, int32_t N, int32_t K, size_t* bytes_out);
  * rows, [2] rows of a chunk, [3] tiles, [4] CTA pairs per tile, [5] tiles cut along k into equal shares, [6] CTA pairs,
  * [7] chains of accumulations per output of a run (fused = 0: fills of an accumulator). */
 int cerb_gemm_plan(int32_t M, int32_t N, int32_t K, int32_t fused, int32_t* out8_host);
+/* Which kernel a bf16 forward of 9 to 256 rows gives one of its products to (host only, for tests and measurement).  product: 0 QKV
+ * (head_dim 128), 1 O or down (above 128 rows where both are taken), 2 gate-up, 3 LM head.  out9_host: [0] 1 if the kernel with a weight tile per SM or
+ * pair of SMs takes it, then [1] groups of eight weight rows per CTA, [2] parts that k is cut into, [3] MMA issuers, [4] accumulators,
+ * [5] the longest chain of tensor-core accumulations, in blocks of 64 k, [6] the root mean square over k of a chain's length, in hundredths of a
+ * block; [7], [8] the same two of the kernel that the product goes to otherwise.  0 in [0]: it goes there. */
+int cerb_forward_gemm_plan(int32_t product, int32_t M, int32_t N, int32_t K, int32_t* out9_host);
 int cerb_gemm(int32_t dtype, const void* X_dev, const void* W_dev, float* out_dev, int32_t M, int32_t N, int32_t K,
               void* scratch_dev, size_t scratch_bytes, void* stream);
 

@@ -32,7 +32,7 @@ EXPORTS = [
     "cerb_attn_scratch_bytes", "cerb_tree_attention", "cerb_tree_ancestors", "cerb_gemm_scratch_bytes", "cerb_gemm",
     "cerb_read_state", "cerb_device_status", "cerb_launch_count", "cerb_strerror", "cerb_profile_enable",
     "cerb_profile_read", "cerb_tree_attention_noalloc", "cerb_set_wait_cycles", "cerb_wait_diagnosis", "cerb_tree_attention_noalloc_status", "cerb_launch_order_table", "cerb_last_forward_rows",
-    "cerb_gemm_plan",
+    "cerb_gemm_plan", "cerb_forward_gemm_plan",
 ]
 
 
@@ -444,6 +444,25 @@ def gemm_plan(M: int, N: int, K: int, fused: bool = False) -> GemmPlan:
     out = (C.c_int32 * 8)()
     _check(lib().cerb_gemm_plan(M, N, K, int(fused), out), "cerb_gemm_plan")
     return GemmPlan(*out)
+
+
+class ForwardGemmPlan(NamedTuple):
+    rows_kernel: int
+    groups: int
+    parts: int
+    issuers: int
+    chains: int
+    longest: int
+    mean_length: int
+    other_longest: int
+    other_mean_length: int
+
+
+def forward_gemm_plan(product: str, M: int, N: int, K: int) -> ForwardGemmPlan:
+    """Which kernel takes a product ("qkv", "o_down", "gate_up", "lm_head") of a forward of 9 to 256 rows, in which chains (see cerb_forward_gemm_plan)."""
+    out = (C.c_int32 * 9)()
+    _check(lib().cerb_forward_gemm_plan(("qkv", "o_down", "gate_up", "lm_head").index(product), M, N, K, out), "cerb_forward_gemm_plan")
+    return ForwardGemmPlan(*out)
 
 
 def gemm(X: torch.Tensor, W: torch.Tensor, scratch: Optional[torch.Tensor] = None) -> torch.Tensor:

@@ -238,13 +238,19 @@ int tree_build(cerb_ctx* c, const int32_t* parent, const int32_t* head_of, const
 
 // Plans and maps of the plain products of 9 to `rows` rows; in no more slots than the workspace has for them.
 int rows_sums_parts(int M, int N, int K) { return M > 128 ? 8 : gemm_plan_split(148, M, N, K); }
+RowsPlan rows_sums_plan(int b, int N, int K) {
+  // Above 128 rows, against output tiles that pairs add up through a fix-up buffer (8-layer forwards of 129 / 192 / 256 rows): 1024 columns 1.26 / 1.28 / 1.29 x,
+  // 2048 1.17 / 1.19 / 1.18 x, 4096 1.03 / 1.02 / 1.035 x, 5120 0.98 / 1.00 / 1.012 x, 8192 0.99 / 1.00 / 0.955 x.  (The wider the output, the fewer
+  // parts and the less there was to add up; and the MMAs of output tiles follow the rows, a pair's are 256 high.)
+  const int limit = rows_class_limit(b);
+  if (limit > 128 && N > (limit == 192 ? 4096 : 6144)) return RowsPlan{};
+  return plan_rows_sums(limit, N, K, rows_sums_parts(limit, N, K));
+}
+// The LM head: up to 128 rows.  (One part: its sums go straight to the logits.  4096 columns and more: 13B forwards 1.005 to 1.015 x; 1024 columns 0.98 x)
+bool lm_head_in_rows(int d_model) { return d_model >= 4096; }
 int make_rows_sums(RowsSums* s, const void* const* W, int layers, int N, int K, int rows) {
-  for (int b = 0; b < kRowsSums && rows_sums_limit(b) <= rows; ++b) {
-    // Above 128 rows, against output tiles that pairs add up through a fix-up buffer (8-layer forwards of 129 / 192 / 256 rows): 1024 columns 1.26 / 1.28 / 1.29 x,
-    // 2048 1.17 / 1.19 / 1.18 x, 4096 1.03 / 1.02 / 1.035 x, 5120 0.98 / 1.00 / 1.012 x, 8192 0.99 / 1.00 / 0.955 x.  (The wider the output, the fewer
-    // parts and the less there was to add up; and the MMAs of output tiles follow the rows, a pair's are 256 high.)
-    if (rows_sums_limit(b) > 128 && N > (rows_sums_limit(b) == 192 ? 4096 : 6144)) continue;
-    s->plan[b] = plan_rows_sums(rows_sums_limit(b), N, K, rows_sums_parts(rows_sums_limit(b), N, K));
+  for (int b = 0; b < kRowsClasses && rows_class_limit(b) <= rows; ++b) {
+    s->plan[b] = rows_sums_plan(b, N, K);
     if (!s->plan[b].tiles) continue;
     s->map[b].resize(layers);
     for (int l = 0; l < layers; ++l) CERB_TRY(make_rows_map(&s->map[b][l], W[l], N, K, s->plan[b].groups * 8));
@@ -351,8 +357,8 @@ int forward_rows(cerb_ctx* c, const cerb_tree* tree, const int32_t* tok, int tok
   const bool small = !c->bf16 && c->f32_aligned && gemm_f32_small(M, 2 * F) && gemm_f32_small(M, 3 * HD) && gemm_f32_small(M, d);
   const bool wide = small || (c->bf16 && (M > 128 || M <= kFewRows));
   // 9 to 128 rows: SwiGLU and RoPE + cache append only, where the matrix is for gemm_rows.cu (which takes some of these up to 256 rows, too).
-  const RowsPlan* rows_gu = c->bf16 && gemm_rows_takes(c->rows_gu, M, d) ? &c->rows_gu : nullptr;
-  const RowsPlan* rows_qkv = c->bf16 && gemm_rows_takes(c->rows_qkv, M, d) ? &c->rows_qkv : nullptr;
+  const RowsPlan* rows_gu = c->bf16 && gemm_rows_takes(c->rows_gu, M) ? &c->rows_gu : nullptr;
+  const RowsPlan* rows_qkv = c->bf16 && gemm_rows_takes(c->rows_qkv, M) ? &c->rows_qkv : nullptr;
   const bool fuse_swiglu = small || rows_gu || (wide && (M <= kFewRows || F % 16 == 0));
   const bool fuse_rope = small || rows_qkv || (wide && g.head_dim == 128);
   // (129 to 256 rows: O and down leave parts of k for the norm to add where both are for gemm_rows.cu)
@@ -567,8 +573,8 @@ int cerb_load(const cerb_config* cfg, const cerb_weights* w, void* workspace_dev
       const int Mr = round_up(c->Mmax, 256);
       c->tm_wqkv.resize(L); c->tm_wo.resize(L); c->tm_wgu.resize(L); c->tm_wd.resize(L);
       c->tm_wqkv_rot.resize(L); c->tm_wgu_pair.resize(L);
-      c->rows_qkv = plan_rows_rope(g.n_heads, g.head_dim);
-      c->rows_gu = plan_rows_swiglu(g.mlp_dim);
+      c->rows_qkv = plan_rows_rope(g.n_heads, g.head_dim, g.d_model);
+      c->rows_gu = plan_rows_swiglu(g.mlp_dim, g.d_model);
       c->tm_wqkv_rows.resize(L); c->tm_wgu_rows.resize(L);
       c->tm_kpool.resize(L); c->tm_vpool.resize(L);
       for (int l = 0; l < L && rc == CERB_OK; ++l) {
@@ -587,8 +593,7 @@ int cerb_load(const cerb_config* cfg, const cerb_weights* w, void* workspace_dev
       if ((rc = make_weight_map(&c->tm_lm_head, c->lm_head, g.vocab, g.d_model)) != CERB_OK) break;
       if ((rc = make_rows_sums(&c->rows_wo, c->wo.data(), L, g.d_model, HD, 256)) != CERB_OK) break;
       if ((rc = make_rows_sums(&c->rows_wd, c->wd.data(), L, g.d_model, g.mlp_dim, 256)) != CERB_OK) break;
-      // (one part: the LM head's sums go straight to the logits.  4096 columns and more: 13B forwards 1.005 to 1.015 x; 1024 columns 0.98 x)
-      if (g.d_model >= 4096 && (rc = make_rows_sums(&c->rows_lm, &c->lm_head, 1, g.vocab, g.d_model, 128)) != CERB_OK) break;
+      if (lm_head_in_rows(g.d_model) && (rc = make_rows_sums(&c->rows_lm, &c->lm_head, 1, g.vocab, g.d_model, 128)) != CERB_OK) break;
       if ((rc = make_act_maps(&c->tm_xn, c->d_xn, Mr, g.d_model)) != CERB_OK) break;
       if ((rc = make_act_maps(&c->tm_hidden, c->d_hidden, Mr, g.d_model)) != CERB_OK) break;
       if ((rc = make_act_maps(&c->tm_attn, c->d_attn, Mr, HD)) != CERB_OK) break;
@@ -863,6 +868,24 @@ int cerb_gemm_plan(int32_t M, int32_t N, int32_t K, int32_t fused, int32_t* o) {
   if (!o || M <= 128 || N < 1 || K < 1) return CERB_E_ARG;
   const TilePlan g = fused ? make_tile_plan(M, N, K, false) : standalone_plan(M, N, K);
   const int32_t v[8] = {g.hf, g.mchunks, g.n_act, (int32_t)g.tiles, g.S, g.sk_tiles, g.pairs, fused ? g.chains : g.fills};
+  memcpy(o, v, sizeof(v));
+  return CERB_OK;
+}
+
+int cerb_forward_gemm_plan(int32_t product, int32_t M, int32_t N, int32_t K, int32_t* o) {
+  const int cls = rows_class(M);
+  if (!o || product < 0 || product > 3 || cls < 0 || N < 1 || K < 1 || (product == 0 && N % 384) || (product == 2 && N % 2)) return CERB_E_ARG;
+  RowsPlan g{};
+  if (product == 0) g = plan_rows_rope(N / 384, 128, K);
+  else if (product == 2) g = plan_rows_swiglu(N / 2, K);
+  else if (product == 1 || (M <= 128 && lm_head_in_rows(K))) g = rows_sums_plan(cls, N, K);
+  const Chains other = gemm_rows_other_chains(rows_class_limit(cls), N, K);
+  int32_t v[9] = {gemm_rows_takes(g, M), g.groups, g.parts ? g.parts : 1, g.ring[cls].issuers, g.ring[cls].chains, 0, 0, other.longest, (int)(100 * sqrt(other.mean_square()) + 0.5)};
+  if (v[0]) {
+    const Chains c = gemm_rows_chains(g, M, K);
+    v[5] = c.longest;
+    v[6] = (int)(100 * sqrt(c.mean_square()) + 0.5);
+  }
   memcpy(o, v, sizeof(v));
   return CERB_OK;
 }

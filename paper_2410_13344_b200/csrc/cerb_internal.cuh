@@ -130,22 +130,47 @@ struct ActMaps {
   const CUtensorMap& box(int rows) const { return m[rows / 16 - 1]; }
 };
 
-// gemm_rows.cu: how a matrix is cut into one tile per SM; no tiles = it is not for that kernel
+// Chains of tensor-core accumulations that a product's sums are made of, in blocks of 64 k.  The tensor cores cut a running sum off towards zero at every
+// step, so the error of a sum grows with the length of its chains: over all sums like the root of `cubes` per block.
+struct Chains {
+  int longest = 0;
+  double cubes = 0, blocks = 0;
+  // a run of n blocks dealt to `chains` accumulators
+  void add(int n, int chains) {
+    for (int i = 0; i < chains && i < n; ++i) chain((n - i + chains - 1) / chains);
+  }
+  void chain(int n) {
+    if (n > longest) longest = n;
+    cubes += (double)n * n * n;
+    blocks += n;
+  }
+  double mean_square() const { return blocks ? cubes / blocks : 0; }
+  // (one per cent of the mean square: blocks are whole)
+  bool no_longer_than(const Chains& o) const { return longest <= o.longest && mean_square() <= 1.01 * o.mean_square(); }
+};
+
+// gemm_rows.cu: how a matrix is cut into one tile per SM, and for up to 32, 64, 96, 128, 192 and 256 rows what runs it; no tiles, or no chains there = not
+// for that kernel
+constexpr int kRowsClasses = 6;
+inline int rows_class_limit(int i) { return i < 4 ? 32 * (i + 1) : 64 * (i - 1); }
+inline int rows_class(int M) { return M <= 8 || M > 256 ? -1 : M <= 128 ? (M - 1) / 32 : (M - 1) / 64 + 2; }
+struct RowsRing {
+  int stages, issuers, chains;
+};
 struct RowsPlan {
   int groups, tiles;
   bool heads;               // cut by heads (RoPE)
   int parts;                // plain sums: pieces that k is cut into, each a slot of the output
+  RowsRing ring[kRowsClasses];
 };
 
-// ... and the plain products of up to 32, 64, 96, 128, 192 and 256 rows: a plan each, with the maps of all layers.
-constexpr int kRowsSums = 6;
-inline int rows_sums_limit(int i) { return i < 4 ? 32 * (i + 1) : 64 * (i - 1); }
+// ... and the plain products: a plan for each of these classes, with the maps of all layers.
 struct RowsSums {
-  RowsPlan plan[kRowsSums];
-  std::vector<CUtensorMap> map[kRowsSums];
+  RowsPlan plan[kRowsClasses];
+  std::vector<CUtensorMap> map[kRowsClasses];
   // which of them is for M rows, or -1
   int at(int M) const {
-    const int i = M <= 8 || M > 256 ? -1 : M <= 128 ? (M - 1) / 32 : (M - 1) / 64 + 2;
+    const int i = rows_class(M);
     return i >= 0 && plan[i].tiles ? i : -1;
   }
 };
@@ -274,6 +299,7 @@ int launch_prefill_commit(cerb_ctx* c, cudaStream_t st);
 // gemm_f32.cu / gemm_bf16.cu : out[split][M][N] fp32 partial sums of X[M][K] . W[N][K]^T
 int launch_gemm_f32(cerb_ctx* c, const float* X, const float* W, float* out, int M, int N, int K, cudaStream_t st);
 int gemm_plan_split(int sm_count, int M, int N, int K);
+Chains gemm_bf16_chains(int N, int K);               // of up to 128 rows
 // What may follow a bf16 GEMM in its epilogue (gemm_few.cu, up to kFewRows rows; gemm_rows.cu, 9 to 256 rows, kinds 1 and 2; gemm_tile.cu, above 128
 // rows).
 // kind 1 (SwiGLU): W is [gate rows F][up rows F]; act[row][f] = SiLU(gate) * up (bf16).
@@ -302,6 +328,7 @@ struct TilePlan {
 };
 TilePlan make_tile_plan(int M, int N, int K, bool plain, size_t max_fix = ~(size_t)0);
 size_t gemm_fix_floats();   // of any plan
+Chains gemm_tile_chains(int M, int N, int K);          // of a product with an epilogue
 int launch_gemm_tile(cerb_ctx* c, const CUtensorMap* tmW, const ActMaps* tmX, const TilePlan& g, float* out, float* fix, unsigned int* tickets,
                      int M, int N, int32_t* status, cudaStream_t st, const GemmEpilogue* epi = nullptr,
                      unsigned long long* clock_slot = nullptr);
@@ -320,10 +347,12 @@ int launch_gemm_f32_fused(cerb_ctx* c, const float* X, const float* W, int M, in
 int launch_gemm_few(cerb_ctx* c, const void* X, const void* W, float* out, int M, int N, int K, cudaStream_t st, const GemmEpilogue* epi = nullptr,
                     const GemmNorm* norm = nullptr, unsigned long long* clock_slot = nullptr);
 bool gemm_few_normalises(int M, int K);
-// gemm_rows.cu: 9 to 256 rows, kinds 1 and 2
-bool gemm_rows_takes(const RowsPlan& g, int M, int K);
-RowsPlan plan_rows_swiglu(int F);
-RowsPlan plan_rows_rope(int n_heads, int head_dim);
+// gemm_rows.cu: 9 to 256 rows, kinds 1 and 2, and plain sums; in chains no longer than those of the kernel that takes the product otherwise
+bool gemm_rows_takes(const RowsPlan& g, int M);
+RowsPlan plan_rows_swiglu(int F, int K);
+RowsPlan plan_rows_rope(int n_heads, int head_dim, int K);
+Chains gemm_rows_chains(const RowsPlan& g, int M, int K);
+Chains gemm_rows_other_chains(int limit, int N, int K);      // of the kernel that takes up to `limit` rows otherwise
 int launch_gemm_rows(cerb_ctx* c, const CUtensorMap* tmW, const ActMaps* tmX, const RowsPlan& g, int M, int N, int K, int32_t* status, cudaStream_t st,
                      const GemmEpilogue* epi, float* out = nullptr, unsigned long long* clock_slot = nullptr);
 RowsPlan plan_rows_sums(int M, int N, int K, int max_parts);

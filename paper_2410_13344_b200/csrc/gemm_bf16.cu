@@ -463,6 +463,17 @@ int gemm_plan_split(int sm_count, int M, int N, int K) {
   return M > BM ? 1 : make_plan(sm_count, N, K).nslots;
 }
 
+Chains gemm_bf16_chains(int N, int K) {
+  const GemmPlan g = make_plan(148, N, K);
+  Chains c;
+  for (long long u = 0; u < g.total;) {
+    const long long share = (u / g.per + 1) * g.per, job = (u / g.num_kb + 1) * g.num_kb, end = share < job ? share : job;
+    c.chain((int)((end < g.total ? end : g.total) - u));
+    u = end;
+  }
+  return c;
+}
+
 // Slots of M x N floats that the scratch of the stand-alone GEMM holds.  Up to 128 rows the slots of the plan.  Above, the
 // size that callers of that entry have been told to provide: the slots of 74 workers walking 512 weight rows at a time,
 // side by side on chunks of 256 rows; the tile plan (gemm_tile.cu) is fitted into it.

@@ -21,9 +21,11 @@
 //
 // Issuers and chains.  One thread waits for a stage, issues four MMAs and commits them in 600 to 670 cycles, whatever the MMAs' size up to 160 columns
 // (80 cycles each are possible); it issues nothing while it waits, and two accumulators of its own change nothing.  Two warps that take the
-// stages in turn need 320 to 340 per stage, three 225.  Each has an accumulator of its own, or two in turn where there is room: the tensor cores
-// cut a running sum off towards zero at every step, so a sum is made of several short chains (at most as long as the partial sums were:
-// keys of the first 7B layer against float64, mean error of 64 rows 3.1e-6 with two chains of 32 k blocks, 2.5e-6 with partial sums of 21).
+// stages in turn need 320 to 340 per stage, three 225.  Each has one accumulator or several in turn: the tensor cores cut a running sum off towards
+// zero at every step, so a sum is made of several short chains, as many as it takes for them to be no longer than those of the kernel that the
+// product goes to otherwise (plan_ring; where they do not fit, it goes there).  V of a first layer against float64, by the bf16 values that round the
+// other way, in 1e-6 of their size, 32 / 128 rows: 2048 columns 0.48 / 0.26 there, 0.75 / 0.39 in three / four chains, 0.27 / 0.30 in six; 2560 columns 0.37 / 0.56,
+// 0.62 / 0.93 in three, 0.29 / 0.39 in six; 4096 columns, 96 rows 1.23, 1.41 in three, 1.09 in four.  Six chains instead of four cost 0.2 us a launch.
 // A pair's tile of more than 256 columns is two MMAs wide (and one issuer keeps the tensor cores busy: 712 cycles of 640 per stage); there is
 // room for three accumulators then, and each half of the columns goes over to another one near the middle: the first half to the third, the
 // second to the first, which the epilogue warps have taken to registers by then.
@@ -45,6 +47,7 @@ constexpr int MAX_STAGES = 18;
 constexpr int ROWS = 128;                                  // accumulator rows of a CTA
 constexpr int kSms = 148;
 constexpr int kIssuers = 3;                                // at most
+constexpr int kChains = 6;                                 // at most
 constexpr int kParts = 3;                                  // epilogue warps per 32 accumulator rows
 constexpr int kThreads = 128 + 128 * kParts;
 constexpr int COLS = 16;                                   // columns an epilogue warp takes at a time (two groups)
@@ -83,7 +86,9 @@ __device__ __forceinline__ void load_groups(uint32_t dst, const CUtensorMap* map
         : "memory");
 }
 
-template <int KIND, int CG>
+// MANY: more than four accumulators.  (An instance of its own: with the loop for them in the others, where it does not run, 8 layers of 4096 columns took 774 instead of
+// 768 us at 9 rows.)
+template <int KIND, int CG, bool MANY>
 __global__ void __launch_bounds__(kThreads, 1) gemm_rows_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtensorMap tmX,
                                                                 const RowsParams p) {
   extern __shared__ uint8_t smem_raw[];
@@ -210,7 +215,9 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_rows_kernel(const __grid_con
       };
       if (!two) {
         const uint32_t idesc = idesc_bf16(CG * (uint32_t)p.m_rows, p.acc_cols, false, false);
-        uint32_t d = tmem_base + (uint32_t)self * p.acc_cols, other = d + (p.chains > p.issuers ? (uint32_t)p.issuers * p.acc_cols : 0u), ph = 0;
+        // this issuer's accumulators, which it takes in turn
+        const uint32_t d0 = tmem_base + (uint32_t)self * p.acc_cols, d_end = tmem_base + (uint32_t)p.chains * p.acc_cols;
+        uint32_t d = d0, ph = 0;
         int s = self;
         for (int i = self; i < num_kb; i += p.issuers) {
           live = __all_sync(0xffffffffu, wait(full_bar[s], ph, 242));
@@ -221,9 +228,8 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_rows_kernel(const __grid_con
             commit(empty_bar[s]);                              // the stage is free once the MMAs have read it
           }
           __syncwarp();
-          const uint32_t t = d;
-          d = other;
-          other = t;
+          d += (uint32_t)p.issuers * p.acc_cols;
+          if (d >= d_end) d = d0;
           if ((s += p.issuers) >= p.stages) { s = self; ph ^= 1u; }
         }
       } else {
@@ -306,24 +312,37 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_rows_kernel(const __grid_con
       tc_fence_after();
       // two blocks of eight columns of all chains
       auto load = [&](uint32_t c0, uint32_t c1, float* v) {
-        float t[COLS];
-        tmem_ld8_nowait(lanes + c0, reinterpret_cast<uint32_t*>(v));
-        tmem_ld8_nowait(lanes + c1, reinterpret_cast<uint32_t*>(v + 8));
-        auto next = [&](int chain, float* t) {
-          tmem_ld8_nowait(lanes + (uint32_t)chain * p.acc_cols + c0, reinterpret_cast<uint32_t*>(t));
-          tmem_ld8_nowait(lanes + (uint32_t)chain * p.acc_cols + c1, reinterpret_cast<uint32_t*>(t + 8));
+        auto fetch = [&](int chain, float* t) {
+          const uint32_t at = lanes + (uint32_t)chain * p.acc_cols;
+          if constexpr (KIND == 2 && CG == 2) {
+            tmem_ld8_nowait(at + c0, reinterpret_cast<uint32_t*>(t));
+            tmem_ld8_nowait(at + c1, reinterpret_cast<uint32_t*>(t + 8));
+          } else {
+            tmem_ld16_nowait(at + c0, reinterpret_cast<uint32_t*>(t));              // (c1 is c0 + 8)
+          }
         };
-        float u[COLS];
-        if (p.chains > 1) next(1, t);
-        if (p.chains > 2) next(2, u);
+        float t[COLS], u[COLS];
+        fetch(0, v);
+        if (p.chains > 1) fetch(1, t);
+        if (p.chains > 2) fetch(2, u);
         tmem_ld_wait();
 #pragma unroll
         for (int j = 0; j < COLS; ++j) v[j] += (p.chains > 1 ? t[j] : 0.f) + (p.chains > 2 ? u[j] : 0.f);
         if (p.chains > 3) {
-          next(3, t);
+          fetch(3, t);
           tmem_ld_wait();
 #pragma unroll
           for (int j = 0; j < COLS; ++j) v[j] += t[j];
+        }
+        if constexpr (MANY) {
+#pragma unroll 1
+          for (int chain = 4; chain < p.chains; chain += 2) {
+            fetch(chain, t);
+            if (chain + 1 < p.chains) fetch(chain + 1, u);
+            tmem_ld_wait();
+#pragma unroll
+            for (int j = 0; j < COLS; ++j) v[j] += t[j] + (chain + 1 < p.chains ? u[j] : 0.f);
+          }
         }
       };
       if constexpr (KIND == 1) {
@@ -468,36 +487,115 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_rows_kernel(const __grid_con
   }
 }
 
-template <int KIND, int CG>
+template <int KIND, int CG, bool MANY>
 int launch_kind(const CUtensorMap& tmW, const CUtensorMap& tmX, const RowsParams& p, int tiles, cudaStream_t st) {
+  auto kern = gemm_rows_kernel<KIND, CG, MANY>;
   static bool configured = false;
   if (!configured) {
-    CERB_CUDA_OK(cudaFuncSetAttribute(gemm_rows_kernel<KIND, CG>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRing));
+    CERB_CUDA_OK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRing));
     configured = true;
   }
   // (always the same request, more than half of an SM: one CTA there, which may own all of its tensor memory)
-  const cudaError_t e = CG == 2 ? launch_pdl_cluster(gemm_rows_kernel<KIND, CG>, dim3((tiles + 1) / 2 * 2), dim3(kThreads), kRing, st, 2u, tmW, tmX, p)
-                                : launch_pdl(gemm_rows_kernel<KIND, CG>, dim3(tiles), dim3(kThreads), kRing, st, tmW, tmX, p);
+  const cudaError_t e = CG == 2 ? launch_pdl_cluster(kern, dim3((tiles + 1) / 2 * 2), dim3(kThreads), kRing, st, 2u, tmW, tmX, p)
+                                : launch_pdl(kern, dim3(tiles), dim3(kThreads), kRing, st, tmW, tmX, p);
   return e == cudaSuccess ? CERB_OK : CERB_E_CUDA;
+}
+
+// (activation tiles of 16 or 48 rows: forwards 2 % slower than with 32 and 64)
+size_t rows_fetched(int M) { return ((M > ROWS ? (M + 1) / 2 : M) + 31) / 32 * 32; }
+// Up to 64 rows: MMAs of 64 rows.  A stream of weights at the HBM rate and half-empty MMAs run into the power limit together: 64-node forwards of the 7B
+// shape, one after the other, 3511 us with MMAs of 128 rows and 3358 with 64; the first ones on an idle GPU take 3280 either way.
+int mma_rows(int M) { return M <= 64 ? 64 : ROWS; }
+int acc_columns(const RowsPlan& g, int M) {
+  const int step = mma_rows(M) == 64 ? 8 : 16;
+  return (g.groups * 8 * (M > ROWS ? 2 : 1) + step - 1) / step * step;
+}
+int ring_stages(const RowsPlan& g, int M) {
+  const size_t stage = (size_t)g.groups * 1024 + rows_fetched(M) * 128;
+  // (the MMAs read all rows of the last stage, too; 1 KB for the alignment of the ring)
+  const int stages = (int)((kRing - 1024 - (mma_rows(M) - rows_fetched(M)) * 128) / stage);
+  return stages < MAX_STAGES ? stages : MAX_STAGES;
+}
+Chains ring_chains(const RowsPlan& g, const RowsRing& r, int num_kb) {
+  Chains c;
+  const int parts = g.parts ? g.parts : 1;
+  for (int s = 0; s < parts; ++s) {
+    const int n = (s + 1) * num_kb / parts - s * num_kb / parts;
+    for (int i = 0; i < r.issuers; ++i) c.add((n - i + r.issuers - 1) / r.issuers, (r.chains - i + r.issuers - 1) / r.issuers);
+  }
+  return c;
+}
+// What runs a plan's product of up to `limit` rows: the ring, the issuers, and as many accumulators as its chains need to be no longer than `other`.
+// A stage belongs to one issuer, which waits for its phases in turn.  (Issuers that took turns at a stage could be a round apart when copies
+// land out of order, and a parity tells neighbouring phases apart only.)  Three issuers or two where the ring loses no stage by it; one
+// where it would and the weights of a stage take as long to come as one issuer needs.
+RowsRing plan_ring(const RowsPlan& g, int limit, int K, const Chains& other) {
+  const int num_kb = (K + BK - 1) / BK, least_kb = g.parts ? num_kb / g.parts : num_kb, cols = acc_columns(g, limit);
+  RowsRing r;
+  r.stages = ring_stages(g, limit);
+  r.issuers = r.stages % 3 == 0 && 3 * cols <= 512 ? 3 : r.stages % 2 == 0 ? 2 : g.groups >= 16 ? 1 : 2;
+  r.stages -= r.stages % r.issuers;
+  if (r.issuers > least_kb) r.issuers = least_kb;
+  int most = 512 / cols < least_kb ? 512 / cols : least_kb;
+  if (most > kChains) most = kChains;
+  r.chains = r.issuers < 3 && 2 * r.issuers <= most ? 2 * r.issuers : r.issuers;
+  while (r.chains <= most && !ring_chains(g, r, num_kb).no_longer_than(other)) ++r.chains;
+  if (r.chains > most) r.chains = 0;
+  return r;
+}
+}  // namespace
+
+Chains gemm_rows_other_chains(int limit, int N, int K) {
+  if (limit <= ROWS) return gemm_bf16_chains(N, K);
+  const Chains a = gemm_tile_chains(limit - 32, N, K), b = gemm_tile_chains(limit, N, K);
+  return a.no_longer_than(b) ? a : b;
+}
+namespace {
+
+// Two MMAs per 16 k: blocks after which each goes over to its second accumulator
+int turn0(int num_kb) { return num_kb * 30 / 64; }
+int turn1(int num_kb) { return num_kb * 34 / 64; }
+Chains two_chains(int num_kb) {
+  Chains c;
+  for (int turn : {turn0(num_kb), turn1(num_kb)}) {
+    c.chain(turn);
+    c.chain(num_kb - turn);
+  }
+  return c;
+}
+void plan_rings(RowsPlan& g, int N, int K) {
+  for (int i = 0; i < kRowsClasses; ++i) {
+    const int limit = rows_class_limit(i);
+    if (g.heads && limit > ROWS && limit <= 192) continue;
+    if (limit > ROWS && g.groups > 16) {
+      if (g.heads || (g.groups + (g.groups + 1) / 2) * 16 > 512 || K < 16 * BK) continue;
+      g.ring[i] = RowsRing{ring_stages(g, limit), 1, 2};
+    } else {
+      g.ring[i] = plan_ring(g, limit, K, gemm_rows_other_chains(limit, N, K));
+    }
+  }
 }
 
 }  // namespace
 
-RowsPlan plan_rows_swiglu(int F) {
-  RowsPlan g{0, 0, false, 0};
+RowsPlan plan_rows_swiglu(int F, int K) {
+  RowsPlan g{};
   const int groups = F / 4, per = (groups + kSms - 1) / kSms;
   if (F % 4 || per < 2 || per > 32) return g;
   g.groups = per;
   g.tiles = (groups + per - 1) / per;
+  plan_rings(g, 2 * F, K);
   return g;
 }
 
-RowsPlan plan_rows_rope(int n_heads, int head_dim) {
-  RowsPlan g{0, 0, true, 0};
+RowsPlan plan_rows_rope(int n_heads, int head_dim, int K) {
+  RowsPlan g{};
+  g.heads = true;
   const int heads = 3 * n_heads, per = (heads + kSms / 16 - 1) / (kSms / 16);
   if (head_dim != 128 || per < 2 || per > 32) return g;
   g.groups = per;
   g.tiles = 16 * ((heads + per - 1) / per);
+  plan_rings(g, heads * 128, K);
   return g;
 }
 
@@ -507,13 +605,18 @@ RowsPlan plan_rows_rope(int n_heads, int head_dim) {
 //   Forwards, plain sums (below) included: 7B width 9 / 64 / 128 rows 1.06 / 1.06 / 1.12 x, 13B 1.02 / 1.09 / 1.13 x, 1024 to 3200 columns 1.04 to 1.25 x.
 //   129 to 256 rows, in pairs, against output tiles of 256 weight rows (gemm_tile.cu): a pair's tile has to fit one MMA, or (SwiGLU, 16 k
 //   blocks and more) three accumulators.  Tiles of 256 rows leave SMs idle or have to be cut along k: 7B width, gate-up of 129 / 256 rows 46 / 53 -> 41 /
-//   43 us.  RoPE from 193 rows on: below, the output tiles are cut and sum shorter chains than the two that fit here (keys of 130 to 180 rows against float64
-//   1.10e-4 to 1.32e-4 there, 1.32e-4 to 1.52e-4 here; from 193 rows on the bits are the same; QKV of 256 rows 32.5 -> 27 us).
-bool gemm_rows_takes(const RowsPlan& g, int M, int K) {
-  if (M <= kFewRows || M > 2 * ROWS || g.tiles < 1) return false;
-  if (M <= ROWS) return true;
-  if (g.groups > 16) return !g.heads && (g.groups + (g.groups + 1) / 2) * 16 <= 512 && K >= 16 * BK;
-  return !g.heads || M > 192;
+//   43 us.  RoPE from 193 rows on: below, the output tiles are cut and sum shorter chains than those that fit here (keys of 130 to 180 rows against float64
+//   1.10e-4 to 1.32e-4 there, 1.32e-4 to 1.52e-4 here).  From 193 rows on they are as long at 4096 columns and more (QKV of 256 rows 32.5 -> 27 us) and fit at 1024
+//   and 1536; from 2048 to 3584 they do not (2048 columns, 2 x 128 rows, 8 layers: 580 us here, 645 with output tiles; V 0.44 against 0.24e-6 from float64).
+bool gemm_rows_takes(const RowsPlan& g, int M) {
+  const int i = rows_class(M);
+  return i >= 0 && g.tiles > 0 && g.ring[i].chains > 0;
+}
+
+Chains gemm_rows_chains(const RowsPlan& g, int M, int K) {
+  const RowsRing& r = g.ring[rows_class(M)];
+  const int num_kb = (K + BK - 1) / BK;
+  return M > ROWS && g.groups > 16 ? two_chains(num_kb) : ring_chains(g, r, num_kb);
 }
 
 // Plain sums of up to 128 rows (O, down, LM head): k is cut into parts, each a sum of its own (a slot) for the kernel behind to add, so that tiles are wide
@@ -523,7 +626,7 @@ bool gemm_rows_takes(const RowsPlan& g, int M, int K) {
 // 4.0 us, O 9.8 -> 8.8, down 17.6 -> 16.5.)
 // 129 to 256 rows, in pairs: the same, a part costing more (4 MB to write and to read back at 256 rows and 4096 columns).
 RowsPlan plan_rows_sums(int M, int N, int K, int max_parts) {
-  RowsPlan best{0, 0, false, 0};
+  RowsPlan best{};
   double best_t = 0;
   const int pair = M > ROWS ? 2 : 1, groups = (N + 7) / 8, num_kb = (K + BK - 1) / BK, x = ((M + pair - 1) / pair + 31) / 32 * 32 / 8;
   if (M <= kFewRows || M > 2 * ROWS) return best;
@@ -536,15 +639,19 @@ RowsPlan plan_rows_sums(int M, int N, int K, int max_parts) {
     const double in = hbm > sm ? hbm : sm, t = (in > least ? in : least) + parts * (pair == 2 ? 0.004 * M : 0.05 + 0.001 * M);
     if (!best_t || t < best_t) {
       best_t = t;
-      best = RowsPlan{per, (groups + pair * per - 1) / (pair * per) * parts * pair, false, parts};
+      best = RowsPlan{per, (groups + pair * per - 1) / (pair * per) * parts * pair, false, parts, {}};
     }
   }
-  return best;
+  if (!best.tiles) return best;
+  RowsRing& r = best.ring[rows_class(M)];
+  r = plan_ring(best, M, K, gemm_rows_other_chains(M, N, K));
+  return r.chains ? best : RowsPlan{};
 }
 
 int launch_gemm_rows(cerb_ctx* c, const CUtensorMap* tmW, const ActMaps* tmX, const RowsPlan& g, int M, int N, int K, int32_t* status, cudaStream_t st,
                      const GemmEpilogue* epi, float* out, unsigned long long* clock_slot) {
-  if (epi ? !gemm_rows_takes(g, M, K) : M < 1 || M > 2 * ROWS || g.parts < 1) return CERB_E_SHAPE;
+  const int i = rows_class(M);
+  if (i < 0 || !g.ring[i].chains || (!epi && g.parts < 1)) return CERB_E_SHAPE;
   const bool pairs = M > ROWS;            // (7B width, 96 and 128 rows: 1062 and 1082 us in pairs, 926 and 974 in single CTAs)
   RowsParams p;
   memset(&p, 0, sizeof(p));
@@ -555,40 +662,27 @@ int launch_gemm_rows(cerb_ctx* c, const CUtensorMap* tmW, const ActMaps* tmX, co
   p.out = out;
   p.N = N;
   p.parts = g.parts;
-  const int least_kb = epi ? p.num_kb : p.num_kb / g.parts;
   p.groups = p.groups0 = g.groups;
-  // (activation tiles of 16 or 48 rows: forwards 2 % slower than with 32 and 64)
-  p.x_rows = ((pairs ? (M + 1) / 2 : M) + 31) / 32 * 32;
-  const size_t stage = (size_t)p.groups * 1024 + (size_t)p.x_rows * 128;
-  // Up to 64 rows: MMAs of 64 rows.  A stream of weights at the HBM rate and half-empty MMAs run into the power limit together: 64-node forwards of the 7B
-  // shape, one after the other, 3511 us with MMAs of 128 rows and 3358 with 64; the first ones on an idle GPU take 3280 either way.
-  p.m_rows = !pairs && M <= 64 ? 64 : ROWS;
-  // (the MMAs read all rows of the last stage, too; 1 KB for the alignment of the ring)
-  p.stages = (int)((kRing - 1024 - (size_t)(p.m_rows - p.x_rows) * 128) / stage);
-  if (p.stages > MAX_STAGES) p.stages = MAX_STAGES;
-  const int step = p.m_rows == 64 ? 8 : 16, cols = (g.groups * 8 * (pairs ? 2 : 1) + step - 1) / step * step;
+  p.x_rows = (int)rows_fetched(M);
+  p.m_rows = mma_rows(M);
+  p.stages = g.ring[i].stages;
+  p.issuers = g.ring[i].issuers;
+  p.chains = g.ring[i].chains;
   if (pairs && g.groups > 16) {
     p.groups0 = (g.groups + 1) / 2;
-    p.issuers = 1;
-    p.turn0 = p.num_kb * 30 / 64;
-    p.turn1 = p.num_kb * 34 / 64;
+    p.turn0 = turn0(p.num_kb);
+    p.turn1 = turn1(p.num_kb);
     p.tmem_cols = 512;
   } else {
-    // A stage belongs to one issuer, which waits for its phases in turn.  (Issuers that took turns at a stage could be a round apart when copies
-    // land out of order, and a parity tells neighbouring phases apart only.)  Three issuers or two where the ring loses no stage by it; one
-    // where it would and the weights of a stage take as long to come as one issuer needs.
-    p.issuers = p.stages % 3 == 0 && 3 * cols <= 512 ? 3 : p.stages % 2 == 0 ? 2 : p.groups >= 16 ? 1 : 2;
-    p.stages -= p.stages % p.issuers;
-    if (p.issuers > least_kb) p.issuers = least_kb;
-    p.chains = p.issuers < 3 && least_kb >= 2 * p.issuers && 2 * p.issuers * cols <= 512 ? 2 * p.issuers : p.issuers;
-    p.acc_cols = (uint32_t)cols;
+    p.acc_cols = (uint32_t)acc_columns(g, M);
     for (p.tmem_cols = 32; p.tmem_cols < p.chains * p.acc_cols; p.tmem_cols *= 2) {}
   }
   p.wait_cycles = wait_cycles();
   p.clk = clock_slot;
   auto run = [&](auto kind, const CUtensorMap& x) {
     constexpr int KIND = decltype(kind)::value;
-    return pairs ? launch_kind<KIND, 2>(*tmW, x, p, g.tiles, st) : launch_kind<KIND, 1>(*tmW, x, p, g.tiles, st);
+    if (p.chains > 4) return pairs ? launch_kind<KIND, 2, true>(*tmW, x, p, g.tiles, st) : launch_kind<KIND, 1, true>(*tmW, x, p, g.tiles, st);
+    return pairs ? launch_kind<KIND, 2, false>(*tmW, x, p, g.tiles, st) : launch_kind<KIND, 1, false>(*tmW, x, p, g.tiles, st);
   };
   int rc;
   if (!epi) {

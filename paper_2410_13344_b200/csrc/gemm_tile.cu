@@ -713,6 +713,22 @@ TilePlan make_tile_plan(int M, int N, int K, bool plain, size_t max_fix) {
   return best;
 }
 
+Chains gemm_tile_chains(int M, int N, int K) {
+  const TilePlan g = make_tile_plan(M, N, K, false);
+  Chains c;
+  for (int t = 0; t < g.tiles; ++t)
+    if (t < g.sk_tiles) {
+      for (int u = t * g.num_kb; u < (t + 1) * g.num_kb;) {
+        const int share = (u / g.per + 1) * g.per, end = share < (t + 1) * g.num_kb ? share : (t + 1) * g.num_kb;
+        c.add(end - u, g.chains);
+        u = end;
+      }
+    } else {
+      for (int s = 0; s < g.S; ++s) c.add((s + 1) * g.num_kb / g.S - s * g.num_kb / g.S, g.chains);
+    }
+  return c;
+}
+
 size_t gemm_fix_floats() { return (size_t)kPairs * 2 * 2 * 128 * TILE_X; }
 
 template <int KIND, int HF>

@@ -21,11 +21,10 @@ SHAPES = {
 }
 # prompt lengths: rows of one accumulator quarter, its edges, all of them; pairs: one row in the second CTA's half and all
 CASES = [(n, m) for n in SHAPES for m in (9, 33, 64, 65, 128, 129, 256)]
+CASES += [("32 and 152 rows, two MMAs per pair", m) for m in (96, 97, 192, 193)]          # ... and both sides of the other plans' edges
 
 
-@pytest.mark.parametrize("name,M", CASES)
-def test_prompts_match_oracle(name, M):
-    d, H, F = SHAPES[name]
+def _prompt_matches_oracle(d, H, F, M):
     ms = synth.ModelShape(1, d, H, 128, F, 512, "bf16")
     rig = Rig(cb, ms, max_tokens=M + 16, max_nodes=16)
     prompt = [int(t) for t in synth.make_prompt(ms.vocab, M, seq=140 + M)]
@@ -40,9 +39,31 @@ def test_prompts_match_oracle(name, M):
         assert close(h_last[0], st.h_last, 0) < TOL["bf16"]
         k, v = rig.eng.gather_kv(0, 0, M)
         assert close(k, st.k[0][:M], 0) < TOL["bf16"] and close(v, st.v[0][:M], 0) < TOL["bf16"]
+    return launches
+
+
+@pytest.mark.parametrize("name,M", CASES)
+def test_prompts_match_oracle(name, M):
+    d, H, F = SHAPES[name]
+    launches = _prompt_matches_oracle(d, H, F, M)
     # live rows, first norm, seven launches of the layer, commit, LM head, argmax
     if M <= 128:
         assert launches == 1 + 1 + 7 + 3
+    # ... of which these are this kernel's
+    assert [cb.forward_gemm_plan(p, M, N, d).rows_kernel for p, N in (("gate_up", 2 * F), ("qkv", 384 * H))] == [1, M <= 128 or M > 192]
+
+
+# More accumulators than two per issuer, and numbers of them that the issuers do not divide: (rows, product, issuers, accumulators)
+@pytest.mark.parametrize("d,H,F,M,product,issuers,chains", [
+    (1024, 8, 2816, 9, "qkv", 3, 6), (1024, 8, 2816, 97, "qkv", 2, 4), (1024, 8, 2816, 256, "qkv", 2, 6), (1536, 12, 4096, 97, "qkv", 2, 6),
+    (1024, 8, 2816, 33, "gate_up", 2, 4), (1024, 8, 4096, 128, "gate_up", 3, 6), (2048, 4, 5632, 9, "gate_up", 3, 5), (3584, 4, 9728, 65, "gate_up", 1, 3),
+    (1024, 8, 1024, 129, "o_down", 3, 5), (1024, 8, 1024, 250, "o_down", 3, 5), (4096, 32, 1184, 96, "qkv", 3, 4),
+])
+def test_accumulators_in_turn_match_oracle(d, H, F, M, product, issuers, chains):
+    N = {"qkv": 384 * H, "gate_up": 2 * F, "o_down": d}[product]
+    g = cb.forward_gemm_plan(product, M, N, d)
+    assert (g.rows_kernel, g.issuers, g.chains) == (1, issuers, chains), g
+    _prompt_matches_oracle(d, H, F, M)
 
 
 @pytest.mark.parametrize("n,live", [(40, (40, 17, 1)), (70, (1, 70, 33))])
