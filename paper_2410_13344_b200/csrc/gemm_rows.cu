@@ -26,9 +26,11 @@
 // product goes to otherwise (plan_ring; where they do not fit, it goes there).  V of a first layer against float64, by the bf16 values that round the
 // other way, in 1e-6 of their size, 32 / 128 rows: 2048 columns 0.48 / 0.26 there, 0.75 / 0.39 in three / four chains, 0.27 / 0.30 in six; 2560 columns 0.37 / 0.56,
 // 0.62 / 0.93 in three, 0.29 / 0.39 in six; 4096 columns, 96 rows 1.23, 1.41 in three, 1.09 in four.  Six chains instead of four cost 0.2 us a launch.
-// A pair's tile of more than 256 columns is two MMAs wide (and one issuer keeps the tensor cores busy: 712 cycles of 640 per stage); there is
-// room for three accumulators then, and each half of the columns goes over to another one near the middle: the first half to the third, the
-// second to the first, which the epilogue warps have taken to registers by then.
+// A pair's tile of more than 256 columns is three MMAs wide: two of 96 columns each, whose accumulators go over to a third one of that size in turn, while
+// the epilogue warps add what the last one holds to their registers (which have room for these 192 columns, and for no more), and one of the
+// rest, with an accumulator for either half of k; two warps issue the two kinds.  (7B width: chains of 8 and 16 k blocks and of 32, 23 in the root mean square, 24 in cut output
+// tiles; activations of 160 / 256 rows 4.4 / 5.0e-6 from float64 as above, 4.8 / 5.7e-6 there.  Two MMAs with one change each, chains of 30 and 34: 6.7 / 7.5e-6,
+// and 0.5 % less for a forward: 1287 / 1297 us of 256 rows, 8 layers.)
 //
 // Roles (512 threads): warp 0 = TMA producer (one lane), which fills the ring with weights ahead of the dependency wait; warps 1 to 3 = MMA
 // issuers (of a pair's first CTA); warps 4 to 15 = epilogue, three per 32 accumulator rows.
@@ -47,11 +49,12 @@ constexpr int MAX_STAGES = 18;
 constexpr int ROWS = 128;                                  // accumulator rows of a CTA
 constexpr int kSms = 148;
 constexpr int kIssuers = 3;                                // at most
-constexpr int kChains = 6;                                 // at most
 constexpr int kParts = 3;                                  // epilogue warps per 32 accumulator rows
 constexpr int kThreads = 128 + 128 * kParts;
 constexpr int COLS = 16;                                   // columns an epilogue warp takes at a time (two groups)
-constexpr int HELD = 4;                                    // blocks of columns that an epilogue thread can hold
+constexpr int HELD = 2;                                    // blocks of columns of each of two MMAs that an epilogue thread holds
+constexpr int kTurnCols = HELD * kParts * COLS;            // columns of such an MMA
+constexpr int kTurnGroups = kTurnCols / 16;                // groups of either CTA in it
 constexpr size_t kRing = 226 * 1024;                       // shared memory of the ring, with what the last stage's missing rows need
 
 struct RowsParams {
@@ -62,11 +65,10 @@ struct RowsParams {
   int32_t* status;
   int M, F, num_kb;
   int groups;               // groups of eight weight rows of a CTA
-  int groups0;              // ... of them in the first MMA (CG = 2; the rest in the second)
   int x_rows;               // activation rows fetched by a CTA
   int m_rows;               // rows of a CTA's accumulator: 128, or (CG = 1) 64, of which each warp quarter has 16
   int stages, issuers, chains;
-  int turn0, turn1;         // two MMAs: k blocks after which each goes over to its second accumulator
+  int turn, turns;          // three MMAs: k blocks from one change of accumulators to the next, and how many of these there are; else 0
   uint32_t acc_cols, tmem_cols;
   long long wait_cycles;
   unsigned long long* clk;
@@ -107,7 +109,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_rows_kernel(const __grid_con
   const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;       // (one value per warp, as the compiler sees)
   const int rank = CG == 2 ? (int)cluster_ctarank() : 0;
   const bool first = rank == 0;
-  const bool two = KIND == 1 && CG == 2 && p.groups0 < p.groups;           // two MMAs per 16 k
+  const bool turning = KIND == 1 && CG == 2 && p.turns > 0;                // three MMAs per 16 k
   // Consecutive groups; RoPE: four rotations of a block of heads.  Plain sums: the parts of a tile are neighbours.
   const int row0 = KIND == 2 ? ((int)blockIdx.x & 15) * 4 : 0;
   const int tile = KIND == 2 ? (int)blockIdx.x >> 4 : KIND == 0 ? (int)blockIdx.x / CG / p.parts : (int)blockIdx.x;
@@ -121,7 +123,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_rows_kernel(const __grid_con
     issued_s = -1;
     for (int s = 0; s < p.stages; ++s) {
       mbar_init(smem_u32(&full_bar[s]), 1);
-      mbar_init(smem_u32(&empty_bar[s]), 1);
+      mbar_init(smem_u32(&empty_bar[s]), turning ? 2 : 1);
     }
     mbar_init(smem_u32(&acc_full), (uint32_t)p.issuers);
     for (int i = 0; i < kIssuers; ++i) mbar_init(smem_u32(&drain_bar[i]), 1);
@@ -213,7 +215,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_rows_kernel(const __grid_con
           else umma_bf16(d, adesc + (uint64_t)(kk * 2), bdesc + (uint64_t)(kk * 2), idesc, acc);
         }
       };
-      if (!two) {
+      if (!turning) {
         const uint32_t idesc = idesc_bf16(CG * (uint32_t)p.m_rows, p.acc_cols, false, false);
         // this issuer's accumulators, which it takes in turn
         const uint32_t d0 = tmem_base + (uint32_t)self * p.acc_cols, d_end = tmem_base + (uint32_t)p.chains * p.acc_cols;
@@ -233,28 +235,44 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_rows_kernel(const __grid_con
           if ((s += p.issuers) >= p.stages) { s = self; ph ^= 1u; }
         }
       } else {
-        const uint32_t n0 = 16u * (uint32_t)p.groups0, n1 = 16u * (uint32_t)p.groups - n0;
-        const uint32_t idesc0 = idesc_bf16(2 * ROWS, n0, false, false), idesc1 = idesc_bf16(2 * ROWS, n1, false, false);
-        uint32_t d0 = tmem_base, d1 = tmem_base + n0;
-        uint32_t ph = 0;
+        const uint32_t idesc_t = idesc_bf16(2 * ROWS, kTurnCols, false, false);
+        const uint32_t rest = 16u * (uint32_t)p.groups - 2 * kTurnCols, idesc_r = idesc_bf16(2 * ROWS, rest, false, false);
+        uint32_t d0 = tmem_base, d1 = d0 + kTurnCols, spare = d1 + kTurnCols, ph = 0;              // the first issuer's
+        uint32_t d = tmem_base + 3 * kTurnCols;                                                   // the second one's
+        bool fresh0 = true, fresh1 = true;
+        int t = 0;                                             // changes so far
         for (int i = 0, s = 0; i < num_kb; ++i) {
-          // to the second accumulators: the third one's columns; the first one's, when they have been taken from there
-          if (i == p.turn0) d0 = tmem_base + n0 + n1;
-          if (i == p.turn1) {
-            live = __all_sync(0xffffffffu, wait(turn_done, 0, 244));
+          if (self == 1) {
+            fresh0 = i == 0 || i == num_kb / 2;
+            if (i > 0 && fresh0) d += rest;
+          } else if (t < p.turns && i == (t + 1) * p.turn) {
+            // the spare accumulator has been taken over since the last change
+            live = t == 0 || __all_sync(0xffffffffu, wait(turn_done, (uint32_t)(t - 1) & 1u, 244));
             if (!live) break;
-            d1 = tmem_base;
+            tc_fence_after();
+            if (elect_one()) commit(turn_full);
+            __syncwarp();
+            uint32_t& mine = t & 1 ? d1 : d0;
+            const uint32_t done = mine;
+            mine = spare;
+            spare = done;
+            (t & 1 ? fresh1 : fresh0) = true;
+            ++t;
           }
           live = __all_sync(0xffffffffu, wait(full_bar[s], ph, 242));
           if (!live) break;
           tc_fence_after();
           if (elect_one()) {
-            issue(s, 0, idesc0, d0, i == 0 || i == p.turn0);
-            if (i + 1 == p.turn0) commit(turn_full);
-            issue(s, p.groups0, idesc1, d1, i == 0 || i == p.turn1);
+            if (self == 0) {
+              issue(s, 0, idesc_t, d0, fresh0);
+              issue(s, kTurnGroups, idesc_t, d1, fresh1);
+            } else {
+              issue(s, 2 * kTurnGroups, idesc_r, d, fresh0);
+            }
             commit(empty_bar[s]);
           }
           __syncwarp();
+          fresh0 = fresh1 = false;
           if (++s == p.stages) { s = 0; ph ^= 1u; }
         }
       }
@@ -292,21 +310,43 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_rows_kernel(const __grid_con
       }
     }
     const uint32_t lanes = tmem_base + ((uint32_t)(quarter * 32) << 16);
-    const uint32_t n0 = 16u * (uint32_t)p.groups0;
     bool live = rank * p.x_rows + quarter * per_quarter < p.M && quarter * per_quarter < p.x_rows;      // (a warp none of whose rows exist reads no accumulator)
-    float held[CG == 2 ? HELD : 1][COLS];
-    if (CG == 2 && two) {
-      if (live) live = __all_sync(0xffffffffu, wait(turn_full, 0, 245));
-      if (live) {
-        tc_fence_after();
+    float held[2][CG == 2 && KIND == 1 ? HELD : 1][COLS];
+    uint32_t at0 = lanes, at1 = at0 + kTurnCols, spare = at1 + kTurnCols;               // as the issuer's
+    if constexpr (KIND == 1 && CG == 2) {
+      // (all warps of the pair, whether their rows exist or not, go through the changes together: their arrivals are counted)
+      bool go = true;
+#pragma unroll
+      for (int m = 0; m < 2; ++m)
 #pragma unroll
         for (int i = 0; i < HELD; ++i)
-          if ((part + i * kParts) * COLS < (int)n0) tmem_ld16_nowait(lanes + (uint32_t)((part + i * kParts) * COLS), reinterpret_cast<uint32_t*>(held[CG == 2 ? i : 0]));
-        tmem_ld_wait();
-        tc_fence_before();
+#pragma unroll
+          for (int j = 0; j < COLS; ++j) held[m][i][j] = 0.f;
+      auto take = [&](uint32_t& at, float (&sum)[HELD][COLS], int t) {
+        if (go) go = __all_sync(0xffffffffu, wait(turn_full, (uint32_t)t & 1u, 245));
+        if (go && live) {
+          tc_fence_after();
+          float v[HELD][COLS];
+#pragma unroll
+          for (int i = 0; i < HELD; ++i) tmem_ld16_nowait(at + (uint32_t)((part + i * kParts) * COLS), reinterpret_cast<uint32_t*>(v[i]));
+          tmem_ld_wait();
+          tc_fence_before();
+#pragma unroll
+          for (int i = 0; i < HELD; ++i)
+#pragma unroll
+            for (int j = 0; j < COLS; ++j) sum[i][j] += v[i][j];
+        }
+        __syncwarp();
+        if (lane == 0) mbar_arrive_cluster(mapa_u32(smem_u32(&turn_done), 0));
+        const uint32_t done = at;
+        at = spare;
+        spare = done;
+      };
+      for (int t = 0; t < p.turns; t += 2) {
+        take(at0, held[0], t);
+        if (t + 1 < p.turns) take(at1, held[1], t + 1);
       }
-      __syncwarp();
-      if (lane == 0) mbar_arrive_cluster(mapa_u32(smem_u32(&turn_done), 0));
+      live = live && go;
     }
     if (live && __all_sync(0xffffffffu, wait(acc_full, 0, 243))) {
       tc_fence_after();
@@ -352,7 +392,8 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_rows_kernel(const __grid_con
           for (int half = 0; half < 2; ++half) {
             int lg = 2 * c + half, r = 0;                    // the column group's place among its CTA's, and which CTA that is
             if constexpr (CG == 2) {
-              const int base = lg < 2 * p.groups0 ? 0 : p.groups0, here = base ? p.groups - base : p.groups0;
+              const int base = !turning || c < kTurnGroups ? 0 : c < 2 * kTurnGroups ? kTurnGroups : 2 * kTurnGroups;
+              const int here = turning && c < 2 * kTurnGroups ? kTurnGroups : p.groups - base;
               lg -= 2 * base;
               r = lg >= here ? 1 : 0;
               lg += base - r * here;
@@ -378,28 +419,29 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_rows_kernel(const __grid_con
             if (4 * g[1] < p.F) *reinterpret_cast<uint2*>(at + 4 * g[1]) = o[1];
           }
         };
-        if (CG == 2 && two) {
-          const uint32_t n = 16u * (uint32_t)p.groups;
+        if (CG == 2 && turning) {
 #pragma unroll
-          for (int i = 0; i < HELD; ++i) {
-            const int c = part + i * kParts;
-            if (c * COLS < (int)n0) {
+          for (int m = 0; m < 2; ++m)
+#pragma unroll
+            for (int i = 0; i < (CG == 2 ? HELD : 1); ++i) {
+              const int c = part + i * kParts;
               float v[COLS];
-              tmem_ld16_nowait(lanes + n + (uint32_t)(c * COLS), reinterpret_cast<uint32_t*>(v));
+              tmem_ld16_nowait((m ? at1 : at0) + (uint32_t)(c * COLS), reinterpret_cast<uint32_t*>(v));
               tmem_ld_wait();
 #pragma unroll
-              for (int j = 0; j < COLS; ++j) v[j] += held[CG == 2 ? i : 0][j];
-              finish(c, v);
+              for (int j = 0; j < COLS; ++j) v[j] += held[m][i][j];
+              finish(c + m * kTurnGroups, v);
             }
-          }
-          for (int c = (int)n0 / COLS + part; c < p.groups; c += kParts) {
+          const int rest = p.groups - 2 * kTurnGroups;
+          for (int c = part; c < rest; c += kParts) {
             float v[COLS], t[COLS];
-            tmem_ld16_nowait(lanes + (uint32_t)(c * COLS), reinterpret_cast<uint32_t*>(v));
-            tmem_ld16_nowait(lanes + (uint32_t)(c * COLS) - n0, reinterpret_cast<uint32_t*>(t));
+            const uint32_t from = lanes + (uint32_t)(3 * kTurnCols + c * COLS);
+            tmem_ld16_nowait(from, reinterpret_cast<uint32_t*>(v));
+            tmem_ld16_nowait(from + (uint32_t)(rest * COLS), reinterpret_cast<uint32_t*>(t));
             tmem_ld_wait();
 #pragma unroll
             for (int j = 0; j < COLS; ++j) v[j] += t[j];
-            finish(c, v);
+            finish(c + 2 * kTurnGroups, v);
           }
         } else {
           for (int c = part; 2 * c < CG * p.groups; c += kParts) {
@@ -536,8 +578,7 @@ RowsRing plan_ring(const RowsPlan& g, int limit, int K, const Chains& other) {
   r.issuers = r.stages % 3 == 0 && 3 * cols <= 512 ? 3 : r.stages % 2 == 0 ? 2 : g.groups >= 16 ? 1 : 2;
   r.stages -= r.stages % r.issuers;
   if (r.issuers > least_kb) r.issuers = least_kb;
-  int most = 512 / cols < least_kb ? 512 / cols : least_kb;
-  if (most > kChains) most = kChains;
+  const int most = 512 / cols < least_kb ? 512 / cols : least_kb;
   r.chains = r.issuers < 3 && 2 * r.issuers <= most ? 2 * r.issuers : r.issuers;
   while (r.chains <= most && !ring_chains(g, r, num_kb).no_longer_than(other)) ++r.chains;
   if (r.chains > most) r.chains = 0;
@@ -552,15 +593,25 @@ Chains gemm_rows_other_chains(int limit, int N, int K) {
 }
 namespace {
 
-// Two MMAs per 16 k: blocks after which each goes over to its second accumulator
-int turn0(int num_kb) { return num_kb * 30 / 64; }
-int turn1(int num_kb) { return num_kb * 34 / 64; }
-Chains two_chains(int num_kb) {
+// Three MMAs per 16 k: a change of accumulators every eighth of k
+int turn_blocks(int num_kb) { return num_kb / 8; }
+int turn_count(int num_kb) { return (num_kb - 1) / turn_blocks(num_kb); }
+bool turns_fit(const RowsPlan& g, int K) {
+  return 3 * kTurnCols + 2 * (16 * g.groups - 2 * kTurnCols) <= 512 && (K + BK - 1) / BK >= 16;
+}
+Chains turn_chains(const RowsPlan& g, int num_kb) {
   Chains c;
-  for (int turn : {turn0(num_kb), turn1(num_kb)}) {
-    c.chain(turn);
-    c.chain(num_kb - turn);
-  }
+  for (int column = 0; column < g.groups; ++column)                // (16 columns at a time)
+    if (column < 2 * kTurnGroups) {
+      int since = 0;
+      for (int t = column / kTurnGroups; t < turn_count(num_kb); t += 2) {
+        c.chain((t + 1) * turn_blocks(num_kb) - since);
+        since = (t + 1) * turn_blocks(num_kb);
+      }
+      c.chain(num_kb - since);
+    } else {
+      c.add(num_kb, 2);
+    }
   return c;
 }
 void plan_rings(RowsPlan& g, int N, int K) {
@@ -568,8 +619,8 @@ void plan_rings(RowsPlan& g, int N, int K) {
     const int limit = rows_class_limit(i);
     if (g.heads && limit > ROWS && limit <= 192) continue;
     if (limit > ROWS && g.groups > 16) {
-      if (g.heads || (g.groups + (g.groups + 1) / 2) * 16 > 512 || K < 16 * BK) continue;
-      g.ring[i] = RowsRing{ring_stages(g, limit), 1, 2};
+      if (g.heads || !turns_fit(g, K) || !turn_chains(g, (K + BK - 1) / BK).no_longer_than(gemm_rows_other_chains(limit, N, K))) continue;
+      g.ring[i] = RowsRing{ring_stages(g, limit), 2, 5};
     } else {
       g.ring[i] = plan_ring(g, limit, K, gemm_rows_other_chains(limit, N, K));
     }
@@ -599,12 +650,11 @@ RowsPlan plan_rows_rope(int n_heads, int head_dim, int K) {
   return g;
 }
 
-// A pair's tile is up to 256 columns wide in one MMA, or has room for three accumulators.
 // Which products come here, from 9 rows on.
 //   Up to 128 rows, against partial sums and kernels behind them: matrices of at least 16 rows per SM (an MMA's N is no less) and at most 256.
 //   Forwards, plain sums (below) included: 7B width 9 / 64 / 128 rows 1.06 / 1.06 / 1.12 x, 13B 1.02 / 1.09 / 1.13 x, 1024 to 3200 columns 1.04 to 1.25 x.
 //   129 to 256 rows, in pairs, against output tiles of 256 weight rows (gemm_tile.cu): a pair's tile has to fit one MMA, or (SwiGLU, 16 k
-//   blocks and more) three accumulators.  Tiles of 256 rows leave SMs idle or have to be cut along k: 7B width, gate-up of 129 / 256 rows 46 / 53 -> 41 /
+//   blocks and more, up to 304 columns) three as above.  Tiles of 256 rows leave SMs idle or have to be cut along k: 7B width, gate-up of 129 / 256 rows 46 / 53 -> 41 /
 //   43 us.  RoPE from 193 rows on: below, the output tiles are cut and sum shorter chains than those that fit here (keys of 130 to 180 rows against float64
 //   1.10e-4 to 1.32e-4 there, 1.32e-4 to 1.52e-4 here).  From 193 rows on they are as long at 4096 columns and more (QKV of 256 rows 32.5 -> 27 us) and fit at 1024
 //   and 1536; from 2048 to 3584 they do not (2048 columns, 2 x 128 rows, 8 layers: 580 us here, 645 with output tiles; V 0.44 against 0.24e-6 from float64).
@@ -616,7 +666,7 @@ bool gemm_rows_takes(const RowsPlan& g, int M) {
 Chains gemm_rows_chains(const RowsPlan& g, int M, int K) {
   const RowsRing& r = g.ring[rows_class(M)];
   const int num_kb = (K + BK - 1) / BK;
-  return M > ROWS && g.groups > 16 ? two_chains(num_kb) : ring_chains(g, r, num_kb);
+  return M > ROWS && g.groups > 16 ? turn_chains(g, num_kb) : ring_chains(g, r, num_kb);
 }
 
 // Plain sums of up to 128 rows (O, down, LM head): k is cut into parts, each a sum of its own (a slot) for the kernel behind to add, so that tiles are wide
@@ -662,16 +712,15 @@ int launch_gemm_rows(cerb_ctx* c, const CUtensorMap* tmW, const ActMaps* tmX, co
   p.out = out;
   p.N = N;
   p.parts = g.parts;
-  p.groups = p.groups0 = g.groups;
+  p.groups = g.groups;
   p.x_rows = (int)rows_fetched(M);
   p.m_rows = mma_rows(M);
   p.stages = g.ring[i].stages;
   p.issuers = g.ring[i].issuers;
   p.chains = g.ring[i].chains;
   if (pairs && g.groups > 16) {
-    p.groups0 = (g.groups + 1) / 2;
-    p.turn0 = turn0(p.num_kb);
-    p.turn1 = turn1(p.num_kb);
+    p.turn = turn_blocks(p.num_kb);
+    p.turns = turn_count(p.num_kb);
     p.tmem_cols = 512;
   } else {
     p.acc_cols = (uint32_t)acc_columns(g, M);
@@ -681,7 +730,7 @@ int launch_gemm_rows(cerb_ctx* c, const CUtensorMap* tmW, const ActMaps* tmX, co
   p.clk = clock_slot;
   auto run = [&](auto kind, const CUtensorMap& x) {
     constexpr int KIND = decltype(kind)::value;
-    if (p.chains > 4) return pairs ? launch_kind<KIND, 2, true>(*tmW, x, p, g.tiles, st) : launch_kind<KIND, 1, true>(*tmW, x, p, g.tiles, st);
+    if (p.chains > 4 && !p.turns) return pairs ? launch_kind<KIND, 2, true>(*tmW, x, p, g.tiles, st) : launch_kind<KIND, 1, true>(*tmW, x, p, g.tiles, st);
     return pairs ? launch_kind<KIND, 2, false>(*tmW, x, p, g.tiles, st) : launch_kind<KIND, 1, false>(*tmW, x, p, g.tiles, st);
   };
   int rc;

@@ -16,12 +16,14 @@ pytestmark = pytest.mark.gpu
 SHAPES = {
     "16 and 16 rows, one k block": (64, 4, 1184),                # the least of both plans
     "16 and 24 rows, ragged k block": (200, 4, 1192),            # one feature group more than two per SM
-    "32 and 152 rows, two MMAs per pair": (1096, 10, 11000),     # odd number of groups; the last tile of SwiGLU half empty
-    "112 and 168 rows": (1024, 40, 12432),                       # the widest pair of MMAs
+    "32 and 152 rows, three MMAs per pair": (1096, 10, 11000),   # odd number of groups; the last tile of SwiGLU half empty; ragged k
+    "112 and 168 rows": (1024, 40, 12432),                       # too wide for a pair: above 128 rows gate-up is the output tiles'
+    "16 and 144 rows, three MMAs per pair": (1024, 4, 10600),    # the fewest k blocks; an even number of groups
+    "16 and 136 rows, three MMAs per pair": (1984, 4, 9504),     # 31 k blocks: the most changes of accumulators; the smallest third MMA
 }
 # prompt lengths: rows of one accumulator quarter, its edges, all of them; pairs: one row in the second CTA's half and all
 CASES = [(n, m) for n in SHAPES for m in (9, 33, 64, 65, 128, 129, 256)]
-CASES += [("32 and 152 rows, two MMAs per pair", m) for m in (96, 97, 192, 193)]          # ... and both sides of the other plans' edges
+CASES += [("32 and 152 rows, three MMAs per pair", m) for m in (96, 97, 192, 193)]          # ... and both sides of the other plans' edges
 
 
 def _prompt_matches_oracle(d, H, F, M):
@@ -50,14 +52,14 @@ def test_prompts_match_oracle(name, M):
     if M <= 128:
         assert launches == 1 + 1 + 7 + 3
     # ... of which these are this kernel's
-    assert [cb.forward_gemm_plan(p, M, N, d).rows_kernel for p, N in (("gate_up", 2 * F), ("qkv", 384 * H))] == [1, M <= 128 or M > 192]
+    assert [cb.forward_gemm_plan(p, M, N, d).rows_kernel for p, N in (("gate_up", 2 * F), ("qkv", 384 * H))] == [M <= 128 or F < 12000, M <= 128 or M > 192]
 
 
 # More accumulators than two per issuer, and numbers of them that the issuers do not divide: (rows, product, issuers, accumulators)
 @pytest.mark.parametrize("d,H,F,M,product,issuers,chains", [
     (1024, 8, 2816, 9, "qkv", 3, 6), (1024, 8, 2816, 97, "qkv", 2, 4), (1024, 8, 2816, 256, "qkv", 2, 6), (1536, 12, 4096, 97, "qkv", 2, 6),
     (1024, 8, 2816, 33, "gate_up", 2, 4), (1024, 8, 4096, 128, "gate_up", 3, 6), (2048, 4, 5632, 9, "gate_up", 3, 5), (3584, 4, 9728, 65, "gate_up", 1, 3),
-    (1024, 8, 1024, 129, "o_down", 3, 5), (1024, 8, 1024, 250, "o_down", 3, 5), (4096, 32, 1184, 96, "qkv", 3, 4),
+    (1024, 8, 1024, 129, "o_down", 3, 5), (1024, 8, 1024, 250, "o_down", 3, 5), (4096, 32, 1184, 96, "qkv", 3, 4), (1984, 4, 1184, 40, "qkv", 3, 9), (1984, 4, 1184, 200, "qkv", 3, 9),
 ])
 def test_accumulators_in_turn_match_oracle(d, H, F, M, product, issuers, chains):
     N = {"qkv": 384 * H, "gate_up": 2 * F, "o_down": d}[product]
@@ -69,7 +71,7 @@ def test_accumulators_in_turn_match_oracle(d, H, F, M, product, issuers, chains)
 @pytest.mark.parametrize("n,live", [(40, (40, 17, 1)), (70, (1, 70, 33))])
 def test_trees_with_dead_nodes_match_oracle(n, live):
     """Three sequences (120 and 210 rows): rows of nodes that are not live write nothing."""
-    d, H, F = SHAPES["32 and 152 rows, two MMAs per pair"]
+    d, H, F = SHAPES["32 and 152 rows, three MMAs per pair"]
     ms = synth.ModelShape(1, d, H, 128, F, 512, "bf16")
     rig = Rig(cb, ms, max_tokens=128, max_batch=3, max_nodes=n)
     lens = [29, 16, 5]
