@@ -170,7 +170,6 @@ __global__ void __launch_bounds__((WQ * WK + 1) * 32) tree_attn_bf16_kernel(cons
   float* mrg = reinterpret_cast<float*>(smem_gen);   // [NQ][ROWF], used after the key loop
 
   if (warp == NW) {
-    int issued = 0;                                    // (lane 0: tiles whose copies it has issued)
     // ---------------- producer warp ----------------
     const int32_t* pt = p.page_table + (size_t)b * p.max_pages;
     const int n_pages = (t_end - t0) * PAGES_PER_TILE;
@@ -185,8 +184,8 @@ __global__ void __launch_bounds__((WQ * WK + 1) * 32) tree_attn_bf16_kernel(cons
       // (the abort flag itself is looked at once, for a launch that starts after a time-out: nothing is issued then;
       // later a wait that gives up says so in its return value, which costs the loop nothing)
       const int t_stop = *aborted ? t0 : t_end;
-      for (int t = t0; t < t_stop; ++t, ++issued) {
-        const int i = issued;
+      int i = 0;
+      for (int t = t0; t < t_stop; ++t, ++i) {
         if (i == early) { griddep_wait(); griddep_launch(); }
         int s = i % STAGES;
         uint32_t ph = (uint32_t)(i / STAGES) & 1u;
@@ -205,10 +204,14 @@ __global__ void __launch_bounds__((WQ * WK + 1) * 32) tree_attn_bf16_kernel(cons
           }
         }
       }
+      if (*aborted) {
+        // give-up path: the copies already issued (units 0 .. i-1) still land in this CTA's shared memory; see each of them in
+        for (int j = i > STAGES ? i - STAGES : 0; j < i; ++j)
+          mbar_wait_drain(smem_u32(&full_bar[j % STAGES]), (uint32_t)(j / STAGES) & 1u, 20000000ll);
+      }
     }
     griddep_wait();      // (a lane that has waited already returns at once)
     griddep_launch();
-    see_own_copies_in(smem_u32(&full_bar[0]), STAGES, issued, lane, 20000000ll);
   } else {
     // ---------------- compute warps ----------------
     griddep_wait();
@@ -678,8 +681,12 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tree_attn_tc_kernel(const __gri
         if (++slot == ring) { slot = 0; ph ^= 1u; }
       }
     }
+    if (lane == 0 && *aborted) {
+      // give-up path: the copies already issued still land in this CTA's shared memory; see each of them in
+      for (int j = issued > ring ? issued - ring : 0; j < issued; ++j)
+        mbar_wait_drain(smem_u32(&full[j % ring]), (uint32_t)(j / ring) & 1u, 20000000ll);
+    }
     enter();             // (a lane that has waited already returns at once)
-    see_own_copies_in(smem_u32(full), ring, issued, lane, 20000000ll);
   } else if (warp == 1) {
     enter();
     // ---------------- QK^T issuer ----------------
@@ -716,7 +723,10 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tree_attn_tc_kernel(const __gri
           if (++slot == SK) { slot = 0; ph ^= 1u; }
         }
       }
-      if (elect_one()) see_mmas_retire<1>(smem_u32(&drain_bar[0]), 20000000ll);
+      if (__any_sync(0xffffffffu, *aborted) && elect_one()) {                                // give-up path: see the MMAs already issued retire
+        umma_commit(smem_u32(&drain_bar[0]));
+        mbar_wait_drain(smem_u32(&drain_bar[0]), 0, 20000000ll);
+      }
     }
   } else if (warp == 10) {
     enter();
@@ -751,7 +761,10 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tree_attn_tc_kernel(const __gri
           if (++slot == SV) { slot = 0; vph ^= 1u; }
         }
       }
-      if (elect_one()) see_mmas_retire<1>(smem_u32(&drain_bar[1]), 20000000ll);
+      if (__any_sync(0xffffffffu, *aborted) && elect_one()) {                                // give-up path: see the MMAs already issued retire
+        umma_commit(smem_u32(&drain_bar[1]));
+        mbar_wait_drain(smem_u32(&drain_bar[1]), 0, 20000000ll);
+      }
     }
   } else {
     // ---------------- softmax groups: thread <-> query row, group g takes tiles g, g+2, ... ----------------

@@ -75,16 +75,6 @@ __device__ __noinline__ bool wait_for_partner(uint32_t bar, long long budget) {
   return mbar_wait_drain(bar, 0, partner_cycles(w));
 }
 
-// What see_own_copies_in is for, of the units of one kind (t-th: unit 2 t + kind, in slot u % nu) that a producer has issued, and of its boxes of the first K unit (of
-// more units than slots the last ones go out only when the first have been used).  A phase also needs the other producers' shares.
-static __device__ __noinline__ void see_units_in(uint32_t first_unit, uint32_t full, int kind, int issued, int nu) {
-  if (kind && issued >= 0 && issued <= nu / 2) mbar_wait_drain(first_unit, 0, 20000000ll);
-  for (int t = issued > nu / 2 ? issued - nu / 2 : 0; t < issued; ++t) {
-    const int u = 2 * t + kind;
-    mbar_wait_drain(full + 8u * (uint32_t)(u % nu), (uint32_t)(u / nu) & 1u, 20000000ll);
-  }
-}
-
 template <bool PART>
 __global__ void __launch_bounds__(KT_THREADS, 1) tree_attn_kt_kernel(const __grid_constant__ CUtensorMap tmK,
                                                                      const __grid_constant__ CUtensorMap tmV,
@@ -222,7 +212,7 @@ __global__ void __launch_bounds__(KT_THREADS, 1) tree_attn_kt_kernel(const __gri
     const int box = (pw >> 1) + (NPROD / 2) * lane;  // lanes 0 .. BOXES-1
     const int pg = box >> 1, hf = box & 1;
     const uint64_t pol = l2_policy(true);            // K/V are read once per step
-    int issued = -1;                                 // units of this warp's kind whose copies it has issued, -1: none of any kind
+    int issued = 0;
     // (the abort flag itself is looked at once, for a launch that starts after a time-out: nothing is issued then;
     // later a wait that gives up says so in its return value, which costs the loop nothing)
     const int t_stop = *aborted ? 0 : T;
@@ -237,7 +227,7 @@ __global__ void __launch_bounds__(KT_THREADS, 1) tree_attn_kt_kernel(const __gri
         tma_load_2d_hint(ring + (uint32_t)hf * KT_HALF + (uint32_t)pg * (CERB_PAGE * 128), &tmK, hf * 64, page_list[pg], smem_u32(&full_u[0][0]), pol);
       issued = 1 - kind;
     }
-    for (int t = max(issued, 0); t < t_stop; ++t) {
+    for (int t = issued; t < t_stop; ++t) {
       if (t == early) enter();
       const int u = 2 * t + kind, slot = u % NU;
       const uint32_t fb = smem_u32(&full_u[kind][slot]);
@@ -254,8 +244,14 @@ __global__ void __launch_bounds__(KT_THREADS, 1) tree_attn_kt_kernel(const __gri
       }
       issued = t + 1;
     }
+    if (lane == 0 && *aborted) {
+      // give-up path: the copies this warp has issued still land in the CTA's shared memory; see them in (the
+      // phase also needs the other producers' shares, hence a limit of its own: 10 ms)
+      if (kind && t_stop > 0) mbar_wait_drain(smem_u32(&full_u[0][0]), 0, 20000000ll);
+      for (int t = issued > NU / 2 ? issued - NU / 2 : 0; t < issued; ++t)
+        mbar_wait_drain(smem_u32(&full_u[kind][(2 * t + kind) % NU]), unit_parity(2 * t + kind), 20000000ll);
+    }
     enter();             // (a lane that has waited already returns at once)
-    if (lane == 0) see_units_in(smem_u32(&full_u[0][0]), smem_u32(&full_u[kind][0]), kind, issued, NU);
   } else if (warp == W_QK) {
     enter();
     // ---------------- QK^T issuer ----------------
@@ -282,7 +278,10 @@ __global__ void __launch_bounds__(KT_THREADS, 1) tree_attn_kt_kernel(const __gri
         }
         __syncwarp();
       }
-      if (elect_one()) see_mmas_retire<1>(smem_u32(&drain_bar[0]), 20000000ll);
+      if (__any_sync(0xffffffffu, *aborted) && elect_one()) {                                // give-up path: see the MMAs already issued retire
+        umma_commit(smem_u32(&drain_bar[0]));
+        mbar_wait_drain(smem_u32(&drain_bar[0]), 0, 20000000ll);
+      }
     }
   } else if (warp == W_PV) {
     enter();
@@ -310,6 +309,10 @@ __global__ void __launch_bounds__(KT_THREADS, 1) tree_attn_kt_kernel(const __gri
         }
         __syncwarp();
       }
+      if (__any_sync(0xffffffffu, *aborted) && elect_one()) {                                // give-up path: see the MMAs already issued retire
+        umma_commit(smem_u32(&drain_bar[1]));
+        mbar_wait_drain(smem_u32(&drain_bar[1]), 0, 20000000ll);
+      }
       if (p.cluster) {
         // Q is staged and every MMA has retired: this CTA's rx may be written.  (Said from here the release costs the softmax warps nothing.)
         __syncwarp();
@@ -318,7 +321,6 @@ __global__ void __launch_bounds__(KT_THREADS, 1) tree_attn_kt_kernel(const __gri
         cluster_start_wait();
         if (lane < p.nsplit) mbar_arrive_cluster(mapa_u32(smem_u32(&cl_bar[0]), (uint32_t)lane));
       }
-      if (elect_one()) see_mmas_retire<1>(smem_u32(&drain_bar[1]), 20000000ll);
     }
   } else {
     // ---------------- softmax: thread = (key lane of the tile, block of QB queries) ----------------

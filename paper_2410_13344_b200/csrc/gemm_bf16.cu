@@ -95,7 +95,7 @@ __global__ void __launch_bounds__(224, 1) gemm_bf16_kernel(const __grid_constant
   __shared__ __align__(8) uint64_t acc_empty[2];
   __shared__ __align__(8) uint64_t drain_bar[2];       // one per MMA issuer: "everything I issued has retired" (give-up path only)
   __shared__ uint32_t tmem_base_slot;
-  __shared__ int aborted_s, issued_s;                  // issued_s: units whose copies the producer has issued, once it has stopped
+  __shared__ int aborted_s;
   volatile int* aborted = &aborted_s;
   const WaitCtx wc{p.wait_cycles, aborted, p.status, p.N + 100000 * (p.M > 999 ? 999 : p.M)};
 
@@ -110,7 +110,6 @@ __global__ void __launch_bounds__(224, 1) gemm_bf16_kernel(const __grid_constant
 
   if (threadIdx.x == 0) {
     aborted_s = 0;
-    issued_s = -1;
     for (int s = 0; s < p.stages; ++s) {
       mbar_init(smem_u32(&full_bar[s]), 1);
       mbar_init(smem_u32(&empty_bar[s]), 2);
@@ -179,7 +178,6 @@ __global__ void __launch_bounds__(224, 1) gemm_bf16_kernel(const __grid_constant
         load_x(i);
         issued = i + 1;
       }
-      *(volatile int*)&issued_s = issued;
       if (*aborted) {
         // give-up path: the copies already issued still land in this CTA's shared memory; see each of them in
         for (int i = issued > p.stages ? issued - p.stages : 0; i < issued; ++i)
@@ -192,7 +190,6 @@ __global__ void __launch_bounds__(224, 1) gemm_bf16_kernel(const __grid_constant
     // its own issuing thread (warp 1: first tile, warp 6: second tile).  A stage is free, and an accumulator
     // complete, once both have committed.
     const int hf = warp == 6 ? 1 : 0;
-    bool live = true;
     if (lane == 0) {
       int u = u0;
       Segment sg;
@@ -200,13 +197,13 @@ __global__ void __launch_bounds__(224, 1) gemm_bf16_kernel(const __grid_constant
       while (next_segment(u, u1, p.num_kb, sg)) {
         const int buf = g & 1;
         const uint32_t use = (uint32_t)(g >> 1);      // how often this buffer was used before
-        if (!mbar_wait(smem_u32(&acc_empty[buf]), (use & 1u) ^ 1u, wc, 202)) { live = false; break; }
+        if (!mbar_wait(smem_u32(&acc_empty[buf]), (use & 1u) ^ 1u, wc, 202)) break;
         tc_fence_after();
         const uint32_t tmem_d = tmem_base + (uint32_t)buf * p.acc_cols;
         for (int k = 0; k < sg.nkb; ++k, ++i) {
           int s = i % p.stages;
           uint32_t ph = (uint32_t)(i / p.stages) & 1u;
-          if (!mbar_wait(smem_u32(&full_bar[s]), ph, wc, 203)) { live = false; break; }
+          if (!mbar_wait(smem_u32(&full_bar[s]), ph, wc, 203)) break;
           tc_fence_after();
           uint32_t a_src = smem_base + (uint32_t)s * stage_bytes;
           uint64_t bdesc = desc_k_sw128(a_src + a_bytes);
@@ -217,13 +214,16 @@ __global__ void __launch_bounds__(224, 1) gemm_bf16_kernel(const __grid_constant
             umma_bf16(d, adesc + (uint64_t)(kk * 2), bdesc + (uint64_t)(kk * 2), p.idesc, (k > 0 || kk > 0) ? 1u : 0u);
           umma_commit(smem_u32(&empty_bar[s]));     // the stage is free once the MMAs have read it
         }
-        if (!live) break;
+        if (*aborted) break;
         umma_commit(smem_u32(&acc_full[buf]));       // this thread's part of the segment's accumulator is complete
         ++g;
       }
-      see_mmas_retire<1>(smem_u32(&drain_bar[hf]), kDrainCycles);
+      if (*aborted) {
+        // give-up path: the MMAs already issued still read shared memory and write tensor memory; see them retire
+        umma_commit(smem_u32(&drain_bar[hf]));
+        mbar_wait_drain(smem_u32(&drain_bar[hf]), 0);
+      }
     }
-    if (!__shfl_sync(0xffffffffu, live, 0)) see_copies_in(smem_u32(&full_bar[0]), p.stages, &issued_s, lane, kDrainCycles);
   } else {
     const int quarter = warp & 3;                    // TMEM lanes 32*quarter .. +31 belong to this warp
     griddep_wait();                                  // the kernel before this one may still be reading the partial buffer

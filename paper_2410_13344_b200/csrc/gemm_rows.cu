@@ -99,7 +99,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_rows_kernel(const __grid_con
   __shared__ __align__(8) uint64_t acc_full, drain_bar[kIssuers];
   __shared__ __align__(8) uint64_t turn_full, turn_done, meet_bar;       // turn_done: first CTA only, all epilogue warps of the pair arrive
   __shared__ uint32_t tmem_base_slot;
-  __shared__ int aborted_s, meet_flag_s, issued_s;           // issued_s: k blocks whose copies the producer has issued, once it has stopped
+  __shared__ int aborted_s, meet_flag_s;
   volatile int* aborted = &aborted_s;
   const WaitCtx wc{p.wait_cycles, aborted, p.status, KIND + 10 * p.num_kb + 100000 * p.M};
 
@@ -120,7 +120,6 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_rows_kernel(const __grid_con
   if (threadIdx.x == 0) {
     aborted_s = 0;
     meet_flag_s = 0;
-    issued_s = -1;
     for (int s = 0; s < p.stages; ++s) {
       mbar_init(smem_u32(&full_bar[s]), 1);
       mbar_init(smem_u32(&empty_bar[s]), turning ? 2 : 1);
@@ -186,13 +185,12 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_rows_kernel(const __grid_con
         issued = i + 1;
         if (++s == p.stages) { s = 0; ph ^= 1u; }
       }
-      *(volatile int*)&issued_s = issued;
       if (*aborted) {
         // give-up path: the copies already issued still land in this CTA's shared memory; see each of them in.  (A pair's are counted on
         // the first CTA's barriers, and the CTAs may have stopped at different stages: both let the time of many round trips pass, too.)
         if (first)
           for (int i = issued > p.stages ? issued - p.stages : 0; i < issued; ++i)
-            mbar_wait_drain(smem_u32(&full_bar[i % p.stages]), (uint32_t)(i / p.stages) & 1u, CG == 2 ? kPairCopyCycles : kDrainCycles);
+            mbar_wait_drain(smem_u32(&full_bar[i % p.stages]), (uint32_t)(i / p.stages) & 1u, CG == 2 ? 2000000ll : kDrainCycles);
         const long long t_land = clock64();
         while (CG == 2 && clock64() - t_land < 400000ll) __nanosleep(1000);
       }
@@ -276,10 +274,15 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_rows_kernel(const __grid_con
           if (++s == p.stages) { s = 0; ph ^= 1u; }
         }
       }
-      if (!live) see_copies_in(smem_u32(&full_bar[0]), p.stages, &issued_s, lane, CG == 2 ? kPairCopyCycles : kDrainCycles);
       if (elect_one()) {
         if (live) commit(acc_full);
-        see_mmas_retire<CG>(smem_u32(&drain_bar[self]), CG == 2 ? 40000000ll : kDrainCycles);
+        if (!live || *aborted) {
+          // give-up path, whoever's wait ran out: the MMAs already issued still read shared memory and write tensor memory; see them retire
+          if constexpr (CG == 2)
+            asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(&drain_bar[self])) : "memory");
+          else umma_commit(smem_u32(&drain_bar[self]));
+          mbar_wait_drain(smem_u32(&drain_bar[self]), 0, CG == 2 ? 40000000ll : kDrainCycles);
+        }
       }
     }
   } else if (warp >= 4) {
@@ -518,10 +521,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_rows_kernel(const __grid_con
   if (p.clk && threadIdx.x == 0) atomicMax(p.clk + kGemmClockSlots, globaltimer_ns());
   if constexpr (CG == 2) {
     // Neither CTA leaves (nor frees its tensor memory) before the other is done: copies, commits and arrivals cross between them until then.
-    if (warp == 2) {
-      if (*aborted) let_pair_copies_land();
-      cluster_meet_before_exit(&meet_bar, 2, lane, wc, &meet_flag_s, 246);
-    }
+    if (warp == 2) cluster_meet_before_exit(&meet_bar, 2, lane, wc, &meet_flag_s, 246);
     __syncthreads();
     if (warp == 1) asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(p.tmem_cols) : "memory");
   } else {

@@ -261,7 +261,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tile_kernel(const __grid_con
   __shared__ __align__(8) uint64_t drain_bar, meet_bar;
   __shared__ int pos_s[KIND == 2 ? TILE_X : 1], kv_s[KIND == 2 ? TILE_X : 1];
   __shared__ uint32_t tmem_base_slot;
-  __shared__ int aborted_s, meet_flag_s, issued_s;            // issued_s: stages whose copies the producer has issued, once it has stopped
+  __shared__ int aborted_s, meet_flag_s;
   volatile int* aborted = &aborted_s;
   const WaitCtx wc{p.wait_cycles, aborted, p.status, p.N + 100000 * (p.M > 999 ? 999 : p.M)};
 
@@ -275,7 +275,6 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tile_kernel(const __grid_con
   if (threadIdx.x == 0) {
     aborted_s = 0;
     meet_flag_s = 0;
-    issued_s = -1;
     for (int s = 0; s < p.stages; ++s) {
       mbar_init(smem_u32(&full_bar[s]), 1);
       mbar_init(smem_u32(&empty_bar[s]), 1);
@@ -340,7 +339,6 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tile_kernel(const __grid_con
         load_w();
         load_x();
       }
-      *(volatile int*)&issued_s = issued;
       if (*aborted) {
         // give-up path: this CTA's copies land in its own shared memory but are counted on the first CTA's
         // barriers, and the two CTAs may have stopped at different stages, so neither can see exactly its own
@@ -348,7 +346,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tile_kernel(const __grid_con
         // many memory round trips pass before they go on to the rendezvous and leave.
         if (first)
           for (int i = issued > p.stages ? issued - p.stages : 0; i < issued; ++i)
-            mbar_wait_drain(smem_u32(&full_bar[i % p.stages]), (uint32_t)(i / p.stages) & 1u, kPairCopyCycles);
+            mbar_wait_drain(smem_u32(&full_bar[i % p.stages]), (uint32_t)(i / p.stages) & 1u, 2000000ll);
         const long long t_land = clock64();
         while (clock64() - t_land < 400000ll) __nanosleep(1000);
       }
@@ -427,8 +425,10 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tile_kernel(const __grid_con
           ++g;
         }
       }
-      if (!live) see_copies_in(smem_u32(&full_bar[0]), p.stages, &issued_s, lane, kPairCopyCycles);
-      if (elect_one()) see_mmas_retire<2>(smem_u32(&drain_bar), 40000000ll);
+      if ((!live || *aborted) && elect_one()) {            // (an issuer whose own waits hold ends like the others, too)
+        asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(&drain_bar)) : "memory");
+        mbar_wait_drain(smem_u32(&drain_bar), 0, 40000000ll);
+      }
     }
   } else {
     const int quarter = warp & 3;                    // tensor-memory lanes 32 * quarter .. + 31 belong to this warp
@@ -620,10 +620,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tile_kernel(const __grid_con
   // Neither CTA leaves (nor frees its tensor memory) before the other is done: copies, commits and arrivals cross
   // between them until then.  The rendezvous keeps a budget of its own, far above that of the other waits, so that a
   // CTA which has given up still finds its partner.
-  if (warp == 2) {
-    if (*aborted) let_pair_copies_land();
-    cluster_meet_before_exit(&meet_bar, 2, lane, wc, &meet_flag_s, 225);
-  }
+  if (warp == 2) cluster_meet_before_exit(&meet_bar, 2, lane, wc, &meet_flag_s, 225);
   __syncthreads();
   if (warp == 1)
     asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(512u) : "memory");

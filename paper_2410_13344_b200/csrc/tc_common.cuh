@@ -40,13 +40,22 @@ struct WaitCtx {
                              // [3] `tag`
   int tag = 0;               // a number identifying the launch (for diagnosis)
 };
+// What the CTA's roles have begun must be over before it leaves, whichever role's wait is the first to run out.  A role that ends after that sees the flag and
+// waits for its copies and MMAs in flight.  One that had ended before saw nothing: so the thread that sets the flag, without which the CTA
+// does not leave, first lets the time of many memory round trips pass.  (This costs a launch whose waits hold nothing.  Roles that wait at their ends
+// in every launch cost 0 to 0.5 us in the GEMMs and 4 to 5 % of persistent attention, a test behind the CTA's last barrier 0.1 to 0.2 us, and
+// this function out of line 0.9 us where a rest of attention items gets a launch of its own.)
+constexpr long long kLandCycles = 400000ll;
 __device__ __forceinline__ void wait_ran_out(const WaitCtx& w, int site) {
+  const bool first = *w.aborted == 0;
   *w.aborted = 1;
   if (atomicExch(w.status, CERB_E_TIMEOUT) == 0) {
     w.status[1] = site;
     w.status[2] = (int)(blockIdx.x + 1000u * blockIdx.y + 1000000u * blockIdx.z);
     w.status[3] = w.tag;
   }
+  const long long t_land = clock64();
+  while (first && clock64() - t_land < kLandCycles) __nanosleep(1000);
 }
 // Once one wait in a CTA has run out (or an earlier kernel already reported a time-out), every later wait
 // of that CTA gives up after this many cycles, so the CTA still runs to its end in bounded time.
@@ -93,42 +102,6 @@ __device__ __forceinline__ bool mbar_wait_drain(uint32_t bar, uint32_t parity, l
       if (mbar_try_wait(bar, parity)) return true;
     if (clock64() - t0 > cycles) return false;
   }
-}
-// What a role of a kernel has begun must be over before its CTA leaves.  That follows from what the other roles wait for, until one of them gives up: which one
-// that is, and how early the others have ended by then, is open.  So a role's look at the CTA's abort flag is not enough.  An issuer waits for its own MMAs
-// at its end, in every launch (the epilogue waits for them as well).  Copies are waited for by the issuers block by block; one that
-// finds a block missing, and therefore leaves, first sees in whatever the producer has issued.  (Tests behind the CTA's last barrier cost 0.1 to 0.2 us a
-// launch, where code is fetched whether it runs or not; a GEMM's producer that waits for its last copies in every launch 0.2 to 0.5 us.)
-// Copies, by a whole warp, a lane to each of up to 32 stages: *issued is how many the producer has issued once it has stopped, -1 before.
-constexpr long long kProducerCycles = 40000000ll;
-static __device__ __noinline__ void see_copies_in(uint32_t full_bar, int stages, const volatile int* issued, int lane, long long cycles) {
-  const long long t0 = clock64();
-  while (*issued < 0 && clock64() - t0 < kProducerCycles) __nanosleep(200);
-  const int n = *issued;
-  if (lane < stages && lane < n) mbar_wait_drain(full_bar + 8u * (uint32_t)lane, (uint32_t)((n - 1 - lane) / stages) & 1u, cycles);
-  __syncwarp();
-}
-// The same for a producer warp whose lane 0 knows the number, in every launch (where it costs nothing).
-__device__ __forceinline__ void see_own_copies_in(uint32_t full_bar, int stages, int issued, int lane, long long cycles) {
-  issued = __shfl_sync(0xffffffffu, issued, 0);
-  if (lane < stages && lane < issued) mbar_wait_drain(full_bar + 8u * (uint32_t)lane, (uint32_t)((issued - 1 - lane) / stages) & 1u, cycles);
-}
-// MMAs of the calling thread read shared memory and write tensor memory; `bar` is used for nothing else.
-template <int CG>
-static __device__ __noinline__ void see_mmas_retire(uint32_t bar, long long cycles) {
-  if constexpr (CG == 2)
-    asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
-  else
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
-  mbar_wait_drain(bar, 0, cycles);
-}
-// A pair's copies are counted on its first CTA's barriers, and once a CTA has given up the two may have stopped at different stages: what see_copies_in
-// finds there (short budget: kPairCopyCycles) need not be all.  So a CTA of a pair that has given up also lets the time of many memory round trips
-// pass before the pair's last rendezvous.
-constexpr long long kPairCopyCycles = 2000000ll;
-static __device__ __noinline__ void let_pair_copies_land() {
-  const long long t_land = clock64();
-  while (clock64() - t_land < 400000ll) __nanosleep(1000);
 }
 // Same bounded wait for a lane whose warp shares an issue port with busy warps: back off between polls.
 __device__ __forceinline__ bool mbar_wait_polite(uint32_t bar, uint32_t parity, const WaitCtx& w, int site = 0) {

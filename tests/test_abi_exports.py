@@ -156,31 +156,32 @@ def test_no_forward_kernel_leaves_ahead_of_its_wait():
     assert seen >= 12
 
 
-def test_every_role_sees_in_what_it_has_begun():
-    """A kernel that gives up must not let a copy outlive its shared memory, nor an MMA its tensor memory.  Any role's wait may be the one that
-    runs out, when the others have already done all of theirs: so an issuer waits for its MMAs at its end in every launch, and copies are waited for in
-    every launch by their producer (attention) or by the issuers, of which one that leaves early sees in all that the producer has issued.  (Of a
-    pair's copies the second CTA cannot see its own: a CTA that has given up also lets them land before the two meet.)"""
+def test_every_role_of_a_kernel_that_gives_up_sees_in_what_it_has_begun():
+    """A kernel that gives up must not let a copy outlive its shared memory, nor an MMA its tensor memory, whichever role's wait is the first to run
+    out.  Roles that end after that look at the CTA's flag, and not only at what became of their own waits; for what roles had begun that ended before, the
+    thread that sets the flag lets the time of many memory round trips pass before it goes on (and the CTA leaves with all of its threads)."""
     src = os.path.join(ROOT, "paper_2410_13344_b200", "csrc")
-    always, leaving = r"see_(own_copies|units)_in\(", r"if \(!(live|__shfl_sync\(0xffffffffu, live, 0\))\) see_copies_in\("
-    # copies; MMAs; pairs
-    roles = {"gemm_bf16_kernel": (leaving, 1, 0), "gemm_tile_kernel": (leaving, 1, 1), "gemm_rows_kernel": (leaving, 1, 1),
-             "tree_attn_bf16_kernel": (always, 0, 0), "tree_attn_tc_kernel": (always, 2, 0), "tree_attn_kt_kernel": (always, 2, 0)}
+    # producers and issuers
+    roles = {"gemm_bf16_kernel": 2, "gemm_tile_kernel": 2, "gemm_rows_kernel": 2, "tree_attn_bf16_kernel": 1, "tree_attn_tc_kernel": 3, "tree_attn_kt_kernel": 3}
     for fn in sorted(os.listdir(src)):
         if not fn.endswith((".cu", ".cuh")):
             continue
         text = re.sub(r"//[^\n]*", "", open(os.path.join(src, fn)).read())
+        if fn == "tc_common.cuh":
+            give_up = text[text.index("void wait_ran_out("):]
+            give_up = give_up[:give_up.index("\n}\n")]
+            assert give_up.index("first = *w.aborted == 0;") < give_up.index("*w.aborted = 1;") < give_up.index("while (first && clock64() - t_land < kLandCycles)")
         for body in re.split(r"__global__", text)[1:]:
             body = body[:body.index("\n}\n")]
             if "WaitCtx wc" not in body:
                 continue
-            copies, mmas, pair = roles.pop(re.search(r"\b(\w+_kernel)\(", body).group(1))
-            assert len(re.findall(copies, body)) == 1 and len(re.findall(r"see_(own_copies|copies|units)_in\(", body)) == 1, fn
-            retire = [s for s in body.split("\n") if "see_mmas_retire" in s]
-            assert len(retire) == mmas and not any(w in s for s in retire for w in ("aborted", "live")), (fn, retire)
-            assert len(re.findall(r"if \(\*aborted\) let_pair_copies_land\(\);\s*cluster_meet_before_exit", body)) == pair, fn
-            if copies == leaving:                        # an issuer that leaves its loop early says so, whatever made it
-                assert not re.search(r"\*aborted\) break", body) and body.count("*(volatile int*)&issued_s = issued;") == 1, fn
+            name = re.search(r"\b(\w+_kernel)\(", body).group(1)
+            guards = []
+            for m in re.finditer(r"mbar_wait_drain\(", body):
+                # the `if` in front of it that looks at the flag, or at a role's own waits only
+                guards.append([g for g in re.findall(r"if \(([^\n{]*(?:aborted|live)[^\n{]*)\) \{", body[:m.start()])][-1])
+            assert guards and all("*aborted" in g for g in guards), (name, guards)
+            assert len(set(re.findall(r"if \([^\n{]*\*aborted[^\n{]*\) \{", body))) >= 1 and len(guards) >= roles.pop(name), (name, guards)
     assert not roles
 
 
