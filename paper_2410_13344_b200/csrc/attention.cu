@@ -1626,9 +1626,10 @@ static int launch_attn_window(cerb_ctx* c, const cerb_attn_args* a, int row0, in
     p.follows = row0 > 0 && use_cluster ? 1 : 0;                     // the second window of a wide tree (150 nodes behind 600 keys 28.4 -> 20.2 us)
     // More items than SMs: where the last round leaves half of the SMs and more without one, its items' keys are split over them in a launch of its
     // own, which needs nothing from the first one.  160 heads of 800 / 1564 / 4096 keys, 64 nodes: 30.7 / 44.9 / 94.9 us in one launch, 26.9 / 35.9 / 65.4 in two;
-    // 512: 65.6 / 95.4 / 217 and 66.1 / 91.8 / 201; below 768 keys the second launch costs as much as it gives (300 keys: 0.88 to 0.97 x).
+    // 512: 65.6 / 95.4 / 217 and 66.1 / 91.8 / 201; below 768 keys the second launch costs as much as it gives (300 keys: 0.88 to 0.97 x), and with a rest of more than 24,
+    // whose keys are cut into few splits, below 1024 (24 nodes behind 740 keys, 352 / 480 / 512 / 640 items: 0.99 / 0.99 / 0.975 / 0.96 x).
     const int rest = items % 148;
-    if (win == 1 && use_cluster && items > 148 && rest > 0 && rest <= 74 && tiles * tile >= 768) {
+    if (win == 1 && use_cluster && items > 148 && rest > 0 && rest <= 74 && tiles * tile >= (rest <= 24 ? 768 : 1024)) {
       const int ns = splits(rest);
       if (ns > 1 && splits(items) == 1) {
         rc = launch(items - rest, 1);
