@@ -25,6 +25,11 @@ pytestmark = pytest.mark.gpu
     # two launches over the rows; the second one with live rows in one sequence only
     (2, 150, 5, 128, [700, 333], [150, 128]),
     (3, 192, 50, 128, [800, 20, 130], [192, 129, 5]),
+    # ... whose second one takes fewer splits than would be there at once: 24 items in three, 32 in two, 64 in one; 40 of 3000 keys do not
+    (6, 150, 4, 128, [1000 - 7 * b for b in range(6)], None),
+    (1, 192, 32, 128, [300], None),
+    (2, 150, 32, 128, [310, 2], [150, 131]),
+    (1, 150, 40, 128, [3000], None),
 ])
 def test_matches_oracle(B, n, H, Dh, lens, n_active):
     for _ in range(2):
