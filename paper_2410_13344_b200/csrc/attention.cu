@@ -1459,7 +1459,7 @@ template <int DH, int WQ, int WK, int STAGES>
 int launch_cfg(AttnParams p, const CUtensorMap* tmK, const CUtensorMap* tmV, int B, int max_len, cudaStream_t st) {
   const int planned = p.nsplit;
   constexpr size_t smem = (size_t)STAGES * 2 * (DH / 64) * TILE * 128 + 1024;
-  static bool configured = false;
+  static std::atomic<bool> configured{false};
   if (!configured) {
     CERB_CUDA_OK(cudaFuncSetAttribute(tree_attn_bf16_kernel<DH, WQ, WK, STAGES>,
                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
@@ -1576,7 +1576,7 @@ static int launch_attn_window(cerb_ctx* c, const cerb_attn_args* a, int row0, in
   }
   const bool kt_path = a->head_dim == 128 && force_tc < 0 && rows <= 64 && (force_kt < 0 ? rows > 16 : force_kt != 0);
   if (kt_path || tensor_path) {
-    static bool configured = false;
+    static std::atomic<bool> configured{false};
     if (!configured) {
       for (auto kern : {tree_attn_kt_kernel<false>, tree_attn_kt_kernel<true>})
         CERB_CUDA_OK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)KT_SMEM));

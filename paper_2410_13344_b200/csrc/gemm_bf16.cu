@@ -519,7 +519,7 @@ int launch_gemm_bf16(cerb_ctx* c, const CUtensorMap* tmW, const ActMaps* tmX, fl
   p.idesc = idesc_bf16(BM, (uint32_t)p.n_mma, false, false);
   size_t smem = (size_t)p.stages * stage_bytes + 1024;
   if (smem < 120 * 1024) smem = 120 * 1024;    // one CTA per SM: a CTA may then own all of tensor memory
-  static bool configured = false;
+  static std::atomic<bool> configured{false};
   if (!configured) {
     CERB_CUDA_OK(cudaFuncSetAttribute(gemm_bf16_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(220 * 1024)));
     configured = true;

@@ -228,7 +228,7 @@ int launch(FewParams p, cudaStream_t st) {
   p.range = rounds * ROUND;
   p.rounds = (rounds + 1) & ~1;
   auto kern = gemm_few_kernel<KIND, NORM>;
-  static bool configured = false;
+  static std::atomic<bool> configured{false};
   if (!configured) {
     // the share of the SM's memory that two CTAs need as shared memory; the rest is L1
     constexpr size_t need = 2 * (2 * WARPS * ROWS * LD * sizeof(float) + (NORM ? kNormSmem : 0) + 1024), all = 228 * 1024;

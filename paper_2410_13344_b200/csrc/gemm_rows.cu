@@ -532,7 +532,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_rows_kernel(const __grid_con
 template <int KIND, int CG, bool MANY>
 int launch_kind(const CUtensorMap& tmW, const CUtensorMap& tmX, const RowsParams& p, int tiles, cudaStream_t st) {
   auto kern = gemm_rows_kernel<KIND, CG, MANY>;
-  static bool configured = false;
+  static std::atomic<bool> configured{false};
   if (!configured) {
     CERB_CUDA_OK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRing));
     configured = true;

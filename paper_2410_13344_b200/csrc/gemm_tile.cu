@@ -735,7 +735,7 @@ static int launch_kind(const CUtensorMap& tmW, const CUtensorMap& tmX, TileParam
   const size_t stage = HF * A_BYTES + (size_t)q.n_act * BK;
   q.stages = (int)(kRing / stage);
   if (q.stages > MAX_STAGES) q.stages = MAX_STAGES;
-  static bool configured = false;
+  static std::atomic<bool> configured{false};
   if (!configured) {
     CERB_CUDA_OK(cudaFuncSetAttribute(gemm_tile_kernel<KIND, HF>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(kRing + 1024)));
     configured = true;

@@ -425,7 +425,7 @@ template <int NT, int MT, int U, int KG, int MB>
 int launch_mma(cerb_ctx* c, const LevelParams& P, int max_rows, cudaStream_t st) {
   constexpr int ROWS = 16 * MT * (HM_WARPS / KG);
   constexpr size_t smem = (size_t)KG * ROWS * (8 * NT + 1) * sizeof(float);
-  static bool configured = false;
+  static std::atomic<bool> configured{false};
   if (!configured) {
     CERB_CUDA_OK(cudaFuncSetAttribute(head_mma_kernel<NT, MT, U, KG, MB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     configured = true;
@@ -456,7 +456,7 @@ int launch_level_mma(cerb_ctx* c, const LevelParams& P, int max_rows, cudaStream
 int launch_level(cerb_ctx* c, const LevelParams& P, int max_rows, int max_w, cudaStream_t st) {
   dim3 grid((max_rows + ROWS_PER_BLOCK - 1) / ROWS_PER_BLOCK, P.Hc);
   size_t smem1 = (size_t)max_w * sizeof(float);
-  static bool configured = false;
+  static std::atomic<bool> configured{false};
   if (!configured) {
     CERB_CUDA_OK(cudaFuncSetAttribute(head_gemv_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
     CERB_CUDA_OK(cudaFuncSetAttribute(head_gemv_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
