@@ -234,3 +234,17 @@ def test_load_refuses_gains_and_embeddings_off_their_boundary():
             for off in (4, step // 2, step - 2):
                 assert load(**{name: off}) == binding.E_ARG, (name, off)
         assert load(wqkv=4, wd=4) == binding.E_NOMEM
+
+
+def test_calls_find_the_current_stream_without_torch_internals(monkeypatch):
+    """The stream comes from two functions that torch does not document; a torch without either of them still has the documented way."""
+    import types
+    from paper_2410_13344_b200 import binding
+    monkeypatch.setattr(binding.torch.cuda, "current_stream", lambda: types.SimpleNamespace(cuda_stream=77))
+    monkeypatch.setattr(binding, "_CURRENT_DEVICE", lambda: 3)
+    monkeypatch.setattr(binding, "_RAW_STREAM", lambda device: 100 + device)
+    assert binding._stream() == 103
+    for name in ("_CURRENT_DEVICE", "_RAW_STREAM"):
+        with monkeypatch.context() as m:
+            m.setattr(binding, name, None)
+            assert binding._stream() == 77
