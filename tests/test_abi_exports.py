@@ -102,12 +102,12 @@ def test_no_kernel_reads_before_its_wait_what_the_kernel_in_front_writes():
     per kernel, the buffers written and the buffers read ahead of the wait; the rule is recomputed here."""
     from paper_2410_13344_b200 import binding
     CONST = 1 << 9
-    for variant in (0, 1, 2):
+    for variant in (0, 1, 2, 4):
         rc, rows = _launch_table(variant)
         assert rc == binding.OK
         names = [r[1] for r in rows]
         assert sum("gemm" in n for n in names) == 3 * 4 + 1 and sum(n == "tree attention" for n in names) == 3
-        assert ("swiglu" in names) == (variant == 0) and ("rope_append" in names) == (variant < 2)
+        assert ("swiglu" in names) == (variant in (0, 4)) and ("rope_append" in names) == (variant < 2)
         for i, (_, name, _, reads) in enumerate(rows):
             for bit in range(9):
                 if not reads >> bit & 1:
@@ -135,6 +135,29 @@ def test_every_forward_kernel_releases_its_dependents_after_its_own_wait():
                 seen += 1
                 assert 0 <= w < t, (fn, body[:80])
     assert seen >= 8
+
+
+def test_a_launch_that_follows_releases_its_dependents_behind_its_final_wait():
+    """A launch of attention that follows another one of the same call reads queries and keys without a wait of its own: its predecessor let it start
+    behind that one's own wait, and writes nothing that it reads.  The kernel behind it still has to find both complete: the launch that follows
+    waits for the first one at its end, and releases only then.  Both kernels that have such a form, form by form."""
+    src = os.path.join(ROOT, "paper_2410_13344_b200", "csrc")
+    seen = 0
+    for fn in ("attention.cu", "attention_kt.cuh"):
+        text = re.sub(r"//[^\n]*", "", open(os.path.join(src, fn)).read())
+        for body in re.split(r"__global__", text)[1:]:
+            body = body[:body.index("\n}\n")]
+            if "p.follows" not in body:
+                continue
+            seen += 1
+            enter = re.search(r"auto enter = \[&\]\(\) \{\s*if \(PART && p\.follows\) return;\s*griddep_wait\(\);\s*griddep_launch\(\);\s*\};", body)
+            end = re.search(r"if \(PART && p\.follows\) \{\s*griddep_wait\(\);\s*griddep_launch\(\);\s*\}\s*tc_fence_before\(\);\s*__syncthreads\(\);", body)
+            assert enter and end and enter.end() < end.start(), fn
+            rest = body[:enter.start()] + body[enter.end():end.start()] + body[end.end():]
+            # no other release, and no CTA leaves without a wait
+            assert "griddep_launch" not in rest and "p.follows" not in rest, fn
+            assert all(re.search(r"griddep_wait\(\);\s*$", rest[:m.start()]) for m in re.finditer(r"\breturn\s*;", rest)), fn
+    assert seen == 2
 
 
 def test_no_forward_kernel_leaves_ahead_of_its_wait():
@@ -187,7 +210,7 @@ def test_every_role_of_a_kernel_that_gives_up_sees_in_what_it_has_begun():
 
 def test_the_read_before_wait_rule_holds_in_every_variant():
     """The rule of test_no_kernel_reads_before_its_wait_what_the_kernel_in_front_writes over all exported launch sequences, those of
-    the forwards (0, 3, 5, 6, 7, 8) among them."""
+    the forwards among them (each is one for some shape and number of rows: fp32 and bf16, head_dim 64 and 128, up to 8, 128 and 256 rows and above)."""
     from paper_2410_13344_b200 import binding
     # variant: SwiGLU in a GEMM, RoPE in a GEMM, residual add in the GEMMs, norms in the GEMMs
     fused = {0: (0, 0, 0, 0), 1: (1, 0, 0, 0), 2: (1, 1, 0, 0), 3: (1, 1, 1, 0), 4: (0, 1, 0, 0), 5: (0, 0, 1, 0), 6: (1, 0, 1, 0), 7: (0, 1, 1, 0), 8: (1, 1, 1, 1)}

@@ -94,18 +94,24 @@ def test_trees_with_dead_nodes_match_oracle(n, live):
     assert changed <= sum(live)
 
 
-def test_launches_of_a_forward_are_the_table():
-    d, H, F = SHAPES["16 and 24 rows, ragged k block"]
+# residual adds in the products (3, 7) where O and down do not leave parts of k for the norm; SwiGLU a kernel of its own (7) in output tiles of 11000 features
+@pytest.mark.parametrize("name,n,B,variant", [("16 and 24 rows, ragged k block", 9, 1, 2), ("16 and 24 rows, ragged k block", 64, 2, 2),
+                                              ("16 and 24 rows, ragged k block", 65, 2, 3), ("32 and 152 rows, three MMAs per pair", 65, 2, 2),
+                                              ("32 and 152 rows, three MMAs per pair", 128, 2, 2), ("32 and 152 rows, three MMAs per pair", 129, 2, 7)])
+def test_launches_of_a_forward_are_the_table(name, n, B, variant):
+    d, H, F = SHAPES[name]
     ms = synth.ModelShape(3, d, H, 128, F, 512, "bf16")
-    for n, B, variant in ((9, 1, 2), (64, 2, 2), (65, 2, 3)):
-        rig = Rig(cb, ms, max_tokens=64, max_batch=B, max_nodes=n)
-        rig.eng.prefill(torch.zeros(B, 4, dtype=torch.int32, device="cuda"), [4] * B)
-        th = rig.eng.tree(synth.random_parent_tree(n, 4, tree_id=3, n_heads=4, kmax=1))
-        before = rig.eng.launch_count()
-        rig.eng.verify(th, torch.zeros(B, n, dtype=torch.int32, device="cuda"))
-        buf = C.create_string_buffer(1 << 14)
-        assert cb.lib().cerb_launch_order_table(variant, buf, len(buf)) == cb.OK
-        assert rig.eng.launch_count() - before == len(buf.value.decode().strip().split("\n"))
+    taken = n * B <= 256 and all(cb.forward_gemm_plan("o_down", n * B, d, k).rows_kernel for k in (128 * H, F))
+    assert taken == (n * B > 128 and variant == 2)
+    rig = Rig(cb, ms, max_tokens=64, max_batch=B, max_nodes=n)
+    rig.eng.prefill(torch.zeros(B, 4, dtype=torch.int32, device="cuda"), [4] * B)
+    th = rig.eng.tree(synth.random_parent_tree(n, 4, tree_id=3, n_heads=4, kmax=1))
+    before = rig.eng.launch_count()
+    rig.eng.verify(th, torch.zeros(B, n, dtype=torch.int32, device="cuda"))
+    buf = C.create_string_buffer(1 << 14)
+    assert cb.lib().cerb_launch_order_table(variant, buf, len(buf)) == cb.OK
+    # (a tree of more than 128 nodes: attention in two launches)
+    assert rig.eng.launch_count() - before == len(buf.value.decode().strip().split("\n")) + (3 if n > 128 else 0)
 
 
 # The LM head in one part, straight to the logits: columns that four divides, that eight does not, that four does not; rows of one and of two MMA heights

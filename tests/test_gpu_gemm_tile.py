@@ -106,9 +106,10 @@ def test_chains_of_accumulations_are_short(M, N, K):
 
 # Forwards whose GEMMs take the schedules above with an epilogue: (model, prompt length, GEMM, what its plan has to be)
 FORWARDS = {
-    "gate-up cut, 76 tiles": (synth.ModelShape(1, 2048, 16, 128, 9728, 512, "bf16"), 256, (19456, 2048), lambda g: g.cut_tiles == 76),
+    "gate-up cut, 76 tiles": (synth.ModelShape(1, 2048, 16, 128, 4864, 512, "bf16"), 300, (9728, 2048), lambda g: g.cut_tiles == 76),
     "gate-up cut, 38 tiles": (synth.ModelShape(1, 3072, 2, 128, 4864, 512, "bf16"), 150, (9728, 3072), lambda g: g.cut_tiles == 38),
     "qkv cut": (synth.ModelShape(1, 4096, 26, 128, 64, 512, "bf16"), 256, (9984, 4096), lambda g: g.cut_tiles > 0),
+    "qkv cut, 7B width": (synth.ModelShape(1, 4096, 32, 128, 64, 512, "bf16"), 150, (12288, 4096), lambda g: g.cut_tiles > 0),
     "down on 512-row tiles, several pairs each": (synth.ModelShape(1, 2048, 2, 128, 4096, 512, "bf16"), 1100, (2048, 4096),
                                                   lambda g: g.halves == 2 and g.pairs_per_tile > 1),
 }
@@ -118,6 +119,7 @@ FORWARDS = {
 def test_scheduled_epilogues_match_oracle(name):
     ms, n, (N, K), right = FORWARDS[name]
     assert right(cb.gemm_plan(n, N, K, fused=True)), cb.gemm_plan(n, N, K, fused=True)
+    assert n > 256 or not cb.forward_gemm_plan(name.split()[0].rstrip(",").replace("-", "_"), n, N, K).rows_kernel      # (the plan is the one that runs)
     rig = Rig(cb, ms, max_tokens=n + 16, max_nodes=16)
     prompt = [int(t) for t in synth.make_prompt(ms.vocab, n, seq=97)]
     tok = torch.tensor([prompt], dtype=torch.int32, device="cuda")

@@ -1,4 +1,4 @@
-"""Forwards of 9 to 128 rows whose products arrive as sums of few and of many slots: the kernels that add them up."""
+"""Forwards of 9 to 256 rows whose products arrive as sums of few and of many slots: the kernels that add them up."""
 import numpy as np
 import pytest
 import torch
@@ -16,25 +16,32 @@ def cb():
     return binding
 
 
-def _slots(cb, M, N, K):
+def _slots(cb, product, M, N, K):
+    """Slots that the product leaves in a forward of M rows; 0: its outputs are finished where they are summed."""
+    if M > 128 and product == "lm_head":
+        return 1
+    g = cb.forward_gemm_plan(product, M, N, K)
+    if g.rows_kernel:
+        return 0 if product == "gate_up" else g.parts
+    if M > 128:
+        return 0 if product == "gate_up" else 1
     nb = cb.C.c_size_t(0)
     assert cb.lib().cerb_gemm_scratch_bytes(M, N, K, cb.C.byref(nb)) == cb.OK
     return (nb.value - 256) // (4 * M * N)
 
 
-# Slots of the gate-up product: one trip to L2 (1, 2, 4), more (9, 17).  Slots of the down product: one trip (1, 4, 8), code of their own
-# (9, 10, 11), two trips (12, 14), two and four pieces of a row per thread.
-# Slots of the LM head: 1, 2, 4 and more; rows of more columns than are on their way at once, and of a length that four does not divide;
-# more rows than SMs (those of the last case, 200, leave no slots).  bf16 storage through one layer: the 2e-2 of every bf16 comparison, with weights of 1 / sqrt(d), so that queries and keys have
+# Slots of the gate-up product (SwiGLU as a kernel of its own: one, four), of the down product (the norm: one trip to L2 for one to eight, two and more for
+# 9 and 16, which only matrices of fewer than 16 rows per SM and part leave; two and four pieces of a row per thread) and of the LM head (one, two, four, eight and more;
+# rows of more columns than are on their way at once, and of a length that four does not divide); more rows than SMs (200 and 250).  bf16 storage through one layer: the 2e-2 of every bf16 comparison, with weights of 1 / sqrt(d), so that queries and keys have
 # elements of size one: rounding them (2^-9) then moves a score of 128 terms over sqrt(128) by 2^-8 or so, and with it a weight by 0.4 %.
 # (With weights of 0.03 at d = 8448 they are 2.8, and scores move by 0.03 x the scores' own spread of 8.)  An argmax is that of the logits.
-@pytest.mark.parametrize("d,mlp,vocab,n,slots", [(256, 256, 33000, 9, (1, 1, 1)), (1024, 2048, 1000, 17, (4, 8, 4)), (1024, 2304, 1002, 17, (4, 9, 4)),
-                                                 (1024, 2560, 1000, 64, (4, 10, 4)), (1024, 2816, 4100, 17, (4, 11, 4)), (1024, 3072, 1000, 33, (4, 12, 4)),
-                                                 (512, 3584, 520, 17, (2, 14, 2)), (4352, 2304, 1000, 17, (9, 8, 17)), (8448, 1024, 1000, 17, (17, 4, 33)),
-                                                 (256, 256, 1004, 100, None)])
+@pytest.mark.parametrize("d,mlp,vocab,n,slots", [(256, 256, 33000, 9, (1, 1, 1)), (1024, 512, 1000, 33, (4, 2, 4)), (1024, 2304, 1002, 17, (0, 8, 4)),
+                                                 (1024, 2560, 1000, 64, (0, 8, 4)), (512, 3584, 520, 17, (0, 8, 2)), (128, 2304, 1000, 17, (0, 9, 1)),
+                                                 (128, 4096, 1000, 33, (0, 16, 1)), (2560, 4096, 1000, 17, (0, 8, 10)), (4096, 11008, 1000, 32, (0, 5, 8)),
+                                                 (4352, 2304, 1000, 17, (0, 4, 8)), (8448, 2304, 1000, 17, (0, 3, 8)), (8448, 1024, 1000, 17, (0, 2, 8)),
+                                                 (256, 256, 1004, 100, (0, 1, 1)), (2048, 5632, 1000, 125, (0, 5, 1))])
 def test_forward_over_slots(cb, d, mlp, vocab, n, slots):
-    if slots:
-        assert (_slots(cb, 2 * n, 2 * mlp, d), _slots(cb, 2 * n, d, mlp), _slots(cb, 2 * n, vocab, d)) == slots
+    assert (_slots(cb, "gate_up", 2 * n, 2 * mlp, d), _slots(cb, "o_down", 2 * n, d, mlp), _slots(cb, "lm_head", 2 * n, vocab, d)) == slots
     ms = synth.ModelShape(1, d, 4, 128, mlp, vocab, "bf16")
     model = synth.make_model(ms, device="cuda", std=d ** -0.5)
     cmodel = {k: v.cpu() for k, v in model.items()}
