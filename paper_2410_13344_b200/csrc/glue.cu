@@ -427,11 +427,12 @@ int launch_fused_norm(cerb_ctx* c, const float* part, int nsplit, size_t split_s
                  tok ? (const T*)c->embed : (const T*)nullptr, tok, tok_stride, tok_off, (const int32_t*)c->d_nactive, n, g.vocab,
                  (const T*)gain, (T*)out, d, g.rms_eps, row_off, c->B);
     };
-    // A product leaves at most eight slots: of up to 8192 columns they are one trip to L2; wider rows take two at a time.  More rows than SMs, with three to
-    // five slots: two blocks of half the threads to an SM (256 rows of 4096 / 5120 columns 6.7 / 7.6 -> 5.0 / 5.0 us).
+    // Products of gemm_rows.cu leave at most eight slots: of up to 8192 columns they are one trip to L2; wider rows take two at a time.  (Matrices that it does not take,
+    // of fewer than 16 rows per SM and part of k, leave up to 16: two trips and more.)  More rows than SMs, with slots: two blocks of half the
+    // threads to an SM (256 rows of 4096 / 5120 columns 6.7 / 7.6 -> 5.0 / 5.0 us; without slots 2048-row forwards of 4096 columns took 26.14 ms so and 26.00 with one block).
     const bool one = d <= NORM_THREADS * 4;
-    if (c->bf16 && rows > c->sm_count && one) go(fused_norm_kernel<bf16, 2, 4, NORM_THREADS / 2>, bf16(), NORM_THREADS / 2);
-    else if (c->bf16 && rows > c->sm_count && d <= NORM_THREADS * 6) go(fused_norm_kernel<bf16, 3, 4, NORM_THREADS / 2>, bf16(), NORM_THREADS / 2);
+    if (c->bf16 && nsplit > 0 && rows > c->sm_count && one) go(fused_norm_kernel<bf16, 2, 4, NORM_THREADS / 2>, bf16(), NORM_THREADS / 2);
+    else if (c->bf16 && nsplit > 0 && rows > c->sm_count && d <= NORM_THREADS * 6) go(fused_norm_kernel<bf16, 3, 4, NORM_THREADS / 2>, bf16(), NORM_THREADS / 2);
     else if (c->bf16 && one) go(fused_norm_kernel<bf16, 1, 8>, bf16());
     else if (c->bf16 && d <= NORM_THREADS * 8) go(fused_norm_kernel<bf16, 2, 8>, bf16());
     else if (c->bf16) go(fused_norm_kernel<bf16, NORM_MAX_ITER, 2>, bf16());
