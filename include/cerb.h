@@ -286,7 +286,8 @@ int cerb_tree_attention_noalloc_status(void* stream);
 /* Ancestor bitmasks of a tree, the form cerb_tree_attention takes: anc_out host [n][CERB_ANC_WORDS]. */
 int cerb_tree_ancestors(const int32_t* parent, int32_t n, uint64_t* anc_out);
 
-/* Stand-alone dense GEMM as the verification forward runs it (Algorithm 1, TL_i / LH):
+/* Stand-alone dense GEMM (Algorithm 1, TL_i / LH; a forward of 9 to 256 rows runs most of its products in another kernel,
+ * see cerb_forward_gemm_plan):
  * out[M][N] (fp32) = X[M][K] . W[N][K]^T, X and W in `dtype`, fp32 accumulation.
  * bf16: X and W 16-byte aligned, K a multiple of 8, weights streamed once; up to 8 rows warp MMAs fed from global
  * memory, up to 128 rows tcgen05 with the split-K partial sums in scratch, above that output tiles on CTA pairs, which use
@@ -294,7 +295,7 @@ int cerb_tree_ancestors(const int32_t* parent, int32_t n, uint64_t* anc_out);
 int cerb_gemm_scratch_bytes(int32_t M, int32_t N, int32_t K, size_t* bytes_out);
 /* How the bf16 GEMM of more than 128 rows cuts this problem up (host only, for tests and measurement; the paper has no
  * counterpart): as cerb_gemm runs it (fused = 0, with the scratch that cerb_gemm_scratch_bytes asks for), or inside the
- * forward with an epilogue (fused = 1).  out8_host: [0] weight tiles of 256 rows that share an activation tile, [1] chunks of
+ * forward with an epilogue (fused = 1: above 256 rows, and up to there what cerb_forward_gemm_plan does not give to the other kernel).  out8_host: [0] weight tiles of 256 rows that share an activation tile, [1] chunks of
  * rows, [2] rows of a chunk, [3] tiles, [4] CTA pairs per tile, [5] tiles cut along k into equal shares, [6] CTA pairs,
  * [7] chains of accumulations per output of a run (fused = 0: fills of an accumulator). */
 int cerb_gemm_plan(int32_t M, int32_t N, int32_t K, int32_t fused, int32_t* out8_host);
@@ -350,13 +351,13 @@ int cerb_set_wait_cycles(int64_t cycles);
 /* The launch sequence of the base-model forward with, per kernel, the buffers it writes and the buffers it reads
  * ahead of its dependency wait (bit masks; the paper has no counterpart, this documents the library's use of
  * programmatic dependent launch).  Writes one line per launch, "id|name|writes|reads-before-wait", for one set-up
- * launch, three layers and the tail, into buf (host).  variant 0: separate SwiGLU and RoPE kernels (steps of 9
- * to 128 rows).  With the residual add inside the O and down GEMMs (steps above 128 rows and of up to 8): 3 with SwiGLU inside the
- * gate-up GEMM and RoPE + cache append inside the QKV GEMM, 5 without either, 6 with SwiGLU, 7 with RoPE; 8: variant 3 with
+ * launch, three layers and the tail, into buf (host).  Sums of O and down left for the norm to add (9 to 128 rows,
+ * and up to 256 where cerb_forward_gemm_plan gives it both products): variant 2 with SwiGLU inside the gate-up GEMM and RoPE + cache append
+ * inside the QKV GEMM, 1 with SwiGLU only, 4 with RoPE only, 0 with separate kernels for both, as the plans of the two products and head_dim say.
+ * With the residual add inside the O and down GEMMs (other steps above 128 rows, and of up to 8): 3 with both, 5 without either, 6 with SwiGLU, 7 with RoPE; 8: variant 3 with
  * the norms inside the QKV and gate-up GEMMs (up to 8 rows, as far as they fit: two of 4096 columns).  fp32 models: 8 with up to 256
  * columns, else 3, while the layers' matrices start on 16-byte boundaries and each of their products has fewer than 296 tiles of 64 x 64
- * outputs; else 0.  1 (SwiGLU alone), 2 (SwiGLU
- * and RoPE) and 4 (RoPE alone) describe no forward any more.  Returns CERB_OK when no kernel reads, ahead of its wait, a buffer
+ * outputs; else 0.  Returns CERB_OK when no kernel reads, ahead of its wait, a buffer
  * that the kernel right in front of it writes, CERB_E_STATE otherwise, CERB_E_NOMEM when buf is too small. */
 int cerb_launch_order_table(int32_t variant, char* buf_host, size_t cap);
 

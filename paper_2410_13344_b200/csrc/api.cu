@@ -240,13 +240,14 @@ int tree_build(cerb_ctx* c, const int32_t* parent, const int32_t* head_of, const
 int rows_sums_parts(int M, int N, int K) { return M > 128 ? 8 : gemm_plan_split(148, M, N, K); }
 RowsPlan rows_sums_plan(int b, int N, int K) {
   // Above 128 rows, against output tiles that pairs add up through a fix-up buffer (8-layer forwards of 129 / 192 / 256 rows): 1024 columns 1.26 / 1.28 / 1.29 x,
-  // 2048 1.17 / 1.19 / 1.18 x, 4096 1.03 / 1.02 / 1.035 x, 5120 0.98 / 1.00 / 1.012 x, 8192 0.99 / 1.00 / 0.955 x.  (The wider the output, the fewer
+  // 2048 1.17 / 1.19 / 1.18 x, 4096 1.03 / 1.02 / 1.035 x, 5120 0.98 / 1.00 / 1.012 x (220 rows 1.00 x), 8192 0.99 / 1.00 / 0.955 x.  (The wider the output, the fewer
   // parts and the less there was to add up; and the MMAs of output tiles follow the rows, a pair's are 256 high.)
   const int limit = rows_class_limit(b);
   if (limit > 128 && N > (limit == 192 ? 4096 : 6144)) return RowsPlan{};
   return plan_rows_sums(limit, N, K, rows_sums_parts(limit, N, K));
 }
-// The LM head: up to 128 rows.  (One part: its sums go straight to the logits.  4096 columns and more: 13B forwards 1.005 to 1.015 x; 1024 columns 0.98 x)
+// The LM head: up to 128 rows.  (One part: its sums go straight to the logits.  4096 columns and more: 13B forwards 1.005 to 1.015 x; 1024 / 1536 / 2048 columns 0.98 to 0.995 /
+// 0.995 to 1.00 / 0.99 to 1.00 x, 3200 0.994 at 9 rows to 1.012 at 96.)
 bool lm_head_in_rows(int d_model) { return d_model >= 4096; }
 int make_rows_sums(RowsSums* s, const void* const* W, int layers, int N, int K, int rows) {
   for (int b = 0; b < kRowsClasses && rows_class_limit(b) <= rows; ++b) {
@@ -352,7 +353,7 @@ int forward_rows(cerb_ctx* c, const cerb_tree* tree, const int32_t* tok, int tok
     if (c->h_len[b] + nb > max_len) max_len = c->h_len[b] + nb;
   }
   // Up to 8 rows and above 128, whatever follows a GEMM runs in its epilogue: SwiGLU, (head_dim 128) RoPE + cache append,
-  // the residual adds.
+  // the residual adds (but for those of up to 256 rows that are left to the norm, below).
   // fp32: the same as long as the GEMMs have few output tiles.
   const bool small = !c->bf16 && c->f32_aligned && gemm_f32_small(M, 2 * F) && gemm_f32_small(M, 3 * HD) && gemm_f32_small(M, d);
   const bool wide = small || (c->bf16 && (M > 128 || M <= kFewRows));

@@ -2,7 +2,7 @@
 // finished where they are summed, and plain sums (O, down, up to 128 rows the LM head) in few parts of k.
 //
 //   CG = 1:  D[128 activation rows][w weight rows] per CTA
-//   CG = 2:  D[256 activation rows][2 w weight rows] per pair of CTAs (cta_group::2), fp32, in tensor memory; one tile, all of k
+//   CG = 2:  D[256 activation rows][2 w weight rows] per pair of CTAs (cta_group::2), fp32, in tensor memory; one tile each, of all of k or of a part of it
 //
 // What bounds it: the weight stream up to 64 rows, then L2 on its way to the SMs.  The activation rows are the MMA's M side (rows that do not exist
 // are whatever lies behind them in shared memory; they only reach accumulator rows that nobody reads), the weight rows its N side, which comes

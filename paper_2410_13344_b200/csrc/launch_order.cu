@@ -73,7 +73,7 @@ const Entry kQkvNorm = {LO_GEMM_QKV, "gemm norm + qkv + rope / append epilogue",
 const Entry kGuNorm = {LO_GEMM_GU, "gemm norm + gate-up + swiglu epilogue", B_ACT, B_CONST};
 
 // Variants 0, 1, 2 and 4 are the steps of 9 to 128 rows (bf16): a tile per SM finishes SwiGLU, RoPE + cache append or both, where the matrix has the size
-// for it (gemm_rows.cu).  Those with a residual add in the GEMMs occur above and up to 8 rows, the norms in
+// for it (gemm_rows.cu); and of up to 256 rows where O and down leave parts of k for the norm.  Those with a residual add in the GEMMs occur above and up to 8 rows, the norms in
 // the GEMMs (8) with as many of those as gemm_few_normalises allows.  fp32 models take 8 or, above kF32NormMax columns, 3 as long as their
 // GEMMs have few output tiles, 0 otherwise.
 constexpr int kVariants = 9;
