@@ -656,8 +656,8 @@ RowsPlan plan_rows_rope(int n_heads, int head_dim, int K) {
 //   Up to 128 rows, against partial sums and kernels behind them: matrices of at least 16 rows per SM (an MMA's N is no less) and at most 256.
 //   Forwards, plain sums (below) included: 7B width 9 / 64 / 128 rows 1.06 / 1.06 / 1.12 x, 13B 1.02 / 1.09 / 1.13 x, 1024 to 3200 columns 1.04 to 1.25 x.
 //   129 to 256 rows, in pairs, against output tiles of 256 weight rows (gemm_tile.cu): a pair's tile has to fit one MMA, or (SwiGLU, 16 k
-//   blocks and more, up to 304 columns) three as above.  Tiles of 256 rows leave SMs idle or have to be cut along k: 7B width, gate-up of 129 / 256 rows 46 / 53 -> 42 /
-//   44 us.  RoPE from 193 rows on: below, the output tiles are cut and sum shorter chains than those that fit here (keys of 130 to 180 rows against float64
+//   blocks and more, up to 304 columns) three as above.  Tiles of 256 rows leave SMs idle or have to be cut along k: 7B width, gate-up of 129 / 256 rows 46 / 53 -> 41 /
+//   43 us with two MMAs a tile, and 1 us more with three (as above).  RoPE from 193 rows on: below, the output tiles are cut and sum shorter chains than those that fit here (keys of 130 to 180 rows against float64
 //   1.10e-4 to 1.32e-4 there, 1.32e-4 to 1.52e-4 here).  From 193 rows on they are as long at 4096 columns and more (QKV of 256 rows 32.5 -> 27 us) and fit at 1024
 //   and 1536; from 2048 to 3584 they do not (2048 columns, 2 x 128 rows, 8 layers: 580 us here, 645 with output tiles; V 0.44 against 0.24e-6 from float64).
 bool gemm_rows_takes(const RowsPlan& g, int M) {
